@@ -563,14 +563,28 @@ static int copy_blob(anakin_t* h, int which, void* ptr, size_t bytes, int ptr_is
                               : ptr_is_device == 2 ? cudaMemcpyDefault
                               : (to_lib ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost);
     cudaError_t e = cudaSuccess;
-    {   // one copy per policy: its blob sits at the same offset inside its sub-workspace
-        unsigned char* user = static_cast<unsigned char*>(ptr);
-        for (int p = 0; p < h->K && e == cudaSuccess; ++p) {
-            const size_t n = p == h->K - 1 ? blob_of(h, which, h->d.B_last).bytes : bl.bytes;
-            unsigned char* mine = static_cast<unsigned char*>(bl.ptr) + (size_t)p * h->sub_bytes;
-            e = to_lib ? cudaMemcpyAsync(mine, user, n, kind, h->stream) : cudaMemcpyAsync(user, mine, n, kind, h->stream);
-            user += n;
-        }
+    if (h->K == 1) {
+        e = to_lib ? cudaMemcpyAsync(bl.ptr, ptr, bytes, kind, h->stream) : cudaMemcpyAsync(ptr, bl.ptr, bytes, kind, h->stream);
+    } else {  // policy p's blob: contiguous on the caller's side, sub_bytes apart here; the last policy may have fewer envs
+        const size_t full = h->K - (h->d.B_last == h->d.B ? 0 : 1), n = bl.bytes;
+        auto move = [&](unsigned char* mine, unsigned char* user, size_t width, size_t rows) {
+            if (rows == 0 || width == 0) return cudaSuccess;
+            void *dst = to_lib ? mine : user, *src = to_lib ? user : mine;
+            const size_t dp = to_lib ? h->sub_bytes : width, sp = to_lib ? width : h->sub_bytes;
+            if (ptr_is_device == 1) {
+                ++h->launches;
+                return launch_copy_blocks(dst, dp, src, sp, width, rows, h->stream);
+            }
+            if (h->sub_bytes <= 0x7FFFFFFFu) return cudaMemcpy2DAsync(dst, dp, src, sp, width, rows, kind, h->stream);
+            cudaError_t er = cudaSuccess;  // beyond the largest pitch a 2-D copy takes
+            for (size_t r = 0; r < rows && er == cudaSuccess; ++r)
+                er = cudaMemcpyAsync((char*)dst + r * dp, (const char*)src + r * sp, width, kind, h->stream);
+            return er;
+        };
+        unsigned char *mine = static_cast<unsigned char*>(bl.ptr), *user = static_cast<unsigned char*>(ptr);
+        e = move(mine, user, n, full);
+        if (e == cudaSuccess && full < (size_t)h->K)
+            e = move(mine + full * h->sub_bytes, user + full * n, blob_of(h, which, h->d.B_last).bytes, 1);
     }
     if (e != cudaSuccess) return fail_cuda(h, e);
     if (to_lib) {

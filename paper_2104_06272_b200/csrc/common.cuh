@@ -340,6 +340,7 @@ cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int apl, int bpl, 
 // kernels (defined in the .cu files) ----------------------------------------------------------------
 cudaError_t launch_reset(const Dims& d, const Buffers& b, uint64_t seed, double density, int prec, const Ctx& c);
 cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c);
+cudaError_t launch_copy_blocks(void* dst, size_t dpitch, const void* src, size_t spitch, size_t bytes, size_t rows, cudaStream_t s);
 cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c);
 cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s);  // cudaErrorNotSupported if not covered
 bool rollout_mma_supported(int H);

@@ -240,3 +240,26 @@ def test_policies_runs_are_bitwise_deterministic_and_limits_are_refused(bnd):
         with pytest.raises(bnd.AnakinError) as e:
             bnd.workspace_bytes(bnd.make_cfg(**args))
         assert e.value.code == code, kw
+
+
+@pytest.mark.parametrize("name", ["k3_h64_ragged", "k64_h64", "k5_h128"])
+def test_policies_blobs_by_device_pinned_and_host_copies_agree(bnd, name):
+    """A blob of many policies moves in one strided copy; the last, smaller policy in a second one: all three kinds of
+    pointer, both directions, blobs whose size is not a multiple of four bytes among them."""
+    w = CASES[name]
+    an = make(bnd, w)
+    an.reset(5)
+    an.run(1)
+    for which in (bnd.PARAMS, bnd.ENV_POS, bnd.ENV_WALLS, bnd.TRAJ_ACTION, bnd.TRAJ_VALUE, bnd.DEBUG_GATES):
+        want = an.get(which).view(np.uint8).reshape(-1)
+        dev = torch.zeros(want.size, dtype=torch.uint8, device="cuda")
+        pin = torch.zeros(want.size, dtype=torch.uint8).pin_memory()
+        an.get_into(which, dev)
+        an.get_into(which, pin, wait=False)
+        assert an.status() == 0
+        assert np.array_equal(dev.cpu().numpy(), want) and np.array_equal(pin.numpy(), want)
+    rev = torch.from_numpy(an.get(bnd.TRAJ_ACTION)).flip(0).contiguous()
+    for value in (rev.cuda(), rev, rev.pin_memory()):
+        an.set(bnd.TRAJ_ACTION, torch.zeros_like(rev).cuda())
+        an.set(bnd.TRAJ_ACTION, value)
+        assert np.array_equal(an.get(bnd.TRAJ_ACTION), rev.numpy())
