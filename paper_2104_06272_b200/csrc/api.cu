@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/anakin.h: configuration checks, workspace carving, state
 // tracking and kernel enqueueing.  The host only schedules (Podracer paper, Section 3.1): no call in the
 // rollout/learn/run path copies data or synchronises.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -113,15 +114,17 @@ size_t carve(const anakin_cfg& c, const Dims& d, int NS, unsigned char* base, Bu
     const bool frags = mma && rollout_uses_fragments(d.H, c.precision);
     b.w2f_hi = frags ? (uint2*)take(H * H * 2) : nullptr;
     b.w2f_lo = frags ? (uint2*)take(H * H * 2) : nullptr;
-    b.w2p_hi = tensor ? (uint16_t*)take(H * H * 2) : nullptr;
+    const bool wide = wide_supported(d.H, c.precision), f32 = c.precision == ANAKIN_PRECISION_FP32;
+    b.w2p_hi = tensor ? (uint16_t*)take(H * H * 2 * (wide && f32 ? 3 : 1)) : nullptr;
     b.w2p_lo = mma ? (uint16_t*)take(H * H * 2) : nullptr;
-    b.h1 = (float*)take(R * H * 4);
+    // wide layers: bf16 planes of h1 (three exact terms in fp32 workloads) with room for the bootstrap step's rows; h2 likewise
+    b.h1 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 6 : 2) : R * H * 4);
     b.gate1 = (dh1_agent_tc_supported(d) && policies_of(c) <= 1) ? (uint8_t*)take(R * (H / 8)) : nullptr;  // what the fused dh1 kernel gates with
-    b.h2 = (float*)take(R * H * 4);
+    b.h2 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 4 : 2) : R * H * 4);
     b.out5 = tensor ? (float*)take(R * 8 * 4) : nullptr;
     b.vboot = tensor ? (float*)take(B * 4) : nullptr;
-    b.dh2 = (float*)take(R * H * 4);
-    b.dh1 = (float*)take(R * H * 4);
+    b.dh2 = (float*)take(R * H * (!wide ? 4 : f32 ? 6 : 2));
+    b.dh1 = (float*)take(!wide ? R * H * 4 : std::max(R * H * (f32 ? 4 : 2), wide_scratch_bytes(d)));
     b.dout = (float*)take(R * 8 * 4);
     b.S = (float*)take(4 * B * H * 4);  // up to four t-slices of two 16-bit planes
     size_t part_floats = (size_t)NS * P, loss_blocks = LOSS_BLOCKS;
@@ -465,7 +468,10 @@ int anakin_learn_ppo(anakin_t* h, int epochs, float clip_eps) {
 int anakin_learn_vtrace(anakin_t* h, int epochs, float rho_bar, float c_bar) {
     if (!h || epochs < 1 || !(rho_bar >= 0.f) || !(c_bar >= 0.f)) return ANAKIN_E_INVALID_ARG;
     if (!h->is_reset || !h->rollout_pending) return ANAKIN_E_BAD_STATE;
-    if (h->K > 1 || !tensor_path_supported(h->d.H, h->cfg.precision)) return ANAKIN_E_UNSUPPORTED_CFG;  // needs the saved head outputs
+    // the hidden widths this objective is offered at
+    const int H = h->d.H;
+    const bool offered = rollout_mma_supported(H) || (h->cfg.precision == ANAKIN_PRECISION_BF16 && (H == 512 || H == 1024));
+    if (h->K > 1 || !offered) return ANAKIN_E_UNSUPPORTED_CFG;
     for (int ep = 0; ep < epochs; ++ep) {
         cudaError_t e;
         if (!h->base_valid) {

@@ -70,7 +70,7 @@ struct Buffers {
     float* base;     // [B][H]  b1 + sum of W1 rows of the wall cells + W1 row of the goal cell
     uint2* w2f_hi;   // [H*H/4] W2 as mma.sync B fragments, high parts (null: the warp-level rollout kernel is not used)
     uint2* w2f_lo;   // [H*H/4] bf16 low parts
-    uint16_t* w2p_hi;  // [H][H] W2 row-major as 16-bit hi / lo planes (B operand of the dh1 kernel)
+    uint16_t* w2p_hi;  // [H][H] W2 row-major as 16-bit hi / lo planes (B operand of the dh1 kernel); wide fp32: three bf16 planes
     uint16_t* w2p_lo;
     float* h1;       // [R][H]
     uint8_t* gate1;  // [R][H/8] layer-1 ReLU gates of every recorded row: bit j%8 of byte j/8 = the 16-bit hi term of h1[j] is not zero (null: not kept)
@@ -348,7 +348,12 @@ bool rollout_uses_fragments(int H, int prec);  // the warp-level kernel (and wit
 cudaError_t launch_rollout_tc128(const RolloutArgs& a, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, fp32, large batches); cudaErrorNotSupported otherwise
 cudaError_t launch_rollout_pair2(const RolloutArgs& a, cudaStream_t s);  // two env groups per CTA pair (H = 256, fp32, large batches); cudaErrorNotSupported otherwise
 cudaError_t launch_rollout_pair(const RolloutArgs& a, cudaStream_t s);  // CTA-pair tcgen05 rollout (H = 256, fp32); cudaErrorNotSupported otherwise
-bool wide_supported(int H, int prec);         // bf16 workload with a hidden layer too wide for the persistent rollout
+bool wide_supported(int H, int prec);         // hidden layer too wide for the persistent rollouts (either precision)
+size_t wide_h1_rows(const Dims& d);           // rows of one h1 / h2 plane on that path: the recorded ones and the bootstrap step's
+size_t wide_scratch_bytes(const Dims& d);     // operands of the base GEMM (kept in the dh1 buffer)
+int agent_plane_splits(const Dims& d);
+// agent plane of dW1 (ns partials) and S from the fp32 dh1 rows
+cudaError_t launch_agent_plane(const LearnArgs& a, int ns, float* part, size_t stride, const Ctx& c);
 bool tensor_path_supported(int H, int prec);  // either tensor-core path: the update reuses activations the rollout saved
 cudaError_t launch_rollout_wide(const RolloutArgs& a, const Ctx& c);  // T+1 forward passes, or the replay of recorded rows
 cudaError_t launch_pack_w2_wide(const Dims& d, const Buffers& b, const Ctx& c);

@@ -252,6 +252,9 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
 //     bound on the weight gradients.)  fp16 has a narrow exponent range, so gradient-side tensors are carried
 //     multiplied by a power of two (LearnArgs::gscale) that is divided out exactly when the partials are reduced.
 //   PREC 1 (bf16 workload): operands are bf16 values already; one bf16 product, no lo term.
+//   PREC 2 (fp32 workloads at the other hidden widths): every fp32 operand is the EXACT sum of three bf16 terms (8 + 8 + 8
+//     significand bits, full fp32 exponent range); six bf16 products (all but mid*lo, lo*mid, lo*lo, which are below 2^-24 of
+//     the product) accumulated in fp32.
 // pack2<PREC> rounds two consecutive elements to the 16-bit format: the lower-index element goes to the low half.
 template <int PREC>
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -267,6 +270,16 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
         lo = *reinterpret_cast<const uint32_t*>(&l);
     }
 }
+// PREC 2: two consecutive elements as three packed bf16 terms, x = t[0] + t[1] + t[2] (both subtractions are exact).
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t (&t)[3]) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+        t[q] = *reinterpret_cast<const uint32_t*>(&h);
+        x0 -= __uint_as_float(t[q] << 16);
+        x1 -= __uint_as_float(t[q] & 0xFFFF0000u);
+    }
+}
 template <int PREC>
 __device__ __forceinline__ void split1(float x, uint16_t& hi, uint16_t& lo) {
     if (PREC == 1) {
@@ -280,7 +293,7 @@ __device__ __forceinline__ void split1(float x, uint16_t& hi, uint16_t& lo) {
 }
 template <int PREC>
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    if (PREC == 1) mma_bf16(d, a, b0, b1);
+    if (PREC >= 1) mma_bf16(d, a, b0, b1);
     else mma_f16(d, a, b0, b1);
 }
 // Two-term bf16 split (used for fp32 sums that feed a bf16 product in the bf16 workload).
@@ -300,6 +313,6 @@ __device__ __forceinline__ uint32_t nonzero_bits16(const uint4& v) {
     return m;
 }
 // 1.0 in the 16-bit operand format
-template <int PREC> __device__ __forceinline__ uint32_t one16() { return PREC == 1 ? 0x3F80u : 0x3C00u; }
+template <int PREC> __device__ __forceinline__ uint32_t one16() { return PREC >= 1 ? 0x3F80u : 0x3C00u; }
 
 }  // namespace anakin

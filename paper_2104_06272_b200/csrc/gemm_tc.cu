@@ -74,7 +74,7 @@ bool make_tensor_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint6
 // synthesized-A modes are bound by their builder threads, and a second CTA hides them).
 template <int BN, int APL, int BPL, bool DEEP, int PREC = 0>
 struct GemmTcCfg {
-    static constexpr int BM = 128, KC = 64, THREADS = 192;
+    static constexpr int BM = 128, KC = 64, THREADS = DEEP && PREC == 2 ? 320 : 192;
     static constexpr int BOX = 64 * 64 * 2;                  // one 64 x 64 box of 16-bit elements
     static constexpr int A_PLANE = (BM / 64) * BOX;          // 16 KB
     static constexpr int B_PLANE = (BN / 64) * BOX;
@@ -85,17 +85,22 @@ struct GemmTcCfg {
     static constexpr size_t smem_bytes = (size_t)STAGES * STAGE + 1024 /*alignment slack*/ + 128 /*barriers, tmem slot*/;
     // plane operands of the fp32 workloads: two accumulators, a group of GROUP 64-row chunks (4096 rows, 768 MMAs) each.
     // The bf16 workload's 2e-2 bound does not need it.
-    static constexpr bool FLUSH = DEEP && PREC == 0;
-    static constexpr int GROUP = 64;
+    static constexpr bool FLUSH = DEEP && PREC != 1;
+    // fp32 as three bf16 terms (plane operands): a stage holds all three terms of both operands, so that a staged byte feeds two
+    // MMAs; every 64-row chunk is an accumulator group of its own (products smallest first, four leading MMAs), and the groups
+    // are added with round-to-nearest in the registers of eight epilogue warps.
+    static constexpr bool X3 = PREC == 2 && DEEP;
+    static constexpr int GROUP = X3 ? 1 : 64;
+    static constexpr int EPI_THREADS = X3 ? 256 : 128;
     static constexpr int TMEM_COLS = FLUSH ? 2 * BN : BN;
 };
 
 struct GemmTcMaps {
-    CUtensorMap a_hi, a_lo, b_hi, b_lo;
+    CUtensorMap a_hi, a_lo, a_lo2, b_hi, b_lo, b_lo2;
 };
 
 template <int BN, int AMODE, int APL, int BPL, int PREC>
-__global__ void __launch_bounds__(192, 1) k_gemm_tn_tc(const __grid_constant__ GemmTcMaps maps, GemmTnArgs g, int* status) {
+__global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>::THREADS), 1) k_gemm_tn_tc(const __grid_constant__ GemmTcMaps maps, GemmTnArgs g, int* status) {
     using Cfg = GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>;
     constexpr int BM = Cfg::BM, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -118,7 +123,7 @@ __global__ void __launch_bounds__(192, 1) k_gemm_tn_tc(const __grid_constant__ G
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&bars[s], 1 + NBUILD); tc::mbar_init(&bars[STAGES + s], 1); }
-        for (int q = 0; q < 2; ++q) { tc::mbar_init(&accfull[q], 1); tc::mbar_init(&accempty[q], 128); }
+        for (int q = 0; q < 2; ++q) { tc::mbar_init(&accfull[q], 1); tc::mbar_init(&accempty[q], Cfg::EPI_THREADS); }
         tc::mbar_fence_init();
     }
     if (wid == 2) tc::tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
@@ -141,14 +146,16 @@ __global__ void __launch_bounds__(192, 1) k_gemm_tn_tc(const __grid_constant__ G
 #pragma unroll
                     for (int bx = 0; bx < BM / 64; ++bx) {
                         tc::tma_load_2d(st + bx * Cfg::BOX, &maps.a_hi, &bars[s], m0 + 64 * bx, k0);
-                        if (APL == 2) tc::tma_load_2d(st + Cfg::A_PLANE + bx * Cfg::BOX, &maps.a_lo, &bars[s], m0 + 64 * bx, k0);
+                        if (APL == 3) tc::tma_load_2d(st + 2 * Cfg::A_PLANE + bx * Cfg::BOX, &maps.a_lo2, &bars[s], m0 + 64 * bx, k0);
+                        if (APL >= 2) tc::tma_load_2d(st + Cfg::A_PLANE + bx * Cfg::BOX, &maps.a_lo, &bars[s], m0 + 64 * bx, k0);
                     }
                 }
                 unsigned char* sb = st + APL * Cfg::A_PLANE;
 #pragma unroll
                 for (int bx = 0; bx < BN / 64; ++bx) {
                     tc::tma_load_2d(sb + bx * Cfg::BOX, &maps.b_hi, &bars[s], n0 + 64 * bx, k0);
-                    if (BPL == 2) tc::tma_load_2d(sb + Cfg::B_PLANE + bx * Cfg::BOX, &maps.b_lo, &bars[s], n0 + 64 * bx, k0);
+                    if (BPL >= 2) tc::tma_load_2d(sb + Cfg::B_PLANE + bx * Cfg::BOX, &maps.b_lo, &bars[s], n0 + 64 * bx, k0);
+                    if (BPL == 3) tc::tma_load_2d(sb + 2 * Cfg::B_PLANE + bx * Cfg::BOX, &maps.b_lo2, &bars[s], n0 + 64 * bx, k0);
                 }
             }
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
@@ -167,6 +174,14 @@ __global__ void __launch_bounds__(192, 1) k_gemm_tn_tc(const __grid_constant__ G
                 tc::tc_fence_after();
                 unsigned char* sa = base + s * Cfg::STAGE;
                 unsigned char* sb = sa + APL * Cfg::A_PLANE;
+                if constexpr (Cfg::X3) {
+#pragma unroll
+                    for (int i = 0; i < tc::X3_PAIRS; ++i)
+#pragma unroll
+                        for (int k16 = 0; k16 < KC / 16; ++k16)
+                            tc::umma(acc, tc::umma_desc(sa + tc::x3_a(i) * Cfg::A_PLANE + k16 * 2048, Cfg::BOX, 1024),
+                                     tc::umma_desc(sb + tc::x3_b(i) * Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, (i > 0 || k16 > 0) ? 1u : 0u);
+                } else
 #pragma unroll
                 for (int k16 = 0; k16 < KC / 16; ++k16) {
                     // 16 k rows = two 8-row groups = 2048 bytes further into every box
@@ -174,7 +189,8 @@ __global__ void __launch_bounds__(192, 1) k_gemm_tn_tc(const __grid_constant__ G
                     const uint64_t b_hi = tc::umma_desc(sb + k16 * 2048, Cfg::BOX, 1024);
                     uint32_t accum = (cg > 0 || k16 > 0) ? 1u : 0u;
                     if (APL == 2) { tc::umma(acc, tc::umma_desc(sa + Cfg::A_PLANE + k16 * 2048, Cfg::BOX, 1024), b_hi, idesc, accum); accum = 1u; }
-                    if (BPL == 2) { tc::umma(acc, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
+                    if (BPL == 3) { tc::umma(acc, a_hi, tc::umma_desc(sb + 2 * Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
+                    if (BPL >= 2) { tc::umma(acc, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
                     tc::umma(acc, a_hi, b_hi, idesc, accum);
                 }
                 tc::umma_commit(&bars[STAGES + s]);  // frees the stage when these MMAs are done
@@ -243,6 +259,36 @@ __global__ void __launch_bounds__(192, 1) k_gemm_tn_tc(const __grid_constant__ G
         const int Mrows = second ? g.M2 : g.M;
         float* part = second ? g.part2 + (size_t)split * g.stride2 : g.part + (size_t)split * g.stride + g.off;
         bool got = true;
+        if constexpr (Cfg::X3) {  // warps 2-9: column half (wid - 2) / 4 of the tile, sums in registers, one store at the end
+            constexpr int COLS = BN / 2;
+            const int half = (wid - 2) >> 2;
+            float sum[COLS];
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) sum[j] = 0.f;  // an empty K range contributes zeros
+            for (int grp = 0; grp < ngroups && got; ++grp) {
+                got = tc::mbar_wait(&accfull[grp & 1], (grp >> 1) & 1);
+                tc::tc_fence_after();
+                __syncwarp();
+                const uint32_t acc = tmem + (uint32_t)((grp & 1) * BN + half * COLS) + ((uint32_t)(32 * q) << 16);
+                if (got) {
+#pragma unroll
+                    for (int c0 = 0; c0 < COLS; c0 += 32) {
+                        uint32_t r[32];
+                        tc::tmem_ld32(acc + (uint32_t)c0, r);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) sum[c0 + j] += __uint_as_float(r[j]);
+                    }
+                }
+                tc::tc_fence_before();
+                if (grp + 2 < ngroups) tc::mbar_arrive(&accempty[grp & 1]);  // hand the accumulator back to the issuer
+            }
+            if (m < Mrows) {
+                float4* dst = reinterpret_cast<float4*>(part + (size_t)m * g.ldc + n0 + half * COLS);
+#pragma unroll
+                for (int j = 0; j < COLS / 4; ++j)
+                    if (n0 + half * COLS + 4 * j < g.N) dst[j] = make_float4(sum[4 * j], sum[4 * j + 1], sum[4 * j + 2], sum[4 * j + 3]);
+            }
+        } else
         for (int grp = 0; grp < (ngroups > 0 ? ngroups : 1); ++grp) {
             if (ngroups > 0 && got) got = tc::mbar_wait(&accfull[grp & 1], (grp >> 1) & 1);
             tc::tc_fence_after();
@@ -288,13 +334,17 @@ static cudaError_t launch_t(const GemmTnArgs& g, int splits, int* status, cudaSt
     using Cfg = GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>;
     GemmTcMaps maps;
     memset(&maps, 0, sizeof(maps));
-    const bool bf = PREC == 1;
+    const bool bf = PREC >= 1;
+    // (every term is a matrix of its own: rows past K read as zeros)
+    auto map = [&](CUtensorMap* m, const __nv_bfloat16* p, int ld) { return make_tensor_map_2d(m, p, (uint64_t)g.K, (uint64_t)ld, 64, bf); };
     if (AMODE == A_PLANES) {
-        if (!make_tensor_map_2d(&maps.a_hi, g.Ahi, (uint64_t)g.K, (uint64_t)g.lda, 64, bf)) return cudaErrorNotSupported;
-        if (APL == 2 && !make_tensor_map_2d(&maps.a_lo, g.Alo, (uint64_t)g.K, (uint64_t)g.lda, 64, bf)) return cudaErrorNotSupported;
+        if (!map(&maps.a_hi, g.Ahi, g.lda)) return cudaErrorNotSupported;
+        if (APL >= 2 && !map(&maps.a_lo, g.Alo, g.lda)) return cudaErrorNotSupported;
+        if (APL == 3 && !map(&maps.a_lo2, g.Alo + (g.Alo - g.Ahi), g.lda)) return cudaErrorNotSupported;
     }
-    if (!make_tensor_map_2d(&maps.b_hi, g.Bhi, (uint64_t)g.K, (uint64_t)g.ldb, 64, bf)) return cudaErrorNotSupported;
-    if (BPL == 2 && !make_tensor_map_2d(&maps.b_lo, g.Blo, (uint64_t)g.K, (uint64_t)g.ldb, 64, bf)) return cudaErrorNotSupported;
+    if (!map(&maps.b_hi, g.Bhi, g.ldb)) return cudaErrorNotSupported;
+    if (BPL >= 2 && !map(&maps.b_lo, g.Blo, g.ldb)) return cudaErrorNotSupported;
+    if (BPL == 3 && !map(&maps.b_lo2, g.Blo + (g.Blo - g.Bhi), g.ldb)) return cudaErrorNotSupported;
     cudaError_t e = cudaFuncSetAttribute(k_gemm_tn_tc<BN, AMODE, APL, BPL, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
     if (e != cudaSuccess) return e;
     dim3 grid(AMODE == A_ENV ? 2 : (g.M + Cfg::BM - 1) / Cfg::BM, (g.N + BN - 1) / BN, splits);
@@ -304,28 +354,37 @@ static cudaError_t launch_t(const GemmTnArgs& g, int splits, int* status, cudaSt
 
 template <int BN, int PREC>
 static cudaError_t launch_bn(const GemmTnArgs& g, int amode, int bpl, int splits, int* status, cudaStream_t s) {
-    constexpr int PL = PREC == 1 ? 1 : 2;
-    if (PREC == 1 && bpl == 2) {  // bf16 workload with a two-term B (the sum over t of dh1): synthesized A only
-        if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, 2, PREC>(g, splits, status, s);
-        if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, 2, PREC>(g, splits, status, s);
+    if constexpr (PREC == 2) {  // fp32 as three bf16 terms (plane operands: 128-column tiles, two stages of 96 KB)
+        if (amode == A_PLANES) return launch_t<128, A_PLANES, 3, 3, PREC>(g, splits, status, s);
+        if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, 3, PREC>(g, splits, status, s);
+        if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, 3, PREC>(g, splits, status, s);
+        if (amode == A_ENV && g.M <= 128 && g.M2 <= 128) return launch_t<BN, A_ENV, 1, 3, PREC>(g, splits, status, s);
+        return cudaErrorNotSupported;
+    } else {
+        constexpr int PL = PREC == 1 ? 1 : 2;
+        if (PREC == 1 && bpl == 2) {  // bf16 workload with a two-term B (the sum over t of dh1): synthesized A only
+            if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, 2, PREC>(g, splits, status, s);
+            if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, 2, PREC>(g, splits, status, s);
+            return cudaErrorNotSupported;
+        }
+        if (amode == A_PLANES) return launch_t<BN, A_PLANES, PL, PL, PREC>(g, splits, status, s);
+        if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, PL, PREC>(g, splits, status, s);
+        if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, PL, PREC>(g, splits, status, s);
+        if (amode == A_ENV && g.M <= 128 && g.M2 <= 128) return launch_t<BN, A_ENV, 1, PL, PREC>(g, splits, status, s);
         return cudaErrorNotSupported;
     }
-    if (amode == A_PLANES) return launch_t<BN, A_PLANES, PL, PL, PREC>(g, splits, status, s);
-    if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, PL, PREC>(g, splits, status, s);
-    if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, PL, PREC>(g, splits, status, s);
-    if (amode == A_ENV && g.M <= 128 && g.M2 <= 128) return launch_t<BN, A_ENV, 1, PL, PREC>(g, splits, status, s);
-    return cudaErrorNotSupported;
 }
 
-// Covered: N = ldb = 64, 128, 256 or a multiple of 256 (column tiles of 256 on grid.y), klen a multiple of 64, A planes or one-hot A,
-// operand planes as the fp32 workloads (hi+lo fp16) or the bf16 workload (one plane) use them.
+// Covered: N = ldb = 64, 128, 256 or a multiple of 64 above (column tiles of 256 on grid.y), klen a multiple of 64, A planes or
+// one-hot A, operand planes as the fp32 workloads (hi+lo fp16; prec 2: three bf16 terms) or the bf16 workload (one plane) use them.
 cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int apl, int bpl, int prec, int splits, int* status, cudaStream_t s) {
-    const int pl = prec == 1 ? 1 : 2;
-    if (g.N != g.ldb || g.klen % 64 != 0 || (bpl != pl && !(prec == 1 && bpl == 2 && amode != A_PLANES)) ||
+    const int pl = prec == 1 ? 1 : prec == 2 ? 3 : 2;
+    if (g.N != g.ldb || g.N % 64 != 0 || g.klen % 64 != 0 || (bpl != pl && !(prec == 1 && bpl == 2 && amode != A_PLANES)) ||
         (amode == A_PLANES && (apl != pl || g.lda % 64 != 0)))
         return cudaErrorNotSupported;
     if (amode != A_PLANES && apl != 1) return cudaErrorNotSupported;
-    const int bn = g.N > 256 && g.N % 256 == 0 ? 256 : g.N;
+    const int bn = g.N > 256 ? 256 : g.N;
+    if (prec == 2) return bn == 256 ? launch_bn<256, 2>(g, amode, bpl, splits, status, s) : cudaErrorNotSupported;
     if (prec == 1) {
         switch (bn) {
             case 64: return launch_bn<64, 1>(g, amode, bpl, splits, status, s);

@@ -391,8 +391,14 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
                 a_wh[cc][3] = fmaf(hv[cc], d0s[0][3], a_wh[cc][3]);
                 a_wh[cc][4] = fmaf(hv[cc], d0s[0][4], a_wh[cc][4]);
             }
-            uint32_t phi, plo;
-            split2<PREC>(dh[0], dh[1], phi, plo);
+            uint32_t phi, plo, pl2 = 0u;
+            if constexpr (PREC == 2) {
+                uint32_t tm[3];
+                split3(dh[0], dh[1], tm);
+                phi = tm[0]; plo = tm[1]; pl2 = tm[2];
+            } else {
+                split2<PREC>(dh[0], dh[1], phi, plo);
+            }
             if (PREC == 1) {  // the bf16 workload rounds dh2: the sums take the rounded values
                 dh[0] = __uint_as_float(phi << 16);
                 dh[1] = __uint_as_float(phi & 0xFFFF0000u);
@@ -401,7 +407,8 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
             a_b2[1] += dh[1];
             if (fullt || r < rows_left) {
                 o_hi[r * (H / 2)] = phi;
-                if (PREC == 0) o_lo[r * (H / 2)] = plo;
+                if (PREC != 1) o_lo[r * (H / 2)] = plo;
+                if (PREC == 2) o_lo[RH / 2 + r * (H / 2)] = pl2;
             }
             if (FUSE) {
                 // element (k = tile row, n = unit 2 cp) of the MN-major tile: box n/64, byte k*128 + (((n%64)/8) ^ (k%8))*16 +
@@ -1049,8 +1056,16 @@ __device__ __forceinline__ void adam_step(const LearnArgs& a, size_t i, float g,
     if (b.w2p_hi && i >= d.oW2 && i < d.ob2) {
         const int H = d.H;
         const int k = (int)((i - d.oW2) / H), n = (int)((i - d.oW2) % H);
+        if (PREC == 2) {
+            uint32_t tm[3];
+            split3(thc, 0.f, tm);
+            const size_t n2 = (size_t)H * H;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) b.w2p_hi[p * n2 + (i - d.oW2)] = (uint16_t)tm[p];
+            return;
+        }
         uint16_t hi, lo;
-        split1<PREC>(thc, hi, lo);
+        split1<PREC == 1 ? 1 : 0>(thc, hi, lo);
         if (b.w2f_hi) {
             const size_t ef = ((size_t)((k >> 4) * (H / 8) + (n >> 3)) * 32 + (n & 7) * 4 + ((k & 7) >> 1)) * 4 + ((k & 15) >> 3) * 2 + (k & 1);
             reinterpret_cast<uint16_t*>(b.w2f_hi)[ef] = hi;
@@ -1260,13 +1275,15 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     const int tiles_ch = ((C + 1 + bt - 1) / bt) * ((H + bt - 1) / bt);
     int tiles_agent = tiles_ch;
     if (H > 256) {  // wide path: 128 x 256 output tiles in the tcgen05 GEMMs
-        tiles_hh = (H / 128) * (H / 256);
-        tiles_agent = ((C + 127) / 128) * (H / 256);
+        tiles_hh = (H / 128) * ((H + 255) / 256);
+        tiles_agent = ((C + 127) / 128) * ((H + 255) / 256);
     }
     p->ns_w2 = splits_for((int)R, tiles_hh, 256);
     p->ns_agent = splits_for((int)R, tiles_agent, 256);
     if (H > 256) {  // the bf16 GEMM CTAs of the wide path take a whole SM each (four 48 KB stages): one wave
         p->ns_w2 = 148 / tiles_hh > 0 ? 148 / tiles_hh : 1;
+        const int ap = agent_plane_splits(d);
+        if (ap > p->ns_agent) p->ns_agent = ap;
     }
     if (dh1_agent_tc_supported(d)) {  // the fused kernel writes one agent-plane partial per (CTA row, t slice)
         int gx, ts;
@@ -1275,7 +1292,7 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     }
     p->ns_env = splits_for(d.B, tiles_ch, 128);
     const size_t tiles32 = (R + 31) / 32;
-    size_t hg = H == 256 ? HEADS_GRID / 2 : HEADS_GRID;  // (the H = 256 kernel takes a whole SM)
+    size_t hg = H >= 256 ? HEADS_GRID / 2 : HEADS_GRID;  // (the kernels for H >= 256 take a whole SM, or walk several column slabs)
     if (d.npol > 1) hg = (size_t)(2 * HEADS_GRID / d.npol > 0 ? 2 * HEADS_GRID / d.npol : 1);  // many policies: the CTAs of all policies fill the GPU together
     p->heads_grid = (int)(tiles32 < hg ? tiles32 : hg);
     // (the fused heads + dW2 kernel writes one dW2 partial per CTA: room for the larger of the two partial counts)
@@ -1307,7 +1324,7 @@ static cudaError_t launch_heads_t(const LearnArgs& a, int grid, cudaStream_t s, 
         }
         return cudaErrorNotSupported;
     }
-    if constexpr ((H == 128 || H == 256) && HS == H && !H2BF) {
+    if constexpr ((H == 128 || H == 256) && HS == H && !H2BF && PREC != 2) {
         if (fuse) {  // also dW2 = h1^T dh2 for the CTA's rows (tcgen05; the h1 tiles by TMA)
             using FCfg = HeadsCfg<H, NW, PREC, HS, H2BF, true>;
             const size_t R = (size_t)a.d.B * a.T, RH = (size_t)a.d.B * a.d.Tmax * H;
@@ -1350,6 +1367,8 @@ static cudaError_t launch_dh1_t(const LearnArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+template <int V> using ic = std::integral_constant<int, V>;
+
 template <int PREC>
 static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const Dims& d = a.d;
@@ -1363,6 +1382,10 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const bool grouped = d.npol > 1;
     LearnPlan pl;
     learn_mma_plan(d, &pl);
+    if (PREC == 2 && wide) {  // 128 x 128 tiles: one wave of CTAs
+        const int one_wave = 148 / ((H / 128) * (H / 128));
+        pl.ns_w2 = one_wave < 1 ? 1 : one_wave < pl.ns_w2 ? one_wave : pl.ns_w2;
+    }
     a.part_small = b.part + pl.off_small;
     a.small_stride = pl.small_stride;
     // parameter regions in flat order: W1 walls | W1 agent | W1 goal | b1 | W2 | b2 | Wh | bh
@@ -1382,16 +1405,23 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     {
         Scope sc(c, K_HEADS_BWD);
         switch (H) {
-            case 64: CK((launch_heads_t<64, 4, PREC>(a, pl.heads_grid, s))); break;
-            case 128: CK((launch_heads_t<128, 8, PREC>(a, pl.heads_grid, s, fuse_dw2))); break;
-            case 256: CK((launch_heads_t<256, 16, PREC>(a, pl.heads_grid, s, fuse_dw2))); break;
+            case 64: if constexpr (PREC != 2) { CK((launch_heads_t<64, 4, PREC>(a, pl.heads_grid, s))); break; }
+            case 128: if constexpr (PREC != 2) { CK((launch_heads_t<128, 8, PREC>(a, pl.heads_grid, s, fuse_dw2))); break; }
+            case 256: if constexpr (PREC != 2) { CK((launch_heads_t<256, 16, PREC>(a, pl.heads_grid, s, fuse_dw2))); break; }
             default:
+                if constexpr (PREC == 2) {  // wide fp32: column slabs; the row warp of each slab takes the softmax again
+                    if (H == 384) { CK((launch_heads_t<384, 8, 2, 128>(a, pl.heads_grid, s))); break; }
+                    if (H == 512) { CK((launch_heads_t<512, 16, 2, 256>(a, pl.heads_grid, s))); break; }
+                    if (H == 768) { CK((launch_heads_t<768, 16, 2, 256>(a, pl.heads_grid, s))); break; }
+                    if (H == 1024) { CK((launch_heads_t<1024, 16, 2, 256>(a, pl.heads_grid, s))); break; }
+                }
                 if constexpr (PREC == 1) {
+                    if (H == 384) { CK((launch_heads_t<384, 8, 1, 128, true>(a, pl.heads_grid, s))); break; }  // (no whole 256-column slabs)
                     if (wide) {  // tensor-pipe version: one partial slot per CTA (slot 4 * CTA of the small region)
                         for (int q = 5; q <= 7; ++q) { a.reg[q].ns = pl.heads_grid; a.reg[q].stride = 4 * pl.small_stride; }
                         if (H == 512) { CK((launch_heads_tc_t<512>(a, pl.heads_grid, s))); break; }
                         if (H == 1024) { CK((launch_heads_tc_t<1024>(a, pl.heads_grid, s))); break; }
-                        if (H == 2048) { CK((launch_heads_tc_t<2048>(a, pl.heads_grid, s))); break; }
+                        if (H == 768) { CK((launch_heads_tc_t<768>(a, pl.heads_grid, s))); break; }
                     }
                 }
                 return cudaErrorNotSupported;
@@ -1426,12 +1456,18 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     if (fused_agent) {
     } else if (wide) {
         CK(launch_dh1_wide(a, c));
+        if (PREC == 2) {
+            a.reg[1].ns = agent_plane_splits(d);
+            CK(launch_agent_plane(a, a.reg[1].ns, b.part + pl.off_agent, CH, c));
+            fused_agent = true;
+        }
     } else {
         Scope sc(c, K_DH1);
         const cudaError_t etc = grouped ? cudaErrorNotSupported : launch_dh1_tc(a, PREC, s);  // tcgen05 where covered, else the mma.sync kernel
         if (etc != cudaErrorNotSupported) CK(etc);
         else a.ts = 1;
-        if (etc == cudaErrorNotSupported) switch (H) {
+        if constexpr (PREC == 2) return cudaErrorNotSupported;
+        else if (etc == cudaErrorNotSupported) switch (H) {
             case 64: CK((launch_dh1_t<64, 64, PREC>(a, s))); break;
             case 128: CK((launch_dh1_t<128, 128, PREC>(a, s))); break;
             case 256: CK((launch_dh1_t<256, 128, PREC>(a, s))); break;
@@ -1442,14 +1478,25 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const __nv_bfloat16* dh2hi = reinterpret_cast<const __nv_bfloat16*>(b.dh2);
     const __nv_bfloat16* dh1hi = reinterpret_cast<const __nv_bfloat16*>(b.dh1);
     const __nv_bfloat16* Shi = reinterpret_cast<const __nv_bfloat16*>(b.S);
-    constexpr int PL = PREC == 1 ? 1 : 2;
+    constexpr int PL = PREC == 1 ? 1 : PREC == 2 ? 3 : 2, SPL = PREC == 2 ? 3 : 2;  // planes of an operand, of S
     auto klen_of = [](int K, int ns) { return ((K + ns - 1) / ns + 63) / 64 * 64; };
     GemmTnArgs g;
     memset(&g, 0, sizeof(g));
     const size_t RH_last = (size_t)d.B_last * d.Tmax * H;  // plane offset inside the last policy's (more compact) buffers
     if (grouped) { g.npol = d.npol; g.pstride = d.pstride; }
-    auto tc_gemm = [&](int amode, int apl, int bpl, int splits) {
-        return grouped ? cudaErrorNotSupported : launch_gemm_tn_tc(g, amode, apl, bpl, PREC, splits, b.status, s);
+    // tcgen05 where covered, else the warp-level kernel
+    auto tn_gemm = [&](auto amode_c, auto apl_c, auto bpl_c, int rows_m, int splits) -> cudaError_t {
+        constexpr int amode = decltype(amode_c)::value, apl = decltype(apl_c)::value, bpl = decltype(bpl_c)::value;
+        if (!grouped) {
+            const cudaError_t e = launch_gemm_tn_tc(g, amode, apl, bpl, PREC, splits, b.status, s);
+            if (e != cudaErrorNotSupported) return e;
+        }
+        if constexpr (PREC == 2 || amode == A_ENV) {
+            return cudaErrorNotSupported;
+        } else {
+            if (H >= 128) return launch_gemm_tn<128, 128, amode, apl, bpl, PREC>(g, rows_m, splits, s);
+            return launch_gemm_tn<64, 64, amode, apl, bpl, PREC>(g, rows_m, splits, s);
+        }
     };
     // dW2 = h1^T dh2
     g.M = H; g.N = H; g.K = (int)R; g.klen = klen_of(g.K, pl.ns_w2);
@@ -1457,14 +1504,10 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     g.Bhi = dh2hi; g.Blo = dh2hi + RH; g.ldb = H;
     g.part = b.part + pl.off_w2; g.stride = (size_t)H * H; g.off = 0; g.ldc = H; g.ones_row = -1;
     g.K_last = d.B_last * T; g.kmod_last = 0; g.alo_off_last = g.blo_off_last = RH_last;
+    if (wide && PREC == 2) g.Alo = h1hi + wide_h1_rows(d) * H;
     if (!fuse_dw2) {
         Scope sc(c, K_DW2);
-        cudaError_t e = tc_gemm(A_PLANES, PL, PL, pl.ns_w2);  // tcgen05 where covered
-        if (e == cudaErrorNotSupported) {
-            if (H >= 128) e = launch_gemm_tn<128, 128, A_PLANES, PL, PL, PREC>(g, H, pl.ns_w2, s);
-            else e = launch_gemm_tn<64, 64, A_PLANES, PL, PL, PREC>(g, H, pl.ns_w2, s);
-        }
-        CK(e);
+        CK(tn_gemm(ic<A_PLANES>{}, ic<PL>{}, ic<PL>{}, H, pl.ns_w2));
     }
     // dW1, agent plane = onehot(pos)^T dh1
     g.M = C; g.K = (int)R; g.klen = klen_of(g.K, pl.ns_agent);
@@ -1473,12 +1516,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     g.part = b.part + pl.off_agent; g.stride = CH; g.off = 0;
     if (!fused_agent) {
         Scope sc(c, K_DW1_AGENT);
-        cudaError_t e = tc_gemm(A_ONEHOT, 1, PL, pl.ns_agent);
-        if (e == cudaErrorNotSupported) {
-            if (H >= 128) e = launch_gemm_tn<128, 128, A_ONEHOT, 1, PL, PREC>(g, C, pl.ns_agent, s);
-            else e = launch_gemm_tn<64, 64, A_ONEHOT, 1, PL, PREC>(g, C, pl.ns_agent, s);
-        }
-        CK(e);
+        CK(tn_gemm(ic<A_ONEHOT>{}, ic<1>{}, ic<PL>{}, C, pl.ns_agent));
     }
     // dW1, wall plane (+ db1 through the all-ones row) = walls^T S; goal plane = onehot(goal)^T S
     g.K = a.ts * B; g.kmod = B; g.klen = klen_of(g.K, pl.ns_env);
@@ -1487,34 +1525,22 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     g.walls = b.walls; g.W = d.W; g.ones_row = C; g.M = C + 1;
     g.part = b.part + pl.off_walls; g.stride = (size_t)(C + 1) * H; g.off = 0; g.off_ones = CH;
     bool env_planes_done = false;
-    if (PREC == 0) {  // both planes in one launch: row tile 0 = wall bits + ones row, row tile 1 = one-hot of the goal cell
+    if (PREC != 1) {  // both planes in one launch: row tile 0 = wall bits + ones row, row tile 1 = one-hot of the goal cell
         g.idx2 = b.goal; g.M2 = C; g.part2 = b.part + pl.off_goal; g.stride2 = CH;
         Scope sc(c, K_DW1_WALLS);
-        const cudaError_t e = tc_gemm(A_ENV, 1, 2, pl.ns_env);
+        const cudaError_t e = tn_gemm(ic<A_ENV>{}, ic<1>{}, ic<SPL>{}, C + 1, pl.ns_env);
         if (e == cudaSuccess) env_planes_done = true;
         else if (e != cudaErrorNotSupported) return e;
     }
     if (!env_planes_done) {
         {
             Scope sc(c, K_DW1_WALLS);
-            cudaError_t e = tc_gemm(A_WALLS, 1, 2, pl.ns_env);
-            if (e == cudaErrorNotSupported) {
-                if (H >= 128) e = launch_gemm_tn<128, 128, A_WALLS, 1, 2, PREC>(g, C + 1, pl.ns_env, s);
-                else e = launch_gemm_tn<64, 64, A_WALLS, 1, 2, PREC>(g, C + 1, pl.ns_env, s);
-            }
-            CK(e);
+            CK(tn_gemm(ic<A_WALLS>{}, ic<1>{}, ic<SPL>{}, C + 1, pl.ns_env));
         }
         g.M = C; g.ones_row = -1; g.idx = b.goal;
         g.part = b.part + pl.off_goal; g.stride = CH;
-        {
-            Scope sc(c, K_DW1_GOAL);
-            cudaError_t e = tc_gemm(A_ONEHOT, 1, 2, pl.ns_env);
-            if (e == cudaErrorNotSupported) {
-                if (H >= 128) e = launch_gemm_tn<128, 128, A_ONEHOT, 1, 2, PREC>(g, C, pl.ns_env, s);
-                else e = launch_gemm_tn<64, 64, A_ONEHOT, 1, 2, PREC>(g, C, pl.ns_env, s);
-            }
-            CK(e);
-        }
+        Scope sc(c, K_DW1_GOAL);
+        CK(tn_gemm(ic<A_ONEHOT>{}, ic<1>{}, ic<SPL>{}, C, pl.ns_env));
     }
     {
         Scope sc(c, K_REDUCE_ADAM);
@@ -1531,7 +1557,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     if (b.dbg_gates) {
         Scope sc(c, K_PACK_GATES);
         if (d.npol > 1) k_pack_gates2<true><<<dim3(64, d.npol), 256, 0, s>>>(DimsBuffers{d, b}, R, 0);
-        else k_pack_gates2<false><<<148 * 8, 256, 0, s>>>(DimsBuffers{d, b}, R, wide ? 1 : 0);
+        else k_pack_gates2<false><<<148 * 8, 256, 0, s>>>(DimsBuffers{d, b}, R, wide && PREC == 1 ? 1 : 0);
         CK(cudaGetLastError());
     }
     return cudaSuccess;
@@ -1544,12 +1570,14 @@ cudaError_t launch_adam_only(const LearnArgs& a, int prec, const Ctx& c) {
         if (prec == 1) return cudaErrorNotSupported;
         k_adam_only<0, true><<<dim3(nb, a.d.npol), 256, 0, c.s>>>(a);
     } else if (prec == 1) k_adam_only<1, false><<<nb, 256, 0, c.s>>>(a);
+    else if (wide_supported(a.d.H, prec)) k_adam_only<2, false><<<nb, 256, 0, c.s>>>(a);
     else k_adam_only<0, false><<<nb, 256, 0, c.s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_learn_mma(const LearnArgs& a, int prec, const Ctx& c) {
-    return prec == 1 ? launch_learn_mma_p<1>(a, c) : launch_learn_mma_p<0>(a, c);
+    if (prec == 1) return launch_learn_mma_p<1>(a, c);
+    return wide_supported(a.d.H, prec) ? launch_learn_mma_p<2>(a, c) : launch_learn_mma_p<0>(a, c);
 }
 
 }  // namespace anakin

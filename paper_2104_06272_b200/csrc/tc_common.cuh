@@ -85,7 +85,7 @@ __device__ __forceinline__ uint64_t umma_desc(const void* smem_ptr, uint32_t lbo
 // bit 15 / 16 = A / B is MN-major, bits 17-22 = N >> 3, bits 24-28 = M >> 4.
 template <int PREC>
 __device__ __forceinline__ uint32_t umma_idesc(int M, int N, bool a_mn_major, bool b_mn_major) {
-    const uint32_t fmt = PREC == 1 ? 1u : 0u;
+    const uint32_t fmt = PREC >= 1 ? 1u : 0u;
     return (1u << 4) | (fmt << 7) | (fmt << 10) | ((a_mn_major ? 1u : 0u) << 15) | ((b_mn_major ? 1u : 0u) << 16) |
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
@@ -229,6 +229,12 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint16_t cta_mas
                  "h"(cta_mask)
                  : "memory");
 }
+
+// PREC 2: the (A term, B term) pairs of an fp32 product, smallest first, so that the accumulator is small while the small
+// terms go in and the leading products are rounded only once per k16 step.
+constexpr int X3_PAIRS = 6;
+__host__ __device__ constexpr int x3_a(int i) { return i == 0 ? 2 : i == 2 ? 1 : i == 3 ? 1 : 0; }
+__host__ __device__ constexpr int x3_b(int i) { return i == 1 ? 2 : i == 2 ? 1 : i == 4 ? 1 : 0; }
 
 }  // namespace tc
 

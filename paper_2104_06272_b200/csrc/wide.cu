@@ -22,22 +22,24 @@
 
 namespace anakin {
 
-bool wide_supported(int H, int prec) { return prec == 1 && (H == 512 || H == 1024 || H == 2048); }
+// Hidden layers too wide for the persistent rollouts, in either precision (bf16 at 512 / 1024 is the headline form).
+bool wide_supported(int H, int prec) { (void)prec; return H == 384 || H == 512 || H == 768 || H == 1024; }
 bool tensor_path_supported(int H, int prec) { return rollout_mma_supported(H) || wide_supported(H, prec); }
 
 namespace {
 
 using namespace widegemm;
 
+template <int BN_>
 struct NtCfg {
-    static constexpr int BM = 128, BN = NT_BN, KC = 64, STAGES = 3, THREADS = 320, MAXN = NT_MAXN;
+    static constexpr int BM = 128, BN = BN_, KC = 64, STAGES = BN == 256 ? 3 : BN == 128 ? 5 : 6, THREADS = 320, MAXN = NT_MAXN;
     static constexpr int A_BYTES = BM * KC * 2, B_BYTES = BN * KC * 2, STAGE = A_BYTES + B_BYTES;
     static constexpr size_t smem_bytes = (size_t)STAGES * STAGE + 1024 /*alignment slack*/ + 256 /*barriers, tmem slot*/ + MAXN * 4 + NT_EPI_WARPS * NT_STAGE_BYTES;
 };
 
-template <int EPI, bool B_MN>
+template <int EPI, bool B_MN, int BN_>
 __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ NtMaps maps, NtArgs g) {
-    using Cfg = NtCfg;
+    using Cfg = NtCfg<BN_>;
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);  // the swizzle needs 1024-byte alignment
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
     float* s_bias = (float*)(base + STAGES * Cfg::STAGE + 256);
     unsigned char* s_stage = (unsigned char*)(s_bias + NT_MAXN);  // [NT_EPI_WARPS][NT_STAGE_BYTES]
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
-    const int nt = g.N / BN, mt = (g.M + BM - 1) / BM, ntiles = mt * nt, nch = g.K / KC;
+    const int nt = (g.N + BN - 1) / BN, mt = (g.M + BM - 1) / BM, ntiles = mt * nt, nch = g.K / KC;
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); }
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
     }
     if (EPI != EPI_GATE)
         for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
-    if (wid == 2) tc::tmem_alloc(tmem_slot, 512);
+    if (wid == 2) tc::tmem_alloc(tmem_slot, 2 * BN);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
@@ -84,8 +86,8 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
 #pragma unroll
                         for (int bx = 0; bx < BN / 64; ++bx) tc::tma_load_2d(sb + bx * 8192, &maps.b, &full[s], n0 + 64 * bx, kc * KC);
                     } else {
-                        tc::tma_load_2d(sb, &maps.b, &full[s], kc * KC, n0);  // two boxes of 128 rows (n)
-                        tc::tma_load_2d(sb + Cfg::B_BYTES / 2, &maps.b, &full[s], kc * KC, n0 + BN / 2);
+#pragma unroll
+                        for (int bx = 0; bx < BN; bx += 128) tc::tma_load_2d(sb + bx * 128, &maps.b, &full[s], kc * KC, n0 + bx);  // boxes of 128 rows (n), 64 for a 64-wide tile
                     }
                 }
             }
@@ -131,12 +133,13 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
             const int m = m0 + 32 * q + lane;
             const bool valid = m < g.M;
             const size_t gi = ((size_t)g.row0 + (valid ? m : 0)) * g.N + n0;
-            if (EPI == EPI_GATE && valid) nt_prefetch_gate(g, gi);  // towards L2 while the MMAs run
+            if (EPI == EPI_GATE && valid) nt_prefetch_gate(g, gi, g.N - n0 < BN ? g.N - n0 : BN);  // towards L2 while the MMAs run
             ok = tc::mbar_wait(&tfull[buf], (u >> 1) & 1);
             if (!ok) break;
             tc::tc_fence_after();
+            constexpr int HW = BN >= 128 ? BN / 2 : 64;  // two column halves; the epilogue takes 64 columns at a time, so a 64-wide tile is one half's
             nt_epilogue_warp<EPI>(g, s_bias, s_stage + (wid - 2) * NT_STAGE_BYTES, tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN), m - lane, n0, lane,
-                                  half * (BN / 2), (half + 1) * (BN / 2));
+                                  half * HW, (half + 1) * HW < BN ? (half + 1) * HW : BN);
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&tempty[buf]);  // the issuer may overwrite this accumulator now
@@ -145,29 +148,66 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
     }
     tc::tc_fence_before();
     __syncthreads();
-    if (wid == 2) tc::tmem_dealloc(tmem, 512);
+    if (wid == 2) tc::tmem_dealloc(tmem, 2 * BN);
 }
 
-template <int EPI, bool B_MN>
-cudaError_t launch_nt(const NtMaps& maps, const NtArgs& g, cudaStream_t s) {
-    if (g.N % NtCfg::BN != 0 || g.K % NtCfg::KC != 0 || g.N > NtCfg::MAXN || g.M < 1) return cudaErrorNotSupported;
-    if (g.M >= 2 * NtCfg::BM) {  // the CTA-pair kernel (256 x 256 tiles) where there are rows for it
-        const cudaError_t ep = launch_nt_pair(EPI, B_MN, maps, g, s);
-        if (ep != cudaErrorNotSupported) return ep;
-    }
-    const cudaError_t e = cudaFuncSetAttribute(k_gemm_nt_tc<EPI, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NtCfg::smem_bytes);
+template <int EPI, bool B_MN, int BN>
+cudaError_t launch_nt_t(const NtMaps& maps, const NtArgs& g, int ntiles, cudaStream_t s) {
+    using Cfg = NtCfg<BN>;
+    const cudaError_t e = cudaFuncSetAttribute(k_gemm_nt_tc<EPI, B_MN, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
     if (e != cudaSuccess) return e;
-    const int ntiles = ((g.M + NtCfg::BM - 1) / NtCfg::BM) * (g.N / NtCfg::BN);
-    const int grid = ntiles < 148 ? ntiles : 148;
-    k_gemm_nt_tc<EPI, B_MN><<<grid, NtCfg::THREADS, NtCfg::smem_bytes, s>>>(maps, g);
+    k_gemm_nt_tc<EPI, B_MN, BN><<<ntiles < 148 ? ntiles : 148, Cfg::THREADS, Cfg::smem_bytes, s>>>(maps, g);
     return cudaGetLastError();
 }
 
+// B: MN-major [K][N] (boxes of 64 x 64) or K-major [N][K].  The CTA-pair kernel (256 x 256 tiles) halves the operand traffic and takes
+// every launch that gives its 74 pairs work; with fewer tiles than half of that, smaller tiles on more SMs are quicker.
+template <int EPI, bool B_MN>
+cudaError_t launch_nt(const void* A, size_t a_rows, const void* B, const NtArgs& g, cudaStream_t s) {
+    if (g.N % 64 != 0 || g.K % 64 != 0 || g.N > NT_MAXN || g.M < 1) return cudaErrorNotSupported;
+    auto tiles = [&](int bm, int bn) { return ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn); };
+    const int np = tiles(256, 256), n128 = tiles(128, 128), n64 = tiles(128, 64);
+    const int bn = EPI == EPI_BASE || np > 37 ? 256 : n64 <= 148 ? 64 : 128;
+    NtMaps maps;
+    memset(&maps, 0, sizeof(maps));
+    if (!make_tensor_map_2d(&maps.a, A, a_rows, g.K, 128, true)) return cudaErrorNotSupported;
+    if (!make_tensor_map_2d(&maps.b, B, B_MN ? g.K : g.N, B_MN ? g.N : g.K, B_MN || bn == 64 ? 64 : 128, true)) return cudaErrorNotSupported;
+    if (bn == 256 && g.M >= 256) return launch_nt_pair(EPI, B_MN, maps, g, s);
+    if constexpr (EPI != EPI_BASE) {
+        if (bn == 64) return launch_nt_t<EPI, B_MN, 64>(maps, g, n64, s);
+        if (bn == 128) return launch_nt_t<EPI, B_MN, 128>(maps, g, n128, s);
+    }
+    return launch_nt_t<EPI, B_MN, 256>(maps, g, tiles(128, 256), s);
+}
+
+// Elements between the bf16 planes of h1 in the fp32 form: the recorded rows and the B rows of the bootstrap step.
+__host__ __device__ inline size_t h1_plane(const Dims& d) { return ((size_t)d.B * d.Tmax + d.B) * d.H; }
+
+// Eight consecutive hidden units of one row of h1 = relu(base + W1 row): bf16-rounded (one plane), or exact as three planes.
+template <bool F32>
+__device__ __forceinline__ void h1_store8(uint16_t* out, size_t plane, const float4& b0, const float4& b1, const float4& w0, const float4& w1) {
+    const float x[8] = {fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f),
+                        fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f)};
+    if (F32) {
+        uint32_t t[4][3];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) split3(x[2 * q], x[2 * q + 1], t[q]);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(out + p * plane) = make_uint4(t[0][p], t[1][p], t[2][p], t[3][p]);
+    } else {
+        uint32_t o[4], unused;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) split2<1>(x[2 * q], x[2 * q + 1], o[q], unused);
+        *reinterpret_cast<uint4*>(out) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
 // h1 rows: 8 hidden units per thread.  pos[i] is the agent cell of row i (env = i mod B).
+template <bool F32>
 __global__ void __launch_bounds__(256) k_h1_wide(Dims d, Buffers b, const uint8_t* pos, size_t rows, size_t row0) {
     const int H = d.H, H8 = H / 8;
     const float* W1a = b.theta_c + d.oW1 + (size_t)d.C * H;  // agent plane of W1
-    uint4* out = reinterpret_cast<uint4*>(b.h1) + row0 * H8;
+    uint16_t* out = reinterpret_cast<uint16_t*>(b.h1) + row0 * H;
     const size_t total = rows * H8;
     for (size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x; idx < total; idx += (size_t)gridDim.x * 256) {
         const size_t i = idx / H8;
@@ -176,25 +216,18 @@ __global__ void __launch_bounds__(256) k_h1_wide(Dims d, Buffers b, const uint8_
         const int p = min((int)pos[i], d.C - 1);  // a position handed in from outside stays inside the plane
         const float4* bp = reinterpret_cast<const float4*>(b.base + (size_t)env * H) + 2 * j8;
         const float4* wp = reinterpret_cast<const float4*>(W1a + (size_t)p * H) + 2 * j8;
-        const float4 b0 = bp[0], b1 = bp[1], w0 = __ldg(wp), w1 = __ldg(wp + 1);
-        uint4 o;
-        o.x = pack_bf16(__float2bfloat16_rn(fmaxf(b0.x + w0.x, 0.f)), __float2bfloat16_rn(fmaxf(b0.y + w0.y, 0.f)));
-        o.y = pack_bf16(__float2bfloat16_rn(fmaxf(b0.z + w0.z, 0.f)), __float2bfloat16_rn(fmaxf(b0.w + w0.w, 0.f)));
-        o.z = pack_bf16(__float2bfloat16_rn(fmaxf(b1.x + w1.x, 0.f)), __float2bfloat16_rn(fmaxf(b1.y + w1.y, 0.f)));
-        o.w = pack_bf16(__float2bfloat16_rn(fmaxf(b1.z + w1.z, 0.f)), __float2bfloat16_rn(fmaxf(b1.w + w1.w, 0.f)));
-        out[idx] = o;
+        h1_store8<F32>(out + idx * 8, h1_plane(d), bp[0], bp[1], __ldg(wp), __ldg(wp + 1));
     }
 }
 
-// Heads, sampling and env step for 32 rows per CTA: eight warps take four rows each for the head products, then warp 0
+// Heads, sampling and env step for RW = 32 or 8 rows per CTA (eight where 32 would leave SMs without a CTA: a step is a
+// dependent launch, so its latency counts): eight warps share the rows for the head products, then warp 0
 // takes one row per lane for the per-env part (its env state and wall words were requested at kernel start).
 //   mode 0: step t of the rollout (row = env): saves the head outputs and the value, samples, steps the env, records.
 //   mode 1: bootstrap forward after the last step: saves the value only.
 //   mode 2: replay of recorded rows (row = t*B + env): saves the head outputs only.
 //   mode 3: forward of the current env state under the current parameters: saves the value to vboot.
-constexpr int HW_ROWS = 32;
-
-template <int H>
+template <int H, bool F32, int HW_ROWS>
 __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mode, size_t rows, size_t row0) {
     constexpr int TRIPS = H / 128;   // a lane covers four consecutive hidden units per trip
     extern __shared__ __align__(16) float s_wh[];  // [H][5] as stored
@@ -227,12 +260,13 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
     }
     const uint16_t* h2b = reinterpret_cast<const uint16_t*>(b.h2);
     // a warp walks rows wid, wid+8, ...; the loads of the next row are in flight while this row is reduced
-    uint2 v[TRIPS], vn[TRIPS];
-    auto load_row = [&](int r, uint2 (&dst)[TRIPS]) {
-        const size_t i = i0 + r;
-        const uint2* hp = reinterpret_cast<const uint2*>(h2b + (row0 + (i < rows ? i : 0)) * H);
+    using H2x4 = typename std::conditional<F32, float4, uint2>::type;  // four consecutive units of h2: fp32, or bf16
+    H2x4 v[TRIPS], vn[TRIPS];
+    auto load_row = [&](int r, H2x4 (&dst)[TRIPS]) {
+        const size_t i = i0 + r, off = (row0 + (i < rows ? i : 0)) * H;
+        const H2x4* hp = F32 ? reinterpret_cast<const H2x4*>(b.h2 + off) : reinterpret_cast<const H2x4*>(h2b + off);
 #pragma unroll
-        for (int q = 0; q < TRIPS; ++q) dst[q] = (r < HW_ROWS && i < rows) ? __ldg(hp + lane + 32 * q) : make_uint2(0u, 0u);
+        for (int q = 0; q < TRIPS; ++q) dst[q] = (r < HW_ROWS && i < rows) ? __ldg(hp + lane + 32 * q) : H2x4{};
     };
     load_row(wid, v);
     __syncthreads();
@@ -242,8 +276,15 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
         float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int q = 0; q < TRIPS; ++q) {
-            const float x[4] = {__uint_as_float(v[q].x << 16), __uint_as_float(v[q].x & 0xFFFF0000u), __uint_as_float(v[q].y << 16),
-                                __uint_as_float(v[q].y & 0xFFFF0000u)};
+            float x[4];
+            if constexpr (F32) {
+                x[0] = v[q].x; x[1] = v[q].y; x[2] = v[q].z; x[3] = v[q].w;
+            } else {
+                x[0] = __uint_as_float(v[q].x << 16);
+                x[1] = __uint_as_float(v[q].x & 0xFFFF0000u);
+                x[2] = __uint_as_float(v[q].y << 16);
+                x[3] = __uint_as_float(v[q].y & 0xFFFF0000u);
+            }
             // this lane's four units are 20 consecutive floats of Wh (80-byte lane stride: conflict-free 16-byte reads)
             const float4* wp = reinterpret_cast<const float4*>(s_wh + 20 * (lane + 32 * q));
             float w[20];
@@ -270,9 +311,9 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
     }
     __syncthreads();
     __shared__ int s_pos[HW_ROWS];
-    if (tid < HW_ROWS) {
+    if (tid < 32) {  // (the whole warp: the counters below are folded over its lanes)
     const size_t i = i0 + tid;
-    const bool valid = i < rows;
+    const bool valid = tid < HW_ROWS && i < rows;
     unsigned long long n_ep = 0, n_goal = 0, n_steps = 0;
     int bad = 0;
     if (valid) {
@@ -320,25 +361,19 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
     }
     if (mode != 0) return;
     // ---- layer 1 of the NEXT step for this CTA's envs, from the positions just produced (rows (t+1)*B + env):
-    // 8 threads per env, 16-byte chunks interleaved so that a row's lanes read and write contiguous memory
+    // 256 / HW_ROWS threads per env, 16-byte chunks interleaved so that a row's lanes read and write contiguous memory
     __syncthreads();
     {
-        const int rl = tid >> 3, q = tid & 7;
+        constexpr int TPR = 256 / HW_ROWS;
+        const int rl = tid / TPR, q = tid % TPR;
         const size_t env = i0 + rl;
         if (env < rows) {
             const float4* bp = reinterpret_cast<const float4*>(b.base + env * H);
             const float4* wp = reinterpret_cast<const float4*>(b.theta_c + d.oW1 + ((size_t)d.C + s_pos[rl]) * H);
-            uint4* out = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(b.h1) + ((size_t)(t + 1) * d.B + env) * H);
+            uint16_t* out = reinterpret_cast<uint16_t*>(b.h1) + ((size_t)(t + 1) * d.B + env) * H;
 #pragma unroll 4
-            for (int ch = q; ch < H / 8; ch += 8) {
-                const float4 b0 = bp[2 * ch], b1 = bp[2 * ch + 1], w0 = __ldg(wp + 2 * ch), w1 = __ldg(wp + 2 * ch + 1);
-                uint4 o;
-                o.x = pack_bf16(__float2bfloat16_rn(fmaxf(b0.x + w0.x, 0.f)), __float2bfloat16_rn(fmaxf(b0.y + w0.y, 0.f)));
-                o.y = pack_bf16(__float2bfloat16_rn(fmaxf(b0.z + w0.z, 0.f)), __float2bfloat16_rn(fmaxf(b0.w + w0.w, 0.f)));
-                o.z = pack_bf16(__float2bfloat16_rn(fmaxf(b1.x + w1.x, 0.f)), __float2bfloat16_rn(fmaxf(b1.y + w1.y, 0.f)));
-                o.w = pack_bf16(__float2bfloat16_rn(fmaxf(b1.z + w1.z, 0.f)), __float2bfloat16_rn(fmaxf(b1.w + w1.w, 0.f)));
-                out[ch] = o;
-            }
+            for (int ch = q; ch < H / 8; ch += TPR)
+                h1_store8<F32>(out + 8 * ch, h1_plane(d), bp[2 * ch], bp[2 * ch + 1], __ldg(wp + 2 * ch), __ldg(wp + 2 * ch + 1));
         }
     }
 }
@@ -380,179 +415,213 @@ __global__ void __launch_bounds__(256) k_sum_t_wide(Dims d, Buffers b, int T) {
     S_lo[idx] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
-// W2 as a row-major bf16 plane (the values are bf16 already in this workload).
+// W2 as row-major bf16 planes: one (the values are bf16 already in the bf16 workload) or the three terms of fp32 weights.
+template <bool F32>
 __global__ void __launch_bounds__(256) k_pack_w2_wide(Dims d, Buffers b) {
-    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (i < (size_t)d.H * d.H) b.w2p_hi[i] = __bfloat16_as_ushort(__float2bfloat16_rn(b.theta_c[d.oW2 + i]));
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x, n = (size_t)d.H * d.H;
+    if (2 * i >= n) return;
+    const float2 w = reinterpret_cast<const float2*>(b.theta_c + d.oW2)[i];
+    uint32_t t[3];
+    split3(w.x, w.y, t);
+    for (int p = 0; p < (F32 ? 3 : 1); ++p) reinterpret_cast<uint32_t*>(b.w2p_hi + p * n)[i] = t[p];
 }
 
-// Operands of the base GEMM: X[env][c] = 1 where cell c of the env is a wall (bf16), and the wall plane of W1 as bf16
-// (exact: the weights are bf16 values in this workload).
-__global__ void __launch_bounds__(256) k_expand_walls(Dims d, Buffers b, uint16_t* X, uint16_t* W1w) {
-    const size_t nx = (size_t)d.B * (d.C / 8), nw = (size_t)d.C * d.H;
+// Operands of the base GEMM: X[env][c] = 1 where cell c of the env is a wall (bf16), and the wall plane of W1 as bf16 planes
+// (one where the weights are bf16 values, else three terms).  Columns / rows from C up to Cp, a multiple of 64, are zero.
+template <bool F32>
+__global__ void __launch_bounds__(256) k_expand_walls(Dims d, Buffers b, uint16_t* X, uint16_t* W1w, int Cp) {
+    const size_t nx = (size_t)d.B * (Cp / 8), nw = (size_t)Cp * d.H / 2, real = (size_t)d.C * d.H / 2;
     for (size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x; idx < nx + nw; idx += (size_t)gridDim.x * 256) {
         if (idx < nx) {
-            const size_t e = idx / (d.C / 8);
-            const int c8 = (int)(idx - e * (d.C / 8));
-            const uint32_t bits = (b.walls[e * d.W + (c8 >> 2)] >> ((c8 & 3) * 8)) & 0xFFu;
+            const size_t e = idx / (Cp / 8);
+            const int c8 = (int)(idx - e * (Cp / 8)), left = d.C - 8 * c8;  // cells of the board in this chunk
+            uint32_t bits = left > 0 ? (b.walls[e * d.W + (c8 >> 2)] >> ((c8 & 3) * 8)) & 0xFFu : 0u;
+            if (left < 8 && left > 0) bits &= (1u << left) - 1u;
             uint32_t o[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) o[q] = ((bits >> (2 * q)) & 1u ? 0x3F80u : 0u) | ((bits >> (2 * q + 1)) & 1u ? 0x3F800000u : 0u);
-            reinterpret_cast<uint4*>(X)[idx] = make_uint4(o[0], o[1], o[2], o[3]);
+            for (int p = 0; p < (F32 ? 3 : 1); ++p) reinterpret_cast<uint4*>(X)[(e * (F32 ? 3 : 1) + p) * (Cp / 8) + c8] = make_uint4(o[0], o[1], o[2], o[3]);
         } else {
             const size_t i = idx - nx;
-            W1w[i] = __bfloat16_as_ushort(__float2bfloat16_rn(b.theta_c[d.oW1 + i]));
+            const float2 w = i < real ? reinterpret_cast<const float2*>(b.theta_c + d.oW1)[i] : make_float2(0.f, 0.f);
+            uint32_t t[3];
+            split3(w.x, w.y, t);
+            for (int p = 0; p < (F32 ? 3 : 1); ++p) reinterpret_cast<uint32_t*>(W1w)[(F32 ? 2 - p : 0) * nw + i] = t[p];
         }
     }
 }
 
 #define CKW(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return e_; } while (0)
 
-cudaError_t heads_wide(const RolloutArgs& a, int t, int mode, size_t rows, size_t row0, cudaStream_t s) {
-    const size_t smem = (size_t)5 * a.d.H * sizeof(float);
-    const unsigned grid = (unsigned)((rows + HW_ROWS - 1) / HW_ROWS);
+template <int H, bool F32>
+cudaError_t heads_wide_t(const RolloutArgs& a, int t, int mode, size_t rows, size_t row0, cudaStream_t s) {
+    const size_t smem = (size_t)5 * H * sizeof(float);
+    if (rows < 148 * 2 * 32) k_heads_wide<H, F32, 8><<<(unsigned)((rows + 7) / 8), 256, smem, s>>>(a, t, mode, rows, row0);
+    else k_heads_wide<H, F32, 32><<<(unsigned)((rows + 31) / 32), 256, smem, s>>>(a, t, mode, rows, row0);
+    return cudaGetLastError();
+}
+cudaError_t heads_wide(const RolloutArgs& a, bool f32, int t, int mode, size_t rows, size_t row0, cudaStream_t s) {
     switch (a.d.H) {
-        case 512: k_heads_wide<512><<<grid, 256, smem, s>>>(a, t, mode, rows, row0); break;
-        case 1024: k_heads_wide<1024><<<grid, 256, smem, s>>>(a, t, mode, rows, row0); break;
-        case 2048: k_heads_wide<2048><<<grid, 256, smem, s>>>(a, t, mode, rows, row0); break;
+        case 384: return f32 ? heads_wide_t<384, true>(a, t, mode, rows, row0, s) : heads_wide_t<384, false>(a, t, mode, rows, row0, s);
+        case 512: return f32 ? heads_wide_t<512, true>(a, t, mode, rows, row0, s) : heads_wide_t<512, false>(a, t, mode, rows, row0, s);
+        case 768: return f32 ? heads_wide_t<768, true>(a, t, mode, rows, row0, s) : heads_wide_t<768, false>(a, t, mode, rows, row0, s);
+        case 1024: return f32 ? heads_wide_t<1024, true>(a, t, mode, rows, row0, s) : heads_wide_t<1024, false>(a, t, mode, rows, row0, s);
         default: return cudaErrorNotSupported;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace
 
+// fp32 workloads compute with the master parameters themselves.
+static bool is_f32(const Buffers& b) { return b.theta_c == b.theta; }
+
 cudaError_t launch_pack_w2_wide(const Dims& d, const Buffers& b, const Ctx& c) {
     Scope sc(c, K_PACK_W2);
-    k_pack_w2_wide<<<(unsigned)(((size_t)d.H * d.H + 255) / 256), 256, 0, c.s>>>(d, b);
+    const unsigned nb = (unsigned)(((size_t)d.H * d.H / 2 + 255) / 256);
+    if (is_f32(b)) k_pack_w2_wide<true><<<nb, 256, 0, c.s>>>(d, b);
+    else k_pack_w2_wide<false><<<nb, 256, 0, c.s>>>(d, b);
     return cudaGetLastError();
 }
 
-// base = b1 + walls x W1[wall plane] + W1[goal row] as one GEMM (K = C cells).  Applies to the buffers of the wide path
-// (bf16 workload: the products 1 x w are exact and the accumulation is fp32); cudaErrorNotSupported otherwise.
-// Uses the dh1 buffer, which is dead outside the update, as scratch for the two bf16 operands.
+size_t wide_scratch_bytes(const Dims& d) {
+    const size_t Cp = (size_t)(d.C + 63) / 64 * 64;
+    return 3 * ((size_t)d.B * Cp + Cp * d.H) * 2;
+}
+size_t wide_h1_rows(const Dims& d) { return (size_t)d.B * d.Tmax + d.B; }
+
+// base = b1 + walls x W1[wall plane] + W1[goal row] as one GEMM (K = C cells, padded to a multiple of 64): the operand X is
+// exact, W1 has one (bf16 workload) or three exact bf16 terms, the accumulation is fp32.  Three terms are one GEMM of three
+// times the K: the smallest term's rows first, X repeated.  cudaErrorNotSupported for the
+// buffers of other paths and for small batches, where the gather kernel's single launch is quicker (B H = 2^20: 11 us each).
+// Uses the dh1 buffer, which is dead outside the update, as scratch for the operands.
 cudaError_t launch_env_base_wide(const Dims& d, const Buffers& b, const Ctx& c) {
-    const bool wide_buffers = b.w2p_hi && d.H >= 512;  // (narrower layers keep fp32-sized activation buffers)
-    if (!wide_buffers || d.C % 64 != 0 || d.H % NtCfg::BN != 0 || d.H > NtCfg::MAXN) return cudaErrorNotSupported;
+    if (!b.w2p_hi || !wide_supported(d.H, 0) || (size_t)d.B * d.H < ((size_t)1 << 20)) return cudaErrorNotSupported;
+    const bool f32 = is_f32(b);
+    const int Cp = (d.C + 63) / 64 * 64, terms = f32 ? 3 : 1;
     uint16_t* X = reinterpret_cast<uint16_t*>(b.dh1);
-    uint16_t* W1w = X + (size_t)d.B * d.C;
-    NtMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.a, X, d.B, d.C, 128, true)) return cudaErrorNotSupported;
-    if (!make_tensor_map_2d(&maps.b, W1w, d.C, d.H, 64, true)) return cudaErrorNotSupported;
+    uint16_t* W1w = X + (size_t)d.B * Cp * terms;
     {
         Scope sc(c, K_ENV_BASE);
-        k_expand_walls<<<148 * 8, 256, 0, c.s>>>(d, b, X, W1w);
+        if (f32) k_expand_walls<true><<<148 * 8, 256, 0, c.s>>>(d, b, X, W1w, Cp);
+        else k_expand_walls<false><<<148 * 8, 256, 0, c.s>>>(d, b, X, W1w, Cp);
         CKW(cudaGetLastError());
     }
     Scope sc(c, K_ENV_BASE);
     NtArgs g;
     memset(&g, 0, sizeof(g));
-    g.M = d.B; g.N = d.H; g.K = d.C; g.row0 = 0;
+    g.M = d.B; g.N = d.H; g.K = Cp * terms; g.row0 = 0;
     g.bias = b.theta_c + d.ob1;
     g.outf = b.base;
     g.addrows = b.theta_c + d.oW1;
     g.addidx = b.goal;
     g.addrow0 = 2 * d.C;
+    g.addmax = d.C - 1;
     g.status = b.status;
-    return launch_nt<EPI_BASE, true>(maps, g, c.s);
+    return launch_nt<EPI_BASE, true>(X, d.B, W1w, g, c.s);
 }
 
-// T+1 forward passes (or, in replay mode, one pass over the recorded rows).
-cudaError_t launch_rollout_wide(const RolloutArgs& a, const Ctx& c) {
+template <bool F32>
+static cudaError_t rollout_wide_t(const RolloutArgs& a, const Ctx& c) {
     const Dims& d = a.d;
     const Buffers& b = a.b;
     const int H = d.H, B = d.B;
-    const size_t cap_rows = (size_t)2 * B * d.Tmax;  // the fp32-sized h1 / h2 buffers hold this many bf16 rows
-    NtMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.a, b.h1, cap_rows, H, 128, true)) return cudaErrorNotSupported;
-    if (!make_tensor_map_2d(&maps.b, b.w2p_hi, H, H, 64, true)) return cudaErrorNotSupported;
-    NtArgs g;
-    memset(&g, 0, sizeof(g));
-    g.N = H; g.K = H;
-    g.out = reinterpret_cast<uint16_t*>(b.h2);
-    g.bias = b.theta_c + d.ob2;
-    g.status = b.status;
-    auto h1_grid = [](size_t rows, int H) { return (unsigned)((rows * (H / 8) + 255) / 256); };
+    const size_t rows = wide_h1_rows(d);
+    auto fwd = [&](size_t n, size_t row0) {  // h2 of n rows
+        if constexpr (F32) {
+            X3Args g;
+            memset(&g, 0, sizeof(g));
+            g.M = (int)n; g.N = g.K = H; g.row0 = (int)row0;
+            g.arows = (int)rows; g.brows = H;
+            g.out = b.h2;
+            g.bias = b.theta_c + d.ob2;
+            g.status = b.status;
+            return launch_x3_nt(EPI_FWD, b.h1, 3 * rows, b.w2p_hi, g, c.s);
+        } else {
+            NtArgs g;
+            memset(&g, 0, sizeof(g));
+            g.M = (int)n; g.N = g.K = H; g.row0 = (int)row0;
+            g.out = reinterpret_cast<uint16_t*>(b.h2);
+            g.bias = b.theta_c + d.ob2;
+            g.status = b.status;
+            return launch_nt<EPI_FWD, true>(b.h1, rows, b.w2p_hi, g, c.s);
+        }
+    };
+    auto h1_rows = [&](const uint8_t* pos, size_t n, size_t row0) {
+        k_h1_wide<F32><<<(unsigned)((n * (H / 8) + 255) / 256), 256, 0, c.s>>>(d, b, pos, n, row0);
+        return cudaGetLastError();
+    };
+    // forward of n rows from row0: (h1,) h2, heads in the given mode
+    auto replay = [&](const uint8_t* pos, size_t n, size_t row0, int mode) {
+        {
+            Scope sc(c, K_REPLAY);
+            CKW(h1_rows(pos, n, row0));
+        }
+        {
+            Scope sc(c, K_REPLAY);
+            CKW(fwd(n, row0));
+        }
+        Scope sc(c, K_REPLAY);
+        return heads_wide(a, F32, 0, mode, n, row0, c.s);
+    };
     if (a.replay) {
         const size_t R = (size_t)B * a.T;
-        {
-            Scope sc(c, K_REPLAY);
-            k_h1_wide<<<h1_grid(R, H), 256, 0, c.s>>>(d, b, b.tpos, R, 0);
-            CKW(cudaGetLastError());
-        }
-        {
-            Scope sc(c, K_REPLAY);
-            g.M = (int)R; g.row0 = 0;
-            CKW((launch_nt<EPI_FWD, true>(maps, g, c.s)));
-        }
-        {
-            Scope sc(c, K_REPLAY);
-            CKW(heads_wide(a, 0, 2, R, 0, c.s));
-        }
-        if (a.replay == 2) {  // one more forward on the env state as it stands, in the B rows after the recorded ones
-            {
-                Scope sc(c, K_REPLAY);
-                k_h1_wide<<<h1_grid(B, H), 256, 0, c.s>>>(d, b, b.pos, B, R);
-                CKW(cudaGetLastError());
-            }
-            {
-                Scope sc(c, K_REPLAY);
-                g.M = B; g.row0 = (int)R;
-                CKW((launch_nt<EPI_FWD, true>(maps, g, c.s)));
-            }
-            Scope sc(c, K_REPLAY);
-            return heads_wide(a, 0, 3, B, R, c.s);
-        }
+        CKW(replay(b.tpos, R, 0, 2));
+        if (a.replay == 2) CKW(replay(b.pos, B, R, 3));  // and the env state as it stands, in the B rows after the recorded ones
         return cudaSuccess;
     }
     for (int t = 0; t <= a.T; ++t) {
         const size_t row0 = (size_t)t * B;
         if (t == 0) {  // later steps: the heads kernel of step t-1 writes the h1 rows of step t
             Scope sc(c, K_H1);
-            k_h1_wide<<<h1_grid(B, H), 256, 0, c.s>>>(d, b, b.pos, B, row0);
-            CKW(cudaGetLastError());
+            CKW(h1_rows(b.pos, B, row0));
         }
         {
             Scope sc(c, K_FWD2);
-            g.M = B; g.row0 = (int)row0;
-            CKW((launch_nt<EPI_FWD, true>(maps, g, c.s)));
+            CKW(fwd(B, row0));
         }
         {
             Scope sc(c, K_ROLLOUT);
-            CKW(heads_wide(a, t, t == a.T ? 1 : 0, B, row0, c.s));
+            CKW(heads_wide(a, F32, t, t == a.T ? 1 : 0, B, row0, c.s));
         }
     }
     return cudaSuccess;
 }
+// T+1 forward passes (or, in replay mode, one pass over the recorded rows).
+cudaError_t launch_rollout_wide(const RolloutArgs& a, const Ctx& c) { return is_f32(a.b) ? rollout_wide_t<true>(a, c) : rollout_wide_t<false>(a, c); }
 
-// dh1 = (dh2 W2^T) gated by h1 > 0 over all R rows, then S = sum over t of dh1.
-cudaError_t launch_dh1_wide(const LearnArgs& a, const Ctx& c) {
+// dh1 = (dh2 W2^T) gated by h1 > 0 over all R rows: fp32 (the agent-plane kernel reads it and forms S), or one bf16 plane and S.
+template <bool F32>
+static cudaError_t dh1_wide_t(const LearnArgs& a, const Ctx& c) {
     const Dims& d = a.d;
     const Buffers& b = a.b;
     const int H = d.H;
-    const size_t R = (size_t)d.B * a.T;
-    NtMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.a, b.dh2, R, H, 128, true)) return cudaErrorNotSupported;
-    if (!make_tensor_map_2d(&maps.b, b.w2p_hi, H, H, 128, true)) return cudaErrorNotSupported;
-    NtArgs g;
-    memset(&g, 0, sizeof(g));
-    g.M = (int)R; g.N = H; g.K = H; g.row0 = 0;
-    g.out = reinterpret_cast<uint16_t*>(b.dh1);
-    g.gate = reinterpret_cast<const uint16_t*>(b.h1);
-    g.status = b.status;
-    {
+    const size_t R = (size_t)d.B * a.T, plane = (size_t)d.B * d.Tmax;
+    if constexpr (F32) {
         Scope sc(c, K_DH1);
-        CKW((launch_nt<EPI_GATE, false>(maps, g, c.s)));
-    }
-    {
+        X3Args g;
+        memset(&g, 0, sizeof(g));
+        g.M = (int)R; g.N = g.K = H;
+        g.arows = (int)plane; g.brows = H;
+        g.out = b.dh1;
+        g.gate = reinterpret_cast<const uint16_t*>(b.h1);
+        g.status = b.status;
+        return launch_x3_nt(EPI_GATE, b.dh2, 3 * plane, b.w2p_hi, g, c.s);
+    } else {
+        NtArgs g;
+        memset(&g, 0, sizeof(g));
+        g.M = (int)R; g.N = g.K = H;
+        g.out = reinterpret_cast<uint16_t*>(b.dh1);
+        g.gate = reinterpret_cast<const uint16_t*>(b.h1);
+        g.status = b.status;
+        {
+            Scope sc(c, K_DH1);
+            CKW((launch_nt<EPI_GATE, false>(b.dh2, R, b.w2p_hi, g, c.s)));
+        }
         Scope sc(c, K_SUM_OVER_T);
         k_sum_t_wide<<<(unsigned)(((size_t)d.B * (H / 8) + 255) / 256), 256, 0, c.s>>>(d, b, a.T);
-        CKW(cudaGetLastError());
+        return cudaGetLastError();
     }
-    return cudaSuccess;
 }
+cudaError_t launch_dh1_wide(const LearnArgs& a, const Ctx& c) { return is_f32(a.b) ? dh1_wide_t<true>(a, c) : dh1_wide_t<false>(a, c); }
 
 }  // namespace anakin

@@ -47,7 +47,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pa
     const uint32_t rank = tc::cluster_ctarank();
     const bool leader = rank == 0;
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-    const int nt = g.N / BN, mt = (g.M + PM - 1) / PM, ntiles = mt * nt, nch = g.K / KC;
+    const int nt = (g.N + BN - 1) / BN, mt = (g.M + PM - 1) / PM, ntiles = mt * nt, nch = g.K / KC;
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); }
@@ -129,7 +129,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pa
             const int m = m0 + 32 * q + lane;
             const bool valid = m < g.M;
             const size_t gi = ((size_t)g.row0 + (valid ? m : 0)) * g.N + n0;
-            if (EPI == EPI_GATE && valid) nt_prefetch_gate(g, gi);  // towards L2 while the MMAs run
+            if (EPI == EPI_GATE && valid) nt_prefetch_gate(g, gi, g.N - n0);  // towards L2 while the MMAs run
             ok = tc::mbar_wait(&tfull[buf], (u >> 1) & 1);
             if (!ok) break;
             tc::tc_fence_after();
@@ -152,7 +152,7 @@ template <int EPI, bool B_MN>
 cudaError_t launch_pair_t(const NtMaps& maps, const NtArgs& g, cudaStream_t s) {
     const cudaError_t e = cudaFuncSetAttribute(k_gemm_nt_pair<EPI, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::smem_bytes);
     if (e != cudaSuccess) return e;
-    const int ntiles = ((g.M + PairCfg::PM - 1) / PairCfg::PM) * (g.N / PairCfg::BN);
+    const int ntiles = ((g.M + PairCfg::PM - 1) / PairCfg::PM) * ((g.N + PairCfg::BN - 1) / PairCfg::BN);
     const int pairs = ntiles < 74 ? ntiles : 74;
     k_gemm_nt_pair<EPI, B_MN><<<2 * pairs, PairCfg::THREADS, PairCfg::smem_bytes, s>>>(maps, g);
     return cudaGetLastError();
@@ -160,10 +160,10 @@ cudaError_t launch_pair_t(const NtMaps& maps, const NtArgs& g, cudaStream_t s) {
 
 }  // namespace
 
-// Needs: N a multiple of 256 (at most 2048), K a multiple of 64, an A map with 128-row boxes and a B map with 64 x 64
+// Needs: N a multiple of 64 (at most 2048), K a multiple of 64, an A map with 128-row boxes and a B map with 64 x 64
 // boxes (MN-major B) or 128-row boxes (K-major B).
 cudaError_t launch_nt_pair(int epi, bool b_mn, const NtMaps& maps, const NtArgs& g, cudaStream_t s) {
-    if (g.N % PairCfg::BN != 0 || g.K % PairCfg::KC != 0 || g.N > NT_MAXN || g.M < 1) return cudaErrorNotSupported;
+    if (g.N % 64 != 0 || g.K % PairCfg::KC != 0 || g.N > NT_MAXN || g.M < 1) return cudaErrorNotSupported;
     if (epi == EPI_FWD && b_mn) return launch_pair_t<EPI_FWD, true>(maps, g, s);
     if (epi == EPI_GATE && !b_mn) return launch_pair_t<EPI_GATE, false>(maps, g, s);
     if (epi == EPI_BASE && b_mn) return launch_pair_t<EPI_BASE, true>(maps, g, s);

@@ -17,7 +17,7 @@ struct NtArgs {
     float* outf;           // EPI_BASE: fp32 [rows][N] = acc + bias[n] + addrows[(addrow0 + addidx[m])*N + n]
     const float* addrows;
     const uint8_t* addidx;
-    int addrow0;
+    int addrow0, addmax;   // (indexes above addmax are taken as addmax)
     int* status;
 };
 
@@ -25,13 +25,26 @@ struct NtMaps {
     CUtensorMap a, b;
 };
 
+// fp32 operands as three exact bf16 planes (x3_gemm.cu): plane p of A / B lies p * arows / p * brows rows further down.
+struct X3Args {
+    int M, N, K, row0;
+    int arows, brows;
+    float* out;            // fp32 [rows][N]
+    const float* bias;     // EPI_FWD
+    const uint16_t* gate;  // EPI_GATE: first plane of the activation
+    int* status;
+};
+// a = planes of A [3 * arows][K], b = planes of B: [3 * brows][N] (MN-major) or [3 * brows][K] (K-major); cudaErrorNotSupported if not covered
+cudaError_t launch_x3_nt(int epi, const void* a, size_t a_rows_total, const void* b, const X3Args& g, cudaStream_t s);
+
 constexpr int NT_BN = 256;    // accumulator columns of an output tile
 constexpr int NT_MAXN = 2048;  // bias staging in shared memory
 
 // Pulls the gate bytes of one output row's tile (512 B) towards L2; called before the accumulator is waited for.
-__device__ __forceinline__ void nt_prefetch_gate(const NtArgs& g, size_t gi) {
+__device__ __forceinline__ void nt_prefetch_gate(const NtArgs& g, size_t gi, int cols) {
 #pragma unroll
-    for (int l = 0; l < 4; ++l) asm volatile("prefetch.global.L2 [%0];" ::"l"(g.gate + gi + 64 * l));
+    for (int l = 0; l < 4; ++l)
+        if (64 * l < cols) asm volatile("prefetch.global.L2 [%0];" ::"l"(g.gate + gi + 64 * l));
 }
 
 constexpr int NT_STAGE_BYTES = 4096;  // per epilogue warp: 32 rows x 64 bf16 columns
@@ -53,12 +66,13 @@ __device__ __forceinline__ void nt_epilogue_warp(const NtArgs& g, const float* s
     const int crow = lane >> 3, cch = lane & 7;                       // coalesced phase: row 4i + crow, 16-byte chunk cch
 #pragma unroll 1
     for (int c0 = c_begin; c0 < c_end; c0 += 64) {
+        if (n0 + c0 >= g.N) break;  // columns past the matrix (its width is a multiple of 64)
         uint32_t r0[32], r1[32];
         if (EPI == EPI_BASE) {
             tc::tmem_ld32(taddr + (uint32_t)c0, r0);
             tc::tmem_ld32(taddr + (uint32_t)(c0 + 32), r1);
             if (valid) {
-                const float4* add = reinterpret_cast<const float4*>(g.addrows + ((size_t)g.addrow0 + g.addidx[m]) * g.N + n0 + c0);
+                const float4* add = reinterpret_cast<const float4*>(g.addrows + ((size_t)g.addrow0 + min((int)g.addidx[m], g.addmax)) * g.N + n0 + c0);
                 float4* dst = reinterpret_cast<float4*>(g.outf + gi + c0);
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
