@@ -105,7 +105,7 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
             if (!ok) atomicOr(g.status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {
-        if (lane == 0 && leader) {  // ---- MMA issuer
+        if (leader) {  // ---- MMA issuer: the whole warp walks the loop, one elected lane issues
             const uint32_t idesc = tc::umma_idesc<2>(PM, BN, false, B_MN);
             int c = 0;
             for (int tile = unit; tile < ntiles && ok; tile += units) {
@@ -113,7 +113,7 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
                     const int s = c % STAGES, buf = c & 1;
                     if (c >= 2) ok = PAIR ? tc::mbar_wait_cluster(&tempty[buf], ((c >> 1) - 1) & 1) : tc::mbar_wait(&tempty[buf], ((c >> 1) - 1) & 1);
                     if (ok) ok = tc::mbar_wait(&full[s], (c / STAGES) & 1);
-                    if (!ok) break;
+                    if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
                     tc::tc_fence_after();
                     const uint32_t acc = tmem + (uint32_t)(buf * BN);
                     unsigned char* sa = base + s * Cfg::STAGE;
@@ -121,26 +121,29 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
                     // K-major: 16 k = 32 bytes along the swizzled 128-byte rows; MN-major: 16 k rows = 2048 bytes (the start address
                     // is the descriptor's low field, in 16-byte units)
                     const uint64_t a0 = tc::umma_desc(sa, 16, 1024), b0 = B_MN ? tc::umma_desc(sb, 8192, 1024) : tc::umma_desc(sb, 16, 1024);
-#pragma unroll 1
-                    for (int i = 0; i < tc::X3_PAIRS; ++i) {
-                        const uint64_t pa = a0 + (uint64_t)(tc::x3_a(i) * (Cfg::A_PLANE >> 4)), pb = b0 + (uint64_t)(tc::x3_b(i) * (Cfg::B_PLANE >> 4));
+                    if (tc::elect_one()) {
 #pragma unroll
-                        for (int k16 = 0; k16 < KC / 16; ++k16) {
-                            const uint64_t ad = pa + (uint64_t)(k16 * 2), bd = pb + (uint64_t)(k16 * (B_MN ? 128 : 2));
-                            if constexpr (PAIR) tc::umma_pair(acc, ad, bd, idesc, (i > 0 || k16 > 0) ? 1u : 0u);
-                            else tc::umma(acc, ad, bd, idesc, (i > 0 || k16 > 0) ? 1u : 0u);
+                        for (int i = 0; i < tc::X3_PAIRS; ++i) {
+#pragma unroll
+                            for (int k16 = 0; k16 < KC / 16; ++k16) {
+                                const uint64_t ad = a0 + (uint64_t)(tc::x3_a(i) * (Cfg::A_PLANE >> 4) + k16 * 2);
+                                const uint64_t bd = b0 + (uint64_t)(tc::x3_b(i) * (Cfg::B_PLANE >> 4) + k16 * (B_MN ? 128 : 2));
+                                if constexpr (PAIR) tc::umma_pair(acc, ad, bd, idesc, (i > 0 || k16 > 0) ? 1u : 0u);
+                                else tc::umma(acc, ad, bd, idesc, (i > 0 || k16 > 0) ? 1u : 0u);
+                            }
+                        }
+                        if constexpr (PAIR) {
+                            tc::umma_commit_pair(&empty[s], 3);
+                            tc::umma_commit_pair(&tfull[buf], 3);
+                        } else {
+                            tc::umma_commit(&empty[s]);
+                            tc::umma_commit(&tfull[buf]);
                         }
                     }
-                    if constexpr (PAIR) {
-                        tc::umma_commit_pair(&empty[s], 3);
-                        tc::umma_commit_pair(&tfull[buf], 3);
-                    } else {
-                        tc::umma_commit(&empty[s]);
-                        tc::umma_commit(&tfull[buf]);
-                    }
+                    __syncwarp();
                 }
             }
-            if (!ok) atomicOr(g.status, DEV_E_WAIT_TIMEOUT);
+            if (!ok && lane == 0) atomicOr(g.status, DEV_E_WAIT_TIMEOUT);
         }
     } else {
         // ---- epilogue warps: accumulator lanes 32*(wid%4)..+31 = output rows, column half (wid-2)/4
