@@ -95,21 +95,22 @@ __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1Tc
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {
-        if (lane == 0) {  // ---- MMA issuer
+        {  // ---- MMA issuer: the whole warp walks the loop, one elected lane issues
             const uint32_t idesc = tc::umma_idesc<PREC>(BM, BN, false, false);
-            ok = tc::mbar_wait(wfull, 0);
+            ok = tc::warp_all(tc::mbar_wait(wfull, 0));
             for (int u = 0; u < nsteps && ok; ++u) {
                 const int buf = u & 1;
-                if (u >= 2) ok = tc::mbar_wait(&tempty[buf], ((u >> 1) - 1) & 1);  // epilogue of step u-2 has drained it
+                if (u >= 2) ok = tc::warp_all(tc::mbar_wait(&tempty[buf], ((u >> 1) - 1) & 1));  // epilogue of step u-2 has drained it
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(buf * BN);
                 for (int kc = 0; kc < NCH && ok; ++kc) {
                     const int c = u * NCH + kc, s = c % STAGES;
-                    ok = tc::mbar_wait(&full[s], (c / STAGES) & 1);
+                    ok = tc::warp_all(tc::mbar_wait(&full[s], (c / STAGES) & 1));
                     if (!ok) break;
                     tc::tc_fence_after();
                     unsigned char* sa = sA + s * Cfg::A_STAGE;
+                    if (tc::elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < KC / 16; ++k16) {
                         // K-major operands: 16 k = 32 bytes further along the swizzled 128-byte rows
@@ -124,10 +125,12 @@ __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1Tc
                         tc::umma(acc, a_hi, w_hi, idesc, accum);
                     }
                     tc::umma_commit(&empty[s]);
+                    if (kc == NCH - 1) tc::umma_commit(&tfull[buf]);
+                    }
+                    __syncwarp();
                 }
-                if (ok) tc::umma_commit(&tfull[buf]);
             }
-            if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
+            if (!ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else {
         // ---- epilogue warps: accumulator lanes 32*(wid%4)..+31 (= envs), column half (wid-2)/4 of the 128-wide tile

@@ -212,14 +212,15 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {
-        if (lane == 0 && leader) {  // ---- MMA issuer (of the pair)
+        if (leader) {  // ---- MMA issuer (of the pair): the whole warp walks the loop, one elected lane issues
             const uint32_t idesc = tc::umma_idesc<PREC>(NCTA * BN, BM, false, false);
             const uint32_t idesc_agent = tc::umma_idesc<PREC>(NCTA * BN, 128, false, true);
             // agent-plane product of step v: 8 k16 steps over the 128 envs per plane of dh1 (the one-hot is exact)
             auto agent_mma = [&](int v) {
-                ok = wait_leader(tiles_full, (uint32_t)v & 1u);
+                ok = tc::warp_all(wait_leader(tiles_full, (uint32_t)v & 1u));
                 if (!ok) return;
                 tc::tc_fence_after();
+                if (tc::elect_one()) {
 #pragma unroll
                 for (int pl = 0; pl < PL; ++pl) {
 #pragma unroll
@@ -234,20 +235,23 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                     }
                 }
                 commit(tiles_free);
+                }
+                __syncwarp();
             };
-            ok = wait_leader(wfull, 0);
+            ok = tc::warp_all(wait_leader(wfull, 0));
             for (int u = 0; u < G && ok; ++u) {
                 const int buf = u & 1;
-                if (u >= 2) ok = wait_leader(&tempty[buf], (uint32_t)((u >> 1) - 1) & 1u);  // the epilogues of step u-2 have drained it
+                if (u >= 2) ok = tc::warp_all(wait_leader(&tempty[buf], (uint32_t)((u >> 1) - 1) & 1u));  // the epilogues of step u-2 have drained it
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(Cfg::ACC_COL + 128 * buf);
                 for (int kc = 0; kc < NCH && ok; ++kc) {
                     const int c = u * NCH + kc, s = c % STAGES;
-                    ok = tc::mbar_wait(&full[s], (c / STAGES) & 1);
+                    ok = tc::warp_all(tc::mbar_wait(&full[s], (c / STAGES) & 1));
                     if (!ok) break;
                     tc::tc_fence_after();
                     unsigned char* sa = sA + s * Cfg::A_STAGE;
+                    if (tc::elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < KC / 16; ++k16) {
                         // W2 rows in tensor memory: 16 k = 8 columns; dh2 (K-major): 16 k = 32 bytes along the swizzled rows
@@ -274,13 +278,15 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                         }
                     }
                     commit(&empty[s]);
+                    if (kc == NCH - 1) commit(&tfull[buf]);
+                    }
+                    __syncwarp();
                 }
                 if (!ok) break;
-                commit(&tfull[buf]);
                 if (u >= 1) agent_mma(u - 1);  // queued behind this step's product: the tensor pipe stays busy
             }
             if (ok && G > 0) agent_mma(G - 1);
-            if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
+            if (!ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 2) {
         if (lane == 0) {  // ---- TMA producer of the gate tiles (rows as for dh2, units n0 .. n0+127 of the h1 hi plane)

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {
-        if (lane == 0) {  // ---- MMA issuer
+        {  // ---- MMA issuer: the whole warp walks the loop, one elected lane issues
             const uint32_t idesc = tc::umma_idesc<PREC>(BM, BN, true, true);
             for (int c = 0; c < nchunks && ok; ++c) {
                 const int s = c % STAGES;
@@ -169,11 +169,12 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
                 const uint32_t acc = tmem + (uint32_t)((grp & 1) * BN);
                 // the third and later groups reuse an accumulator: wait until the epilogue warps have read it out
                 if (FLUSH && cg == 0 && grp >= 2) ok = tc::mbar_wait(&accempty[grp & 1], ((grp >> 1) - 1) & 1);
-                if (ok) ok = tc::mbar_wait(&bars[s], (c / STAGES) & 1);
+                ok = tc::warp_all(ok && tc::mbar_wait(&bars[s], (c / STAGES) & 1));
                 if (!ok) break;
                 tc::tc_fence_after();
                 unsigned char* sa = base + s * Cfg::STAGE;
                 unsigned char* sb = sa + APL * Cfg::A_PLANE;
+                if (tc::elect_one()) {
                 if constexpr (Cfg::X3) {
 #pragma unroll
                     for (int i = 0; i < tc::X3_PAIRS; ++i)
@@ -195,8 +196,10 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
                 }
                 tc::umma_commit(&bars[STAGES + s]);  // frees the stage when these MMAs are done
                 if (c == nchunks - 1 || (FLUSH && cg == GROUP - 1)) tc::umma_commit(&accfull[grp & 1]);  // this group's sum is complete
+                }
+                __syncwarp();
             }
-            if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
+            if (!ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else {
         // ---- warps 2-5: builders of a synthesized A tile, then the epilogue

@@ -106,15 +106,16 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
     const int my_its = (ntiles > (int)blockIdx.x) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;  // tiles of this CTA
 
     if (FUSE && tid >= NTHREADS + 32) {
-        // ---- the MMA warp (one lane): per tile, dW2[i][j] += sum over the tile's 32 rows of h1[r][i] dh2[r][j] with the h1
+        // ---- the MMA warp: per tile, dW2[i][j] += sum over the tile's 32 rows of h1[r][i] dh2[r][j] with the h1
         // tile (TMA, MN-major boxes) as A and the dh2 tile the column warps wrote as B; both are double-buffered.
         const uint32_t tmem = *tmem_slot;
-        if (tid == NTHREADS + 32) {
+        {  // (the whole warp walks the loop, one elected lane issues the copies and the MMAs)
             constexpr int PL = Cfg::PL;
             const uint32_t idesc = tc::umma_idesc<PREC>(128, H, true, true);
             constexpr int AB = Cfg::A_BUFS;
             auto load_h1 = [&](int it) {
                 const int buf = it % AB, row = ((int)blockIdx.x + it * (int)gridDim.x) * TR;
+                if (!tc::elect_one()) return;
                 tc::mbar_expect_tx(&a_full[buf], Cfg::OP_TILE);
 #pragma unroll
                 for (int bx = 0; bx < H / 64; ++bx) {
@@ -123,16 +124,17 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
                 }
             };
             for (int q = 0; q < AB; ++q)
-                if (my_its > q) load_h1(q);
+                if (my_its > q) { load_h1(q); __syncwarp(); }
             for (int it = 0; it < my_its && ok; ++it) {
                 const int buf = it & 1, abuf = it % AB;
                 const uint32_t ph = (uint32_t)(it >> 1) & 1u;
                 ok = tc::mbar_wait(&a_full[abuf], (uint32_t)(it / AB) & 1u);
-                if (ok) ok = tc::mbar_wait(&t_ready[buf], ph);
+                ok = tc::warp_all(ok && tc::mbar_wait(&t_ready[buf], ph));
                 if (!ok) break;
                 tc::tc_fence_after();
                 const unsigned char* ta = s_a + abuf * Cfg::OP_TILE;
                 const unsigned char* tb = s_t + buf * Cfg::OP_TILE;
+                if (tc::elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < TR / 16; ++k16) {
                     // MN-major operands: 16 k rows = 2048 bytes into each box, consecutive 64-wide boxes one box apart
@@ -152,12 +154,15 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
                     }
                 }
                 tc::umma_commit(&mma_done[buf]);
+                }
+                __syncwarp();
                 if (it + AB < my_its) {  // refill this h1 buffer once the MMAs that read it have finished
-                    ok = tc::mbar_wait(&mma_done[buf], ph);
+                    ok = tc::warp_all(tc::mbar_wait(&mma_done[buf], ph));
                     if (ok) load_h1(it + AB);
+                    __syncwarp();
                 }
             }
-            if (!ok) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
+            if (!ok && (tid & 31) == 0) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
         }
         // tensor memory is freed once every column warp has read its part of the accumulators
         __syncwarp();

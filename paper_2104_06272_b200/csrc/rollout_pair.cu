@@ -218,13 +218,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
         const bool acting = owner && !a.replay && t < a.T;
         StepPre pre;
         if (acting) pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
-        // ---- layer 2: the leader's issuer thread drives both tensor cores, k block by k block.  A block's sixteen
-        // arrivals also say that those warps have read last step's accumulators.
-        if (tid == NWT && rank == 0) {
+        // ---- layer 2: the leader's owner warp drives both tensor cores, k block by k block (the whole warp waits, one elected
+        // lane issues).  A block's sixteen arrivals also say that those warps have read last step's accumulators.
+        if (!worker && rank == 0) {
 #pragma unroll
             for (int kb = 0; kb < 4; ++kb) {
-                if (ok) ok = tc::mbar_wait_cluster(&ready[kb], (uint32_t)t & 1u);
+                ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[kb], (uint32_t)t & 1u));
                 tc::tc_fence_after();
+                if (tc::elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16) {
                     // A (MN-major): 16 k rows = 2048 bytes into each box, 8192 bytes between the two 64-column boxes
@@ -235,8 +236,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                     tc::umma_pair(tmem, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
                     tc::umma_pair(tmem + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
                 }
+                if (kb == 3) tc::umma_commit_pair(tfull, 3);
+                }
+                __syncwarp();
             }
-            tc::umma_commit_pair(tfull, 3);
         }
         // ---- heads (workers): thread = hidden unit j, 32 envs of CTA rE
         if (worker) {

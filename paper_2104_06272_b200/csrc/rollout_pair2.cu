@@ -174,10 +174,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     const int t_end = a.replay == 1 ? a.T - 1 : a.T;  // replay recomputes the T recorded rows (mode 2: and the current state)
 
     if (wid == iwarp) {
-        // ---- layer 2: one thread of the leader CTA drives both tensor cores for both groups, k block by k block, in the
+        // ---- layer 2: this warp of the leader CTA drives both tensor cores for both groups (one elected lane issues), k block by k block, in the
         // order the groups' operand blocks are written.  A block's sixteen arrivals also say that those warps have read
         // the group's accumulators of the step before.
-        if (issuer && rank == 0) {
+        if (rank == 0) {
             const uint32_t idesc_w = tc::umma_idesc<0>(256, 128, true, false), idesc_n = tc::umma_idesc<0>(256, 64, true, false);
             for (int t = 0; t <= t_end; ++t) {
                 for (int g = 0; g < NG; ++g) {
@@ -185,8 +185,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                     unsigned char* bop = s_bop + g * Cfg::B_BYTES;
 #pragma unroll
                     for (int kb = 0; kb < 4; ++kb) {
-                        if (ok) ok = tc::mbar_wait_cluster(&ready[4 * g + kb], (uint32_t)t & 1u);
+                        ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[4 * g + kb], (uint32_t)t & 1u));
                         tc::tc_fence_after();
+                        if (tc::elect_one()) {
 #pragma unroll
                         for (int k16 = 0; k16 < 4; ++k16) {
                             // A (MN-major): 16 k rows = 2048 bytes into each box, 8192 bytes between the two 64-column boxes
@@ -197,8 +198,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                             tc::umma_pair(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
                             tc::umma_pair(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
                         }
+                        if (kb == 3) tc::umma_commit_pair(&tfull[g], 3);
+                        }
+                        __syncwarp();
                     }
-                    tc::umma_commit_pair(&tfull[g], 3);
                 }
             }
         }

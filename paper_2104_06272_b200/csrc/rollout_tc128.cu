@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
     const int t_end = a.replay == 1 ? a.T - 1 : a.T;  // replay recomputes the T recorded rows (mode 2: and the current state)
 
-    if (issuer) {
-        // ---- layer 2: one thread drives the tensor core for both groups, k block by k block, in the order the groups'
+    if (wid == (NWT + NOWN) / 32) {
+        // ---- layer 2: one warp drives the tensor core for both groups (an elected lane issues), k block by k block, in the order the groups'
         // operand blocks are written (group 0, then group 1, every step).  A block's eight arrivals also say that those
         // warps have read the group's accumulators of the step before.
         const uint32_t idesc_w = tc::umma_idesc<0>(128, 128, true, false), idesc_n = tc::umma_idesc<0>(128, 64, true, false);
@@ -178,8 +178,9 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                 unsigned char* bop = s_bop + g * Cfg::B_BYTES;
 #pragma unroll
                 for (int kb = 0; kb < 2; ++kb) {
-                    if (ok) ok = tc::mbar_wait(&ready[2 * g + kb], (uint32_t)t & 1u);
+                    ok = tc::warp_all(ok && tc::mbar_wait(&ready[2 * g + kb], (uint32_t)t & 1u));
                     tc::tc_fence_after();
+                    if (tc::elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16) {
                         // A (MN-major): 16 k rows = 2048 bytes into each box, one box further per 64 columns
@@ -190,8 +191,10 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                         tc::umma(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
                         tc::umma(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
                     }
+                    if (kb == 1) tc::umma_commit(&tfull[g]);
+                    }
+                    __syncwarp();
                 }
-                tc::umma_commit(&tfull[g]);
             }
         }
     } else if (worker) {

@@ -160,6 +160,9 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
+// Every lane of the warp says yes: after a bounded wait that all lanes take, so that they leave or go on together.
+__device__ __forceinline__ bool warp_all(bool ok) { return __all_sync(0xFFFFFFFFu, ok); }
+
 // ---- CTA pairs (clusters of two): one thread of the leader CTA issues MMAs that span both CTAs' tensor cores ----
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;

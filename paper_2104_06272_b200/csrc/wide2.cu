@@ -90,22 +90,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pa
             if (!ok) atomicOr(g.status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {
-        if (lane == 0 && leader) {  // ---- MMA issuer of the pair
+        if (leader) {  // ---- MMA issuer of the pair: the whole warp walks the loop, one elected lane issues
             const uint32_t idesc = tc::umma_idesc<1>(PM, BN, false, B_MN);
             int c = 0, u = 0;
             for (int tile = pair; tile < ntiles && ok; tile += npairs, ++u) {
                 const int buf = u & 1;
-                if (u >= 2) ok = tc::mbar_wait_cluster(&tempty[buf], ((u >> 1) - 1) & 1);  // both epilogues have drained tile u-2
+                if (u >= 2) ok = tc::warp_all(tc::mbar_wait_cluster(&tempty[buf], ((u >> 1) - 1) & 1));  // both epilogues have drained tile u-2
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(buf * BN);
                 for (int kc = 0; kc < nch; ++kc, ++c) {
                     const int s = c % STAGES;
-                    ok = tc::mbar_wait(&full[s], (c / STAGES) & 1);
+                    ok = tc::warp_all(tc::mbar_wait(&full[s], (c / STAGES) & 1));
                     if (!ok) break;
                     tc::tc_fence_after();
                     unsigned char* sa = base + s * Cfg::STAGE;
                     unsigned char* sb = sa + Cfg::A_BYTES;
+                    if (tc::elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < KC / 16; ++k16) {
                         // K-major: 16 k = 32 bytes along the swizzled 128-byte rows; MN-major: 16 k rows = 2048 bytes
@@ -114,10 +115,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pa
                         tc::umma_pair(acc, ad, bd, idesc, (kc > 0 || k16 > 0) ? 1u : 0u);
                     }
                     tc::umma_commit_pair(&empty[s], 3);
+                    if (kc == nch - 1) tc::umma_commit_pair(&tfull[buf], 3);
+                    }
+                    __syncwarp();
                 }
-                if (ok) tc::umma_commit_pair(&tfull[buf], 3);
             }
-            if (!ok) atomicOr(g.status, DEV_E_WAIT_TIMEOUT);
+            if (!ok && lane == 0) atomicOr(g.status, DEV_E_WAIT_TIMEOUT);
         }
     } else {
         // ---- epilogue warps: accumulator lanes 32*(wid%4)..+31 = this CTA's output rows

@@ -113,7 +113,8 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
                     const int s = c % STAGES, buf = c & 1;
                     if (c >= 2) ok = PAIR ? tc::mbar_wait_cluster(&tempty[buf], ((c >> 1) - 1) & 1) : tc::mbar_wait(&tempty[buf], ((c >> 1) - 1) & 1);
                     if (ok) ok = tc::mbar_wait(&full[s], (c / STAGES) & 1);
-                    if (!__all_sync(0xFFFFFFFFu, ok)) { ok = false; break; }
+                    ok = tc::warp_all(ok);
+                    if (!ok) break;
                     tc::tc_fence_after();
                     const uint32_t acc = tmem + (uint32_t)(buf * BN);
                     unsigned char* sa = base + s * Cfg::STAGE;
