@@ -25,7 +25,6 @@ struct anakin_handle {
     bool adv_valid;   // ADV/RET were computed from the pending trajectory (by the rollout's fused GAE scan)
     bool acts_valid;  // the saved h1/h2 belong to the pending trajectory and the current parameters
     int last_T;
-    int NS;
     int K;             // policies (>= 1)
     size_t sub_bytes;  // size of one policy's sub-workspace
     uint64_t seed;
@@ -67,19 +66,8 @@ int validate(const anakin_cfg* c) {
 int policies_of(const anakin_cfg& c) { return c.n_policies >= 2 ? c.n_policies : 1; }
 int envs_per_policy(const anakin_cfg& c) { const int K = policies_of(c); return (c.B + K - 1) / K; }
 
-int choose_splits(const Dims& d) {
-    const int tiles = ((d.H + 63) / 64) * ((d.H + 63) / 64);
-    int ns = (4 * 148 + tiles - 1) / tiles;
-    if (ns > 64) ns = 64;
-    const size_t R = (size_t)d.B * d.Tmax;
-    const size_t cap = R / 64 > 0 ? R / 64 : 1;
-    if ((size_t)ns > cap) ns = (int)cap;
-    if (ns < 1) ns = 1;
-    return ns;
-}
-
 // Carves the workspace; with base == nullptr only sizes it.
-size_t carve(const anakin_cfg& c, const Dims& d, int NS, unsigned char* base, Buffers* out) {
+size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* out) {
     size_t off = 0;
     auto take = [&](size_t bytes) -> void* {
         void* p = base ? base + off : nullptr;
@@ -110,32 +98,28 @@ size_t carve(const anakin_cfg& c, const Dims& d, int NS, unsigned char* base, Bu
     b.dbg_logits = c.debug_logits ? (float*)take(R * 16) : nullptr;
     b.dbg_gates = c.debug_logits ? (uint32_t*)take(2 * R * (H / 32) * 4) : nullptr;
     b.base = (float*)take(B * H * 4);
-    const bool mma = rollout_mma_supported(d.H), tensor = tensor_path_supported(d.H, c.precision);
+    const bool mma = rollout_mma_supported(d.H);
     const bool frags = mma && rollout_uses_fragments(d.H, c.precision);
     b.w2f_hi = frags ? (uint2*)take(H * H * 2) : nullptr;
     b.w2f_lo = frags ? (uint2*)take(H * H * 2) : nullptr;
     const bool wide = wide_supported(d.H, c.precision), f32 = c.precision == ANAKIN_PRECISION_FP32;
-    b.w2p_hi = tensor ? (uint16_t*)take(H * H * 2 * (wide && f32 ? 3 : 1)) : nullptr;
-    b.w2p_lo = mma ? (uint16_t*)take(H * H * 2) : nullptr;
+    const bool x3 = three_terms(d.H, c.precision);
+    b.w2f_lo2 = frags && x3 ? (uint2*)take(H * H * 2) : nullptr;
+    b.w2p_hi = (uint16_t*)take(H * H * 2 * (x3 ? 3 : 1));
+    b.w2p_lo = mma && !x3 ? (uint16_t*)take(H * H * 2) : nullptr;
     // wide layers: bf16 planes of h1 (three exact terms in fp32 workloads) with room for the bootstrap step's rows; h2 likewise
-    b.h1 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 6 : 2) : R * H * 4);
+    b.h1 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 6 : 2) : R * H * (x3 ? 6 : 4));
     b.gate1 = (dh1_agent_tc_supported(d) && policies_of(c) <= 1) ? (uint8_t*)take(R * (H / 8)) : nullptr;  // what the fused dh1 kernel gates with
     b.h2 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 4 : 2) : R * H * 4);
-    b.out5 = tensor ? (float*)take(R * 8 * 4) : nullptr;
-    b.vboot = tensor ? (float*)take(B * 4) : nullptr;
-    b.dh2 = (float*)take(R * H * (!wide ? 4 : f32 ? 6 : 2));
+    b.out5 = (float*)take(R * 8 * 4);
+    b.vboot = (float*)take(B * 4);
+    b.dh2 = (float*)take(R * H * (x3 ? 6 : wide ? 2 : 4));
     b.dh1 = (float*)take(!wide ? R * H * 4 : std::max(R * H * (f32 ? 4 : 2), wide_scratch_bytes(d)));
-    b.dout = (float*)take(R * 8 * 4);
-    b.S = (float*)take(4 * B * H * 4);  // up to four t-slices of two 16-bit planes
-    size_t part_floats = (size_t)NS * P, loss_blocks = LOSS_BLOCKS;
-    if (tensor) {
-        LearnPlan pl;
-        learn_mma_plan(d, &pl);
-        if (pl.part_floats > part_floats) part_floats = pl.part_floats;
-        if ((size_t)pl.loss_blocks > loss_blocks) loss_blocks = pl.loss_blocks;
-    }
-    b.part = (float*)take(part_floats * 4);
-    b.loss_part = (float*)take(loss_blocks * 4 * 4);
+    b.S = (float*)take(4 * B * H * 4);  // up to four t-slices of two 16-bit planes, or three planes
+    LearnPlan pl;
+    learn_mma_plan(d, &pl);
+    b.part = (float*)take(pl.part_floats * 4);
+    b.loss_part = (float*)take((size_t)pl.loss_blocks * 4 * 4);
     b.stats = (anakin_stats*)take(sizeof(anakin_stats));
     b.status = (int*)take(sizeof(int));
     if (out) *out = b;
@@ -234,7 +218,7 @@ int do_rollout(anakin_t* h, int T, const int8_t* forced) {
     h->gstep += T;
     h->last_T = T;
     h->rollout_pending = true;
-    h->acts_valid = tensor_path_supported(h->d.H, h->cfg.precision);  // the tensor-core rollouts save h1 and h2 of every row
+    h->acts_valid = true;  // the rollouts save h1 and h2 of every row
     h->adv_valid = a.fuse_gae != 0;
     return ANAKIN_OK;
 }
@@ -286,7 +270,7 @@ int anakin_workspace_bytes(const anakin_cfg* cfg, size_t* bytes) {
     if (rc != ANAKIN_OK) return rc;
     Dims d = make_dims(envs_per_policy(*cfg), cfg->N, cfg->H, cfg->T_max);
     d.npol = policies_of(*cfg);  // (the update's launch plan, and with it the partial buffers, depend on it)
-    *bytes = carve(*cfg, d, choose_splits(d), nullptr, nullptr) * (size_t)policies_of(*cfg);  // one sub-workspace per policy
+    *bytes = carve(*cfg, d, nullptr, nullptr) * (size_t)policies_of(*cfg);  // one sub-workspace per policy
     return ANAKIN_OK;
 }
 
@@ -300,8 +284,7 @@ int anakin_create(const anakin_cfg* cfg, void* dev_workspace, size_t bytes, void
     Dims d = make_dims(Bp, cfg->N, cfg->H, cfg->T_max);
     d.env0 = cfg->env_offset;
     d.npol = K;
-    const int NS = choose_splits(d);
-    const size_t sub = carve(*cfg, d, NS, nullptr, nullptr), need = sub * (size_t)K;
+    const size_t sub = carve(*cfg, d, nullptr, nullptr), need = sub * (size_t)K;
     d.B_last = cfg->B - (K - 1) * Bp;
     d.pstride = sub;
     if (bytes < need) return ANAKIN_E_WORKSPACE_TOO_SMALL;
@@ -315,13 +298,12 @@ int anakin_create(const anakin_cfg* cfg, void* dev_workspace, size_t bytes, void
     h->cuda_err[0] = 0;
     h->cfg = *cfg;
     h->d = d;
-    h->NS = NS;
     h->K = K;
     h->sub_bytes = sub;
     h->ws = (unsigned char*)dev_workspace;
     h->ws_bytes = bytes;
     h->stream = (cudaStream_t)cuda_stream;
-    carve(*cfg, d, NS, h->ws, &h->b);
+    carve(*cfg, d, h->ws, &h->b);
     int cur = -1;
     cudaError_t e = cudaGetDevice(&cur);
     if (e == cudaSuccess && cur != cfg->device) e = cudaSetDevice(cfg->device);
@@ -344,6 +326,7 @@ int anakin_destroy(anakin_t* h) {
 int anakin_reset(anakin_t* h, uint64_t seed) {
     if (!h) return ANAKIN_E_INVALID_ARG;
     cudaError_t e = launch_reset(h->d, h->b, seed, h->cfg.wall_density, h->cfg.precision, h->ctx());
+    if (e == cudaSuccess) e = pack_w2(h);
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->seed = seed;
     h->gstep = 0;
@@ -351,7 +334,7 @@ int anakin_reset(anakin_t* h, uint64_t seed) {
     h->is_reset = true;
     h->rollout_pending = false;
     h->base_valid = false;
-    h->frags_valid = false;
+    h->frags_valid = true;
     h->acts_valid = false;
     h->adv_valid = false;
     h->last_T = 0;
@@ -391,7 +374,6 @@ static int learn_after_gae(anakin_t* h, int phase, float ppo_clip = 0.f, bool co
     a.d = h->d;
     a.b = h->b;
     a.T = h->last_T;
-    a.NS = h->NS;
     a.c_v = h->cfg.value_coef;
     a.c_e = h->cfg.entropy_coef;
     a.lr = h->cfg.lr;
@@ -411,15 +393,11 @@ static int learn_after_gae(anakin_t* h, int phase, float ppo_clip = 0.f, bool co
         a.gscale = (float)ldexp(1.0, ex);
         a.inv_gscale = (float)ldexp(1.0, -ex);
     }
-    if (tensor_path_supported(h->d.H, h->cfg.precision)) {
-        if (!h->acts_valid) {
-            const int rc = replay_activations(h);
-            if (rc != ANAKIN_OK) return rc;
-        }
-        e = launch_learn_mma(a, h->cfg.precision, h->ctx());
-    } else {
-        e = launch_learn(a, h->cfg.precision, h->ctx());
+    if (!h->acts_valid) {
+        const int rc = replay_activations(h);
+        if (rc != ANAKIN_OK) return rc;
     }
+    e = launch_learn_mma(a, h->cfg.precision, h->ctx());
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->acts_valid = false;  // saved activations belong to the parameters they were computed with
     if (consume) {
@@ -429,7 +407,7 @@ static int learn_after_gae(anakin_t* h, int phase, float ppo_clip = 0.f, bool co
     if (phase == 0) {
         h->adam_k += 1;
         h->base_valid = false;  // parameters changed
-        h->frags_valid = tensor_path_supported(h->d.H, h->cfg.precision);  // the tensor-core update refreshes the 16-bit copies itself
+        h->frags_valid = true;  // the update refreshes the 16-bit copies itself
     }
     return ANAKIN_OK;
 }
@@ -470,7 +448,7 @@ int anakin_learn_vtrace(anakin_t* h, int epochs, float rho_bar, float c_bar) {
     if (!h->is_reset || !h->rollout_pending) return ANAKIN_E_BAD_STATE;
     // the hidden widths this objective is offered at
     const int H = h->d.H;
-    const bool offered = rollout_mma_supported(H) || (h->cfg.precision == ANAKIN_PRECISION_BF16 && (H == 512 || H == 1024));
+    const bool offered = H == 64 || H == 128 || H == 256 || (h->cfg.precision == ANAKIN_PRECISION_BF16 && (H == 512 || H == 1024));
     if (h->K > 1 || !offered) return ANAKIN_E_UNSUPPORTED_CFG;
     for (int ep = 0; ep < epochs; ++ep) {
         cudaError_t e;
@@ -532,7 +510,7 @@ int anakin_apply_grads_mean(anakin_t* h, int n_replicas) {
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->adam_k += 1;
     h->base_valid = false;  // parameters changed
-    h->frags_valid = tensor_path_supported(h->d.H, h->cfg.precision);  // every element of the 16-bit copies of W2 was rewritten
+    h->frags_valid = true;  // every element of the 16-bit copies of W2 was rewritten
     return ANAKIN_OK;
 }
 
@@ -651,8 +629,8 @@ int anakin_kernel_count(void) { return K_COUNT; }
 
 const char* anakin_kernel_name(int id) {
     static const char* names[K_COUNT] = {"reset_env", "reset_params", "refresh_params", "env_base", "rollout", "gae", "h1",
-                                         "fwd2", "heads_loss", "dh1", "dw2", "colsums", "sum_over_t", "dw1_agent",
-                                         "dw1_walls", "dw1_goal", "reduce_adam", "loss_total", "pack_gates", "pack_w2", "heads_bwd", "replay", "vtrace"};
+                                         "fwd2", "dh1", "dw2", "sum_over_t", "dw1_agent",
+                                         "dw1_walls", "dw1_goal", "reduce_adam", "pack_gates", "pack_w2", "heads_bwd", "replay", "vtrace"};
     return (id >= 0 && id < K_COUNT) ? names[id] : "";
 }
 

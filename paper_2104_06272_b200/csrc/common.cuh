@@ -69,7 +69,8 @@ struct Buffers {
     uint32_t* dbg_gates;  // [2][R][H/32] or null: ReLU gates of the last update
     float* base;     // [B][H]  b1 + sum of W1 rows of the wall cells + W1 row of the goal cell
     uint2* w2f_hi;   // [H*H/4] W2 as mma.sync B fragments, high parts (null: the warp-level rollout kernel is not used)
-    uint2* w2f_lo;   // [H*H/4] bf16 low parts
+    uint2* w2f_lo;   // [H*H/4] low parts
+    uint2* w2f_lo2;  // [H*H/4] third terms (null unless fp32 operands have three)
     uint16_t* w2p_hi;  // [H][H] W2 row-major as 16-bit hi / lo planes (B operand of the dh1 kernel); wide fp32: three bf16 planes
     uint16_t* w2p_lo;
     float* h1;       // [R][H]
@@ -79,15 +80,13 @@ struct Buffers {
     float* vboot;    // [B] value of the state after the last recorded step under the CURRENT parameters (replay mode 2)
     float* dh2;      // [R][H]
     float* dh1;      // [R][H]
-    float* dout;     // [R][8]  (5 used)
     float* S;        // [B][H]  sum over t of dh1
-    float* part;     // [NS][P] split-K partial gradients
-    float* loss_part;  // [LOSS_BLOCKS][4]
+    float* part;     // split-K partial gradients (LearnPlan)
+    float* loss_part;  // [loss_blocks][4]
     anakin_stats* stats;
     int* status;
 };
 
-constexpr int LOSS_BLOCKS = 592;
 
 // ---- many policies: a kernel launched with one grid slice per policy moves every workspace pointer to its policy ----
 #ifdef __CUDACC__
@@ -101,9 +100,9 @@ __device__ __forceinline__ void shift_buffers(Buffers& b, size_t off) {
     shift_ptr(b.walls, off); shift_ptr(b.start, off); shift_ptr(b.goal, off); shift_ptr(b.pos, off); shift_ptr(b.tep, off);
     shift_ptr(b.tpos, off); shift_ptr(b.tact, off); shift_ptr(b.tdone, off); shift_ptr(b.trew, off); shift_ptr(b.tval, off);
     shift_ptr(b.tlogp, off); shift_ptr(b.adv, off); shift_ptr(b.ret, off); shift_ptr(b.dbg_logits, off); shift_ptr(b.dbg_gates, off);
-    shift_ptr(b.base, off); shift_ptr(b.w2f_hi, off); shift_ptr(b.w2f_lo, off);
+    shift_ptr(b.base, off); shift_ptr(b.w2f_hi, off); shift_ptr(b.w2f_lo, off); shift_ptr(b.w2f_lo2, off);
     shift_ptr(b.w2p_hi, off); shift_ptr(b.w2p_lo, off); shift_ptr(b.h1, off); shift_ptr(b.gate1, off); shift_ptr(b.h2, off); shift_ptr(b.out5, off);
-    shift_ptr(b.vboot, off); shift_ptr(b.dh2, off); shift_ptr(b.dh1, off); shift_ptr(b.dout, off); shift_ptr(b.S, off);
+    shift_ptr(b.vboot, off); shift_ptr(b.dh2, off); shift_ptr(b.dh1, off); shift_ptr(b.S, off);
     shift_ptr(b.part, off); shift_ptr(b.loss_part, off); shift_ptr(b.stats, off);
 }
 __device__ __forceinline__ void select_policy(Dims& d, Buffers& b, int pol) {
@@ -185,7 +184,6 @@ struct LearnArgs {
     Dims d;
     Buffers b;
     int T;
-    int NS;  // split-K factor of the weight-gradient GEMMs (FFMA path)
     float c_v, c_e;
     float lr, beta1, beta2, eps;
     int adam_k;  // step index after the increment
@@ -252,8 +250,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p);
 
 // Kernel identifiers (anakin_kernel_name / anakin_profile_read index by these).
 enum KernelId : int {
-    K_RESET_ENV = 0, K_RESET_PARAMS, K_REFRESH_PARAMS, K_ENV_BASE, K_ROLLOUT, K_GAE, K_H1, K_FWD2, K_HEADS_LOSS, K_DH1,
-    K_DW2, K_COLSUMS, K_SUM_OVER_T, K_DW1_AGENT, K_DW1_WALLS, K_DW1_GOAL, K_REDUCE_ADAM, K_LOSS_TOTAL, K_PACK_GATES, K_PACK_W2, K_HEADS_BWD, K_REPLAY, K_VTRACE, K_COUNT
+    K_RESET_ENV = 0, K_RESET_PARAMS, K_REFRESH_PARAMS, K_ENV_BASE, K_ROLLOUT, K_GAE, K_H1, K_FWD2, K_DH1,
+    K_DW2, K_SUM_OVER_T, K_DW1_AGENT, K_DW1_WALLS, K_DW1_GOAL, K_REDUCE_ADAM, K_PACK_GATES, K_PACK_W2, K_HEADS_BWD, K_REPLAY, K_VTRACE, K_COUNT
 };
 
 // Optional per-kernel timing with CUDA events on the launching stream (off by default).
@@ -344,6 +342,7 @@ cudaError_t launch_copy_blocks(void* dst, size_t dpitch, const void* src, size_t
 cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c);
 cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s);  // cudaErrorNotSupported if not covered
 bool rollout_mma_supported(int H);
+bool three_terms(int H, int prec);             // fp32 operands as three bf16 terms instead of two fp16 terms
 bool rollout_uses_fragments(int H, int prec);  // the warp-level kernel (and with it the fragment copies of W2) serves this shape
 cudaError_t launch_rollout_tc128(const RolloutArgs& a, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, fp32, large batches); cudaErrorNotSupported otherwise
 cudaError_t launch_rollout_pair2(const RolloutArgs& a, cudaStream_t s);  // two env groups per CTA pair (H = 256, fp32, large batches); cudaErrorNotSupported otherwise
@@ -354,7 +353,6 @@ size_t wide_scratch_bytes(const Dims& d);     // operands of the base GEMM (kept
 int agent_plane_splits(const Dims& d);
 // agent plane of dW1 (ns partials) and S from the fp32 dh1 rows
 cudaError_t launch_agent_plane(const LearnArgs& a, int ns, float* part, size_t stride, const Ctx& c);
-bool tensor_path_supported(int H, int prec);  // either tensor-core path: the update reuses activations the rollout saved
 cudaError_t launch_rollout_wide(const RolloutArgs& a, const Ctx& c);  // T+1 forward passes, or the replay of recorded rows
 cudaError_t launch_pack_w2_wide(const Dims& d, const Buffers& b, const Ctx& c);
 cudaError_t launch_dh1_wide(const LearnArgs& a, const Ctx& c);
@@ -363,7 +361,6 @@ cudaError_t launch_pack_w2(const Dims& d, const Buffers& b, int prec, const Ctx&
 cudaError_t launch_gae(const Dims& d, const Buffers& b, int T, float gamma, float lambda, const Ctx& c);
 // V-trace scan over the recorded rows: current-policy logits and values from out5, bootstrap values from `boot` [B].
 cudaError_t launch_vtrace(const Dims& d, const Buffers& b, int T, float gamma, float rho_bar, float c_bar, const float* boot, const Ctx& c);
-cudaError_t launch_learn(const LearnArgs& a, int prec, const Ctx& c);
 cudaError_t launch_learn_mma(const LearnArgs& a, int prec, const Ctx& c);
 cudaError_t launch_adam_only(const LearnArgs& a, int prec, const Ctx& c);  // Adam from GRADS as they stand
 constexpr int DH1A_UNITS = 128;  // hidden units (columns of dh1) one CTA of the fused dh1 + agent-plane kernel owns

@@ -92,7 +92,10 @@ struct GemmTcCfg {
     static constexpr bool X3 = PREC == 2 && DEEP;
     static constexpr int GROUP = X3 ? 1 : 64;
     static constexpr int EPI_THREADS = X3 ? 256 : 128;
-    static constexpr int TMEM_COLS = FLUSH ? 2 * BN : BN;
+    // three-term B beside an exact synthesized A: the leading products in one accumulator, the small terms in a second one (every
+    // MMA rounds toward zero at its accumulator's magnitude), added at the end
+    static constexpr bool SPLIT = PREC == 2 && !DEEP;
+    static constexpr int TMEM_COLS = FLUSH || SPLIT ? 2 * BN : BN;
 };
 
 struct GemmTcMaps {
@@ -190,8 +193,11 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
                     const uint64_t b_hi = tc::umma_desc(sb + k16 * 2048, Cfg::BOX, 1024);
                     uint32_t accum = (cg > 0 || k16 > 0) ? 1u : 0u;
                     if (APL == 2) { tc::umma(acc, tc::umma_desc(sa + Cfg::A_PLANE + k16 * 2048, Cfg::BOX, 1024), b_hi, idesc, accum); accum = 1u; }
-                    if (BPL == 3) { tc::umma(acc, a_hi, tc::umma_desc(sb + 2 * Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
-                    if (BPL >= 2) { tc::umma(acc, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
+                    if (Cfg::SPLIT) {
+                        tc::umma(acc + BN, a_hi, tc::umma_desc(sb + 2 * Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum);
+                        tc::umma(acc + BN, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, 1u);
+                    }
+                    if (BPL == 2) { tc::umma(acc, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
                     tc::umma(acc, a_hi, b_hi, idesc, accum);
                 }
                 tc::umma_commit(&bars[STAGES + s]);  // frees the stage when these MMAs are done
@@ -301,6 +307,12 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
                 uint32_t r[32];
                 if (ngroups > 0 && got) {
                     tc::tmem_ld32(acc + (uint32_t)c0, r);
+                    if constexpr (Cfg::SPLIT) {
+                        uint32_t r2[32];
+                        tc::tmem_ld32(acc + (uint32_t)(BN + c0), r2);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
+                    }
                 } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) r[j] = 0u;  // an empty K range contributes zeros
@@ -382,12 +394,16 @@ static cudaError_t launch_bn(const GemmTnArgs& g, int amode, int bpl, int splits
 // one-hot A, operand planes as the fp32 workloads (hi+lo fp16; prec 2: three bf16 terms) or the bf16 workload (one plane) use them.
 cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int apl, int bpl, int prec, int splits, int* status, cudaStream_t s) {
     const int pl = prec == 1 ? 1 : prec == 2 ? 3 : 2;
-    if (g.N != g.ldb || g.N % 64 != 0 || g.klen % 64 != 0 || (bpl != pl && !(prec == 1 && bpl == 2 && amode != A_PLANES)) ||
-        (amode == A_PLANES && (apl != pl || g.lda % 64 != 0)))
+    if (g.N != g.ldb || g.N % (prec == 2 ? 32 : 64) != 0 || g.klen % 64 != 0 || (bpl != pl && !(prec == 1 && bpl == 2 && amode != A_PLANES)) ||
+        (amode == A_PLANES && (apl != pl || g.lda % (prec == 2 ? 32 : 64) != 0)))
         return cudaErrorNotSupported;
     if (amode != A_PLANES && apl != 1) return cudaErrorNotSupported;
     const int bn = g.N > 256 ? 256 : g.N;
-    if (prec == 2) return bn == 256 ? launch_bn<256, 2>(g, amode, bpl, splits, status, s) : cudaErrorNotSupported;
+    if (prec == 2) {  // (columns past N read as zeros and are not stored)
+        if (bn > 128) return launch_bn<256, 2>(g, amode, bpl, splits, status, s);
+        if (bn > 64) return launch_bn<128, 2>(g, amode, bpl, splits, status, s);
+        return launch_bn<64, 2>(g, amode, bpl, splits, status, s);
+    }
     if (prec == 1) {
         switch (bn) {
             case 64: return launch_bn<64, 1>(g, amode, bpl, splits, status, s);

@@ -675,13 +675,14 @@ __global__ void __launch_bounds__(512, 2) k_heads_bwd_tc(LearnArgs a) {
 
 // ----------------------------------------------------------------------------------------------------
 // k_dh1: dh1 = (dh2 W2^T) gated by h1 > 0 on the tensor pipe, and S = sum over t of dh1.
-// A CTA owns 64 envs x BN output columns and walks t = 0..T-1.  Its slice of W2 (BN rows, all K, hi and lo planes)
-// stays in shared memory for the whole kernel; the dh2 planes stream through a cp.async ring in 64-wide k chunks
+// A CTA owns 64 envs x BN output columns and walks its slice of the steps (grid.y = column tile + tiles * slice; S then has one
+// row per slice and env: 64 envs on one CTA took 28 us for 16 steps, four slices take 9).  Its slice of W2 (BN rows, all K, hi
+// and lo planes) stays in shared memory for the whole kernel; the dh2 planes stream through a cp.async ring in 64-wide k chunks
 // that runs across the t boundaries without draining.
 // ----------------------------------------------------------------------------------------------------
 template <int H, int BN, int PREC>
 struct Dh1Cfg {
-    static constexpr int BM = 64, KC = 64, STAGES = 4;
+    static constexpr int BM = 64, KC = H % 64 == 0 ? 64 : 32, STAGES = 4;
     static constexpr int PL = PREC == 1 ? 1 : 2;
     static constexpr int LDW = H + 8;     // 16-bit pitch of the resident W2 planes
     static constexpr int LDA = KC + 8;    // 16-bit pitch of an A chunk
@@ -711,7 +712,8 @@ __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnAr
     const int wm = wid / Cfg::WARPS_N, wn = wid % Cfg::WARPS_N;
     const int g = lane >> 2, t4 = lane & 3;
     const int B = d.B, T = a.T;
-    const int e0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+    const int slice = (int)blockIdx.y / (H / BN), t_len = (T + a.ts - 1) / a.ts, t_beg = slice * t_len;
+    const int e0 = blockIdx.x * BM, n0 = ((int)blockIdx.y % (H / BN)) * BN;
     const size_t RH = (size_t)B * d.Tmax * H;
     const uint16_t* g_dh2hi = reinterpret_cast<const uint16_t*>(b.dh2);
     const uint16_t* g_h1hi = reinterpret_cast<const uint16_t*>(b.h1);
@@ -725,9 +727,9 @@ __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnAr
     }
     cp_async_commit();
 
-    const int nchunks = T * NCH;
+    const int nchunks = t_beg < T ? min(t_len, T - t_beg) * NCH : 0;
     auto issue = [&](int c, int stage) {
-        const int t = c / NCH, k0 = (c - t * NCH) * KC;
+        const int t = t_beg + c / NCH, k0 = (c % NCH) * KC;
         uint16_t* a_s = sA + stage * Cfg::A_STAGE;
         for (int q = tid; q < BM * (KC / 8); q += NTH) {
             const int r = q / (KC / 8), k = 8 * (q - r * (KC / 8));
@@ -754,7 +756,7 @@ __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnAr
     const int jm = lane >> 3, r8 = lane & 7;
 
     for (int c = 0; c < nchunks; ++c) {
-        const int t = c / NCH, kc = c - t * NCH;
+        const int t = t_beg + c / NCH, kc = c % NCH;
         cp_async_wait<STAGES - 2>();  // chunk c (and, the first time, the W2 slice) has landed
         __syncthreads();
         {
@@ -831,8 +833,9 @@ __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnAr
     }
     cp_async_wait<0>();
     // S (sum over t of dh1) as two 16-bit planes [B][H]: S is an fp32 sum, so it keeps two terms in either workload
-    uint16_t* S_hi = reinterpret_cast<uint16_t*>(b.S);
-    uint16_t* S_lo = S_hi + (size_t)B * H;
+    // (row slice * B + env of each plane)
+    uint16_t* S_hi = reinterpret_cast<uint16_t*>(b.S) + (size_t)slice * B * H;
+    uint16_t* S_lo = S_hi + (size_t)a.ts * B * H;
 #pragma unroll
     for (int i = 0; i < MT; ++i)
 #pragma unroll
@@ -929,14 +932,14 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
                 const int k = k0 + kk;
                 uint32_t w[4] = {0u, 0u, 0u, 0u};
                 if (k < kend) {
+                    // the chunk's eight cells are one byte of the env's wall mask
+                    const int m = m0 + mm;
+                    uint32_t bits = (m >> 5) < g.W ? (g.walls[(size_t)(g.kmod ? k % g.kmod : k) * g.W + (m >> 5)] >> (m & 31)) & 0xFFu : 0u;
+                    const int r1 = g.ones_row - m;  // position of the ones row in this chunk
+                    if (r1 < 8) bits = r1 <= 0 ? 0u : bits & ((1u << r1) - 1u);
+                    if (r1 >= 0 && r1 < 8) bits |= 1u << r1;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int m = m0 + mm + q;
-                        bool on = false;
-                        if (m < g.ones_row) on = (g.walls[(size_t)(g.kmod ? k % g.kmod : k) * g.W + (m >> 5)] >> (m & 31)) & 1u;
-                        else if (m == g.ones_row) on = true;
-                        if (on) w[q >> 1] |= (q & 1) ? (one16<PREC>() << 16) : one16<PREC>();
-                    }
+                    for (int q = 0; q < 4; ++q) w[q] = ((bits >> (2 * q)) & 1u) * one16<PREC>() | ((bits >> (2 * q + 1)) & 1u) * (one16<PREC>() << 16);
                 }
                 *reinterpret_cast<uint4*>(a_s + kk * LDA + mm) = make_uint4(w[0], w[1], w[2], w[3]);
             }
@@ -1042,6 +1045,10 @@ static cudaError_t launch_gemm_tn(const GemmTnArgs& g, int rows_m, int splits, c
 __device__ __forceinline__ AdamIn adam_load(const LearnArgs& a, size_t i) {
     return AdamIn{a.b.adam_m[i], a.b.adam_v[i], a.b.theta[i]};
 }
+// 16-bit element (k, n) of W2 inside a fragment copy (layout as in k_pack_w2).
+__device__ __forceinline__ size_t frag_index(int k, int n, int H) {
+    return ((size_t)((k >> 4) * (H / 8) + (n >> 3)) * 32 + (n & 7) * 4 + ((k & 7) >> 1)) * 4 + ((k & 15) >> 3) * 2 + (k & 1);
+}
 template <int PREC>
 __device__ __forceinline__ void adam_step(const LearnArgs& a, size_t i, float g, const AdamIn& in) {
     const Dims& d = a.d;
@@ -1067,12 +1074,18 @@ __device__ __forceinline__ void adam_step(const LearnArgs& a, size_t i, float g,
             const size_t n2 = (size_t)H * H;
 #pragma unroll
             for (int p = 0; p < 3; ++p) b.w2p_hi[p * n2 + (i - d.oW2)] = (uint16_t)tm[p];
+            if (b.w2f_hi) {
+                const size_t ef = frag_index(k, n, H);
+                reinterpret_cast<uint16_t*>(b.w2f_hi)[ef] = (uint16_t)tm[0];
+                reinterpret_cast<uint16_t*>(b.w2f_lo)[ef] = (uint16_t)tm[1];
+                reinterpret_cast<uint16_t*>(b.w2f_lo2)[ef] = (uint16_t)tm[2];
+            }
             return;
         }
         uint16_t hi, lo;
         split1<PREC == 1 ? 1 : 0>(thc, hi, lo);
         if (b.w2f_hi) {
-            const size_t ef = ((size_t)((k >> 4) * (H / 8) + (n >> 3)) * 32 + (n & 7) * 4 + ((k & 7) >> 1)) * 4 + ((k & 15) >> 3) * 2 + (k & 1);
+            const size_t ef = frag_index(k, n, H);
             reinterpret_cast<uint16_t*>(b.w2f_hi)[ef] = hi;
             reinterpret_cast<uint16_t*>(b.w2f_lo)[ef] = lo;
         }
@@ -1272,10 +1285,18 @@ static bool heads_fuse_dw2(const Dims& d, size_t R, int heads_grid, int prec) {
     return (d.H == 128 || d.H == 256) && d.npol <= 1 && heads_grid >= 1;
 }
 
+// dW2 with three-term operands: 128 x 128 tiles, one wave of CTAs, ranges of at least 256 rows.
+static int x3_w2_splits(int H, size_t R) {
+    const int tiles = ((H + 127) / 128) * ((H + 127) / 128);
+    size_t ns = 148 / tiles > 0 ? 148 / tiles : 1;
+    const size_t cap = R / 256 > 0 ? R / 256 : 1;
+    return (int)(ns < cap ? ns : cap);
+}
+
 void learn_mma_plan(const Dims& d, LearnPlan* p) {
     const int H = d.H, C = d.C;
     const size_t R = (size_t)d.B * d.Tmax;
-    const int bt = H >= 128 ? 128 : 64;  // gemm tile side
+    const int bt = H == 128 || H >= 256 ? 128 : 64;  // gemm tile side
     int tiles_hh = ((H + bt - 1) / bt) * ((H + bt - 1) / bt);
     const int tiles_ch = ((C + 1 + bt - 1) / bt) * ((H + bt - 1) / bt);
     int tiles_agent = tiles_ch;
@@ -1287,6 +1308,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     p->ns_agent = splits_for((int)R, tiles_agent, 256);
     if (H > 256) {  // the bf16 GEMM CTAs of the wide path take a whole SM each (four 48 KB stages): one wave
         p->ns_w2 = 148 / tiles_hh > 0 ? 148 / tiles_hh : 1;
+    }
+    if (three_terms(H, 0)) {  // (the plan serves both precisions: room for the larger of their partial counts)
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
     }
@@ -1301,7 +1324,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     if (d.npol > 1) hg = (size_t)(2 * HEADS_GRID / d.npol > 0 ? 2 * HEADS_GRID / d.npol : 1);  // many policies: the CTAs of all policies fill the GPU together
     p->heads_grid = (int)(tiles32 < hg ? tiles32 : hg);
     // (the fused heads + dW2 kernel writes one dW2 partial per CTA: room for the larger of the two partial counts)
-    const int w2_slots = heads_fuse_dw2(d, R, p->heads_grid, 1) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;
+    int w2_slots = heads_fuse_dw2(d, R, p->heads_grid, 1) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;
+    if (three_terms(H, 0) && x3_w2_splits(H, R) > w2_slots) w2_slots = x3_w2_splits(H, R);
     p->ns_small = 4 * p->heads_grid;
     p->small_stride = (size_t)6 * H + 8;
     size_t off = 0;
@@ -1357,7 +1381,7 @@ static cudaError_t launch_heads_tc_t(const LearnArgs& a, int grid, cudaStream_t 
 template <int H, int BN, int PREC>
 static cudaError_t launch_dh1_t(const LearnArgs& a, cudaStream_t s) {
     using Cfg = Dh1Cfg<H, BN, PREC>;
-    dim3 grid((a.d.B + Cfg::BM - 1) / Cfg::BM, H / BN);
+    dim3 grid((a.d.B + Cfg::BM - 1) / Cfg::BM, H / BN * a.ts);
     if (a.d.npol > 1) {
         if constexpr (PREC == 0) {
             CK(cudaFuncSetAttribute(k_dh1<H, BN, PREC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes));
@@ -1387,10 +1411,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const bool grouped = d.npol > 1;
     LearnPlan pl;
     learn_mma_plan(d, &pl);
-    if (PREC == 2 && wide) {  // 128 x 128 tiles: one wave of CTAs
-        const int one_wave = 148 / ((H / 128) * (H / 128));
-        pl.ns_w2 = one_wave < 1 ? 1 : one_wave < pl.ns_w2 ? one_wave : pl.ns_w2;
-    }
+    if (PREC == 2) pl.ns_w2 = x3_w2_splits(H, R);
     a.part_small = b.part + pl.off_small;
     a.small_stride = pl.small_stride;
     // parameter regions in flat order: W1 walls | W1 agent | W1 goal | b1 | W2 | b2 | Wh | bh
@@ -1414,6 +1435,11 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
             case 128: if constexpr (PREC != 2) { CK((launch_heads_t<128, 8, PREC>(a, pl.heads_grid, s, fuse_dw2))); break; }
             case 256: if constexpr (PREC != 2) { CK((launch_heads_t<256, 16, PREC>(a, pl.heads_grid, s, fuse_dw2))); break; }
             default:
+                if constexpr (PREC != 0) {
+                    if (H == 32) { CK((launch_heads_t<32, 2, PREC>(a, pl.heads_grid, s))); break; }
+                    if (H == 96) { CK((launch_heads_t<96, 6, PREC>(a, pl.heads_grid, s))); break; }
+                    if (H == 192) { CK((launch_heads_t<192, 12, PREC>(a, pl.heads_grid, s))); break; }
+                }
                 if constexpr (PREC == 2) {  // wide fp32: column slabs; the row warp of each slab takes the softmax again
                     if (H == 384) { CK((launch_heads_t<384, 8, 2, 128>(a, pl.heads_grid, s))); break; }
                     if (H == 512) { CK((launch_heads_t<512, 16, 2, 256>(a, pl.heads_grid, s))); break; }
@@ -1459,9 +1485,9 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         if (ts >= 2) a.ts = ts;
     }
     if (fused_agent) {
-    } else if (wide) {
+    } else if (PREC == 2 || wide) {
         CK(launch_dh1_wide(a, c));
-        if (PREC == 2) {
+        if (PREC == 2) {  // fp32 dh1 rows: the agent plane and S in one pass over them
             a.reg[1].ns = agent_plane_splits(d);
             CK(launch_agent_plane(a, a.reg[1].ns, b.part + pl.off_agent, CH, c));
             fused_agent = true;
@@ -1469,14 +1495,28 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     } else {
         Scope sc(c, K_DH1);
         const cudaError_t etc = grouped ? cudaErrorNotSupported : launch_dh1_tc(a, PREC, s);  // tcgen05 where covered, else the mma.sync kernel
-        if (etc != cudaErrorNotSupported) CK(etc);
-        else a.ts = 1;
-        if constexpr (PREC == 2) return cudaErrorNotSupported;
-        else if (etc == cudaErrorNotSupported) switch (H) {
-            case 64: CK((launch_dh1_t<64, 64, PREC>(a, s))); break;
-            case 128: CK((launch_dh1_t<128, 128, PREC>(a, s))); break;
-            case 256: CK((launch_dh1_t<256, 128, PREC>(a, s))); break;
-            default: return cudaErrorNotSupported;
+        if (etc != cudaErrorNotSupported) {
+            CK(etc);
+        } else if constexpr (PREC == 2) {
+            return cudaErrorNotSupported;
+        } else {
+            const int ctas = ((B + 63) / 64) * (H > 128 ? 2 : 1);  // slices of at least two steps while SMs are without a CTA
+            a.ts = grouped ? 1 : 148 / ctas;
+            if (a.ts > 4) a.ts = 4;
+            if (a.ts > T / 2) a.ts = T / 2;
+            if (a.ts < 1) a.ts = 1;
+            switch (H) {
+                case 64: CK((launch_dh1_t<64, 64, PREC>(a, s))); break;
+                case 128: CK((launch_dh1_t<128, 128, PREC>(a, s))); break;
+                case 256: CK((launch_dh1_t<256, 128, PREC>(a, s))); break;
+                default:
+                    if constexpr (PREC == 1) {
+                        if (H == 32) { CK((launch_dh1_t<32, 32, PREC>(a, s))); break; }
+                        if (H == 96) { CK((launch_dh1_t<96, 96, PREC>(a, s))); break; }
+                        if (H == 192) { CK((launch_dh1_t<192, 96, PREC>(a, s))); break; }
+                    }
+                    return cudaErrorNotSupported;
+            }
         }
     }
     const __nv_bfloat16* h1hi = reinterpret_cast<const __nv_bfloat16*>(b.h1);
@@ -1499,7 +1539,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         if constexpr (PREC == 2 || amode == A_ENV) {
             return cudaErrorNotSupported;
         } else {
-            if (H >= 128) return launch_gemm_tn<128, 128, amode, apl, bpl, PREC>(g, rows_m, splits, s);
+            if (H == 128 || H == 256) return launch_gemm_tn<128, 128, amode, apl, bpl, PREC>(g, rows_m, splits, s);
             return launch_gemm_tn<64, 64, amode, apl, bpl, PREC>(g, rows_m, splits, s);
         }
     };
@@ -1575,14 +1615,14 @@ cudaError_t launch_adam_only(const LearnArgs& a, int prec, const Ctx& c) {
         if (prec == 1) return cudaErrorNotSupported;
         k_adam_only<0, true><<<dim3(nb, a.d.npol), 256, 0, c.s>>>(a);
     } else if (prec == 1) k_adam_only<1, false><<<nb, 256, 0, c.s>>>(a);
-    else if (wide_supported(a.d.H, prec)) k_adam_only<2, false><<<nb, 256, 0, c.s>>>(a);
+    else if (three_terms(a.d.H, prec)) k_adam_only<2, false><<<nb, 256, 0, c.s>>>(a);
     else k_adam_only<0, false><<<nb, 256, 0, c.s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_learn_mma(const LearnArgs& a, int prec, const Ctx& c) {
     if (prec == 1) return launch_learn_mma_p<1>(a, c);
-    return wide_supported(a.d.H, prec) ? launch_learn_mma_p<2>(a, c) : launch_learn_mma_p<0>(a, c);
+    return three_terms(a.d.H, prec) ? launch_learn_mma_p<2>(a, c) : launch_learn_mma_p<0>(a, c);
 }
 
 }  // namespace anakin

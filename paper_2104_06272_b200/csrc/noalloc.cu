@@ -91,7 +91,12 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
     b.tlogp = dev_traj_logp;
     b.base = reinterpret_cast<float*>(scratch);
     unsigned char* frag = scratch + kMaxBaseFloats * sizeof(float);
-    if (rollout_mma_supported(cfg->H)) {  // same kernel choice as the handle-based rollout
+    if (rollout_mma_supported(cfg->H) && three_terms(cfg->H, cfg->precision)) {  // three fragment planes (H <= 192: 216 KiB)
+        const size_t plane = (size_t)cfg->H * cfg->H * 2;
+        b.w2f_hi = reinterpret_cast<uint2*>(frag);
+        b.w2f_lo = reinterpret_cast<uint2*>(frag + plane);
+        b.w2f_lo2 = reinterpret_cast<uint2*>(frag + 2 * plane);
+    } else if (rollout_mma_supported(cfg->H)) {  // same kernel choice as the handle-based rollout
         if (rollout_uses_fragments(cfg->H, cfg->precision)) {
             b.w2f_hi = reinterpret_cast<uint2*>(frag);
             b.w2f_lo = reinterpret_cast<uint2*>(frag + kW2FragBytes / 2);

@@ -65,12 +65,13 @@ cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c) {
 }
 
 // ----------------------------------------------------------------------------------------------------
-// Persistent rollout.  256 threads = 8 warps; H = 32*HJ hidden units; ME = 8*RR envs per CTA.
+// Persistent FFMA rollout: the wide hidden layers (above 256) of callers without a workspace, whose fixed scratch has no room for
+// the tensor-core path's operands.  256 threads = 8 warps; H = 32*HJ hidden units; ME = 8*RR envs per CTA.
 // Per step: h1 = relu(base + W1[agent row]) -> h2 = relu(h1 W2 + b2) (register-tiled FFMA, W2 streamed through
 // L1/L2) -> 5 head outputs by warp reduction -> one thread per env: softmax, inverse-CDF sample with the
 // Philox uniform of (env, global step), env step, coalesced time-major stores.
 // ----------------------------------------------------------------------------------------------------
-template <int HJ, int RR, int PREC>
+template <int HJ, int RR>
 __global__ void __launch_bounds__(256) k_rollout(RolloutArgs a) {
     constexpr int H = 32 * HJ, ME = 8 * RR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(256) k_rollout(RolloutArgs a) {
         for (int idx = tid; idx < ME * H; idx += 256) {
             const int e = idx / H, j = idx - e * H;
             const float z = s_base[idx] + W1[(size_t)(C + s_pos[e]) * H + j];
-            s_h1[idx] = rnd<PREC>(fmaxf(z, 0.f));
+            s_h1[idx] = (fmaxf(z, 0.f));
         }
         __syncthreads();
         // ---- layer 2: thread (wid, lane) owns rows wid+8*rr and columns lane+32*jj
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(256) k_rollout(RolloutArgs a) {
                 const float bias = __ldg(b2 + lane + 32 * jj);
 #pragma unroll
                 for (int rr = 0; rr < RR; ++rr)
-                    s_h2[(wid + 8 * rr) * H + lane + 32 * jj] = rnd<PREC>(fmaxf(acc[rr][jj] + bias, 0.f));
+                    s_h2[(wid + 8 * rr) * H + lane + 32 * jj] = (fmaxf(acc[rr][jj] + bias, 0.f));
             }
         }
         __syncthreads();
@@ -223,39 +224,27 @@ __global__ void __launch_bounds__(256) k_rollout(RolloutArgs a) {
     }
 }
 
-template <int HJ, int RR, int PREC>
+template <int HJ, int RR>
 static cudaError_t launch_rollout_t(const RolloutArgs& a, cudaStream_t s) {
     constexpr int H = 32 * HJ, ME = 8 * RR;
     const size_t smem = (size_t)(3 * ME * H + ME * 8) * sizeof(float) + ME * 8 * sizeof(uint32_t) + ME * sizeof(int);
-    cudaError_t e = cudaFuncSetAttribute(k_rollout<HJ, RR, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_rollout<HJ, RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_rollout<HJ, RR, PREC><<<(a.d.B + ME - 1) / ME, 256, smem, s>>>(a);
+    k_rollout<HJ, RR><<<(a.d.B + ME - 1) / ME, 256, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int PREC>
-static cudaError_t launch_rollout_p(const RolloutArgs& a, cudaStream_t s) {
+cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
+    if (wide_supported(a.d.H, prec) && a.b.w2p_hi) return launch_rollout_wide(a, c);  // two launches per step
+    Scope sc(c, K_ROLLOUT);
+    if (rollout_mma_supported(a.d.H)) return launch_rollout_mma(a, prec, c.s);
     switch (a.d.H / 32) {
-        case 1: return launch_rollout_t<1, 4, PREC>(a, s);
-        case 2: return launch_rollout_t<2, 4, PREC>(a, s);
-        case 3: return launch_rollout_t<3, 4, PREC>(a, s);
-        case 4: return launch_rollout_t<4, 4, PREC>(a, s);
-        case 6: return launch_rollout_t<6, 4, PREC>(a, s);
-        case 8: return launch_rollout_t<8, 4, PREC>(a, s);
-        case 12: return launch_rollout_t<12, 4, PREC>(a, s);
-        case 16: return launch_rollout_t<16, 2, PREC>(a, s);
-        case 24: return launch_rollout_t<24, 2, PREC>(a, s);
-        case 32: return launch_rollout_t<32, 2, PREC>(a, s);
+        case 12: return launch_rollout_t<12, 4>(a, c.s);
+        case 16: return launch_rollout_t<16, 2>(a, c.s);
+        case 24: return launch_rollout_t<24, 2>(a, c.s);
+        case 32: return launch_rollout_t<32, 2>(a, c.s);
         default: return cudaErrorInvalidValue;
     }
-}
-
-cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
-    if (wide_supported(a.d.H, prec) && a.b.w2p_hi) return launch_rollout_wide(a, c);  // three launches per step
-    Scope sc(c, K_ROLLOUT);
-    const cudaError_t e = launch_rollout_mma(a, prec, c.s);  // tensor-pipe kernel where the shape is covered
-    if (e != cudaErrorNotSupported) return e;
-    return prec == 1 ? launch_rollout_p<1>(a, c.s) : launch_rollout_p<0>(a, c.s);
 }
 
 // ----------------------------------------------------------------------------------------------------

@@ -31,18 +31,35 @@ __global__ void __launch_bounds__(256) k_pack_w2(DimsBuffers in) {
     const float* W2 = b.theta_c + d.oW2;
     if (b.w2f_hi) {
         const int ks4[4] = {k0, k0 + 1, k0 + 8, k0 + 9};
-        uint2 hi, lo;
-        split2<PREC>(W2[(size_t)ks4[0] * H + n], W2[(size_t)ks4[1] * H + n], hi.x, lo.x);
-        split2<PREC>(W2[(size_t)ks4[2] * H + n], W2[(size_t)ks4[3] * H + n], hi.y, lo.y);
-        b.w2f_hi[idx] = hi;
-        b.w2f_lo[idx] = lo;
+        if constexpr (PREC == 2) {
+            uint32_t x[3], y[3];
+            split3(W2[(size_t)ks4[0] * H + n], W2[(size_t)ks4[1] * H + n], x);
+            split3(W2[(size_t)ks4[2] * H + n], W2[(size_t)ks4[3] * H + n], y);
+            b.w2f_hi[idx] = make_uint2(x[0], y[0]);
+            b.w2f_lo[idx] = make_uint2(x[1], y[1]);
+            b.w2f_lo2[idx] = make_uint2(x[2], y[2]);
+        } else {
+            uint2 hi, lo;
+            split2<PREC>(W2[(size_t)ks4[0] * H + n], W2[(size_t)ks4[1] * H + n], hi.x, lo.x);
+            split2<PREC>(W2[(size_t)ks4[2] * H + n], W2[(size_t)ks4[3] * H + n], hi.y, lo.y);
+            b.w2f_hi[idx] = hi;
+            b.w2f_lo[idx] = lo;
+        }
     }
     // and W2 itself as row-major hi / lo planes: this thread covers elements 4*idx .. 4*idx+3
-    if (!b.w2p_hi || !b.w2p_lo) return;
+    if (!b.w2p_hi || (PREC != 2 && !b.w2p_lo)) return;
+    if constexpr (PREC == 2) {  // three planes one after the other
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            uint32_t tm[3];
+            split3(W2[(size_t)4 * idx + 2 * q], W2[(size_t)4 * idx + 2 * q + 1], tm);
+            for (int p = 0; p < 3; ++p) reinterpret_cast<uint32_t*>(b.w2p_hi + (size_t)p * H * H)[2 * idx + q] = tm[p];
+        }
+    } else
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         uint16_t h16, l16;
-        split1<PREC>(W2[(size_t)4 * idx + q], h16, l16);
+        split1<PREC == 1 ? 1 : 0>(W2[(size_t)4 * idx + q], h16, l16);
         b.w2p_hi[(size_t)4 * idx + q] = h16;
         b.w2p_lo[(size_t)4 * idx + q] = l16;
     }
@@ -56,6 +73,7 @@ cudaError_t launch_pack_w2(const Dims& d, const Buffers& b, int prec, const Ctx&
         if (prec == 1) return cudaErrorNotSupported;
         k_pack_w2<0, true><<<dim3(nb, d.npol), 256, 0, c.s>>>(DimsBuffers{d, b});
     } else if (prec == 1) k_pack_w2<1, false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
+    else if (three_terms(d.H, prec)) k_pack_w2<2, false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
     else k_pack_w2<0, false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
     return cudaGetLastError();
 }
@@ -67,9 +85,10 @@ struct RolloutMmaCfg {
     static constexpr int NT = NC / 8;        // n8 tiles per warp
     static constexpr int KS = H / 16;        // k16 steps
     static constexpr int LD = H + 8;         // bf16 row pitch of the h1 planes (16-byte skew: conflict-free ldmatrix)
-    static constexpr int PLANES = PREC == 1 ? 1 : 2;
+    static constexpr int PLANES = PREC == 1 ? 1 : PREC == 2 ? 3 : 2;
+    static constexpr int WSM = PREC == 2 ? 2 : 1;  // planes of W2 fragments in shared memory (the last plane: registers)
     static constexpr size_t smem_bytes =
-        (size_t)H * H * 2                    // W2 hi fragments
+        (size_t)H * H * 2 * WSM              // W2 leading fragments
         + (size_t)ME * H * 4                 // base
         + (size_t)PLANES * ME * LD * 2       // h1 hi (and lo)
         + (size_t)NW * ME * 5 * 4            // per-warp head partials
@@ -88,9 +107,11 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
     constexpr int ME = Cfg::ME, NT = Cfg::NT, KS = Cfg::KS, LD = Cfg::LD, NTHREADS = NW * 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint2* s_w2hi = reinterpret_cast<uint2*>(smem_raw);                        // [KS][H/8][32]
-    float* s_base = reinterpret_cast<float*>(smem_raw + (size_t)H * H * 2);    // [ME][H]
+    uint2* s_w2mid = s_w2hi + (size_t)H * H / 4;                               // (PREC 2) the second terms
+    float* s_base = reinterpret_cast<float*>(smem_raw + (size_t)H * H * 2 * Cfg::WSM);  // [ME][H]
     __nv_bfloat16* s_h1hi = reinterpret_cast<__nv_bfloat16*>(s_base + ME * H); // [ME][LD]
     __nv_bfloat16* s_h1lo = s_h1hi + (PREC == 1 ? 0 : ME * LD);               // [ME][LD] (fp32 workloads only)
+    __nv_bfloat16* s_h1lo2 = s_h1hi + (PREC == 2 ? 2 * ME * LD : 0);           // (PREC 2)
     float* s_red = reinterpret_cast<float*>(s_h1hi + Cfg::PLANES * ME * LD);   // [NW][ME][5]
     float* s_wh = s_red + NW * ME * 5;                                         // [H][5]
     float* s_b2 = s_wh + H * 5;                                                // [H]
@@ -112,6 +133,8 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
     // ---- prologue: weights and per-env constants on chip
     // asynchronous copies: every 16-byte chunk is in flight at once, nothing is staged in registers
     for (int i = tid; i < H * H * 2 / 16; i += NTHREADS) cp_async16(reinterpret_cast<uint4*>(s_w2hi) + i, reinterpret_cast<const uint4*>(b.w2f_hi) + i, 16);
+    if (PREC == 2)
+        for (int i = tid; i < H * H * 2 / 16; i += NTHREADS) cp_async16(reinterpret_cast<uint4*>(s_w2mid) + i, reinterpret_cast<const uint4*>(b.w2f_lo) + i, 16);
     for (int i = tid; i < ME * H / 4; i += NTHREADS) {
         const int e = i / (H / 4), j = 4 * (i - e * (H / 4));
         const bool ok = e0 + e < B;
@@ -122,11 +145,12 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
     for (int i = tid; i < H; i += NTHREADS) s_b2[i] = b.theta_c[d.ob2 + i];
     if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
     uint2 blo[PREC == 1 ? 1 : KS][NT];
-    if (PREC == 0) {
+    if (PREC != 1) {
+        const uint2* last = PREC == 2 ? b.w2f_lo2 : b.w2f_lo;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
 #pragma unroll
-            for (int j = 0; j < NT; ++j) blo[ks][j] = b.w2f_lo[(ks * (H / 8) + wid * NT + j) * 32 + lane];
+            for (int j = 0; j < NT; ++j) blo[ks][j] = last[(ks * (H / 8) + wid * NT + j) * 32 + lane];
     }
     EnvLane s;
     s.pos = s.tep = s.start = s.goal = 0;
@@ -149,9 +173,12 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
 
     // Saved activations (the update reuses the policy's forward pass: Section 3.1): row i = t*B + env.
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
-    __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
-    const int t_end = a.replay == 1 ? a.T - 1 : a.T;  // replay recomputes the T recorded rows (mode 2: and the current state)
-    for (int t = 0; t <= t_end; ++t) {
+    const size_t h1_plane = (size_t)B * d.Tmax * H;
+    // Replay recomputes the T recorded rows (mode 2: and the current state).  Its steps are independent of one another, so a
+    // launch for few envs cuts them into slices (grid.y).
+    const int t_last = a.replay == 1 ? a.T - 1 : a.T, slices = GROUPED ? 1 : (int)gridDim.y, t_len = (t_last + slices) / slices;
+    const int t_beg = GROUPED ? 0 : (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
+    for (int t = t_beg; t <= t_end; ++t) {
         if (a.replay) {  // positions come from the recorded trajectory (row T: the env state as it stands)
             if (tid < ME) s_pos[tid] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + tid] : b.pos[e0 + tid]), C - 1) : 0;
             __syncthreads();
@@ -178,18 +205,33 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
                 const int e = p / (H / 8), k = 8 * (p - e * (H / 8));
                 const float4 b0 = *reinterpret_cast<const float4*>(s_base + e * H + k);
                 const float4 b1 = *reinterpret_cast<const float4*>(s_base + e * H + k + 4);
-                uint4 hi, lo;
-                split2<PREC>(fmaxf(b0.x + w[i][0].x, 0.f), fmaxf(b0.y + w[i][0].y, 0.f), hi.x, lo.x);
-                split2<PREC>(fmaxf(b0.z + w[i][0].z, 0.f), fmaxf(b0.w + w[i][0].w, 0.f), hi.y, lo.y);
-                split2<PREC>(fmaxf(b1.x + w[i][1].x, 0.f), fmaxf(b1.y + w[i][1].y, 0.f), hi.z, lo.z);
-                split2<PREC>(fmaxf(b1.z + w[i][1].z, 0.f), fmaxf(b1.w + w[i][1].w, 0.f), hi.w, lo.w);
-                if (PREC == 0) *reinterpret_cast<uint4*>(s_h1lo + e * LD + k) = lo;
-                *reinterpret_cast<uint4*>(s_h1hi + e * LD + k) = hi;
-                if (save_h1 && e0 + e < B) {
-                    const size_t gi = ((size_t)t * B + e0 + e) * H + k;
-                    *reinterpret_cast<uint4*>(g_h1hi + gi) = hi;
-                    if (PREC == 0) *reinterpret_cast<uint4*>(g_h1lo + gi) = lo;
-                    if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi);  // the gates of these eight units
+                const bool save = save_h1 && e0 + e < B;
+                const size_t gi = ((size_t)t * B + e0 + e) * H + k;
+                if constexpr (PREC == 2) {
+                    uint32_t x[4][3];
+                    split3(fmaxf(b0.x + w[i][0].x, 0.f), fmaxf(b0.y + w[i][0].y, 0.f), x[0]);
+                    split3(fmaxf(b0.z + w[i][0].z, 0.f), fmaxf(b0.w + w[i][0].w, 0.f), x[1]);
+                    split3(fmaxf(b1.x + w[i][1].x, 0.f), fmaxf(b1.y + w[i][1].y, 0.f), x[2]);
+                    split3(fmaxf(b1.z + w[i][1].z, 0.f), fmaxf(b1.w + w[i][1].w, 0.f), x[3]);
+#pragma unroll
+                    for (int p3 = 0; p3 < 3; ++p3) {
+                        const uint4 v = make_uint4(x[0][p3], x[1][p3], x[2][p3], x[3][p3]);
+                        *reinterpret_cast<uint4*>(s_h1hi + p3 * ME * LD + e * LD + k) = v;
+                        if (save) *reinterpret_cast<uint4*>(g_h1hi + p3 * h1_plane + gi) = v;
+                    }
+                } else {
+                    uint4 hi, lo;
+                    split2<PREC>(fmaxf(b0.x + w[i][0].x, 0.f), fmaxf(b0.y + w[i][0].y, 0.f), hi.x, lo.x);
+                    split2<PREC>(fmaxf(b0.z + w[i][0].z, 0.f), fmaxf(b0.w + w[i][0].w, 0.f), hi.y, lo.y);
+                    split2<PREC>(fmaxf(b1.x + w[i][1].x, 0.f), fmaxf(b1.y + w[i][1].y, 0.f), hi.z, lo.z);
+                    split2<PREC>(fmaxf(b1.z + w[i][1].z, 0.f), fmaxf(b1.w + w[i][1].w, 0.f), hi.w, lo.w);
+                    if (PREC == 0) *reinterpret_cast<uint4*>(s_h1lo + e * LD + k) = lo;
+                    *reinterpret_cast<uint4*>(s_h1hi + e * LD + k) = hi;
+                    if (save) {
+                        *reinterpret_cast<uint4*>(g_h1hi + gi) = hi;
+                        if (PREC == 0) *reinterpret_cast<uint4*>(g_h1hi + h1_plane + gi) = lo;
+                        if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi);  // the gates of these eight units
+                    }
                 }
             }
         }
@@ -211,20 +253,41 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
 #pragma unroll
                 for (int q = 0; q < 4; ++q) acc[mt][j][q] = 0.f;
         {
+            // PREC 2: the leading products and the others in accumulators of their own (the tensor core rounds toward zero
+            // at every MMA: the small terms do that at their own magnitude)
+            float accx[PREC == 2 ? 2 : 1][PREC == 2 ? NT : 1][4];
+            if (PREC == 2) {
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) accx[mt][j][q] = 0.f;
+            }
             const int arow = (lane & 7) + ((lane >> 3) & 1) * 8, acol = (lane >> 4) * 8;
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks) {
-                uint32_t ahi[2][4], alo[2][4];
+                uint32_t ahi[2][4], alo[2][4], alo2[2][4];
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt) {
                     ldmatrix_x4(ahi[mt], s_h1hi + (16 * mt + arow) * LD + 16 * ks + acol);
-                    if (PREC == 0) ldmatrix_x4(alo[mt], s_h1lo + (16 * mt + arow) * LD + 16 * ks + acol);
+                    if (PREC != 1) ldmatrix_x4(alo[mt], s_h1lo + (16 * mt + arow) * LD + 16 * ks + acol);
+                    if (PREC == 2) ldmatrix_x4(alo2[mt], s_h1lo2 + (16 * mt + arow) * LD + 16 * ks + acol);
                 }
 #pragma unroll
                 for (int j = 0; j < NT; ++j) {
                     const uint2 bhi = s_w2hi[(ks * (H / 8) + wid * NT + j) * 32 + lane];
+                    uint2 bmid = make_uint2(0u, 0u);
+                    if (PREC == 2) bmid = s_w2mid[(ks * (H / 8) + wid * NT + j) * 32 + lane];
 #pragma unroll
                     for (int mt = 0; mt < 2; ++mt) {
+                        if (PREC == 2) {
+                            mma16816<PREC>(accx[mt][j], alo2[mt], bhi.x, bhi.y);
+                            mma16816<PREC>(accx[mt][j], ahi[mt], blo[ks][j].x, blo[ks][j].y);
+                            mma16816<PREC>(accx[mt][j], alo[mt], bmid.x, bmid.y);
+                            mma16816<PREC>(accx[mt][j], alo[mt], bhi.x, bhi.y);
+                            mma16816<PREC>(accx[mt][j], ahi[mt], bmid.x, bmid.y);
+                        }
                         if (PREC == 0) {
                             mma16816<PREC>(acc[mt][j], alo[mt], bhi.x, bhi.y);
                             mma16816<PREC>(acc[mt][j], ahi[mt], blo[ks][j].x, blo[ks][j].y);
@@ -232,6 +295,14 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
                         mma16816<PREC>(acc[mt][j], ahi[mt], bhi.x, bhi.y);
                     }
                 }
+            }
+            if (PREC == 2) {
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) acc[mt][j][q] += accx[mt][j][q];
             }
         }
         // ---- epilogue: bias, ReLU, head partials over this warp's columns
@@ -359,12 +430,22 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
     }
     cudaError_t e = cudaFuncSetAttribute(k_rollout_mma<H, NW, PREC, GROUPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM);
     if (e != cudaSuccess) return e;
-    const dim3 grid((a.d.B + Cfg::ME - 1) / Cfg::ME, GROUPED ? a.d.npol : 1);
+    const int ctas = (a.d.B + Cfg::ME - 1) / Cfg::ME;
+    int slices = 1;
+    if (a.replay && !GROUPED) {  // independent steps: enough CTAs for every SM (two per SM up to H = 128), at least two steps each
+        const int want = (H <= 128 ? 2 : 1) * 148, steps = a.T + (a.replay == 2 ? 1 : 0);
+        slices = (want + ctas - 1) / ctas;
+        if (slices > (steps + 1) / 2) slices = (steps + 1) / 2;
+    }
+    const dim3 grid(ctas, GROUPED ? a.d.npol : slices);
     k_rollout_mma<H, NW, PREC, GROUPED><<<grid, NW * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-bool rollout_mma_supported(int H) { return H == 64 || H == 128 || H == 256; }
+// Hidden widths whose second-layer weights fit on chip beside a CTA's activations.
+bool rollout_mma_supported(int H) { return H == 32 || H == 64 || H == 96 || H == 128 || H == 192 || H == 256; }
+// fp32 operands as three exact bf16 terms (the widths beside 64, 128 and 256, which take two fp16 terms).
+bool three_terms(int H, int prec) { return prec == 0 && !(H == 64 || H == 128 || H == 256); }
 // fp32 at H = 256 runs the CTA-pair tcgen05 kernel, which reads the row-major planes of W2 only.
 bool rollout_uses_fragments(int H, int prec) { return rollout_mma_supported(H) && !(H == 256 && prec == 0); }
 
@@ -391,14 +472,20 @@ cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s) {
     }
     if (prec == 1) {
         switch (a.d.H) {
+            case 32: return launch_t<32, 2, 1>(a, s);
             case 64: return launch_t<64, 4, 1>(a, s);
+            case 96: return launch_t<96, 6, 1>(a, s);
             case 128: return launch_t<128, 8, 1>(a, s);
+            case 192: return launch_t<192, 12, 1>(a, s);
             case 256: return launch_t<256, 16, 1>(a, s);
         }
     } else {
         switch (a.d.H) {
+            case 32: return launch_t<32, 2, 2>(a, s);
             case 64: return launch_t<64, 4, 0>(a, s);
+            case 96: return launch_t<96, 6, 2>(a, s);
             case 128: return launch_t<128, 8, 0>(a, s);
+            case 192: return launch_t<192, 12, 2>(a, s);
         }
     }
     return cudaErrorNotSupported;

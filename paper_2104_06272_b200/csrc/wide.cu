@@ -24,7 +24,6 @@ namespace anakin {
 
 // Hidden layers too wide for the persistent rollouts, in either precision (bf16 at 512 / 1024 is the headline form).
 bool wide_supported(int H, int prec) { (void)prec; return H == 384 || H == 512 || H == 768 || H == 1024; }
-bool tensor_path_supported(int H, int prec) { return rollout_mma_supported(H) || wide_supported(H, prec); }
 
 namespace {
 
@@ -598,7 +597,7 @@ static cudaError_t dh1_wide_t(const LearnArgs& a, const Ctx& c) {
     const Dims& d = a.d;
     const Buffers& b = a.b;
     const int H = d.H;
-    const size_t R = (size_t)d.B * a.T, plane = (size_t)d.B * d.Tmax;
+    const size_t R = (size_t)d.B * a.T, plane = (size_t)d.B * d.Tmax;  // (dh2 planes)
     if constexpr (F32) {
         Scope sc(c, K_DH1);
         X3Args g;

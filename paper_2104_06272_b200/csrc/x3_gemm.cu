@@ -53,7 +53,7 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
     const int rank = PAIR ? (int)tc::cluster_ctarank() : 0;
     const bool leader = rank == 0;
     const int unit = PAIR ? blockIdx.x >> 1 : blockIdx.x, units = PAIR ? gridDim.x >> 1 : gridDim.x;
-    const int nt = (g.N + BN - 1) / BN, mt = (g.M + PM - 1) / PM, ntiles = mt * nt, nkc = g.K / KC;
+    const int nt = (g.N + BN - 1) / BN, mt = (g.M + PM - 1) / PM, ntiles = mt * nt, nkc = (g.K + KC - 1) / KC;  // (columns of A past K read as zeros)
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); }
@@ -194,7 +194,7 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
             if (EPI == EPI_GATE) load_gates(0);
 #pragma unroll
             for (int c0 = 0; c0 < COLS; c0 += 16) {
-                if (n0 + c0 < g.N) {  // (the matrix's width is a multiple of 64)
+                if (n0 + c0 < g.N) {  // (the matrix's width is a multiple of 32)
 #pragma unroll
                     for (int ch = 0; ch < 4; ++ch)
                         *reinterpret_cast<float4*>(stage + lane * 64 + ((ch ^ ((lane >> 1) & 3)) << 4)) =
@@ -264,13 +264,13 @@ cudaError_t launch_x3_t(const NtMaps& maps, const X3Args& g, int bn, int tiles, 
 
 }  // namespace
 
-// Tile rule: pairs (256 x 256) while more than half of the 74 pairs get a tile; below that 128 x 128 tiles, or 128 x 64 where even
+// Tile rule: no tile more than twice as wide as the matrix; pairs (256 x 256) while more than half of the 74 pairs get a tile; below that 128 x 128 tiles, or 128 x 64 where even
 // those fit one wave (an idle SM costs more than a narrow MMA).
 cudaError_t launch_x3_nt(int epi, const void* a, size_t a_rows_total, const void* b, const X3Args& g, cudaStream_t s) {
-    if (g.N % 64 != 0 || g.K % 64 != 0 || g.N > X3Cfg<true, 256>::MAXN || g.M < 1) return cudaErrorNotSupported;
+    if (g.N % 32 != 0 || g.K % 32 != 0 || g.N > X3Cfg<true, 256>::MAXN || g.M < 1) return cudaErrorNotSupported;
     auto tiles = [&](int bm, int bn) { return ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn); };
     const int np = tiles(256, 256), n128 = tiles(128, 128), n64 = tiles(128, 64);
-    const int bn = np > 37 ? 256 : n64 <= 148 ? 64 : 128, n = bn == 256 ? np : bn == 128 ? n128 : n64;
+    const int bn = g.N <= 64 ? 64 : np > 37 && g.N > 128 ? 256 : n64 <= 148 ? 64 : 128, n = bn == 256 ? np : bn == 128 ? n128 : n64;
     const bool b_mn = epi == EPI_FWD;  // W2 as stored: rows = k for h1 W2, rows = n for dh2 W2^T
     NtMaps maps;
     memset(&maps, 0, sizeof(maps));
