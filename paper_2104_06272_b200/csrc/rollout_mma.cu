@@ -99,12 +99,15 @@ struct RolloutMmaCfg {
     static constexpr size_t gae_bytes(int T) { return (size_t)(T + 1) * ME * 4 + (size_t)T * ME; }
 };
 
-template <int H, int NW, int PREC, bool GROUPED>
-__global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(RolloutArgs a_in) {
+// OWN: the per-env part of a step (one lane per env) has a warp of its own beside the NW workers, which meets them at named
+// barriers: the logits-independent half of an interaction runs under the gather, and the records are written after the workers
+// have been given the new positions.  Otherwise warp 0 does both (the wide kernels' registers leave no room for another warp).
+template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
+__global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(RolloutArgs a_in) {
     const PolicyArgs<GROUPED, RolloutArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
     const RolloutArgs& a = pa.a;
     using Cfg = RolloutMmaCfg<H, NW, PREC>;
-    constexpr int ME = Cfg::ME, NT = Cfg::NT, KS = Cfg::KS, LD = Cfg::LD, NTHREADS = NW * 32;
+    constexpr int ME = Cfg::ME, NT = Cfg::NT, KS = Cfg::KS, LD = Cfg::LD, NTHREADS = NW * 32 /*workers*/, NALL = NTHREADS + (OWN ? 32 : 0);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint2* s_w2hi = reinterpret_cast<uint2*>(smem_raw);                        // [KS][H/8][32]
     uint2* s_w2mid = s_w2hi + (size_t)H * H / 4;                               // (PREC 2) the second terms
@@ -130,22 +133,25 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
     const int B = d.B, C = d.C;
     const float* W1 = b.theta_c + d.oW1;
 
+    const int ow = OWN ? tid - NTHREADS : tid;  // env of this thread (0 .. ME-1: an owner)
+    const bool worker = !OWN || tid < NTHREADS, ownw = ow >= 0 && ow < ME;
+
     // ---- prologue: weights and per-env constants on chip
     // asynchronous copies: every 16-byte chunk is in flight at once, nothing is staged in registers
-    for (int i = tid; i < H * H * 2 / 16; i += NTHREADS) cp_async16(reinterpret_cast<uint4*>(s_w2hi) + i, reinterpret_cast<const uint4*>(b.w2f_hi) + i, 16);
+    for (int i = tid; i < H * H * 2 / 16; i += NALL) cp_async16(reinterpret_cast<uint4*>(s_w2hi) + i, reinterpret_cast<const uint4*>(b.w2f_hi) + i, 16);
     if (PREC == 2)
-        for (int i = tid; i < H * H * 2 / 16; i += NTHREADS) cp_async16(reinterpret_cast<uint4*>(s_w2mid) + i, reinterpret_cast<const uint4*>(b.w2f_lo) + i, 16);
-    for (int i = tid; i < ME * H / 4; i += NTHREADS) {
+        for (int i = tid; i < H * H * 2 / 16; i += NALL) cp_async16(reinterpret_cast<uint4*>(s_w2mid) + i, reinterpret_cast<const uint4*>(b.w2f_lo) + i, 16);
+    for (int i = tid; i < ME * H / 4; i += NALL) {
         const int e = i / (H / 4), j = 4 * (i - e * (H / 4));
         const bool ok = e0 + e < B;
         cp_async16(s_base + e * H + j, b.base + (size_t)(ok ? e0 + e : 0) * H + j, ok ? 16 : 0);
     }
     cp_async_commit();
-    for (int i = tid; i < H * 5; i += NTHREADS) s_wh[i] = b.theta_c[d.oWh + i];
-    for (int i = tid; i < H; i += NTHREADS) s_b2[i] = b.theta_c[d.ob2 + i];
+    for (int i = tid; i < H * 5; i += NALL) s_wh[i] = b.theta_c[d.oWh + i];
+    for (int i = tid; i < H; i += NALL) s_b2[i] = b.theta_c[d.ob2 + i];
     if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
     uint2 blo[PREC == 1 ? 1 : KS][NT];
-    if (PREC != 1) {
+    if (PREC != 1 && worker) {
         const uint2* last = PREC == 2 ? b.w2f_lo2 : b.w2f_lo;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks)
@@ -156,17 +162,17 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
     s.pos = s.tep = s.start = s.goal = 0;
     s.n_episodes = s.n_goals = s.n_epsteps = 0;
     s.bad = 0;
-    const bool owner = tid < ME && e0 + tid < B;
-    if (tid < ME) {
-        for (int wi = 0; wi < 8; ++wi) s_walls[tid * 8 + wi] = (owner && wi < d.W) ? b.walls[(size_t)(e0 + tid) * d.W + wi] : 0u;
+    const bool owner = ownw && e0 + ow < B;
+    if (ownw) {
+        for (int wi = 0; wi < 8; ++wi) s_walls[ow * 8 + wi] = (owner && wi < d.W) ? b.walls[(size_t)(e0 + ow) * d.W + wi] : 0u;
         if (owner) {
-            s.pos = b.pos[e0 + tid];
-            s.tep = b.tep[e0 + tid];
-            s.start = b.start[e0 + tid];
-            s.goal = b.goal[e0 + tid];
-            check_env_state(s, C, s_walls + tid * 8);
+            s.pos = b.pos[e0 + ow];
+            s.tep = b.tep[e0 + ow];
+            s.start = b.start[e0 + ow];
+            s.goal = b.goal[e0 + ow];
+            check_env_state(s, C, s_walls + ow * 8);
         }
-        s_pos[tid] = s.pos;
+        s_pos[ow] = s.pos;
     }
     cp_async_wait<0>();
     __syncthreads();
@@ -178,11 +184,14 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
     // launch for few envs cuts them into slices (grid.y).
     const int t_last = a.replay == 1 ? a.T - 1 : a.T, slices = GROUPED ? 1 : (int)gridDim.y, t_len = (t_last + slices) / slices;
     const int t_beg = GROUPED ? 0 : (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
-    for (int t = t_beg; t <= t_end; ++t) {
-        if (a.replay) {  // positions come from the recorded trajectory (row T: the env state as it stands)
-            if (tid < ME) s_pos[tid] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + tid] : b.pos[e0 + tid]), C - 1) : 0;
-            __syncthreads();
-        }
+    auto recorded_pos = [&](int t) {  // replay: the position of this thread's env at step t (row T: the env state as it stands)
+        return owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
+    };
+    if (a.replay) {
+        if (ownw) s_pos[ow] = recorded_pos(t_beg);
+        __syncthreads();
+    }
+    auto layer1 = [&](int t) {
         // ---- layer 1: eight consecutive hidden units per thread and trip.  All gathers of the agent's W1 row are issued
         // before any is used (one L2 round trip per step, not one per trip); the fp16 planes go to shared memory for
         // the MMAs and, for the update's reuse, straight to global memory (16 bytes per lane).
@@ -235,15 +244,8 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
                 }
             }
         }
-        __syncthreads();
-        // The logits-independent half of the interaction (the Philox uniform, the four candidate cells) is taken by the
-        // owner threads now, under the other warps' tensor work, so that only softmax and selection follow the heads.
-        // It waits in shared memory (two words per env) rather than in registers, which the MMA loop needs.
-        const bool acting = owner && !a.replay && t < a.T;
-        if (acting) {
-            const StepPre pre = step_prepare(s, a, e0 + tid, t, s_walls + tid * 8);
-            s_pre[tid] = make_uint2(__float_as_uint(pre.u), (uint32_t)pre.np[0] | ((uint32_t)pre.np[1] << 8) | ((uint32_t)pre.np[2] << 16) | ((uint32_t)pre.np[3] << 24));
-        }
+    };
+    auto layer2_heads = [&](int t) {
         // ---- layer 2 on the tensor pipe: acc[mt][j] = rows 16mt.. x columns 8(wid*NT+j)..
         float acc[2][NT][4];
 #pragma unroll
@@ -370,18 +372,32 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
                 s_red[(wid * ME + row) * 5 + c] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 2);
             }
         }
-        __syncthreads();
-        // ---- one thread per env: fixed-order sum of the warps' partials, then act and step
+    };
+    // ---- one thread per env: fixed-order sum of the warps' partials, then act and step; `publish` comes between the new
+    // position and the records
+    auto per_env = [&](int t, bool acting, const StepPre& pre, auto&& publish) {
+        float o[5];
+        ActOut ao;
+        ao.la_mx = ao.Z = ao.rew = 0.f;
+        ao.act = ao.done = ao.pos0 = 0;
         if (owner) {
-            float o[5];
 #pragma unroll
             for (int c = 0; c < 5; ++c) o[c] = 0.f;
+#pragma unroll
             for (int w = 0; w < NW; ++w)
 #pragma unroll
-                for (int c = 0; c < 5; ++c) o[c] += s_red[(w * ME + tid) * 5 + c];
+                for (int c = 0; c < 5; ++c) o[c] += s_red[(w * ME + ow) * 5 + c];
 #pragma unroll
             for (int c = 0; c < 5; ++c) o[c] += s_bh[c];
-            const int env = e0 + tid;
+            if (acting) {
+                ao = act_decide(s, a, e0 + ow, t, o[0], o[1], o[2], o[3], pre);
+                s_pos[ow] = s.pos;
+            }
+        }
+        if (a.replay && ownw && t < t_end) s_pos[ow] = recorded_pos(t + 1);
+        publish();
+        if (owner) {
+            const int env = e0 + ow;
             if (b.out5 && t < a.T) {  // the update reuses the head outputs of every recorded row
                 float4* o5 = reinterpret_cast<float4*>(b.out5 + ((size_t)t * B + env) * 8);
                 o5[0] = make_float4(o[0], o[1], o[2], o[3]);
@@ -390,33 +406,81 @@ __global__ void __launch_bounds__(NW * 32, (H <= 128 ? 2 : 1)) k_rollout_mma(Rol
             if (a.replay == 2 && t == a.T) b.vboot[env] = o[4];
             if (!a.replay) {
                 b.tval[(size_t)t * B + env] = o[4];
-                if (a.gae_smem) s_gv[t * ME + tid] = o[4];
+                if (a.gae_smem) s_gv[t * ME + ow] = o[4];
                 if (acting) {
-                    const uint2 pk = s_pre[tid];
-                    StepPre pre;
-                    pre.u = __uint_as_float(pk.x);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) pre.np[q] = (pk.y >> (8 * q)) & 0xFF;
-                    const int code = act_and_step_pre(s, a, env, t, o[0], o[1], o[2], o[3], pre);
-                    if (a.gae_smem) s_gc[t * ME + tid] = (uint8_t)code;
-                    s_pos[tid] = s.pos;
+                    act_record(a, env, t, o[0], o[1], o[2], o[3], ao);
+                    if (a.gae_smem) s_gc[t * ME + ow] = (uint8_t)(ao.done | (ao.rew != 0.f ? 2 : 0));
                 }
             }
         }
-        __syncthreads();
+    };
+    if constexpr (OWN) {
+        // Named barriers: 3 = the workers have written the h1 tile; 2 = head partials written (workers arrive, the owner warp
+        // waits); 1 = positions published and every worker past its reads of the h1 tile (the owner warp arrives).
+        if (worker) {
+            for (int t = t_beg; t <= t_end; ++t) {
+                layer1(t);
+                asm volatile("bar.sync 3, %0;" ::"n"(NTHREADS) : "memory");
+                layer2_heads(t);
+                asm volatile("bar.arrive 2, %0;" ::"n"(NALL) : "memory");
+                asm volatile("bar.sync 1, %0;" ::"n"(NALL) : "memory");
+            }
+        } else {
+            for (int t = t_beg; t <= t_end; ++t) {
+                const bool acting = owner && !a.replay && t < a.T;
+                StepPre pre;
+                if (acting) pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
+                asm volatile("bar.sync 2, %0;" ::"n"(NALL) : "memory");
+                per_env(t, acting, pre, [&]() {
+                    __syncwarp();
+                    asm volatile("bar.arrive 1, %0;" ::"n"(NALL) : "memory");
+                });
+            }
+        }
+    } else {
+        for (int t = t_beg; t <= t_end; ++t) {
+            layer1(t);
+            __syncthreads();
+            // the logits-independent half of the interaction waits in shared memory (two words per env) rather than in
+            // registers, which the MMA loop needs
+            const bool acting = owner && !a.replay && t < a.T;
+            if (acting) {
+                const StepPre pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
+                s_pre[ow] = make_uint2(__float_as_uint(pre.u), (uint32_t)pre.np[0] | ((uint32_t)pre.np[1] << 8) | ((uint32_t)pre.np[2] << 16) | ((uint32_t)pre.np[3] << 24));
+            }
+            layer2_heads(t);
+            __syncthreads();
+            StepPre pre;
+            if (acting) {
+                const uint2 pk = s_pre[ow];
+                pre.u = __uint_as_float(pk.x);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) pre.np[q] = (pk.y >> (8 * q)) & 0xFF;
+            }
+            per_env(t, acting, pre, []() {});
+            __syncthreads();
+        }
     }
     if (a.replay) return;
     if (owner) {
-        b.pos[e0 + tid] = (uint8_t)s.pos;
-        b.tep[e0 + tid] = (uint8_t)s.tep;
+        b.pos[e0 + ow] = (uint8_t)s.pos;
+        b.tep[e0 + ow] = (uint8_t)s.tep;
         // the owner thread wrote this env's rewards, values and done flags itself: it can scan them right away
-        if (a.gae_smem) gae_scan_env_smem(b, B, a.T, e0 + tid, a.gamma, a.lambda, s_gv, s_gc, ME, tid);
-        else if (a.fuse_gae) gae_scan_env(b, B, a.T, e0 + tid, a.gamma, a.lambda);
+        if (a.gae_smem) gae_scan_env_smem(b, B, a.T, e0 + ow, a.gamma, a.lambda, s_gv, s_gc, ME, ow);
+        else if (a.fuse_gae) gae_scan_env(b, B, a.T, e0 + ow, a.gamma, a.lambda);
     }
-    if (tid < 32) flush_env_stats(s, a);
+    if (OWN ? !worker : tid < 32) flush_env_stats(s, a);
 }
 
 constexpr size_t MAX_DYN_SMEM = 232448;  // 227 KB of dynamic shared memory per CTA
+
+template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
+static cudaError_t launch_k(const RolloutArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
+    const cudaError_t e = cudaFuncSetAttribute(k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM);
+    if (e != cudaSuccess) return e;
+    k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN><<<grid, NW * 32 + (OWN ? 32 : 0), smem, s>>>(a);
+    return cudaGetLastError();
+}
 
 template <int H, int NW, int PREC, bool GROUPED = false>
 static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
@@ -428,8 +492,6 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
         a.gae_smem = 1;
         smem += Cfg::gae_bytes(a.T);
     }
-    cudaError_t e = cudaFuncSetAttribute(k_rollout_mma<H, NW, PREC, GROUPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM);
-    if (e != cudaSuccess) return e;
     const int ctas = (a.d.B + Cfg::ME - 1) / Cfg::ME;
     int slices = 1;
     if (a.replay && !GROUPED) {  // independent steps: enough CTAs for every SM (two per SM up to H = 128), at least two steps each
@@ -438,8 +500,15 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
         if (slices > (steps + 1) / 2) slices = (steps + 1) / 2;
     }
     const dim3 grid(ctas, GROUPED ? a.d.npol : slices);
-    k_rollout_mma<H, NW, PREC, GROUPED><<<grid, NW * 32, smem, s>>>(a);
-    return cudaGetLastError();
+    // The owner warp costs a CTA of the 128-wide kernel its second place on an SM: only where every CTA gets an SM of its own.
+    // (H = 64: three CTAs per SM where there are that many)
+    if constexpr (H == 64)
+        if ((size_t)grid.x * grid.y > 296) return launch_k<H, NW, PREC, GROUPED, 3, true>(a, grid, smem, s);
+    if constexpr (H < 128) return launch_k<H, NW, PREC, GROUPED, 2, true>(a, grid, smem, s);
+    else if constexpr (H == 128) {
+        if ((size_t)grid.x * grid.y <= 148) return launch_k<H, NW, PREC, GROUPED, 1, true>(a, grid, smem, s);
+        return launch_k<H, NW, PREC, GROUPED, 2, false>(a, grid, smem, s);
+    } else return launch_k<H, NW, PREC, GROUPED, 1, H == 192>(a, grid, smem, s);
 }
 
 // Hidden widths whose second-layer weights fit on chip beside a CTA's activations.
