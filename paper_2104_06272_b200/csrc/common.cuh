@@ -5,6 +5,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 #include <vector>
 
@@ -334,6 +335,49 @@ __device__ __forceinline__ void select_policy(GemmTnArgs& g, int pol) {
 
 // tcgen05 version (tensor memory accumulators, TMA-fed); cudaErrorNotSupported when the shape is not covered.
 cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int apl, int bpl, int prec, int splits, int* status, cudaStream_t s);
+
+// ---- launches ----
+// Every kernel of the library is launched as a programmatic dependent of the one before it on the stream: its CTAs may be placed,
+// and its set-up may run, while that one drains.  A kernel calls pdl_wait() before it touches anything another kernel reads or
+// writes (all earlier grids have then completed and their writes are visible), and pdl_trigger() where its own successor may
+// be placed.  Launch gaps of the small workloads were 1.3 us each, a fifth of the tiny pass.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// (Not in a GEMM whose CTAs finish unevenly or leave SMs idle: the successor's CTAs would all crowd onto the first free SMs.)
+#define PDL_START() do { anakin::pdl_wait(); anakin::pdl_trigger(); } while (0)
+
+// Launches kernel K.  Its limit of dynamic shared memory is raised to all there is, once per device instead of before every launch.
+template <auto K, class... A>
+inline cudaError_t launch(dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    if (smem > 48 * 1024) {
+        constexpr int MAXDEV = 64;
+        static std::atomic<bool> raised[MAXDEV];  // (zero-initialised)
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev >= MAXDEV || !raised[dev].load(std::memory_order_acquire)) {
+            cudaFuncAttributes fa;
+            e = cudaFuncGetAttributes(&fa, K);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - (int)fa.sharedSizeBytes);
+            if (e != cudaSuccess) return e;
+            if (dev < MAXDEV) raised[dev].store(true, std::memory_order_release);
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, K, args...);
+}
+#endif
 
 // kernels (defined in the .cu files) ----------------------------------------------------------------
 cudaError_t launch_reset(const Dims& d, const Buffers& b, uint64_t seed, double density, int prec, const Ctx& c);

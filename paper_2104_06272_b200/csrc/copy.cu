@@ -9,6 +9,7 @@ namespace anakin {
 // costs 3.5 us on the stream), one launch takes 20 us.
 template <class W>
 __global__ void __launch_bounds__(256) k_copy_blocks(W* dst, size_t dpitch, const W* src, size_t spitch, size_t words, size_t rows) {
+    PDL_START();
     for (size_t r = blockIdx.y; r < rows; r += gridDim.y) {
         const W* s = src + r * spitch;
         W* o = dst + r * dpitch;
@@ -30,8 +31,8 @@ cudaError_t launch_copy_blocks(void* dst, size_t dpitch, const void* src, size_t
     const size_t words = w4 ? bytes / 4 : bytes;
     const size_t gx = (words + 1023) / 1024;
     const dim3 grid((unsigned)(gx < 1024 ? gx : 1024), (unsigned)(rows < 65535 ? rows : 65535));
-    if (w4) k_copy_blocks<uint32_t><<<grid, 256, 0, s>>>((uint32_t*)dst, dpitch / 4, (const uint32_t*)src, spitch / 4, words, rows);
-    else k_copy_blocks<uint8_t><<<grid, 256, 0, s>>>((uint8_t*)dst, dpitch, (const uint8_t*)src, spitch, words, rows);
+    if (w4) launch<k_copy_blocks<uint32_t>>(grid, 256, 0, s, (uint32_t*)dst, dpitch / 4, (const uint32_t*)src, spitch / 4, words, rows);
+    else launch<k_copy_blocks<uint8_t>>(grid, 256, 0, s, (uint8_t*)dst, dpitch, (const uint8_t*)src, spitch, words, rows);
     return cudaGetLastError();
 }
 

@@ -34,6 +34,7 @@ struct Dh1TcMaps {
 
 template <int H, int PREC>
 __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1TcMaps maps, LearnArgs a) {
+    PDL_START();
     using Cfg = Dh1TcCfg<H, PREC>;
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, PL = Cfg::PL, NCH = Cfg::NCH, STAGES = Cfg::STAGES, BOX = Cfg::BOX;
     extern __shared__ unsigned char smem_raw[];
@@ -241,11 +242,8 @@ static cudaError_t launch_t(const LearnArgs& a, cudaStream_t s) {
         if (!make_tensor_map_2d(&maps.a_lo, dh2hi + RH, R, H, 128, bf)) return cudaErrorNotSupported;
         if (!make_tensor_map_2d(&maps.w_lo, b.w2p_lo, H, H, 128, bf)) return cudaErrorNotSupported;
     }
-    cudaError_t e = cudaFuncSetAttribute(k_dh1_tc<H, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-    if (e != cudaSuccess) return e;
     dim3 grid((d.B + Cfg::BM - 1) / Cfg::BM, H / Cfg::BN, a.ts);
-    k_dh1_tc<H, PREC><<<grid, Cfg::THREADS, Cfg::smem_bytes, s>>>(maps, a);
-    return cudaGetLastError();
+    return launch<k_dh1_tc<H, PREC>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, a);
 }
 
 // Covered: H = 128 or 256.  cudaErrorNotSupported otherwise (the caller falls back to the mma.sync kernel).

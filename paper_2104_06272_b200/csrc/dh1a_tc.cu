@@ -473,11 +473,13 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
 template <int H, int PREC>
 __global__ void __launch_bounds__(Dh1aCfg<H, PREC>::THREADS, 1)
     k_dh1a_tc(const __grid_constant__ Dh1aMaps maps, LearnArgs a, float* part_agent, size_t part_stride) {
+    PDL_START();
     dh1a_body<H, PREC>(maps, a, part_agent, part_stride);
 }
 template <int H, int PREC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Dh1aCfg<H, PREC>::THREADS, 1)
     k_dh1a_pair(const __grid_constant__ Dh1aMaps maps, LearnArgs a, float* part_agent, size_t part_stride) {
+    PDL_START();
     dh1a_body<H, PREC>(maps, a, part_agent, part_stride);
 }
 
@@ -497,13 +499,9 @@ cudaError_t launch_t(const LearnArgs& a, int grid_x, float* part_agent, size_t p
     if (!make_tensor_map_2d(&maps.w_hi, b.w2p_hi, H, H, 128, bf)) return cudaErrorNotSupported;
     if (Cfg::PL == 2 && !make_tensor_map_2d(&maps.w_lo, b.w2p_lo, H, H, 128, bf)) return cudaErrorNotSupported;
     if constexpr (Cfg::PAIR) {  // the two CTAs of a pair are neighbours in x; each pair takes all H units
-        cudaError_t e = cudaFuncSetAttribute(k_dh1a_pair<H, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-        if (e != cudaSuccess) return e;
-        k_dh1a_pair<H, PREC><<<dim3(2 * grid_x, 1, a.ts), Cfg::THREADS, Cfg::smem_bytes, s>>>(maps, a, part_agent, part_stride);
+        launch<k_dh1a_pair<H, PREC>>(dim3(2 * grid_x, 1, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
     } else {
-        cudaError_t e = cudaFuncSetAttribute(k_dh1a_tc<H, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-        if (e != cudaSuccess) return e;
-        k_dh1a_tc<H, PREC><<<dim3(grid_x, H / Cfg::BN, a.ts), Cfg::THREADS, Cfg::smem_bytes, s>>>(maps, a, part_agent, part_stride);
+        launch<k_dh1a_tc<H, PREC>>(dim3(grid_x, H / Cfg::BN, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
     }
     return cudaGetLastError();
 }

@@ -24,6 +24,7 @@ int agent_warps(int C) {
 }
 
 __global__ void __launch_bounds__(256) k_agent_plane(LearnArgs a, float* part, size_t stride) {
+    PDL_START();
     extern __shared__ float s_acc[];  // [warps][C + 1][32]
     const Dims& d = a.d;
     const Buffers& b = a.b;
@@ -118,10 +119,7 @@ cudaError_t launch_agent_plane(const LearnArgs& a, int ns, float* part, size_t s
     const int w = agent_warps(a.d.C);
     const size_t smem = (size_t)w * (a.d.C + 1) * 128;
     Scope sc(c, K_DW1_AGENT);
-    const cudaError_t e = cudaFuncSetAttribute(k_agent_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_agent_plane<<<dim3(a.d.H / 32, ns), 32 * w, smem, c.s>>>(a, part, stride);
-    return cudaGetLastError();
+    return launch<k_agent_plane>(dim3(a.d.H / 32, ns), 32 * w, smem, c.s, a, part, stride);
 }
 
 }  // namespace anakin

@@ -46,28 +46,56 @@ EncodeTiledFn encode_fn() {
 
 }  // namespace
 
-bool make_tensor_map_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool bf16) {
+namespace {
+
+// A tensor map is a pure function of these values, and a training loop asks for the same dozen every iteration: each thread keeps
+// the last 64 it encoded (an encode costs about a microsecond of host time, a tenth of tiny's launch work in all).
+struct MapKey {
+    const void* base;
+    uint64_t rows, cols;
+    uint32_t box_rows, box_cols, type;
+    bool operator==(const MapKey& o) const {
+        return base == o.base && rows == o.rows && cols == o.cols && box_rows == o.box_rows && box_cols == o.box_cols && type == o.type;
+    }
+};
+struct MapSlot {
+    MapKey key;
+    CUtensorMap map;
+};
+
+bool encode_cached(CUtensorMap* map, const MapKey& k, CUtensorMapDataType type, uint32_t elem, CUtensorMapSwizzle swizzle) {
+    constexpr int SLOTS = 64;
+    static thread_local MapSlot slots[SLOTS] = {};
+    const uint64_t h = ((uint64_t)(uintptr_t)k.base * 0x9E3779B97F4A7C15ull) ^ (k.rows * 0xC2B2AE3D27D4EB4Full) ^ (k.cols << 7) ^ (k.box_rows << 3) ^ k.type;
+    MapSlot& s = slots[(h ^ (h >> 29)) >> 20 & (SLOTS - 1)];
+    if (s.key == k) { *map = s.map; return true; }
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols * 2};
-    cuuint32_t box[2] = {64, box_rows};
+    cuuint64_t dims[2] = {k.cols, k.rows};
+    cuuint64_t strides[1] = {k.cols * elem};
+    cuuint32_t box[2] = {k.box_cols, k.box_rows};
     cuuint32_t estr[2] = {1, 1};
-    return enc(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    if (enc(&s.map, type, 2, const_cast<void*>(k.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+        s.key = MapKey{};
+        return false;
+    }
+    s.key = k;
+    *map = s.map;
+    return true;
+}
+
+}  // namespace
+
+bool make_tensor_map_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool bf16) {
+    return encode_cached(map, MapKey{base, rows, cols, box_rows, 64, bf16 ? 1u : 0u}, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
+                         CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // The same over a row-major byte matrix [rows][cols] (cols a multiple of 16) with a box of box_cols x box_rows bytes, not swizzled.
 bool make_tensor_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_cols) {
-    EncodeTiledFn enc = encode_fn();
-    if (!enc || cols % 16 != 0 || box_cols % 16 != 0) return false;
-    cuuint64_t dims[2] = {cols, rows};
-    cuuint64_t strides[1] = {cols};
-    cuuint32_t box[2] = {box_cols, box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    if (cols % 16 != 0 || box_cols % 16 != 0) return false;
+    return encode_cached(map, MapKey{base, rows, cols, box_rows, box_cols, 2u}, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 // DEEP: as many stages as fit (plane operands, TMA-latency-bound); otherwise two, so that two CTAs share an SM (the
@@ -104,6 +132,7 @@ struct GemmTcMaps {
 
 template <int BN, int AMODE, int APL, int BPL, int PREC>
 __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>::THREADS), 1) k_gemm_tn_tc(const __grid_constant__ GemmTcMaps maps, GemmTnArgs g, int* status) {
+    PDL_START();
     using Cfg = GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>;
     constexpr int BM = Cfg::BM, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -360,11 +389,8 @@ static cudaError_t launch_t(const GemmTnArgs& g, int splits, int* status, cudaSt
     if (!map(&maps.b_hi, g.Bhi, g.ldb)) return cudaErrorNotSupported;
     if (BPL >= 2 && !map(&maps.b_lo, g.Blo, g.ldb)) return cudaErrorNotSupported;
     if (BPL == 3 && !map(&maps.b_lo2, g.Blo + (g.Blo - g.Bhi), g.ldb)) return cudaErrorNotSupported;
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tn_tc<BN, AMODE, APL, BPL, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-    if (e != cudaSuccess) return e;
     dim3 grid(AMODE == A_ENV ? 2 : (g.M + Cfg::BM - 1) / Cfg::BM, (g.N + BN - 1) / BN, splits);
-    k_gemm_tn_tc<BN, AMODE, APL, BPL, PREC><<<grid, Cfg::THREADS, Cfg::smem_bytes, s>>>(maps, g, status);
-    return cudaGetLastError();
+    return launch<k_gemm_tn_tc<BN, AMODE, APL, BPL, PREC>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, g, status);
 }
 
 template <int BN, int PREC>

@@ -61,6 +61,7 @@ struct HeadsMaps {
 template <int H, int NW, int PREC, int HS = H, bool H2BF = false, bool GROUPED = false, bool FUSE = false>
 __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREADS), (HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::PER_SM))
     k_heads_bwd(LearnArgs a_in, const __grid_constant__ HeadsMaps maps) {
+    PDL_START();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.z);  // many policies: grid.z = policy
     const LearnArgs& a = pa.a;
     using Cfg = HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>;
@@ -472,6 +473,7 @@ struct HeadsTcCfg {
 
 template <int H>
 __global__ void __launch_bounds__(512, 2) k_heads_bwd_tc(LearnArgs a) {
+    PDL_START();
     using Cfg = HeadsTcCfg<H>;
     constexpr int TR = Cfg::TR, HS = Cfg::HS, NW = Cfg::NW, NST = Cfg::NST, LD = Cfg::LD, LDT = TR + 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -696,6 +698,7 @@ struct Dh1Cfg {
 
 template <int H, int BN, int PREC, bool GROUPED = false>
 __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnArgs a_in) {
+    PDL_START();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.z);  // many policies: grid.z = policy
     const LearnArgs& a = pa.a;
     using Cfg = Dh1Cfg<H, BN, PREC>;
@@ -876,6 +879,7 @@ struct GemmTnCfg {
 
 template <int BM, int BN, int AMODE, int APL, int BPL, int PREC, bool GROUPED = false>
 __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
+    PDL_START();
     // many policies: grid.z = policy * nsplit + split
     const PolicyArgs<GROUPED, GemmTnArgs> pa(g_in, GROUPED ? (int)blockIdx.z / g_in.nsplit : 0);
     const GemmTnArgs& g = pa.a;
@@ -1023,21 +1027,15 @@ static cudaError_t launch_gemm_tn(const GemmTnArgs& g, int rows_m, int splits, c
     dim3 grid((rows_m + BM - 1) / BM, (g.N + BN - 1) / BN, splits);
     if (g.npol > 1) {  // many policies: grid.z = policy * splits + split
         if constexpr (PREC == 0) {
-            cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-            if (e != cudaSuccess) return e;
             if ((size_t)g.npol * splits > 65535) return cudaErrorNotSupported;
             grid.z = g.npol * splits;
             GemmTnArgs gg = g;
             gg.nsplit = splits;
-            k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC, true><<<grid, 256, Cfg::smem_bytes, s>>>(gg);
-            return cudaGetLastError();
+            return launch<k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC, true>>(grid, 256, Cfg::smem_bytes, s, gg);
         }
         return cudaErrorNotSupported;
     }
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-    if (e != cudaSuccess) return e;
-    k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC><<<grid, 256, Cfg::smem_bytes, s>>>(g);
-    return cudaGetLastError();
+    return launch<k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC>>(grid, 256, Cfg::smem_bytes, s, g);
 }
 
 // One Adam step of parameter i with gradient g (Kingma & Ba, Algorithm 1), plus the refreshed 16-bit copies.
@@ -1097,6 +1095,7 @@ __device__ __forceinline__ void adam_step(const LearnArgs& a, size_t i, float g,
 // Adam from the GRADS blob as it stands (the second half of an update whose gradient was averaged over replicas).
 template <int PREC, bool GROUPED>
 __global__ void __launch_bounds__(256) k_adam_only(LearnArgs a_in) {
+    PDL_START();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
     const LearnArgs& a = pa.a;
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
@@ -1115,6 +1114,7 @@ __global__ void __launch_bounds__(256) k_adam_only(LearnArgs a_in) {
 // ----------------------------------------------------------------------------------------------------
 template <int PREC, bool GROUPED>
 __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_in, int loss_blocks) {
+    PDL_START();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
     const LearnArgs& a = pa.a;
     const size_t R = GROUPED ? (size_t)a.d.B * a.T : R_in;  // rows of THIS policy
@@ -1233,6 +1233,7 @@ __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_i
 // Debug record of the ReLU gates from the saved activations (h1 hi plane, h2).
 template <bool GROUPED>
 __global__ void __launch_bounds__(256) k_pack_gates2(DimsBuffers in, size_t R_in, int h2_bf16) {
+    PDL_START();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);  // many policies: grid.y = policy
     const Dims& d = pa.a.d;
     const Buffers& b = pa.a.b;
@@ -1347,9 +1348,7 @@ static cudaError_t launch_heads_t(const LearnArgs& a, int grid, cudaStream_t s, 
     memset(&maps, 0, sizeof(maps));
     if (a.d.npol > 1) {
         if constexpr (PREC == 0 && HS == H && !H2BF) {
-            CK(cudaFuncSetAttribute(k_heads_bwd<H, NW, PREC, HS, H2BF, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes));
-            k_heads_bwd<H, NW, PREC, HS, H2BF, true><<<dim3(grid, 1, a.d.npol), Cfg::THREADS, Cfg::smem_bytes, s>>>(a, maps);
-            return cudaGetLastError();
+            return launch<k_heads_bwd<H, NW, PREC, HS, H2BF, true>>(dim3(grid, 1, a.d.npol), Cfg::THREADS, Cfg::smem_bytes, s, a, maps);
         }
         return cudaErrorNotSupported;
     }
@@ -1360,22 +1359,16 @@ static cudaError_t launch_heads_t(const LearnArgs& a, int grid, cudaStream_t s, 
             const uint16_t* h1hi = reinterpret_cast<const uint16_t*>(a.b.h1);
             if (!make_tensor_map_2d(&maps.h1_hi, h1hi, R, H, FCfg::TR, PREC == 1)) return cudaErrorNotSupported;
             if (PREC == 0 && !make_tensor_map_2d(&maps.h1_lo, h1hi + RH, R, H, FCfg::TR, false)) return cudaErrorNotSupported;
-            CK(cudaFuncSetAttribute(k_heads_bwd<H, NW, PREC, HS, H2BF, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FCfg::smem_bytes));
-            k_heads_bwd<H, NW, PREC, HS, H2BF, false, true><<<dim3(grid, 1), FCfg::THREADS, FCfg::smem_bytes, s>>>(a, maps);
-            return cudaGetLastError();
+            return launch<k_heads_bwd<H, NW, PREC, HS, H2BF, false, true>>(dim3(grid, 1), FCfg::THREADS, FCfg::smem_bytes, s, a, maps);
         }
     }
-    CK(cudaFuncSetAttribute(k_heads_bwd<H, NW, PREC, HS, H2BF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes));
-    k_heads_bwd<H, NW, PREC, HS, H2BF><<<dim3(grid, H / HS), Cfg::THREADS, Cfg::smem_bytes, s>>>(a, maps);
-    return cudaGetLastError();
+    return launch<k_heads_bwd<H, NW, PREC, HS, H2BF>>(dim3(grid, H / HS), Cfg::THREADS, Cfg::smem_bytes, s, a, maps);
 }
 
 template <int H>
 static cudaError_t launch_heads_tc_t(const LearnArgs& a, int grid, cudaStream_t s) {
     using Cfg = HeadsTcCfg<H>;
-    CK(cudaFuncSetAttribute(k_heads_bwd_tc<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes));
-    k_heads_bwd_tc<H><<<dim3(grid, H / Cfg::HS), 512, Cfg::smem_bytes, s>>>(a);
-    return cudaGetLastError();
+    return launch<k_heads_bwd_tc<H>>(dim3(grid, H / Cfg::HS), 512, Cfg::smem_bytes, s, a);
 }
 
 template <int H, int BN, int PREC>
@@ -1384,16 +1377,12 @@ static cudaError_t launch_dh1_t(const LearnArgs& a, cudaStream_t s) {
     dim3 grid((a.d.B + Cfg::BM - 1) / Cfg::BM, H / BN * a.ts);
     if (a.d.npol > 1) {
         if constexpr (PREC == 0) {
-            CK(cudaFuncSetAttribute(k_dh1<H, BN, PREC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes));
             grid.z = a.d.npol;
-            k_dh1<H, BN, PREC, true><<<grid, Cfg::THREADS, Cfg::smem_bytes, s>>>(a);
-            return cudaGetLastError();
+            return launch<k_dh1<H, BN, PREC, true>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, a);
         }
         return cudaErrorNotSupported;
     }
-    CK(cudaFuncSetAttribute(k_dh1<H, BN, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes));
-    k_dh1<H, BN, PREC><<<grid, Cfg::THREADS, Cfg::smem_bytes, s>>>(a);
-    return cudaGetLastError();
+    return launch<k_dh1<H, BN, PREC>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, a);
 }
 
 template <int V> using ic = std::integral_constant<int, V>;
@@ -1592,17 +1581,17 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         const unsigned nb = (unsigned)((d.ob2 + 255) / 256 + (d.P - d.ob2 + 7) / 8);
         if (d.npol > 1) {
             const unsigned per_policy = d.npol >= 74 ? 8u : (nb < 592u / d.npol ? nb : 592u / d.npol);  // at least four CTAs per SM in all, at most eight per policy
-            if constexpr (PREC == 0) k_reduce_adam2<PREC, true><<<dim3(per_policy, d.npol), 256, 0, s>>>(a, R, pl.loss_blocks);
+            if constexpr (PREC == 0) launch<k_reduce_adam2<PREC, true>>(dim3(per_policy, d.npol), 256, 0, s, a, R, pl.loss_blocks);
             else return cudaErrorNotSupported;
         } else {
-            k_reduce_adam2<PREC, false><<<nb, 256, 0, s>>>(a, R, pl.loss_blocks);
+            launch<k_reduce_adam2<PREC, false>>(nb, 256, 0, s, a, R, pl.loss_blocks);
         }
         CK(cudaGetLastError());
     }
     if (b.dbg_gates) {
         Scope sc(c, K_PACK_GATES);
-        if (d.npol > 1) k_pack_gates2<true><<<dim3(64, d.npol), 256, 0, s>>>(DimsBuffers{d, b}, R, 0);
-        else k_pack_gates2<false><<<148 * 8, 256, 0, s>>>(DimsBuffers{d, b}, R, wide && PREC == 1 ? 1 : 0);
+        if (d.npol > 1) launch<k_pack_gates2<true>>(dim3(64, d.npol), 256, 0, s, DimsBuffers{d, b}, R, 0);
+        else launch<k_pack_gates2<false>>(148 * 8, 256, 0, s, DimsBuffers{d, b}, R, wide && PREC == 1 ? 1 : 0);
         CK(cudaGetLastError());
     }
     return cudaSuccess;
@@ -1613,10 +1602,10 @@ cudaError_t launch_adam_only(const LearnArgs& a, int prec, const Ctx& c) {
     const unsigned nb = (unsigned)((a.d.P + 255) / 256);
     if (a.d.npol > 1) {
         if (prec == 1) return cudaErrorNotSupported;
-        k_adam_only<0, true><<<dim3(nb, a.d.npol), 256, 0, c.s>>>(a);
-    } else if (prec == 1) k_adam_only<1, false><<<nb, 256, 0, c.s>>>(a);
-    else if (three_terms(a.d.H, prec)) k_adam_only<2, false><<<nb, 256, 0, c.s>>>(a);
-    else k_adam_only<0, false><<<nb, 256, 0, c.s>>>(a);
+        launch<k_adam_only<0, true>>(dim3(nb, a.d.npol), 256, 0, c.s, a);
+    } else if (prec == 1) launch<k_adam_only<1, false>>(nb, 256, 0, c.s, a);
+    else if (three_terms(a.d.H, prec)) launch<k_adam_only<2, false>>(nb, 256, 0, c.s, a);
+    else launch<k_adam_only<0, false>>(nb, 256, 0, c.s, a);
     return cudaGetLastError();
 }
 

@@ -9,6 +9,7 @@ namespace anakin {
 // cells); counter (b,1+c/4,0) word (c%4) below floor(density*2^32) makes cell c a wall; start and goal stay free.
 template <bool GROUPED>
 __global__ void __launch_bounds__(128) k_reset_env(DimsBuffers in, uint32_t k0, uint32_t k1, uint32_t thr) {
+    PDL_START();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);  // many policies: grid.y = policy
     const Dims& d = pa.a.d;
     const Buffers& b = pa.a.b;
@@ -45,6 +46,7 @@ __global__ void __launch_bounds__(128) k_reset_env(DimsBuffers in, uint32_t k0, 
 // draws counter (i,p,0): its own, independent initialisation (policy 0 = the single-policy one).
 template <bool GROUPED>
 __global__ void __launch_bounds__(256) k_reset_params(DimsBuffers in, uint32_t k0, uint32_t k1) {
+    PDL_START();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);
     const Dims& d = pa.a.d;
     const Buffers& b = pa.a.b;
@@ -77,6 +79,7 @@ __global__ void __launch_bounds__(256) k_reset_params(DimsBuffers in, uint32_t k
 
 // bf16 mode: the network computes with bf16-rounded weight matrices and unrounded biases.
 __global__ void __launch_bounds__(256) k_refresh_compute_params(Dims d, Buffers b) {
+    PDL_START();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d.P) return;
     const bool is_bias = (i >= d.ob1 && i < d.oW2) || (i >= d.ob2 && i < d.oWh) || i >= d.obh;
@@ -87,8 +90,7 @@ __global__ void __launch_bounds__(256) k_refresh_compute_params(Dims d, Buffers 
 cudaError_t launch_refresh_compute_params(const Dims& d, const Buffers& b, int prec, const Ctx& c) {
     if (prec != 1) return cudaSuccess;
     Scope sc(c, K_REFRESH_PARAMS);
-    k_refresh_compute_params<<<(unsigned)((d.P + 255) / 256), 256, 0, c.s>>>(d, b);
-    return cudaGetLastError();
+    return launch<k_refresh_compute_params>((unsigned)((d.P + 255) / 256), 256, 0, c.s, d, b);
 }
 
 cudaError_t launch_reset(const Dims& d, const Buffers& b, uint64_t seed, double density, int prec, const Ctx& c) {
@@ -97,16 +99,16 @@ cudaError_t launch_reset(const Dims& d, const Buffers& b, uint64_t seed, double 
     cudaError_t e;
     {
         Scope sc(c, K_RESET_ENV);
-        if (d.npol > 1) k_reset_env<true><<<dim3((d.B + 127) / 128, d.npol), 128, 0, c.s>>>(DimsBuffers{d, b}, k0, k1, thr);
-        else k_reset_env<false><<<(d.B + 127) / 128, 128, 0, c.s>>>(DimsBuffers{d, b}, k0, k1, thr);
+        if (d.npol > 1) launch<k_reset_env<true>>(dim3((d.B + 127) / 128, d.npol), 128, 0, c.s, DimsBuffers{d, b}, k0, k1, thr);
+        else launch<k_reset_env<false>>((d.B + 127) / 128, 128, 0, c.s, DimsBuffers{d, b}, k0, k1, thr);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
     {
         Scope sc(c, K_RESET_PARAMS);
         const unsigned nb = (unsigned)((d.P + 255) / 256);
-        if (d.npol > 1) k_reset_params<true><<<dim3(nb, d.npol), 256, 0, c.s>>>(DimsBuffers{d, b}, k0, k1);
-        else k_reset_params<false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b}, k0, k1);
+        if (d.npol > 1) launch<k_reset_params<true>>(dim3(nb, d.npol), 256, 0, c.s, DimsBuffers{d, b}, k0, k1);
+        else launch<k_reset_params<false>>(nb, 256, 0, c.s, DimsBuffers{d, b}, k0, k1);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;

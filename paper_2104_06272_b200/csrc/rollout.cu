@@ -12,6 +12,7 @@ namespace anakin {
 // ascending cell order, the goal row last.
 template <bool GROUPED>
 __global__ void __launch_bounds__(256) k_env_base(DimsBuffers in) {
+    PDL_START();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);  // many policies: grid.y = policy
     const Dims& d = pa.a.d;
     const Buffers& b = pa.a.b;
@@ -59,8 +60,8 @@ cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c) {
     }
     Scope sc(c, K_ENV_BASE);
     const unsigned nb = (unsigned)(((size_t)d.B * (d.H / 4) + 255) / 256);
-    if (d.npol > 1) k_env_base<true><<<dim3(nb, d.npol), 256, 0, c.s>>>(DimsBuffers{d, b});
-    else k_env_base<false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
+    if (d.npol > 1) launch<k_env_base<true>>(dim3(nb, d.npol), 256, 0, c.s, DimsBuffers{d, b});
+    else launch<k_env_base<false>>(nb, 256, 0, c.s, DimsBuffers{d, b});
     return cudaGetLastError();
 }
 
@@ -73,6 +74,7 @@ cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c) {
 // ----------------------------------------------------------------------------------------------------
 template <int HJ, int RR>
 __global__ void __launch_bounds__(256) k_rollout(RolloutArgs a) {
+    PDL_START();
     constexpr int H = 32 * HJ, ME = 8 * RR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* s_base = reinterpret_cast<float*>(smem_raw);  // [ME][H]
@@ -228,10 +230,7 @@ template <int HJ, int RR>
 static cudaError_t launch_rollout_t(const RolloutArgs& a, cudaStream_t s) {
     constexpr int H = 32 * HJ, ME = 8 * RR;
     const size_t smem = (size_t)(3 * ME * H + ME * 8) * sizeof(float) + ME * 8 * sizeof(uint32_t) + ME * sizeof(int);
-    cudaError_t e = cudaFuncSetAttribute(k_rollout<HJ, RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_rollout<HJ, RR><<<(a.d.B + ME - 1) / ME, 256, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch<k_rollout<HJ, RR>>((a.d.B + ME - 1) / ME, 256, smem, s, a);
 }
 
 cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
@@ -253,6 +252,7 @@ cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
 // ----------------------------------------------------------------------------------------------------
 template <bool GROUPED>
 __global__ void __launch_bounds__(128) k_gae(DimsBuffers in, int T, float gamma, float lambda) {
+    PDL_START();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);
     const Dims& d = pa.a.d;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(128) k_gae(DimsBuffers in, int T, float gamma,
 
 cudaError_t launch_gae(const Dims& d, const Buffers& b, int T, float gamma, float lambda, const Ctx& c) {
     Scope sc(c, K_GAE);
-    if (d.npol > 1) k_gae<true><<<dim3((d.B + 127) / 128, d.npol), 128, 0, c.s>>>(DimsBuffers{d, b}, T, gamma, lambda);
-    else k_gae<false><<<(d.B + 127) / 128, 128, 0, c.s>>>(DimsBuffers{d, b}, T, gamma, lambda);
+    if (d.npol > 1) launch<k_gae<true>>(dim3((d.B + 127) / 128, d.npol), 128, 0, c.s, DimsBuffers{d, b}, T, gamma, lambda);
+    else launch<k_gae<false>>((d.B + 127) / 128, 128, 0, c.s, DimsBuffers{d, b}, T, gamma, lambda);
     return cudaGetLastError();
 }
 
@@ -275,6 +275,7 @@ cudaError_t launch_gae(const Dims& d, const Buffers& b, int T, float gamma, floa
 // Four steps per memory round trip.
 // ----------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_vtrace(Dims d, Buffers b, int T, float gamma, float rho_bar, float c_bar, const float* boot) {
+    PDL_START();
     const int env = blockIdx.x * blockDim.x + threadIdx.x;
     if (env >= d.B) return;
     const int B = d.B;
@@ -323,8 +324,7 @@ __global__ void __launch_bounds__(128) k_vtrace(Dims d, Buffers b, int T, float 
 
 cudaError_t launch_vtrace(const Dims& d, const Buffers& b, int T, float gamma, float rho_bar, float c_bar, const float* boot, const Ctx& c) {
     Scope sc(c, K_VTRACE);
-    k_vtrace<<<(d.B + 127) / 128, 128, 0, c.s>>>(d, b, T, gamma, rho_bar, c_bar, boot);
-    return cudaGetLastError();
+    return launch<k_vtrace>((d.B + 127) / 128, 128, 0, c.s, d, b, T, gamma, rho_bar, c_bar, boot);
 }
 
 }  // namespace anakin

@@ -18,6 +18,7 @@ namespace anakin {
 // n = 8*nt + g:  x = {W2[16ks+2t][n], W2[16ks+2t+1][n]},  y = {W2[16ks+2t+8][n], W2[16ks+2t+9][n]}  (low half first).
 template <int PREC, bool GROUPED>
 __global__ void __launch_bounds__(256) k_pack_w2(DimsBuffers in) {
+    PDL_START();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);  // many policies: grid.y = policy
     const Dims& d = pa.a.d;
     const Buffers& b = pa.a.b;
@@ -71,10 +72,10 @@ cudaError_t launch_pack_w2(const Dims& d, const Buffers& b, int prec, const Ctx&
     const unsigned nb = (d.H * d.H / 4 + 255) / 256;
     if (d.npol > 1) {
         if (prec == 1) return cudaErrorNotSupported;
-        k_pack_w2<0, true><<<dim3(nb, d.npol), 256, 0, c.s>>>(DimsBuffers{d, b});
-    } else if (prec == 1) k_pack_w2<1, false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
-    else if (three_terms(d.H, prec)) k_pack_w2<2, false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
-    else k_pack_w2<0, false><<<nb, 256, 0, c.s>>>(DimsBuffers{d, b});
+        launch<k_pack_w2<0, true>>(dim3(nb, d.npol), 256, 0, c.s, DimsBuffers{d, b});
+    } else if (prec == 1) launch<k_pack_w2<1, false>>(nb, 256, 0, c.s, DimsBuffers{d, b});
+    else if (three_terms(d.H, prec)) launch<k_pack_w2<2, false>>(nb, 256, 0, c.s, DimsBuffers{d, b});
+    else launch<k_pack_w2<0, false>>(nb, 256, 0, c.s, DimsBuffers{d, b});
     return cudaGetLastError();
 }
 
@@ -104,6 +105,7 @@ struct RolloutMmaCfg {
 // have been given the new positions.  Otherwise warp 0 does both (the wide kernels' registers leave no room for another warp).
 template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
 __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(RolloutArgs a_in) {
+    PDL_START();
     const PolicyArgs<GROUPED, RolloutArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
     const RolloutArgs& a = pa.a;
     using Cfg = RolloutMmaCfg<H, NW, PREC>;
@@ -476,10 +478,7 @@ constexpr size_t MAX_DYN_SMEM = 232448;  // 227 KB of dynamic shared memory per 
 
 template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
 static cudaError_t launch_k(const RolloutArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-    const cudaError_t e = cudaFuncSetAttribute(k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM);
-    if (e != cudaSuccess) return e;
-    k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN><<<grid, NW * 32 + (OWN ? 32 : 0), smem, s>>>(a);
-    return cudaGetLastError();
+    return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
 }
 
 template <int H, int NW, int PREC, bool GROUPED = false>

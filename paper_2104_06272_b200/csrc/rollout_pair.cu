@@ -56,6 +56,7 @@ __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uin
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(const __grid_constant__ PairMaps maps, RolloutArgs a) {
+    PDL_START();
     using Cfg = PairCfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NWT = Cfg::NWORK * 32;
     extern __shared__ unsigned char smem_raw[];
@@ -401,11 +402,8 @@ cudaError_t launch_rollout_pair(const RolloutArgs& a0, cudaStream_t s) {
     memset(&maps, 0, sizeof(maps));
     if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     if (!make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    const cudaError_t e = cudaFuncSetAttribute(k_rollout_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
     const int pairs = (a.d.B + 2 * Cfg::ME - 1) / (2 * Cfg::ME);
-    k_rollout_pair<<<2 * pairs, Cfg::THREADS, smem, s>>>(maps, a);
-    return cudaGetLastError();
+    return launch<k_rollout_pair>(2 * pairs, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

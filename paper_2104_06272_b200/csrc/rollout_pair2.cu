@@ -60,6 +60,7 @@ __device__ __forceinline__ void st_async_f32_2(uint32_t cluster_addr, float v, u
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1) k_rollout_pair2(const __grid_constant__ Pair2Maps maps, RolloutArgs a) {
+    PDL_START();
     using Cfg = Pair2Cfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
     extern __shared__ unsigned char smem_raw[];
@@ -436,11 +437,8 @@ cudaError_t launch_rollout_pair2(const RolloutArgs& a0, cudaStream_t s) {
     memset(&maps, 0, sizeof(maps));
     if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     if (!make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    const cudaError_t e = cudaFuncSetAttribute(k_rollout_pair2, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
     const int pairs = (a.d.B + PER_PAIR - 1) / PER_PAIR;
-    k_rollout_pair2<<<2 * pairs, Cfg::THREADS, smem, s>>>(maps, a);
-    return cudaGetLastError();
+    return launch<k_rollout_pair2>(2 * pairs, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

@@ -52,6 +52,7 @@ struct Tc128Maps {
 };
 
 __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __grid_constant__ Tc128Maps maps, RolloutArgs a) {
+    PDL_START();
     using Cfg = Tc128Cfg;
     constexpr int H = Cfg::H, NE = Cfg::NE, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
     extern __shared__ unsigned char smem_raw[];
@@ -433,10 +434,7 @@ cudaError_t launch_rollout_tc128(const RolloutArgs& a0, cudaStream_t s) {
     memset(&maps, 0, sizeof(maps));
     if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     if (!make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    const cudaError_t e = cudaFuncSetAttribute(k_rollout_tc128, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    k_rollout_tc128<<<(a.d.B + Cfg::NOWN - 1) / Cfg::NOWN, Cfg::THREADS, smem, s>>>(maps, a);
-    return cudaGetLastError();
+    return launch<k_rollout_tc128>((a.d.B + Cfg::NOWN - 1) / Cfg::NOWN, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

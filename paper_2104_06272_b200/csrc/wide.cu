@@ -38,6 +38,7 @@ struct NtCfg {
 
 template <int EPI, bool B_MN, int BN_>
 __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ NtMaps maps, NtArgs g) {
+    pdl_wait();
     using Cfg = NtCfg<BN_>;
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -156,10 +157,7 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
 template <int EPI, bool B_MN, int BN>
 cudaError_t launch_nt_t(const NtMaps& maps, const NtArgs& g, int ntiles, cudaStream_t s) {
     using Cfg = NtCfg<BN>;
-    const cudaError_t e = cudaFuncSetAttribute(k_gemm_nt_tc<EPI, B_MN, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_bytes);
-    if (e != cudaSuccess) return e;
-    k_gemm_nt_tc<EPI, B_MN, BN><<<ntiles < 148 ? ntiles : 148, Cfg::THREADS, Cfg::smem_bytes, s>>>(maps, g);
-    return cudaGetLastError();
+    return launch<k_gemm_nt_tc<EPI, B_MN, BN>>(ntiles < 148 ? ntiles : 148, Cfg::THREADS, Cfg::smem_bytes, s, maps, g);
 }
 
 // B: MN-major [K][N] (boxes of 64 x 64) or K-major [N][K].  The CTA-pair kernel (256 x 256 tiles) halves the operand traffic and takes
@@ -207,6 +205,7 @@ __device__ __forceinline__ void h1_store8(uint16_t* out, size_t plane, const flo
 // h1 rows: 8 hidden units per thread.  pos[i] is the agent cell of row i (env = i mod B).
 template <bool F32>
 __global__ void __launch_bounds__(256) k_h1_wide(Dims d, Buffers b, const uint8_t* pos, size_t rows, size_t row0) {
+    PDL_START();
     const int H = d.H, H8 = H / 8;
     const float* W1a = b.theta_c + d.oW1 + (size_t)d.C * H;  // agent plane of W1
     uint16_t* out = reinterpret_cast<uint16_t*>(b.h1) + row0 * H;
@@ -231,6 +230,7 @@ __global__ void __launch_bounds__(256) k_h1_wide(Dims d, Buffers b, const uint8_
 //   mode 3: forward of the current env state under the current parameters: saves the value to vboot.
 template <int H, bool F32, int HW_ROWS>
 __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mode, size_t rows, size_t row0) {
+    PDL_START();
     constexpr int TRIPS = H / 128;   // a lane covers four consecutive hidden units per trip
     extern __shared__ __align__(16) float s_wh[];  // [H][5] as stored
     __shared__ float s_out[HW_ROWS][8];
@@ -382,6 +382,7 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
 
 // S[env][j] = sum over t of dh1[t*B + env][j], kept as two bf16 terms (hi and lo planes) for the K = B GEMMs of dW1.
 __global__ void __launch_bounds__(256) k_sum_t_wide(Dims d, Buffers b, int T) {
+    PDL_START();
     const int H8 = d.H / 8;
     const size_t total = (size_t)d.B * H8;
     const size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x;
@@ -420,6 +421,7 @@ __global__ void __launch_bounds__(256) k_sum_t_wide(Dims d, Buffers b, int T) {
 // W2 as row-major bf16 planes: one (the values are bf16 already in the bf16 workload) or the three terms of fp32 weights.
 template <bool F32>
 __global__ void __launch_bounds__(256) k_pack_w2_wide(Dims d, Buffers b) {
+    PDL_START();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x, n = (size_t)d.H * d.H;
     if (2 * i >= n) return;
     const float2 w = reinterpret_cast<const float2*>(b.theta_c + d.oW2)[i];
@@ -432,6 +434,7 @@ __global__ void __launch_bounds__(256) k_pack_w2_wide(Dims d, Buffers b) {
 // (one where the weights are bf16 values, else three terms).  Columns / rows from C up to Cp, a multiple of 64, are zero.
 template <bool F32>
 __global__ void __launch_bounds__(256) k_expand_walls(Dims d, Buffers b, uint16_t* X, uint16_t* W1w, int Cp) {
+    PDL_START();
     const size_t nx = (size_t)d.B * (Cp / 8), nw = (size_t)Cp * d.H / 2, real = (size_t)d.C * d.H / 2;
     for (size_t idx = (size_t)blockIdx.x * 256 + threadIdx.x; idx < nx + nw; idx += (size_t)gridDim.x * 256) {
         if (idx < nx) {
@@ -458,8 +461,8 @@ __global__ void __launch_bounds__(256) k_expand_walls(Dims d, Buffers b, uint16_
 template <int H, bool F32>
 cudaError_t heads_wide_t(const RolloutArgs& a, int t, int mode, size_t rows, size_t row0, cudaStream_t s) {
     const size_t smem = (size_t)5 * H * sizeof(float);
-    if (rows < 148 * 2 * 32) k_heads_wide<H, F32, 8><<<(unsigned)((rows + 7) / 8), 256, smem, s>>>(a, t, mode, rows, row0);
-    else k_heads_wide<H, F32, 32><<<(unsigned)((rows + 31) / 32), 256, smem, s>>>(a, t, mode, rows, row0);
+    if (rows < 148 * 2 * 32) launch<k_heads_wide<H, F32, 8>>((unsigned)((rows + 7) / 8), 256, smem, s, a, t, mode, rows, row0);
+    else launch<k_heads_wide<H, F32, 32>>((unsigned)((rows + 31) / 32), 256, smem, s, a, t, mode, rows, row0);
     return cudaGetLastError();
 }
 cudaError_t heads_wide(const RolloutArgs& a, bool f32, int t, int mode, size_t rows, size_t row0, cudaStream_t s) {
@@ -480,8 +483,8 @@ static bool is_f32(const Buffers& b) { return b.theta_c == b.theta; }
 cudaError_t launch_pack_w2_wide(const Dims& d, const Buffers& b, const Ctx& c) {
     Scope sc(c, K_PACK_W2);
     const unsigned nb = (unsigned)(((size_t)d.H * d.H / 2 + 255) / 256);
-    if (is_f32(b)) k_pack_w2_wide<true><<<nb, 256, 0, c.s>>>(d, b);
-    else k_pack_w2_wide<false><<<nb, 256, 0, c.s>>>(d, b);
+    if (is_f32(b)) launch<k_pack_w2_wide<true>>(nb, 256, 0, c.s, d, b);
+    else launch<k_pack_w2_wide<false>>(nb, 256, 0, c.s, d, b);
     return cudaGetLastError();
 }
 
@@ -504,8 +507,8 @@ cudaError_t launch_env_base_wide(const Dims& d, const Buffers& b, const Ctx& c) 
     uint16_t* W1w = X + (size_t)d.B * Cp * terms;
     {
         Scope sc(c, K_ENV_BASE);
-        if (f32) k_expand_walls<true><<<148 * 8, 256, 0, c.s>>>(d, b, X, W1w, Cp);
-        else k_expand_walls<false><<<148 * 8, 256, 0, c.s>>>(d, b, X, W1w, Cp);
+        if (f32) launch<k_expand_walls<true>>(148 * 8, 256, 0, c.s, d, b, X, W1w, Cp);
+        else launch<k_expand_walls<false>>(148 * 8, 256, 0, c.s, d, b, X, W1w, Cp);
         CKW(cudaGetLastError());
     }
     Scope sc(c, K_ENV_BASE);
@@ -549,8 +552,7 @@ static cudaError_t rollout_wide_t(const RolloutArgs& a, const Ctx& c) {
         }
     };
     auto h1_rows = [&](const uint8_t* pos, size_t n, size_t row0) {
-        k_h1_wide<F32><<<(unsigned)((n * (H / 8) + 255) / 256), 256, 0, c.s>>>(d, b, pos, n, row0);
-        return cudaGetLastError();
+        return launch<k_h1_wide<F32>>((unsigned)((n * (H / 8) + 255) / 256), 256, 0, c.s, d, b, pos, n, row0);
     };
     // forward of n rows from row0: (h1,) h2, heads in the given mode
     auto replay = [&](const uint8_t* pos, size_t n, size_t row0, int mode) {
@@ -620,8 +622,7 @@ static cudaError_t dh1_wide_t(const LearnArgs& a, const Ctx& c) {
             CKW((launch_nt<EPI_GATE, false>(b.dh2, R, b.w2p_hi, g, c.s)));
         }
         Scope sc(c, K_SUM_OVER_T);
-        k_sum_t_wide<<<(unsigned)(((size_t)d.B * (H / 8) + 255) / 256), 256, 0, c.s>>>(d, b, a.T);
-        return cudaGetLastError();
+        return launch<k_sum_t_wide>((unsigned)(((size_t)d.B * (H / 8) + 255) / 256), 256, 0, c.s, d, b, a.T);
     }
 }
 cudaError_t launch_dh1_wide(const LearnArgs& a, const Ctx& c) { return is_f32(a.b) ? dh1_wide_t<true>(a, c) : dh1_wide_t<false>(a, c); }

@@ -30,6 +30,7 @@ struct PairCfg {
 
 template <int EPI, bool B_MN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pair(const __grid_constant__ NtMaps maps, NtArgs g) {
+    pdl_wait();
     using Cfg = PairCfg;
     constexpr int BM = Cfg::BM, PM = Cfg::PM, BN = Cfg::BN, BNH = Cfg::BNH, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -153,12 +154,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pa
 
 template <int EPI, bool B_MN>
 cudaError_t launch_pair_t(const NtMaps& maps, const NtArgs& g, cudaStream_t s) {
-    const cudaError_t e = cudaFuncSetAttribute(k_gemm_nt_pair<EPI, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PairCfg::smem_bytes);
-    if (e != cudaSuccess) return e;
     const int ntiles = ((g.M + PairCfg::PM - 1) / PairCfg::PM) * ((g.N + PairCfg::BN - 1) / PairCfg::BN);
     const int pairs = ntiles < 74 ? ntiles : 74;
-    k_gemm_nt_pair<EPI, B_MN><<<2 * pairs, PairCfg::THREADS, PairCfg::smem_bytes, s>>>(maps, g);
-    return cudaGetLastError();
+    return launch<k_gemm_nt_pair<EPI, B_MN>>(2 * pairs, PairCfg::THREADS, PairCfg::smem_bytes, s, maps, g);
 }
 
 }  // namespace

@@ -242,24 +242,20 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
 
 template <int EPI, bool B_MN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_x3_pair(const __grid_constant__ NtMaps maps, X3Args g) {
+    pdl_wait();
     x3_body<EPI, B_MN, true, 256>(maps, g);
 }
 template <int EPI, bool B_MN, int BN>
 __global__ void __launch_bounds__(320, 1) k_x3_one(const __grid_constant__ NtMaps maps, X3Args g) {
+    pdl_wait();
     x3_body<EPI, B_MN, false, BN>(maps, g);
 }
 
 template <int EPI, bool B_MN>
 cudaError_t launch_x3_t(const NtMaps& maps, const X3Args& g, int bn, int tiles, cudaStream_t s) {
-    auto go = [&](auto kern, size_t smem, int grid) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<grid, 320, smem, s>>>(maps, g);
-        return cudaGetLastError();
-    };
-    if (bn == 256) return go(k_x3_pair<EPI, B_MN>, X3Cfg<true, 256>::smem_bytes, 2 * (tiles < 74 ? tiles : 74));
-    if (bn == 128) return go(k_x3_one<EPI, B_MN, 128>, X3Cfg<false, 128>::smem_bytes, tiles < 148 ? tiles : 148);
-    return go(k_x3_one<EPI, B_MN, 64>, X3Cfg<false, 64>::smem_bytes, tiles < 148 ? tiles : 148);
+    if (bn == 256) return launch<k_x3_pair<EPI, B_MN>>(2 * (tiles < 74 ? tiles : 74), 320, X3Cfg<true, 256>::smem_bytes, s, maps, g);
+    if (bn == 128) return launch<k_x3_one<EPI, B_MN, 128>>(tiles < 148 ? tiles : 148, 320, X3Cfg<false, 128>::smem_bytes, s, maps, g);
+    return launch<k_x3_one<EPI, B_MN, 64>>(tiles < 148 ? tiles : 148, 320, X3Cfg<false, 64>::smem_bytes, s, maps, g);
 }
 
 }  // namespace
