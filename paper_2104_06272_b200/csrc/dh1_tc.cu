@@ -34,7 +34,6 @@ struct Dh1TcMaps {
 
 template <int H, int PREC>
 __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1TcMaps maps, LearnArgs a) {
-    PDL_START();
     using Cfg = Dh1TcCfg<H, PREC>;
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, PL = Cfg::PL, NCH = Cfg::NCH, STAGES = Cfg::STAGES, BOX = Cfg::BOX;
     extern __shared__ unsigned char smem_raw[];
@@ -72,6 +71,7 @@ __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1Tc
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     const int nchunks = nsteps * NCH;
     bool ok = true;
 

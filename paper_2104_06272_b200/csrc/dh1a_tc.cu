@@ -146,6 +146,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     tc::tc_fence_after();
     if (PAIR) tc::cluster_sync_all();  // both CTAs' barriers exist before either signals the other
     const uint32_t tmem = *tmem_slot;
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     const uint32_t acc_agent = tmem + (uint32_t)Cfg::AGENT_COL;
     int my_tiles = 0;  // env tiles this CTA walks
     for (int mt = xi; mt < m_tiles; mt += nx) ++my_tiles;
@@ -473,13 +474,11 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
 template <int H, int PREC>
 __global__ void __launch_bounds__(Dh1aCfg<H, PREC>::THREADS, 1)
     k_dh1a_tc(const __grid_constant__ Dh1aMaps maps, LearnArgs a, float* part_agent, size_t part_stride) {
-    PDL_START();
     dh1a_body<H, PREC>(maps, a, part_agent, part_stride);
 }
 template <int H, int PREC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Dh1aCfg<H, PREC>::THREADS, 1)
     k_dh1a_pair(const __grid_constant__ Dh1aMaps maps, LearnArgs a, float* part_agent, size_t part_stride) {
-    PDL_START();
     dh1a_body<H, PREC>(maps, a, part_agent, part_stride);
 }
 

@@ -132,7 +132,6 @@ struct GemmTcMaps {
 
 template <int BN, int AMODE, int APL, int BPL, int PREC>
 __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>::THREADS), 1) k_gemm_tn_tc(const __grid_constant__ GemmTcMaps maps, GemmTnArgs g, int* status) {
-    PDL_START();
     using Cfg = GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PREC>;
     constexpr int BM = Cfg::BM, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -163,6 +162,7 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     bool ok = true;
 
     if (wid == 0) {

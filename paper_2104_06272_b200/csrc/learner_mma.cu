@@ -61,7 +61,6 @@ struct HeadsMaps {
 template <int H, int NW, int PREC, int HS = H, bool H2BF = false, bool GROUPED = false, bool FUSE = false>
 __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREADS), (HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::PER_SM))
     k_heads_bwd(LearnArgs a_in, const __grid_constant__ HeadsMaps maps) {
-    PDL_START();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.z);  // many policies: grid.z = policy
     const LearnArgs& a = pa.a;
     using Cfg = HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>;
@@ -103,6 +102,7 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
     if (FUSE) tc::tc_fence_before();
     __syncthreads();
     if (FUSE) tc::tc_fence_after();
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     bool ok = true;
     const int my_its = (ntiles > (int)blockIdx.x) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;  // tiles of this CTA
 

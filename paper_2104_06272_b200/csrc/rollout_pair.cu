@@ -56,7 +56,6 @@ __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uin
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(const __grid_constant__ PairMaps maps, RolloutArgs a) {
-    PDL_START();
     using Cfg = PairCfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NWT = Cfg::NWORK * 32;
     extern __shared__ unsigned char smem_raw[];
@@ -101,6 +100,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     if (tid == NWT) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
         tc::mbar_expect_tx(wbar, 2 * Cfg::A_PLANE);
 #pragma unroll

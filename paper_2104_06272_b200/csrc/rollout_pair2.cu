@@ -60,7 +60,6 @@ __device__ __forceinline__ void st_async_f32_2(uint32_t cluster_addr, float v, u
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1) k_rollout_pair2(const __grid_constant__ Pair2Maps maps, RolloutArgs a) {
-    PDL_START();
     using Cfg = Pair2Cfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
     extern __shared__ unsigned char smem_raw[];
@@ -111,6 +110,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     if (issuer) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
         tc::mbar_expect_tx(wbar, 2 * Cfg::A_PLANE);
 #pragma unroll

@@ -52,7 +52,6 @@ struct Tc128Maps {
 };
 
 __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __grid_constant__ Tc128Maps maps, RolloutArgs a) {
-    PDL_START();
     using Cfg = Tc128Cfg;
     constexpr int H = Cfg::H, NE = Cfg::NE, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
     extern __shared__ unsigned char smem_raw[];
@@ -101,6 +100,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    PDL_START();  // (the set-up above runs under the predecessor's tail)
     if (issuer) {  // all of W2: box (kb, bx) = k rows 64kb.., columns 64bx..
         tc::mbar_expect_tx(wbar, 2 * Cfg::A_PLANE);
 #pragma unroll

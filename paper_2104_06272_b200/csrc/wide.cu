@@ -38,7 +38,6 @@ struct NtCfg {
 
 template <int EPI, bool B_MN, int BN_>
 __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ NtMaps maps, NtArgs g) {
-    pdl_wait();
     using Cfg = NtCfg<BN_>;
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -59,13 +58,16 @@ __global__ void __launch_bounds__(320, 1) k_gemm_nt_tc(const __grid_constant__ N
         for (int i = 0; i < 2; ++i) { tc::mbar_init(&tfull[i], 1); tc::mbar_init(&tempty[i], NT_EPI_WARPS); }
         tc::mbar_fence_init();
     }
-    if (EPI != EPI_GATE)
-        for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
     if (wid == 2) tc::tmem_alloc(tmem_slot, 2 * BN);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
+    if (EPI != EPI_GATE) {
+        for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
+        __syncthreads();
+    }
     bool ok = true;
 
     if (wid == 0) {

@@ -30,7 +30,6 @@ struct PairCfg {
 
 template <int EPI, bool B_MN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pair(const __grid_constant__ NtMaps maps, NtArgs g) {
-    pdl_wait();
     using Cfg = PairCfg;
     constexpr int BM = Cfg::BM, PM = Cfg::PM, BN = Cfg::BN, BNH = Cfg::BNH, KC = Cfg::KC, STAGES = Cfg::STAGES;
     extern __shared__ unsigned char smem_raw[];
@@ -55,14 +54,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_gemm_nt_pa
         for (int i = 0; i < 2; ++i) { tc::mbar_init(&tfull[i], 1); tc::mbar_init(&tempty[i], 2 * NT_EPI_WARPS); }
         tc::mbar_fence_init();
     }
-    if (EPI != EPI_GATE)
-        for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
     if (wid == 2) tc::tmem_alloc_pair(tmem_slot, 512);
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     tc::cluster_sync_all();  // both CTAs' barriers exist before either signals the other
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
+    if (EPI != EPI_GATE) {
+        for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
+        __syncthreads();
+    }
     bool ok = true;
 
     if (wid == 0) {

@@ -60,8 +60,6 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
         for (int i = 0; i < 2; ++i) { tc::mbar_init(&tfull[i], 1); tc::mbar_init(&tempty[i], (PAIR ? 2 : 1) * Cfg::EPI_WARPS); }
         tc::mbar_fence_init();
     }
-    if (EPI == EPI_FWD)
-        for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
     if (wid == 2) {
         if constexpr (PAIR) tc::tmem_alloc_pair(tmem_slot, 2 * BN);
         else tc::tmem_alloc(tmem_slot, 2 * BN);
@@ -71,6 +69,11 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
     tc::tc_fence_after();
     if constexpr (PAIR) tc::cluster_sync_all();  // both CTAs' barriers exist before either signals the other
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
+    if (EPI == EPI_FWD) {
+        for (int i = tid; i < g.N; i += Cfg::THREADS) s_bias[i] = g.bias[i];
+        __syncthreads();
+    }
     bool ok = true;
 
     if (wid == 0) {
@@ -242,12 +245,10 @@ __device__ __forceinline__ void x3_body(const NtMaps& maps, const X3Args& g) {
 
 template <int EPI, bool B_MN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(320, 1) k_x3_pair(const __grid_constant__ NtMaps maps, X3Args g) {
-    pdl_wait();
     x3_body<EPI, B_MN, true, 256>(maps, g);
 }
 template <int EPI, bool B_MN, int BN>
 __global__ void __launch_bounds__(320, 1) k_x3_one(const __grid_constant__ NtMaps maps, X3Args g) {
-    pdl_wait();
     x3_body<EPI, B_MN, false, BN>(maps, g);
 }
 
