@@ -388,9 +388,20 @@ cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s); 
 bool rollout_mma_supported(int H);
 bool three_terms(int H, int prec);             // fp32 operands as three bf16 terms instead of two fp16 terms
 bool rollout_uses_fragments(int H, int prec);  // the warp-level kernel (and with it the fragment copies of W2) serves this shape
-cudaError_t launch_rollout_tc128(const RolloutArgs& a, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, fp32, large batches); cudaErrorNotSupported otherwise
-cudaError_t launch_rollout_pair2(const RolloutArgs& a, cudaStream_t s);  // two env groups per CTA pair (H = 256, fp32, large batches); cudaErrorNotSupported otherwise
-cudaError_t launch_rollout_pair(const RolloutArgs& a, cudaStream_t s);  // CTA-pair tcgen05 rollout (H = 256, fp32); cudaErrorNotSupported otherwise
+cudaError_t launch_rollout_tc128(const RolloutArgs& a, int prec, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, large batches); cudaErrorNotSupported otherwise
+cudaError_t launch_rollout_pair2(const RolloutArgs& a, int prec, cudaStream_t s);  // two env groups per CTA pair (H = 256, large batches); cudaErrorNotSupported otherwise
+// Slices of a replay (grid.y) for kernels of one CTA per SM: its steps are independent, so few CTAs take fewer steps each; at least
+// two steps (the weights' load is paid per slice), none empty.
+inline int replay_slices(const RolloutArgs& a, int ctas) {
+    if (!a.replay) return 1;
+    const int steps = a.T + (a.replay == 2 ? 1 : 0);
+    int n = 148 / ctas;
+    if (n > steps / 2) n = steps / 2;
+    if (n < 1) n = 1;
+    const int len = (steps + n - 1) / n;
+    return (steps + len - 1) / len;
+}
+cudaError_t launch_rollout_pair(const RolloutArgs& a, int prec, cudaStream_t s);  // CTA-pair tcgen05 rollout (H = 256); cudaErrorNotSupported otherwise
 bool wide_supported(int H, int prec);         // hidden layer too wide for the persistent rollouts (either precision)
 size_t wide_h1_rows(const Dims& d);           // rows of one h1 / h2 plane on that path: the recorded ones and the bootstrap step's
 size_t wide_scratch_bytes(const Dims& d);     // operands of the base GEMM (kept in the dh1 buffer)

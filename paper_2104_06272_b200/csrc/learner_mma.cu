@@ -1112,7 +1112,10 @@ __global__ void __launch_bounds__(256) k_adam_only(LearnArgs a_in) {
 // ----------------------------------------------------------------------------------------------------
 // k_reduce_adam2: fixed-order sums of each parameter region's partials, then Adam (Kingma & Ba, Algorithm 1).
 // ----------------------------------------------------------------------------------------------------
-template <int PREC, bool GROUPED>
+// G threads share a parameter of the main part (64 or 256 parameters per piece): thread group g adds partials g, g + G, ... in
+// order, then the G sums are added in group order.  One thread per parameter is a chain of ns / 32 memory round trips: with 148
+// to 296 partials per weight (the fused heads + dW2 kernel leaves one per CTA) four threads take a quarter of it.
+template <int PREC, bool GROUPED, int G = 1>
 __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_in, int loss_blocks) {
     PDL_START();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
@@ -1142,10 +1145,48 @@ __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_i
     // parameter group, see below.
     // The work is cut into nb_total block-sized pieces; a launch with fewer CTAs per policy (many policies: a handful of
     // fat CTAs each instead of tens of thousands of tiny ones) walks them in a stride loop.
-    const int nb_main = (int)((d.ob2 + 255) / 256);
+    constexpr int PPB = 256 / G;  // parameters per piece of the main part
+    static_assert(!GROUPED || G == 1, "many policies have a handful of partials");
+    const int nb_main = (int)((d.ob2 + PPB - 1) / PPB);
     const int nb_total = nb_main + (int)(GROUPED ? (d.P - d.ob2 + 255) / 256 : (d.P - d.ob2 + 7) / 8);
     for (int bx = blockIdx.x; bx < nb_total; bx += gridDim.x) {
-        if (bx < nb_main || GROUPED) {
+        if (G > 1 && bx < nb_main) {
+            const int pi = threadIdx.x % PPB, grp = threadIdx.x / PPB;
+            const size_t i = (size_t)bx * PPB + pi;
+            float gsum = 0.f;
+            AdamIn in{0.f, 0.f, 0.f};
+            if (i < d.ob2) {
+                if (grp == 0) in = state_of(i);
+                const PartRegion& rg = a_in.reg[region_of(i)];
+                const float* p = rg.part + (i - rg.start);
+                constexpr int NF = 16;
+                const int ns = rg.ns;
+                const size_t step = rg.stride * G;
+                p += (size_t)grp * rg.stride;
+                int s = grp;
+                for (; s + (NF - 1) * G < ns; s += NF * G, p += NF * step) {
+                    float v[NF];
+#pragma unroll
+                    for (int q = 0; q < NF; ++q) v[q] = __ldg(p + q * step);
+#pragma unroll
+                    for (int q = 0; q < NF; ++q) gsum += v[q];
+                }
+                float v[NF];
+#pragma unroll
+                for (int q = 0; q < NF; ++q) v[q] = s + G * q < ns ? __ldg(p + q * step) : 0.f;
+#pragma unroll
+                for (int q = 0; q < NF; ++q) gsum += v[q];
+            }
+            __shared__ float s_grp[G][PPB];
+            __syncthreads();
+            s_grp[grp][pi] = gsum;
+            __syncthreads();
+            if (grp == 0 && i < d.ob2) {
+#pragma unroll
+                for (int g2 = 1; g2 < G; ++g2) gsum += s_grp[g2][pi];
+                apply(i, gsum, in);
+            }
+        } else if (bx < nb_main || GROUPED) {
             // (many policies: few partials everywhere, so the tail is cut into pieces of 256 parameters like the rest)
             const size_t i = bx < nb_main ? (size_t)bx * 256 + threadIdx.x : d.ob2 + (size_t)(bx - nb_main) * 256 + threadIdx.x;
             if (i < (bx < nb_main ? d.ob2 : d.P)) {
@@ -1578,13 +1619,17 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     }
     {
         Scope sc(c, K_REDUCE_ADAM);
-        const unsigned nb = (unsigned)((d.ob2 + 255) / 256 + (d.P - d.ob2 + 7) / 8);
+        int most = 0;  // partials of a main-part parameter
+        for (int q = 0; q < 5; ++q) most = a.reg[q].ns > most ? a.reg[q].ns : most;
+        const int grp = most > 48 ? 4 : 1;
+        const unsigned nb = (unsigned)((d.ob2 * grp + 255) / 256 + (d.P - d.ob2 + 7) / 8);
         if (d.npol > 1) {
             const unsigned per_policy = d.npol >= 74 ? 8u : (nb < 592u / d.npol ? nb : 592u / d.npol);  // at least four CTAs per SM in all, at most eight per policy
-            if constexpr (PREC == 0) launch<k_reduce_adam2<PREC, true>>(dim3(per_policy, d.npol), 256, 0, s, a, R, pl.loss_blocks);
+            if constexpr (PREC == 0) launch<k_reduce_adam2<PREC, true, 1>>(dim3(per_policy, d.npol), 256, 0, s, a, R, pl.loss_blocks);
             else return cudaErrorNotSupported;
         } else {
-            launch<k_reduce_adam2<PREC, false>>(nb, 256, 0, s, a, R, pl.loss_blocks);
+            if (grp > 1) launch<k_reduce_adam2<PREC, false, 4>>(nb, 256, 0, s, a, R, pl.loss_blocks);
+            else launch<k_reduce_adam2<PREC, false, 1>>(nb, 256, 0, s, a, R, pl.loss_blocks);
         }
         CK(cudaGetLastError());
     }

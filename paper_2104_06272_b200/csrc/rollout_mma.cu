@@ -514,19 +514,19 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
 bool rollout_mma_supported(int H) { return H == 32 || H == 64 || H == 96 || H == 128 || H == 192 || H == 256; }
 // fp32 operands as three exact bf16 terms (the widths beside 64, 128 and 256, which take two fp16 terms).
 bool three_terms(int H, int prec) { return prec == 0 && !(H == 64 || H == 128 || H == 256); }
-// fp32 at H = 256 runs the CTA-pair tcgen05 kernel, which reads the row-major planes of W2 only.
-bool rollout_uses_fragments(int H, int prec) { return rollout_mma_supported(H) && !(H == 256 && prec == 0); }
+// H = 256 runs the CTA-pair tcgen05 kernels, which read the row-major planes of W2 only.
+bool rollout_uses_fragments(int H, int prec) { (void)prec; return rollout_mma_supported(H) && H != 256; }
 
 // Returns cudaErrorNotSupported when the shape is not covered by the tensor-pipe kernel.
 cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s) {
     if (!rollout_mma_supported(a.d.H)) return cudaErrorNotSupported;
-    if (prec == 0 && a.d.npol <= 1 && a.d.H == 256) {  // the CTA-pair kernels on the 5th-generation tensor cores
-        const cudaError_t e = launch_rollout_pair2(a, s);  // large batches: two env groups per pair
+    if (a.d.npol <= 1 && a.d.H == 256) {  // the CTA-pair kernels on the 5th-generation tensor cores
+        const cudaError_t e = launch_rollout_pair2(a, prec, s);  // large batches: two env groups per pair
         if (e != cudaErrorNotSupported) return e;
-        return launch_rollout_pair(a, s);
+        return launch_rollout_pair(a, prec, s);
     }
-    if (prec == 0 && a.d.npol <= 1 && a.d.H == 128) {  // large batches: two env groups per CTA on the 5th-generation tensor cores
-        const cudaError_t e = launch_rollout_tc128(a, s);
+    if (a.d.npol <= 1 && a.d.H == 128) {  // large batches: two env groups per CTA on the 5th-generation tensor cores
+        const cudaError_t e = launch_rollout_tc128(a, prec, s);
         if (e != cudaErrorNotSupported) return e;
     }
     if (!a.b.w2f_hi) return cudaErrorNotSupported;
@@ -545,7 +545,6 @@ cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s) {
             case 96: return launch_t<96, 6, 1>(a, s);
             case 128: return launch_t<128, 8, 1>(a, s);
             case 192: return launch_t<192, 12, 1>(a, s);
-            case 256: return launch_t<256, 16, 1>(a, s);
         }
     } else {
         switch (a.d.H) {

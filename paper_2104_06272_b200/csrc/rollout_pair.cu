@@ -55,6 +55,7 @@ __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uin
                  : "memory");
 }
 
+template <int PREC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(const __grid_constant__ PairMaps maps, RolloutArgs a) {
     using Cfg = PairCfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NWT = Cfg::NWORK * 32;
@@ -102,13 +103,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
     const uint32_t tmem = *tmem_slot;
     PDL_START();  // (the set-up above runs under the predecessor's tail)
     if (tid == NWT) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
-        tc::mbar_expect_tx(wbar, 2 * Cfg::A_PLANE);
+        tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
 #pragma unroll
         for (int kb = 0; kb < H / 64; ++kb)
 #pragma unroll
             for (int bx = 0; bx < 2; ++bx) {
                 tc::tma_load_2d(s_ahi + (kb * 2 + bx) * Cfg::BOX, &maps.w_hi, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
-                tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
+                if (PREC == 0) tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
             }
     }
     // hidden unit of this thread in the heads phase, and its constants
@@ -139,7 +140,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                     const int jj = 128 * (int)rank + 32 * q + 16 * ks + 8 * hh + 2 * t4;
                     const float w0 = n < 5 ? b.theta_c[d.oWh + (size_t)jj * 5 + n] : 0.f;
                     const float w1 = n < 5 ? b.theta_c[d.oWh + (size_t)(jj + 1) * 5 + n] : 0.f;
-                    split2<0>(w0, w1, whf_hi[ks][hh], whf_lo[ks][hh]);
+                    split2<PREC>(w0, w1, whf_hi[ks][hh], whf_lo[ks][hh]);
                 }
         }
         if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
@@ -162,10 +163,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
-    const uint32_t idesc_w = tc::umma_idesc<0>(256, 128, true, false), idesc_n = tc::umma_idesc<0>(256, 64, true, false);
+    const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, true, false), idesc_n = tc::umma_idesc<PREC>(256, 64, true, false);
 
-    const int t_end = a.replay == 1 ? a.T - 1 : a.T;  // replay recomputes the T recorded rows (mode 2: and the current state)
-    for (int t = 0; t <= t_end; ++t) {
+    // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
+    const int t_last = a.replay == 1 ? a.T - 1 : a.T, t_len = (t_last + (int)gridDim.y) / (int)gridDim.y;
+    const int t_beg = (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
+    for (int t = t_beg; t <= t_end; ++t) {
         if (a.replay) {  // positions come from the recorded trajectory
             if (ow >= 0) s_pos[ow] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
             __syncthreads();
@@ -193,13 +196,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                 const int k = 64 * kb + 8 * c8;
                 const float4 b0 = *reinterpret_cast<const float4*>(s_base + e * H + k);
                 const float4 b1 = *reinterpret_cast<const float4*>(s_base + e * H + k + 4);
-                split2<0>(fmaxf(b0.x + w[kb][0].x, 0.f), fmaxf(b0.y + w[kb][0].y, 0.f), hi[kb].x, lo[kb].x);
-                split2<0>(fmaxf(b0.z + w[kb][0].z, 0.f), fmaxf(b0.w + w[kb][0].w, 0.f), hi[kb].y, lo[kb].y);
-                split2<0>(fmaxf(b1.x + w[kb][1].x, 0.f), fmaxf(b1.y + w[kb][1].y, 0.f), hi[kb].z, lo[kb].z);
-                split2<0>(fmaxf(b1.z + w[kb][1].z, 0.f), fmaxf(b1.w + w[kb][1].w, 0.f), hi[kb].w, lo[kb].w);
+                split2<PREC>(fmaxf(b0.x + w[kb][0].x, 0.f), fmaxf(b0.y + w[kb][0].y, 0.f), hi[kb].x, lo[kb].x);
+                split2<PREC>(fmaxf(b0.z + w[kb][0].z, 0.f), fmaxf(b0.w + w[kb][0].w, 0.f), hi[kb].y, lo[kb].y);
+                split2<PREC>(fmaxf(b1.x + w[kb][1].x, 0.f), fmaxf(b1.y + w[kb][1].y, 0.f), hi[kb].z, lo[kb].z);
+                split2<PREC>(fmaxf(b1.z + w[kb][1].z, 0.f), fmaxf(b1.w + w[kb][1].w, 0.f), hi[kb].w, lo[kb].w);
                 unsigned char* row = s_bop + kb * Cfg::B_CHUNK + e * 128 + ((c8 ^ (e & 7)) << 4);
                 *reinterpret_cast<uint4*>(row) = hi[kb];
-                *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
+                if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
                 tc::fence_proxy_async();  // ordinary stores -> visible to the tensor cores
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[kb]), 0));
@@ -210,7 +213,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                 for (int kb = 0; kb < 4; ++kb) {
                     const size_t gi = ((size_t)t * B + e0 + e) * H + 64 * kb + 8 * c8;
                     *reinterpret_cast<uint4*>(g_h1hi + gi) = hi[kb];
-                    *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb];
+                    if (PREC == 0) *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb];
                     if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi[kb]);  // the gates of these eight units
                 }
             }
@@ -224,7 +227,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
         if (!worker && rank == 0) {
 #pragma unroll
             for (int kb = 0; kb < 4; ++kb) {
-                ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[kb], (uint32_t)t & 1u));
+                ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[kb], (uint32_t)(t - t_beg) & 1u));
                 tc::tc_fence_after();
                 if (tc::elect_one()) {
 #pragma unroll
@@ -234,8 +237,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                     const uint64_t alo = tc::umma_desc(s_alo + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
                     // B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
                     const uint64_t bd = tc::umma_desc(s_bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
-                    tc::umma_pair(tmem, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                    tc::umma_pair(tmem + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                    if (PREC == 0) {
+                        tc::umma_pair(tmem, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
+                        tc::umma_pair(tmem + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                    } else {  // bf16 operands: one product, the hi rows of the operand tile only
+                        tc::umma_pair(tmem, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                    }
                 }
                 if (kb == 3) tc::umma_commit_pair(tfull, 3);
                 }
@@ -244,18 +251,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
         }
         // ---- heads (workers): thread = hidden unit j, 32 envs of CTA rE
         if (worker) {
-            if (ok) ok = tc::mbar_wait(tfull, (uint32_t)t & 1u);
+            if (ok) ok = tc::mbar_wait(tfull, (uint32_t)(t - t_beg) & 1u);
             tc::tc_fence_after();
             float v[32];
             {
                 uint32_t r0[32], r1[32], r2[32];
                 const uint32_t lanes = tmem + ((uint32_t)(32 * q) << 16);
-                tc::tmem_ld32_nowait(lanes + (uint32_t)(64 * rE), r0);        // W2hi x h1hi
-                tc::tmem_ld32_nowait(lanes + (uint32_t)(64 * rE + 32), r1);   // W2hi x h1lo
-                tc::tmem_ld32_nowait(lanes + 128u + (uint32_t)(32 * rE), r2); // W2lo x h1hi
+                tc::tmem_ld32_nowait(lanes + (uint32_t)((PREC == 0 ? 64 : 32) * rE), r0);  // W2hi x h1hi
+                if (PREC == 0) {
+                    tc::tmem_ld32_nowait(lanes + (uint32_t)(64 * rE + 32), r1);   // W2hi x h1lo
+                    tc::tmem_ld32_nowait(lanes + 128u + (uint32_t)(32 * rE), r2); // W2lo x h1hi
+                }
                 tc::tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) v[e] = fmaxf(((__uint_as_float(r0[e]) + __uint_as_float(r1[e])) + __uint_as_float(r2[e])) + b2j, 0.f);
+                for (int e = 0; e < 32; ++e) {
+                    float z = __uint_as_float(r0[e]);
+                    if (PREC == 0) z = (z + __uint_as_float(r1[e])) + __uint_as_float(r2[e]);
+                    v[e] = rnd<PREC>(fmaxf(z + b2j, 0.f));
+                }
             }
             // head partials over this warp's 32 hidden units on the warp-level tensor path.  The operand tile is free
             // once the step's MMAs have finished: warp w keeps [32 units][32 envs] fp16 hi and lo planes in its 4 KB of it,
@@ -264,13 +277,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
 #pragma unroll
             for (int c4 = 0; c4 < 4; ++c4) {
                 uint4 hi, lo;
-                split2<0>(v[8 * c4 + 0], v[8 * c4 + 1], hi.x, lo.x);
-                split2<0>(v[8 * c4 + 2], v[8 * c4 + 3], hi.y, lo.y);
-                split2<0>(v[8 * c4 + 4], v[8 * c4 + 5], hi.z, lo.z);
-                split2<0>(v[8 * c4 + 6], v[8 * c4 + 7], hi.w, lo.w);
+                split2<PREC>(v[8 * c4 + 0], v[8 * c4 + 1], hi.x, lo.x);
+                split2<PREC>(v[8 * c4 + 2], v[8 * c4 + 3], hi.y, lo.y);
+                split2<PREC>(v[8 * c4 + 4], v[8 * c4 + 5], hi.z, lo.z);
+                split2<PREC>(v[8 * c4 + 6], v[8 * c4 + 7], hi.w, lo.w);
                 const int off = lane * 64 + ((c4 ^ ((lane >> 1) & 3)) << 4);
                 *reinterpret_cast<uint4*>(wsm + off) = hi;
-                *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
+                if (PREC == 0) *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
             }
             __syncwarp();
             float acc[2][4];
@@ -291,11 +304,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                         const int off = krow * 64 + ((chunk ^ ((krow >> 1) & 3)) << 4);
                         uint32_t ahi[4], alo[4];
                         ldmatrix_x4_trans(ahi, wsm + off);
-                        ldmatrix_x4_trans(alo, wsm + 2048 + off);
+                        if (PREC == 0) ldmatrix_x4_trans(alo, wsm + 2048 + off);
                         // the x4 order above is (k lo, m lo), (k lo, m hi), (k hi, m lo), (k hi, m hi) = a0, a1, a2, a3
-                        mma_f16(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
-                        mma_f16(acc[mt], ahi, whf_lo[ks][0], whf_lo[ks][1]);
-                        mma_f16(acc[mt], ahi, whf_hi[ks][0], whf_hi[ks][1]);
+                        if (PREC == 0) {
+                            mma16816<PREC>(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
+                            mma16816<PREC>(acc[mt], ahi, whf_lo[ks][0], whf_lo[ks][1]);
+                        }
+                        mma16816<PREC>(acc[mt], ahi, whf_hi[ks][0], whf_hi[ks][1]);
                     }
                 }
             }
@@ -322,7 +337,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             }
         }
         // ---- one thread per env: once the eight partials are in, their fixed-order sum, then act and step
-        if (!worker && ok) ok = tc::mbar_wait_cluster(pfull, (uint32_t)t & 1u);
+        if (!worker && ok) ok = tc::mbar_wait_cluster(pfull, (uint32_t)(t - t_beg) & 1u);
         // The new positions are all the next step's gather needs: the owners publish them and release the workers (named
         // barrier 1: the workers wait on it, the owner warp only arrives, once and as a whole warp) before they write the
         // step's records.
@@ -388,9 +403,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
 
 // Covers hidden width 256 with fp32 parameters (two-term fp16 operands) when the row-major 16-bit planes of W2 exist;
 // anything else returns cudaErrorNotSupported and the caller takes the warp-level kernel.
-cudaError_t launch_rollout_pair(const RolloutArgs& a0, cudaStream_t s) {
+cudaError_t launch_rollout_pair(const RolloutArgs& a0, int prec, cudaStream_t s) {
     using Cfg = PairCfg;
-    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || !a0.b.w2p_lo || !a0.b.base) return cudaErrorNotSupported;
+    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base) return cudaErrorNotSupported;
     RolloutArgs a = a0;
     size_t smem = Cfg::fixed_bytes + 1024;  // alignment slack
     a.gae_smem = 0;
@@ -400,10 +415,12 @@ cudaError_t launch_rollout_pair(const RolloutArgs& a0, cudaStream_t s) {
     }
     PairMaps maps;
     memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    if (!make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
+    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, prec == 1)) return cudaErrorNotSupported;
+    if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int pairs = (a.d.B + 2 * Cfg::ME - 1) / (2 * Cfg::ME);
-    return launch<k_rollout_pair>(2 * pairs, Cfg::THREADS, smem, s, maps, a);
+    const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
+    if (prec == 1) return launch<k_rollout_pair<1>>(grid, Cfg::THREADS, smem, s, maps, a);
+    return launch<k_rollout_pair<0>>(grid, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

@@ -59,6 +59,7 @@ __device__ __forceinline__ void st_async_f32_2(uint32_t cluster_addr, float v, u
                  : "memory");
 }
 
+template <int PREC>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1) k_rollout_pair2(const __grid_constant__ Pair2Maps maps, RolloutArgs a) {
     using Cfg = Pair2Cfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
@@ -111,14 +112,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     PDL_START();  // (the set-up above runs under the predecessor's tail)
+    // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
+    const int t_last = a.replay == 1 ? a.T - 1 : a.T, t_len = (t_last + (int)gridDim.y) / (int)gridDim.y;
+    const int t_beg = (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
     if (issuer) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
-        tc::mbar_expect_tx(wbar, 2 * Cfg::A_PLANE);
+        tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
 #pragma unroll
         for (int kb = 0; kb < H / 64; ++kb)
 #pragma unroll
             for (int bx = 0; bx < 2; ++bx) {
                 tc::tma_load_2d(s_ahi + (kb * 2 + bx) * Cfg::BOX, &maps.w_hi, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
-                tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
+                if (PREC == 0) tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
             }
     }
     // worker constants
@@ -149,7 +153,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                     const int jj = 128 * (int)rank + 32 * q + 16 * ks + 8 * hh + 2 * t4;
                     const float w0 = n < 5 ? b.theta_c[d.oWh + (size_t)jj * 5 + n] : 0.f;
                     const float w1 = n < 5 ? b.theta_c[d.oWh + (size_t)(jj + 1) * 5 + n] : 0.f;
-                    split2<0>(w0, w1, whf_hi[ks][hh], whf_lo[ks][hh]);
+                    split2<PREC>(w0, w1, whf_hi[ks][hh], whf_lo[ks][hh]);
                 }
         }
         if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
@@ -161,7 +165,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
             s.start = b.start[oenv];
             s.goal = b.goal[oenv];
             check_env_state(s, C, s_walls + ow * 8);
-            if (a.replay) s.pos = min((int)(a.T > 0 ? b.tpos[oenv] : b.pos[oenv]), C - 1);  // row 0 of the recorded positions
+            if (a.replay) s.pos = min((int)(t_beg < a.T ? b.tpos[(size_t)t_beg * B + oenv] : b.pos[oenv]), C - 1);  // the slice's first position
         }
         s_pos[ow] = s.pos;
     }
@@ -172,21 +176,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
-    const int t_end = a.replay == 1 ? a.T - 1 : a.T;  // replay recomputes the T recorded rows (mode 2: and the current state)
 
     if (wid == iwarp) {
         // ---- layer 2: this warp of the leader CTA drives both tensor cores for both groups (one elected lane issues), k block by k block, in the
         // order the groups' operand blocks are written.  A block's sixteen arrivals also say that those warps have read
         // the group's accumulators of the step before.
         if (rank == 0) {
-            const uint32_t idesc_w = tc::umma_idesc<0>(256, 128, true, false), idesc_n = tc::umma_idesc<0>(256, 64, true, false);
-            for (int t = 0; t <= t_end; ++t) {
+            const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, true, false), idesc_n = tc::umma_idesc<PREC>(256, 64, true, false);
+            for (int t = t_beg; t <= t_end; ++t) {
                 for (int g = 0; g < NG; ++g) {
                     const uint32_t acc = tmem + (uint32_t)(g * Cfg::ACC);
                     unsigned char* bop = s_bop + g * Cfg::B_BYTES;
 #pragma unroll
                     for (int kb = 0; kb < 4; ++kb) {
-                        ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[4 * g + kb], (uint32_t)t & 1u));
+                        ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[4 * g + kb], (uint32_t)(t - t_beg) & 1u));
                         tc::tc_fence_after();
                         if (tc::elect_one()) {
 #pragma unroll
@@ -196,8 +199,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                             const uint64_t alo = tc::umma_desc(s_alo + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
                             // B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
                             const uint64_t bd = tc::umma_desc(bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
-                            tc::umma_pair(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                            tc::umma_pair(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            if (PREC == 0) {
+                                tc::umma_pair(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
+                                tc::umma_pair(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            } else {  // bf16 operands: one product, the hi rows of the operand tile only
+                                tc::umma_pair(acc, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            }
                         }
                         if (kb == 3) tc::umma_commit_pair(&tfull[g], 3);
                         }
@@ -236,13 +243,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 for (int kk = 0; kk < 2; ++kk) {
                     const int kb = 2 * half + kk;
                     const float4 b0 = bs[kk][0], b1 = bs[kk][1], w0 = w[kk][0], w1 = w[kk][1];
-                    split2<0>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), hi[kb].x, lo[kb].x);
-                    split2<0>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), hi[kb].y, lo[kb].y);
-                    split2<0>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), hi[kb].z, lo[kb].z);
-                    split2<0>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), hi[kb].w, lo[kb].w);
+                    split2<PREC>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), hi[kb].x, lo[kb].x);
+                    split2<PREC>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), hi[kb].y, lo[kb].y);
+                    split2<PREC>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), hi[kb].z, lo[kb].z);
+                    split2<PREC>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), hi[kb].w, lo[kb].w);
                     unsigned char* row = bop + kb * Cfg::B_CHUNK + e * 128 + ((c8 ^ (e & 7)) << 4);
                     *reinterpret_cast<uint4*>(row) = hi[kb];
-                    *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
+                    if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
                     tc::fence_proxy_async();  // ordinary stores -> visible to the tensor cores
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[4 * g + kb]), 0));
@@ -254,14 +261,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 for (int kb = 0; kb < 4; ++kb) {
                     const size_t gi = ((size_t)t * B + env) * H + 64 * kb + 8 * c8;
                     *reinterpret_cast<uint4*>(g_h1hi + gi) = hi[kb];
-                    *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb];
+                    if (PREC == 0) *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb];
                     if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi[kb]);  // the gates of these eight units
                 }
             }
         };
         // ---- heads of group g for step t: thread = hidden unit j, the group's 32 envs of CTA rE
         auto heads = [&](int g, int t) {
-            if (ok) ok = tc::mbar_wait(&tfull[g], (uint32_t)t & 1u);
+            if (ok) ok = tc::mbar_wait(&tfull[g], (uint32_t)(t - t_beg) & 1u);
             tc::tc_fence_after();
             // sixteen envs at a time (registers): accumulator columns -> bias, ReLU -> the h2 rows for the update -> the
             // fp16 (hi, lo) terms for the head products.  The group's operand tile is free once the step's MMAs have
@@ -276,12 +283,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 float v[16];
                 {
                     uint32_t r0[16], r1[16], r2[16];
-                    tc::tmem_ld16_nowait(lanes + (uint32_t)(64 * rE + 16 * hf), r0);         // W2hi x h1hi
-                    tc::tmem_ld16_nowait(lanes + (uint32_t)(64 * rE + 32 + 16 * hf), r1);    // W2hi x h1lo
-                    tc::tmem_ld16_nowait(lanes + 128u + (uint32_t)(32 * rE + 16 * hf), r2);  // W2lo x h1hi
+                    tc::tmem_ld16_nowait(lanes + (uint32_t)((PREC == 0 ? 64 : 32) * rE + 16 * hf), r0);             // W2hi x h1hi
+                    if (PREC == 0) {
+                        tc::tmem_ld16_nowait(lanes + (uint32_t)(64 * rE + 32 + 16 * hf), r1);         // W2hi x h1lo
+                        tc::tmem_ld16_nowait(lanes + 128u + (uint32_t)(32 * rE + 16 * hf), r2);  // W2lo x h1hi
+                    }
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = fmaxf(((__uint_as_float(r0[e]) + __uint_as_float(r1[e])) + __uint_as_float(r2[e])) + b2j, 0.f);
+                    for (int e = 0; e < 16; ++e) {
+                        float z = __uint_as_float(r0[e]);
+                        if (PREC == 0) z = (z + __uint_as_float(r1[e])) + __uint_as_float(r2[e]);
+                        v[e] = rnd<PREC>(fmaxf(z + b2j, 0.f));
+                    }
                 }
                 if (save_h2) {  // one 128-byte line per env and warp
 #pragma unroll
@@ -292,13 +305,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 for (int c2 = 0; c2 < 2; ++c2) {
                     const int c4 = 2 * hf + c2;
                     uint4 hi, lo;
-                    split2<0>(v[8 * c2 + 0], v[8 * c2 + 1], hi.x, lo.x);
-                    split2<0>(v[8 * c2 + 2], v[8 * c2 + 3], hi.y, lo.y);
-                    split2<0>(v[8 * c2 + 4], v[8 * c2 + 5], hi.z, lo.z);
-                    split2<0>(v[8 * c2 + 6], v[8 * c2 + 7], hi.w, lo.w);
+                    split2<PREC>(v[8 * c2 + 0], v[8 * c2 + 1], hi.x, lo.x);
+                    split2<PREC>(v[8 * c2 + 2], v[8 * c2 + 3], hi.y, lo.y);
+                    split2<PREC>(v[8 * c2 + 4], v[8 * c2 + 5], hi.z, lo.z);
+                    split2<PREC>(v[8 * c2 + 6], v[8 * c2 + 7], hi.w, lo.w);
                     const int off = lane * 64 + ((c4 ^ ((lane >> 1) & 3)) << 4);
                     *reinterpret_cast<uint4*>(wsm + off) = hi;
-                    *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
+                    if (PREC == 0) *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
                 }
             }
             __syncwarp();
@@ -320,10 +333,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                         const int off = krow * 64 + ((chunk ^ ((krow >> 1) & 3)) << 4);
                         uint32_t ahi[4], alo[4];
                         ldmatrix_x4_trans(ahi, wsm + off);
-                        ldmatrix_x4_trans(alo, wsm + 2048 + off);
-                        mma_f16(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
-                        mma_f16(acc[mt], ahi, whf_lo[ks][0], whf_lo[ks][1]);
-                        mma_f16(acc[mt], ahi, whf_hi[ks][0], whf_hi[ks][1]);
+                        if (PREC == 0) ldmatrix_x4_trans(alo, wsm + 2048 + off);
+                        if (PREC == 0) {
+                            mma16816<PREC>(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
+                            mma16816<PREC>(acc[mt], ahi, whf_lo[ks][0], whf_lo[ks][1]);
+                        }
+                        mma16816<PREC>(acc[mt], ahi, whf_hi[ks][0], whf_hi[ks][1]);
                     }
                 }
             }
@@ -346,22 +361,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
             }
         };
         // a group's eight warps walk its steps on their own
-        gather(wg, 0);
-        for (int t = 0; t <= t_end; ++t) {
+        if (t_beg <= t_end) gather(wg, t_beg);
+        for (int t = t_beg; t <= t_end; ++t) {
             heads(wg, t);
             if (t < t_end) {
-                if (ok) ok = tc::mbar_wait(&posrdy[wg], (uint32_t)t & 1u);  // the owners have published the positions after step t
+                if (ok) ok = tc::mbar_wait(&posrdy[wg], (uint32_t)(t - t_beg) & 1u);  // the owners have published the positions after step t
                 gather(wg, t + 1);
             }
         }
     } else if (ownerw) {
         // ---- one thread per env of this CTA (owner warp og serves group og)
-        for (int t = 0; t <= t_end; ++t) {
+        for (int t = t_beg; t <= t_end; ++t) {
             if (lane == 0) tc::mbar_expect_tx(&pfull[og], 8 * ME * 5 * 4);  // this step's head partials, counted as they land
             const bool acting = owner && !a.replay && t < a.T;
             StepPre pre;
             if (acting) pre = step_prepare(s, a, oenv, t, s_walls + ow * 8);
-            if (ok) ok = tc::mbar_wait_cluster(&pfull[og], (uint32_t)t & 1u);
+            if (ok) ok = tc::mbar_wait_cluster(&pfull[og], (uint32_t)(t - t_beg) & 1u);
             float o[5];
 #pragma unroll
             for (int c = 0; c < 5; ++c) o[c] = 0.f;
@@ -421,11 +436,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
 
 // Covers hidden width 256 with fp32 parameters on batches large enough to give every SM pair a cluster of 128 envs;
 // anything else returns cudaErrorNotSupported and the caller takes the one-group CTA-pair kernel.
-cudaError_t launch_rollout_pair2(const RolloutArgs& a0, cudaStream_t s) {
+cudaError_t launch_rollout_pair2(const RolloutArgs& a0, int prec, cudaStream_t s) {
     using Cfg = Pair2Cfg;
     constexpr int PER_PAIR = 2 * Cfg::NG * Cfg::ME;
-    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || !a0.b.w2p_lo || !a0.b.base || a0.d.npol > 1) return cudaErrorNotSupported;
-    if (a0.d.B < 74 * PER_PAIR) return cudaErrorNotSupported;
+    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base || a0.d.npol > 1) return cudaErrorNotSupported;
+    // Acting: beyond one wave of the one-group kernel (74 pairs of 64 envs), whose second wave would cost more than the longer
+    // steps here (6.8 us for 128 envs against 4.3 us for 64).  Replay: whenever a pair has its two groups.
+    if (a0.replay ? a0.d.B < PER_PAIR : a0.d.B <= 74 * PER_PAIR / 2) return cudaErrorNotSupported;
     RolloutArgs a = a0;
     size_t smem = Cfg::fixed_bytes + 1024;  // alignment slack
     a.gae_smem = 0;
@@ -435,10 +452,12 @@ cudaError_t launch_rollout_pair2(const RolloutArgs& a0, cudaStream_t s) {
     }
     Pair2Maps maps;
     memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    if (!make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
+    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, prec == 1)) return cudaErrorNotSupported;
+    if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int pairs = (a.d.B + PER_PAIR - 1) / PER_PAIR;
-    return launch<k_rollout_pair2>(2 * pairs, Cfg::THREADS, smem, s, maps, a);
+    const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
+    if (prec == 1) return launch<k_rollout_pair2<1>>(grid, Cfg::THREADS, smem, s, maps, a);
+    return launch<k_rollout_pair2<0>>(grid, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

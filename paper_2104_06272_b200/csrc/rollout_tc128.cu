@@ -51,6 +51,7 @@ struct Tc128Maps {
     CUtensorMap w_hi, w_lo;  // W2 row-major [k][j] as fp16 planes, boxes of 64 j x 64 k
 };
 
+template <int PREC>
 __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __grid_constant__ Tc128Maps maps, RolloutArgs a) {
     using Cfg = Tc128Cfg;
     constexpr int H = Cfg::H, NE = Cfg::NE, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
@@ -101,14 +102,17 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     PDL_START();  // (the set-up above runs under the predecessor's tail)
+    // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
+    const int t_last = a.replay == 1 ? a.T - 1 : a.T, t_len = (t_last + (int)gridDim.y) / (int)gridDim.y;
+    const int t_beg = (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
     if (issuer) {  // all of W2: box (kb, bx) = k rows 64kb.., columns 64bx..
-        tc::mbar_expect_tx(wbar, 2 * Cfg::A_PLANE);
+        tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
 #pragma unroll
         for (int kb = 0; kb < H / 64; ++kb)
 #pragma unroll
             for (int bx = 0; bx < H / 64; ++bx) {
                 tc::tma_load_2d(s_ahi + (kb * (H / 64) + bx) * Cfg::BOX, &maps.w_hi, wbar, 64 * bx, 64 * kb);
-                tc::tma_load_2d(s_alo + (kb * (H / 64) + bx) * Cfg::BOX, &maps.w_lo, wbar, 64 * bx, 64 * kb);
+                if (PREC == 0) tc::tma_load_2d(s_alo + (kb * (H / 64) + bx) * Cfg::BOX, &maps.w_lo, wbar, 64 * bx, 64 * kb);
             }
     }
     // worker constants: hidden unit of this thread in the heads phase (its accumulator lane) and the env half it reads
@@ -143,7 +147,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                     const int jj = 32 * q + 16 * ks + 8 * hh + 2 * t4;
                     const float w0 = n < 5 ? b.theta_c[d.oWh + (size_t)jj * 5 + n] : 0.f;
                     const float w1 = n < 5 ? b.theta_c[d.oWh + (size_t)(jj + 1) * 5 + n] : 0.f;
-                    split2<0>(w0, w1, whf_hi[ks][hh], whf_lo[ks][hh]);
+                    split2<PREC>(w0, w1, whf_hi[ks][hh], whf_lo[ks][hh]);
                 }
         }
         if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
@@ -156,7 +160,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
             s.start = b.start[e0 + ow];
             s.goal = b.goal[e0 + ow];
             check_env_state(s, C, s_walls + ow * 8);
-            if (a.replay) s.pos = min((int)(a.T > 0 ? b.tpos[e0 + ow] : b.pos[e0 + ow]), C - 1);  // row 0 of the recorded positions
+            if (a.replay) s.pos = min((int)(t_beg < a.T ? b.tpos[(size_t)t_beg * B + e0 + ow] : b.pos[e0 + ow]), C - 1);  // the slice's first position
         }
         s_pos[ow] = s.pos;
     }
@@ -166,20 +170,19 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
-    const int t_end = a.replay == 1 ? a.T - 1 : a.T;  // replay recomputes the T recorded rows (mode 2: and the current state)
 
     if (wid == (NWT + NOWN) / 32) {
         // ---- layer 2: one warp drives the tensor core for both groups (an elected lane issues), k block by k block, in the order the groups'
         // operand blocks are written (group 0, then group 1, every step).  A block's eight arrivals also say that those
         // warps have read the group's accumulators of the step before.
-        const uint32_t idesc_w = tc::umma_idesc<0>(128, 128, true, false), idesc_n = tc::umma_idesc<0>(128, 64, true, false);
-        for (int t = 0; t <= t_end; ++t) {
+        const uint32_t idesc_w = tc::umma_idesc<PREC>(128, 128, true, false), idesc_n = tc::umma_idesc<PREC>(128, 64, true, false);
+        for (int t = t_beg; t <= t_end; ++t) {
             for (int g = 0; g < NG; ++g) {
                 const uint32_t acc = tmem + (uint32_t)(g * Cfg::ACC);
                 unsigned char* bop = s_bop + g * Cfg::B_BYTES;
 #pragma unroll
                 for (int kb = 0; kb < 2; ++kb) {
-                    ok = tc::warp_all(ok && tc::mbar_wait(&ready[2 * g + kb], (uint32_t)t & 1u));
+                    ok = tc::warp_all(ok && tc::mbar_wait(&ready[2 * g + kb], (uint32_t)(t - t_beg) & 1u));
                     tc::tc_fence_after();
                     if (tc::elect_one()) {
 #pragma unroll
@@ -189,8 +192,12 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                         const uint64_t alo = tc::umma_desc(s_alo + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
                         // B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
                         const uint64_t bd = tc::umma_desc(bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
-                        tc::umma(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                        tc::umma(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                        if (PREC == 0) {
+                            tc::umma(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
+                            tc::umma(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                        } else {  // bf16 operands: one product, the hi rows of the operand tile only
+                            tc::umma(acc, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                        }
                     }
                     if (kb == 1) tc::umma_commit(&tfull[g]);
                     }
@@ -229,13 +236,13 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                     const float4 b0 = *reinterpret_cast<const float4*>(bp);
                     const float4 b1 = *reinterpret_cast<const float4*>(bp + 4);
                     const float4 w0 = w[kb][p][0], w1 = w[kb][p][1];
-                    split2<0>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), hi[kb][p].x, lo[kb][p].x);
-                    split2<0>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), hi[kb][p].y, lo[kb][p].y);
-                    split2<0>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), hi[kb][p].z, lo[kb][p].z);
-                    split2<0>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), hi[kb][p].w, lo[kb][p].w);
+                    split2<PREC>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), hi[kb][p].x, lo[kb][p].x);
+                    split2<PREC>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), hi[kb][p].y, lo[kb][p].y);
+                    split2<PREC>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), hi[kb][p].z, lo[kb][p].z);
+                    split2<PREC>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), hi[kb][p].w, lo[kb][p].w);
                     unsigned char* row = bop + kb * Cfg::B_CHUNK + er * 128 + ((c8 ^ (er & 7)) << 4);
                     *reinterpret_cast<uint4*>(row) = hi[kb][p];
-                    *reinterpret_cast<uint4*>(row + NE * 128) = lo[kb][p];
+                    if (PREC == 0) *reinterpret_cast<uint4*>(row + NE * 128) = lo[kb][p];
                 }
                 tc::fence_proxy_async();  // ordinary stores -> visible to the tensor core
                 __syncwarp();
@@ -251,7 +258,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                         for (int kb = 0; kb < 2; ++kb) {
                             const size_t gi = ((size_t)t * B + env) * H + 64 * kb + 8 * c8;
                             *reinterpret_cast<uint4*>(g_h1hi + gi) = hi[kb][p];
-                            *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb][p];
+                            if (PREC == 0) *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb][p];
                             if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi[kb][p]);  // the gates of these eight units
                         }
                     }
@@ -260,7 +267,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         };
         // ---- heads of group g for step t: thread = hidden unit j, the 32 envs of its half of the group
         auto heads = [&](int g, int t) {
-            if (ok) ok = tc::mbar_wait(&tfull[g], (uint32_t)t & 1u);
+            if (ok) ok = tc::mbar_wait(&tfull[g], (uint32_t)(t - t_beg) & 1u);
             tc::tc_fence_after();
             // sixteen envs at a time (registers): accumulator columns -> bias, ReLU -> the h2 rows for the update -> the
             // fp16 (hi, lo) terms for the head products.  The group's operand tile is free once the step's MMAs have
@@ -275,12 +282,18 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                 float v[16];
                 {
                     uint32_t r0[16], r1[16], r2[16];
-                    tc::tmem_ld16_nowait(lanes + (uint32_t)(32 * half + 16 * hf), r0);         // W2hi x h1hi
-                    tc::tmem_ld16_nowait(lanes + (uint32_t)(NE + 32 * half + 16 * hf), r1);    // W2hi x h1lo
-                    tc::tmem_ld16_nowait(lanes + 128u + (uint32_t)(32 * half + 16 * hf), r2);  // W2lo x h1hi
+                    tc::tmem_ld16_nowait(lanes + (uint32_t)(32 * half + 16 * hf), r0);             // W2hi x h1hi
+                    if (PREC == 0) {
+                        tc::tmem_ld16_nowait(lanes + (uint32_t)(NE + 32 * half + 16 * hf), r1);         // W2hi x h1lo
+                        tc::tmem_ld16_nowait(lanes + 128u + (uint32_t)(32 * half + 16 * hf), r2);  // W2lo x h1hi
+                    }
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = fmaxf(((__uint_as_float(r0[e]) + __uint_as_float(r1[e])) + __uint_as_float(r2[e])) + b2j, 0.f);
+                    for (int e = 0; e < 16; ++e) {
+                        float z = __uint_as_float(r0[e]);
+                        if (PREC == 0) z = (z + __uint_as_float(r1[e])) + __uint_as_float(r2[e]);
+                        v[e] = rnd<PREC>(fmaxf(z + b2j, 0.f));
+                    }
                 }
                 if (save_h2) {  // one 128-byte line per env and warp
 #pragma unroll
@@ -291,13 +304,13 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                 for (int c2 = 0; c2 < 2; ++c2) {
                     const int c4 = 2 * hf + c2;
                     uint4 hi, lo;
-                    split2<0>(v[8 * c2 + 0], v[8 * c2 + 1], hi.x, lo.x);
-                    split2<0>(v[8 * c2 + 2], v[8 * c2 + 3], hi.y, lo.y);
-                    split2<0>(v[8 * c2 + 4], v[8 * c2 + 5], hi.z, lo.z);
-                    split2<0>(v[8 * c2 + 6], v[8 * c2 + 7], hi.w, lo.w);
+                    split2<PREC>(v[8 * c2 + 0], v[8 * c2 + 1], hi.x, lo.x);
+                    split2<PREC>(v[8 * c2 + 2], v[8 * c2 + 3], hi.y, lo.y);
+                    split2<PREC>(v[8 * c2 + 4], v[8 * c2 + 5], hi.z, lo.z);
+                    split2<PREC>(v[8 * c2 + 6], v[8 * c2 + 7], hi.w, lo.w);
                     const int off = lane * 64 + ((c4 ^ ((lane >> 1) & 3)) << 4);
                     *reinterpret_cast<uint4*>(wsm + off) = hi;
-                    *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
+                    if (PREC == 0) *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
                 }
             }
             __syncwarp();
@@ -319,10 +332,12 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                         const int off = krow * 64 + ((chunk ^ ((krow >> 1) & 3)) << 4);
                         uint32_t ahi[4], alo[4];
                         ldmatrix_x4_trans(ahi, wsm + off);
-                        ldmatrix_x4_trans(alo, wsm + 2048 + off);
-                        mma_f16(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
-                        mma_f16(acc[mt], ahi, whf_lo[ks][0], whf_lo[ks][1]);
-                        mma_f16(acc[mt], ahi, whf_hi[ks][0], whf_hi[ks][1]);
+                        if (PREC == 0) ldmatrix_x4_trans(alo, wsm + 2048 + off);
+                        if (PREC == 0) {
+                            mma16816<PREC>(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
+                            mma16816<PREC>(acc[mt], ahi, whf_lo[ks][0], whf_lo[ks][1]);
+                        }
+                        mma16816<PREC>(acc[mt], ahi, whf_hi[ks][0], whf_hi[ks][1]);
                     }
                 }
             }
@@ -344,11 +359,11 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         };
         // a group's eight warps walk its steps on their own; the two groups drift apart by themselves, so that one group's
         // tensor-core and sampling phases fall into the other's gather and heads phases
-        gather(wg, 0);
-        for (int t = 0; t <= t_end; ++t) {
+        if (t_beg <= t_end) gather(wg, t_beg);
+        for (int t = t_beg; t <= t_end; ++t) {
             heads(wg, t);
             if (t < t_end) {
-                if (ok) ok = tc::mbar_wait(&posrdy[wg], (uint32_t)t & 1u);  // the owners have published the positions after step t
+                if (ok) ok = tc::mbar_wait(&posrdy[wg], (uint32_t)(t - t_beg) & 1u);  // the owners have published the positions after step t
                 gather(wg, t + 1);
             }
         }
@@ -356,12 +371,12 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         // ---- one thread per env
         const int env = e0 + ow;
         const int oe = ow - og * NE;  // env index within the group
-        for (int t = 0; t <= t_end; ++t) {
+        for (int t = t_beg; t <= t_end; ++t) {
             // the logits-independent half of the interaction, while the workers gather and the tensor core runs
             const bool acting = owner && !a.replay && t < a.T;
             StepPre pre;
             if (acting) pre = step_prepare(s, a, env, t, s_walls + ow * 8);
-            if (ok) ok = tc::mbar_wait(&pdone[og], (uint32_t)t & 1u);
+            if (ok) ok = tc::mbar_wait(&pdone[og], (uint32_t)(t - t_beg) & 1u);
             float o[5];
 #pragma unroll
             for (int c = 0; c < 5; ++c) o[c] = 0.f;
@@ -419,10 +434,12 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
 
 // Covers hidden width 128 with fp32 parameters (two-term fp16 operands) on batches large enough to give every SM a CTA
 // of 128 envs; anything else returns cudaErrorNotSupported and the caller takes the warp-level kernel.
-cudaError_t launch_rollout_tc128(const RolloutArgs& a0, cudaStream_t s) {
+cudaError_t launch_rollout_tc128(const RolloutArgs& a0, int prec, cudaStream_t s) {
     using Cfg = Tc128Cfg;
-    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || !a0.b.w2p_lo || !a0.b.base || a0.d.npol > 1) return cudaErrorNotSupported;
-    if (a0.d.B < 148 * Cfg::NOWN) return cudaErrorNotSupported;
+    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base || a0.d.npol > 1) return cudaErrorNotSupported;
+    // Acting: beyond one wave of the warp-level kernel (two CTAs of 32 envs per SM), whose step takes 4.4 us against 5.8 us here.
+    // Replay: whenever a CTA's two groups have envs.
+    if (a0.replay ? a0.d.B <= Cfg::NE : a0.d.B <= 148 * 64) return cudaErrorNotSupported;
     RolloutArgs a = a0;
     size_t smem = Cfg::fixed_bytes + 1024;  // alignment slack
     a.gae_smem = 0;
@@ -432,9 +449,12 @@ cudaError_t launch_rollout_tc128(const RolloutArgs& a0, cudaStream_t s) {
     }
     Tc128Maps maps;
     memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    if (!make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
-    return launch<k_rollout_tc128>((a.d.B + Cfg::NOWN - 1) / Cfg::NOWN, Cfg::THREADS, smem, s, maps, a);
+    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, prec == 1)) return cudaErrorNotSupported;
+    if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
+    const int ctas = (a.d.B + Cfg::NOWN - 1) / Cfg::NOWN;
+    const dim3 grid(ctas, replay_slices(a, ctas));
+    if (prec == 1) return launch<k_rollout_tc128<1>>(grid, Cfg::THREADS, smem, s, maps, a);
+    return launch<k_rollout_tc128<0>>(grid, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

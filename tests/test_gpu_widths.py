@@ -15,6 +15,8 @@ CASES = [
     # the warp-level kernels' widths: batches around a CTA's 32 envs and a dh1 tile's 64, one and several t-slices
     (32, 0, 33, 5, 3), (32, 1, 65, 4, 2), (96, 0, 2, 3, 4), (96, 0, 777, 7, 20), (96, 1, 64, 12, 5), (192, 0, 100, 6, 9),
     (192, 0, 5, 4, 55), (192, 1, 2100, 5, 3), (64, 0, 1500, 5, 9), (64, 1, 31, 6, 33),
+    # just beyond one wave of the smaller-batch rollouts at H = 128 and 256
+    (128, 0, 9473, 4, 2), (128, 1, 9500, 5, 3), (256, 0, 4737, 4, 2), (256, 1, 4800, 5, 3),
 ]
 
 
@@ -37,3 +39,23 @@ def test_width_one_iteration_stage_by_stage(bnd, H, prec, B, N, T):
         par.check_iteration(an, bnd, w, 11)
     finally:
         print(w.name, "worst error / bound:", {k: round(v, 3) for k, v in par.MARGINS.items()})
+
+
+@pytest.mark.parametrize("H,prec,B,T", [(32, 0, 40, 7), (64, 0, 33, 9), (96, 1, 70, 5), (128, 0, 65, 11), (128, 1, 200, 4), (256, 0, 127, 6), (256, 0, 300, 9),
+                                        (256, 1, 129, 7), (384, 0, 70, 5)])
+def test_replayed_forward_pass_equals_the_rollouts_own(bnd, H, prec, B, T):
+    """The update of a trajectory handed back through set() recomputes the forward pass in slices of steps (few envs), and must
+    give the gradient of the update that reuses the rollout's activations."""
+    w = Workload("replay", B=B, N=5, H=H, T=T, iters=1, precision=prec, episode_cap=6)
+    grads = []
+    for hand_back in (False, True):
+        an = bnd.Anakin(bnd.cfg_from_workload(w))
+        an.reset(3)
+        an.set(bnd.PARAMS, random_params(5, w.P, 0.15 if H <= 256 else 0.05))
+        an.rollout()
+        if hand_back:
+            an.set(bnd.TRAJ_POS, an.get(bnd.TRAJ_POS))
+        an.learn()
+        grads.append(an.get(bnd.GRADS))
+        assert an.status() == 0
+    par.assert_close(grads[1], grads[0], par.rtol_of(prec), "replayed gradient")
