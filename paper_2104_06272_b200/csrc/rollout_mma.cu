@@ -103,7 +103,7 @@ struct RolloutMmaCfg {
 // OWN: the per-env part of a step (one lane per env) has a warp of its own beside the NW workers, which meets them at named
 // barriers: the logits-independent half of an interaction runs under the gather, and the records are written after the workers
 // have been given the new positions.  Otherwise warp 0 does both (the wide kernels' registers leave no room for another warp).
-template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
+template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN, bool REPLAY>
 __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(RolloutArgs a_in) {
     PDL_START();
     const PolicyArgs<GROUPED, RolloutArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
@@ -184,12 +184,13 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
     const size_t h1_plane = (size_t)B * d.Tmax * H;
     // Replay recomputes the T recorded rows (mode 2: and the current state).  Its steps are independent of one another, so a
     // launch for few envs cuts them into slices (grid.y).
-    const int t_last = a.replay == 1 ? a.T - 1 : a.T, slices = GROUPED ? 1 : (int)gridDim.y, t_len = (t_last + slices) / slices;
-    const int t_beg = GROUPED ? 0 : (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
+    constexpr bool SLICED = REPLAY && !GROUPED;
+    const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = SLICED ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
+    const int t_beg = SLICED ? (int)blockIdx.y * t_len : 0, t_end = SLICED ? min(t_last, t_beg + t_len - 1) : t_last;
     auto recorded_pos = [&](int t) {  // replay: the position of this thread's env at step t (row T: the env state as it stands)
         return owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
     };
-    if (a.replay) {
+    if (REPLAY) {
         if (ownw) s_pos[ow] = recorded_pos(t_beg);
         __syncthreads();
     }
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
                 s_pos[ow] = s.pos;
             }
         }
-        if (a.replay && ownw && t < t_end) s_pos[ow] = recorded_pos(t + 1);
+        if (REPLAY && ownw && t < t_end) s_pos[ow] = recorded_pos(t + 1);
         publish();
         if (owner) {
             const int env = e0 + ow;
@@ -405,8 +406,8 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
                 o5[0] = make_float4(o[0], o[1], o[2], o[3]);
                 o5[1] = make_float4(o[4], 0.f, 0.f, 0.f);
             }
-            if (a.replay == 2 && t == a.T) b.vboot[env] = o[4];
-            if (!a.replay) {
+            if (REPLAY && a.replay == 2 && t == a.T) b.vboot[env] = o[4];
+            if (!REPLAY) {
                 b.tval[(size_t)t * B + env] = o[4];
                 if (a.gae_smem) s_gv[t * ME + ow] = o[4];
                 if (acting) {
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             }
         } else {
             for (int t = t_beg; t <= t_end; ++t) {
-                const bool acting = owner && !a.replay && t < a.T;
+                const bool acting = owner && !REPLAY && t < a.T;
                 StepPre pre;
                 if (acting) pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
                 asm volatile("bar.sync 2, %0;" ::"n"(NALL) : "memory");
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             __syncthreads();
             // the logits-independent half of the interaction waits in shared memory (two words per env) rather than in
             // registers, which the MMA loop needs
-            const bool acting = owner && !a.replay && t < a.T;
+            const bool acting = owner && !REPLAY && t < a.T;
             if (acting) {
                 const StepPre pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
                 s_pre[ow] = make_uint2(__float_as_uint(pre.u), (uint32_t)pre.np[0] | ((uint32_t)pre.np[1] << 8) | ((uint32_t)pre.np[2] << 16) | ((uint32_t)pre.np[3] << 24));
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             __syncthreads();
         }
     }
-    if (a.replay) return;
+    if (REPLAY) return;
     if (owner) {
         b.pos[e0 + ow] = (uint8_t)s.pos;
         b.tep[e0 + ow] = (uint8_t)s.tep;
@@ -478,7 +479,8 @@ constexpr size_t MAX_DYN_SMEM = 232448;  // 227 KB of dynamic shared memory per 
 
 template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
 static cudaError_t launch_k(const RolloutArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-    return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
+    if (a.replay) return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN, true>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
+    return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN, false>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
 }
 
 template <int H, int NW, int PREC, bool GROUPED = false>

@@ -55,7 +55,7 @@ __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uin
                  : "memory");
 }
 
-template <int PREC>
+template <int PREC, bool REPLAY>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(const __grid_constant__ PairMaps maps, RolloutArgs a) {
     using Cfg = PairCfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NWT = Cfg::NWORK * 32;
@@ -166,10 +166,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
     const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, true, false), idesc_n = tc::umma_idesc<PREC>(256, 64, true, false);
 
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
-    const int t_last = a.replay == 1 ? a.T - 1 : a.T, t_len = (t_last + (int)gridDim.y) / (int)gridDim.y;
-    const int t_beg = (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
+    const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
+    const int t_beg = REPLAY ? (int)blockIdx.y * t_len : 0, t_end = REPLAY ? min(t_last, t_beg + t_len - 1) : t_last;
     for (int t = t_beg; t <= t_end; ++t) {
-        if (a.replay) {  // positions come from the recorded trajectory
+        if (REPLAY) {  // positions come from the recorded trajectory
             if (ow >= 0) s_pos[ow] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
             __syncthreads();
         }
@@ -219,7 +219,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             }
         }
         // the logits-independent half of the interaction, taken by the owner warp while the workers gather
-        const bool acting = owner && !a.replay && t < a.T;
+        const bool acting = owner && !REPLAY && t < a.T;
         StepPre pre;
         if (acting) pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
         // ---- layer 2: the leader's owner warp drives both tensor cores, k block by k block (the whole warp waits, one elected
@@ -369,8 +369,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                     o5[0] = make_float4(o[0], o[1], o[2], o[3]);
                     o5[1] = make_float4(o[4], 0.f, 0.f, 0.f);
                 }
-                if (a.replay == 2 && t == a.T) b.vboot[env] = o[4];
-                if (!a.replay) {
+                if (REPLAY && a.replay == 2 && t == a.T) b.vboot[env] = o[4];
+                if (!REPLAY) {
                     b.tval[(size_t)t * B + env] = o[4];
                     if (a.gae_smem) s_gv[t * ME + ow] = o[4];
                 }
@@ -384,13 +384,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             asm volatile("bar.sync 1, %0;" ::"n"(Cfg::THREADS) : "memory");
         }
     }
-    if (owner && !a.replay) {
+    if (owner && !REPLAY) {
         b.pos[e0 + ow] = (uint8_t)s.pos;
         b.tep[e0 + ow] = (uint8_t)s.tep;
         if (a.gae_smem) gae_scan_env_smem(b, B, a.T, e0 + ow, a.gamma, a.lambda, s_gv, s_gc, ME, ow);
         else if (a.fuse_gae) gae_scan_env(b, B, a.T, e0 + ow, a.gamma, a.lambda);
     }
-    if (!worker && !a.replay) flush_env_stats(s, a);
+    if (!worker && !REPLAY) flush_env_stats(s, a);
     if (!ok && lane == 0) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
     // neither CTA frees tensor memory or leaves while the other may still signal it
     tc::tc_fence_before();
@@ -419,8 +419,8 @@ cudaError_t launch_rollout_pair(const RolloutArgs& a0, int prec, cudaStream_t s)
     if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int pairs = (a.d.B + 2 * Cfg::ME - 1) / (2 * Cfg::ME);
     const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
-    if (prec == 1) return launch<k_rollout_pair<1>>(grid, Cfg::THREADS, smem, s, maps, a);
-    return launch<k_rollout_pair<0>>(grid, Cfg::THREADS, smem, s, maps, a);
+    if (prec == 1) return a.replay ? launch<k_rollout_pair<1, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_pair<1, false>>(grid, Cfg::THREADS, smem, s, maps, a);
+    return a.replay ? launch<k_rollout_pair<0, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_pair<0, false>>(grid, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

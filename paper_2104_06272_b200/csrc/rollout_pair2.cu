@@ -59,7 +59,7 @@ __device__ __forceinline__ void st_async_f32_2(uint32_t cluster_addr, float v, u
                  : "memory");
 }
 
-template <int PREC>
+template <int PREC, bool REPLAY>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1) k_rollout_pair2(const __grid_constant__ Pair2Maps maps, RolloutArgs a) {
     using Cfg = Pair2Cfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
@@ -113,8 +113,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     const uint32_t tmem = *tmem_slot;
     PDL_START();  // (the set-up above runs under the predecessor's tail)
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
-    const int t_last = a.replay == 1 ? a.T - 1 : a.T, t_len = (t_last + (int)gridDim.y) / (int)gridDim.y;
-    const int t_beg = (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
+    const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
+    const int t_beg = REPLAY ? (int)blockIdx.y * t_len : 0, t_end = REPLAY ? min(t_last, t_beg + t_len - 1) : t_last;
     if (issuer) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
         tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
 #pragma unroll
@@ -165,7 +165,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
             s.start = b.start[oenv];
             s.goal = b.goal[oenv];
             check_env_state(s, C, s_walls + ow * 8);
-            if (a.replay) s.pos = min((int)(t_beg < a.T ? b.tpos[(size_t)t_beg * B + oenv] : b.pos[oenv]), C - 1);  // the slice's first position
+            if (REPLAY) s.pos = min((int)(t_beg < a.T ? b.tpos[(size_t)t_beg * B + oenv] : b.pos[oenv]), C - 1);  // the slice's first position
         }
         s_pos[ow] = s.pos;
     }
@@ -373,7 +373,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
         // ---- one thread per env of this CTA (owner warp og serves group og)
         for (int t = t_beg; t <= t_end; ++t) {
             if (lane == 0) tc::mbar_expect_tx(&pfull[og], 8 * ME * 5 * 4);  // this step's head partials, counted as they land
-            const bool acting = owner && !a.replay && t < a.T;
+            const bool acting = owner && !REPLAY && t < a.T;
             StepPre pre;
             if (acting) pre = step_prepare(s, a, oenv, t, s_walls + ow * 8);
             if (ok) ok = tc::mbar_wait_cluster(&pfull[og], (uint32_t)(t - t_beg) & 1u);
@@ -393,7 +393,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 if (acting) {
                     ao = act_decide(s, a, oenv, t, o[0], o[1], o[2], o[3], pre);
                     s_pos[ow] = s.pos;
-                } else if (a.replay && t < t_end) {  // positions come from the recorded trajectory (row T: the env state as it stands)
+                } else if (REPLAY && t < t_end) {  // positions come from the recorded trajectory (row T: the env state as it stands)
                     s_pos[ow] = min((int)(t + 1 < a.T ? b.tpos[(size_t)(t + 1) * B + oenv] : b.pos[oenv]), C - 1);
                 }
             }
@@ -405,8 +405,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                     o5[0] = make_float4(o[0], o[1], o[2], o[3]);
                     o5[1] = make_float4(o[4], 0.f, 0.f, 0.f);
                 }
-                if (a.replay == 2 && t == a.T) b.vboot[oenv] = o[4];
-                if (!a.replay) {
+                if (REPLAY && a.replay == 2 && t == a.T) b.vboot[oenv] = o[4];
+                if (!REPLAY) {
                     b.tval[(size_t)t * B + oenv] = o[4];
                     if (a.gae_smem) s_gv[t * NOWN + ow] = o[4];
                 }
@@ -416,13 +416,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 }
             }
         }
-        if (owner && !a.replay) {
+        if (owner && !REPLAY) {
             b.pos[oenv] = (uint8_t)s.pos;
             b.tep[oenv] = (uint8_t)s.tep;
             if (a.gae_smem) gae_scan_env_smem(b, B, a.T, oenv, a.gamma, a.lambda, s_gv, s_gc, NOWN, ow);
             else if (a.fuse_gae) gae_scan_env(b, B, a.T, oenv, a.gamma, a.lambda);
         }
-        if (!a.replay) flush_env_stats(s, a, wid == NWT / 32);
+        if (!REPLAY) flush_env_stats(s, a, wid == NWT / 32);
     }
     if (!ok && lane == 0) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
     // neither CTA frees tensor memory or leaves while the other may still signal it
@@ -456,8 +456,8 @@ cudaError_t launch_rollout_pair2(const RolloutArgs& a0, int prec, cudaStream_t s
     if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int pairs = (a.d.B + PER_PAIR - 1) / PER_PAIR;
     const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
-    if (prec == 1) return launch<k_rollout_pair2<1>>(grid, Cfg::THREADS, smem, s, maps, a);
-    return launch<k_rollout_pair2<0>>(grid, Cfg::THREADS, smem, s, maps, a);
+    if (prec == 1) return a.replay ? launch<k_rollout_pair2<1, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_pair2<1, false>>(grid, Cfg::THREADS, smem, s, maps, a);
+    return a.replay ? launch<k_rollout_pair2<0, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_pair2<0, false>>(grid, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin

@@ -51,7 +51,7 @@ struct Tc128Maps {
     CUtensorMap w_hi, w_lo;  // W2 row-major [k][j] as fp16 planes, boxes of 64 j x 64 k
 };
 
-template <int PREC>
+template <int PREC, bool REPLAY>
 __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __grid_constant__ Tc128Maps maps, RolloutArgs a) {
     using Cfg = Tc128Cfg;
     constexpr int H = Cfg::H, NE = Cfg::NE, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
     const uint32_t tmem = *tmem_slot;
     PDL_START();  // (the set-up above runs under the predecessor's tail)
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
-    const int t_last = a.replay == 1 ? a.T - 1 : a.T, t_len = (t_last + (int)gridDim.y) / (int)gridDim.y;
-    const int t_beg = (int)blockIdx.y * t_len, t_end = min(t_last, t_beg + t_len - 1);
+    const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
+    const int t_beg = REPLAY ? (int)blockIdx.y * t_len : 0, t_end = REPLAY ? min(t_last, t_beg + t_len - 1) : t_last;
     if (issuer) {  // all of W2: box (kb, bx) = k rows 64kb.., columns 64bx..
         tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
 #pragma unroll
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
             s.start = b.start[e0 + ow];
             s.goal = b.goal[e0 + ow];
             check_env_state(s, C, s_walls + ow * 8);
-            if (a.replay) s.pos = min((int)(t_beg < a.T ? b.tpos[(size_t)t_beg * B + e0 + ow] : b.pos[e0 + ow]), C - 1);  // the slice's first position
+            if (REPLAY) s.pos = min((int)(t_beg < a.T ? b.tpos[(size_t)t_beg * B + e0 + ow] : b.pos[e0 + ow]), C - 1);  // the slice's first position
         }
         s_pos[ow] = s.pos;
     }
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         const int oe = ow - og * NE;  // env index within the group
         for (int t = t_beg; t <= t_end; ++t) {
             // the logits-independent half of the interaction, while the workers gather and the tensor core runs
-            const bool acting = owner && !a.replay && t < a.T;
+            const bool acting = owner && !REPLAY && t < a.T;
             StepPre pre;
             if (acting) pre = step_prepare(s, a, env, t, s_walls + ow * 8);
             if (ok) ok = tc::mbar_wait(&pdone[og], (uint32_t)(t - t_beg) & 1u);
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                 if (acting) {
                     ao = act_decide(s, a, env, t, o[0], o[1], o[2], o[3], pre);
                     s_pos[ow] = s.pos;
-                } else if (a.replay && t < t_end) {  // positions come from the recorded trajectory (row T: the env state as it stands)
+                } else if (REPLAY && t < t_end) {  // positions come from the recorded trajectory (row T: the env state as it stands)
                     s_pos[ow] = min((int)(t + 1 < a.T ? b.tpos[(size_t)(t + 1) * B + env] : b.pos[env]), C - 1);
                 }
             }
@@ -405,8 +405,8 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                     o5[0] = make_float4(o[0], o[1], o[2], o[3]);
                     o5[1] = make_float4(o[4], 0.f, 0.f, 0.f);
                 }
-                if (a.replay == 2 && t == a.T) b.vboot[env] = o[4];
-                if (!a.replay) {
+                if (REPLAY && a.replay == 2 && t == a.T) b.vboot[env] = o[4];
+                if (!REPLAY) {
                     b.tval[(size_t)t * B + env] = o[4];
                     if (a.gae_smem) s_gv[t * NOWN + ow] = o[4];
                 }
@@ -416,13 +416,13 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                 }
             }
         }
-        if (owner && !a.replay) {
+        if (owner && !REPLAY) {
             b.pos[env] = (uint8_t)s.pos;
             b.tep[env] = (uint8_t)s.tep;
             if (a.gae_smem) gae_scan_env_smem(b, B, a.T, env, a.gamma, a.lambda, s_gv, s_gc, NOWN, ow);
             else if (a.fuse_gae) gae_scan_env(b, B, a.T, env, a.gamma, a.lambda);
         }
-        if (!a.replay) flush_env_stats(s, a, wid == NWT / 32);
+        if (!REPLAY) flush_env_stats(s, a, wid == NWT / 32);
     }
     if (!ok && lane == 0) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
     tc::tc_fence_before();
@@ -453,8 +453,8 @@ cudaError_t launch_rollout_tc128(const RolloutArgs& a0, int prec, cudaStream_t s
     if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int ctas = (a.d.B + Cfg::NOWN - 1) / Cfg::NOWN;
     const dim3 grid(ctas, replay_slices(a, ctas));
-    if (prec == 1) return launch<k_rollout_tc128<1>>(grid, Cfg::THREADS, smem, s, maps, a);
-    return launch<k_rollout_tc128<0>>(grid, Cfg::THREADS, smem, s, maps, a);
+    if (prec == 1) return a.replay ? launch<k_rollout_tc128<1, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_tc128<1, false>>(grid, Cfg::THREADS, smem, s, maps, a);
+    return a.replay ? launch<k_rollout_tc128<0, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_tc128<0, false>>(grid, Cfg::THREADS, smem, s, maps, a);
 }
 
 }  // namespace anakin
