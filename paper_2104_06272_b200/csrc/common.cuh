@@ -195,7 +195,7 @@ struct LearnArgs {
     // tensor-pipe path
     int ts;               // t-slices of the dh1 kernel: S holds ts*B rows (slice z, env b at row z*B + b)
     float gscale, inv_gscale;  // power of two carried by every gradient-side tensor, divided out in the reduction
-    float* part_small;    // per (CTA, row group) partials of dWh | db2 | dbh
+    float* part_small;    // per-CTA partials of dWh | db2 | dbh
     size_t small_stride;
     PartRegion reg[NREG];
 };
@@ -422,6 +422,9 @@ constexpr int DH1A_UNITS = 128;  // hidden units (columns of dh1) one CTA of the
 bool dh1_agent_tc_supported(const Dims& d);
 // dh1, S and the agent plane of dW1 in one tcgen05 kernel; cudaErrorNotSupported if not covered
 cudaError_t launch_dh1_agent_tc(const LearnArgs& a, int prec, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s);
+void back64_shape(const Dims& d, int T, int* nx, int* ts);  // hidden width 64: dh1, S, dW2 and the agent plane in one kernel
+constexpr int BACK64_SLICES = 16;
+cudaError_t launch_back64(const LearnArgs& a, int prec, int nx, float* part_w2, float* part_agent, size_t stride_agent, cudaStream_t s);
 cudaError_t launch_dh1_tc(const LearnArgs& a, int prec, cudaStream_t s);  // tcgen05 dh1 kernel; cudaErrorNotSupported if not covered  // needs the activations the rollout saved
 cudaError_t launch_selftest_wait(int* status, long long limit_clocks, long long* waited_clocks, cudaStream_t s);
 cudaError_t launch_refresh_compute_params(const Dims& d, const Buffers& b, int prec, const Ctx& c);

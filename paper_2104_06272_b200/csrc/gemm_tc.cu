@@ -52,30 +52,31 @@ namespace {
 // the last 64 it encoded (an encode costs about a microsecond of host time, a tenth of tiny's launch work in all).
 struct MapKey {
     const void* base;
-    uint64_t rows, cols;
-    uint32_t box_rows, box_cols, type;
-    bool operator==(const MapKey& o) const {
-        return base == o.base && rows == o.rows && cols == o.cols && box_rows == o.box_rows && box_cols == o.box_cols && type == o.type;
-    }
+    uint64_t dims[4], strides[3];  // innermost first; strides in bytes, of dimension 1 and up
+    uint32_t box[4], rank, type;   // type: 0 = fp16, 1 = bf16 (both 128-byte swizzle), 2 = bytes
+    bool operator==(const MapKey& o) const { return memcmp(this, &o, sizeof(MapKey)) == 0; }
 };
+static_assert(sizeof(MapKey) == 8 + 7 * 8 + 6 * 4, "compared as bytes: no padding");
 struct MapSlot {
     MapKey key;
     CUtensorMap map;
 };
 
-bool encode_cached(CUtensorMap* map, const MapKey& k, CUtensorMapDataType type, uint32_t elem, CUtensorMapSwizzle swizzle) {
+bool encode_cached(CUtensorMap* map, const MapKey& k) {
     constexpr int SLOTS = 64;
     static thread_local MapSlot slots[SLOTS] = {};
-    const uint64_t h = ((uint64_t)(uintptr_t)k.base * 0x9E3779B97F4A7C15ull) ^ (k.rows * 0xC2B2AE3D27D4EB4Full) ^ (k.cols << 7) ^ (k.box_rows << 3) ^ k.type;
+    const uint64_t h = ((uint64_t)(uintptr_t)k.base * 0x9E3779B97F4A7C15ull) ^ (k.dims[1] * 0xC2B2AE3D27D4EB4Full) ^ (k.dims[0] << 7) ^ (k.box[1] << 3) ^ k.type;
     MapSlot& s = slots[(h ^ (h >> 29)) >> 20 & (SLOTS - 1)];
     if (s.key == k) { *map = s.map; return true; }
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
-    cuuint64_t dims[2] = {k.cols, k.rows};
-    cuuint64_t strides[1] = {k.cols * elem};
-    cuuint32_t box[2] = {k.box_cols, k.box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    if (enc(&s.map, type, 2, const_cast<void*>(k.base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    cuuint64_t dims[4], strides[3];
+    for (int i = 0; i < 4; ++i) dims[i] = k.dims[i];
+    for (int i = 0; i < 3; ++i) strides[i] = k.strides[i];
+    const CUtensorMapDataType type = k.type == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : k.type == 1 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    if (enc(&s.map, type, k.rank, const_cast<void*>(k.base), dims, strides, k.box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            k.type == 2 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
         s.key = MapKey{};
         return false;
@@ -88,14 +89,18 @@ bool encode_cached(CUtensorMap* map, const MapKey& k, CUtensorMapDataType type, 
 }  // namespace
 
 bool make_tensor_map_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool bf16) {
-    return encode_cached(map, MapKey{base, rows, cols, box_rows, 64, bf16 ? 1u : 0u}, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
-                         CU_TENSOR_MAP_SWIZZLE_128B);
+    return encode_cached(map, MapKey{base, {cols, rows}, {cols * 2}, {64, box_rows}, 2, bf16 ? 1u : 0u});
+}
+
+bool make_tensor_map_4d(CUtensorMap* map, const void* base, uint64_t envs, uint64_t steps, uint64_t policies, uint64_t pol_stride, uint32_t box_envs,
+                        uint32_t box_steps, bool bf16) {
+    return encode_cached(map, MapKey{base, {64, envs, steps, policies}, {128, envs * 128, pol_stride}, {64, box_envs, box_steps, 1}, 4, bf16 ? 1u : 0u});
 }
 
 // The same over a row-major byte matrix [rows][cols] (cols a multiple of 16) with a box of box_cols x box_rows bytes, not swizzled.
 bool make_tensor_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_cols) {
     if (cols % 16 != 0 || box_cols % 16 != 0) return false;
-    return encode_cached(map, MapKey{base, rows, cols, box_rows, box_cols, 2u}, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, CU_TENSOR_MAP_SWIZZLE_NONE);
+    return encode_cached(map, MapKey{base, {cols, rows}, {cols}, {box_cols, box_rows}, 2, 2u});
 }
 
 // DEEP: as many stages as fit (plane operands, TMA-latency-bound); otherwise two, so that two CTAs share an SM (the

@@ -16,6 +16,8 @@
 //   k_reduce_adam2  fixed-order sum of every region's partials (= the batch-mean gradient, the single-device form of
 //                 the paper's cross-core average), Adam, loss statistics.
 // No floating-point atomics: every sum has a fixed order, so runs are bitwise reproducible.
+#include <algorithm>
+
 #include "tc_common.cuh"
 
 namespace anakin {
@@ -31,12 +33,15 @@ namespace anakin {
 // HS = width of the column slab one CTA covers (blockIdx.y picks the slab; HS = H for H <= 256); H2BF: h2 is stored as
 // bf16 (the wide bf16 path) instead of fp32.
 // FUSE (H = 256 only): the kernel also takes dW2 = h1^T dh2 for its rows on the tcgen05 pipe (see k_heads_bwd).
+__host__ __device__ constexpr int heads_per_sm(int H) { return H == 32 ? 8 : H == 64 ? 5 : H == 96 ? 4 : 2; }
 template <int H, int NW, int PREC, int HS = H, bool H2BF = false, bool FUSE = false>
 struct HeadsCfg {
     static constexpr int TR = 32;  // rows per tile
     static constexpr int ESZ = H2BF ? 2 : 4;
-    // the widest slab (32 KB tiles, 17 warps) runs one CTA per SM with a deep ring; the narrower ones two CTAs per SM
-    static constexpr int PER_SM = TR * HS * ESZ >= 32768 ? 1 : 2;
+    // the widest slab (32 KB tiles, 17 warps) runs one CTA per SM with a deep ring; the narrower ones two CTAs per SM, and below
+    // H = 128, where a tile is so little work that the one row warp of a CTA sets its pace (about a microsecond a tile), as
+    // many as shared memory holds: B200, H = 64, 2.0 M rows, two CTAs per SM 215 us
+    static constexpr int PER_SM = TR * HS * ESZ >= 32768 ? 1 : heads_per_sm(H);
     static constexpr int PL = PREC == 1 ? 1 : 2;
     static constexpr int BOX = TR * 128;                     // 32 rows x 64 16-bit elements, MN-major (4 KB)
     static constexpr int OP_TILE = PL * (H / 64) * BOX;      // one operand tile: [plane][64-column box]
@@ -102,7 +107,10 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
     if (FUSE) tc::tc_fence_before();
     __syncthreads();
     if (FUSE) tc::tc_fence_after();
-    PDL_START();  // (the set-up above runs under the predecessor's tail)
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
+    // The fused kernel takes its SMs whole.  The other one triggers after its tiles: with CTAs of the next kernel placed beside
+    // it from the start it ran a third slower (B200, H = 64, 2.0 M rows: 215 -> 283 us; H = 32: 54 -> 84 us).
+    if (FUSE) pdl_trigger();
     bool ok = true;
     const int my_its = (ntiles > (int)blockIdx.x) ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;  // tiles of this CTA
 
@@ -254,11 +262,8 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 if (rr == c) {
-                    if (c < 5) {
-                        for (int q = 0; q < 4; ++q) a.part_small[(size_t)(4 * blockIdx.x + q) * a.small_stride + (size_t)H * 6 + c] = q == 0 ? vals[c] : 0.f;
-                    } else {
-                        b.loss_part[(size_t)blockIdx.x * 4 + (c - 5)] = vals[c];
-                    }
+                    if (c < 5) a.part_small[(size_t)blockIdx.x * a.small_stride + (size_t)H * 6 + c] = vals[c];
+                    else b.loss_part[(size_t)blockIdx.x * 4 + (c - 5)] = vals[c];
                 }
             }
         }
@@ -436,14 +441,36 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
         if (FUSE && (it + 1) % Cfg::GROUP == 0 && it + 1 < my_its) ok = dw2_out(it) && ok;
     }
     cp_async_wait<0>();
-    // ---- per-CTA results: dWh, db2 partials (split index = 4*CTA + row group)
+    if (!FUSE) pdl_trigger();
+    // ---- this CTA's dWh and db2 partial: the row groups are added, in order, through the idle ring
     {
-        float* part = a.part_small + (size_t)(4 * blockIdx.x + rg) * a.small_stride;
+        float* red = reinterpret_cast<float*>(s_h2);  // [row group 1..3][12][HP2]
+        asm volatile("bar.sync 1, %0;" ::"n"(NTHREADS) : "memory");
+        if (rg > 0) {
 #pragma unroll
-        for (int cc = 0; cc < 2; ++cc) {
+            for (int cc = 0; cc < 2; ++cc) {
 #pragma unroll
-            for (int c = 0; c < 5; ++c) part[(size_t)(c_base + 2 * cp + cc) * 5 + c] = a_wh[cc][c];
-            part[(size_t)H * 5 + c_base + 2 * cp + cc] = a_b2[cc];
+                for (int c = 0; c < 5; ++c) red[((rg - 1) * 12 + 6 * cc + c) * HP2 + cp] = a_wh[cc][c];
+                red[((rg - 1) * 12 + 6 * cc + 5) * HP2 + cp] = a_b2[cc];
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(NTHREADS) : "memory");
+        if (rg == 0) {
+            float* part = a.part_small + (size_t)blockIdx.x * a.small_stride;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int cc = 0; cc < 2; ++cc) {
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) a_wh[cc][c] += red[(q * 12 + 6 * cc + c) * HP2 + cp];
+                    a_b2[cc] += red[(q * 12 + 6 * cc + 5) * HP2 + cp];
+                }
+#pragma unroll
+            for (int cc = 0; cc < 2; ++cc) {
+#pragma unroll
+                for (int c = 0; c < 5; ++c) part[(size_t)(c_base + 2 * cp + cc) * 5 + c] = a_wh[cc][c];
+                part[(size_t)H * 5 + c_base + 2 * cp + cc] = a_b2[cc];
+            }
         }
     }
     if (FUSE) {
@@ -637,7 +664,7 @@ __global__ void __launch_bounds__(512, 2) k_heads_bwd_tc(LearnArgs a) {
     __syncthreads();
     if (prev_tile >= 0) copy_out(prev_tile, (it - 1) & 1);
     // ---- per-CTA results (split index = CTA): dWh from the accumulator fragments, db2 folded over the 8 row lanes
-    float* part = a.part_small + (size_t)(4 * blockIdx.x) * a.small_stride;
+    float* part = a.part_small + (size_t)blockIdx.x * a.small_stride;
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
         const int col = c_base + col0 + g + 8 * hh;
@@ -879,7 +906,7 @@ struct GemmTnCfg {
 
 template <int BM, int BN, int AMODE, int APL, int BPL, int PREC, bool GROUPED = false>
 __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
-    PDL_START();
+    pdl_wait();  // (the trigger comes after the products: CTAs of the next kernel beside these from the start cost more than the gap)
     // many policies: grid.z = policy * nsplit + split
     const PolicyArgs<GROUPED, GemmTnArgs> pa(g_in, GROUPED ? (int)blockIdx.z / g_in.nsplit : 0);
     const GemmTnArgs& g = pa.a;
@@ -1002,6 +1029,7 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
         }
     }
     cp_async_wait<0>();
+    pdl_trigger();
     // ---- split-K partial out
     const int gq = lane >> 2, t4 = lane & 3;
     float* part = g.part + (size_t)split * g.stride;
@@ -1295,7 +1323,8 @@ __global__ void __launch_bounds__(256) k_pack_gates2(DimsBuffers in, size_t R_in
 // ----------------------------------------------------------------------------------------------------
 // host side
 // ----------------------------------------------------------------------------------------------------
-constexpr int HEADS_GRID = 2 * 148;  // persistent CTAs of k_heads_bwd (two per SM)
+// Persistent CTAs of k_heads_bwd.  (The kernels for H >= 256 take a whole SM, or walk several column slabs.)
+static int heads_grid_max(int H) { return H >= 256 ? 148 : heads_per_sm(H) * 148; }
 
 static int splits_for(int K, int tiles, int min_k) {
     int ns = (2 * 148 + tiles - 1) / tiles;
@@ -1361,14 +1390,18 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         if (gx * ts > p->ns_agent) p->ns_agent = gx * ts;
     }
     p->ns_env = splits_for(d.B, tiles_ch, 128);
+    if (H == 64) {  // (one partial per CTA of the fused kernel; its slices of the steps are rows of S)
+        p->ns_w2 = p->ns_agent = 148 / d.npol > 0 ? 148 / d.npol : 1;
+        p->ns_env = splits_for(std::max(4 * d.B, std::min(BACK64_SLICES * d.B, 148 * 128)), tiles_ch, 256);
+    }
     const size_t tiles32 = (R + 31) / 32;
-    size_t hg = H >= 256 ? HEADS_GRID / 2 : HEADS_GRID;  // (the kernels for H >= 256 take a whole SM, or walk several column slabs)
-    if (d.npol > 1) hg = (size_t)(2 * HEADS_GRID / d.npol > 0 ? 2 * HEADS_GRID / d.npol : 1);  // many policies: the CTAs of all policies fill the GPU together
+    size_t hg = (size_t)heads_grid_max(H);
+    if (d.npol > 1) hg = (size_t)std::max(std::max(heads_grid_max(H), 4 * 148) / d.npol, 1);  // many policies: the CTAs of all policies fill the GPU together
     p->heads_grid = (int)(tiles32 < hg ? tiles32 : hg);
     // (the fused heads + dW2 kernel writes one dW2 partial per CTA: room for the larger of the two partial counts)
     int w2_slots = heads_fuse_dw2(d, R, p->heads_grid, 1) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;
     if (three_terms(H, 0) && x3_w2_splits(H, R) > w2_slots) w2_slots = x3_w2_splits(H, R);
-    p->ns_small = 4 * p->heads_grid;
+    p->ns_small = p->heads_grid;
     p->small_stride = (size_t)6 * H + 8;
     size_t off = 0;
     p->off_w2 = off; off += (size_t)w2_slots * H * H;
@@ -1478,8 +1511,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
                 }
                 if constexpr (PREC == 1) {
                     if (H == 384) { CK((launch_heads_t<384, 8, 1, 128, true>(a, pl.heads_grid, s))); break; }  // (no whole 256-column slabs)
-                    if (wide) {  // tensor-pipe version: one partial slot per CTA (slot 4 * CTA of the small region)
-                        for (int q = 5; q <= 7; ++q) { a.reg[q].ns = pl.heads_grid; a.reg[q].stride = 4 * pl.small_stride; }
+                    if (wide) {  // tensor-pipe version
                         if (H == 512) { CK((launch_heads_tc_t<512>(a, pl.heads_grid, s))); break; }
                         if (H == 1024) { CK((launch_heads_tc_t<1024>(a, pl.heads_grid, s))); break; }
                         if (H == 768) { CK((launch_heads_tc_t<768>(a, pl.heads_grid, s))); break; }
@@ -1492,7 +1524,17 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     // CTAs covers the SMs.  The mma.sync fall-back keeps one slice.
     a.ts = 1;
     bool fused_agent = false;  // dh1, S and the agent plane of dW1 in one kernel (dh1 stays on chip)
-    if (!wide && !grouped && dh1_agent_tc_supported(d)) {
+    const bool back64 = H == 64;  // ... and dW2 too
+    if (back64) {
+        int nx;
+        back64_shape(d, T, &nx, &a.ts);
+        a.reg[1].ns = a.reg[4].ns = nx;
+        const int tiles = (C + 1 + 63) / 64;
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = splits_for(a.ts * B, tiles, 256);
+        Scope sc(c, K_DH1);
+        CK(launch_back64(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
+        fused_agent = true;
+    } else if (!wide && !grouped && dh1_agent_tc_supported(d)) {
         int gx, ts;
         dh1a_shape(d, T, &gx, &ts);
         a.ts = ts;
@@ -1536,8 +1578,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
             if (a.ts > T / 2) a.ts = T / 2;
             if (a.ts < 1) a.ts = 1;
             switch (H) {
-                case 64: CK((launch_dh1_t<64, 64, PREC>(a, s))); break;
-                case 128: CK((launch_dh1_t<128, 128, PREC>(a, s))); break;
+                    case 128: CK((launch_dh1_t<128, 128, PREC>(a, s))); break;
                 case 256: CK((launch_dh1_t<256, 128, PREC>(a, s))); break;
                 default:
                     if constexpr (PREC == 1) {
@@ -1580,7 +1621,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     g.part = b.part + pl.off_w2; g.stride = (size_t)H * H; g.off = 0; g.ldc = H; g.ones_row = -1;
     g.K_last = d.B_last * T; g.kmod_last = 0; g.alo_off_last = g.blo_off_last = RH_last;
     if (wide && PREC == 2) g.Alo = h1hi + wide_h1_rows(d) * H;
-    if (!fuse_dw2) {
+    if (!fuse_dw2 && !back64) {
         Scope sc(c, K_DW2);
         CK(tn_gemm(ic<A_PLANES>{}, ic<PL>{}, ic<PL>{}, H, pl.ns_w2));
     }

@@ -50,6 +50,16 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
+// The same over a 4-D map (x = innermost).
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w)
+                 : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* map, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(map), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
 // Makes generic-proxy writes to shared memory (ordinary stores) visible to the async proxy (TMA, tcgen05.mma).
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -251,6 +261,9 @@ __host__ __device__ constexpr int x3_b(int i) { return i == 1 ? 2 : i == 2 ? 1 :
 // Host: encodes a 2-D tensor map over a row-major 16-bit matrix [rows][cols] with a box of 64 columns x box_rows rows
 // and the 128-byte swizzle.  Returns false if the driver entry point is missing or the encode fails.
 bool make_tensor_map_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, bool bf16);
+// Host: the same over [policy][step][env][64] (policies pol_stride bytes apart) with a box of box_envs x box_steps rows.
+bool make_tensor_map_4d(CUtensorMap* map, const void* base, uint64_t envs, uint64_t steps, uint64_t policies, uint64_t pol_stride, uint32_t box_envs,
+                        uint32_t box_steps, bool bf16);
 // Host: the same over a row-major byte matrix [rows][cols] (cols a multiple of 16), box of box_cols x box_rows bytes, no swizzle.
 bool make_tensor_map_u8(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_cols);
 
