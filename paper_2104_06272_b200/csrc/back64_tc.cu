@@ -15,7 +15,7 @@
 //               (A = one-hot cells, 128 or 256 of them; B = dh1)
 //   warps 2-9   thread = (row, half of the units): tcgen05.ld, gate, S +=, 16-bit split; the dh1 planes go over the dh2 planes
 //               of the same stage once dW2 has read them
-// dW2 changes accumulator every FLUSH tiles (4096 rows, as in the plain GEMM) and the groups are added in registers.
+// dW2 restarts its accumulator every FLUSH tiles (4096 rows, as in the plain GEMM); the groups are added in registers.
 #include <cstring>
 
 #include "tc_common.cuh"
@@ -30,13 +30,18 @@ struct Back64Cfg {
     static constexpr int PL = PREC == 1 ? 1 : 2;
     static constexpr int EPI_WARPS = 8, FIRST_EPI = 2, THREADS = 32 * (FIRST_EPI + EPI_WARPS);
     static constexpr int BOX = BM * 128;             // 128 rows x 64 16-bit elements
-    static constexpr int STAGE = 2 * PL * BOX;       // [h1 planes][dh2 planes]
-    static constexpr int STAGES = PREC == 1 ? 4 : 2;
+    static constexpr int STAGE = PL * BOX;           // the planes of one operand
+    static constexpr int HST = PREC == 1 ? 3 : 2;    // h1 ring
+    static constexpr int DST = PREC == 1 ? 4 : NC == 1 ? 3 : 2;  // dh2 ring (a stage then holds the dh1 planes: it is busy longer)
     static constexpr int W_BOX = H * 128, W_BYTES = PL * W_BOX;
     static constexpr int O_TILE = 2 * NC * BOX;      // one-hot: 128 rows x NC * 128 cells in 64-wide boxes
     static constexpr int FLUSH = 32;                 // tiles per dW2 accumulator
-    static constexpr int ACC_COL = 0, W2_COL = 128, AGENT_COL = 256, TMEM_COLS = 512;
-    static constexpr size_t smem_bytes = (size_t)STAGES * STAGE + W_BYTES + O_TILE + 256 + 1024;
+    // Two planes of the N operand are one MMA of 128 columns (half of them the lo plane's): the M operand is then read from shared
+    // memory once, and shared memory is what bounds these products.  (At NC = 2 tensor memory has no room for it in dh1.)
+    static constexpr int W2_N = PL * H, AGENT_N = PL * H, ACC_N = PL == 2 && NC == 1 ? 2 * H : H;
+    static constexpr int ACC_COL = 0, W2_COL = 2 * ACC_N, AGENT_COL = W2_COL + W2_N, TMEM_COLS = 512;
+    static_assert(AGENT_COL + NC * AGENT_N <= TMEM_COLS, "tensor memory");
+    static constexpr size_t smem_bytes = (size_t)(HST + DST) * STAGE + W_BYTES + O_TILE + 256 + 1024;
     static_assert(smem_bytes <= 232448, "227 KB per CTA");
 };
 
@@ -54,17 +59,20 @@ struct Back64Args {
 template <int PREC, int NC, bool GROUPED>
 __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(const __grid_constant__ Back64Maps maps, const __grid_constant__ Back64Args in) {
     using Cfg = Back64Cfg<PREC, NC>;
-    constexpr int H = Cfg::H, BM = Cfg::BM, PL = Cfg::PL, STAGES = Cfg::STAGES, BOX = Cfg::BOX;
+    constexpr int H = Cfg::H, BM = Cfg::BM, PL = Cfg::PL, HST = Cfg::HST, DST = Cfg::DST, BOX = Cfg::BOX;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* sT = base;                              // [STAGES] of [h1 planes][dh2 planes]
-    unsigned char* sW = sT + STAGES * Cfg::STAGE;          // W2 planes, 64 rows x 64 k each
+    unsigned char* sH = base;                              // [HST] h1 planes
+    unsigned char* sD = sH + HST * Cfg::STAGE;             // [DST] dh2 planes, then dh1 planes
+    unsigned char* sW = sD + DST * Cfg::STAGE;             // W2 planes, 64 rows x 64 k each
     unsigned char* sO = sW + Cfg::W_BYTES;                 // one-hot tile
     uint64_t* bars = (uint64_t*)(sO + Cfg::O_TILE);
-    uint64_t* full = bars;                 // [STAGES] planes landed
-    uint64_t* empty = full + STAGES;       // [STAGES] the agent MMAs of the tile have finished (the last readers of the stage)
-    uint64_t* w2done = empty + STAGES;     // [STAGES] dW2 (and dh1) of the tile have finished: the dh2 planes may be overwritten
-    uint64_t* tfull = w2done + STAGES;     // [2] dh1 accumulator written
+    uint64_t* hfull = bars;                // [HST] h1 planes landed
+    uint64_t* hempty = hfull + HST;        // [HST] dW2 has read them (commit) and the gates have been taken (the epilogue warps arrive)
+    uint64_t* full = hempty + HST;         // [DST] dh2 planes landed
+    uint64_t* empty = full + DST;          // [DST] the agent MMAs of the tile have finished
+    uint64_t* w2done = empty + DST;        // [DST] dW2 (and dh1) of the tile have finished: the dh2 planes may be overwritten
+    uint64_t* tfull = w2done + DST;        // [2] dh1 accumulator written
     uint64_t* tempty = tfull + 2;          // [2] dh1 accumulator drained (the epilogue warps arrive)
     uint64_t* wfull = tempty + 2;          // W2 planes in shared memory (the epilogue warps arrive)
     uint64_t* tiles_full = wfull + 1;      // dh1 planes and one-hot of a tile written (the epilogue warps arrive)
@@ -87,7 +95,8 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
     auto t_end = [&](int u) { return min((u / m_tiles) * tl + tl, T); };
 
     if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); tc::mbar_init(&w2done[s], 1); }
+        for (int s = 0; s < HST; ++s) { tc::mbar_init(&hfull[s], 1); tc::mbar_init(&hempty[s], 1 + Cfg::EPI_WARPS); }
+        for (int s = 0; s < DST; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); tc::mbar_init(&w2done[s], 1); }
         for (int i = 0; i < 2; ++i) { tc::mbar_init(&tfull[i], 1); tc::mbar_init(&tempty[i], Cfg::EPI_WARPS); }
         tc::mbar_init(wfull, Cfg::EPI_WARPS);
         tc::mbar_init(tiles_full, Cfg::EPI_WARPS);
@@ -96,8 +105,8 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
     if (wid == 1) tc::tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
     // the one-hot tile starts all zero (every tile clears the elements of the one before); so do the rows that no box fills
     for (int i = tid; i < Cfg::O_TILE / 16; i += Cfg::THREADS) reinterpret_cast<uint4*>(sO)[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (SP > 1)
-        for (int i = tid; i < STAGES * Cfg::STAGE / 16; i += Cfg::THREADS) reinterpret_cast<uint4*>(sT)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (SP * TE < BM)
+        for (int i = tid; i < (HST + DST) * Cfg::STAGE / 16; i += Cfg::THREADS) reinterpret_cast<uint4*>(sH)[i] = make_uint4(0u, 0u, 0u, 0u);
     tc::fence_proxy_async();
     tc::tc_fence_before();
     __syncthreads();
@@ -115,85 +124,99 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
             const CUtensorMap* dh = last ? &maps.ld_hi : &maps.d_hi;
             const CUtensorMap* dl = last ? &maps.ld_lo : &maps.d_lo;
             const int w = last ? 0 : pol;
-            const uint32_t bytes = 2 * PL * (uint32_t)(SP * TE) * 128u;
+            const uint32_t bytes = PL * (uint32_t)(SP * TE) * 128u;
             int g = 0;
             for (int u = xi; u < units && ok; u += nx) {
                 const int env0 = (u % m_tiles) * BM, t1 = t_end(u);
                 for (int t = t_begin(u); t < t1; t += SP, ++g) {
-                    const int s = g % STAGES;
-                    if (t + STAGES * SP < t1) {  // pull a later tile of this unit towards L2
-                        const int tp = t + STAGES * SP;
+                    const int hs = g % HST, ds = g % DST, tp = t + DST * SP;
+                    if (tp < t1) {  // pull a later tile of this unit towards L2
                         tc::tma_prefetch_4d(dh, 0, env0, tp, w);
                         tc::tma_prefetch_4d(mh, 0, env0, tp, w);
                         if (PL == 2) { tc::tma_prefetch_4d(dl, 0, env0, tp, w); tc::tma_prefetch_4d(ml, 0, env0, tp, w); }
                     }
-                    if (g >= STAGES) ok = tc::mbar_wait(&empty[s], (uint32_t)(g / STAGES - 1) & 1u);
+                    if (g >= DST) ok = tc::mbar_wait(&empty[ds], (uint32_t)(g / DST - 1) & 1u);
                     if (!ok) break;
-                    unsigned char* st = sT + s * Cfg::STAGE;
-                    tc::mbar_expect_tx(&full[s], bytes);
-                    tc::tma_load_4d(st + PL * BOX, dh, &full[s], 0, env0, t, w);
-                    if (PL == 2) tc::tma_load_4d(st + 3 * BOX, dl, &full[s], 0, env0, t, w);
-                    tc::tma_load_4d(st, mh, &full[s], 0, env0, t, w);
-                    if (PL == 2) tc::tma_load_4d(st + BOX, ml, &full[s], 0, env0, t, w);
+                    tc::mbar_expect_tx(&full[ds], bytes);
+                    tc::tma_load_4d(sD + ds * Cfg::STAGE, dh, &full[ds], 0, env0, t, w);
+                    if (PL == 2) tc::tma_load_4d(sD + ds * Cfg::STAGE + BOX, dl, &full[ds], 0, env0, t, w);
+                    if (g >= HST) ok = tc::mbar_wait(&hempty[hs], (uint32_t)(g / HST - 1) & 1u);
+                    if (!ok) break;
+                    tc::mbar_expect_tx(&hfull[hs], bytes);
+                    tc::tma_load_4d(sH + hs * Cfg::STAGE, mh, &hfull[hs], 0, env0, t, w);
+                    if (PL == 2) tc::tma_load_4d(sH + hs * Cfg::STAGE + BOX, ml, &hfull[hs], 0, env0, t, w);
                 }
             }
             if (!ok) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {  // ---- MMA issuer: the whole warp walks the loop, one elected lane issues
-        const uint32_t id_dh1 = tc::umma_idesc<PREC>(BM, H, false, false), id_mn = tc::umma_idesc<PREC>(128, H, true, true);
-        auto agent_mma = [&](int v) {
-            const int s = v % STAGES;
+        const uint32_t id_dh1 = tc::umma_idesc<PREC>(BM, H, false, false), id_dh1_2 = tc::umma_idesc<PREC>(BM, 2 * H, false, false);
+        const uint32_t id_w2 = tc::umma_idesc<PREC>(128, Cfg::W2_N, true, true), id_agent = tc::umma_idesc<PREC>(128, Cfg::AGENT_N, true, true);
+        auto agent_mma = [&](int v) {  // 16 rows = 2048 bytes further in the MN-major boxes; the lo plane of dh1 one box on
+            const int s = v % DST;
             ok = tc::warp_all(tc::mbar_wait(tiles_full, (uint32_t)v & 1u));
             if (!ok) return;
             tc::tc_fence_after();
             if (tc::elect_one()) {
-                const unsigned char* sd = sT + s * Cfg::STAGE + PL * BOX;
 #pragma unroll
-                for (int pl = PL - 1; pl >= 0; --pl)
+                for (int k16 = 0; k16 < BM / 16; ++k16) {
+                    const uint64_t dd = tc::umma_desc(sD + s * Cfg::STAGE + k16 * 2048, BOX, 1024);
 #pragma unroll
-                    for (int k16 = 0; k16 < BM / 16; ++k16) {
-                        const uint64_t dd = tc::umma_desc(sd + pl * BOX + k16 * 2048, BOX, 1024);
-#pragma unroll
-                        for (int c = 0; c < NC; ++c)
-                            tc::umma(tmem + (uint32_t)(Cfg::AGENT_COL + 64 * c), tc::umma_desc(sO + 2 * c * BOX + k16 * 2048, BOX, 1024), dd, id_mn,
-                                     v > 0 || pl < PL - 1 || k16 > 0);
-                    }
+                    for (int c = 0; c < NC; ++c)
+                        tc::umma(tmem + (uint32_t)(Cfg::AGENT_COL + Cfg::AGENT_N * c), tc::umma_desc(sO + 2 * c * BOX + k16 * 2048, BOX, 1024), dd, id_agent,
+                                 v > 0 || k16 > 0);
+                }
                 tc::umma_commit(&empty[s]);
             }
             __syncwarp();
         };
         ok = tc::warp_all(tc::mbar_wait(wfull, 0));
         for (int g = 0; g < G && ok; ++g) {
-            const int s = g % STAGES, buf = g & 1;
+            const int hs = g % HST, ds = g % DST, buf = g & 1;
             if (g >= 2) ok = tc::warp_all(tc::mbar_wait(&tempty[buf], (uint32_t)((g >> 1) - 1) & 1u));
-            if (ok) ok = tc::warp_all(tc::mbar_wait(&full[s], (uint32_t)(g / STAGES) & 1u));
+            if (ok) ok = tc::warp_all(tc::mbar_wait(&full[ds], (uint32_t)(g / DST) & 1u));
             if (!ok) break;
             tc::tc_fence_after();
+            const unsigned char* sh = sH + hs * Cfg::STAGE;
+            const unsigned char* sd = sD + ds * Cfg::STAGE;
             if (tc::elect_one()) {
-                const unsigned char* sh = sT + s * Cfg::STAGE;
-                const unsigned char* sd = sh + PL * BOX;
-                const uint32_t acc = tmem + (uint32_t)(Cfg::ACC_COL + 64 * buf);
-                // dh1: W lo x dh2 hi, W hi x dh2 lo, W hi x dh2 hi per k16 (32 bytes along the swizzled rows)
+                const uint32_t acc = tmem + (uint32_t)(Cfg::ACC_COL + Cfg::ACC_N * buf);
+                // dh1 per k16 (32 bytes along the swizzled rows): dh2 hi x [W hi | W lo] where there is room for both halves (they
+                // are added in the epilogue), dh2 lo x W hi
 #pragma unroll
                 for (int k16 = 0; k16 < H / 16; ++k16) {
                     const uint64_t d_hi = tc::umma_desc(sd + k16 * 32, 16, 1024), w_hi = tc::umma_desc(sW + k16 * 32, 16, 1024);
-                    if (PL == 2) {
-                        tc::umma(acc, d_hi, tc::umma_desc(sW + Cfg::W_BOX + k16 * 32, 16, 1024), id_dh1, k16 > 0);
-                        tc::umma(acc, tc::umma_desc(sd + BOX + k16 * 32, 16, 1024), w_hi, id_dh1, 1u);
+                    if (PL == 1) {
+                        tc::umma(acc, d_hi, w_hi, id_dh1, k16 > 0);
+                    } else {
+                        const uint64_t d_lo = tc::umma_desc(sd + BOX + k16 * 32, 16, 1024);
+                        if (NC == 1) {
+                            tc::umma(acc, d_hi, w_hi, id_dh1_2, k16 > 0);
+                            tc::umma(acc, d_lo, w_hi, id_dh1, 1u);
+                        } else {
+                            tc::umma(acc, d_hi, tc::umma_desc(sW + Cfg::W_BOX + k16 * 32, 16, 1024), id_dh1, k16 > 0);
+                            tc::umma(acc, d_lo, w_hi, id_dh1, 1u);
+                            tc::umma(acc, d_hi, w_hi, id_dh1, 1u);
+                        }
                     }
-                    tc::umma(acc, d_hi, w_hi, id_dh1, PL == 2 || k16 > 0);
                 }
                 tc::umma_commit(&tfull[buf]);
-                // dW2: 16 rows = 2048 bytes further; M = units of the hi plane, then of the lo plane one box on (bf16: the box
-                // behind h1 is dh2, its 64 lanes are not read)
-                const uint32_t acc2 = tmem + (uint32_t)(Cfg::W2_COL + 64 * ((g / Cfg::FLUSH) & 1));
+            }
+            __syncwarp();
+            ok = tc::warp_all(tc::mbar_wait(&hfull[hs], (uint32_t)(g / HST) & 1u));
+            // a new group of dW2: the accumulator of the one before has been read (the epilogue does so ahead of its own dh1)
+            if (ok && g > 0 && g % Cfg::FLUSH == 0) ok = tc::warp_all(tc::mbar_wait(&tempty[buf], (uint32_t)(g >> 1) & 1u));
+            if (!ok) break;
+            tc::tc_fence_after();
+            if (tc::elect_one()) {
+                // dW2: M = units of the hi plane of h1, then of the lo plane one box on (bf16: whatever follows, 64 lanes that are not
+                // read); N = units of dh2, the lo plane's behind the hi plane's
+                const uint32_t acc2 = tmem + (uint32_t)Cfg::W2_COL;
 #pragma unroll
-                for (int pl = PL - 1; pl >= 0; --pl)
-#pragma unroll
-                    for (int k16 = 0; k16 < BM / 16; ++k16)
-                        tc::umma(acc2, tc::umma_desc(sh + k16 * 2048, BOX, 1024), tc::umma_desc(sd + pl * BOX + k16 * 2048, BOX, 1024), id_mn,
-                                 g % Cfg::FLUSH != 0 || pl < PL - 1 || k16 > 0);
-                tc::umma_commit(&w2done[s]);
+                for (int k16 = 0; k16 < BM / 16; ++k16)
+                    tc::umma(acc2, tc::umma_desc(sh + k16 * 2048, BOX, 1024), tc::umma_desc(sd + k16 * 2048, BOX, 1024), id_w2, g % Cfg::FLUSH != 0 || k16 > 0);
+                tc::umma_commit(&w2done[ds]);
+                tc::umma_commit(&hempty[hs]);
             }
             __syncwarp();
             if (g >= 1) agent_mma(g - 1);
@@ -220,11 +243,20 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
         for (int i = 0; i < 32; ++i) w_acc[i] = 0.f;
         uint16_t* const S_hi = reinterpret_cast<uint16_t*>(b.S);
         uint16_t* const S_lo = S_hi + (size_t)a.ts * B * H;
-        auto add_w2 = [&](int group) {  // += this thread's 32 columns of a finished dW2 accumulator
-            uint32_t v[32];
-            tc::tmem_ld32(tmem + lane_base + (uint32_t)(Cfg::W2_COL + 64 * (group & 1) + 32 * half), v);
+        // 32 columns of this thread's lane: those of the hi half of the accumulator and, behind them, of the lo half, added
+        auto read_pair = [&](uint32_t col, bool two, float (&v)[32]) {
+            uint32_t x0[32], x1[32];
+            tc::tmem_ld32_nowait(tmem + lane_base + col + 32 * half, x0);
+            if (two) tc::tmem_ld32_nowait(tmem + lane_base + col + 64 + 32 * half, x1);
+            tc::tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 32; ++i) w_acc[i] += __uint_as_float(v[i]);
+            for (int i = 0; i < 32; ++i) v[i] = two ? __uint_as_float(x0[i]) + __uint_as_float(x1[i]) : __uint_as_float(x0[i]);
+        };
+        auto add_w2 = [&]() {  // += this thread's 32 columns of the finished dW2 accumulator
+            float v[32];
+            read_pair(Cfg::W2_COL, PL == 2, v);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) w_acc[i] += v[i];
         };
         auto store_S = [&](size_t row, const float (&v)[32]) {  // 32 units of one row, two 16-bit planes
             uint32_t hi[16], lo[16];
@@ -254,43 +286,45 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
 #pragma unroll
             for (int i = 0; i < 32; ++i) s_acc[i] = 0.f;
             for (int t = t_begin(u); t < t1; t += SP, ++g) {
-                const int buf = g & 1, s = g % STAGES;
+                const int buf = g & 1, s = g % DST, hs = g % HST;
                 const int cell = half == 0 && have && t + row_dt < t1 ? (int)b.tpos[(size_t)(t + row_dt) * B + env] : -1;
                 ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g >> 1) & 1u);
                 if (!ok) break;
                 tc::tc_fence_after();
-                if (g > 0 && g % Cfg::FLUSH == 0) add_w2(g / Cfg::FLUSH - 1);  // (finished: w2done of the tile before was waited for)
-                uint32_t x[32];
-                tc::tmem_ld32(tmem + lane_base + (uint32_t)(Cfg::ACC_COL + 64 * buf + 32 * half), x);
+                if (g > 0 && g % Cfg::FLUSH == 0) add_w2();  // (finished: w2done of the tile before was waited for)
+                float x[32];
+                read_pair((uint32_t)(Cfg::ACC_COL + Cfg::ACC_N * buf), Cfg::ACC_N > H, x);
                 tc::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&tempty[buf]);
-                ok = tc::mbar_wait(&full[s], (uint32_t)(g / STAGES) & 1u);  // (the loads themselves, for this thread's own reads)
+                ok = tc::mbar_wait(&hfull[hs], (uint32_t)(g / HST) & 1u);  // (the loads themselves, for this thread's own reads)
                 if (!ok) break;
-                unsigned char* st = sT + s * Cfg::STAGE;
+                uint32_t hi[16];
                 uint32_t lo[16];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {  // 16-byte chunks of 8 units: gate, S, split; the hi words replace the products
-                    const uint4 gt = *reinterpret_cast<const uint4*>(st + r * 128 + (((4 * half + c) ^ (r & 7)) << 4));
+                for (int c = 0; c < 4; ++c) {  // 16-byte chunks of 8 units: gate, S, split
+                    const uint4 gt = *reinterpret_cast<const uint4*>(sH + hs * Cfg::STAGE + r * 128 + (((4 * half + c) ^ (r & 7)) << 4));
                     const uint32_t gw[4] = {gt.x, gt.y, gt.z, gt.w};
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
                         const int i = 8 * c + 2 * p;
-                        const float v0 = rnd<PREC>((gw[p] & 0x00007FFFu) ? __uint_as_float(x[i]) : 0.f);
-                        const float v1 = rnd<PREC>((gw[p] & 0x7FFF0000u) ? __uint_as_float(x[i + 1]) : 0.f);
+                        const float v0 = rnd<PREC>((gw[p] & 0x00007FFFu) ? x[i] : 0.f);
+                        const float v1 = rnd<PREC>((gw[p] & 0x7FFF0000u) ? x[i + 1] : 0.f);
                         s_acc[i] += v0;
                         s_acc[i + 1] += v1;
-                        split2<PREC>(v0, v1, x[i / 2], lo[i / 2]);
+                        split2<PREC>(v0, v1, hi[i / 2], lo[i / 2]);
                     }
                 }
-                ok = tc::mbar_wait(&w2done[s], (uint32_t)(g / STAGES) & 1u);
-                if (ok && g >= 1) ok = tc::mbar_wait(&empty[(g - 1) % STAGES], (uint32_t)((g - 1) / STAGES) & 1u);  // the one-hot tile is free
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&hempty[hs]);
+                ok = tc::mbar_wait(&w2done[s], (uint32_t)(g / DST) & 1u);
+                if (ok && g >= 1) ok = tc::mbar_wait(&empty[(g - 1) % DST], (uint32_t)((g - 1) / DST) & 1u);  // the one-hot tile is free
                 if (!ok) break;
-                unsigned char* drow = st + PL * BOX + r * 128;
+                unsigned char* drow = sD + s * Cfg::STAGE + r * 128;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int off = ((4 * half + c) ^ (r & 7)) << 4;
-                    *reinterpret_cast<uint4*>(drow + off) = make_uint4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+                    *reinterpret_cast<uint4*>(drow + off) = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
                     if (PL == 2) *reinterpret_cast<uint4*>(drow + BOX + off) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
                 }
                 if (prev_off >= 0) *reinterpret_cast<uint16_t*>(sO + prev_off) = 0;
@@ -308,14 +342,14 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
         }
         if (!ok && lane == 0) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
         bool got = ok && G > 0;
-        if (got) got = tc::mbar_wait(&empty[(G - 1) % STAGES], (uint32_t)((G - 1) / STAGES) & 1u);  // the last MMAs; the stages are idle now
+        if (got) got = tc::mbar_wait(&empty[(G - 1) % DST], (uint32_t)((G - 1) / DST) & 1u);  // the last MMAs; the stages are idle now
         if (!got && ok && G > 0 && lane == 0) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
         tc::tc_fence_after();
         __syncwarp();
-        if (got) add_w2((G - 1) / Cfg::FLUSH);
+        if (got) add_w2();
         // the lo half of dW2 (lanes 64..) and, where a tile holds several steps, S go through the idle stages
-        float* const x_w2 = reinterpret_cast<float*>(sT);             // [64][64 + 4]
-        float* const x_s = reinterpret_cast<float*>(sT + 2 * BOX);    // [128][64]
+        float* const x_w2 = reinterpret_cast<float*>(sH);             // [64][64 + 4]
+        float* const x_s = reinterpret_cast<float*>(sH + 2 * BOX);    // [128][64]
         if (PL == 2 && q >= 2) {
 #pragma unroll
             for (int i = 0; i < 32; i += 4)
@@ -354,18 +388,18 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
         if (GROUPED) pagent = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(pagent) + (size_t)pol * in.a.d.pstride);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {  // accumulator lane = cell, column = unit
-            uint32_t v[32];
+            float v[32];
             if (got) {
-                tc::tmem_ld32(tmem + lane_base + (uint32_t)(Cfg::AGENT_COL + 64 * c + 32 * half), v);
+                read_pair((uint32_t)(Cfg::AGENT_COL + Cfg::AGENT_N * c), PL == 2, v);
             } else {
 #pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = 0u;
+                for (int i = 0; i < 32; ++i) v[i] = 0.f;
             }
             const int cell = 128 * c + r;
             if (cell < C) {
 #pragma unroll
                 for (int i = 0; i < 32; i += 4)
-                    *reinterpret_cast<uint4*>(pagent + (size_t)cell * H + 32 * half + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                    *reinterpret_cast<float4*>(pagent + (size_t)cell * H + 32 * half + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
             }
         }
     }

@@ -725,7 +725,7 @@ struct Dh1Cfg {
 
 template <int H, int BN, int PREC, bool GROUPED = false>
 __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnArgs a_in) {
-    PDL_START();
+    pdl_wait();
     const PolicyArgs<GROUPED, LearnArgs> pa(a_in, blockIdx.z);  // many policies: grid.z = policy
     const LearnArgs& a = pa.a;
     using Cfg = Dh1Cfg<H, BN, PREC>;
@@ -862,6 +862,7 @@ __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnAr
         }
     }
     cp_async_wait<0>();
+    pdl_trigger();
     // S (sum over t of dh1) as two 16-bit planes [B][H]: S is an fp32 sum, so it keeps two terms in either workload
     // (row slice * B + env of each plane)
     uint16_t* S_hi = reinterpret_cast<uint16_t*>(b.S) + (size_t)slice * B * H;
@@ -1396,7 +1397,7 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     }
     const size_t tiles32 = (R + 31) / 32;
     size_t hg = (size_t)heads_grid_max(H);
-    if (d.npol > 1) hg = (size_t)std::max(std::max(heads_grid_max(H), 4 * 148) / d.npol, 1);  // many policies: the CTAs of all policies fill the GPU together
+    if (d.npol > 1) hg = (size_t)std::max(4 * heads_grid_max(H) / d.npol, 1);  // many policies: the CTAs of all policies fill the GPU together
     p->heads_grid = (int)(tiles32 < hg ? tiles32 : hg);
     // (the fused heads + dW2 kernel writes one dW2 partial per CTA: room for the larger of the two partial counts)
     int w2_slots = heads_fuse_dw2(d, R, p->heads_grid, 1) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;

@@ -12,7 +12,7 @@ namespace anakin {
 // ascending cell order, the goal row last.
 template <bool GROUPED>
 __global__ void __launch_bounds__(256) k_env_base(DimsBuffers in) {
-    PDL_START();
+    pdl_wait();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);  // many policies: grid.y = policy
     const Dims& d = pa.a.d;
     const Buffers& b = pa.a.b;
@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(256) k_env_base(DimsBuffers in) {
         }
         if (rows[7] < 0) break;
     }
+    pdl_trigger();
     reinterpret_cast<float4*>(b.base)[idx] = acc;
 }
 
@@ -252,7 +253,7 @@ cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
 // ----------------------------------------------------------------------------------------------------
 template <bool GROUPED>
 __global__ void __launch_bounds__(128) k_gae(DimsBuffers in, int T, float gamma, float lambda) {
-    PDL_START();
+    pdl_wait();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);
     const Dims& d = pa.a.d;
     const int e = blockIdx.x * blockDim.x + threadIdx.x;

@@ -105,7 +105,7 @@ struct RolloutMmaCfg {
 // have been given the new positions.  Otherwise warp 0 does both (the wide kernels' registers leave no room for another warp).
 template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN, bool REPLAY>
 __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(RolloutArgs a_in) {
-    PDL_START();
+    pdl_wait();
     const PolicyArgs<GROUPED, RolloutArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
     const RolloutArgs& a = pa.a;
     using Cfg = RolloutMmaCfg<H, NW, PREC>;
@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             __syncthreads();
         }
     }
+    pdl_trigger();
     if (REPLAY) return;
     if (owner) {
         b.pos[e0 + ow] = (uint8_t)s.pos;
