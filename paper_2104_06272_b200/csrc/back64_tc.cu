@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    PDL_START();  // (the set-up above runs under the predecessor's tail)
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
     int G = 0;  // tiles of this CTA
     for (int u = xi; u < units; u += nx) G += (t_end(u) - t_begin(u) + SP - 1) / SP;
     bool ok = true;
@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
                     if (PL == 2) tc::tma_load_4d(sH + hs * Cfg::STAGE + BOX, ml, &hfull[hs], 0, env0, t, w);
                 }
             }
+            pdl_trigger();  // (the last loads are on their way)
             if (!ok) atomicOr(b.status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {  // ---- MMA issuer: the whole warp walks the loop, one elected lane issues

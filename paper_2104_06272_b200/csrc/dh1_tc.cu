@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1Tc
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    PDL_START();  // (the set-up above runs under the predecessor's tail)
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
     const int nchunks = nsteps * NCH;
     bool ok = true;
 
@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(320, 1) k_dh1_tc(const __grid_constant__ Dh1Tc
                 tc::tma_load_2d(sA + s * Cfg::A_STAGE, &maps.a_hi, &full[s], kc * KC, t * B + e0);
                 if (PL == 2) tc::tma_load_2d(sA + s * Cfg::A_STAGE + BOX, &maps.a_lo, &full[s], kc * KC, t * B + e0);
             }
+            pdl_trigger();  // (the last loads are on their way)
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {

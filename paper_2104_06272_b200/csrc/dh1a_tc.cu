@@ -146,7 +146,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     tc::tc_fence_after();
     if (PAIR) tc::cluster_sync_all();  // both CTAs' barriers exist before either signals the other
     const uint32_t tmem = *tmem_slot;
-    PDL_START();  // (the set-up above runs under the predecessor's tail)
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
     const uint32_t acc_agent = tmem + (uint32_t)Cfg::AGENT_COL;
     int my_tiles = 0;  // env tiles this CTA walks
     for (int mt = xi; mt < m_tiles; mt += nx) ++my_tiles;
@@ -210,6 +210,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                     if (PL == 2) tc::tma_load_2d(sA + s * Cfg::A_STAGE + Cfg::A_BOX, &maps.a_lo, &full[s], kc * KC, row);
                 }
             }
+            pdl_trigger();  // (the last loads are on their way)
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    PDL_START();  // (the set-up above runs under the predecessor's tail)
+    pdl_wait();  // (the set-up above runs under the predecessor's tail)
     bool ok = true;
 
     if (wid == 0) {
@@ -195,6 +195,7 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
                     if (BPL == 3) tc::tma_load_2d(sb + 2 * Cfg::B_PLANE + bx * Cfg::BOX, &maps.b_lo2, &bars[s], n0 + 64 * bx, k0);
                 }
             }
+            pdl_trigger();  // (the last loads are on their way)
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
     } else if (wid == 1) {
