@@ -293,7 +293,7 @@ struct Scope {
 };
 
 // Operands of the split-K "TN" GEMMs  C[m][n] = sum_k A[k][m] B[k][n]  (weight gradients).
-enum : int { A_PLANES = 0, A_ONEHOT = 1, A_WALLS = 2, A_ENV = 3 };  // A_ENV: row tile 0 = A_WALLS, row tile 1 = A_ONEHOT of idx2
+enum : int { A_PLANES = 0, A_ONEHOT = 1, A_WALLS = 2, A_ENV = 3 };  // A_ENV: the row tiles of A_WALLS, then those of A_ONEHOT of idx2
 
 struct GemmTnArgs {
     int M, N, K, klen;
@@ -308,7 +308,7 @@ struct GemmTnArgs {
     float* part;                     // out: part[split*stride + off + m*ldc + n]; row ones_row goes to off_ones + n
     size_t stride, off, off_ones;
     int ldc;
-    // A_ENV only: the second row tile is the one-hot of idx2 (M2 rows), written to part2[split*stride2 + m*ldc + n]
+    // A_ENV only: the second group of row tiles is the one-hot of idx2 (M2 rows), written to part2[split*stride2 + m*ldc + n]
     const uint8_t* idx2;
     int M2;
     float* part2;
@@ -334,7 +334,7 @@ __device__ __forceinline__ void select_policy(GemmTnArgs& g, int pol) {
 #endif
 
 // tcgen05 version (tensor memory accumulators, TMA-fed); cudaErrorNotSupported when the shape is not covered.
-cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int apl, int bpl, int prec, int splits, int* status, cudaStream_t s);
+cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int prec, int splits, int* status, cudaStream_t s);
 
 // ---- launches ----
 // Every kernel of the library is launched as a programmatic dependent of the one before it on the stream: its CTAs may be placed,
@@ -427,7 +427,6 @@ cudaError_t launch_dh1_agent_tc(const LearnArgs& a, int prec, int grid_x, float*
 void back64_shape(const Dims& d, int T, int* nx, int* ts);  // hidden width 64: dh1, S, dW2 and the agent plane in one kernel
 constexpr int BACK64_SLICES = 16;
 cudaError_t launch_back64(const LearnArgs& a, int prec, int nx, float* part_w2, float* part_agent, size_t stride_agent, cudaStream_t s);
-cudaError_t launch_dh1_tc(const LearnArgs& a, int prec, cudaStream_t s);  // tcgen05 dh1 kernel; cudaErrorNotSupported if not covered  // needs the activations the rollout saved
 cudaError_t launch_selftest_wait(int* status, long long limit_clocks, long long* waited_clocks, cudaStream_t s);
 cudaError_t launch_refresh_compute_params(const Dims& d, const Buffers& b, int prec, const Ctx& c);
 

@@ -38,7 +38,8 @@ namespace anakin {
 
 namespace {
 
-template <int H, int PREC>
+// NC: groups of 128 board cells (boards of more than 128 cells take a second agent accumulator and one dh1 accumulator)
+template <int H, int PREC, int NC>
 struct Dh1aCfg {
     static constexpr bool PAIR = H == 2 * DH1A_UNITS;  // two CTAs share an env tile, 128 units each
     static constexpr int NCTA = PAIR ? 2 : 1;
@@ -53,16 +54,17 @@ struct Dh1aCfg {
     static constexpr int A_STAGE = PL * A_BOX;
     static constexpr int D_BOX = BN * 128;               // dh1^T: 128 unit rows x 64 envs (16 KB), K-major
     static constexpr int D_TILE = PL * 2 * D_BOX;        // [plane][env half]
-    static constexpr int O_TILE = (2 / NCTA) * BM * 128; // one-hot: 128 k-rows (envs) x this CTA's cells (64-wide boxes), MN-major
+    static constexpr int O_TILE = (2 * NC / NCTA) * BM * 128; // one-hot: 128 k-rows (envs) x this CTA's cells (64-wide boxes), MN-major
     static constexpr int G_TILE = BM * (BN / 8);         // gates: 128 env rows x 16 bytes (one bit per unit)
     // W2 rows in tensor memory: two k per 32-bit column, hi plane then lo.  At H = 256 only the hi plane fits beside the
     // accumulators; the lo plane (needed for one of the three fp16 terms) stays in shared memory as K-major boxes.
     static constexpr bool W_LO_SMEM = PL == 2 && H == 256;
     static constexpr int WT_PL = W_LO_SMEM ? 1 : PL;     // planes of W2 held in tensor memory
     static constexpr int W_COLS = WT_PL * H / 2;
-    static constexpr int ACC_COL = W_COLS, AGENT_COL = W_COLS + 2 * 128;  // two dh1 accumulators, then the agent plane's
+    static constexpr int ACCS = NC == 1 ? 2 : 1;  // dh1 accumulators
+    static constexpr int ACC_COL = W_COLS, AGENT_COL = W_COLS + ACCS * 128;  // ... then the agent plane's
     static constexpr int TMEM_COLS = 512;
-    static_assert(AGENT_COL + 128 <= TMEM_COLS, "tensor memory: W2 planes + three 128-column accumulators");
+    static_assert(AGENT_COL + NC * 128 <= TMEM_COLS, "tensor memory: W2 planes + three 128-column accumulators");
     static constexpr int W_BOX = BN * 128;               // W2 lo: 128 unit rows x 64 k (16 KB), K-major
     static constexpr int W_BYTES = W_LO_SMEM ? NCH * W_BOX : 0;
     // the planes bound for tensor memory are staged by TMA in the (still unused) dh1^T tile where they fit
@@ -79,9 +81,10 @@ struct Dh1aMaps {
     CUtensorMap a_hi, a_lo, gate, w_hi, w_lo;
 };
 
-template <int H, int PREC>
+template <int H, int PREC, int NC>
 __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs& a, float* part_agent, size_t part_stride) {
-    using Cfg = Dh1aCfg<H, PREC>;
+    using Cfg = Dh1aCfg<H, PREC, NC>;
+    constexpr int ACCS = Cfg::ACCS, CTA_CELLS = 128 * NC / Cfg::NCTA;  // cells whose one-hot columns this CTA keeps
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, PL = Cfg::PL, NCH = Cfg::NCH, STAGES = Cfg::STAGES;
     constexpr bool PAIR = Cfg::PAIR;
     constexpr int NCTA = Cfg::NCTA;
@@ -216,7 +219,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     } else if (wid == 1) {
         if (leader) {  // ---- MMA issuer (of the pair): the whole warp walks the loop, one elected lane issues
             const uint32_t idesc = tc::umma_idesc<PREC>(NCTA * BN, BM, false, false);
-            const uint32_t idesc_agent = tc::umma_idesc<PREC>(NCTA * BN, 128, false, true);
+            const uint32_t idesc_agent = tc::umma_idesc<PREC>(NCTA * BN, 128 * NC, false, true);
             // agent-plane product of step v: 8 k16 steps over the 128 envs per plane of dh1 (the one-hot is exact)
             auto agent_mma = [&](int v) {
                 ok = tc::warp_all(wait_leader(tiles_full, (uint32_t)v & 1u));
@@ -242,8 +245,8 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             };
             ok = tc::warp_all(wait_leader(wfull, 0));
             for (int u = 0; u < G && ok; ++u) {
-                const int buf = u & 1;
-                if (u >= 2) ok = tc::warp_all(wait_leader(&tempty[buf], (uint32_t)((u >> 1) - 1) & 1u));  // the epilogues of step u-2 have drained it
+                const int buf = u % ACCS;
+                if (u >= ACCS) ok = tc::warp_all(wait_leader(&tempty[buf], (uint32_t)(u / ACCS - 1) & 1u));  // the epilogues of step u - ACCS have drained it
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(Cfg::ACC_COL + 128 * buf);
@@ -360,8 +363,8 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             for (int i = 0; i < 64; ++i) s_acc[i] = 0.f;
             for (int t = t0; t < t1; ++t, ++g) {
                 const int cell = (half == 0 && oh_env < B) ? (int)b.tpos[(size_t)t * B + oh_env] : -1;
-                const int buf = g & 1;
-                if (ok) ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g >> 1) & 1u);
+                const int buf = g % ACCS;
+                if (ok) ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g / ACCS) & 1u);
                 if (!ok) break;
                 tc::tc_fence_after();
                 uint32_t r0[32], r1[32];
@@ -403,9 +406,9 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                 if (lane == 0) tc::mbar_arrive(gempty);  // the gate tile may be overwritten
                 if (prev_off >= 0) *reinterpret_cast<uint16_t*>(sO + prev_off) = 0;
                 prev_off = -1;
-                if (cell >= 0 && cell < 128 && (!PAIR || (uint32_t)(cell >> 6) == rank)) {  // (pair: this CTA holds the box of its 64 cells)
+                if (cell >= 0 && cell < 128 * NC && (!PAIR || (uint32_t)(cell / CTA_CELLS) == rank)) {  // (pair: this CTA holds the boxes of its cells)
                     // element (k = env j, n = cell) of the MN-major tile: byte k*128 + ((n/8) ^ (k%8))*16 + (n%8)*2
-                    prev_off = (PAIR ? 0 : (cell >> 6) * (BM * 128)) + j * 128 + ((((cell & 63) >> 3) ^ (j & 7)) << 4) + (cell & 7) * 2;
+                    prev_off = ((cell % CTA_CELLS) >> 6) * (BM * 128) + j * 128 + ((((cell & 63) >> 3) ^ (j & 7)) << 4) + (cell & 7) * 2;
                     *reinterpret_cast<uint16_t*>(sO + prev_off) = (uint16_t)one16<PREC>();
                 }
                 tc::fence_proxy_async();  // generic-proxy stores -> visible to the tensor cores
@@ -447,17 +450,17 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
         __syncwarp();
         float* part = part_agent + (size_t)(blockIdx.z * nx + xi) * part_stride + n0 + j;
 #pragma unroll
-        for (int c0 = 0; c0 < 64; c0 += 32) {
+        for (int c0 = 0; c0 < 64 * NC; c0 += 32) {
             uint32_t r[32];
             if (got && G > 0) {
-                tc::tmem_ld32(acc_agent + lane_base + (uint32_t)(64 * half + c0), r);
+                tc::tmem_ld32(acc_agent + lane_base + (uint32_t)(64 * NC * half + c0), r);
             } else {
 #pragma unroll
                 for (int i = 0; i < 32; ++i) r[i] = 0u;  // an empty slice contributes zeros
             }
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
-                const int cell = 64 * half + c0 + i;
+                const int cell = 64 * NC * half + c0 + i;
                 if (cell < C) part[(size_t)cell * H] = __uint_as_float(r[i]);
             }
         }
@@ -472,20 +475,20 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     }
 }
 
-template <int H, int PREC>
-__global__ void __launch_bounds__(Dh1aCfg<H, PREC>::THREADS, 1)
+template <int H, int PREC, int NC>
+__global__ void __launch_bounds__(Dh1aCfg<H, PREC, NC>::THREADS, 1)
     k_dh1a_tc(const __grid_constant__ Dh1aMaps maps, LearnArgs a, float* part_agent, size_t part_stride) {
-    dh1a_body<H, PREC>(maps, a, part_agent, part_stride);
+    dh1a_body<H, PREC, NC>(maps, a, part_agent, part_stride);
 }
-template <int H, int PREC>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Dh1aCfg<H, PREC>::THREADS, 1)
+template <int H, int PREC, int NC>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Dh1aCfg<H, PREC, NC>::THREADS, 1)
     k_dh1a_pair(const __grid_constant__ Dh1aMaps maps, LearnArgs a, float* part_agent, size_t part_stride) {
-    dh1a_body<H, PREC>(maps, a, part_agent, part_stride);
+    dh1a_body<H, PREC, NC>(maps, a, part_agent, part_stride);
 }
 
-template <int H, int PREC>
+template <int H, int PREC, int NC>
 cudaError_t launch_t(const LearnArgs& a, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s) {
-    using Cfg = Dh1aCfg<H, PREC>;
+    using Cfg = Dh1aCfg<H, PREC, NC>;
     const Dims& d = a.d;
     const Buffers& b = a.b;
     const size_t R = (size_t)d.B * a.T, RH = (size_t)d.B * d.Tmax * H;
@@ -499,24 +502,29 @@ cudaError_t launch_t(const LearnArgs& a, int grid_x, float* part_agent, size_t p
     if (!make_tensor_map_2d(&maps.w_hi, b.w2p_hi, H, H, 128, bf)) return cudaErrorNotSupported;
     if (Cfg::PL == 2 && !make_tensor_map_2d(&maps.w_lo, b.w2p_lo, H, H, 128, bf)) return cudaErrorNotSupported;
     if constexpr (Cfg::PAIR) {  // the two CTAs of a pair are neighbours in x; each pair takes all H units
-        launch<k_dh1a_pair<H, PREC>>(dim3(2 * grid_x, 1, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
+        launch<k_dh1a_pair<H, PREC, NC>>(dim3(2 * grid_x, 1, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
     } else {
-        launch<k_dh1a_tc<H, PREC>>(dim3(grid_x, H / Cfg::BN, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
+        launch<k_dh1a_tc<H, PREC, NC>>(dim3(grid_x, H / Cfg::BN, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
     }
     return cudaGetLastError();
 }
 
+template <int NC>
+cudaError_t launch_nc(const LearnArgs& a, int prec, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s) {
+    if (a.d.H == 256) return prec == 1 ? launch_t<256, 1, NC>(a, grid_x, part_agent, part_stride, s) : launch_t<256, 0, NC>(a, grid_x, part_agent, part_stride, s);
+    return prec == 1 ? launch_t<128, 1, NC>(a, grid_x, part_agent, part_stride, s) : launch_t<128, 0, NC>(a, grid_x, part_agent, part_stride, s);
+}
+
 }  // namespace
 
-bool dh1_agent_tc_supported(const Dims& d) { return (d.H == 128 || d.H == 256) && d.C <= 128; }
+bool dh1_agent_tc_supported(const Dims& d) { return d.H == 128 || d.H == 256; }
 
 // grid_x CTAs share the 128-env tiles (grid_x <= ceil(B/128)); a.ts slices the steps.  The agent-plane partials go to
 // part_agent[split * part_stride + cell * H + col] with split = t slice * grid_x + blockIdx.x: grid_x * a.ts splits.
 // cudaErrorNotSupported when the shape is not covered.
 cudaError_t launch_dh1_agent_tc(const LearnArgs& a, int prec, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s) {
     if (!dh1_agent_tc_supported(a.d) || !a.b.w2p_hi || (prec != 1 && !a.b.w2p_lo)) return cudaErrorNotSupported;
-    if (a.d.H == 256) return prec == 1 ? launch_t<256, 1>(a, grid_x, part_agent, part_stride, s) : launch_t<256, 0>(a, grid_x, part_agent, part_stride, s);
-    return prec == 1 ? launch_t<128, 1>(a, grid_x, part_agent, part_stride, s) : launch_t<128, 0>(a, grid_x, part_agent, part_stride, s);
+    return a.d.C > 128 ? launch_nc<2>(a, prec, grid_x, part_agent, part_stride, s) : launch_nc<1>(a, prec, grid_x, part_agent, part_stride, s);
 }
 
 }  // namespace anakin

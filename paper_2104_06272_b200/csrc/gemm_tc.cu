@@ -148,9 +148,12 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
     constexpr bool FLUSH = Cfg::FLUSH;
     constexpr int GROUP = Cfg::GROUP;
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
-    // A_ENV: two row tiles with different synthesized A operands (wall bits + ones row; one-hot of idx2), each with its own M space
-    const int amode = AMODE == A_ENV ? (blockIdx.x == 0 ? A_WALLS : A_ONEHOT) : AMODE;
-    const int m0 = AMODE == A_ENV ? 0 : blockIdx.x * BM, n0 = blockIdx.y * BN, split = blockIdx.z;
+    // A_ENV: two groups of row tiles with different synthesized A operands (wall bits + ones row; one-hot of idx2), each with its
+    // own M space
+    const int wall_tiles = AMODE == A_ENV ? (g.M + BM - 1) / BM : 0;
+    const bool second = AMODE == A_ENV && (int)blockIdx.x >= wall_tiles;
+    const int amode = AMODE == A_ENV ? (second ? A_ONEHOT : A_WALLS) : AMODE;
+    const int m0 = ((int)blockIdx.x - (second ? wall_tiles : 0)) * BM, n0 = blockIdx.y * BN, split = blockIdx.z;
     const uint8_t* oh_idx = (AMODE == A_ENV) ? g.idx2 : g.idx;
     const int kbeg = split * g.klen, kend = min(g.K, kbeg + g.klen);
     const int nchunks = kend > kbeg ? (kend - kbeg + KC - 1) / KC : 0;
@@ -299,7 +302,6 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
         // later group adds to what this same thread wrote (program order; round-to-nearest additions in group order).
         const int q = wid & 3;
         const int m = m0 + 32 * q + lane;
-        const bool second = AMODE == A_ENV && blockIdx.x == 1;
         const int Mrows = second ? g.M2 : g.M;
         float* part = second ? g.part2 + (size_t)split * g.stride2 : g.part + (size_t)split * g.stride + g.off;
         bool got = true;
@@ -395,61 +397,34 @@ static cudaError_t launch_t(const GemmTnArgs& g, int splits, int* status, cudaSt
     if (!map(&maps.b_hi, g.Bhi, g.ldb)) return cudaErrorNotSupported;
     if (BPL >= 2 && !map(&maps.b_lo, g.Blo, g.ldb)) return cudaErrorNotSupported;
     if (BPL == 3 && !map(&maps.b_lo2, g.Blo + (g.Blo - g.Bhi), g.ldb)) return cudaErrorNotSupported;
-    dim3 grid(AMODE == A_ENV ? 2 : (g.M + Cfg::BM - 1) / Cfg::BM, (g.N + BN - 1) / BN, splits);
+    dim3 grid((g.M + Cfg::BM - 1) / Cfg::BM + (AMODE == A_ENV ? (g.M2 + Cfg::BM - 1) / Cfg::BM : 0), (g.N + BN - 1) / BN, splits);
     return launch<k_gemm_tn_tc<BN, AMODE, APL, BPL, PREC>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, g, status);
 }
 
 template <int BN, int PREC>
-static cudaError_t launch_bn(const GemmTnArgs& g, int amode, int bpl, int splits, int* status, cudaStream_t s) {
-    if constexpr (PREC == 2) {  // fp32 as three bf16 terms (plane operands: 128-column tiles, two stages of 96 KB)
-        if (amode == A_PLANES) return launch_t<128, A_PLANES, 3, 3, PREC>(g, splits, status, s);
-        if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, 3, PREC>(g, splits, status, s);
-        if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, 3, PREC>(g, splits, status, s);
-        if (amode == A_ENV && g.M <= 128 && g.M2 <= 128) return launch_t<BN, A_ENV, 1, 3, PREC>(g, splits, status, s);
-        return cudaErrorNotSupported;
-    } else {
-        constexpr int PL = PREC == 1 ? 1 : 2;
-        if (PREC == 1 && bpl == 2) {  // bf16 workload with a two-term B (the sum over t of dh1): synthesized A only
-            if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, 2, PREC>(g, splits, status, s);
-            if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, 2, PREC>(g, splits, status, s);
-            return cudaErrorNotSupported;
-        }
-        if (amode == A_PLANES) return launch_t<BN, A_PLANES, PL, PL, PREC>(g, splits, status, s);
-        if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, PL, PREC>(g, splits, status, s);
-        if (amode == A_WALLS) return launch_t<BN, A_WALLS, 1, PL, PREC>(g, splits, status, s);
-        if (amode == A_ENV && g.M <= 128 && g.M2 <= 128) return launch_t<BN, A_ENV, 1, PL, PREC>(g, splits, status, s);
-        return cudaErrorNotSupported;
-    }
-}
-
-// Covered: N = ldb = 64, 128, 256 or a multiple of 64 above (column tiles of 256 on grid.y), klen a multiple of 64, A planes or
-// one-hot A, operand planes as the fp32 workloads (hi+lo fp16; prec 2: three bf16 terms) or the bf16 workload (one plane) use them.
-cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int apl, int bpl, int prec, int splits, int* status, cudaStream_t s) {
-    const int pl = prec == 1 ? 1 : prec == 2 ? 3 : 2;
-    if (g.N != g.ldb || g.N % (prec == 2 ? 32 : 64) != 0 || g.klen % 64 != 0 || (bpl != pl && !(prec == 1 && bpl == 2 && amode != A_PLANES)) ||
-        (amode == A_PLANES && (apl != pl || g.lda % (prec == 2 ? 32 : 64) != 0)))
-        return cudaErrorNotSupported;
-    if (amode != A_PLANES && apl != 1) return cudaErrorNotSupported;
-    const int bn = g.N > 256 ? 256 : g.N;
-    if (prec == 2) {  // (columns past N read as zeros and are not stored)
-        if (bn > 128) return launch_bn<256, 2>(g, amode, bpl, splits, status, s);
-        if (bn > 64) return launch_bn<128, 2>(g, amode, bpl, splits, status, s);
-        return launch_bn<64, 2>(g, amode, bpl, splits, status, s);
-    }
-    if (prec == 1) {
-        switch (bn) {
-            case 64: return launch_bn<64, 1>(g, amode, bpl, splits, status, s);
-            case 128: return launch_bn<128, 1>(g, amode, bpl, splits, status, s);
-            case 256: return launch_bn<256, 1>(g, amode, bpl, splits, status, s);
-        }
-    } else {
-        switch (bn) {
-            case 64: return launch_bn<64, 0>(g, amode, bpl, splits, status, s);
-            case 128: return launch_bn<128, 0>(g, amode, bpl, splits, status, s);
-            case 256: return launch_bn<256, 0>(g, amode, bpl, splits, status, s);
-        }
+static cudaError_t launch_bn(const GemmTnArgs& g, int amode, int splits, int* status, cudaStream_t s) {
+    constexpr int PL = PREC == 1 ? 1 : PREC == 2 ? 3 : 2, SPL = PREC == 2 ? 3 : 2;  // terms of an activation, of S
+    // (fp32 as three bf16 terms, plane operands: 128-column tiles, two stages of 96 KB)
+    if (amode == A_PLANES) return launch_t<PREC == 2 ? 128 : BN, A_PLANES, PL, PL, PREC>(g, splits, status, s);
+    if (amode == A_ENV) return launch_t<BN, A_ENV, 1, SPL, PREC>(g, splits, status, s);
+    if constexpr (PREC == 1) {  // the agent plane of the wide layers
+        if (amode == A_ONEHOT) return launch_t<BN, A_ONEHOT, 1, 1, PREC>(g, splits, status, s);
     }
     return cudaErrorNotSupported;
+}
+
+template <int PREC>
+static cudaError_t launch_p(const GemmTnArgs& g, int amode, int splits, int* status, cudaStream_t s) {
+    if (g.N > 128) return launch_bn<256, PREC>(g, amode, splits, status, s);
+    if (g.N > 64) return launch_bn<128, PREC>(g, amode, splits, status, s);
+    return launch_bn<64, PREC>(g, amode, splits, status, s);
+}
+
+// Covered: N = ldb a multiple of 32 (column tiles of 64, 128 or 256; columns past N read as zeros and are not stored), klen a
+// multiple of 64, the planes of the workload's precision.
+cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int prec, int splits, int* status, cudaStream_t s) {
+    if (g.N != g.ldb || g.N % 32 != 0 || g.klen % 64 != 0 || (amode == A_PLANES && g.lda % 32 != 0)) return cudaErrorNotSupported;
+    return prec == 2 ? launch_p<2>(g, amode, splits, status, s) : prec == 1 ? launch_p<1>(g, amode, splits, status, s) : launch_p<0>(g, amode, splits, status, s);
 }
 
 }  // namespace anakin

@@ -893,10 +893,11 @@ __global__ void __launch_bounds__(Dh1Cfg<H, BN, PREC>::THREADS, 1) k_dh1(LearnAr
 }
 
 // ----------------------------------------------------------------------------------------------------
-// k_gemm_tn: C[m][n] = sum_k A[k][m] B[k][n], split-K partial outputs.
+// k_gemm_tn (many policies, fp32 workloads): C[m][n] = sum_k A[k][m] B[k][n], split-K partial outputs.
 // ----------------------------------------------------------------------------------------------------
-template <int BM, int BN, int AMODE, int APL, int BPL, int PREC>
+template <int BM, int BN, int AMODE>
 struct GemmTnCfg {
+    static constexpr int APL = AMODE == A_PLANES ? 2 : 1, BPL = 2;
     static constexpr int BK = 32, STAGES = 3, THREADS = 256;
     static constexpr int LDA = BM + 8, LDB = BN + 8;  // bf16 pitches
     static constexpr int A_STAGE = APL * BK * LDA, B_STAGE = BPL * BK * LDB;  // elements
@@ -905,13 +906,14 @@ struct GemmTnCfg {
     static constexpr int MT = WM / 16, NT = WN / 8;
 };
 
-template <int BM, int BN, int AMODE, int APL, int BPL, int PREC, bool GROUPED = false>
+template <int BM, int BN, int AMODE>
 __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
     pdl_wait();  // (the trigger comes after the products: CTAs of the next kernel beside these from the start cost more than the gap)
     // many policies: grid.z = policy * nsplit + split
-    const PolicyArgs<GROUPED, GemmTnArgs> pa(g_in, GROUPED ? (int)blockIdx.z / g_in.nsplit : 0);
+    const PolicyArgs<true, GemmTnArgs> pa(g_in, (int)blockIdx.z / g_in.nsplit);
     const GemmTnArgs& g = pa.a;
-    using Cfg = GemmTnCfg<BM, BN, AMODE, APL, BPL, PREC>;
+    using Cfg = GemmTnCfg<BM, BN, AMODE>;
+    constexpr int APL = Cfg::APL, BPL = Cfg::BPL, PREC = 0;
     constexpr int BK = Cfg::BK, STAGES = Cfg::STAGES, LDA = Cfg::LDA, LDB = Cfg::LDB, MT = Cfg::MT, NT = Cfg::NT;
     static_assert(NT % 2 == 0, "B fragments are loaded two n-tiles at a time");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -919,7 +921,7 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
     __nv_bfloat16* sB = sA + STAGES * Cfg::A_STAGE;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int wm = wid >> 2, wn = wid & 3;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN, split = GROUPED ? (int)blockIdx.z % g.nsplit : (int)blockIdx.z;
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN, split = (int)blockIdx.z % g.nsplit;
     const int kbeg = split * g.klen, kend = min(g.K, kbeg + g.klen);
     const int ntiles = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
 
@@ -1050,21 +1052,13 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
             }
 }
 
-template <int BM, int BN, int AMODE, int APL, int BPL, int PREC>
+template <int BM, int BN, int AMODE>
 static cudaError_t launch_gemm_tn(const GemmTnArgs& g, int rows_m, int splits, cudaStream_t s) {
-    using Cfg = GemmTnCfg<BM, BN, AMODE, APL, BPL, PREC>;
-    dim3 grid((rows_m + BM - 1) / BM, (g.N + BN - 1) / BN, splits);
-    if (g.npol > 1) {  // many policies: grid.z = policy * splits + split
-        if constexpr (PREC == 0) {
-            if ((size_t)g.npol * splits > 65535) return cudaErrorNotSupported;
-            grid.z = g.npol * splits;
-            GemmTnArgs gg = g;
-            gg.nsplit = splits;
-            return launch<k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC, true>>(grid, 256, Cfg::smem_bytes, s, gg);
-        }
-        return cudaErrorNotSupported;
-    }
-    return launch<k_gemm_tn<BM, BN, AMODE, APL, BPL, PREC>>(grid, 256, Cfg::smem_bytes, s, g);
+    using Cfg = GemmTnCfg<BM, BN, AMODE>;
+    if ((size_t)g.npol * splits > 65535) return cudaErrorNotSupported;
+    GemmTnArgs gg = g;
+    gg.nsplit = splits;
+    return launch<k_gemm_tn<BM, BN, AMODE>>(dim3((rows_m + BM - 1) / BM, (g.N + BN - 1) / BN, g.npol * splits), 256, Cfg::smem_bytes, s, gg);
 }
 
 // One Adam step of parameter i with gradient g (Kingma & Ba, Algorithm 1), plus the refreshed 16-bit copies.
@@ -1381,6 +1375,10 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     if (H > 256) {  // the bf16 GEMM CTAs of the wide path take a whole SM each (four 48 KB stages): one wave
         p->ns_w2 = 148 / tiles_hh > 0 ? 148 / tiles_hh : 1;
     }
+    if (H == 32 || H == 96 || H == 192) {  // (bf16: tiles of 128 rows x all columns in the tcgen05 GEMMs, one wave where a CTA takes an SM)
+        p->ns_w2 = std::min(splits_for((int)R, 1, 256), 148 / ((H + 127) / 128));
+        p->ns_agent = splits_for((int)R, (C + 127) / 128, 256);
+    }
     if (three_terms(H, 0)) {  // (the plan serves both precisions: room for the larger of their partial counts)
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
@@ -1450,14 +1448,8 @@ template <int H, int BN, int PREC>
 static cudaError_t launch_dh1_t(const LearnArgs& a, cudaStream_t s) {
     using Cfg = Dh1Cfg<H, BN, PREC>;
     dim3 grid((a.d.B + Cfg::BM - 1) / Cfg::BM, H / BN * a.ts);
-    if (a.d.npol > 1) {
-        if constexpr (PREC == 0) {
-            grid.z = a.d.npol;
-            return launch<k_dh1<H, BN, PREC, true>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, a);
-        }
-        return cudaErrorNotSupported;
-    }
-    return launch<k_dh1<H, BN, PREC>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, a);
+    grid.z = a.d.npol;
+    return launch<k_dh1<H, BN, PREC, PREC == 0>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, a);
 }
 
 template <int V> using ic = std::integral_constant<int, V>;
@@ -1521,9 +1513,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
                 return cudaErrorNotSupported;
         }
     }
-    // t-slices: the tcgen05 dh1 kernel has ceil(B/128)*(H/128) CTAs per slice; slice the T steps so that one wave of
-    // CTAs covers the SMs.  The mma.sync fall-back keeps one slice.
-    a.ts = 1;
+    a.ts = 1;  // slices of the steps (rows of S per env)
     bool fused_agent = false;  // dh1, S and the agent plane of dW1 in one kernel (dh1 stays on chip)
     const bool back64 = H == 64;  // ... and dW2 too
     if (back64) {
@@ -1536,28 +1526,12 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         CK(launch_back64(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
     } else if (!wide && !grouped && dh1_agent_tc_supported(d)) {
-        int gx, ts;
-        dh1a_shape(d, T, &gx, &ts);
-        a.ts = ts;
+        int gx;
+        dh1a_shape(d, T, &gx, &a.ts);
         Scope sc(c, K_DH1);
-        const cudaError_t ef = launch_dh1_agent_tc(a, PREC, gx, b.part + pl.off_agent, CH, s);
-        if (ef == cudaSuccess) {
-            fused_agent = true;
-            a.reg[1].ns = gx * ts;
-        } else if (ef != cudaErrorNotSupported) {
-            return ef;
-        } else {
-            a.ts = 1;
-        }
-    }
-    if (!fused_agent && !grouped && (H == 128 || H == 256)) {  // (the warp-level dh1 kernel walks all steps itself)
-        const int per_slice = ((B + 127) / 128) * (H / 128);
-        int ts = 148 / per_slice;
-        if (ts > 4) ts = 4;
-        if (ts > T) ts = T;
-        if (ts >= 2) a.ts = ts;
-    }
-    if (fused_agent) {
+        CK(launch_dh1_agent_tc(a, PREC, gx, b.part + pl.off_agent, CH, s));
+        fused_agent = true;
+        a.reg[1].ns = gx * a.ts;
     } else if (PREC == 2 || wide) {
         CK(launch_dh1_wide(a, c));
         if (PREC == 2) {  // fp32 dh1 rows: the agent plane and S in one pass over them
@@ -1565,29 +1539,18 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
             CK(launch_agent_plane(a, a.reg[1].ns, b.part + pl.off_agent, CH, c));
             fused_agent = true;
         }
-    } else {
+    } else {  // many policies at H = 128, bf16 at the narrow widths: the warp-level kernel
         Scope sc(c, K_DH1);
-        const cudaError_t etc = grouped ? cudaErrorNotSupported : launch_dh1_tc(a, PREC, s);  // tcgen05 where covered, else the mma.sync kernel
-        if (etc != cudaErrorNotSupported) {
-            CK(etc);
-        } else if constexpr (PREC == 2) {
-            return cudaErrorNotSupported;
-        } else {
-            const int ctas = ((B + 63) / 64) * (H > 128 ? 2 : 1);  // slices of at least two steps while SMs are without a CTA
-            a.ts = grouped ? 1 : 148 / ctas;
-            if (a.ts > 4) a.ts = 4;
-            if (a.ts > T / 2) a.ts = T / 2;
-            if (a.ts < 1) a.ts = 1;
+        const int ctas = (B + 63) / 64 * (H > 128 ? 2 : 1);  // slices of at least two steps while SMs are without a CTA
+        a.ts = grouped ? 1 : std::max(1, std::min(std::min(148 / ctas, 4), T / 2));
+        if constexpr (PREC == 0) {
+            CK((launch_dh1_t<128, 128, PREC>(a, s)));
+        } else if constexpr (PREC == 1) {
             switch (H) {
-                    case 128: CK((launch_dh1_t<128, 128, PREC>(a, s))); break;
-                case 256: CK((launch_dh1_t<256, 128, PREC>(a, s))); break;
-                default:
-                    if constexpr (PREC == 1) {
-                        if (H == 32) { CK((launch_dh1_t<32, 32, PREC>(a, s))); break; }
-                        if (H == 96) { CK((launch_dh1_t<96, 96, PREC>(a, s))); break; }
-                        if (H == 192) { CK((launch_dh1_t<192, 96, PREC>(a, s))); break; }
-                    }
-                    return cudaErrorNotSupported;
+                case 32: CK((launch_dh1_t<32, 32, PREC>(a, s))); break;
+                case 96: CK((launch_dh1_t<96, 96, PREC>(a, s))); break;
+                case 192: CK((launch_dh1_t<192, 96, PREC>(a, s))); break;
+                default: return cudaErrorNotSupported;
             }
         }
     }
@@ -1595,25 +1558,20 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const __nv_bfloat16* dh2hi = reinterpret_cast<const __nv_bfloat16*>(b.dh2);
     const __nv_bfloat16* dh1hi = reinterpret_cast<const __nv_bfloat16*>(b.dh1);
     const __nv_bfloat16* Shi = reinterpret_cast<const __nv_bfloat16*>(b.S);
-    constexpr int PL = PREC == 1 ? 1 : PREC == 2 ? 3 : 2, SPL = PREC == 2 ? 3 : 2;  // planes of an operand, of S
     auto klen_of = [](int K, int ns) { return ((K + ns - 1) / ns + 63) / 64 * 64; };
     GemmTnArgs g;
     memset(&g, 0, sizeof(g));
     const size_t RH_last = (size_t)d.B_last * d.Tmax * H;  // plane offset inside the last policy's (more compact) buffers
     if (grouped) { g.npol = d.npol; g.pstride = d.pstride; }
-    // tcgen05 where covered, else the warp-level kernel
-    auto tn_gemm = [&](auto amode_c, auto apl_c, auto bpl_c, int rows_m, int splits) -> cudaError_t {
-        constexpr int amode = decltype(amode_c)::value, apl = decltype(apl_c)::value, bpl = decltype(bpl_c)::value;
-        if (!grouped) {
-            const cudaError_t e = launch_gemm_tn_tc(g, amode, apl, bpl, PREC, splits, b.status, s);
-            if (e != cudaErrorNotSupported) return e;
+    // one policy: tcgen05; many policies (every operand moves with the policy): the warp-level kernel
+    auto tn_gemm = [&](auto amode_c, int rows_m, int splits) -> cudaError_t {
+        constexpr int amode = decltype(amode_c)::value;
+        if (!grouped) return launch_gemm_tn_tc(g, amode, PREC, splits, b.status, s);
+        if constexpr (PREC == 0 && amode != A_ENV) {
+            if (H == 128) return launch_gemm_tn<128, 128, amode>(g, rows_m, splits, s);
+            if constexpr (amode != A_PLANES) return launch_gemm_tn<64, 64, amode>(g, rows_m, splits, s);  // (H = 64: the walls and the goal)
         }
-        if constexpr (PREC == 2 || amode == A_ENV) {
-            return cudaErrorNotSupported;
-        } else {
-            if (H == 128 || H == 256) return launch_gemm_tn<128, 128, amode, apl, bpl, PREC>(g, rows_m, splits, s);
-            return launch_gemm_tn<64, 64, amode, apl, bpl, PREC>(g, rows_m, splits, s);
-        }
+        return cudaErrorNotSupported;
     };
     // dW2 = h1^T dh2
     g.M = H; g.N = H; g.K = (int)R; g.klen = klen_of(g.K, pl.ns_w2);
@@ -1624,7 +1582,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     if (wide && PREC == 2) g.Alo = h1hi + wide_h1_rows(d) * H;
     if (!fuse_dw2 && !back64) {
         Scope sc(c, K_DW2);
-        CK(tn_gemm(ic<A_PLANES>{}, ic<PL>{}, ic<PL>{}, H, pl.ns_w2));
+        CK(tn_gemm(ic<A_PLANES>{}, H, pl.ns_w2));
     }
     // dW1, agent plane = onehot(pos)^T dh1
     g.M = C; g.K = (int)R; g.klen = klen_of(g.K, pl.ns_agent);
@@ -1633,7 +1591,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     g.part = b.part + pl.off_agent; g.stride = CH; g.off = 0;
     if (!fused_agent) {
         Scope sc(c, K_DW1_AGENT);
-        CK(tn_gemm(ic<A_ONEHOT>{}, ic<1>{}, ic<PL>{}, C, pl.ns_agent));
+        CK(tn_gemm(ic<A_ONEHOT>{}, C, pl.ns_agent));
     }
     // dW1, wall plane (+ db1 through the all-ones row) = walls^T S; goal plane = onehot(goal)^T S
     g.K = a.ts * B; g.kmod = B; g.klen = klen_of(g.K, pl.ns_env);
@@ -1641,23 +1599,19 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     g.Bhi = Shi; g.Blo = Shi + (size_t)a.ts * B * H;
     g.walls = b.walls; g.W = d.W; g.ones_row = C; g.M = C + 1;
     g.part = b.part + pl.off_walls; g.stride = (size_t)(C + 1) * H; g.off = 0; g.off_ones = CH;
-    bool env_planes_done = false;
-    if (PREC != 1) {  // both planes in one launch: row tile 0 = wall bits + ones row, row tile 1 = one-hot of the goal cell
+    if (!grouped) {  // both planes in one launch: the row tiles of the wall bits + ones row, then those of the goal cell's one-hot
         g.idx2 = b.goal; g.M2 = C; g.part2 = b.part + pl.off_goal; g.stride2 = CH;
         Scope sc(c, K_DW1_WALLS);
-        const cudaError_t e = tn_gemm(ic<A_ENV>{}, ic<1>{}, ic<SPL>{}, C + 1, pl.ns_env);
-        if (e == cudaSuccess) env_planes_done = true;
-        else if (e != cudaErrorNotSupported) return e;
-    }
-    if (!env_planes_done) {
+        CK(tn_gemm(ic<A_ENV>{}, C + 1, pl.ns_env));
+    } else {
         {
             Scope sc(c, K_DW1_WALLS);
-            CK(tn_gemm(ic<A_WALLS>{}, ic<1>{}, ic<SPL>{}, C + 1, pl.ns_env));
+            CK(tn_gemm(ic<A_WALLS>{}, C + 1, pl.ns_env));
         }
         g.M = C; g.ones_row = -1; g.idx = b.goal;
         g.part = b.part + pl.off_goal; g.stride = CH;
         Scope sc(c, K_DW1_GOAL);
-        CK(tn_gemm(ic<A_ONEHOT>{}, ic<1>{}, ic<SPL>{}, C, pl.ns_env));
+        CK(tn_gemm(ic<A_ONEHOT>{}, C, pl.ns_env));
     }
     {
         Scope sc(c, K_REDUCE_ADAM);

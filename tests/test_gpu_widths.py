@@ -15,6 +15,10 @@ CASES = [
     # the warp-level kernels' widths: batches around a CTA's 32 envs and a dh1 tile's 64, one and several t-slices
     (32, 0, 33, 5, 3), (32, 1, 65, 4, 2), (96, 0, 2, 3, 4), (96, 0, 777, 7, 20), (96, 1, 64, 12, 5), (192, 0, 100, 6, 9),
     (192, 0, 5, 4, 55), (192, 1, 2100, 5, 3), (64, 0, 1500, 5, 9), (64, 1, 31, 6, 33),
+    # width 64: several steps in a 128-row tile (rows left over, slices that end short), one env more than fits, a CTA that walks
+    # more than 32 tiles; boards of more than 128 cells there and at 128 and 256
+    (64, 0, 1, 12, 5), (64, 0, 5, 16, 40), (64, 1, 64, 12, 7), (64, 0, 65, 5, 20), (64, 1, 129, 16, 3), (64, 0, 18945, 3, 17),
+    (128, 0, 130, 16, 5), (128, 1, 77, 12, 9), (256, 0, 40, 12, 7), (256, 1, 300, 16, 4), (32, 1, 300, 16, 9), (192, 1, 70, 13, 6),
     # just beyond one wave of the smaller-batch rollouts at H = 128 and 256
     (128, 0, 9473, 4, 2), (128, 1, 9500, 5, 3), (256, 0, 4737, 4, 2), (256, 1, 4800, 5, 3),
 ]
