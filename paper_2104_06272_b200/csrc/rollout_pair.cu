@@ -3,9 +3,11 @@
 //
 // Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top), hidden width 256, fp32 workloads.
 // The second layer is computed transposed,  D[j][env] = sum_k W2[k][j] h1[env][k],  as tcgen05.mma.cta_group::2 with
-// M = 256 hidden units, so that each CTA keeps only ITS 128 columns of W2 on chip (two fp16 planes, 128 KB, loaded once
-// by TMA) and builds only the h1 rows of ITS 32 envs; the tensor cores of the pair read both CTAs' h1 rows, and each
-// CTA receives its 128 hidden units x all 64 envs in its own tensor memory.  Per step:
+// M = 256 hidden units, so that each CTA keeps only ITS 128 columns of W2 on chip (two fp16 planes in TENSOR memory, the A
+// operand of every MMA, transposed into it once) and builds only the h1 rows of ITS 32 envs; the tensor cores of the pair read
+// both CTAs' h1 rows, and each CTA receives its 128 hidden units x all 64 envs in its own tensor memory.  What bounds a step
+// is the chain gather -> layer 1 -> MMAs -> heads -> action, so the agent rows of W1 stay in shared memory on boards of up to
+// 144 cells (with W2 in shared memory and these rows in L2 the gather was 950-1900 and the MMAs 2200 clocks of 7400).  Per step:
 //   layer 1   h1 = relu(base + W1[agent row])       gather-add; the fp16 (hi, lo) terms go straight into the swizzled
 //                                                   K-major operand tile [32 hi rows | 32 lo rows] x 256 k
 //   layer 2   two MMAs per k16:  W2hi x [h1hi | h1lo]  (N = 128 over the pair)  and  W2lo x h1hi  (N = 64), fp32
@@ -20,7 +22,7 @@
 // workers; partials landed -> owners) and each CTA has one barrier of its own (new positions); the cluster barrier is
 // used at start and exit only.  Every mbarrier wait is bounded; a timeout raises DEV_E_WAIT_TIMEOUT and the threads keep
 // walking through the barriers to the exit, where tensor memory is freed.
-#include <cstring>
+#include <type_traits>
 
 #include "tc_common.cuh"
 
@@ -30,52 +32,48 @@ namespace {
 
 struct PairCfg {
     static constexpr int H = 256, ME = 32, NWORK = 8, THREADS = (NWORK + 1) * 32;
-    static constexpr int BOX = 64 * 64 * 2;                   // one 64 x 64 box of 16-bit elements
-    static constexpr int A_PLANE = (128 / 64) * (H / 64) * BOX;  // this CTA's 128 columns of W2, all k: 64 KB
     static constexpr int B_CHUNK = 64 * 128;                  // 64 operand rows (32 hi + 32 lo) x 64 k
     static constexpr int B_BYTES = (H / 64) * B_CHUNK;        // 32 KB
-    static constexpr int TMEM_COLS = 256;                     // [0,128): W2hi x [hi|lo] of both CTAs, [128,192): W2lo x hi
+    // [0,128): W2hi x [hi|lo] of both CTAs, [128,192): W2lo x hi; then this CTA's 128 columns of W2 as rows (lane = hidden unit, two
+    // k per 32-bit column), hi plane and lo plane
+    static constexpr int W_COL = 256, TMEM_COLS = 512;
+    static constexpr int W1_CELLS = 144;                      // boards whose agent rows of W1 fit in shared memory
     static constexpr size_t fixed_bytes =
-        2 * (size_t)A_PLANE + B_BYTES + (size_t)ME * H * 4    // W2 planes, operand tile, base
+        (size_t)B_BYTES + (size_t)ME * H * 4                  // operand tile, base
         + 64                                                  // barriers, tensor-memory slot
-        + (size_t)8 * ME * 5 * 4                              // head partials: 8 blocks of 32 hidden units
+        + (size_t)8 * ME * 6 * 4                              // head partials: 8 blocks of 32 hidden units
         + 8 * 4 + (size_t)ME * 8 * 4 + ME * 4;                // bh, walls, pos
     static constexpr size_t gae_bytes(int T) { return (size_t)(T + 1) * ME * 4 + (size_t)T * ME; }
 };
 
-struct PairMaps {
-    CUtensorMap w_hi, w_lo;  // W2 row-major [k][j] as fp16 planes, boxes of 64 j x 64 k
-};
-
-// Asynchronous store of one float into the shared memory of a CTA of the cluster; when it has landed it counts its
-// four bytes on the mbarrier (same CTA as the destination), so the reader needs no fence from the writer.
-__device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uint32_t cluster_bar_addr) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(cluster_addr), "f"(v),
+// Asynchronous store of two floats into the shared memory of a CTA of the cluster; when it has landed it counts its
+// eight bytes on the mbarrier (same CTA as the destination), so the reader needs no fence from the writer.
+__device__ __forceinline__ void st_async_f32x2(uint32_t cluster_addr, float v0, float v1, uint32_t cluster_bar_addr) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(cluster_addr), "f"(v0), "f"(v1),
                  "r"(cluster_bar_addr)
                  : "memory");
 }
 
-template <int PREC, bool REPLAY>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(const __grid_constant__ PairMaps maps, RolloutArgs a) {
+template <int PREC, bool REPLAY, bool W1S>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(RolloutArgs a) {
     using Cfg = PairCfg;
     constexpr int H = Cfg::H, ME = Cfg::ME, NWT = Cfg::NWORK * 32;
     extern __shared__ unsigned char smem_raw[];
     // the dynamic shared memory starts at the same offset in both CTAs, so the rounded base does too
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* s_ahi = sm;
-    unsigned char* s_alo = s_ahi + Cfg::A_PLANE;
-    unsigned char* s_bop = s_alo + Cfg::A_PLANE;
+    unsigned char* s_bop = sm;
     float* s_base = reinterpret_cast<float*>(s_bop + Cfg::B_BYTES);                 // [ME][H]
-    uint64_t* wbar = reinterpret_cast<uint64_t*>(s_base + ME * H);                  // weights landed
+    uint64_t* wbar = reinterpret_cast<uint64_t*>(s_base + ME * H);                  // the agent rows of W1 landed
     uint64_t* tfull = wbar + 1;                                                     // this step's MMAs finished
-    uint64_t* ready = tfull + 1;   // [4] leader's copy: k block kb of both CTAs' operand rows written (16 warps arrive)
-    uint64_t* pfull = ready + 4;   // the eight head partials of this CTA's envs have landed (counted in bytes)
+    uint64_t* ready = tfull + 1;   // [2] leader's copy: k blocks 2i, 2i + 1 of both CTAs' operand rows written (16 warps arrive)
+    uint64_t* pfull = ready + 2;   // the eight head partials of this CTA's envs have landed (counted in bytes)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pfull + 1);
-    float* s_red = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(wbar) + 64);  // [8][ME][5]
-    float* s_bh = s_red + 8 * ME * 5;                                               // [8]
+    float* s_red = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(wbar) + 64);  // [8][ME][6]
+    float* s_bh = s_red + 8 * ME * 6;                                               // [8]
     uint32_t* s_walls = reinterpret_cast<uint32_t*>(s_bh + 8);                      // [ME][8]
     int* s_pos = reinterpret_cast<int*>(s_walls + ME * 8);                          // [ME]
-    float* s_gv = reinterpret_cast<float*>(s_pos + ME);                             // [T+1][ME] (a.gae_smem only)
+    float* s_w1 = reinterpret_cast<float*>(s_pos + ME);                             // [C][H] (W1S only)
+    float* s_gv = s_w1 + (W1S ? a.d.C * H : 0);                                     // [T+1][ME] (a.gae_smem only)
     uint8_t* s_gc = reinterpret_cast<uint8_t*>(s_gv + (a.T + 1) * ME);              // [T][ME]
 
     const Dims& d = a.d;
@@ -92,7 +90,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
     if (tid == 0) {
         tc::mbar_init(wbar, 1);
         tc::mbar_init(tfull, 1);
-        for (int kb = 0; kb < 4; ++kb) tc::mbar_init(&ready[kb], 2 * Cfg::NWORK);
+        for (int i = 0; i < 2; ++i) tc::mbar_init(&ready[i], 2 * Cfg::NWORK);
         tc::mbar_init(pfull, 1);
         tc::mbar_fence_init();
     }
@@ -102,15 +100,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     PDL_START();  // (the set-up above runs under the predecessor's tail)
-    if (tid == NWT) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
-        tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
-#pragma unroll
-        for (int kb = 0; kb < H / 64; ++kb)
-#pragma unroll
-            for (int bx = 0; bx < 2; ++bx) {
-                tc::tma_load_2d(s_ahi + (kb * 2 + bx) * Cfg::BOX, &maps.w_hi, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
-                if (PREC == 0) tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
-            }
+    if (W1S && tid == NWT) {
+        tc::mbar_expect_tx(wbar, (uint32_t)(C * H * 4));
+        tc::bulk_load(s_w1, W1 + (size_t)C * H, wbar, (uint32_t)(C * H * 4));
     }
     // hidden unit of this thread in the heads phase, and its constants
     const int q = wid & 3, rE = (wid >> 2) & 1;  // accumulator lanes 32q.., envs of CTA rE
@@ -130,6 +122,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             cp_async16(s_base + e * H + k, b.base + (size_t)(okb ? e0 + e : 0) * H + k, okb ? 16 : 0);
         }
         cp_async_commit();
+        // W2 into tensor memory, transposed: lane = hidden unit j, 32-bit column = k 2c (low half), 2c + 1.  The two warps of a lane
+        // quarter take 64 columns each of every plane.
+#pragma unroll 1
+        for (int pc = 0; pc < (PREC == 0 ? 4 : 2); ++pc) {
+            const int col0 = 64 * rE + 32 * (pc & 1);
+            const uint16_t* src = ((pc >> 1) ? b.w2p_lo : b.w2p_hi) + (size_t)(2 * col0) * H + j;
+            uint32_t r[32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) r[c] = (uint32_t)__ldg(src + (size_t)(2 * c) * H) | ((uint32_t)__ldg(src + (size_t)(2 * c + 1) * H) << 16);
+            tc::tmem_st32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(Cfg::W_COL + 128 * (pc >> 1) + col0), r);
+        }
+        tc::tmem_st_wait();
+        tc::tc_fence_before();
         b2j = b.theta_c[d.ob2 + j];
         {   // fragment element (k, n): lane = 4n + t holds k = 2t, 2t+1 (first register) and 2t+8, 2t+9 (second)
             const int n = lane >> 2, t4 = lane & 3;
@@ -157,13 +162,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
         s_pos[ow] = s.pos;
     }
     bool ok = true;
-    if (tid == NWT) ok = tc::mbar_wait(wbar, 0);  // the issuer's thread vouches for the weights of its CTA
+    if (W1S) ok = tc::mbar_wait(wbar, 0);
     __syncthreads();
     tc::cluster_sync_all();  // both CTAs' barriers, tensor memory and weights exist before the first MMA
+    tc::tc_fence_after();
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
-    const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, true, false), idesc_n = tc::umma_idesc<PREC>(256, 64, true, false);
+    const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, false, false), idesc_n = tc::umma_idesc<PREC>(256, 64, false, false);
 
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
     const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
@@ -173,39 +179,50 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             if (ow >= 0) s_pos[ow] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
             __syncthreads();
         }
-        if (tid == NWT) tc::mbar_expect_tx(pfull, 8 * ME * 5 * 4);  // this step's head partials, counted as they land
-        // ---- layer 1 (workers): 16-byte chunks of eight hidden units; all gathers of the agent's W1 row are in flight
-        // before any is used.  Trip kb covers k block kb (64 hidden units of layer 1) of all 32 envs: chunk c8 of env e goes
-        // to operand row e (hi) and 32 + e (lo) of that block, at the 16-byte position c8 ^ (e % 8) of the 128-byte row
-        // (the 128-byte swizzle of a K-major operand).  Each finished block is announced to the issuer at once, so the
-        // tensor cores start on block 0 while the later blocks are still being written.
+        if (tid == NWT) tc::mbar_expect_tx(pfull, 8 * ME * 6 * 4);  // this step's head partials, counted as they land
+        // ---- layer 1 (workers): 16-byte chunks of eight hidden units.  Trip kb covers k block kb (64 hidden units of layer 1)
+        // of all 32 envs: chunk c8 of env e goes to operand row e (hi) and 32 + e (lo) of that block, at the 16-byte position
+        // c8 ^ (e % 8) of the 128-byte row (the 128-byte swizzle of a K-major operand).  Two finished blocks are announced to
+        // the issuer together (the proxy fence costs some 300 clocks each time), so the tensor cores start on the first two
+        // while the others are being written.  Lanes 4-7 of an env read their two 16-byte pieces of a row in the other order,
+        // so that the eight lanes cover all banks.
         if (worker) {
-            const int e = tid >> 3, c8 = tid & 7;
+            const int e = tid >> 3, c8 = tid & 7, sw = (c8 >> 2) & 1;
             uint4 hi[4], lo[4];
-            const float* wrow = W1 + (size_t)(C + s_pos[e]) * H + 8 * c8;
+            const float* wrow = (W1S ? s_w1 + (size_t)s_pos[e] * H : W1 + (size_t)(C + s_pos[e]) * H) + 8 * c8;
+            const float* brow = s_base + e * H + 8 * c8;
             float4 w[4][2];
+            if (!W1S) {  // all gathers of the agent's W1 row are in flight before any is used
 #pragma unroll
-            for (int kb = 0; kb < 4; ++kb) {
-                const float4* wp = reinterpret_cast<const float4*>(wrow + 64 * kb);
-                w[kb][0] = __ldg(wp);
-                w[kb][1] = __ldg(wp + 1);
+                for (int kb = 0; kb < 4; ++kb) {
+                    w[kb][0] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * sw));
+                    w[kb][1] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ 1)));
+                }
             }
             tc::tc_fence_before();  // this thread's reads of last step's accumulators precede the arrivals below
 #pragma unroll
             for (int kb = 0; kb < 4; ++kb) {
-                const int k = 64 * kb + 8 * c8;
-                const float4 b0 = *reinterpret_cast<const float4*>(s_base + e * H + k);
-                const float4 b1 = *reinterpret_cast<const float4*>(s_base + e * H + k + 4);
-                split2<PREC>(fmaxf(b0.x + w[kb][0].x, 0.f), fmaxf(b0.y + w[kb][0].y, 0.f), hi[kb].x, lo[kb].x);
-                split2<PREC>(fmaxf(b0.z + w[kb][0].z, 0.f), fmaxf(b0.w + w[kb][0].w, 0.f), hi[kb].y, lo[kb].y);
-                split2<PREC>(fmaxf(b1.x + w[kb][1].x, 0.f), fmaxf(b1.y + w[kb][1].y, 0.f), hi[kb].z, lo[kb].z);
-                split2<PREC>(fmaxf(b1.z + w[kb][1].z, 0.f), fmaxf(b1.w + w[kb][1].w, 0.f), hi[kb].w, lo[kb].w);
+                if (W1S) {
+                    w[kb][0] = *reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * sw);
+                    w[kb][1] = *reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ 1));
+                }
+                const float4 b0 = *reinterpret_cast<const float4*>(brow + 64 * kb + 4 * sw);
+                const float4 b1 = *reinterpret_cast<const float4*>(brow + 64 * kb + 4 * (sw ^ 1));
+                uint2 h0, h1, l0, l1;
+                split2<PREC>(fmaxf(b0.x + w[kb][0].x, 0.f), fmaxf(b0.y + w[kb][0].y, 0.f), h0.x, l0.x);
+                split2<PREC>(fmaxf(b0.z + w[kb][0].z, 0.f), fmaxf(b0.w + w[kb][0].w, 0.f), h0.y, l0.y);
+                split2<PREC>(fmaxf(b1.x + w[kb][1].x, 0.f), fmaxf(b1.y + w[kb][1].y, 0.f), h1.x, l1.x);
+                split2<PREC>(fmaxf(b1.z + w[kb][1].z, 0.f), fmaxf(b1.w + w[kb][1].w, 0.f), h1.y, l1.y);
+                hi[kb] = sw ? make_uint4(h1.x, h1.y, h0.x, h0.y) : make_uint4(h0.x, h0.y, h1.x, h1.y);
+                lo[kb] = sw ? make_uint4(l1.x, l1.y, l0.x, l0.y) : make_uint4(l0.x, l0.y, l1.x, l1.y);
                 unsigned char* row = s_bop + kb * Cfg::B_CHUNK + e * 128 + ((c8 ^ (e & 7)) << 4);
                 *reinterpret_cast<uint4*>(row) = hi[kb];
                 if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
-                tc::fence_proxy_async();  // ordinary stores -> visible to the tensor cores
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[kb]), 0));
+                if (kb & 1) {
+                    tc::fence_proxy_async();  // ordinary stores -> visible to the tensor cores
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[kb >> 1]), 0));
+                }
             }
             // the copies for the update leave after the arrivals (their CTA-scope release does not wait for global stores)
             if (b.h1 != nullptr && t < a.T && e0 + e < B) {
@@ -222,29 +239,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
         const bool acting = owner && !REPLAY && t < a.T;
         StepPre pre;
         if (acting) pre = step_prepare(s, a, e0 + ow, t, s_walls + ow * 8);
-        // ---- layer 2: the leader's owner warp drives both tensor cores, k block by k block (the whole warp waits, one elected
-        // lane issues).  A block's sixteen arrivals also say that those warps have read last step's accumulators.
+        // ---- layer 2: the leader's owner warp drives both tensor cores, two k blocks at a time (the whole warp waits, one elected
+        // lane issues).  Their sixteen arrivals also say that those warps have read last step's accumulators.
         if (!worker && rank == 0) {
 #pragma unroll
-            for (int kb = 0; kb < 4; ++kb) {
-                ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[kb], (uint32_t)(t - t_beg) & 1u));
+            for (int i = 0; i < 2; ++i) {
+                ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[i], (uint32_t)(t - t_beg) & 1u));
                 tc::tc_fence_after();
                 if (tc::elect_one()) {
 #pragma unroll
-                for (int k16 = 0; k16 < 4; ++k16) {
-                    // A (MN-major): 16 k rows = 2048 bytes into each box, 8192 bytes between the two 64-column boxes
-                    const uint64_t ahi = tc::umma_desc(s_ahi + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
-                    const uint64_t alo = tc::umma_desc(s_alo + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
-                    // B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
-                    const uint64_t bd = tc::umma_desc(s_bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
-                    if (PREC == 0) {
-                        tc::umma_pair(tmem, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                        tc::umma_pair(tmem + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
-                    } else {  // bf16 operands: one product, the hi rows of the operand tile only
-                        tc::umma_pair(tmem, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                    for (int k16 = 8 * i; k16 < 8 * i + 8; ++k16) {
+                        // A: 16 k = 8 columns.  B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
+                        const uint32_t ahi = tmem + (uint32_t)(Cfg::W_COL + 8 * k16), alo = ahi + 128u;
+                        const uint64_t bd = tc::umma_desc(s_bop + (k16 >> 2) * Cfg::B_CHUNK + (k16 & 3) * 32, 16, 1024);
+                        if (PREC == 0) {
+                            tc::umma_pair_ta(tmem, ahi, bd, idesc_w, k16 ? 1u : 0u);
+                            tc::umma_pair_ta(tmem + 128u, alo, bd, idesc_n, k16 ? 1u : 0u);
+                        } else {  // bf16 operands: one product, the hi rows of the operand tile only
+                            tc::umma_pair_ta(tmem, ahi, bd, idesc_n, k16 ? 1u : 0u);
+                        }
                     }
-                }
-                if (kb == 3) tc::umma_commit_pair(tfull, 3);
+                    if (i == 1) tc::umma_commit_pair(tfull, 3);
                 }
                 __syncwarp();
             }
@@ -323,9 +338,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
                         const int e = 16 * mt + 8 * hh + g;
-                        const uint32_t dst = tc::mapa(tc::smem_u32(s_red + ((4 * (int)rank + q) * ME + e) * 5 + 2 * t4), (uint32_t)rE);
-                        if (t4 < 3) st_async_f32(dst, acc[mt][2 * hh], pbar);
-                        if (t4 < 2) st_async_f32(dst + 4u, acc[mt][2 * hh + 1], pbar);
+                        const uint32_t dst = tc::mapa(tc::smem_u32(s_red + ((4 * (int)rank + q) * ME + e) * 6 + 2 * t4), (uint32_t)rE);
+                        if (t4 < 3) st_async_f32x2(dst, acc[mt][2 * hh], acc[mt][2 * hh + 1], pbar);
                     }
             }
             // h2 for the update: one 128-byte line per env
@@ -351,9 +365,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             const int env = e0 + ow;
             if (owner) {
 #pragma unroll
-                for (int blk = 0; blk < 8; ++blk)
-#pragma unroll
-                    for (int c = 0; c < 5; ++c) o[c] += s_red[(blk * ME + ow) * 5 + c];
+                for (int blk = 0; blk < 8; ++blk) {
+                    const float2* p2 = reinterpret_cast<const float2*>(s_red + (blk * ME + ow) * 6);
+                    const float2 x0 = p2[0], x1 = p2[1];
+                    o[0] += x0.x; o[1] += x0.y; o[2] += x1.x; o[3] += x1.y;
+                    o[4] += s_red[(blk * ME + ow) * 6 + 4];
+                }
 #pragma unroll
                 for (int c = 0; c < 5; ++c) o[c] += s_bh[c];
                 if (acting) {
@@ -407,20 +424,21 @@ cudaError_t launch_rollout_pair(const RolloutArgs& a0, int prec, cudaStream_t s)
     using Cfg = PairCfg;
     if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base) return cudaErrorNotSupported;
     RolloutArgs a = a0;
-    size_t smem = Cfg::fixed_bytes + 1024;  // alignment slack
+    const bool w1s = a.d.C <= Cfg::W1_CELLS;  // (144 KB of shared memory; larger boards gather from L2)
+    size_t smem = Cfg::fixed_bytes + 1024 /*alignment slack*/ + (w1s ? (size_t)a.d.C * Cfg::H * 4 : 0);
     a.gae_smem = 0;
     if (a.fuse_gae && !a.replay && smem + Cfg::gae_bytes(a.T) <= 232448) {
         a.gae_smem = 1;
         smem += Cfg::gae_bytes(a.T);
     }
-    PairMaps maps;
-    memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, prec == 1)) return cudaErrorNotSupported;
-    if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int pairs = (a.d.B + 2 * Cfg::ME - 1) / (2 * Cfg::ME);
     const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
-    if (prec == 1) return a.replay ? launch<k_rollout_pair<1, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_pair<1, false>>(grid, Cfg::THREADS, smem, s, maps, a);
-    return a.replay ? launch<k_rollout_pair<0, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_pair<0, false>>(grid, Cfg::THREADS, smem, s, maps, a);
+    auto go = [&](auto w1s) {
+        constexpr bool W = decltype(w1s)::value;
+        if (prec == 1) return a.replay ? launch<k_rollout_pair<1, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_pair<1, false, W>>(grid, Cfg::THREADS, smem, s, a);
+        return a.replay ? launch<k_rollout_pair<0, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_pair<0, false, W>>(grid, Cfg::THREADS, smem, s, a);
+    };
+    return w1s ? go(std::true_type{}) : go(std::false_type{});
 }
 
 }  // namespace anakin
