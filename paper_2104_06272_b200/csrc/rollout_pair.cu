@@ -30,14 +30,17 @@ namespace anakin {
 
 namespace {
 
+// ME: envs per CTA, 32 or 16.  A smaller batch takes 16: the chain of a step has half the operand rows to build, half the MMA
+// columns and half the head work, on twice the SMs.
+template <int ME_>
 struct PairCfg {
-    static constexpr int H = 256, ME = 32, NWORK = 8, THREADS = (NWORK + 1) * 32;
-    static constexpr int B_CHUNK = 64 * 128;                  // 64 operand rows (32 hi + 32 lo) x 64 k
-    static constexpr int B_BYTES = (H / 64) * B_CHUNK;        // 32 KB
-    // [0,128): W2hi x [hi|lo] of both CTAs, [128,192): W2lo x hi; then this CTA's 128 columns of W2 as rows (lane = hidden unit, two
+    static constexpr int H = 256, ME = ME_, NWORK = 8, THREADS = (NWORK + 1) * 32;
+    static constexpr int B_CHUNK = 2 * ME * 128;              // operand rows (ME hi + ME lo) x 64 k
+    static constexpr int B_BYTES = (H / 64) * B_CHUNK;
+    // [0, 4 ME): W2hi x [hi|lo] of both CTAs, [128, 128 + 2 ME): W2lo x hi; then this CTA's 128 columns of W2 as rows (lane = hidden unit, two
     // k per 32-bit column), hi plane and lo plane
     static constexpr int W_COL = 256, TMEM_COLS = 512;
-    static constexpr int W1_CELLS = 144;                      // boards whose agent rows of W1 fit in shared memory
+    static constexpr int W1_CELLS = ME == 32 ? 144 : 169;     // boards whose agent rows of W1 fit in shared memory
     static constexpr size_t fixed_bytes =
         (size_t)B_BYTES + (size_t)ME * H * 4                  // operand tile, base
         + 64                                                  // barriers, tensor-memory slot
@@ -54,9 +57,9 @@ __device__ __forceinline__ void st_async_f32x2(uint32_t cluster_addr, float v0, 
                  : "memory");
 }
 
-template <int PREC, bool REPLAY, bool W1S>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1) k_rollout_pair(RolloutArgs a) {
-    using Cfg = PairCfg;
+template <int ME_, int PREC, bool REPLAY, bool W1S>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<ME_>::THREADS, 1) k_rollout_pair(RolloutArgs a) {
+    using Cfg = PairCfg<ME_>;
     constexpr int H = Cfg::H, ME = Cfg::ME, NWT = Cfg::NWORK * 32;
     extern __shared__ unsigned char smem_raw[];
     // the dynamic shared memory starts at the same offset in both CTAs, so the rounded base does too
@@ -114,7 +117,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
     s.n_episodes = s.n_goals = s.n_epsteps = 0;
     s.bad = 0;
     const int ow = tid - NWT;  // warp 8: lane = env of this CTA (its lane 0 also issues the pair's MMAs)
-    const bool owner = ow >= 0 && e0 + ow < B;
+    const bool owner = ow >= 0 && ow < ME && e0 + ow < B;
     if (worker) {
         for (int i = tid; i < ME * H / 4; i += NWT) {
             const int e = i / (H / 4), k = 4 * (i - e * (H / 4));
@@ -151,7 +154,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
         if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
         cp_async_wait<0>();
     } else {
-        for (int wi = 0; wi < 8; ++wi) s_walls[ow * 8 + wi] = (owner && wi < d.W) ? b.walls[(size_t)(e0 + ow) * d.W + wi] : 0u;
+        if (ow < ME)
+            for (int wi = 0; wi < 8; ++wi) s_walls[ow * 8 + wi] = (owner && wi < d.W) ? b.walls[(size_t)(e0 + ow) * d.W + wi] : 0u;
         if (owner) {
             s.pos = b.pos[e0 + ow];
             s.tep = b.tep[e0 + ow];
@@ -159,7 +163,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             s.goal = b.goal[e0 + ow];
             check_env_state(s, C, s_walls + ow * 8);
         }
-        s_pos[ow] = s.pos;
+        if (ow < ME) s_pos[ow] = s.pos;
     }
     bool ok = true;
     if (W1S) ok = tc::mbar_wait(wbar, 0);
@@ -169,69 +173,73 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
-    const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, false, false), idesc_n = tc::umma_idesc<PREC>(256, 64, false, false);
+    const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 4 * ME, false, false), idesc_n = tc::umma_idesc<PREC>(256, 2 * ME, false, false);
 
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
     const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
     const int t_beg = REPLAY ? (int)blockIdx.y * t_len : 0, t_end = REPLAY ? min(t_last, t_beg + t_len - 1) : t_last;
     for (int t = t_beg; t <= t_end; ++t) {
         if (REPLAY) {  // positions come from the recorded trajectory
-            if (ow >= 0) s_pos[ow] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
+            if (ow >= 0 && ow < ME) s_pos[ow] = owner ? min((int)(t < a.T ? b.tpos[(size_t)t * B + e0 + ow] : b.pos[e0 + ow]), C - 1) : 0;
             __syncthreads();
         }
         if (tid == NWT) tc::mbar_expect_tx(pfull, 8 * ME * 6 * 4);  // this step's head partials, counted as they land
         // ---- layer 1 (workers): 16-byte chunks of eight hidden units.  Trip kb covers k block kb (64 hidden units of layer 1)
-        // of all 32 envs: chunk c8 of env e goes to operand row e (hi) and 32 + e (lo) of that block, at the 16-byte position
+        // (ME = 16: warps 0-3 the even blocks, warps 4-7 the odd ones) of all envs: chunk c8 of env e goes to operand row e (hi)
+        // and ME + e (lo) of that block, at the 16-byte position
         // c8 ^ (e % 8) of the 128-byte row (the 128-byte swizzle of a K-major operand).  Two finished blocks are announced to
         // the issuer together (the proxy fence costs some 300 clocks each time), so the tensor cores start on the first two
         // while the others are being written.  Lanes 4-7 of an env read their two 16-byte pieces of a row in the other order,
         // so that the eight lanes cover all banks.
         if (worker) {
-            const int e = tid >> 3, c8 = tid & 7, sw = (c8 >> 2) & 1;
-            uint4 hi[4], lo[4];
+            const int e = (tid >> 3) % ME, c8 = tid & 7, sw = (c8 >> 2) & 1;
+            constexpr int NB = ME / 8;  // chunks of this thread: block kb_of(0), kb_of(1), ...
+            auto kb_of = [&](int i) { return ME == 32 ? i : 2 * i + (wid >> 2); };
+            uint4 hi[NB], lo[NB];
             const float* wrow = (W1S ? s_w1 + (size_t)s_pos[e] * H : W1 + (size_t)(C + s_pos[e]) * H) + 8 * c8;
             const float* brow = s_base + e * H + 8 * c8;
-            float4 w[4][2];
+            float4 w[NB][2];
             if (!W1S) {  // all gathers of the agent's W1 row are in flight before any is used
 #pragma unroll
-                for (int kb = 0; kb < 4; ++kb) {
-                    w[kb][0] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * sw));
-                    w[kb][1] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ 1)));
+                for (int i = 0; i < NB; ++i) {
+                    w[i][0] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb_of(i) + 4 * sw));
+                    w[i][1] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb_of(i) + 4 * (sw ^ 1)));
                 }
             }
             tc::tc_fence_before();  // this thread's reads of last step's accumulators precede the arrivals below
 #pragma unroll
-            for (int kb = 0; kb < 4; ++kb) {
+            for (int i = 0; i < NB; ++i) {
+                const int kb = kb_of(i);
                 if (W1S) {
-                    w[kb][0] = *reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * sw);
-                    w[kb][1] = *reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ 1));
+                    w[i][0] = *reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * sw);
+                    w[i][1] = *reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ 1));
                 }
                 const float4 b0 = *reinterpret_cast<const float4*>(brow + 64 * kb + 4 * sw);
                 const float4 b1 = *reinterpret_cast<const float4*>(brow + 64 * kb + 4 * (sw ^ 1));
                 uint2 h0, h1, l0, l1;
-                split2<PREC>(fmaxf(b0.x + w[kb][0].x, 0.f), fmaxf(b0.y + w[kb][0].y, 0.f), h0.x, l0.x);
-                split2<PREC>(fmaxf(b0.z + w[kb][0].z, 0.f), fmaxf(b0.w + w[kb][0].w, 0.f), h0.y, l0.y);
-                split2<PREC>(fmaxf(b1.x + w[kb][1].x, 0.f), fmaxf(b1.y + w[kb][1].y, 0.f), h1.x, l1.x);
-                split2<PREC>(fmaxf(b1.z + w[kb][1].z, 0.f), fmaxf(b1.w + w[kb][1].w, 0.f), h1.y, l1.y);
-                hi[kb] = sw ? make_uint4(h1.x, h1.y, h0.x, h0.y) : make_uint4(h0.x, h0.y, h1.x, h1.y);
-                lo[kb] = sw ? make_uint4(l1.x, l1.y, l0.x, l0.y) : make_uint4(l0.x, l0.y, l1.x, l1.y);
+                split2<PREC>(fmaxf(b0.x + w[i][0].x, 0.f), fmaxf(b0.y + w[i][0].y, 0.f), h0.x, l0.x);
+                split2<PREC>(fmaxf(b0.z + w[i][0].z, 0.f), fmaxf(b0.w + w[i][0].w, 0.f), h0.y, l0.y);
+                split2<PREC>(fmaxf(b1.x + w[i][1].x, 0.f), fmaxf(b1.y + w[i][1].y, 0.f), h1.x, l1.x);
+                split2<PREC>(fmaxf(b1.z + w[i][1].z, 0.f), fmaxf(b1.w + w[i][1].w, 0.f), h1.y, l1.y);
+                hi[i] = sw ? make_uint4(h1.x, h1.y, h0.x, h0.y) : make_uint4(h0.x, h0.y, h1.x, h1.y);
+                lo[i] = sw ? make_uint4(l1.x, l1.y, l0.x, l0.y) : make_uint4(l0.x, l0.y, l1.x, l1.y);
                 unsigned char* row = s_bop + kb * Cfg::B_CHUNK + e * 128 + ((c8 ^ (e & 7)) << 4);
-                *reinterpret_cast<uint4*>(row) = hi[kb];
-                if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
-                if (kb & 1) {
+                *reinterpret_cast<uint4*>(row) = hi[i];
+                if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[i];
+                if (ME == 16 || (i & 1)) {
                     tc::fence_proxy_async();  // ordinary stores -> visible to the tensor cores
                     __syncwarp();
-                    if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[kb >> 1]), 0));
+                    if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[ME == 16 ? i : i >> 1]), 0));
                 }
             }
             // the copies for the update leave after the arrivals (their CTA-scope release does not wait for global stores)
             if (b.h1 != nullptr && t < a.T && e0 + e < B) {
 #pragma unroll
-                for (int kb = 0; kb < 4; ++kb) {
-                    const size_t gi = ((size_t)t * B + e0 + e) * H + 64 * kb + 8 * c8;
-                    *reinterpret_cast<uint4*>(g_h1hi + gi) = hi[kb];
-                    if (PREC == 0) *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[kb];
-                    if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi[kb]);  // the gates of these eight units
+                for (int i = 0; i < NB; ++i) {
+                    const size_t gi = ((size_t)t * B + e0 + e) * H + 64 * kb_of(i) + 8 * c8;
+                    *reinterpret_cast<uint4*>(g_h1hi + gi) = hi[i];
+                    if (PREC == 0) *reinterpret_cast<uint4*>(g_h1lo + gi) = lo[i];
+                    if (b.gate1) b.gate1[gi >> 3] = (uint8_t)nonzero_bits16(hi[i]);  // the gates of these eight units
                 }
             }
         }
@@ -264,46 +272,53 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                 __syncwarp();
             }
         }
-        // ---- heads (workers): thread = hidden unit j, 32 envs of CTA rE
+        // ---- heads (workers): thread = hidden unit j, the ME envs of CTA rE
         if (worker) {
             if (ok) ok = tc::mbar_wait(tfull, (uint32_t)(t - t_beg) & 1u);
             tc::tc_fence_after();
-            float v[32];
+            float v[ME];
             {
-                uint32_t r0[32], r1[32], r2[32];
+                uint32_t r0[ME], r1[ME], r2[ME];
                 const uint32_t lanes = tmem + ((uint32_t)(32 * q) << 16);
-                tc::tmem_ld32_nowait(lanes + (uint32_t)((PREC == 0 ? 64 : 32) * rE), r0);  // W2hi x h1hi
+                auto load = [&](uint32_t col, uint32_t (&x)[ME]) {
+                    if constexpr (ME == 32) tc::tmem_ld32_nowait(lanes + col, x);
+                    else tc::tmem_ld16_nowait(lanes + col, x);
+                };
+                load((uint32_t)((PREC == 0 ? 2 * ME : ME) * rE), r0);  // W2hi x h1hi
                 if (PREC == 0) {
-                    tc::tmem_ld32_nowait(lanes + (uint32_t)(64 * rE + 32), r1);   // W2hi x h1lo
-                    tc::tmem_ld32_nowait(lanes + 128u + (uint32_t)(32 * rE), r2); // W2lo x h1hi
+                    load((uint32_t)(2 * ME * rE + ME), r1);    // W2hi x h1lo
+                    load(128u + (uint32_t)(ME * rE), r2);      // W2lo x h1hi
                 }
                 tc::tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
+                for (int e = 0; e < ME; ++e) {
                     float z = __uint_as_float(r0[e]);
                     if (PREC == 0) z = (z + __uint_as_float(r1[e])) + __uint_as_float(r2[e]);
                     v[e] = rnd<PREC>(fmaxf(z + b2j, 0.f));
                 }
             }
             // head partials over this warp's 32 hidden units on the warp-level tensor path.  The operand tile is free
-            // once the step's MMAs have finished: warp w keeps [32 units][32 envs] fp16 hi and lo planes in its 4 KB of it,
-            // rows of 64 bytes whose 16-byte chunks are XOR-swizzled by (row / 2) % 4 (conflict-free both ways).
-            unsigned char* wsm = s_bop + wid * 4096;
+            // once the step's MMAs have finished: warp w keeps [32 units][ME envs] fp16 hi and lo planes in its eighth of it,
+            // rows of 64 (32) bytes whose 16-byte chunks are XOR-swizzled by (row / 2) % 4 ((row / 4) % 2): conflict-free both ways.
+            unsigned char* wsm = s_bop + wid * (Cfg::B_BYTES / 8);
+            constexpr int PLANE = 32 * 2 * ME;
+            auto stage_off = [](int unit, int chunk) { return unit * (2 * ME) + ((ME == 32 ? chunk ^ ((unit >> 1) & 3) : chunk ^ ((unit >> 2) & 1)) << 4); };
 #pragma unroll
-            for (int c4 = 0; c4 < 4; ++c4) {
+            for (int c4 = 0; c4 < ME / 8; ++c4) {
                 uint4 hi, lo;
                 split2<PREC>(v[8 * c4 + 0], v[8 * c4 + 1], hi.x, lo.x);
                 split2<PREC>(v[8 * c4 + 2], v[8 * c4 + 3], hi.y, lo.y);
                 split2<PREC>(v[8 * c4 + 4], v[8 * c4 + 5], hi.z, lo.z);
                 split2<PREC>(v[8 * c4 + 6], v[8 * c4 + 7], hi.w, lo.w);
-                const int off = lane * 64 + ((c4 ^ ((lane >> 1) & 3)) << 4);
+                const int off = stage_off(lane, c4);
                 *reinterpret_cast<uint4*>(wsm + off) = hi;
-                if (PREC == 0) *reinterpret_cast<uint4*>(wsm + 2048 + off) = lo;
+                if (PREC == 0) *reinterpret_cast<uint4*>(wsm + PLANE + off) = lo;
             }
             __syncwarp();
-            float acc[2][4];
+            constexpr int MT = ME / 16;
+            float acc[MT][4];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[mt][i] = 0.f;
             {
@@ -314,12 +329,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                 for (int ks = 0; ks < 2; ++ks) {
                     const int krow = 16 * ks + 8 * (mi >> 1) + r8;
 #pragma unroll
-                    for (int mt = 0; mt < 2; ++mt) {
+                    for (int mt = 0; mt < MT; ++mt) {
                         const int chunk = 2 * mt + (mi & 1);
-                        const int off = krow * 64 + ((chunk ^ ((krow >> 1) & 3)) << 4);
+                        const int off = stage_off(krow, chunk);
                         uint32_t ahi[4], alo[4];
                         ldmatrix_x4_trans(ahi, wsm + off);
-                        if (PREC == 0) ldmatrix_x4_trans(alo, wsm + 2048 + off);
+                        if (PREC == 0) ldmatrix_x4_trans(alo, wsm + PLANE + off);
                         // the x4 order above is (k lo, m lo), (k lo, m hi), (k hi, m lo), (k hi, m hi) = a0, a1, a2, a3
                         if (PREC == 0) {
                             mma16816<PREC>(acc[mt], alo, whf_hi[ks][0], whf_hi[ks][1]);
@@ -334,7 +349,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
                 const int g = lane >> 2, t4 = lane & 3;
                 const uint32_t pbar = tc::mapa(tc::smem_u32(pfull), (uint32_t)rE);
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt)
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
                         const int e = 16 * mt + 8 * hh + g;
@@ -346,7 +361,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
             const int env0 = pair * 2 * ME + rE * ME;  // first env of the block this warp holds
             if (b.h2 != nullptr && t < a.T) {
 #pragma unroll
-                for (int e = 0; e < 32; ++e)
+                for (int e = 0; e < ME; ++e)
                     if (env0 + e < B) b.h2[((size_t)t * B + env0 + e) * H + j] = v[e];
             }
         }
@@ -420,25 +435,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg::THREADS, 1)
 
 // Covers hidden width 256 with fp32 parameters (two-term fp16 operands) when the row-major 16-bit planes of W2 exist;
 // anything else returns cudaErrorNotSupported and the caller takes the warp-level kernel.
-cudaError_t launch_rollout_pair(const RolloutArgs& a0, int prec, cudaStream_t s) {
-    using Cfg = PairCfg;
-    if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base) return cudaErrorNotSupported;
+template <int ME>
+static cudaError_t launch_pair(const RolloutArgs& a0, int prec, cudaStream_t s) {
+    using Cfg = PairCfg<ME>;
     RolloutArgs a = a0;
-    const bool w1s = a.d.C <= Cfg::W1_CELLS;  // (144 KB of shared memory; larger boards gather from L2)
+    const bool w1s = a.d.C <= Cfg::W1_CELLS;  // (larger boards gather from L2)
     size_t smem = Cfg::fixed_bytes + 1024 /*alignment slack*/ + (w1s ? (size_t)a.d.C * Cfg::H * 4 : 0);
     a.gae_smem = 0;
     if (a.fuse_gae && !a.replay && smem + Cfg::gae_bytes(a.T) <= 232448) {
         a.gae_smem = 1;
         smem += Cfg::gae_bytes(a.T);
     }
-    const int pairs = (a.d.B + 2 * Cfg::ME - 1) / (2 * Cfg::ME);
+    const int pairs = (a.d.B + 2 * ME - 1) / (2 * ME);
     const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
-    auto go = [&](auto w1s) {
-        constexpr bool W = decltype(w1s)::value;
-        if (prec == 1) return a.replay ? launch<k_rollout_pair<1, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_pair<1, false, W>>(grid, Cfg::THREADS, smem, s, a);
-        return a.replay ? launch<k_rollout_pair<0, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_pair<0, false, W>>(grid, Cfg::THREADS, smem, s, a);
+    auto go = [&](auto w1) {
+        constexpr bool W = decltype(w1)::value;
+        if constexpr (ME == 32) {
+            if (a.replay) return prec == 1 ? launch<k_rollout_pair<ME, 1, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_pair<ME, 0, true, W>>(grid, Cfg::THREADS, smem, s, a);
+        }
+        return prec == 1 ? launch<k_rollout_pair<ME, 1, false, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_pair<ME, 0, false, W>>(grid, Cfg::THREADS, smem, s, a);
     };
     return w1s ? go(std::true_type{}) : go(std::false_type{});
+}
+
+cudaError_t launch_rollout_pair(const RolloutArgs& a, int prec, cudaStream_t s) {
+    if (a.d.H != 256 || !a.b.w2p_hi || (prec == 0 && !a.b.w2p_lo) || !a.b.base) return cudaErrorNotSupported;
+    // 16 envs per CTA while one wave of pairs covers the batch
+    return !a.replay && a.d.B <= 74 * 32 ? launch_pair<16>(a, prec, s) : launch_pair<32>(a, prec, s);
 }
 
 }  // namespace anakin
