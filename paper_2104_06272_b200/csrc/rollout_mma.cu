@@ -79,9 +79,10 @@ cudaError_t launch_pack_w2(const Dims& d, const Buffers& b, int prec, const Ctx&
     return cudaGetLastError();
 }
 
-template <int H, int NW, int PREC>
+template <int H, int NW, int PREC, int ME_ = 32>
 struct RolloutMmaCfg {
-    static constexpr int ME = 32;            // envs per CTA (two m16 tiles)
+    static constexpr int ME = ME_;           // envs per CTA (two m16 tiles, or one: see the launch)
+    static constexpr int MT = ME / 16;
     static constexpr int NC = H / NW;        // output columns per warp
     static constexpr int NT = NC / 8;        // n8 tiles per warp
     static constexpr int KS = H / 16;        // k16 steps
@@ -103,13 +104,14 @@ struct RolloutMmaCfg {
 // OWN: the per-env part of a step (one lane per env) has a warp of its own beside the NW workers, which meets them at named
 // barriers: the logits-independent half of an interaction runs under the gather, and the records are written after the workers
 // have been given the new positions.  Otherwise warp 0 does both (the wide kernels' registers leave no room for another warp).
-template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN, bool REPLAY>
+// W1S: the agent rows of W1 in shared memory (the gather from L2 is a quarter of a small batch's step).
+template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN, bool REPLAY, int ME_, bool W1S>
 __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(RolloutArgs a_in) {
     pdl_wait();
     const PolicyArgs<GROUPED, RolloutArgs> pa(a_in, blockIdx.y);  // many policies: grid.y = policy
     const RolloutArgs& a = pa.a;
-    using Cfg = RolloutMmaCfg<H, NW, PREC>;
-    constexpr int ME = Cfg::ME, NT = Cfg::NT, KS = Cfg::KS, LD = Cfg::LD, NTHREADS = NW * 32 /*workers*/, NALL = NTHREADS + (OWN ? 32 : 0);
+    using Cfg = RolloutMmaCfg<H, NW, PREC, ME_>;
+    constexpr int ME = Cfg::ME, MT = Cfg::MT, NT = Cfg::NT, KS = Cfg::KS, LD = Cfg::LD, NTHREADS = NW * 32 /*workers*/, NALL = NTHREADS + (OWN ? 32 : 0);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint2* s_w2hi = reinterpret_cast<uint2*>(smem_raw);                        // [KS][H/8][32]
     uint2* s_w2mid = s_w2hi + (size_t)H * H / 4;                               // (PREC 2) the second terms
@@ -126,6 +128,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
     uint2* s_pre = reinterpret_cast<uint2*>(s_pos + ME);                       // [ME]
     float* s_gv = reinterpret_cast<float*>(s_pre + ME);                        // [T+1][ME] (a.gae_smem only)
     uint8_t* s_gc = reinterpret_cast<uint8_t*>(s_gv + (a.T + 1) * ME);         // [T][ME]
+    float* s_w1 = a.gae_smem ? reinterpret_cast<float*>(s_gc + a.T * ME) : s_gv;  // [C][H] (W1S only)
 
     const Dims& d = a.d;
     const Buffers& b = a.b;
@@ -148,6 +151,8 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
         const bool ok = e0 + e < B;
         cp_async16(s_base + e * H + j, b.base + (size_t)(ok ? e0 + e : 0) * H + j, ok ? 16 : 0);
     }
+    if (W1S)
+        for (int i = tid; i < C * H / 4; i += NALL) cp_async16(s_w1 + 4 * i, W1 + (size_t)C * H + 4 * i, 16);
     cp_async_commit();
     for (int i = tid; i < H * 5; i += NALL) s_wh[i] = b.theta_c[d.oWh + i];
     for (int i = tid; i < H; i += NALL) s_b2[i] = b.theta_c[d.ob2 + i];
@@ -207,9 +212,15 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             for (int i = 0; i < TRIPS; ++i) {
                 const int p = tid + i * NTHREADS;
                 const int e = p / (H / 8), k = 8 * (p - e * (H / 8));
-                const float4* wp = reinterpret_cast<const float4*>(W1 + (size_t)(C + s_pos[e]) * H + k);
-                w[i][0] = __ldg(wp);
-                w[i][1] = __ldg(wp + 1);
+                if (W1S) {
+                    const float4* wp = reinterpret_cast<const float4*>(s_w1 + s_pos[e] * H + k);
+                    w[i][0] = wp[0];
+                    w[i][1] = wp[1];
+                } else {
+                    const float4* wp = reinterpret_cast<const float4*>(W1 + (size_t)(C + s_pos[e]) * H + k);
+                    w[i][0] = __ldg(wp);
+                    w[i][1] = __ldg(wp + 1);
+                }
             }
 #pragma unroll
             for (int i = 0; i < TRIPS; ++i) {
@@ -250,9 +261,9 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
     };
     auto layer2_heads = [&](int t) {
         // ---- layer 2 on the tensor pipe: acc[mt][j] = rows 16mt.. x columns 8(wid*NT+j)..
-        float acc[2][NT][4];
+        float acc[MT][NT][4];
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
             for (int j = 0; j < NT; ++j)
 #pragma unroll
@@ -260,10 +271,10 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
         {
             // PREC 2: the leading products and the others in accumulators of their own (the tensor core rounds toward zero
             // at every MMA: the small terms do that at their own magnitude)
-            float accx[PREC == 2 ? 2 : 1][PREC == 2 ? NT : 1][4];
+            float accx[PREC == 2 ? MT : 1][PREC == 2 ? NT : 1][4];
             if (PREC == 2) {
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt)
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int j = 0; j < NT; ++j)
 #pragma unroll
@@ -272,9 +283,9 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             const int arow = (lane & 7) + ((lane >> 3) & 1) * 8, acol = (lane >> 4) * 8;
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks) {
-                uint32_t ahi[2][4], alo[2][4], alo2[2][4];
+                uint32_t ahi[MT][4], alo[MT][4], alo2[MT][4];
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
+                for (int mt = 0; mt < MT; ++mt) {
                     ldmatrix_x4(ahi[mt], s_h1hi + (16 * mt + arow) * LD + 16 * ks + acol);
                     if (PREC != 1) ldmatrix_x4(alo[mt], s_h1lo + (16 * mt + arow) * LD + 16 * ks + acol);
                     if (PREC == 2) ldmatrix_x4(alo2[mt], s_h1lo2 + (16 * mt + arow) * LD + 16 * ks + acol);
@@ -285,7 +296,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
                     uint2 bmid = make_uint2(0u, 0u);
                     if (PREC == 2) bmid = s_w2mid[(ks * (H / 8) + wid * NT + j) * 32 + lane];
 #pragma unroll
-                    for (int mt = 0; mt < 2; ++mt) {
+                    for (int mt = 0; mt < MT; ++mt) {
                         if (PREC == 2) {
                             mma16816<PREC>(accx[mt][j], alo2[mt], bhi.x, bhi.y);
                             mma16816<PREC>(accx[mt][j], ahi[mt], blo[ks][j].x, blo[ks][j].y);
@@ -303,7 +314,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
             }
             if (PREC == 2) {
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt)
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int j = 0; j < NT; ++j)
 #pragma unroll
@@ -312,9 +323,9 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
         }
         // ---- epilogue: bias, ReLU, head partials over this warp's columns
         {
-            float ps[4][5];  // rows g, g+8, 16+g, 24+g
+            float ps[2 * MT][5];  // rows g, g+8, (16+g, 24+g)
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int r = 0; r < 2 * MT; ++r)
 #pragma unroll
                 for (int c = 0; c < 5; ++c) ps[r][c] = 0.f;
             const bool save_h2 = b.h2 != nullptr && t < a.T;
@@ -325,12 +336,12 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
                 for (int cc = 0; cc < 2; ++cc) {
                     const float bias = s_b2[col0 + cc];
 #pragma unroll
-                    for (int mt = 0; mt < 2; ++mt)
+                    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                         for (int hh = 0; hh < 2; ++hh) acc[mt][j][2 * hh + cc] = rnd<PREC>(fmaxf(acc[mt][j][2 * hh + cc] + bias, 0.f));
                 }
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt)
+                for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
                         const int row = 16 * mt + 8 * hh + g;
@@ -344,7 +355,7 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
 #pragma unroll
                     for (int c = 0; c < 5; ++c) wh[c] = s_wh[(col0 + cc) * 5 + c];
 #pragma unroll
-                    for (int mt = 0; mt < 2; ++mt)
+                    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                         for (int hh = 0; hh < 2; ++hh) {
                             const float h2 = acc[mt][j][2 * hh + cc];
@@ -354,25 +365,35 @@ __global__ void __launch_bounds__(NW * 32 + (OWN ? 32 : 0), MINB) k_rollout_mma(
                 }
             }
             // sum over the four lanes of a quad with a transposing exchange: after two rounds lane t4 holds the total
-            // of ONE of the four rows (15 shuffles instead of 40), and every lane stores its row
-            float q2[2][5];
+            // of ONE of the four rows (15 shuffles instead of 40; ME = 16: of one of two), and every lane stores its row
             const bool b0 = t4 & 1, b1 = t4 & 2;
+            if constexpr (MT == 2) {
+                float q2[2][5];
 #pragma unroll
-            for (int c = 0; c < 5; ++c) {
+                for (int c = 0; c < 5; ++c) {
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const float send = b0 ? ps[i][c] : ps[2 + i][c];
-                    const float keep = b0 ? ps[2 + i][c] : ps[i][c];
-                    q2[i][c] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 1);
+                    for (int i = 0; i < 2; ++i) {
+                        const float send = b0 ? ps[i][c] : ps[2 + i][c];
+                        const float keep = b0 ? ps[2 + i][c] : ps[i][c];
+                        q2[i][c] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 1);
+                    }
                 }
-            }
-            const int r = (b0 ? 2 : 0) + (b1 ? 1 : 0);
-            const int row = 16 * (r >> 1) + 8 * (r & 1) + g;
+                const int r = (b0 ? 2 : 0) + (b1 ? 1 : 0);
+                const int row = 16 * (r >> 1) + 8 * (r & 1) + g;
 #pragma unroll
-            for (int c = 0; c < 5; ++c) {
-                const float send = b1 ? q2[0][c] : q2[1][c];
-                const float keep = b1 ? q2[1][c] : q2[0][c];
-                s_red[(wid * ME + row) * 5 + c] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 2);
+                for (int c = 0; c < 5; ++c) {
+                    const float send = b1 ? q2[0][c] : q2[1][c];
+                    const float keep = b1 ? q2[1][c] : q2[0][c];
+                    s_red[(wid * ME + row) * 5 + c] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 2);
+                }
+            } else {
+                const int row = 8 * b0 + g;
+#pragma unroll
+                for (int c = 0; c < 5; ++c) {
+                    float x = (b0 ? ps[1][c] : ps[0][c]) + __shfl_xor_sync(0xFFFFFFFFu, b0 ? ps[0][c] : ps[1][c], 1);
+                    x += __shfl_xor_sync(0xFFFFFFFFu, x, 2);
+                    if (!b1) s_red[(wid * ME + row) * 5 + c] = x;
+                }
             }
         }
     };
@@ -480,14 +501,32 @@ constexpr size_t MAX_DYN_SMEM = 232448;  // 227 KB of dynamic shared memory per 
 
 template <int H, int NW, int PREC, bool GROUPED, int MINB, bool OWN>
 static cudaError_t launch_k(const RolloutArgs& a, dim3 grid, size_t smem, cudaStream_t s) {
-    if (a.replay) return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN, true>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
-    return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN, false>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
+    if (a.replay) return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN, true, 32, false>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
+    return launch<k_rollout_mma<H, NW, PREC, GROUPED, MINB, OWN, false, 32, false>>(grid, NW * 32 + (OWN ? 32 : 0), smem, s, a);
+}
+
+// Small batches: 16 envs per CTA, half the chain of a step for each, while every CTA finds an SM of its own (the narrow widths:
+// up to three to an SM; bf16 at 96: two).  B200, T = 16, 64 and 2368 envs: H = 32 22 -> 15 and 17 us, 64 24 -> 18 and 22, 96 49 -> 30
+// and 31, 128 43 -> 29 and 30, 192 113 -> 63 and 65; past the line (3000 envs): 96 50 -> 59, 128 44 -> 56, 192 116 -> 126.
+template <int H, int PREC> constexpr int small_ctas() { return H <= 64 ? 444 : H == 96 && PREC == 1 ? 296 : 148; }
+template <int H, int NW, int PREC>
+static cudaError_t launch_small(RolloutArgs a, cudaStream_t s) {
+    using Cfg = RolloutMmaCfg<H, NW, PREC, 16>;
+    size_t smem = Cfg::smem_bytes;
+    a.gae_smem = a.fuse_gae && smem + Cfg::gae_bytes(a.T) <= MAX_DYN_SMEM;
+    if (a.gae_smem) smem += Cfg::gae_bytes(a.T);
+    const unsigned ctas = (a.d.B + 15) / 16;
+    const size_t w1 = (size_t)a.d.C * H * 4;
+    if (smem + w1 <= MAX_DYN_SMEM) return launch<k_rollout_mma<H, NW, PREC, false, 1, true, false, 16, true>>(ctas, NW * 32 + 32, smem + w1, s, a);
+    return launch<k_rollout_mma<H, NW, PREC, false, 1, true, false, 16, false>>(ctas, NW * 32 + 32, smem, s, a);
 }
 
 template <int H, int NW, int PREC, bool GROUPED = false>
 static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
     using Cfg = RolloutMmaCfg<H, NW, PREC>;
     RolloutArgs a = a0;
+    if constexpr (!GROUPED)
+        if (!a.replay && a.d.B <= 16 * small_ctas<H, PREC>()) return launch_small<H, NW, PREC>(a, s);
     size_t smem = Cfg::smem_bytes;
     a.gae_smem = 0;
     if (a.fuse_gae && !a.replay && smem + Cfg::gae_bytes(a.T) <= MAX_DYN_SMEM) {
