@@ -541,6 +541,11 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
         if (slices > (steps + 1) / 2) slices = (steps + 1) / 2;
     }
     const dim3 grid(ctas, GROUPED ? a.d.npol : slices);
+    // Three-term operands at H = 96, a CTA to an SM: the registers of a whole SM, and the agent rows of W1 (B200, T = 16, 4736 envs:
+    // 70 -> 48 us; the other widths and bf16 gain nothing from these rows, their gathers hide behind twice the MMAs).
+    const size_t w1 = (size_t)a.d.C * H * 4;
+    if constexpr (!GROUPED && H == 96 && PREC == 2)
+        if (!a.replay && ctas <= 148 && smem + w1 <= MAX_DYN_SMEM) return launch<k_rollout_mma<H, NW, PREC, false, 1, true, false, 32, true>>(grid, NW * 32 + 32, smem + w1, s, a);
     // The owner warp costs a CTA of the 128-wide kernel its second place on an SM: only where every CTA gets an SM of its own.
     // (H = 64: three CTAs per SM where there are that many)
     if constexpr (H == 64)

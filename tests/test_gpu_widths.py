@@ -23,7 +23,7 @@ CASES = [
     (128, 0, 9473, 4, 2), (128, 1, 9500, 5, 3), (256, 0, 4737, 4, 2), (256, 1, 4800, 5, 3),
     # 16 and 32 envs per CTA, agent rows of W1 in shared memory and not
     (256, 0, 2368, 4, 2), (256, 0, 2369, 12, 2), (256, 1, 2500, 13, 2), (256, 0, 19, 13, 3), (256, 1, 33, 14, 3),
-    (192, 0, 17, 16, 3), (192, 0, 2369, 3, 2), (128, 1, 2368, 16, 2), (128, 0, 2400, 5, 2), (96, 0, 2368, 5, 2),
+    (192, 0, 17, 16, 3), (192, 0, 2369, 3, 2), (128, 1, 2368, 16, 2), (128, 0, 2400, 5, 2), (96, 0, 2368, 5, 2), (96, 0, 2380, 5, 3), (96, 0, 4737, 3, 2),
 ]
 
 
