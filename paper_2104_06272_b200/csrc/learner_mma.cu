@@ -1390,7 +1390,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     }
     p->ns_env = splits_for(d.B, tiles_ch, 128);
     if (H == 64) {  // (one partial per CTA of the fused kernel; its slices of the steps are rows of S)
-        p->ns_w2 = p->ns_agent = 148 / d.npol > 0 ? 148 / d.npol : 1;
+        const int units = d.B > 64 ? (d.B + 127) / 128 * std::min(BACK64_SLICES, d.Tmax) : (d.Tmax + 128 / d.B - 1) / (128 / d.B);  // (of any T <= Tmax)
+        p->ns_w2 = p->ns_agent = std::min(std::max(148 / d.npol, 1), units);
         p->ns_env = splits_for(std::max(4 * d.B, std::min(BACK64_SLICES * d.B, 148 * 128)), tiles_ch, 256);
     }
     const size_t tiles32 = (R + 31) / 32;
