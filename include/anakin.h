@@ -231,7 +231,7 @@ int anakin_learn_ppo(anakin_t* h, int epochs, float clip_eps);
  *   3. runs the update of anakin_update (policy gradient with ADV, value regression to RET, entropy bonus, Adam).
  * With pi = mu and both levels >= 1 it is the A2C update with GAE at lambda = 1.  Consumes the pending rollout.
  * Errors: BAD_STATE if none is pending; INVALID_ARG for epochs < 1 or a negative level; UNSUPPORTED_CFG on hidden widths
- * whose rollout does not save the head outputs (the generic non-tensor path).
+ * other than 64, 128, 256 and, in bf16, 512 and 1024.
  */
 int anakin_learn_vtrace(anakin_t* h, int epochs, float rho_bar, float c_bar);
 
