@@ -9,8 +9,9 @@
 //   layer 1   h1 = relu(base + W1[agent row])       gather-add; the fp16 (hi, lo) terms go straight into the swizzled
 //                                                   K-major operand tile [64 hi rows | 64 lo rows] x 128 k
 //   layer 2   transposed, D[j][env] = sum_k W2[k][j] h1[env][k], M = 128 hidden units: two tcgen05 MMAs per k16,
-//             W2hi x [h1hi | h1lo] (N = 128) and W2lo x h1hi (N = 64), fp32 accumulators in tensor memory; both fp16
-//             planes of W2 (64 KB) are loaded once by TMA; one thread of a dedicated warp issues the MMAs of both groups
+//             W2hi x [h1hi | h1lo] (N = 128) and W2lo x h1hi (N = 64), fp32 accumulators in tensor memory beside both
+//             planes of W2 (the A operand, transposed into it once: shared memory then holds the agent rows of W1 and is left
+//             to the workers; 2336 -> 2224 us on 131072 envs, T = 64); a dedicated warp issues the MMAs of both groups
 //   heads     a worker thread = one hidden unit j (its accumulator lane): bias, ReLU, h2 stores (one 128-byte line per
 //             env and warp); the warp's 32 units x 32 envs go to shared memory as fp16 (hi, lo) terms and come back
 //             transposed (ldmatrix.trans) as A fragments of warp-level MMAs against Wh; the four 32-unit partials of an
@@ -20,7 +21,7 @@
 // The phases meet through mbarriers only (operand blocks written -> issuer; MMAs finished -> workers; partials stored ->
 // owners; positions published -> workers).  Every wait is bounded; a timeout raises DEV_E_WAIT_TIMEOUT and the threads
 // keep walking through the barriers to the exit, where tensor memory is freed.
-#include <cstring>
+#include <type_traits>
 
 #include "tc_common.cuh"
 
@@ -33,35 +34,28 @@ struct Tc128Cfg {
     static constexpr int NWT = NG * NWORK * 32;                 // worker threads
     static constexpr int NOWN = NG * NE;                        // owner threads: one per env
     static constexpr int THREADS = NWT + NOWN + 32;             // + the issuer warp
-    static constexpr int BOX = 64 * 64 * 2;                     // one 64 x 64 box of 16-bit elements
-    static constexpr int A_PLANE = (H / 64) * (H / 64) * BOX;   // all of W2 as one fp16 plane: 32 KB
     static constexpr int B_CHUNK = 2 * NE * 128;                // 128 operand rows (64 hi + 64 lo) x 64 k: 16 KB
     static constexpr int B_BYTES = (H / 64) * B_CHUNK;          // a group's operand tile: 32 KB
     static constexpr int ACC = 192;                             // TMEM columns of a group: [0,128) W2hi x [hi|lo], [128,192) W2lo x hi
-    static constexpr int TMEM_COLS = 512;
+    static constexpr int W_COL = NG * ACC, TMEM_COLS = 512;     // W2: 64 columns a plane (two k per column), hi then lo
     static constexpr size_t fixed_bytes =
-        2 * (size_t)A_PLANE + (size_t)NG * B_BYTES + (size_t)NG * NE * H * 4  // W2 planes, operand tiles, base
+        (size_t)NG * B_BYTES + (size_t)NG * NE * H * 4                        // operand tiles, base
         + 256                                                                 // barriers, tensor-memory slot
         + (size_t)NG * 4 * NE * 5 * 4                                         // head partials: 4 blocks of 32 hidden units
         + 8 * 4 + (size_t)NOWN * 8 * 4 + NOWN * 4;                            // bh, walls, pos
     static constexpr size_t gae_bytes(int T) { return (size_t)(T + 1) * NOWN * 4 + (size_t)T * NOWN; }
 };
 
-struct Tc128Maps {
-    CUtensorMap w_hi, w_lo;  // W2 row-major [k][j] as fp16 planes, boxes of 64 j x 64 k
-};
-
-template <int PREC, bool REPLAY>
-__global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __grid_constant__ Tc128Maps maps, RolloutArgs a) {
+// W1S: the agent rows of W1 in shared memory too (512 bytes a cell; larger boards gather from L2).
+template <int PREC, bool REPLAY, bool W1S>
+__global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(RolloutArgs a) {
     using Cfg = Tc128Cfg;
     constexpr int H = Cfg::H, NE = Cfg::NE, NG = Cfg::NG, NWT = Cfg::NWT, NOWN = Cfg::NOWN;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);  // the swizzle needs 1024-byte alignment
-    unsigned char* s_ahi = sm;
-    unsigned char* s_alo = s_ahi + Cfg::A_PLANE;
-    unsigned char* s_bop = s_alo + Cfg::A_PLANE;                                     // [NG] operand tiles
+    unsigned char* s_bop = sm;                                                       // [NG] operand tiles
     float* s_base = reinterpret_cast<float*>(s_bop + NG * Cfg::B_BYTES);             // [NG][NE][H]
-    uint64_t* wbar = reinterpret_cast<uint64_t*>(s_base + NG * NE * H);              // weights landed
+    uint64_t* wbar = reinterpret_cast<uint64_t*>(s_base + NG * NE * H);              // the agent rows of W1 landed
     uint64_t* tfull = wbar + 1;     // [NG] this step's MMAs of the group finished
     uint64_t* ready = tfull + NG;   // [NG][2] k block of the group's operand rows written (8 worker warps arrive)
     uint64_t* pdone = ready + NG * 2;  // [NG] the four head partials of every env of the group are stored (8 warps arrive)
@@ -71,7 +65,8 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
     float* s_bh = s_red + NG * 4 * NE * 5;                                           // [8]
     uint32_t* s_walls = reinterpret_cast<uint32_t*>(s_bh + 8);                       // [NOWN][8]
     int* s_pos = reinterpret_cast<int*>(s_walls + NOWN * 8);                         // [NOWN]
-    float* s_gv = reinterpret_cast<float*>(s_pos + NOWN);                            // [T+1][NOWN] (a.gae_smem only)
+    float* s_w1 = reinterpret_cast<float*>(s_pos + NOWN);                            // [C][H] (W1S only)
+    float* s_gv = s_w1 + (W1S ? a.d.C * H : 0);                                      // [T+1][NOWN] (a.gae_smem only)
     uint8_t* s_gc = reinterpret_cast<uint8_t*>(s_gv + (a.T + 1) * NOWN);             // [T][NOWN]
 
     const Dims& d = a.d;
@@ -105,15 +100,9 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
     const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
     const int t_beg = REPLAY ? (int)blockIdx.y * t_len : 0, t_end = REPLAY ? min(t_last, t_beg + t_len - 1) : t_last;
-    if (issuer) {  // all of W2: box (kb, bx) = k rows 64kb.., columns 64bx..
-        tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
-#pragma unroll
-        for (int kb = 0; kb < H / 64; ++kb)
-#pragma unroll
-            for (int bx = 0; bx < H / 64; ++bx) {
-                tc::tma_load_2d(s_ahi + (kb * (H / 64) + bx) * Cfg::BOX, &maps.w_hi, wbar, 64 * bx, 64 * kb);
-                if (PREC == 0) tc::tma_load_2d(s_alo + (kb * (H / 64) + bx) * Cfg::BOX, &maps.w_lo, wbar, 64 * bx, 64 * kb);
-            }
+    if (W1S && issuer) {
+        tc::mbar_expect_tx(wbar, (uint32_t)(C * H * 4));
+        tc::bulk_load(s_w1, W1 + (size_t)C * H, wbar, (uint32_t)(C * H * 4));
     }
     // worker constants: hidden unit of this thread in the heads phase (its accumulator lane) and the env half it reads
     const int wg = worker ? wid / Cfg::NWORK : 0;   // the worker's group
@@ -137,6 +126,19 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
             cp_async16(s_base + e * H + k, b.base + (size_t)(okb ? e0 + e : 0) * H + k, okb ? 16 : 0);
         }
         cp_async_commit();
+        {   // W2 into tensor memory, transposed: lane = hidden unit j, 32-bit column = k 2c (low half), 2c + 1; the four warps of a
+            // lane quarter take half a plane each
+            const int pc = wid >> 2, col0 = 32 * (pc & 1);
+            if (PREC == 0 || pc < 2) {
+                const uint16_t* src = ((pc >> 1) ? b.w2p_lo : b.w2p_hi) + (size_t)(2 * col0) * H + j;
+                uint32_t r[32];
+#pragma unroll
+                for (int c = 0; c < 32; ++c) r[c] = (uint32_t)__ldg(src + (size_t)(2 * c) * H) | ((uint32_t)__ldg(src + (size_t)(2 * c + 1) * H) << 16);
+                tc::tmem_st32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(Cfg::W_COL + 64 * (pc >> 1) + col0), r);
+                tc::tmem_st_wait();
+            }
+            tc::tc_fence_before();
+        }
         b2j = b.theta_c[d.ob2 + j];
         {   // fragment element (k, n): lane = 4n + t holds k = 2t, 2t+1 (first register) and 2t+8, 2t+9 (second)
             const int n = lane >> 2, t4 = lane & 3;
@@ -165,8 +167,9 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         s_pos[ow] = s.pos;
     }
     bool ok = true;
-    if (issuer) ok = tc::mbar_wait(wbar, 0);
+    if (W1S && worker) ok = tc::mbar_wait(wbar, 0);
     __syncthreads();
+    tc::tc_fence_after();
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         // ---- layer 2: one warp drives the tensor core for both groups (an elected lane issues), k block by k block, in the order the groups'
         // operand blocks are written (group 0, then group 1, every step).  A block's eight arrivals also say that those
         // warps have read the group's accumulators of the step before.
-        const uint32_t idesc_w = tc::umma_idesc<PREC>(128, 128, true, false), idesc_n = tc::umma_idesc<PREC>(128, 64, true, false);
+        const uint32_t idesc_w = tc::umma_idesc<PREC>(128, 128, false, false), idesc_n = tc::umma_idesc<PREC>(128, 64, false, false);
         for (int t = t_beg; t <= t_end; ++t) {
             for (int g = 0; g < NG; ++g) {
                 const uint32_t acc = tmem + (uint32_t)(g * Cfg::ACC);
@@ -187,16 +190,14 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                     if (tc::elect_one()) {
 #pragma unroll
                     for (int k16 = 0; k16 < 4; ++k16) {
-                        // A (MN-major): 16 k rows = 2048 bytes into each box, one box further per 64 columns
-                        const uint64_t ahi = tc::umma_desc(s_ahi + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
-                        const uint64_t alo = tc::umma_desc(s_alo + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
-                        // B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
+                        // A: 16 k = 8 columns.  B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
+                        const uint32_t ahi = tmem + (uint32_t)(Cfg::W_COL + 32 * kb + 8 * k16);
                         const uint64_t bd = tc::umma_desc(bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
                         if (PREC == 0) {
-                            tc::umma(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                            tc::umma(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            tc::umma_ta(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
+                            tc::umma_ta(acc + 128u, ahi + 64u, bd, idesc_n, (kb | k16) ? 1u : 0u);
                         } else {  // bf16 operands: one product, the hi rows of the operand tile only
-                            tc::umma(acc, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            tc::umma_ta(acc, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
                         }
                     }
                     if (kb == 1) tc::umma_commit(&tfull[g]);
@@ -212,18 +213,21 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
         // 16-byte position c8 ^ (row % 8) of the 128-byte row (the 128-byte swizzle of a K-major operand).  Each finished
         // block is announced to the issuer at once.
         auto gather = [&](int g, int t) {
-            const int e = tidg >> 3, c8 = tidg & 7;
+            // (lanes 4-7 of an env read their two 16-byte pieces of a row in the other order: the eight lanes cover all banks)
+            const int e = tidg >> 3, c8 = tidg & 7, sw = (c8 >> 2) & 1;
             unsigned char* bop = s_bop + g * Cfg::B_BYTES;
             float4 w[2][2][2];
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                const float* wrow = W1 + (size_t)(C + s_pos[g * NE + e + 32 * p]) * H + 8 * c8;
+                const int pos = s_pos[g * NE + e + 32 * p];
+                const float* wrow = (W1S ? s_w1 + pos * H : W1 + (size_t)(C + pos) * H) + 8 * c8;
 #pragma unroll
-                for (int kb = 0; kb < 2; ++kb) {
-                    const float4* wp = reinterpret_cast<const float4*>(wrow + 64 * kb);
-                    w[kb][p][0] = __ldg(wp);
-                    w[kb][p][1] = __ldg(wp + 1);
-                }
+                for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const float4* wp = reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ x));
+                        w[kb][p][x] = W1S ? *wp : __ldg(wp);
+                    }
             }
             tc::tc_fence_before();  // this thread's reads of the group's accumulators precede the arrivals below
             uint4 hi[2][2], lo[2][2];
@@ -233,13 +237,15 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(const __
                 for (int p = 0; p < 2; ++p) {
                     const int er = e + 32 * p, k = 64 * kb + 8 * c8;  // row within the group
                     const float* bp = s_base + (g * NE + er) * H + k;
-                    const float4 b0 = *reinterpret_cast<const float4*>(bp);
-                    const float4 b1 = *reinterpret_cast<const float4*>(bp + 4);
+                    const float4 b0 = *reinterpret_cast<const float4*>(bp + 4 * sw), b1 = *reinterpret_cast<const float4*>(bp + 4 * (sw ^ 1));
                     const float4 w0 = w[kb][p][0], w1 = w[kb][p][1];
-                    split2<PREC>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), hi[kb][p].x, lo[kb][p].x);
-                    split2<PREC>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), hi[kb][p].y, lo[kb][p].y);
-                    split2<PREC>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), hi[kb][p].z, lo[kb][p].z);
-                    split2<PREC>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), hi[kb][p].w, lo[kb][p].w);
+                    uint2 h0, h1, l0, l1;
+                    split2<PREC>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), h0.x, l0.x);
+                    split2<PREC>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), h0.y, l0.y);
+                    split2<PREC>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), h1.x, l1.x);
+                    split2<PREC>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), h1.y, l1.y);
+                    hi[kb][p] = sw ? make_uint4(h1.x, h1.y, h0.x, h0.y) : make_uint4(h0.x, h0.y, h1.x, h1.y);
+                    lo[kb][p] = sw ? make_uint4(l1.x, l1.y, l0.x, l0.y) : make_uint4(l0.x, l0.y, l1.x, l1.y);
                     unsigned char* row = bop + kb * Cfg::B_CHUNK + er * 128 + ((c8 ^ (er & 7)) << 4);
                     *reinterpret_cast<uint4*>(row) = hi[kb][p];
                     if (PREC == 0) *reinterpret_cast<uint4*>(row + NE * 128) = lo[kb][p];
@@ -442,19 +448,22 @@ cudaError_t launch_rollout_tc128(const RolloutArgs& a0, int prec, cudaStream_t s
     if (a0.replay ? a0.d.B <= Cfg::NE : a0.d.B <= 148 * 64) return cudaErrorNotSupported;
     RolloutArgs a = a0;
     size_t smem = Cfg::fixed_bytes + 1024;  // alignment slack
+    const size_t w1 = (size_t)a.d.C * Cfg::H * 4;
+    const bool w1s = smem + w1 <= 232448;
+    if (w1s) smem += w1;
     a.gae_smem = 0;
     if (a.fuse_gae && !a.replay && smem + Cfg::gae_bytes(a.T) <= 232448) {
         a.gae_smem = 1;
         smem += Cfg::gae_bytes(a.T);
     }
-    Tc128Maps maps;
-    memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, prec == 1)) return cudaErrorNotSupported;
-    if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int ctas = (a.d.B + Cfg::NOWN - 1) / Cfg::NOWN;
     const dim3 grid(ctas, replay_slices(a, ctas));
-    if (prec == 1) return a.replay ? launch<k_rollout_tc128<1, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_tc128<1, false>>(grid, Cfg::THREADS, smem, s, maps, a);
-    return a.replay ? launch<k_rollout_tc128<0, true>>(grid, Cfg::THREADS, smem, s, maps, a) : launch<k_rollout_tc128<0, false>>(grid, Cfg::THREADS, smem, s, maps, a);
+    auto go = [&](auto w) {
+        constexpr bool W = decltype(w)::value;
+        if (prec == 1) return a.replay ? launch<k_rollout_tc128<1, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_tc128<1, false, W>>(grid, Cfg::THREADS, smem, s, a);
+        return a.replay ? launch<k_rollout_tc128<0, true, W>>(grid, Cfg::THREADS, smem, s, a) : launch<k_rollout_tc128<0, false, W>>(grid, Cfg::THREADS, smem, s, a);
+    };
+    return w1s ? go(std::true_type{}) : go(std::false_type{});
 }
 
 }  // namespace anakin

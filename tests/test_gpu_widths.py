@@ -20,7 +20,7 @@ CASES = [
     (64, 0, 1, 12, 5), (64, 0, 5, 16, 40), (64, 1, 64, 12, 7), (64, 0, 65, 5, 20), (64, 1, 129, 16, 3), (64, 0, 18945, 3, 17),
     (128, 0, 130, 16, 5), (128, 1, 77, 12, 9), (256, 0, 40, 12, 7), (256, 1, 300, 16, 4), (32, 1, 300, 16, 9), (192, 1, 70, 13, 6),
     # just beyond one wave of the smaller-batch rollouts at H = 128 and 256
-    (128, 0, 9473, 4, 2), (128, 1, 9500, 5, 3), (256, 0, 4737, 4, 2), (256, 1, 4800, 5, 3),
+    (128, 0, 9473, 4, 2), (128, 1, 9500, 5, 3), (128, 0, 9480, 14, 2), (256, 0, 4737, 4, 2), (256, 1, 4800, 5, 3),
     # 16 and 32 envs per CTA, agent rows of W1 in shared memory and not
     (256, 0, 2368, 4, 2), (256, 0, 2369, 12, 2), (256, 1, 2500, 13, 2), (256, 0, 19, 13, 3), (256, 1, 33, 14, 3),
     (192, 0, 17, 16, 3), (192, 0, 2369, 3, 2), (128, 1, 2368, 16, 2), (128, 0, 2400, 5, 2), (96, 0, 2368, 5, 2), (96, 0, 2380, 5, 3), (96, 0, 4737, 3, 2),
