@@ -112,6 +112,11 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (tid == 0) {
+        tc::prefetch_map(last ? &maps.ld_hi : &maps.d_hi);
+        tc::prefetch_map(last ? &maps.lh_hi : &maps.h_hi);
+        if (PL == 2) { tc::prefetch_map(last ? &maps.ld_lo : &maps.d_lo); tc::prefetch_map(last ? &maps.lh_lo : &maps.h_lo); }
+    }
     pdl_wait();  // (the set-up above runs under the predecessor's tail)
     int G = 0;  // tiles of this CTA
     for (int u = xi; u < units; u += nx) G += (t_end(u) - t_begin(u) + SP - 1) / SP;
@@ -228,10 +233,19 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
         // ---- epilogue: thread = row r (accumulator lane) x 32 of the 64 units
         const int q = wid & 3, r = 32 * q + lane, half = (wid - Cfg::FIRST_EPI) >> 2, etid = tid - 32 * Cfg::FIRST_EPI;
         const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-        for (int i = etid; i < PL * H * 8; i += 256) {  // W2 rows, 16-byte pieces permuted by row % 8
-            const int pl = i / (H * 8), row = (i / 8) % H, c = i & 7;
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>((pl ? b.w2p_lo : b.w2p_hi) + row * H) + c);
-            *reinterpret_cast<uint4*>(sW + pl * Cfg::W_BOX + row * 128 + ((c ^ (row & 7)) << 4)) = v;
+        {   // W2 rows, 16-byte pieces permuted by row % 8
+            constexpr int TRIPS = PL * H * 8 / 256;
+            uint4 v[TRIPS];
+#pragma unroll
+            for (int k = 0; k < TRIPS; ++k) {
+                const int i = etid + 256 * k;
+                v[k] = __ldg(reinterpret_cast<const uint4*>((i / (H * 8) ? b.w2p_lo : b.w2p_hi) + ((i / 8) % H) * H) + (i & 7));
+            }
+#pragma unroll
+            for (int k = 0; k < TRIPS; ++k) {
+                const int i = etid + 256 * k, row = (i / 8) % H;
+                *reinterpret_cast<uint4*>(sW + (i / (H * 8)) * Cfg::W_BOX + row * 128 + (((i & 7) ^ (row & 7)) << 4)) = v[k];
+            }
         }
         tc::fence_proxy_async();
         __syncwarp();

@@ -392,15 +392,19 @@ bool three_terms(int H, int prec);             // fp32 operands as three bf16 te
 bool rollout_uses_fragments(int H, int prec);  // the warp-level kernel (and with it the fragment copies of W2) serves this shape
 cudaError_t launch_rollout_tc128(const RolloutArgs& a, int prec, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, large batches); cudaErrorNotSupported otherwise
 cudaError_t launch_rollout_pair2(const RolloutArgs& a, int prec, cudaStream_t s);  // two env groups per CTA pair (H = 256, large batches); cudaErrorNotSupported otherwise
-// Slices of a replay (grid.y) for kernels of one CTA per SM: its steps are independent, so few CTAs take fewer steps each; at least
-// two steps (the weights' load is paid per slice), none empty.
+// Slices of a replay (grid.y) for kernels of one CTA per SM: its steps are independent, so few CTAs take fewer steps each, at least
+// two.  The number that takes the fewest steps over all waves, with one more per slice for the weights' load; none empty.
 inline int replay_slices(const RolloutArgs& a, int ctas) {
     if (!a.replay) return 1;
     const int steps = a.T + (a.replay == 2 ? 1 : 0);
-    int n = 148 / ctas;
-    if (n > steps / 2) n = steps / 2;
-    if (n < 1) n = 1;
-    const int len = (steps + n - 1) / n;
+    long long best = 1ll << 60;
+    int len = steps;
+    for (int n = 1; n <= 16 || n <= 148 / ctas; ++n) {
+        const int l = (steps + n - 1) / n;
+        if (l < 2 && n > 1) break;
+        const long long t = (long long)(((long long)n * ctas + 147) / 148) * (l + 1);
+        if (t < best) { best = t; len = l; }
+    }
     return (steps + len - 1) / len;
 }
 cudaError_t launch_rollout_pair(const RolloutArgs& a, int prec, cudaStream_t s);  // CTA-pair tcgen05 rollout (H = 256); cudaErrorNotSupported otherwise

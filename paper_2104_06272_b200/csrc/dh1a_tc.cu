@@ -149,6 +149,12 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     tc::tc_fence_after();
     if (PAIR) tc::cluster_sync_all();  // both CTAs' barriers exist before either signals the other
     const uint32_t tmem = *tmem_slot;
+    if (tid == 0) {
+        tc::prefetch_map(&maps.w_hi);
+        tc::prefetch_map(&maps.a_hi);
+        if (PL == 2) { tc::prefetch_map(&maps.w_lo); tc::prefetch_map(&maps.a_lo); }
+    }
+    if (tid == 64) tc::prefetch_map(&maps.gate);
     pdl_wait();  // (the set-up above runs under the predecessor's tail)
     const uint32_t acc_agent = tmem + (uint32_t)Cfg::AGENT_COL;
     int my_tiles = 0;  // env tiles this CTA walks

@@ -170,6 +170,11 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (tid == 0) {
+        tc::prefetch_map(&maps.b_hi);
+        if (BPL >= 2) tc::prefetch_map(&maps.b_lo);
+        if (AMODE == A_PLANES) tc::prefetch_map(&maps.a_hi);
+    }
     pdl_wait();  // (the set-up above runs under the predecessor's tail)
     bool ok = true;
 

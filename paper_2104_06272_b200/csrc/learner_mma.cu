@@ -107,6 +107,10 @@ __global__ void __launch_bounds__((HeadsCfg<H, NW, PREC, HS, H2BF, FUSE>::THREAD
     if (FUSE) tc::tc_fence_before();
     __syncthreads();
     if (FUSE) tc::tc_fence_after();
+    if (FUSE && tid == NTHREADS + 32) {
+        tc::prefetch_map(&maps.h1_hi);
+        if (PREC == 0) tc::prefetch_map(&maps.h1_lo);
+    }
     pdl_wait();  // (the set-up above runs under the predecessor's tail)
     // The fused kernel takes its SMs whole.  The other one triggers after its tiles: with CTAs of the next kernel placed beside
     // it from the start it ran a third slower (B200, H = 64, 2.0 M rows: 215 -> 283 us; H = 32: 54 -> 84 us).

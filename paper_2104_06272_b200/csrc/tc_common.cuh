@@ -38,6 +38,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     return false;
 }
 
+// Fetches a tensor map (a kernel parameter) ahead of its first use.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
+
 // 2-D tiled TMA load into shared memory, completion counted in bytes on an mbarrier.  x = innermost coordinate
 // (elements; x * element size must be a multiple of 16 bytes), y = row.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
