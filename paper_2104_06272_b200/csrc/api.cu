@@ -116,8 +116,8 @@ size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* o
     b.dh2 = (float*)take(R * H * (x3 ? 6 : wide ? 2 : 4));
     const bool dh1_on_chip = H == 64 || (dh1_agent_tc_supported(d) && policies_of(c) <= 1);
     b.dh1 = dh1_on_chip ? nullptr : (float*)take(!wide ? R * H * 4 : std::max(R * H * (f32 ? 4 : 2), wide_scratch_bytes(d)));
-    // up to four t-slices of two 16-bit planes, or three planes (width 64: more slices while they keep to one 128-env tile per SM)
-    b.S = (float*)take(std::max(4 * B, H == 64 ? std::min((size_t)BACK64_SLICES * B, (size_t)148 * 128) : 0) * H * 4);
+    // t-slices of two 16-bit planes, or three planes
+    b.S = (float*)take((dh1_on_chip ? (size_t)most_s_rows((int)B) : 4 * B) * H * 4);
     LearnPlan pl;
     learn_mma_plan(d, &pl);
     b.part = (float*)take(pl.part_floats * 4);

@@ -455,26 +455,15 @@ cudaError_t launch_t(const LearnArgs& a, int nx, float* part_w2, float* part_age
 
 }  // namespace
 
-// CTAs per policy and slices of the steps.  The CTAs of all policies fill the GPU once where there are fewer than 148 policies;
-// the slices (at most BACK64_SLICES while S keeps to one 128-env tile per CTA, else at most 4, and one per CTA where a tile holds several
-// steps) are the number that leaves the fewest tiles on the busiest CTA, the smallest within one part in sixteen: a slice costs
-// a row of S per env.
+// CTAs per policy (all policies together fill the GPU once where there are fewer than 148) and slices of the steps; one slice per
+// CTA where a tile holds several steps.
 void back64_shape(const Dims& d, int T, int* nx, int* ts) {
     const int cap = 148 / d.npol > 0 ? 148 / d.npol : 1;
     const int sp = d.B <= 64 ? (128 / d.B < T ? 128 / d.B : T) : 1, m_tiles = sp > 1 ? 1 : (d.B + 127) / 128, steps = (T + sp - 1) / sp;
-    auto busiest = [&](int n) {
-        const int units = m_tiles * n, ctas = units < cap ? units : cap;
-        return (long long)((units + ctas - 1) / ctas) * ((steps + n - 1) / n);
-    };
-    int most = m_tiles * 4 > cap ? 4 : (cap / m_tiles < BACK64_SLICES ? cap / m_tiles : BACK64_SLICES);
+    int most = most_slices(m_tiles, cap);
     if (sp > 1 && most > cap) most = cap;
-    if (most > steps) most = steps;
-    long long best = busiest(1);
-    for (int n = 2; n <= most; ++n) best = busiest(n) < best ? busiest(n) : best;
-    int n = 1;
-    while (n < most && busiest(n) * 16 > best * 17) ++n;
-    *ts = n;
-    const int units = m_tiles * n;
+    *ts = slices_for(m_tiles, cap, steps, most);
+    const int units = m_tiles * *ts;
     *nx = units < cap ? units : cap;
 }
 

@@ -428,8 +428,25 @@ constexpr int DH1A_UNITS = 128;  // hidden units (columns of dh1) one CTA of the
 bool dh1_agent_tc_supported(const Dims& d);
 // dh1, S and the agent plane of dW1 in one tcgen05 kernel; cudaErrorNotSupported if not covered
 cudaError_t launch_dh1_agent_tc(const LearnArgs& a, int prec, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s);
+// Slices of the steps for a kernel whose units of work are (env tile, slice), `cap` CTAs (or pairs) walking them: the number that
+// leaves the fewest tiles on the busiest CTA, the smallest within one part in sixteen (a slice costs a row of S per env).
+constexpr int MAX_SLICES = 16;
+inline int slices_for(int m_tiles, int cap, int steps, int most) {
+    auto busiest = [&](int n) {
+        const int units = m_tiles * n, ctas = units < cap ? units : cap;
+        return (long long)((units + ctas - 1) / ctas) * ((steps + n - 1) / n);
+    };
+    if (most > steps) most = steps;
+    long long best = busiest(1);
+    for (int n = 2; n <= most; ++n) best = busiest(n) < best ? busiest(n) : best;
+    int n = 1;
+    while (n < most && busiest(n) * 16 > best * 17) ++n;
+    return n;
+}
+// ... at most four, or, while S keeps to one 128-env tile per CTA, MAX_SLICES.
+inline int most_slices(int m_tiles, int cap) { return m_tiles * 4 > cap ? 4 : (cap / m_tiles < MAX_SLICES ? cap / m_tiles : MAX_SLICES); }
+inline int most_s_rows(int B) { return 4 * B > 148 * 128 ? 4 * B : (MAX_SLICES * B < 148 * 128 ? MAX_SLICES * B : 148 * 128); }
 void back64_shape(const Dims& d, int T, int* nx, int* ts);  // hidden width 64: dh1, S, dW2 and the agent plane in one kernel
-constexpr int BACK64_SLICES = 16;
 cudaError_t launch_back64(const LearnArgs& a, int prec, int nx, float* part_w2, float* part_agent, size_t stride_agent, cudaStream_t s);
 cudaError_t launch_selftest_wait(int* status, long long limit_clocks, long long* waited_clocks, cudaStream_t s);
 cudaError_t launch_refresh_compute_params(const Dims& d, const Buffers& b, int prec, const Ctx& c);

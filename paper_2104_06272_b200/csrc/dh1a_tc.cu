@@ -7,8 +7,8 @@
 // The product is taken transposed, dh1^T[unit][env] = W2[unit][:] . dh2[env][:], so that the RESIDENT operand (the
 // CTA's 128 rows of W2, both 16-bit planes) is the A operand and lives in TENSOR memory for the whole kernel: an MMA
 // then fetches only the streamed dh2 box from shared memory, which is what bounds a one-CTA MMA on this part.  A CTA
-// owns 128 hidden units (accumulator lanes) and walks tiles of 128 envs (tile index blockIdx.x, blockIdx.x + gridDim.x,
-// ...) and, per tile, the steps t of its slice:
+// owns 128 hidden units (accumulator lanes) and walks units of (128 envs, slice of the steps), unit blockIdx.x,
+// blockIdx.x + gridDim.x, ..., step by step:
 //   warp 0 (one lane)  TMA producer: the dh2 planes of every step through a ring of 128 x 64 K-major boxes
 //   warp 1 (one lane)  tcgen05.mma issuer.  Per step: the dh1 product (K = H; three fp16 terms per k16, one in the bf16
 //                      workload, all into one of two 128-column accumulators); then, for the step before, the agent-plane
@@ -20,7 +20,7 @@
 //   warps 3-10         epilogue, thread = (unit, half of the envs): tcgen05.ld, gate, S +=, 16-bit split; writes its
 //                      dh1^T row (hi and lo planes, K-major) and the one-hot elements in the 128-byte-swizzled layout
 // At the end the epilogue warps store S (two 16-bit planes) and the agent accumulator as one split-K partial per
-// (env tile, t slice).  Tensor memory: [W2 planes | two dh1 accumulators | agent accumulator]; at H = 256 only the hi plane
+// CTA.  Tensor memory: [W2 planes | two dh1 accumulators | agent accumulator]; at H = 256 only the hi plane
 // of W2 fits (128 + 256 + 128 = 512 columns) and the lo plane is an ordinary shared-memory operand.
 //
 // H = 256 runs as a CTA PAIR (a cluster of two, tcgen05 cta_group::2): the pair owns all 256 units of an env tile, each
@@ -88,7 +88,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     constexpr int BM = Cfg::BM, BN = Cfg::BN, KC = Cfg::KC, PL = Cfg::PL, NCH = Cfg::NCH, STAGES = Cfg::STAGES;
     constexpr bool PAIR = Cfg::PAIR;
     constexpr int NCTA = Cfg::NCTA;
-    constexpr int PREFETCH = 3 * NCH;  // chunks between the L2 prefetch of a box and its load (three steps)
+    constexpr int PREFETCH = 3;  // steps between the L2 prefetch of a box and its load
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sW = base;                                   // W2 lo plane, one box per k chunk (H = 256 only)
@@ -108,6 +108,9 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     uint64_t* gempty = gfull + 1;           // gate tile read (the epilogue warps arrive)
     uint64_t* wstage = gempty + 1;          // the W2 rows bound for tensor memory have landed in their staging boxes
     uint32_t* tmem_slot = (uint32_t*)(wstage + 1);
+    // units of work u = tile + tiles * slice, this CTA's are xi, xi + nx, ...; in shared memory, read where needed: the epilogue's
+    // sums leave no registers for them
+    volatile int* shape = (volatile int*)(tmem_slot + 1);  // [4] tiles, steps of a slice, units, this CTA's steps (all units together)
 
     const Dims& d = a.d;
     const Buffers& b = a.b;
@@ -117,12 +120,17 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     const bool leader = rank == 0;
     const int xi = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, nx = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;  // tile walker
     const int n0 = PAIR ? (int)rank * BN : (int)blockIdx.y * BN;
-    const int m_tiles = (B + BM - 1) / BM;
     int* status = b.status;
-    const int tl = (T + a.ts - 1) / a.ts;  // this CTA's slice of the steps
-    const int t0 = blockIdx.z * tl, t1 = min(T, t0 + tl);
-    const int nsteps = t1 > t0 ? t1 - t0 : 0;
 
+    if (tid == 32) {
+        const int m_tiles = (B + BM - 1) / BM, tl = (T + a.ts - 1) / a.ts, units = m_tiles * a.ts;
+        int steps = 0;
+        for (int u = xi; u < units; u += nx) steps += min((u / m_tiles) * tl + tl, T) - min((u / m_tiles) * tl, T);
+        shape[0] = m_tiles;
+        shape[1] = tl;
+        shape[2] = units;
+        shape[3] = steps;
+    }
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(&full[s], 1); tc::mbar_init(&empty[s], 1); }
         for (int i = 0; i < 2; ++i) {
@@ -157,12 +165,24 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
     if (tid == 64) tc::prefetch_map(&maps.gate);
     pdl_wait();  // (the set-up above runs under the predecessor's tail)
     const uint32_t acc_agent = tmem + (uint32_t)Cfg::AGENT_COL;
-    int my_tiles = 0;  // env tiles this CTA walks
-    for (int mt = xi; mt < m_tiles; mt += nx) ++my_tiles;
-    const int G = my_tiles * nsteps;  // steps of this CTA, all env tiles together (the pipelines run across tiles)
+    const int G = shape[3];  // (the pipelines run across the units)
     bool ok = true;
-    // first row (t*B + env) of running step g
-    auto row_of = [&](int g) { return (t0 + g % nsteps) * B + (xi + (g / nsteps) * nx) * BM; };
+    // walks the running steps; row_of = first row (t*B + env) of the one it stands at (past the last one it stays in its unit)
+    struct Walk {
+        int u, t, end, env0;
+    };
+    auto enter = [&](Walk& w) {
+        const int m_tiles = shape[0], tl = shape[1], slice = w.u / m_tiles;
+        w.t = min(slice * tl, T);
+        w.end = min(slice * tl + tl, T);
+        w.env0 = (w.u - slice * m_tiles) * BM;
+    };
+    auto settle = [&](Walk& w) {
+        while (w.t >= w.end && w.u + nx < shape[2]) { w.u += nx; enter(w); }
+    };
+    auto walk = [&]() { Walk w; w.u = xi; enter(w); settle(w); return w; };
+    auto advance = [&](Walk& w) { ++w.t; settle(w); };
+    auto row_of = [&](const Walk& w) { return w.t * B + w.env0; };
     // arrival on / wait for a barrier of the leader CTA (pair: the peer's arrivals cross the cluster)
     // (release at CTA scope: what these arrivals publish is this warp's finished tensor-memory accesses and its stores to
     // its own CTA's shared memory; a cluster-scope release costs well over a thousand clocks per arrival)
@@ -194,22 +214,22 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                     else tc::tma_load_2d(sW + kc * Cfg::W_BOX, &maps.w_lo, wfull, kc * KC, n0);
                 }
             }
+            Walk now = walk(), ahead = now;
+            for (int i = 0; i < PREFETCH; ++i) advance(ahead);
             for (int c = 0; c < G * NCH && ok; ++c) {
-                const int s = c % STAGES, g = c / NCH, kc = c - g * NCH;
-                {   // pull the boxes of a later chunk towards L2 now, so that their TMA load is an L2 hit
-                    const int cp = c + PREFETCH;
-                    if (cp < G * NCH) {
-                        const int gp = cp / NCH, kp = cp - gp * NCH;
-                        tc::tma_prefetch_2d(&maps.a_hi, kp * KC, row_of(gp) + Cfg::ROWS * (int)rank);
-                        if (PL == 2) tc::tma_prefetch_2d(&maps.a_lo, kp * KC, row_of(gp) + Cfg::ROWS * (int)rank);
-                    }
+                const int s = c % STAGES, kc = c % NCH;
+                if (kc == 0 && c > 0) { advance(now); advance(ahead); }
+                if (c + PREFETCH * NCH < G * NCH) {  // pull the boxes of a later step towards L2 now, so that their TMA load is an L2 hit
+                    const int row = row_of(ahead) + Cfg::ROWS * (int)rank;
+                    tc::tma_prefetch_2d(&maps.a_hi, kc * KC, row);
+                    if (PL == 2) tc::tma_prefetch_2d(&maps.a_lo, kc * KC, row);
                 }
                 if (c >= STAGES) ok = tc::mbar_wait(&empty[s], ((c / STAGES) - 1) & 1);
                 if (!ok) break;
                 if (leader) tc::mbar_expect_tx(&full[s], NCTA * Cfg::A_STAGE);  // the loads of both CTAs
                 // rows t*B + e0 .. +127 of the dh2 planes (rows past the batch end belong to the next step or are
                 // zero-filled past the last row; their results are discarded by the epilogue)
-                const int row = row_of(g) + Cfg::ROWS * (int)rank;
+                const int row = row_of(now) + Cfg::ROWS * (int)rank;
                 if (PAIR) {
                     const uint32_t bar = tc::mapa(tc::smem_u32(&full[s]), 0);
                     tc::tma_load_2d_pair(sA + s * Cfg::A_STAGE, &maps.a_hi, bar, kc * KC, row);
@@ -301,12 +321,15 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
         }
     } else if (wid == 2) {
         if (lane == 0) {  // ---- TMA producer of the gate tiles (rows as for dh2, units n0 .. n0+127 of the h1 hi plane)
-            for (int g = 0; g < G && ok; ++g) {
-                if (g + 2 < G) tc::tma_prefetch_2d(&maps.gate, n0 / 8, row_of(g + 2));
+            Walk now = walk(), ahead = now;
+            advance(ahead);
+            advance(ahead);
+            for (int g = 0; g < G && ok; ++g, advance(now), advance(ahead)) {
+                if (g + 2 < G) tc::tma_prefetch_2d(&maps.gate, n0 / 8, row_of(ahead));
                 if (g >= 1) ok = tc::mbar_wait(gempty, (uint32_t)(g - 1) & 1u);
                 if (!ok) break;
                 tc::mbar_expect_tx(gfull, Cfg::G_TILE);
-                tc::tma_load_2d(sG, &maps.gate, gfull, n0 / 8, row_of(g));  // (x in bytes: 0 or 16)
+                tc::tma_load_2d(sG, &maps.gate, gfull, n0 / 8, row_of(now));  // (x in bytes: 0 or 16)
             }
             if (!ok) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         }
@@ -360,14 +383,15 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
         unsigned char* drow = sD + half * Cfg::D_BOX + j * 128;  // this thread's row of the dh1^T hi box of its env half
         int prev_off = -1;  // byte offset of the one-hot element this thread set the step before
         int g = 0;          // running step index of this CTA
-        for (int mt = xi; mt < m_tiles && ok; mt += nx) {
+        for (int u = xi; u < shape[2] && ok; u += nx) {
+            const int slice = u / shape[0], mt = u - slice * shape[0], t1 = min(slice * shape[1] + shape[1], T);
             const int env0 = mt * BM + 64 * half;              // first env of this thread's half
             const int nvalid = min(64, max(0, B - env0));      // envs of the half that exist
             const int oh_env = mt * BM + j;                    // (half 0 only) the env whose one-hot row this thread keeps
             float s_acc[64];
 #pragma unroll
             for (int i = 0; i < 64; ++i) s_acc[i] = 0.f;
-            for (int t = t0; t < t1; ++t, ++g) {
+            for (int t = min(slice * shape[1], T); t < t1; ++t, ++g) {
                 const int cell = (half == 0 && oh_env < B) ? (int)b.tpos[(size_t)t * B + oh_env] : -1;
                 const int buf = g % ACCS;
                 if (ok) ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g / ACCS) & 1u);
@@ -428,7 +452,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             if (ok) {
                 uint16_t* S_hi = reinterpret_cast<uint16_t*>(b.S);
                 uint16_t* S_lo = S_hi + (size_t)a.ts * B * H;
-                const size_t si = ((size_t)blockIdx.z * B + env0) * H + n0 + j;  // an empty slice writes zeros
+                const size_t si = ((size_t)(u / shape[0]) * B + env0) * H + n0 + j;  // an empty slice writes zeros
 #pragma unroll
                 for (int i = 0; i < 64; ++i) {
                     if (i < nvalid) {
@@ -448,13 +472,13 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             }
         }
         if (!ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
-        // agent-plane partial of this (env tile, t slice): accumulator lane = unit, column = cell
+        // agent-plane partial of this CTA: accumulator lane = unit, column = cell
         bool got = ok;
         if (got && G > 0) got = tc::mbar_wait(tiles_free, (uint32_t)(G - 1) & 1u);
         if (!got && ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         tc::tc_fence_after();
         __syncwarp();
-        float* part = part_agent + (size_t)(blockIdx.z * nx + xi) * part_stride + n0 + j;
+        float* part = part_agent + (size_t)xi * part_stride + n0 + j;
 #pragma unroll
         for (int c0 = 0; c0 < 64 * NC; c0 += 32) {
             uint32_t r[32];
@@ -508,9 +532,9 @@ cudaError_t launch_t(const LearnArgs& a, int grid_x, float* part_agent, size_t p
     if (!make_tensor_map_2d(&maps.w_hi, b.w2p_hi, H, H, 128, bf)) return cudaErrorNotSupported;
     if (Cfg::PL == 2 && !make_tensor_map_2d(&maps.w_lo, b.w2p_lo, H, H, 128, bf)) return cudaErrorNotSupported;
     if constexpr (Cfg::PAIR) {  // the two CTAs of a pair are neighbours in x; each pair takes all H units
-        launch<k_dh1a_pair<H, PREC, NC>>(dim3(2 * grid_x, 1, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
+        launch<k_dh1a_pair<H, PREC, NC>>(dim3(2 * grid_x), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
     } else {
-        launch<k_dh1a_tc<H, PREC, NC>>(dim3(grid_x, H / Cfg::BN, a.ts), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
+        launch<k_dh1a_tc<H, PREC, NC>>(dim3(grid_x, H / Cfg::BN), Cfg::THREADS, Cfg::smem_bytes, s, maps, a, part_agent, part_stride);
     }
     return cudaGetLastError();
 }
@@ -525,8 +549,8 @@ cudaError_t launch_nc(const LearnArgs& a, int prec, int grid_x, float* part_agen
 
 bool dh1_agent_tc_supported(const Dims& d) { return d.H == 128 || d.H == 256; }
 
-// grid_x CTAs share the 128-env tiles (grid_x <= ceil(B/128)); a.ts slices the steps.  The agent-plane partials go to
-// part_agent[split * part_stride + cell * H + col] with split = t slice * grid_x + blockIdx.x: grid_x * a.ts splits.
+// grid_x CTAs (pairs) share the (128-env tile, slice) units, a.ts slices of the steps.  The agent-plane partials go to
+// part_agent[split * part_stride + cell * H + col], one split per CTA (pair).
 // cudaErrorNotSupported when the shape is not covered.
 cudaError_t launch_dh1_agent_tc(const LearnArgs& a, int prec, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s) {
     if (!dh1_agent_tc_supported(a.d) || !a.b.w2p_hi || (prec != 1 && !a.b.w2p_lo)) return cudaErrorNotSupported;

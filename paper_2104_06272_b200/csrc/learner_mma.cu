@@ -1333,20 +1333,19 @@ static int splits_for(int K, int tiles, int min_k) {
     return ns < 1 ? 1 : ns;
 }
 
-// Launch shape of the fused dh1 + agent-plane kernel: one CTA per SM.  Few env tiles: slice the steps; many: let a CTA
-// walk several tiles, so that the number of agent-plane partials stays at most one per CTA row.
-static void dh1a_shape(const Dims& d, int T, int* grid_x, int* ts) {
-    const int m_tiles = (d.B + 127) / 128, n_tiles = d.H / DH1A_UNITS;
-    *grid_x = m_tiles;
-    *ts = 1;
-    if (m_tiles * n_tiles >= 148) {
-        *grid_x = 148 / n_tiles > 0 ? 148 / n_tiles : 1;
-    } else {
-        int t = 148 / (m_tiles * n_tiles);
-        if (t > 4) t = 4;
-        if (t > T) t = T;
-        if (t >= 2) *ts = t;
-    }
+// Launch shape of the fused dh1 + agent-plane kernel: nx CTAs (H = 256: pairs), one per SM, walk the units (128-env tile, slice of
+// the steps); one agent-plane partial each.  (Four slices at most and one unit per CTA: 2500 envs, H = 128, T = 24 21.3 -> 18.8 us,
+// 6000 envs, H = 256, T = 20 58 -> 44 us.)
+static void dh1a_shape(const Dims& d, int T, int* nx, int* ts) {
+    const int m_tiles = (d.B + 127) / 128, cap = 148 / (d.H / DH1A_UNITS);
+    *ts = slices_for(m_tiles, cap, T, most_slices(m_tiles, cap));
+    *nx = std::min(m_tiles * *ts, cap);
+}
+
+// Splits of the wall and goal planes' K range (rows of S).
+static int env_splits(const Dims& d, int rows) {
+    const int bt = d.H == 128 || d.H >= 256 ? 128 : 64;
+    return splits_for(rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
 }
 
 // dW2 inside the heads kernel: hidden width 128 or 256, one policy.
@@ -1387,16 +1386,16 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
     }
-    if (dh1_agent_tc_supported(d)) {  // the fused kernel writes one agent-plane partial per (CTA row, t slice)
-        int gx, ts;
-        dh1a_shape(d, d.Tmax, &gx, &ts);
-        if (gx * ts > p->ns_agent) p->ns_agent = gx * ts;
-    }
     p->ns_env = splits_for(d.B, tiles_ch, 128);
+    if (dh1_agent_tc_supported(d) && d.npol <= 1) {  // (one agent-plane partial per CTA of the fused kernel, any T <= Tmax)
+        const int cap = 148 / (H / DH1A_UNITS);
+        p->ns_agent = std::max(p->ns_agent, std::min(cap, (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax)));
+        p->ns_env = env_splits(d, most_s_rows(d.B));
+    }
     if (H == 64) {  // (one partial per CTA of the fused kernel; its slices of the steps are rows of S)
-        const int units = d.B > 64 ? (d.B + 127) / 128 * std::min(BACK64_SLICES, d.Tmax) : (d.Tmax + 128 / d.B - 1) / (128 / d.B);  // (of any T <= Tmax)
+        const int units = d.B > 64 ? (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax) : (d.Tmax + 128 / d.B - 1) / (128 / d.B);  // (of any T <= Tmax)
         p->ns_w2 = p->ns_agent = std::min(std::max(148 / d.npol, 1), units);
-        p->ns_env = splits_for(std::max(4 * d.B, std::min(BACK64_SLICES * d.B, 148 * 128)), tiles_ch, 256);
+        p->ns_env = env_splits(d, most_s_rows(d.B));
     }
     const size_t tiles32 = (R + 31) / 32;
     size_t hg = (size_t)heads_grid_max(H);
@@ -1525,18 +1524,18 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         int nx;
         back64_shape(d, T, &nx, &a.ts);
         a.reg[1].ns = a.reg[4].ns = nx;
-        const int tiles = (C + 1 + 63) / 64;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = splits_for(a.ts * B, tiles, 256);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
         Scope sc(c, K_DH1);
         CK(launch_back64(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
     } else if (!wide && !grouped && dh1_agent_tc_supported(d)) {
-        int gx;
-        dh1a_shape(d, T, &gx, &a.ts);
+        int nx;
+        dh1a_shape(d, T, &nx, &a.ts);
+        a.reg[1].ns = nx;
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
         Scope sc(c, K_DH1);
-        CK(launch_dh1_agent_tc(a, PREC, gx, b.part + pl.off_agent, CH, s));
+        CK(launch_dh1_agent_tc(a, PREC, nx, b.part + pl.off_agent, CH, s));
         fused_agent = true;
-        a.reg[1].ns = gx * a.ts;
     } else if (PREC == 2 || wide) {
         CK(launch_dh1_wide(a, c));
         if (PREC == 2) {  // fp32 dh1 rows: the agent plane and S in one pass over them
