@@ -69,7 +69,7 @@ struct Dh1aCfg {
     static constexpr int W_BYTES = W_LO_SMEM ? NCH * W_BOX : 0;
     // the planes bound for tensor memory are staged by TMA in the (still unused) dh1^T tile where they fit
     static constexpr bool W_STAGED = WT_PL * NCH * W_BOX <= PL * 2 * BN * 128;
-    static constexpr int BARS = 256;
+    static constexpr int BARS = 320;
     static constexpr int MAX_SMEM = 232448 - 1024;       // 227 KB per CTA minus alignment slack
     static constexpr int RING = MAX_SMEM - BARS - W_BYTES - D_TILE - O_TILE - G_TILE;
     static constexpr int STAGES = RING / A_STAGE >= 6 ? 6 : RING / A_STAGE;
@@ -383,15 +383,19 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
         unsigned char* drow = sD + half * Cfg::D_BOX + j * 128;  // this thread's row of the dh1^T hi box of its env half
         int prev_off = -1;  // byte offset of the one-hot element this thread set the step before
         int g = 0;          // running step index of this CTA
-        for (int u = xi; u < shape[2] && ok; u += nx) {
-            const int slice = u / shape[0], mt = u - slice * shape[0], t1 = min(slice * shape[1] + shape[1], T);
+        volatile int* own = shape + 4 + 3 * (wid - Cfg::FIRST_EPI);  // this warp's unit, the end of its steps, its row of S
+        own[0] = xi;
+        while (ok && own[0] < shape[2]) {
+            const int slice = own[0] / shape[0], mt = own[0] - slice * shape[0];
             const int env0 = mt * BM + 64 * half;              // first env of this thread's half
             const int nvalid = min(64, max(0, B - env0));      // envs of the half that exist
             const int oh_env = mt * BM + j;                    // (half 0 only) the env whose one-hot row this thread keeps
             float s_acc[64];
 #pragma unroll
             for (int i = 0; i < 64; ++i) s_acc[i] = 0.f;
-            for (int t = min(slice * shape[1], T); t < t1; ++t, ++g) {
+            own[1] = min(slice * shape[1] + shape[1], T);
+            own[2] = slice * B + env0;
+            for (int t = min(slice * shape[1], T); t < own[1]; ++t, ++g) {
                 const int cell = (half == 0 && oh_env < B) ? (int)b.tpos[(size_t)t * B + oh_env] : -1;
                 const int buf = g % ACCS;
                 if (ok) ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g / ACCS) & 1u);
@@ -452,7 +456,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             if (ok) {
                 uint16_t* S_hi = reinterpret_cast<uint16_t*>(b.S);
                 uint16_t* S_lo = S_hi + (size_t)a.ts * B * H;
-                const size_t si = ((size_t)(u / shape[0]) * B + env0) * H + n0 + j;  // an empty slice writes zeros
+                const size_t si = (size_t)own[2] * H + n0 + j;  // an empty slice writes zeros
 #pragma unroll
                 for (int i = 0; i < 64; ++i) {
                     if (i < nvalid) {
@@ -470,6 +474,9 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                     }
                 }
             }
+            __syncwarp();
+            if (lane == 0) own[0] = own[0] + nx;
+            __syncwarp();
         }
         if (!ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
         // agent-plane partial of this CTA: accumulator lane = unit, column = cell
