@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_h1_wide(Dims d, Buffers b, const uint8_
 //   mode 2: replay of recorded rows (row = t*B + env): saves the head outputs only.
 //   mode 3: forward of the current env state under the current parameters: saves the value to vboot.
 template <int H, bool F32, int HW_ROWS>
-__global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mode, size_t rows, size_t row0) {
+__global__ void __launch_bounds__(256, HW_ROWS >= 16 && H >= 768 ? 4 : 5) k_heads_wide(RolloutArgs a, int t, int mode, size_t rows, size_t row0) {
     PDL_START();
     constexpr int TRIPS = H / 128;   // a lane covers four consecutive hidden units per trip
     extern __shared__ __align__(16) float s_wh[];  // [H][5] as stored
@@ -263,32 +263,33 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
         }
     }
     const uint16_t* h2b = reinterpret_cast<const uint16_t*>(b.h2);
-    // a warp walks rows wid, wid+8, ...; the loads of the next row are in flight while this row is reduced
+    // A warp walks rows wid, wid + 8, ...; WIN trips of h2 are in flight.  The widest layers take two rows at a time, so that a piece of
+    // Wh read from shared memory serves both (B200, H = 1024: 16384 rows in bf16 37.8 -> 32.2 us, 12000 in fp32 33.1 -> 28.8 us; below
+    // H = 768 the registers cost the fifth CTA per SM, 22.5 -> 23.7 us for 20000 rows of 512 in bf16).
+    constexpr int RB = HW_ROWS >= 16 && H >= 768 ? 2 : 1, WIN = RB == 2 && F32 ? (TRIPS % 2 == 0 ? 2 : 3) : TRIPS % 4 == 0 ? 4 : 3;
     using H2x4 = typename std::conditional<F32, float4, uint2>::type;  // four consecutive units of h2: fp32, or bf16
-    H2x4 v[TRIPS], vn[TRIPS];
-    auto load_row = [&](int r, H2x4 (&dst)[TRIPS]) {
-        const size_t i = i0 + r, off = (row0 + (i < rows ? i : 0)) * H;
-        const H2x4* hp = F32 ? reinterpret_cast<const H2x4*>(b.h2 + off) : reinterpret_cast<const H2x4*>(h2b + off);
+    static_assert(TRIPS % WIN == 0, "a trip keeps its slot from one pass to the next");
+    H2x4 v[WIN][RB];
+    auto load_trip = [&](int r, int q, H2x4 (&dst)[RB]) {
 #pragma unroll
-        for (int q = 0; q < TRIPS; ++q) dst[q] = (r < HW_ROWS && i < rows) ? __ldg(hp + lane + 32 * q) : H2x4{};
+        for (int k = 0; k < RB; ++k) {
+            const size_t i = i0 + r + 8 * k, off = (row0 + (i < rows ? i : 0)) * H;
+            const H2x4* hp = F32 ? reinterpret_cast<const H2x4*>(b.h2 + off) : reinterpret_cast<const H2x4*>(h2b + off);
+            dst[k] = i < rows ? __ldg(hp + lane + 32 * q) : H2x4{};
+        }
     };
-    load_row(wid, v);
+#pragma unroll
+    for (int q = 0; q < WIN; ++q) load_trip(wid, q, v[q]);
     __syncthreads();
 #pragma unroll 1
-    for (int r = wid; r < HW_ROWS; r += 8) {
-        load_row(r + 8, vn);
-        float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int r = wid; r < HW_ROWS; r += 8 * RB) {
+        float acc[RB][5];
+#pragma unroll
+        for (int k = 0; k < RB; ++k)
+#pragma unroll
+            for (int c = 0; c < 5; ++c) acc[k][c] = 0.f;
 #pragma unroll
         for (int q = 0; q < TRIPS; ++q) {
-            float x[4];
-            if constexpr (F32) {
-                x[0] = v[q].x; x[1] = v[q].y; x[2] = v[q].z; x[3] = v[q].w;
-            } else {
-                x[0] = __uint_as_float(v[q].x << 16);
-                x[1] = __uint_as_float(v[q].x & 0xFFFF0000u);
-                x[2] = __uint_as_float(v[q].y << 16);
-                x[3] = __uint_as_float(v[q].y & 0xFFFF0000u);
-            }
             // this lane's four units are 20 consecutive floats of Wh (80-byte lane stride: conflict-free 16-byte reads)
             const float4* wp = reinterpret_cast<const float4*>(s_wh + 20 * (lane + 32 * q));
             float w[20];
@@ -298,20 +299,39 @@ __global__ void __launch_bounds__(256) k_heads_wide(RolloutArgs a, int t, int mo
                 w[4 * j] = f.x; w[4 * j + 1] = f.y; w[4 * j + 2] = f.z; w[4 * j + 3] = f.w;
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int k = 0; k < RB; ++k) {
+                const H2x4 y = v[q % WIN][k];
+                float x[4];
+                if constexpr (F32) {
+                    x[0] = y.x; x[1] = y.y; x[2] = y.z; x[3] = y.w;
+                } else {
+                    x[0] = __uint_as_float(y.x << 16);
+                    x[1] = __uint_as_float(y.x & 0xFFFF0000u);
+                    x[2] = __uint_as_float(y.y << 16);
+                    x[3] = __uint_as_float(y.y & 0xFFFF0000u);
+                }
 #pragma unroll
-                for (int c = 0; c < 5; ++c) acc[c] = fmaf(x[u], w[5 * u + c], acc[c]);
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) acc[k][c] = fmaf(x[u], w[5 * u + c], acc[k][c]);
+            }
+            if (q + WIN < TRIPS) load_trip(r, q + WIN, v[q % WIN]);
+            else if (r + 8 * RB < HW_ROWS) load_trip(r + 8 * RB, (q + WIN) % TRIPS, v[q % WIN]);  // (the next rows' first trips)
         }
+        // sums over the lanes; two rows: the first round of the tree hands each half of the warp one of them
+        float o5[5];
+        const bool up = lane & 16;
 #pragma unroll
-        for (int c = 0; c < 5; ++c)
+        for (int c = 0; c < 5; ++c) {
+            if constexpr (RB == 2) o5[c] = (up ? acc[1][c] : acc[0][c]) + __shfl_xor_sync(0xFFFFFFFFu, up ? acc[0][c] : acc[1][c], 16);
+            else o5[c] = acc[0][c] + __shfl_xor_sync(0xFFFFFFFFu, acc[0][c], 16);
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) acc[c] += __shfl_xor_sync(0xFFFFFFFFu, acc[c], off);
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 5; ++c) s_out[r][c] = acc[c] + b.theta_c[d.obh + c];
+            for (int off = 8; off > 0; off >>= 1) o5[c] += __shfl_xor_sync(0xFFFFFFFFu, o5[c], off);
         }
+        if ((lane & 15) == 0 && (RB == 2 || lane == 0)) {
 #pragma unroll
-        for (int q = 0; q < TRIPS; ++q) v[q] = vn[q];
+            for (int c = 0; c < 5; ++c) s_out[r + (RB == 2 && up ? 8 : 0)][c] = o5[c] + b.theta_c[d.obh + c];
+        }
     }
     __syncthreads();
     __shared__ int s_pos[HW_ROWS];
