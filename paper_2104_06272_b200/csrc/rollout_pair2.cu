@@ -3,13 +3,12 @@
 //
 // Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top), fp32 workloads.  The layout of one
 // group is that of the one-group CTA-pair kernel: layer 2 transposed, D[j][env] = sum_k W2[k][j] h1[env][k], as
-// tcgen05.mma.cta_group::2 with M = 256 hidden units, each CTA keeping ITS 128 columns of W2 on chip (two fp16 planes,
-// 128 KB, loaded once by TMA) and building the h1 rows of ITS 32 envs of the group.  With many envs per SM the rollout is a
+// tcgen05.mma.cta_group::2 with M = 256 hidden units, each CTA keeping ITS 128 columns of W2 on chip (the fp16 hi
+// plane transposed in tensor memory as the A operand, the lo plane in shared memory) and building the h1 rows of ITS 32 envs of the group.  With many envs per SM the rollout is a
 // throughput problem, but one group walks a strictly serial chain per step (gather -> tensor cores -> heads -> sample);
 // so a CTA holds two groups, each with eight worker warps and an owner warp of its own, and one group's tensor-core and
 // sampling phases fall into the other's gather and heads phases.  Per group and step:
-//   layer 1   h1 = relu(base + W1[agent row])       gather-add (base read from L2: shared memory holds W2 and two
-//                                                   operand tiles); fp16 (hi, lo) terms straight into the swizzled
+//   layer 1   h1 = relu(base + W1[agent row])       gather-add (base in shared memory); fp16 (hi, lo) terms straight into the swizzled
 //                                                   K-major operand tile [32 hi rows | 32 lo rows] x 256 k
 //   layer 2   two MMAs per k16:  W2hi x [h1hi | h1lo]  (N = 128 over the pair)  and  W2lo x h1hi  (N = 64), fp32
 //             accumulators in tensor memory; one thread of the leader CTA's issuer warp drives both groups
@@ -18,6 +17,8 @@
 //             memory of the CTA that owns it, sent as asynchronous remote stores that count their bytes on its mbarrier
 //   env       (owner warps) one thread per env: softmax, Philox inverse-CDF sample, gridworld step, time-major records;
 //             the new position is published before the records are written
+// (B200, 65536 envs, T = 32: 1450 us with both planes of W2 in shared memory, base read from L2, a proxy fence per k block and
+// conflicting reads; 1120 us so.)
 // The phases meet through mbarriers only; the cluster barrier is used at start and exit.  Every wait is bounded; a timeout
 // raises DEV_E_WAIT_TIMEOUT and the threads keep walking through the barriers to the exit, where tensor memory is freed.
 #include <cstring>
@@ -34,27 +35,27 @@ struct Pair2Cfg {
     static constexpr int NOWN = NG * ME;                            // owner threads: one per env of this CTA
     static constexpr int THREADS = NWT + NOWN + 32;                 // + the issuer warp
     static constexpr int BOX = 64 * 64 * 2;                         // one 64 x 64 box of 16-bit elements
-    static constexpr int A_PLANE = (128 / 64) * (H / 64) * BOX;     // this CTA's 128 columns of W2, all k: 64 KB
+    static constexpr int A_PLANE = (128 / 64) * (H / 64) * BOX;     // this CTA's 128 columns of W2, all k: 64 KB (the lo plane)
     static constexpr int B_CHUNK = 64 * 128;                        // 64 operand rows (32 hi + 32 lo) x 64 k
     static constexpr int B_BYTES = (H / 64) * B_CHUNK;              // a group's operand tile: 32 KB
     static constexpr int ACC = 192;                                 // TMEM columns of a group
-    static constexpr int TMEM_COLS = 512;
+    static constexpr int W_COL = NG * ACC, TMEM_COLS = 512;         // W2 hi: 128 columns (lane = hidden unit, two k per column)
     static constexpr size_t fixed_bytes =
-        2 * (size_t)A_PLANE + (size_t)NG * B_BYTES                  // W2 planes, operand tiles
+        (size_t)A_PLANE + (size_t)NG * B_BYTES + (size_t)NG * ME * H * 4  // W2 lo, operand tiles, base
         + 256                                                       // barriers, tensor-memory slot
-        + (size_t)NG * 8 * ME * 5 * 4                               // head partials: 8 blocks of 32 hidden units per group
+        + (size_t)NG * 8 * ME * 6 * 4                               // head partials: 8 blocks of 32 hidden units per group
         + 8 * 4 + (size_t)NOWN * 8 * 4 + NOWN * 4;                  // bh, walls, pos
     static constexpr size_t gae_bytes(int T) { return (size_t)(T + 1) * NOWN * 4 + (size_t)T * NOWN; }
 };
 
 struct Pair2Maps {
-    CUtensorMap w_hi, w_lo;  // W2 row-major [k][j] as fp16 planes, boxes of 64 j x 64 k
+    CUtensorMap w_lo;  // W2 row-major [k][j], the fp16 lo plane, boxes of 64 j x 64 k
 };
 
-// Asynchronous store of one float into the shared memory of a CTA of the cluster; when it has landed it counts its
-// four bytes on the mbarrier (same CTA as the destination), so the reader needs no fence from the writer.
-__device__ __forceinline__ void st_async_f32_2(uint32_t cluster_addr, float v, uint32_t cluster_bar_addr) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(cluster_addr), "f"(v),
+// Asynchronous store of two floats into the shared memory of a CTA of the cluster; when it has landed it counts its
+// eight bytes on the mbarrier (same CTA as the destination), so the reader needs no fence from the writer.
+__device__ __forceinline__ void st_async_f32x2(uint32_t cluster_addr, float v0, float v1, uint32_t cluster_bar_addr) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(cluster_addr), "f"(v0), "f"(v1),
                  "r"(cluster_bar_addr)
                  : "memory");
 }
@@ -66,17 +67,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     extern __shared__ unsigned char smem_raw[];
     // the dynamic shared memory starts at the same offset in both CTAs, so the rounded base does too
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* s_ahi = sm;
-    unsigned char* s_alo = s_ahi + Cfg::A_PLANE;
+    unsigned char* s_alo = sm;
     unsigned char* s_bop = s_alo + Cfg::A_PLANE;                                     // [NG] operand tiles
-    uint64_t* wbar = reinterpret_cast<uint64_t*>(s_bop + NG * Cfg::B_BYTES);         // weights landed
+    float* s_base = reinterpret_cast<float*>(s_bop + NG * Cfg::B_BYTES);             // [NG][ME][H]
+    uint64_t* wbar = reinterpret_cast<uint64_t*>(s_base + NG * ME * H);              // W2 lo landed
     uint64_t* tfull = wbar + 1;      // [NG] this step's MMAs of the group finished
-    uint64_t* ready = tfull + NG;    // [NG][4] leader's copy: k block of both CTAs' operand rows written (16 warps arrive)
-    uint64_t* pfull = ready + NG * 4;  // [NG] the eight head partials of this CTA's envs of the group have landed (bytes)
+    uint64_t* ready = tfull + NG;    // [NG][2] leader's copy: two k blocks of both CTAs' operand rows written (16 warps arrive)
+    uint64_t* pfull = ready + NG * 2;  // [NG] the eight head partials of this CTA's envs of the group have landed (bytes)
     uint64_t* posrdy = pfull + NG;     // [NG] this CTA's positions of the group for the next step are published
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(posrdy + NG);
-    float* s_red = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(wbar) + 256);  // [NG][8][ME][5]
-    float* s_bh = s_red + NG * 8 * ME * 5;                                           // [8]
+    float* s_red = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(wbar) + 256);  // [NG][8][ME][6]
+    float* s_bh = s_red + NG * 8 * ME * 6;                                           // [8]
     uint32_t* s_walls = reinterpret_cast<uint32_t*>(s_bh + 8);                       // [NOWN][8]
     int* s_pos = reinterpret_cast<int*>(s_walls + NOWN * 8);                         // [NOWN]
     float* s_gv = reinterpret_cast<float*>(s_pos + NOWN);                            // [T+1][NOWN] (a.gae_smem only)
@@ -100,7 +101,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
         tc::mbar_init(wbar, 1);
         for (int g = 0; g < NG; ++g) {
             tc::mbar_init(&tfull[g], 1);
-            for (int kb = 0; kb < 4; ++kb) tc::mbar_init(&ready[4 * g + kb], 2 * Cfg::NWORK);
+            for (int i = 0; i < 2; ++i) tc::mbar_init(&ready[2 * g + i], 2 * Cfg::NWORK);
             tc::mbar_init(&pfull[g], 1);
             tc::mbar_init(&posrdy[g], 1);
         }
@@ -115,15 +116,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     // Replay recomputes the T recorded rows (mode 2: and the current state), in independent slices of steps (grid.y).
     const int t_last = REPLAY && a.replay == 1 ? a.T - 1 : a.T, t_len = REPLAY ? (t_last + (int)gridDim.y) / (int)gridDim.y : 0;
     const int t_beg = REPLAY ? (int)blockIdx.y * t_len : 0, t_end = REPLAY ? min(t_last, t_beg + t_len - 1) : t_last;
-    if (issuer) {  // this CTA's 128 columns of W2: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
-        tc::mbar_expect_tx(wbar, (PREC == 0 ? 2 : 1) * Cfg::A_PLANE);
+    if (PREC == 0 && issuer) {  // this CTA's 128 columns of the lo plane: box (kb, bx) = k rows 64kb.., columns 128 rank + 64 bx..
+        tc::mbar_expect_tx(wbar, Cfg::A_PLANE);
 #pragma unroll
         for (int kb = 0; kb < H / 64; ++kb)
 #pragma unroll
-            for (int bx = 0; bx < 2; ++bx) {
-                tc::tma_load_2d(s_ahi + (kb * 2 + bx) * Cfg::BOX, &maps.w_hi, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
-                if (PREC == 0) tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
-            }
+            for (int bx = 0; bx < 2; ++bx) tc::tma_load_2d(s_alo + (kb * 2 + bx) * Cfg::BOX, &maps.w_lo, wbar, 128 * (int)rank + 64 * bx, 64 * kb);
     }
     // worker constants
     const int wg = worker ? wid / Cfg::NWORK : 0;   // the worker's group
@@ -143,6 +141,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     const int oenv = pair * (2 * NG * ME) + og * (2 * ME) + (int)rank * ME + oe;  // global env of an owner thread
     const bool owner = ownerw && oenv < B;
     if (worker) {
+        for (int i = tid; i < NG * ME * H / 4; i += NWT) {
+            const int e = i / (H / 4), k = 4 * (i - e * (H / 4));
+            const int env = pair * (2 * NG * ME) + (e / ME) * (2 * ME) + (int)rank * ME + e % ME;
+            cp_async16(s_base + e * H + k, b.base + (size_t)(env < B ? env : 0) * H + k, env < B ? 16 : 0);
+        }
+        cp_async_commit();
+        {   // W2 hi into tensor memory, transposed: lane = hidden unit j, 32-bit column = k 2c (low half), 2c + 1; the four warps of a
+            // lane quarter take 32 columns each
+            const int col0 = 32 * (wid >> 2);
+            const uint16_t* src = b.w2p_hi + (size_t)(2 * col0) * H + j;
+            uint32_t r[32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) r[c] = (uint32_t)__ldg(src + (size_t)(2 * c) * H) | ((uint32_t)__ldg(src + (size_t)(2 * c + 1) * H) << 16);
+            tc::tmem_st32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(Cfg::W_COL + col0), r);
+            tc::tmem_st_wait();
+            tc::tc_fence_before();
+        }
         b2j = b.theta_c[d.ob2 + j];
         {   // fragment element (k, n): lane = 4n + t holds k = 2t, 2t+1 (first register) and 2t+8, 2t+9 (second)
             const int n = lane >> 2, t4 = lane & 3;
@@ -157,6 +172,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
                 }
         }
         if (tid < 5) s_bh[tid] = b.theta_c[d.obh + tid];
+        cp_async_wait<0>();
     } else if (ownerw) {
         for (int wi = 0; wi < 8; ++wi) s_walls[ow * 8 + wi] = (owner && wi < d.W) ? b.walls[(size_t)oenv * d.W + wi] : 0u;
         if (owner) {
@@ -170,9 +186,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
         s_pos[ow] = s.pos;
     }
     bool ok = true;
-    if (issuer) ok = tc::mbar_wait(wbar, 0);  // the issuer's thread vouches for the weights of its CTA
+    if (PREC == 0 && issuer) ok = tc::mbar_wait(wbar, 0);  // the issuer's thread vouches for the weights of its CTA
     __syncthreads();
     tc::cluster_sync_all();  // both CTAs' barriers, tensor memory and weights exist before the first MMA
+    tc::tc_fence_after();
 
     __nv_bfloat16* g_h1hi = reinterpret_cast<__nv_bfloat16*>(b.h1);
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
@@ -182,31 +199,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
         // order the groups' operand blocks are written.  A block's sixteen arrivals also say that those warps have read
         // the group's accumulators of the step before.
         if (rank == 0) {
-            const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, true, false), idesc_n = tc::umma_idesc<PREC>(256, 64, true, false);
+            const uint32_t idesc_w = tc::umma_idesc<PREC>(256, 128, false, false), idesc_n = tc::umma_idesc<PREC>(256, 64, false, false);
+            const uint32_t idesc_lo = tc::umma_idesc<PREC>(256, 64, true, false);
             for (int t = t_beg; t <= t_end; ++t) {
                 for (int g = 0; g < NG; ++g) {
                     const uint32_t acc = tmem + (uint32_t)(g * Cfg::ACC);
                     unsigned char* bop = s_bop + g * Cfg::B_BYTES;
 #pragma unroll
-                    for (int kb = 0; kb < 4; ++kb) {
-                        ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[4 * g + kb], (uint32_t)(t - t_beg) & 1u));
+                    for (int i = 0; i < 2; ++i) {
+                        ok = tc::warp_all(ok && tc::mbar_wait_cluster(&ready[2 * g + i], (uint32_t)(t - t_beg) & 1u));
                         tc::tc_fence_after();
                         if (tc::elect_one()) {
 #pragma unroll
-                        for (int k16 = 0; k16 < 4; ++k16) {
-                            // A (MN-major): 16 k rows = 2048 bytes into each box, 8192 bytes between the two 64-column boxes
-                            const uint64_t ahi = tc::umma_desc(s_ahi + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
-                            const uint64_t alo = tc::umma_desc(s_alo + kb * 2 * Cfg::BOX + k16 * 2048, Cfg::BOX, 1024);
-                            // B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
-                            const uint64_t bd = tc::umma_desc(bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
-                            if (PREC == 0) {
-                                tc::umma_pair(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                                tc::umma_pair(acc + 128u, alo, bd, idesc_n, (kb | k16) ? 1u : 0u);
-                            } else {  // bf16 operands: one product, the hi rows of the operand tile only
-                                tc::umma_pair(acc, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            for (int k16 = 8 * i; k16 < 8 * i + 8; ++k16) {
+                                // A hi (tensor memory): 16 k = 8 columns.  A lo (MN-major): 16 k rows = 2048 bytes into each box, 8192
+                                // bytes between the two 64-column boxes.  B (K-major): 16 k = 32 bytes along the swizzled rows
+                                const uint32_t ahi = tmem + (uint32_t)(Cfg::W_COL + 8 * k16);
+                                const uint64_t bd = tc::umma_desc(bop + (k16 >> 2) * Cfg::B_CHUNK + (k16 & 3) * 32, 16, 1024);
+                                if (PREC == 0) {
+                                    tc::umma_pair_ta(acc, ahi, bd, idesc_w, k16 ? 1u : 0u);
+                                    tc::umma_pair(acc + 128u, tc::umma_desc(s_alo + (k16 >> 2) * 2 * Cfg::BOX + (k16 & 3) * 2048, Cfg::BOX, 1024), bd, idesc_lo, k16 ? 1u : 0u);
+                                } else {  // bf16 operands: one product, the hi rows of the operand tile only
+                                    tc::umma_pair_ta(acc, ahi, bd, idesc_n, k16 ? 1u : 0u);
+                                }
                             }
-                        }
-                        if (kb == 3) tc::umma_commit_pair(&tfull[g], 3);
+                            if (i == 1) tc::umma_commit_pair(&tfull[g], 3);
                         }
                         __syncwarp();
                     }
@@ -214,45 +231,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
             }
         }
     } else if (worker) {
-        // ---- layer 1 of group g for step t: 16-byte chunks of eight hidden units; all gathers are in flight before any is
+        // ---- layer 1 of group g for step t: 16-byte chunks of eight hidden units; two k blocks' gathers are in flight before any is
         // used.  Thread (e, c8) covers chunk c8 of the four k blocks of env e: the chunk goes to operand row e (hi) and
         // 32 + e (lo) of its block, at the 16-byte position c8 ^ (e % 8) of the 128-byte row (the 128-byte swizzle of a
-        // K-major operand).  Each finished block is announced to the leader's issuer at once.
+        // K-major operand).  Two finished blocks at a time are announced to the leader's issuer (one proxy fence).  Lanes 4-7 of an
+        // env read their two 16-byte pieces of a row in the other order, so that the eight lanes cover all banks.
         auto gather = [&](int g, int t) {
-            const int e = tidg >> 3, c8 = tidg & 7;
+            const int e = tidg >> 3, c8 = tidg & 7, sw = (c8 >> 2) & 1;
             const int env = pair * (2 * NG * ME) + g * (2 * ME) + (int)rank * ME + e;
             unsigned char* bop = s_bop + g * Cfg::B_BYTES;
             const float* wrow = W1 + (size_t)(C + s_pos[g * ME + e]) * H + 8 * c8;
-            const float* brow = b.base + (size_t)(env < B ? env : 0) * H + 8 * c8;
+            const float* brow = s_base + (g * ME + e) * H + 8 * c8;
             uint4 hi[4], lo[4];
+            float4 w[4][2];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {  // two k blocks at a time (registers)
-                float4 w[2][2], bs[2][2];
+            for (int kb = 0; kb < 4; ++kb)
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    const int kb = 2 * half + kk;
-                    const float4* wp = reinterpret_cast<const float4*>(wrow + 64 * kb);
-                    const float4* bp = reinterpret_cast<const float4*>(brow + 64 * kb);
-                    w[kk][0] = __ldg(wp);
-                    w[kk][1] = __ldg(wp + 1);
-                    bs[kk][0] = __ldg(bp);
-                    bs[kk][1] = __ldg(bp + 1);
-                }
-                if (half == 0) tc::tc_fence_before();  // this thread's reads of the group's accumulators precede the arrivals below
+                for (int x = 0; x < 2; ++x) w[kb][x] = __ldg(reinterpret_cast<const float4*>(wrow + 64 * kb + 4 * (sw ^ x)));
+            tc::tc_fence_before();  // this thread's reads of the group's accumulators precede the arrivals below
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    const int kb = 2 * half + kk;
-                    const float4 b0 = bs[kk][0], b1 = bs[kk][1], w0 = w[kk][0], w1 = w[kk][1];
-                    split2<PREC>(fmaxf(b0.x + w0.x, 0.f), fmaxf(b0.y + w0.y, 0.f), hi[kb].x, lo[kb].x);
-                    split2<PREC>(fmaxf(b0.z + w0.z, 0.f), fmaxf(b0.w + w0.w, 0.f), hi[kb].y, lo[kb].y);
-                    split2<PREC>(fmaxf(b1.x + w1.x, 0.f), fmaxf(b1.y + w1.y, 0.f), hi[kb].z, lo[kb].z);
-                    split2<PREC>(fmaxf(b1.z + w1.z, 0.f), fmaxf(b1.w + w1.w, 0.f), hi[kb].w, lo[kb].w);
-                    unsigned char* row = bop + kb * Cfg::B_CHUNK + e * 128 + ((c8 ^ (e & 7)) << 4);
-                    *reinterpret_cast<uint4*>(row) = hi[kb];
-                    if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
+            for (int kb = 0; kb < 4; ++kb) {
+                const float4 b0 = *reinterpret_cast<const float4*>(brow + 64 * kb + 4 * sw), b1 = *reinterpret_cast<const float4*>(brow + 64 * kb + 4 * (sw ^ 1));
+                uint2 h0, h1, l0, l1;
+                split2<PREC>(fmaxf(b0.x + w[kb][0].x, 0.f), fmaxf(b0.y + w[kb][0].y, 0.f), h0.x, l0.x);
+                split2<PREC>(fmaxf(b0.z + w[kb][0].z, 0.f), fmaxf(b0.w + w[kb][0].w, 0.f), h0.y, l0.y);
+                split2<PREC>(fmaxf(b1.x + w[kb][1].x, 0.f), fmaxf(b1.y + w[kb][1].y, 0.f), h1.x, l1.x);
+                split2<PREC>(fmaxf(b1.z + w[kb][1].z, 0.f), fmaxf(b1.w + w[kb][1].w, 0.f), h1.y, l1.y);
+                hi[kb] = sw ? make_uint4(h1.x, h1.y, h0.x, h0.y) : make_uint4(h0.x, h0.y, h1.x, h1.y);
+                lo[kb] = sw ? make_uint4(l1.x, l1.y, l0.x, l0.y) : make_uint4(l0.x, l0.y, l1.x, l1.y);
+                unsigned char* row = bop + kb * Cfg::B_CHUNK + e * 128 + ((c8 ^ (e & 7)) << 4);
+                *reinterpret_cast<uint4*>(row) = hi[kb];
+                if (PREC == 0) *reinterpret_cast<uint4*>(row + ME * 128) = lo[kb];
+                if (kb & 1) {
                     tc::fence_proxy_async();  // ordinary stores -> visible to the tensor cores
                     __syncwarp();
-                    if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[4 * g + kb]), 0));
+                    if (lane == 0) tc::mbar_arrive_remote_cta_release(tc::mapa(tc::smem_u32(&ready[2 * g + (kb >> 1)]), 0));
                 }
             }
             // the copies for the update leave after the arrivals (their CTA-scope release does not wait for global stores)
@@ -354,9 +367,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
                         const int e = 16 * mt + 8 * hh + g8;
-                        const uint32_t dst = tc::mapa(tc::smem_u32(s_red + (((g * 8) + 4 * (int)rank + q) * ME + e) * 5 + 2 * t4), (uint32_t)rE);
-                        if (t4 < 3) st_async_f32_2(dst, acc[mt][2 * hh], pbar);
-                        if (t4 < 2) st_async_f32_2(dst + 4u, acc[mt][2 * hh + 1], pbar);
+                        const uint32_t dst = tc::mapa(tc::smem_u32(s_red + (((g * 8) + 4 * (int)rank + q) * ME + e) * 6 + 2 * t4), (uint32_t)rE);
+                        if (t4 < 3) st_async_f32x2(dst, acc[mt][2 * hh], acc[mt][2 * hh + 1], pbar);
                     }
             }
         };
@@ -372,7 +384,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
     } else if (ownerw) {
         // ---- one thread per env of this CTA (owner warp og serves group og)
         for (int t = t_beg; t <= t_end; ++t) {
-            if (lane == 0) tc::mbar_expect_tx(&pfull[og], 8 * ME * 5 * 4);  // this step's head partials, counted as they land
+            if (lane == 0) tc::mbar_expect_tx(&pfull[og], 8 * ME * 6 * 4);  // this step's head partials, counted as they land
             const bool acting = owner && !REPLAY && t < a.T;
             StepPre pre;
             if (acting) pre = step_prepare(s, a, oenv, t, s_walls + ow * 8);
@@ -387,7 +399,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
 #pragma unroll
                 for (int blk = 0; blk < 8; ++blk)
 #pragma unroll
-                    for (int c = 0; c < 5; ++c) o[c] += s_red[((og * 8 + blk) * ME + oe) * 5 + c];
+                    for (int c = 0; c < 5; ++c) o[c] += s_red[((og * 8 + blk) * ME + oe) * 6 + c];
 #pragma unroll
                 for (int c = 0; c < 5; ++c) o[c] += s_bh[c];
                 if (acting) {
@@ -441,7 +453,7 @@ cudaError_t launch_rollout_pair2(const RolloutArgs& a0, int prec, cudaStream_t s
     constexpr int PER_PAIR = 2 * Cfg::NG * Cfg::ME;
     if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base || a0.d.npol > 1) return cudaErrorNotSupported;
     // Acting: beyond one wave of the one-group kernel (74 pairs of 64 envs), whose second wave would cost more than the longer
-    // steps here (6.8 us for 128 envs against 4.3 us for 64).  Replay: whenever a pair has its two groups.
+    // steps here (5.2 us for 128 envs against 3.6 us for 64).  Replay: whenever a pair has its two groups.
     if (a0.replay ? a0.d.B < PER_PAIR : a0.d.B <= 74 * PER_PAIR / 2) return cudaErrorNotSupported;
     RolloutArgs a = a0;
     size_t smem = Cfg::fixed_bytes + 1024;  // alignment slack
@@ -452,7 +464,6 @@ cudaError_t launch_rollout_pair2(const RolloutArgs& a0, int prec, cudaStream_t s
     }
     Pair2Maps maps;
     memset(&maps, 0, sizeof(maps));
-    if (!make_tensor_map_2d(&maps.w_hi, a.b.w2p_hi, Cfg::H, Cfg::H, 64, prec == 1)) return cudaErrorNotSupported;
     if (prec == 0 && !make_tensor_map_2d(&maps.w_lo, a.b.w2p_lo, Cfg::H, Cfg::H, 64, false)) return cudaErrorNotSupported;
     const int pairs = (a.d.B + PER_PAIR - 1) / PER_PAIR;
     const dim3 grid(2 * pairs, replay_slices(a, 2 * pairs));
