@@ -11,7 +11,7 @@
 //   layer 2   transposed, D[j][env] = sum_k W2[k][j] h1[env][k], M = 128 hidden units: two tcgen05 MMAs per k16,
 //             W2hi x [h1hi | h1lo] (N = 128) and W2lo x h1hi (N = 64), fp32 accumulators in tensor memory beside both
 //             planes of W2 (the A operand, transposed into it once: shared memory then holds the agent rows of W1 and is left
-//             to the workers; 2336 -> 2224 us on 131072 envs, T = 64); a dedicated warp issues the MMAs of both groups
+//             to the workers; 2336 -> 2118 us on 131072 envs, T = 64, with one proxy fence a step); a dedicated warp issues the MMAs of both groups
 //   heads     a worker thread = one hidden unit j (its accumulator lane): bias, ReLU, h2 stores (one 128-byte line per
 //             env and warp); the warp's 32 units x 32 envs go to shared memory as fp16 (hi, lo) terms and come back
 //             transposed (ldmatrix.trans) as A fragments of warp-level MMAs against Wh; the four 32-unit partials of an
@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(RolloutA
     float* s_base = reinterpret_cast<float*>(s_bop + NG * Cfg::B_BYTES);             // [NG][NE][H]
     uint64_t* wbar = reinterpret_cast<uint64_t*>(s_base + NG * NE * H);              // the agent rows of W1 landed
     uint64_t* tfull = wbar + 1;     // [NG] this step's MMAs of the group finished
-    uint64_t* ready = tfull + NG;   // [NG][2] k block of the group's operand rows written (8 worker warps arrive)
-    uint64_t* pdone = ready + NG * 2;  // [NG] the four head partials of every env of the group are stored (8 warps arrive)
+    uint64_t* ready = tfull + NG;   // [NG] the group's operand rows written (8 worker warps arrive)
+    uint64_t* pdone = ready + NG;  // [NG] the four head partials of every env of the group are stored (8 warps arrive)
     uint64_t* posrdy = pdone + NG;     // [NG] the group's positions for the next step are published (2 owner warps arrive)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(posrdy + NG);
     float* s_red = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(wbar) + 256);  // [NG][4][NE][5]
@@ -84,8 +84,7 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(RolloutA
         tc::mbar_init(wbar, 1);
         for (int g = 0; g < NG; ++g) {
             tc::mbar_init(&tfull[g], 1);
-            tc::mbar_init(&ready[2 * g], Cfg::NWORK);
-            tc::mbar_init(&ready[2 * g + 1], Cfg::NWORK);
+            tc::mbar_init(&ready[g], Cfg::NWORK);
             tc::mbar_init(&pdone[g], Cfg::NWORK);
             tc::mbar_init(&posrdy[g], NE / 32);
         }
@@ -175,43 +174,40 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(RolloutA
     __nv_bfloat16* g_h1lo = g_h1hi + (size_t)B * d.Tmax * H;
 
     if (wid == (NWT + NOWN) / 32) {
-        // ---- layer 2: one warp drives the tensor core for both groups (an elected lane issues), k block by k block, in the order the groups'
-        // operand blocks are written (group 0, then group 1, every step).  A block's eight arrivals also say that those
-        // warps have read the group's accumulators of the step before.
+        // ---- layer 2: one warp drives the tensor core for both groups (an elected lane issues), in the order the groups' operand
+        // tiles are written (group 0, then group 1, every step).  A tile's eight arrivals also say that those warps have read the
+        // group's accumulators of the step before.
         const uint32_t idesc_w = tc::umma_idesc<PREC>(128, 128, false, false), idesc_n = tc::umma_idesc<PREC>(128, 64, false, false);
         for (int t = t_beg; t <= t_end; ++t) {
             for (int g = 0; g < NG; ++g) {
                 const uint32_t acc = tmem + (uint32_t)(g * Cfg::ACC);
                 unsigned char* bop = s_bop + g * Cfg::B_BYTES;
+                ok = tc::warp_all(ok && tc::mbar_wait(&ready[g], (uint32_t)(t - t_beg) & 1u));
+                tc::tc_fence_after();
+                if (tc::elect_one()) {
 #pragma unroll
-                for (int kb = 0; kb < 2; ++kb) {
-                    ok = tc::warp_all(ok && tc::mbar_wait(&ready[2 * g + kb], (uint32_t)(t - t_beg) & 1u));
-                    tc::tc_fence_after();
-                    if (tc::elect_one()) {
-#pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16) {
+                    for (int k16 = 0; k16 < 8; ++k16) {
                         // A: 16 k = 8 columns.  B (K-major): 16 k = 32 bytes along the swizzled rows, 1024 bytes between 8-row groups
-                        const uint32_t ahi = tmem + (uint32_t)(Cfg::W_COL + 32 * kb + 8 * k16);
-                        const uint64_t bd = tc::umma_desc(bop + kb * Cfg::B_CHUNK + k16 * 32, 16, 1024);
+                        const uint32_t ahi = tmem + (uint32_t)(Cfg::W_COL + 8 * k16);
+                        const uint64_t bd = tc::umma_desc(bop + (k16 >> 2) * Cfg::B_CHUNK + (k16 & 3) * 32, 16, 1024);
                         if (PREC == 0) {
-                            tc::umma_ta(acc, ahi, bd, idesc_w, (kb | k16) ? 1u : 0u);
-                            tc::umma_ta(acc + 128u, ahi + 64u, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            tc::umma_ta(acc, ahi, bd, idesc_w, k16 ? 1u : 0u);
+                            tc::umma_ta(acc + 128u, ahi + 64u, bd, idesc_n, k16 ? 1u : 0u);
                         } else {  // bf16 operands: one product, the hi rows of the operand tile only
-                            tc::umma_ta(acc, ahi, bd, idesc_n, (kb | k16) ? 1u : 0u);
+                            tc::umma_ta(acc, ahi, bd, idesc_n, k16 ? 1u : 0u);
                         }
                     }
-                    if (kb == 1) tc::umma_commit(&tfull[g]);
-                    }
-                    __syncwarp();
+                    tc::umma_commit(&tfull[g]);
                 }
+                __syncwarp();
             }
         }
     } else if (worker) {
         // ---- layer 1 of group g for step t: 16-byte chunks of eight hidden units; all gathers of the agents' W1 rows are
         // in flight before any is used.  Thread (e, c8) covers chunk c8 of both k blocks of envs e and e + 32 (eight lanes
         // read 256 contiguous bytes of one row): chunk c8 goes to operand row (hi) and 64 + row (lo) of its block, at the
-        // 16-byte position c8 ^ (row % 8) of the 128-byte row (the 128-byte swizzle of a K-major operand).  Each finished
-        // block is announced to the issuer at once.
+        // 16-byte position c8 ^ (row % 8) of the 128-byte row (the 128-byte swizzle of a K-major operand).  The finished
+        // tile is announced to the issuer.
         auto gather = [&](int g, int t) {
             // (lanes 4-7 of an env read their two 16-byte pieces of a row in the other order: the eight lanes cover all banks)
             const int e = tidg >> 3, c8 = tidg & 7, sw = (c8 >> 2) & 1;
@@ -250,10 +246,10 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(RolloutA
                     *reinterpret_cast<uint4*>(row) = hi[kb][p];
                     if (PREC == 0) *reinterpret_cast<uint4*>(row + NE * 128) = lo[kb][p];
                 }
-                tc::fence_proxy_async();  // ordinary stores -> visible to the tensor core
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&ready[2 * g + kb]);
             }
+            tc::fence_proxy_async();  // ordinary stores -> visible to the tensor core (once: it costs some 300 clocks)
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&ready[g]);
             // the copies for the update leave after the arrivals
             if (b.h1 != nullptr && t < a.T) {
 #pragma unroll
