@@ -1174,10 +1174,86 @@ __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_i
     // fat CTAs each instead of tens of thousands of tiny ones) walks them in a stride loop.
     constexpr int PPB = 256 / G;  // parameters per piece of the main part
     static_assert(!GROUPED || G == 1, "many policies have a handful of partials");
-    const int nb_main = (int)((d.ob2 + PPB - 1) / PPB);
+    // Many policies: a thread takes four parameters of the main part (16 loads in flight instead of four), in W1 and b1 four in a row,
+    // in W2 the four of an 8-byte element of the fragment copies, so that those leave as whole sectors (1024 policies of 9349
+    // parameters: 127 us with one parameter a thread and 2-byte stores).
+    const int nb_w1 = (int)((d.oW2 + 1023) / 1024), nb_w2 = d.H * d.H / 1024;
+    const int nb_main = GROUPED ? nb_w1 + nb_w2 : (int)((d.ob2 + PPB - 1) / PPB);
     const int nb_total = nb_main + (int)(GROUPED ? (d.P - d.ob2 + 255) / 256 : (d.P - d.ob2 + 7) / 8);
     for (int bx = blockIdx.x; bx < nb_total; bx += gridDim.x) {
-        if (G > 1 && bx < nb_main) {
+        if (GROUPED && bx < nb_main) {
+            const bool w2 = bx >= nb_w1;
+            const int q = (w2 ? bx - nb_w1 : bx) * 256 + (int)threadIdx.x;
+            const int H = d.H, kt = (q >> 5) / (H / 8), nt = (q >> 5) % (H / 8);
+            const size_t i0 = w2 ? d.oW2 + (size_t)(kt * 16 + 2 * ((q >> 3) & 3)) * H + nt * 8 + (q & 7) : (size_t)q * 4;
+            if (w2 || i0 < d.oW2) {
+                const PartRegion& rg = a_in.reg[w2 ? 4 : region_of(i0)];
+                const float* p = reinterpret_cast<const float*>(reinterpret_cast<const unsigned char*>(rg.part) + poff) + (i0 - rg.start);
+                AdamIn in[4];
+                float g4[4] = {0.f, 0.f, 0.f, 0.f};
+                if (!w2) {
+                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const bool st = a.phase == 0;
+                    const float4 m = st ? *reinterpret_cast<const float4*>(b.adam_m + i0) : z, v = st ? *reinterpret_cast<const float4*>(b.adam_v + i0) : z;
+                    const float4 th = st ? *reinterpret_cast<const float4*>(b.theta + i0) : z;
+                    in[0] = {m.x, v.x, th.x}; in[1] = {m.y, v.y, th.y}; in[2] = {m.z, v.z, th.z}; in[3] = {m.w, v.w, th.w};
+#pragma unroll 4
+                    for (int s = 0; s < rg.ns; ++s) {
+                        const float4 x = *reinterpret_cast<const float4*>(p + (size_t)s * rg.stride);
+                        g4[0] += x.x; g4[1] += x.y; g4[2] += x.z; g4[3] += x.w;
+                    }
+                    float4 mo = z, vo = z, to = z;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) g4[u] *= a.inv_gscale;  // exact: a power of two
+                    *reinterpret_cast<float4*>(b.grads + i0) = make_float4(g4[0], g4[1], g4[2], g4[3]);
+                    if (st) {
+                        const AdamIn o0 = adam_arith(a, in[0], g4[0]), o1 = adam_arith(a, in[1], g4[1]), o2 = adam_arith(a, in[2], g4[2]), o3 = adam_arith(a, in[3], g4[3]);
+                        mo = make_float4(o0.m, o1.m, o2.m, o3.m);
+                        vo = make_float4(o0.v, o1.v, o2.v, o3.v);
+                        to = make_float4(o0.theta, o1.theta, o2.theta, o3.theta);
+                        *reinterpret_cast<float4*>(b.adam_m + i0) = mo;
+                        *reinterpret_cast<float4*>(b.adam_v + i0) = vo;
+                        *reinterpret_cast<float4*>(b.theta + i0) = to;
+                    }
+                } else {
+                    const size_t at[4] = {0, (size_t)H, (size_t)8 * H, (size_t)9 * H};  // k, k + 1, k + 8, k + 9
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) in[u] = state_of(i0 + at[u]);
+#pragma unroll 4
+                    for (int s = 0; s < rg.ns; ++s) {
+                        float v[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) v[u] = p[(size_t)s * rg.stride + at[u]];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) g4[u] += v[u];
+                    }
+                    uint32_t hi[4], lo[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const size_t i = i0 + at[u];
+                        const float gm = g4[u] * a.inv_gscale;
+                        b.grads[i] = gm;
+                        if (a.phase == 0) {
+                            const AdamIn o = adam_arith(a, in[u], gm);
+                            b.adam_m[i] = o.m;
+                            b.adam_v[i] = o.v;
+                            b.theta[i] = o.theta;
+                            uint16_t h16, l16;
+                            split1<0>(o.theta, h16, l16);
+                            b.w2p_hi[i - d.oW2] = h16;
+                            b.w2p_lo[i - d.oW2] = l16;
+                            hi[u] = h16;
+                            lo[u] = l16;
+                        }
+                    }
+                    if (a.phase == 0) {
+                        const int ef = (kt * (H / 8) + nt) * 32 + (q & 7) * 4 + ((q >> 3) & 3);
+                        b.w2f_hi[ef] = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
+                        b.w2f_lo[ef] = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
+                    }
+                }
+            }
+        } else if (G > 1 && bx < nb_main) {
             const int pi = threadIdx.x % PPB, grp = threadIdx.x / PPB;
             const size_t i = (size_t)bx * PPB + pi;
             float gsum = 0.f;
@@ -1624,7 +1700,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         const int grp = most > 48 ? 4 : 1;
         const unsigned nb = (unsigned)((d.ob2 * grp + 255) / 256 + (d.P - d.ob2 + 7) / 8);
         if (d.npol > 1) {
-            const unsigned per_policy = d.npol >= 74 ? 8u : (nb < 592u / d.npol ? nb : 592u / d.npol);  // at least four CTAs per SM in all, at most eight per policy
+            const unsigned per_policy = d.npol >= 74 ? (H == 64 ? 6u : 12u) : (nb < 592u / d.npol ? nb : 592u / d.npol);  // (many: two pieces a CTA)
             if constexpr (PREC == 0) launch<k_reduce_adam2<PREC, true, 1>>(dim3(per_policy, d.npol), 256, 0, s, a, R, pl.loss_blocks);
             else return cudaErrorNotSupported;
         } else {
