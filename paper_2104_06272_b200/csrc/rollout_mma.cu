@@ -548,6 +548,14 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
         if (!a.replay && ctas <= 148 && smem + w1 <= MAX_DYN_SMEM) return launch<k_rollout_mma<H, NW, PREC, false, 1, true, false, 32, true>>(grid, NW * 32 + 32, smem + w1, s, a);
     // The owner warp costs a CTA of the 128-wide kernel its second place on an SM: only where every CTA gets an SM of its own.
     // (H = 64: three CTAs per SM where there are that many)
+    // ... in fp32 with the agent rows of W1 beside them where the steps gather many times what the load takes and the GPU is full more
+    // than once (B200: 44158 envs, 100 cells, T = 45 425 -> 390 us, 30000 envs, 81 cells, T = 16 124 -> 113 us; but 104889 envs, 81
+    // cells, T = 6 145 -> 147 us, 12000 envs 76.4 -> 77.6 us, bf16 44158 envs 333 -> 345 us)
+    if constexpr (H == 64 && PREC == 0) {
+        const size_t w1b = (size_t)a.d.C * H * 4;
+        if (!a.replay && (size_t)grid.x * grid.y > 444 && a.T * Cfg::ME >= 6 * a.d.C && smem + w1b <= 75 * 1024)
+            return launch<k_rollout_mma<H, NW, PREC, GROUPED, 3, true, false, 32, true>>(grid, NW * 32 + 32, smem + w1b, s, a);
+    }
     if constexpr (H == 64)
         if ((size_t)grid.x * grid.y > 296) return launch_k<H, NW, PREC, GROUPED, 3, true>(a, grid, smem, s);
     if constexpr (H < 128) return launch_k<H, NW, PREC, GROUPED, 2, true>(a, grid, smem, s);
