@@ -66,185 +66,10 @@ cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c) {
     return cudaGetLastError();
 }
 
-// ----------------------------------------------------------------------------------------------------
-// Persistent FFMA rollout: the wide hidden layers (above 256) of callers without a workspace, whose fixed scratch has no room for
-// the tensor-core path's operands.  256 threads = 8 warps; H = 32*HJ hidden units; ME = 8*RR envs per CTA.
-// Per step: h1 = relu(base + W1[agent row]) -> h2 = relu(h1 W2 + b2) (register-tiled FFMA, W2 streamed through
-// L1/L2) -> 5 head outputs by warp reduction -> one thread per env: softmax, inverse-CDF sample with the
-// Philox uniform of (env, global step), env step, coalesced time-major stores.
-// ----------------------------------------------------------------------------------------------------
-template <int HJ, int RR>
-__global__ void __launch_bounds__(256) k_rollout(RolloutArgs a) {
-    PDL_START();
-    constexpr int H = 32 * HJ, ME = 8 * RR;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* s_base = reinterpret_cast<float*>(smem_raw);  // [ME][H]
-    float* s_h1 = s_base + ME * H;                       // [ME][H]
-    float* s_h2 = s_h1 + ME * H;                         // [ME][H]
-    float* s_out = s_h2 + ME * H;                        // [ME][8]
-    uint32_t* s_walls = reinterpret_cast<uint32_t*>(s_out + ME * 8);  // [ME][8]
-    int* s_pos = reinterpret_cast<int*>(s_walls + ME * 8);            // [ME]
-
-    const Dims& d = a.d;
-    const Buffers& b = a.b;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int e0 = blockIdx.x * ME;
-    const int B = d.B, C = d.C;
-    const float* W1 = b.theta_c + d.oW1;
-    const float* W2 = b.theta_c + d.oW2;
-    const float* b2 = b.theta_c + d.ob2;
-    const float* Wh = b.theta_c + d.oWh;
-    const float* bh = b.theta_c + d.obh;
-
-    for (int idx = tid; idx < ME * H; idx += 256) {
-        const int e = idx / H, j = idx - e * H;
-        s_base[idx] = (e0 + e < B) ? b.base[(size_t)(e0 + e) * H + j] : 0.f;
-    }
-    // per-env state lives in the registers of thread `tid` (tid < ME)
-    int my_pos = 0, my_tep = 0, my_start = 0, my_goal = 0;
-    const bool owner = tid < ME && e0 + tid < B;
-    if (tid < ME) {
-        if (owner) {
-            my_pos = b.pos[e0 + tid];
-            my_tep = b.tep[e0 + tid];
-            my_start = b.start[e0 + tid];
-            my_goal = b.goal[e0 + tid];
-            for (int wi = 0; wi < 8; ++wi) s_walls[tid * 8 + wi] = wi < d.W ? b.walls[(size_t)(e0 + tid) * d.W + wi] : 0u;
-        }
-    }
-    unsigned long long n_episodes = 0, n_goals = 0, n_epsteps = 0;
-    int bad = 0;
-    if (tid < ME) {
-        if (owner) {
-            EnvLane es;
-            es.pos = my_pos; es.tep = my_tep; es.start = my_start; es.goal = my_goal;
-            es.bad = 0;
-            check_env_state(es, C, s_walls + tid * 8);
-            my_pos = es.pos; my_start = es.start; my_goal = es.goal;
-            bad |= es.bad;
-        }
-        s_pos[tid] = my_pos;
-    }
-    __syncthreads();
-
-    for (int t = 0; t <= a.T; ++t) {
-        // ---- layer 1: only the agent plane changes from step to step
-        for (int idx = tid; idx < ME * H; idx += 256) {
-            const int e = idx / H, j = idx - e * H;
-            const float z = s_base[idx] + W1[(size_t)(C + s_pos[e]) * H + j];
-            s_h1[idx] = (fmaxf(z, 0.f));
-        }
-        __syncthreads();
-        // ---- layer 2: thread (wid, lane) owns rows wid+8*rr and columns lane+32*jj
-        {
-            float acc[RR][HJ];
-#pragma unroll
-            for (int rr = 0; rr < RR; ++rr)
-#pragma unroll
-                for (int jj = 0; jj < HJ; ++jj) acc[rr][jj] = 0.f;
-#pragma unroll 2
-            for (int k = 0; k < H; ++k) {
-                float w[HJ];
-#pragma unroll
-                for (int jj = 0; jj < HJ; ++jj) w[jj] = __ldg(W2 + (size_t)k * H + lane + 32 * jj);
-#pragma unroll
-                for (int rr = 0; rr < RR; ++rr) {
-                    const float x = s_h1[(wid + 8 * rr) * H + k];
-#pragma unroll
-                    for (int jj = 0; jj < HJ; ++jj) acc[rr][jj] = fmaf(x, w[jj], acc[rr][jj]);
-                }
-            }
-#pragma unroll
-            for (int jj = 0; jj < HJ; ++jj) {
-                const float bias = __ldg(b2 + lane + 32 * jj);
-#pragma unroll
-                for (int rr = 0; rr < RR; ++rr)
-                    s_h2[(wid + 8 * rr) * H + lane + 32 * jj] = (fmaxf(acc[rr][jj] + bias, 0.f));
-            }
-        }
-        __syncthreads();
-        // ---- heads: warp `wid` reduces its RR envs
-#pragma unroll
-        for (int rr = 0; rr < RR; ++rr) {
-            const int e = wid + 8 * rr;
-            float o[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-            for (int k = lane; k < H; k += 32) {
-                const float x = s_h2[e * H + k];
-#pragma unroll
-                for (int c = 0; c < 5; ++c) o[c] = fmaf(x, __ldg(Wh + k * 5 + c), o[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < 5; ++c) {
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) o[c] += __shfl_xor_sync(0xFFFFFFFFu, o[c], off);
-            }
-            if (lane < 5) s_out[e * 8 + lane] = o[lane] + __ldg(bh + lane);
-        }
-        __syncthreads();
-        // ---- one thread per env: value, sample, env step, records
-        if (owner) {
-            const int env = e0 + tid;
-            const float l0 = s_out[tid * 8 + 0], l1 = s_out[tid * 8 + 1], l2 = s_out[tid * 8 + 2], l3 = s_out[tid * 8 + 3];
-            b.tval[(size_t)t * B + env] = s_out[tid * 8 + 4];
-            if (t < a.T) {  // the shared per-env step (env_step.cuh): sample, transition rule of the configured env, records
-                EnvLane es;
-                es.pos = my_pos; es.tep = my_tep; es.start = my_start; es.goal = my_goal;
-                es.n_episodes = es.n_goals = es.n_epsteps = 0;
-                es.bad = 0;
-                act_and_step(es, a, env, t, l0, l1, l2, l3, s_walls + tid * 8);
-                my_pos = es.pos;
-                my_tep = es.tep;
-                n_episodes += es.n_episodes;
-                n_goals += es.n_goals;
-                n_epsteps += es.n_epsteps;
-                bad |= es.bad;
-                s_pos[tid] = my_pos;
-            }
-        }
-        __syncthreads();
-    }
-    if (owner) {
-        b.pos[e0 + tid] = (uint8_t)my_pos;
-        b.tep[e0 + tid] = (uint8_t)my_tep;
-    }
-    // statistics: integer atomics only, so totals do not depend on arrival order
-    if (tid < 32) {
-        // ME <= 32: all owners are in warp 0
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            n_episodes += __shfl_xor_sync(0xFFFFFFFFu, n_episodes, off);
-            n_goals += __shfl_xor_sync(0xFFFFFFFFu, n_goals, off);
-            n_epsteps += __shfl_xor_sync(0xFFFFFFFFu, n_epsteps, off);
-            bad |= __shfl_xor_sync(0xFFFFFFFFu, bad, off);
-        }
-        if (tid == 0) {
-            if (n_episodes) atomicAdd((unsigned long long*)&b.stats->episodes, n_episodes);
-            if (n_goals) atomicAdd((unsigned long long*)&b.stats->goals, n_goals);
-            if (n_epsteps) atomicAdd((unsigned long long*)&b.stats->episode_steps, n_epsteps);
-            if (blockIdx.x == 0) atomicAdd((unsigned long long*)&b.stats->frames, (unsigned long long)B * a.T);
-            if (bad) atomicOr(b.status, bad);
-        }
-    }
-}
-
-template <int HJ, int RR>
-static cudaError_t launch_rollout_t(const RolloutArgs& a, cudaStream_t s) {
-    constexpr int H = 32 * HJ, ME = 8 * RR;
-    const size_t smem = (size_t)(3 * ME * H + ME * 8) * sizeof(float) + ME * 8 * sizeof(uint32_t) + ME * sizeof(int);
-    return launch<k_rollout<HJ, RR>>((a.d.B + ME - 1) / ME, 256, smem, s, a);
-}
-
 cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
-    if (wide_supported(a.d.H, prec) && a.b.w2p_hi) return launch_rollout_wide(a, c);  // two launches per step
+    if (wide_supported(a.d.H, prec)) return launch_rollout_wide(a, c);  // two launches per step
     Scope sc(c, K_ROLLOUT);
-    if (rollout_mma_supported(a.d.H)) return launch_rollout_mma(a, prec, c.s);
-    switch (a.d.H / 32) {
-        case 12: return launch_rollout_t<12, 4>(a, c.s);
-        case 16: return launch_rollout_t<16, 2>(a, c.s);
-        case 24: return launch_rollout_t<24, 2>(a, c.s);
-        case 32: return launch_rollout_t<32, 2>(a, c.s);
-        default: return cudaErrorInvalidValue;
-    }
+    return launch_rollout_mma(a, prec, c.s);
 }
 
 // ----------------------------------------------------------------------------------------------------

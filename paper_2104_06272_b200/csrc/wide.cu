@@ -183,6 +183,8 @@ cudaError_t launch_nt(const void* A, size_t a_rows, const void* B, const NtArgs&
 }
 
 // Elements between the bf16 planes of h1 in the fp32 form: the recorded rows and the B rows of the bootstrap step.
+// First activation row of step t.  Tmax = 0: h1 and h2 hold the rows of one step only (acting without a workspace).
+__host__ __device__ inline size_t step_row0(const Dims& d, int t) { return d.Tmax ? (size_t)t * d.B : 0; }
 __host__ __device__ inline size_t h1_plane(const Dims& d) { return ((size_t)d.B * d.Tmax + d.B) * d.H; }
 
 // Eight consecutive hidden units of one row of h1 = relu(base + W1 row): bf16-rounded (one plane), or exact as three planes.
@@ -348,9 +350,11 @@ __global__ void __launch_bounds__(256, HW_ROWS >= 16 && H >= 768 ? 4 : 5) k_head
             b.vboot[i] = v4;
         } else {
             const size_t row = mode == 0 ? (size_t)t * d.B + i : i;
-            float4* o = reinterpret_cast<float4*>(b.out5 + row * 8);
-            o[0] = make_float4(o0, o1, o2, o3);
-            o[1] = make_float4(v4, 0.f, 0.f, 0.f);
+            if (b.out5) {
+                float4* o = reinterpret_cast<float4*>(b.out5 + row * 8);
+                o[0] = make_float4(o0, o1, o2, o3);
+                o[1] = make_float4(v4, 0.f, 0.f, 0.f);
+            }
             if (mode == 0) {
                 b.tval[row] = v4;
                 const int env = (int)i;
@@ -394,7 +398,7 @@ __global__ void __launch_bounds__(256, HW_ROWS >= 16 && H >= 768 ? 4 : 5) k_head
         if (env < rows) {
             const float4* bp = reinterpret_cast<const float4*>(b.base + env * H);
             const float4* wp = reinterpret_cast<const float4*>(b.theta_c + d.oW1 + ((size_t)d.C + s_pos[rl]) * H);
-            uint16_t* out = reinterpret_cast<uint16_t*>(b.h1) + ((size_t)(t + 1) * d.B + env) * H;
+            uint16_t* out = reinterpret_cast<uint16_t*>(b.h1) + (step_row0(d, t + 1) + env) * H;
 #pragma unroll 4
             for (int ch = q; ch < H / 8; ch += TPR)
                 h1_store8<F32>(out + 8 * ch, h1_plane(d), bp[2 * ch], bp[2 * ch + 1], __ldg(wp + 2 * ch), __ldg(wp + 2 * ch + 1));
@@ -596,7 +600,7 @@ static cudaError_t rollout_wide_t(const RolloutArgs& a, const Ctx& c) {
         return cudaSuccess;
     }
     for (int t = 0; t <= a.T; ++t) {
-        const size_t row0 = (size_t)t * B;
+        const size_t row0 = step_row0(d, t);
         if (t == 0) {  // later steps: the heads kernel of step t-1 writes the h1 rows of step t
             Scope sc(c, K_H1);
             CKW(h1_rows(b.pos, B, row0));

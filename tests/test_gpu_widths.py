@@ -70,3 +70,33 @@ def test_replayed_forward_pass_equals_the_rollouts_own(bnd, H, prec, B, T):
         grads.append(an.get(bnd.GRADS))
         assert an.status() == 0
     par.assert_close(grads[1], grads[0], par.rtol_of(prec), "replayed gradient")
+
+
+@pytest.mark.parametrize("B,H", [(3, 384), (130, 512), (77, 768), (1024, 1024)])
+def test_acting_without_a_workspace_at_the_wide_widths(bnd, B, H):
+    """One step's activations in the library's own scratch give the trajectory of the handle-based rollout."""
+    import numpy as np
+    import torch
+
+    T, N = 5, 6
+    cfg = bnd.make_cfg(B, N, H, T)
+    an = bnd.Anakin(cfg)
+    an.reset(7)
+
+    def dev(which):
+        x = an.get(which)
+        return torch.from_numpy(x.view(np.int32) if x.dtype == np.uint32 else x).cuda()
+
+    env = [dev(w) for w in (bnd.PARAMS, bnd.ENV_WALLS, bnd.ENV_START, bnd.ENV_GOAL, bnd.ENV_POS, bnd.ENV_TEP)]
+    traj = [torch.zeros(n, dtype=t, device="cuda") for n, t in ((T * B, torch.uint8), (T * B, torch.int8), (T * B, torch.uint8),
+                                                               (T * B, torch.float32), ((T + 1) * B, torch.float32), (T * B, torch.float32))]
+    for call in range(2):
+        assert bnd.rollout_noalloc(cfg, 7, call * T, T, *env, *traj) == bnd.OK
+        an.rollout()
+        for x, which in zip(traj, (bnd.TRAJ_POS, bnd.TRAJ_ACTION, bnd.TRAJ_DONE, bnd.TRAJ_REWARD, bnd.TRAJ_VALUE, bnd.TRAJ_LOGP)):
+            want = an.get(which)
+            if want.dtype == np.float32:
+                par.assert_close(x.cpu().numpy(), want, 1e-5, "trajectory")
+            else:
+                assert (x.cpu().numpy() == want.reshape(-1)).all()
+    assert an.status() == 0 and bnd.noalloc_status()[1] == 0
