@@ -512,6 +512,7 @@ int anakin_apply_grads_mean(anakin_t* h, int n_replicas) {
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->adam_k += 1;
     h->base_valid = false;  // parameters changed
+    h->acts_valid = false;  // ... and a pending trajectory's saved activations belong to the old ones
     h->frags_valid = true;  // every element of the 16-bit copies of W2 was rewritten
     return ANAKIN_OK;
 }

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from paper_2104_06272_b200.workloads import WORKLOADS
+from tests import parity as par
 
 pytestmark = pytest.mark.gpu
 
@@ -53,6 +54,27 @@ def test_split_update_equals_the_fused_update_bitwise(bnd, name):
     b.apply_grads()
     assert np.array_equal(a.get(bnd.PARAMS), b.get(bnd.PARAMS))
     assert a.status() == 0 and b.status() == 0
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_an_update_after_apply_grads_differentiates_under_the_new_parameters(bnd, name):
+    """A step applied between a rollout and its update changes the parameters: the activations that rollout saved are the old
+    ones', and the update must recompute them (as it does for a trajectory handed back through set())."""
+    w = CASES[name].scaled(lr=0.05)
+    got = []
+    for hand_back in (False, True):
+        an = make(bnd, w)
+        an.reset(3)
+        an.rollout()
+        an.grads()
+        an.rollout()
+        an.apply_grads()
+        if hand_back:
+            an.set(bnd.TRAJ_POS, an.get(bnd.TRAJ_POS))
+        an.grads()
+        got.append(an.get(bnd.GRADS))
+        assert an.status() == 0
+    par.assert_close(got[0], got[1], par.rtol_of(w.precision), "gradient after the step")
 
 
 def bnd_params_after_reset(bnd, w, seed):
