@@ -534,6 +534,23 @@ size_t anakin_blob_bytes(anakin_t* h, int which) {
     return blob_total(h, which);
 }
 
+// Whether a kernel launched now may address [p, p + bytes): the current device is the handle's, and both ends are plain memory of
+// that GPU.  Anything else (another GPU's memory, which needs peer access; managed or host memory; a range that runs out of its
+// allocation) is left to the runtime's copies, which take or refuse it themselves.
+static bool kernel_can_copy(const anakin_t* h, const void* p, size_t bytes) {
+    int cur = -1;
+    if (cudaGetDevice(&cur) != cudaSuccess || cur != h->cfg.device) return false;
+    for (const size_t at : {(size_t)0, bytes - 1}) {
+        cudaPointerAttributes pa;
+        if (cudaPointerGetAttributes(&pa, static_cast<const char*>(p) + at) != cudaSuccess) {
+            cudaGetLastError();  // (not this call's error)
+            return false;
+        }
+        if (pa.type != cudaMemoryTypeDevice || pa.device != h->cfg.device) return false;
+    }
+    return true;
+}
+
 static int copy_blob(anakin_t* h, int which, void* ptr, size_t bytes, int ptr_is_device, bool to_lib) {
     if (!h || !ptr) return ANAKIN_E_INVALID_ARG;
     const Blob bl = blob_of(h, which, h->d.B);
@@ -554,16 +571,17 @@ static int copy_blob(anakin_t* h, int which, void* ptr, size_t bytes, int ptr_is
         e = to_lib ? cudaMemcpyAsync(bl.ptr, ptr, bytes, kind, h->stream) : cudaMemcpyAsync(ptr, bl.ptr, bytes, kind, h->stream);
     } else {  // policy p's blob: contiguous on the caller's side, sub_bytes apart here; the last policy may have fewer envs
         const size_t full = h->K - (h->d.B_last == h->d.B ? 0 : 1), n = bl.bytes;
+        const bool by_kernel = ptr_is_device == 1 && kernel_can_copy(h, ptr, bytes);
         auto move = [&](unsigned char* mine, unsigned char* user, size_t width, size_t rows) {
             if (rows == 0 || width == 0) return cudaSuccess;
             void *dst = to_lib ? mine : user, *src = to_lib ? user : mine;
             const size_t dp = to_lib ? h->sub_bytes : width, sp = to_lib ? width : h->sub_bytes;
-            if (ptr_is_device == 1) {
+            if (by_kernel) {
                 ++h->launches;
                 return launch_copy_blocks(dst, dp, src, sp, width, rows, h->stream);
             }
-            if (h->sub_bytes <= 0x7FFFFFFFu) return cudaMemcpy2DAsync(dst, dp, src, sp, width, rows, kind, h->stream);
-            cudaError_t er = cudaSuccess;  // beyond the largest pitch a 2-D copy takes
+            if (ptr_is_device != 1 && h->sub_bytes <= 0x7FFFFFFFu) return cudaMemcpy2DAsync(dst, dp, src, sp, width, rows, kind, h->stream);
+            cudaError_t er = cudaSuccess;  // a pointer that is no host pointer, or beyond the largest pitch a 2-D copy takes
             for (size_t r = 0; r < rows && er == cudaSuccess; ++r)
                 er = cudaMemcpyAsync((char*)dst + r * dp, (const char*)src + r * sp, width, kind, h->stream);
             return er;

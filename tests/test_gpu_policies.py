@@ -263,3 +263,29 @@ def test_policies_blobs_by_device_pinned_and_host_copies_agree(bnd, name):
         an.set(bnd.TRAJ_ACTION, torch.zeros_like(rev).cuda())
         an.set(bnd.TRAJ_ACTION, value)
         assert np.array_equal(an.get(bnd.TRAJ_ACTION), rev.numpy())
+
+
+@pytest.mark.parametrize("name", ["k3_h64_ragged", "k5_h128"])
+def test_policies_blobs_outside_the_handles_gpu_go_by_the_runtimes_copies(bnd, name):
+    """The strided copy kernel may address memory of the handle's own GPU only.  Page-locked host memory stands in for the rest
+    (another GPU's memory needs a second one): passed as a device pointer it must take the runtime's copies, one per policy,
+    and come out the same; a tensor of this GPU takes the kernel, counted as a launch."""
+    w = CASES[name]
+    an = make(bnd, w, debug=0)
+    an.reset(3)
+    an.run(1)
+    want = an.get(bnd.ENV_POS)
+    n = an.blob_bytes(bnd.ENV_POS)
+    there, here = torch.zeros(n, dtype=torch.uint8).pin_memory(), torch.zeros(n, dtype=torch.uint8, device="cuda")
+    for out, by_kernel in ((there, False), (here, True)):
+        before = an.launch_count()
+        assert bnd.lib().anakin_get(an._h, bnd.ENV_POS, out.data_ptr(), n, 1) == bnd.OK
+        assert (an.launch_count() > before) == by_kernel
+        assert an.status() == 0 and (out.cpu().numpy() == want).all()
+        out += 1
+        torch.cuda.synchronize()
+        before = an.launch_count()
+        assert bnd.lib().anakin_set(an._h, bnd.ENV_POS, out.data_ptr(), n, 1) == bnd.OK
+        assert (an.launch_count() > before) == by_kernel
+        assert (an.get(bnd.ENV_POS) == (want + 1).astype(np.uint8)).all()
+        an.set(bnd.ENV_POS, want)
