@@ -289,10 +289,10 @@ const char* anakin_kernel_name(int id);
  * allocator, a process that must never synchronise the device (cudaMalloc and cudaFree may).  This call needs no
  * handle and no workspace.  The caller passes the rollout's inputs and outputs as DEVICE pointers; the only
  * scratch the rollout uses (B*H floats, repacked copies of the second-layer weights, one step's activations of layers wider
- * than 256) is a fixed
- * array compiled into the library, so
- *     B * H  <=  ANAKIN_NOALLOC_MAX_BH  (1,048,576 floats = 4 MiB),
- * and every GPU that loads the library holds the scratch (20.5 MiB in all) until the process exits.  Larger sizes return
+ * than 256) are fixed arrays compiled into the library, so
+ *     B * H  <=  ANAKIN_NOALLOC_MAX_BH  (1,048,576 floats = 4 MiB).
+ * A GPU holds 4.5 MiB of scratch from the first call on it, and 16 MiB more from the first call with H > 256, until the
+ * process exits (under CUDA_MODULE_LOADING=EAGER all of it from the library's load).  Larger sizes return
  * ANAKIN_E_WORKSPACE_TOO_SMALL (with a message on stderr); precision must be ANAKIN_PRECISION_FP32
  * (ANAKIN_E_UNSUPPORTED_CFG otherwise).  The call itself calls no cudaMalloc / cudaFree and no allocating library
  * routine; it enqueues one small memset and the rollout's kernels on `cuda_stream` and returns without synchronising.
@@ -306,8 +306,8 @@ const char* anakin_kernel_name(int id);
  *   global_step   env steps taken since the seed's reset (the caller adds T after each call); 1 <= T <= cfg->T_max
  * All buffers are the caller's and must stay alive until the stream has run the call.
  *
- * Set-up: the FIRST call on each device looks up the array's device address (cudaGetSymbolAddress) with that
- * device current; make that first call outside any stream capture.  The device that is current at the call must be
+ * Set-up: the FIRST call on each device, and the first one with H > 256, looks up an array's device address
+ * (cudaGetSymbolAddress, which loads it) with that device current; make those calls outside any stream capture.  The device that is current at the call must be
  * the one the pointers and the stream belong to.
  * Sharing: every call on a device uses the same array, which keeps the previous call's contents; the call
  * overwrites or clears all of it that it reads, so sequential calls are independent, but two calls that overlap

@@ -408,6 +408,7 @@ inline int replay_slices(const RolloutArgs& a, int ctas) {
     return (steps + len - 1) / len;
 }
 cudaError_t launch_rollout_pair(const RolloutArgs& a, int prec, cudaStream_t s);  // CTA-pair tcgen05 rollout (H = 256); cudaErrorNotSupported otherwise
+cudaError_t noalloc_wide_scratch(Buffers* b);  // acting without a workspace: h1, h2 and W2's planes of the wide layers
 bool wide_supported(int H, int prec);         // hidden layer too wide for the persistent rollouts (either precision)
 size_t wide_h1_rows(const Dims& d);           // rows of one h1 / h2 plane on that path: the recorded ones and the bootstrap step's
 size_t wide_scratch_bytes(const Dims& d);     // operands of the base GEMM (kept in the dh1 buffer)

@@ -4,13 +4,15 @@
 // fixed memory budget handed out at start-up, a plug-in inside a host application that owns the allocator, a
 // process that must not synchronise the device (cudaMalloc and cudaFree may) -- and that therefore cannot size
 // and provide the library's workspace either.  Such a caller passes only the rollout's inputs and outputs; the
-// scratch the rollout needs (the per-env first-layer constant `base`, B*H floats, two repacked copies of the
-// second-layer weights and, above 256 hidden units, the activations of one step) lives in a file-scope device array of
-// fixed size inside this library.
+// scratch the rollout needs (the per-env first-layer constant `base`, B*H floats, and two repacked copies of the
+// second-layer weights) lives in a file-scope device array of fixed size inside this library.  Above 256 hidden units
+// one step's activations and W2's planes come on top, in an array of their own (noalloc_wide.cu).
 //
-// The array below is device memory reserved in every CUDA context that loads the library, from load to exit,
-// whether or not this entry point is ever called.  Its name is a host-side stand-in in host code: the device
-// address is obtained once per device with cudaGetSymbolAddress and only that pointer is handed to kernels.
+// Each array is device memory of the module that holds it: reserved when CUDA loads that module into a context (by
+// default at the first call that needs it, with CUDA_MODULE_LOADING=EAGER with the library) and until exit.  Two files
+// are two modules, so that callers with narrow layers hold 4.5 MiB (measured: 6 MiB of the GPU's memory) and not the wide
+// layers' 16 MiB too (one array: 22 MiB).  The name is a host-side stand-in in host code: the device address is obtained
+// once per device with cudaGetSymbolAddress and only that pointer is handed to kernels.
 #include <cstdio>
 #include <cstring>
 
@@ -23,15 +25,11 @@ namespace {
 constexpr size_t kMaxBaseFloats = ANAKIN_NOALLOC_MAX_BH;  // B*H limit (floats)
 constexpr size_t kW2FragBytes = 2 * 256 * 256 * 2;          // W2 as tensor-pipe fragments, hi and lo planes (H <= 256)
 constexpr size_t kW2PlaneBytes = 2 * 256 * 256 * 2;         // W2 row-major as 16-bit hi and lo planes (H <= 256)
-// Wide layers (H > 256) run the tcgen05 GEMMs of the handle-based rollout on one step's activations: h1 as three bf16 terms, h2, and
-// three planes of W2.  (On the FFMA kernel they ran before, 2730 envs, H = 384, T = 24 took 4.8 ms.)
-constexpr size_t kH1Bytes = 3 * kMaxBaseFloats * 2, kH2Bytes = kMaxBaseFloats * 4, kW2WideBytes = 3ull * 1024 * 1024 * 2;
 constexpr size_t kTailBytes = 256;                          // statistics block + status word
 constexpr int kMaxDevices = 64;
 
-// [ base: kMaxBaseFloats floats | W2 fragments hi, lo | W2 planes hi, lo | anakin_stats | status word | h1 | h2 | W2 planes (wide) ]
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kMaxBaseFloats * sizeof(float) + kW2FragBytes + kW2PlaneBytes + kTailBytes +
-                                                                    kH1Bytes + kH2Bytes + kW2WideBytes];
+// [ base: kMaxBaseFloats floats | W2 fragments hi, lo | W2 planes hi, lo | anakin_stats | status word ]
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kMaxBaseFloats * sizeof(float) + kW2FragBytes + kW2PlaneBytes + kTailBytes];
 
 unsigned char* g_scratch_ptr[kMaxDevices] = {nullptr};  // device address of the array, per device ordinal
 
@@ -127,9 +125,7 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
     const Ctx ctx{s, &launches, nullptr};
     if (launch_env_base(a.d, b, ctx) != cudaSuccess) return ANAKIN_E_CUDA;  // fills `base`: nothing of the last call survives
     if (wide_supported(cfg->H, cfg->precision)) {
-        b.h1 = reinterpret_cast<float*>(tail + kTailBytes);
-        b.h2 = reinterpret_cast<float*>(tail + kTailBytes + kH1Bytes);
-        b.w2p_hi = reinterpret_cast<uint16_t*>(tail + kTailBytes + kH1Bytes + kH2Bytes);
+        if (noalloc_wide_scratch(&b) != cudaSuccess) return ANAKIN_E_CUDA;
         a.d.Tmax = 0;  // the activations of one step
         if (launch_pack_w2_wide(a.d, b, ctx) != cudaSuccess) return ANAKIN_E_CUDA;
     } else if (launch_pack_w2(a.d, b, cfg->precision, ctx) != cudaSuccess) {  // likewise the weight fragments

@@ -5,6 +5,10 @@ the allocator, loops that must not synchronise the device): they pass inputs and
 scratch is a fixed array inside the library.  It must give what the handle-based rollout gives, call after call,
 although every call reuses the same array.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -55,6 +59,41 @@ def test_noalloc_rollout_matches_handle_rollout_twice_in_a_row():
             else:
                 assert (got == want).all(), (call, name)
         assert (pos.cpu().numpy() == an.get(bnd.ENV_POS)).all() and (tep.cpu().numpy() == an.get(bnd.ENV_TEP)).all()
+
+
+_MEMORY_PROBE = """
+import numpy as np, torch
+from paper_2104_06272_b200 import binding as bnd
+
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+for H in (64, 256, 512, 1024):
+    B, N, T = 64, 5, 3
+    cfg = bnd.make_cfg(B, N, H, T)
+    an = bnd.Anakin(cfg)
+    an.reset(1)
+    dev = lambda w: torch.from_numpy(an.get(w).view(np.uint8)).cuda()
+    env = [dev(w) for w in (bnd.PARAMS, bnd.ENV_WALLS, bnd.ENV_START, bnd.ENV_GOAL, bnd.ENV_POS, bnd.ENV_TEP)]
+    out = [torch.empty(n * 4, dtype=torch.uint8, device="cuda") for n in (T * B, T * B, T * B, T * B, (T + 1) * B, T * B)]
+    an.rollout()  # loads the kernels
+    before = free()
+    assert bnd.rollout_noalloc(cfg, 1, 0, T, *env, *out) == bnd.OK
+    print(H, before - free())
+"""
+
+
+def test_noalloc_scratch_of_the_wide_layers_is_not_held_for_narrow_ones():
+    """What a first call takes of the GPU's memory (a fresh process; CUDA's default lazy loading; steps of 2 MiB): 4.5 MiB up to 256
+    hidden units, 16 MiB more above, nothing on later calls."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = {**os.environ, "PYTHONPATH": root, "CUDA_MODULE_LOADING": "LAZY"}
+    r = subprocess.run([sys.executable, "-c", _MEMORY_PROBE], env=env, cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    took = {int(h): int(n) / 2**20 for h, n in (ln.split() for ln in r.stdout.splitlines())}
+    assert took[64] <= 8 and took[256] == 0, took
+    assert took[512] <= 20 and took[1024] == 0, took
 
 
 def test_noalloc_status_reports_a_start_position_on_a_wall():
