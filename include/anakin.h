@@ -298,7 +298,7 @@ const char* anakin_kernel_name(int id);
  * routine; it enqueues one small memset and the rollout's kernels on `cuda_stream` and returns without synchronising.
  *
  * It computes exactly what anakin_rollout(h, T) computes on a handle with the same cfg, seed, GLOBAL_STEP, PARAMS
- * and env blobs: same kernels, same results.
+ * and env blobs: same kernels, bit for bit the same results.
  *   in      dev_params f32[P]; dev_walls u32[B][ceil(C/32)]; dev_start, dev_goal u8[B]   (read only)
  *   in/out  dev_pos, dev_tep u8[B]   (env dynamic state, advanced by T steps)
  *   out     dev_traj_pos u8[T][B]; dev_traj_action i8[T][B]; dev_traj_done u8[T][B]; dev_traj_reward f32[T][B];

@@ -523,10 +523,11 @@ size_t wide_h1_rows(const Dims& d) { return (size_t)d.B * d.Tmax + d.B; }
 // base = b1 + walls x W1[wall plane] + W1[goal row] as one GEMM (K = C cells, padded to a multiple of 64): the operand X is
 // exact, W1 has one (bf16 workload) or three exact bf16 terms, the accumulation is fp32.  Three terms are one GEMM of three
 // times the K: the smallest term's rows first, X repeated.  cudaErrorNotSupported for the
-// buffers of other paths and for small batches, where the gather kernel's single launch is quicker (B H = 2^20: 11 us each).
+// buffers of other paths and for small batches, where the gather kernel's single launch is quicker (B H = 2^20: 11 us each): up to the
+// sizes that act without a workspace, which has no room for the operands, so that both give the same bits.
 // Uses the dh1 buffer, which is dead outside the update, as scratch for the operands.
 cudaError_t launch_env_base_wide(const Dims& d, const Buffers& b, const Ctx& c) {
-    if (!b.w2p_hi || !wide_supported(d.H, 0) || (size_t)d.B * d.H < ((size_t)1 << 20)) return cudaErrorNotSupported;
+    if (!b.w2p_hi || !wide_supported(d.H, 0) || (size_t)d.B * d.H <= ANAKIN_NOALLOC_MAX_BH) return cudaErrorNotSupported;
     const bool f32 = is_f32(b);
     const int Cp = (d.C + 63) / 64 * 64, terms = f32 ? 3 : 1;
     uint16_t* X = reinterpret_cast<uint16_t*>(b.dh1);

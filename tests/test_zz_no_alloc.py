@@ -61,6 +61,33 @@ def test_noalloc_rollout_matches_handle_rollout_twice_in_a_row():
         assert (pos.cpu().numpy() == an.get(bnd.ENV_POS)).all() and (tep.cpu().numpy() == an.get(bnd.ENV_TEP)).all()
 
 
+@pytest.mark.parametrize("H,B,N", [
+    (32, 700, 5), (64, 31, 12), (64, 16384, 3), (96, 2400, 7), (128, 33, 16), (128, 8192, 5), (192, 777, 6), (256, 33, 13), (256, 4096, 4),
+    (384, 2730, 3), (512, 130, 9), (512, 2047, 5), (512, 2048, 5), (768, 1365, 4), (1024, 9, 16), (1024, 1024, 6),
+])
+def test_noalloc_rollout_is_the_handles_bit_for_bit_at_every_width(H, B, N):
+    """Every hidden width, batches on both sides of the kernels' own size rules, up to the largest the call takes (B H = 2^20)."""
+    from paper_2104_06272_b200 import binding as bnd
+    from paper_2104_06272_b200.workloads import random_params
+
+    T, seed = 4, 7
+    cfg = bnd.make_cfg(B, N, H, T, episode_cap=3)
+    an = bnd.Anakin(cfg)
+    an.reset(seed)
+    an.set(bnd.PARAMS, random_params(5, an.P, 0.15 if H <= 256 else 0.05))
+    dev = lambda which: torch.from_numpy(an.get(which).view(np.uint8)).cuda()  # noqa: E731
+    ins = [dev(w) for w in (bnd.PARAMS, bnd.ENV_WALLS, bnd.ENV_START, bnd.ENV_GOAL, bnd.ENV_POS, bnd.ENV_TEP)]
+    blobs = (bnd.TRAJ_POS, bnd.TRAJ_ACTION, bnd.TRAJ_DONE, bnd.TRAJ_REWARD, bnd.TRAJ_VALUE, bnd.TRAJ_LOGP)
+    an.rollout()
+    want = [an.get(w).view(np.uint8) for w in blobs]
+    outs = [torch.zeros(x.size, dtype=torch.uint8, device="cuda") for x in want]
+    assert bnd.rollout_noalloc(cfg, seed, 0, T, *ins, *outs) == bnd.OK
+    assert bnd.noalloc_status() == (bnd.OK, 0) and an.status() == 0
+    for got, x in zip(outs, want):
+        assert (got.cpu().numpy() == x).all()
+    assert (ins[4].cpu().numpy() == an.get(bnd.ENV_POS)).all() and (ins[5].cpu().numpy() == an.get(bnd.ENV_TEP)).all()
+
+
 _MEMORY_PROBE = """
 import numpy as np, torch
 from paper_2104_06272_b200 import binding as bnd
