@@ -13,14 +13,14 @@
 //   warp 1 (one lane)  tcgen05.mma issuer.  Per step: the dh1 product (K = H; three fp16 terms per k16, one in the bf16
 //                      workload, all into one of two 128-column accumulators); then, for the step before, the agent-plane
 //                      product  D[unit][cell] += sum over the 128 envs of dh1[env][unit] * onehot[env][cell]  (K = 128,
-//                      operand tiles that the epilogue warps wrote) into a third accumulator that lives for the whole
-//                      kernel
+//                      operand tiles that the epilogue warps wrote) into a third accumulator, restarted after every GROUP
+//                      steps
 //   warp 2 (one lane)  TMA loads of the layer-1 gates (the bit mask the rollout recorded, 128 envs x 16 bytes per step)
 //                      into a box the epilogue reads
 //   warps 3-10         epilogue, thread = (unit, half of the envs): tcgen05.ld, gate, S +=, 16-bit split; writes its
 //                      dh1^T row (hi and lo planes, K-major) and the one-hot elements in the 128-byte-swizzled layout
-// At the end the epilogue warps store S (two 16-bit planes) and the agent accumulator as one split-K partial per
-// CTA.  Tensor memory: [W2 planes | two dh1 accumulators | agent accumulator]; at H = 256 only the hi plane
+// The epilogue warps store S (two 16-bit planes) at the end of a unit and add the agent accumulator, after every GROUP steps and
+// at the end, into one split-K partial per CTA.  Tensor memory: [W2 planes | two dh1 accumulators | agent accumulator]; at H = 256 only the hi plane
 // of W2 fits (128 + 256 + 128 = 512 columns) and the lo plane is an ordinary shared-memory operand.
 //
 // H = 256 runs as a CTA PAIR (a cluster of two, tcgen05 cta_group::2): the pair owns all 256 units of an env tile, each
@@ -69,6 +69,11 @@ struct Dh1aCfg {
     static constexpr int W_BYTES = W_LO_SMEM ? NCH * W_BOX : 0;
     // the planes bound for tensor memory are staged by TMA in the (still unused) dh1^T tile where they fit
     static constexpr bool W_STAGED = WT_PL * NCH * W_BOX <= PL * 2 * BN * 128;
+    // fp32 workloads: the agent-plane accumulator restarts every GROUP steps (768 MMAs) and the groups are added with round-to-nearest in
+    // the CTA's partial: the tensor core's own accumulation rounds toward zero, and on a board of few cells nearly every MMA hits
+    // a cell.  Left to run, 85,000 rows a CTA on 2 x 2 cells (H = 128) came out 1.2e-4 low, now 8e-6; the restarts cost nothing that
+    // shows (131072 envs, 8 x 8, T = 64: 6.21 -> 6.23 ms for the whole iteration, runs 0.7 % apart).
+    static constexpr int GROUP = PREC == 1 ? (1 << 30) : 48;
     static constexpr int BARS = 320;
     static constexpr int MAX_SMEM = 232448 - 1024;       // 227 KB per CTA minus alignment slack
     static constexpr int RING = MAX_SMEM - BARS - W_BYTES - D_TILE - O_TILE - G_TILE;
@@ -260,7 +265,7 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
                         // env rows = 2048 bytes further, cells 64.. one box further
                         const uint64_t dd = tc::umma_desc(sD + (pl * 2 + (k16 >> 2)) * Cfg::D_BOX + (k16 & 3) * 32, 16, 1024);
                         const uint64_t od = tc::umma_desc(sO + k16 * 2048, BM * 128, 1024);
-                        const uint32_t accum = (v > 0 || pl > 0 || k16 > 0) ? 1u : 0u;
+                        const uint32_t accum = (v % Cfg::GROUP > 0 || pl > 0 || k16 > 0) ? 1u : 0u;  // (a group's first MMA restarts the sum)
                         if (PAIR) tc::umma_pair(acc_agent, dd, od, idesc_agent, accum);
                         else tc::umma(acc_agent, dd, od, idesc_agent, accum);
                     }
@@ -383,6 +388,38 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
         unsigned char* drow = sD + half * Cfg::D_BOX + j * 128;  // this thread's row of the dh1^T hi box of its env half
         int prev_off = -1;  // byte offset of the one-hot element this thread set the step before
         int g = 0;          // running step index of this CTA
+        float* const part = part_agent + (size_t)xi * part_stride + n0 + j;
+        // The agent accumulator (lane = unit, column = cell) into this CTA's partial: the first group is written, every later one added to
+        // what this same thread wrote.  The MMAs of the steps so far have been waited for; no other is issued before this warp's next
+        // arrival on tiles_full.
+        auto drain_agent = [&](bool first, bool got) {
+            tc::tc_fence_after();
+            __syncwarp();
+#pragma unroll 1
+            for (int c0 = 0; c0 < 64 * NC; c0 += 32) {
+                const int cell0 = 64 * NC * half + c0;
+                if (cell0 >= C) break;
+                float* const p = part + (size_t)cell0 * H;
+                uint32_t r[32];
+                float o[32];
+#pragma unroll
+                for (int i = 0; i < 32; ++i) o[i] = 0.f;
+                if (!first) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = cell0 + i < C ? p[(size_t)i * H] : 0.f;
+                }
+                if (got) {
+                    tc::tmem_ld32(acc_agent + lane_base + (uint32_t)cell0, r);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) r[i] = 0u;  // an empty slice contributes zeros
+                }
+#pragma unroll
+                for (int i = 0; i < 32; ++i)
+                    if (cell0 + i < C) p[(size_t)i * H] = o[i] + __uint_as_float(r[i]);
+            }
+            tc::tc_fence_before();
+        };
         volatile int* own = shape + 4 + 3 * (wid - Cfg::FIRST_EPI);  // this warp's unit, the end of its steps, its row of S
         own[0] = xi;
         while (ok && own[0] < shape[2]) {
@@ -398,6 +435,11 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             for (int t = min(slice * shape[1], T); t < own[1]; ++t, ++g) {
                 const int cell = (half == 0 && oh_env < B) ? (int)b.tpos[(size_t)t * B + oh_env] : -1;
                 const int buf = g % ACCS;
+                if (PREC != 1 && g > 0 && g % Cfg::GROUP == 0) {  // a whole group of the agent plane
+                    ok = tc::mbar_wait(tiles_free, (uint32_t)(g - 1) & 1u);
+                    if (!ok) break;
+                    drain_agent(g == Cfg::GROUP, true);
+                }
                 if (ok) ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g / ACCS) & 1u);
                 if (!ok) break;
                 tc::tc_fence_after();
@@ -479,28 +521,11 @@ __device__ __forceinline__ void dh1a_body(const Dh1aMaps& maps, const LearnArgs&
             __syncwarp();
         }
         if (!ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
-        // agent-plane partial of this CTA: accumulator lane = unit, column = cell
+        // the last group (or zeros)
         bool got = ok;
         if (got && G > 0) got = tc::mbar_wait(tiles_free, (uint32_t)(G - 1) & 1u);
         if (!got && ok && lane == 0) atomicOr(status, DEV_E_WAIT_TIMEOUT);
-        tc::tc_fence_after();
-        __syncwarp();
-        float* part = part_agent + (size_t)xi * part_stride + n0 + j;
-#pragma unroll
-        for (int c0 = 0; c0 < 64 * NC; c0 += 32) {
-            uint32_t r[32];
-            if (got && G > 0) {
-                tc::tmem_ld32(acc_agent + lane_base + (uint32_t)(64 * NC * half + c0), r);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) r[i] = 0u;  // an empty slice contributes zeros
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int cell = 64 * NC * half + c0 + i;
-                if (cell < C) part[(size_t)cell * H] = __uint_as_float(r[i]);
-            }
-        }
+        drain_agent(PREC == 1 || G <= Cfg::GROUP, got && G > 0);
     }
     // (pair) neither CTA leaves or frees tensor memory while the other may still signal it or run MMAs that touch it
     tc::tc_fence_before();

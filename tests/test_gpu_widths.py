@@ -52,6 +52,38 @@ def test_width_one_iteration_stage_by_stage(bnd, H, prec, B, N, T):
         print(w.name, "worst error / bound:", {k: round(v, 3) for k, v in par.MARGINS.items()})
 
 
+LONG_SUMS = [
+    # (H, precision, B, N, T, bias of the value head).  Many rows a CTA: the accumulators of the backward kernels are emptied and
+    # restarted on the way (the agent plane every 48 tiles of 128 rows at H = 128 and 256).  However the tiles are dealt out, one of
+    # the 148 CTAs (74 pairs at H = 256) has at least the mean of them.
+    # The tensor core rounds toward zero, so a sum that is left in one accumulator is biased, most where nearly every MMA adds to
+    # it: four cells, and a value head that is off by 3 (every row pulls the same way).
+    (128, 0, 131072, 2, 96, 3.0),
+    (128, 0, 18945, 13, 49, 0.0), (256, 0, 30000, 3, 20, 3.0), (256, 0, 7000, 12, 70, 0.0),
+]
+
+
+@pytest.mark.parametrize("H,prec,B,N,T,bias", LONG_SUMS)
+def test_gradients_of_long_sums(bnd, H, prec, B, N, T, bias):
+    """One whole update on the library's own trajectory, element by element against the oracle."""
+    w = Workload(f"long_h{H}_p{prec}", B=B, N=N, H=H, T=T, iters=1, precision=prec)
+    an = bnd.Anakin(bnd.cfg_from_workload(w, debug_logits=1))
+    an.reset(11)
+    theta = random_params(5, w.P, 0.15)
+    theta[-1] = bias
+    an.set(bnd.PARAMS, theta)
+    st = par.gpu_state(an, bnd)
+    an.rollout()
+    an.gae()
+    row = lambda which: an.get(which).reshape(T, B)  # noqa: E731
+    par.MARGINS.clear()
+    try:
+        par.check_learn(an, bnd, w, st, dict(pos=row(bnd.TRAJ_POS), action=row(bnd.TRAJ_ACTION)), row(bnd.ADV), row(bnd.RET))
+    finally:
+        print(w.name, "worst error / bound:", {k: round(v, 3) for k, v in par.MARGINS.items()})
+    assert an.status() == 0
+
+
 @pytest.mark.parametrize("H,prec,B,T", [(32, 0, 40, 7), (64, 0, 33, 9), (96, 1, 70, 5), (128, 0, 65, 11), (128, 1, 200, 4), (256, 0, 127, 6), (256, 0, 300, 9),
                                         (256, 1, 129, 7), (384, 0, 70, 5)])
 def test_replayed_forward_pass_equals_the_rollouts_own(bnd, H, prec, B, T):
