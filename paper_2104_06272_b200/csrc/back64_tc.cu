@@ -15,7 +15,10 @@
 //               (A = one-hot cells, 128 or 256 of them; B = dh1)
 //   warps 2-9   thread = (row, half of the units): tcgen05.ld, gate, S +=, 16-bit split; the dh1 planes go over the dh2 planes
 //               of the same stage once dW2 has read them
-// dW2 restarts its accumulator every FLUSH tiles (4096 rows, as in the plain GEMM); the groups are added in registers.
+// The tensor core rounds toward zero, so a long sum in one accumulator comes out low.  dW2 restarts its accumulator every FLUSH tiles
+// (4096 rows, as in the plain GEMM) and the groups are added in registers; the agent plane restarts every AGENT_FLUSH tiles (768 MMAs
+// an accumulator, fp32 workloads) and the groups are added in the CTA's partial.  Left to run, 142,000 rows a CTA on 2 x 2 cells came
+// out 1.1e-4 low.
 #include <cstring>
 
 #include "tc_common.cuh"
@@ -23,6 +26,9 @@
 namespace anakin {
 
 namespace {
+
+__device__ __forceinline__ void tmem_cols(uint32_t taddr, uint32_t (&r)[16]) { tc::tmem_ld16_nowait(taddr, r); }
+__device__ __forceinline__ void tmem_cols(uint32_t taddr, uint32_t (&r)[32]) { tc::tmem_ld32_nowait(taddr, r); }
 
 template <int PREC, int NC>
 struct Back64Cfg {
@@ -36,6 +42,10 @@ struct Back64Cfg {
     static constexpr int W_BOX = H * 128, W_BYTES = PL * W_BOX;
     static constexpr int O_TILE = 2 * NC * BOX;      // one-hot: 128 rows x NC * 128 cells in 64-wide boxes
     static constexpr int FLUSH = 32;                 // tiles per dW2 accumulator
+    // tiles per agent-plane accumulator, and of the first one.  Its last tile is never the one before a restart of dW2: there the issuer
+    // waits for the epilogue of the new tile before it issues the agent MMAs of the old one, which that epilogue would be waiting for.
+    static constexpr int AGENT_FLUSH = 96, AGENT_FIRST = 80;
+    static_assert(AGENT_FLUSH % FLUSH == 0 && AGENT_FIRST % FLUSH != 0, "the agent plane and dW2 never restart at the same tile");
     // Two planes of the N operand are one MMA of 128 columns (half of them the lo plane's): the M operand is then read from shared
     // memory once, and shared memory is what bounds these products.  (At NC = 2 tensor memory has no room for it in dh1.)
     static constexpr int W2_N = PL * H, AGENT_N = PL * H, ACC_N = PL == 2 && NC == 1 ? 2 * H : H;
@@ -56,7 +66,8 @@ struct Back64Args {
     int nx;  // CTAs per policy: one partial of dW2 and of the agent plane each
 };
 
-template <int PREC, int NC, bool GROUPED>
+// LONG: a CTA may walk more than AGENT_FIRST tiles.
+template <int PREC, int NC, bool GROUPED, bool LONG>
 __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(const __grid_constant__ Back64Maps maps, const __grid_constant__ Back64Args in) {
     using Cfg = Back64Cfg<PREC, NC>;
     constexpr int H = Cfg::H, BM = Cfg::BM, PL = Cfg::PL, HST = Cfg::HST, DST = Cfg::DST, BOX = Cfg::BOX;
@@ -170,7 +181,7 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
 #pragma unroll
                     for (int c = 0; c < NC; ++c)
                         tc::umma(tmem + (uint32_t)(Cfg::AGENT_COL + Cfg::AGENT_N * c), tc::umma_desc(sO + 2 * c * BOX + k16 * 2048, BOX, 1024), dd, id_agent,
-                                 v > 0 || k16 > 0);
+                                 (v > 0 && !(LONG && v % Cfg::AGENT_FLUSH == Cfg::AGENT_FIRST)) || k16 > 0);  // (a group's first MMA restarts the sum)
                 }
                 tc::umma_commit(&empty[s]);
             }
@@ -273,6 +284,46 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
 #pragma unroll
             for (int i = 0; i < 32; ++i) w_acc[i] += v[i];
         };
+        // The agent accumulators (lane = cell, column = unit) into this CTA's partial: the first group is written, every later one added
+        // to what this same thread wrote.  The MMAs of the tiles so far have been waited for; no other is issued before this warp's
+        // next arrival on tiles_full.
+        // W columns at a time: 16 inside the loop, which leaves few registers; 32 and unrolled at the end, where nothing runs beside it.
+        auto drain_agent = [&](auto width, bool first, bool got) {
+            constexpr int W = decltype(width)::value, PIECES = NC * (32 / W);
+            float* pagent = in.part_agent + (size_t)xi * in.stride_agent;
+            if (GROUPED) pagent = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(pagent) + (size_t)pol * in.a.d.pstride);
+            tc::tc_fence_after();
+            __syncwarp();
+#pragma unroll(W == 32 ? PIECES : 1)
+            for (int k = 0; k < PIECES; ++k) {
+                const int c = k / (32 / W), cell = 128 * c + r, c0 = 32 * half + W * (k % (32 / W));
+                float v[W];
+#pragma unroll
+                for (int i = 0; i < W; ++i) v[i] = 0.f;
+                if (got) {
+                    uint32_t x0[W], x1[W];
+                    const uint32_t at = tmem + lane_base + (uint32_t)(Cfg::AGENT_COL + Cfg::AGENT_N * c + c0);
+                    tmem_cols(at, x0);
+                    if (PL == 2) tmem_cols(at + 64, x1);
+                    tc::tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < W; ++i) v[i] = PL == 2 ? __uint_as_float(x0[i]) + __uint_as_float(x1[i]) : __uint_as_float(x0[i]);
+                }
+                if (cell < C) {
+                    float4* p = reinterpret_cast<float4*>(pagent + (size_t)cell * H + c0);
+                    if (!first) {
+#pragma unroll
+                        for (int i = 0; i < W / 4; ++i) {
+                            const float4 o = p[i];
+                            v[4 * i] += o.x; v[4 * i + 1] += o.y; v[4 * i + 2] += o.z; v[4 * i + 3] += o.w;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < W / 4; ++i) p[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                }
+            }
+            tc::tc_fence_before();
+        };
         auto store_S = [&](size_t row, const float (&v)[32]) {  // 32 units of one row, two 16-bit planes
             uint32_t hi[16], lo[16];
 #pragma unroll
@@ -302,6 +353,11 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
             for (int i = 0; i < 32; ++i) s_acc[i] = 0.f;
             for (int t = t_begin(u); t < t1; t += SP, ++g) {
                 const int buf = g & 1, s = g % DST, hs = g % HST;
+                if (LONG && g % Cfg::AGENT_FLUSH == Cfg::AGENT_FIRST) {  // a whole group of the agent plane
+                    ok = tc::mbar_wait(&empty[(g - 1) % DST], (uint32_t)((g - 1) / DST) & 1u);
+                    if (!ok) break;
+                    drain_agent(std::integral_constant<int, 16>{}, g == Cfg::AGENT_FIRST, true);
+                }
                 const int cell = half == 0 && have && t + row_dt < t1 ? (int)b.tpos[(size_t)(t + row_dt) * B + env] : -1;
                 ok = tc::mbar_wait(&tfull[buf], (uint32_t)(g >> 1) & 1u);
                 if (!ok) break;
@@ -399,24 +455,7 @@ __global__ void __launch_bounds__(Back64Cfg<PREC, NC>::THREADS, 1) k_back64(cons
             }
             store_S((size_t)(xi / m_tiles) * B + r, s_acc);
         }
-        float* pagent = in.part_agent + (size_t)xi * in.stride_agent;
-        if (GROUPED) pagent = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(pagent) + (size_t)pol * in.a.d.pstride);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {  // accumulator lane = cell, column = unit
-            float v[32];
-            if (got) {
-                read_pair((uint32_t)(Cfg::AGENT_COL + Cfg::AGENT_N * c), PL == 2, v);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = 0.f;
-            }
-            const int cell = 128 * c + r;
-            if (cell < C) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 4)
-                    *reinterpret_cast<float4*>(pagent + (size_t)cell * H + 32 * half + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            }
-        }
+        drain_agent(std::integral_constant<int, 32>{}, !LONG || G <= Cfg::AGENT_FIRST, got);  // the last group (or zeros)
     }
     tc::tc_fence_before();
     __syncthreads();
@@ -446,11 +485,21 @@ cudaError_t launch_t(const LearnArgs& a, int nx, float* part_w2, float* part_age
         if (Cfg::PL == 2 && (!map(&maps.lh_lo, h1 + off + RHl, d.B_last, 1) || !map(&maps.ld_lo, dh2 + off + RHl, d.B_last, 1))) return cudaErrorNotSupported;
     }
     const Back64Args in{a, part_w2, part_agent, stride_agent, nx};
-    if (d.npol > 1) {
-        if constexpr (PREC == 0) return launch<k_back64<PREC, NC, true>>(dim3(nx, 1, d.npol), Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
-        return cudaErrorNotSupported;
+    // The restarts cost registers in the tile loop (1024 policies x 64 envs, 8 tiles a CTA: 191 -> 195 us), so launches without a CTA that
+    // needs them do without.  Where they are taken: 131072 envs, 9 cells, T = 60 747 -> 740 us, 25 cells, T = 16 237 -> 229 us, 144
+    // cells, T = 16 303 -> 311 us.
+    const int m_tiles = sp > 1 ? 1 : (d.B + Cfg::BM - 1) / Cfg::BM, steps = (a.T + sp - 1) / sp;
+    const bool many = (m_tiles * a.ts + nx - 1) / nx * ((steps + a.ts - 1) / a.ts) > Cfg::AGENT_FIRST;
+    const dim3 grid(nx, 1, d.npol);
+    if constexpr (PREC == 1) {
+        if (d.npol > 1) return cudaErrorNotSupported;
+        return launch<k_back64<1, NC, false, false>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
+    } else {
+        if (d.npol > 1 && many) return launch<k_back64<0, NC, true, true>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
+        if (d.npol > 1) return launch<k_back64<0, NC, true, false>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
+        if (many) return launch<k_back64<0, NC, false, true>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
+        return launch<k_back64<0, NC, false, false>>(grid, Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
     }
-    return launch<k_back64<PREC, NC, false>>(dim3(nx, 1, 1), Cfg::THREADS, Cfg::smem_bytes, s, maps, in);
 }
 
 }  // namespace

@@ -289,3 +289,27 @@ def test_policies_blobs_outside_the_handles_gpu_go_by_the_runtimes_copies(bnd, n
         assert (an.launch_count() > before) == by_kernel
         assert (an.get(bnd.ENV_POS) == (want + 1).astype(np.uint8)).all()
         an.set(bnd.ENV_POS, want)
+
+
+def test_policies_gradients_of_long_sums(bnd):
+    """Two policies share the 148 CTAs of the fused backward kernel at H = 64: 74 tiles of 128 envs times 97 steps are at least 97 tiles
+    for the busiest of a policy's 74 CTAs, so both accumulators are emptied and restarted on the way (dW2 every 32, the agent plane
+    every 96 tiles).  The last policy is a few envs short."""
+    w = Workload("k2_h64_long", B=2 * 9472 - 50, N=3, H=64, T=97, iters=1, n_policies=2)
+    an = make(bnd, w)
+    an.reset(21)
+    thetas = policy_thetas(w, an.K, seed=31)
+    an.set(bnd.PARAMS, thetas)
+    an.rollout()
+    an.gae()
+    an.learn()
+    walls, goal = an.get(bnd.ENV_WALLS).reshape(w.B, -1), an.get(bnd.ENV_GOAL)
+    ograds, _, reps = orc.learn_policies(an.K, w.N, w.H, 0, w.T, thetas, walls, goal, an.get(bnd.TRAJ_POS), an.get(bnd.TRAJ_ACTION),
+                                         an.get(bnd.ADV), an.get(bnd.RET), np.float32(w.value_coef), np.float32(w.entropy_coef),
+                                         gates=split_gates(an, bnd, w))
+    grads = an.get(bnd.GRADS).reshape(an.K, an.P)
+    for p in range(an.K):
+        assert reps[p]["layer1"]["mismatched"] + reps[p]["layer2"]["mismatched"] <= 10 + 1e-5 * w.B * w.T * w.H
+        for nm, sl in orc.Dims(w.N, w.H).slices().items():
+            par.assert_close(grads[p][sl], ograds[p][sl], par.RTOL_FP32, f"policy {p} grad {nm}")
+    assert an.status() == 0

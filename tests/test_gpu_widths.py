@@ -54,12 +54,13 @@ def test_width_one_iteration_stage_by_stage(bnd, H, prec, B, N, T):
 
 LONG_SUMS = [
     # (H, precision, B, N, T, bias of the value head).  Many rows a CTA: the accumulators of the backward kernels are emptied and
-    # restarted on the way (the agent plane every 48 tiles of 128 rows at H = 128 and 256).  However the tiles are dealt out, one of
+    # restarted on the way (the agent plane every 48 tiles of 128 rows at H = 128 and 256, 96 tiles at 64; dW2 at 64 every 32).  However the tiles are dealt out, one of
     # the 148 CTAs (74 pairs at H = 256) has at least the mean of them.
     # The tensor core rounds toward zero, so a sum that is left in one accumulator is biased, most where nearly every MMA adds to
     # it: four cells, and a value head that is off by 3 (every row pulls the same way).
-    (128, 0, 131072, 2, 96, 3.0),
+    (128, 0, 131072, 2, 96, 3.0), (64, 0, 131072, 2, 160, 3.0),
     (128, 0, 18945, 13, 49, 0.0), (256, 0, 30000, 3, 20, 3.0), (256, 0, 7000, 12, 70, 0.0),
+    (64, 0, 18945, 3, 98, 0.0), (64, 0, 18945, 12, 98, 0.0), (64, 1, 18945, 5, 34, 0.0), (64, 1, 18945, 12, 34, 0.0),
 ]
 
 
