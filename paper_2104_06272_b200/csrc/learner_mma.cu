@@ -1142,6 +1142,11 @@ __global__ void __launch_bounds__(256) k_adam_only(LearnArgs a_in) {
 // G threads share a parameter of the main part (64 or 256 parameters per piece): thread group g adds partials g, g + G, ... in
 // order, then the G sums are added in group order.  One thread per parameter is a chain of ns / 32 memory round trips: with 148
 // to 296 partials per weight (the fused heads + dW2 kernel leaves one per CTA) four threads take a quarter of it.
+// Pieces of one policy's parameters (many policies): W1 and b1, W2, the tail.
+__host__ __device__ inline int w1_pieces(const Dims& d) { return (int)((d.oW2 + 1023) / 1024); }
+__host__ __device__ inline int w2_pieces(const Dims& d) { return d.H * d.H / 1024; }
+__host__ __device__ inline int policy_pieces(const Dims& d) { return w1_pieces(d) + w2_pieces(d) + (int)((d.P - d.ob2 + 255) / 256); }
+
 template <int PREC, bool GROUPED, int G = 1>
 __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_in, int loss_blocks) {
     PDL_START();
@@ -1177,9 +1182,9 @@ __global__ void __launch_bounds__(256) k_reduce_adam2(LearnArgs a_in, size_t R_i
     // Many policies: a thread takes four parameters of the main part (16 loads in flight instead of four), in W1 and b1 four in a row,
     // in W2 the four of an 8-byte element of the fragment copies, so that those leave as whole sectors (1024 policies of 9349
     // parameters: 127 us with one parameter a thread and 2-byte stores).
-    const int nb_w1 = (int)((d.oW2 + 1023) / 1024), nb_w2 = d.H * d.H / 1024;
-    const int nb_main = GROUPED ? nb_w1 + nb_w2 : (int)((d.ob2 + PPB - 1) / PPB);
-    const int nb_total = nb_main + (int)(GROUPED ? (d.P - d.ob2 + 255) / 256 : (d.P - d.ob2 + 7) / 8);
+    const int nb_w1 = w1_pieces(d);
+    const int nb_main = GROUPED ? nb_w1 + w2_pieces(d) : (int)((d.ob2 + PPB - 1) / PPB);
+    const int nb_total = GROUPED ? policy_pieces(d) : nb_main + (int)((d.P - d.ob2 + 7) / 8);
     for (int bx = blockIdx.x; bx < nb_total; bx += gridDim.x) {
         if (GROUPED && bx < nb_main) {
             const bool w2 = bx >= nb_w1;
@@ -1700,7 +1705,12 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         const int grp = most > 48 ? 4 : 1;
         const unsigned nb = (unsigned)((d.ob2 * grp + 255) / 256 + (d.P - d.ob2 + 7) / 8);
         if (d.npol > 1) {
-            const unsigned per_policy = d.npol >= 74 ? (H == 64 ? 6u : 12u) : (nb < 592u / d.npol ? nb : 592u / d.npol);  // (many: two pieces a CTA)
+            // One piece a CTA up to about 48 of them to an SM (six waves of eight), then two to four a CTA, whose loads of one overlap the stores
+            // of the last.  B200, 64 envs each, one / two / four pieces a CTA: 1024 policies at H = 64 on 9, 81, 256 cells (8, 22, 55
+            // pieces) 62 / 60 / 62, 156 / 150 / 150, 412 / 387 / 373 us; 64 policies at H = 128 on 9, 256 cells (24, 117 pieces) 21 / 25 /
+            // 25, 68 / 64 / 66 us; 16 policies at H = 64 on 25 cells 13 / 13 / 17 us.
+            const unsigned pieces = (unsigned)policy_pieces(d), all = pieces * (unsigned)d.npol;
+            const unsigned each = std::min(std::max((all + 16 * 148) / (32 * 148), 1u), 4u), per_policy = (pieces + each - 1) / each;
             if constexpr (PREC == 0) launch<k_reduce_adam2<PREC, true, 1>>(dim3(per_policy, d.npol), 256, 0, s, a, R, pl.loss_blocks);
             else return cudaErrorNotSupported;
         } else {

@@ -313,3 +313,27 @@ def test_policies_gradients_of_long_sums(bnd):
         for nm, sl in orc.Dims(w.N, w.H).slices().items():
             par.assert_close(grads[p][sl], ograds[p][sl], par.RTOL_FP32, f"policy {p} grad {nm}")
     assert an.status() == 0
+
+
+@pytest.mark.parametrize("K,H,N", [(40, 64, 5), (64, 128, 16), (300, 64, 16), (1024, 64, 9)])
+def test_policies_every_parameter_is_reduced_and_stepped_once(bnd, K, H, N):
+    """One, two, three and four pieces of a policy's parameters per CTA of the reduction: gradient, moments and parameters of every policy."""
+    w = Workload(f"k{K}_h{H}_n{N}", B=2 * K - 1, N=N, H=H, T=2, iters=1, n_policies=K)
+    an = make(bnd, w)
+    an.reset(21)
+    thetas = policy_thetas(w, K, seed=31)
+    an.set(bnd.PARAMS, thetas)
+    an.rollout()
+    an.gae()
+    an.learn()
+    walls, goal = an.get(bnd.ENV_WALLS).reshape(w.B, -1), an.get(bnd.ENV_GOAL)
+    ograds, _, _ = orc.learn_policies(K, N, H, 0, w.T, thetas, walls, goal, an.get(bnd.TRAJ_POS), an.get(bnd.TRAJ_ACTION), an.get(bnd.ADV),
+                                      an.get(bnd.RET), np.float32(w.value_coef), np.float32(w.entropy_coef), gates=split_gates(an, bnd, w))
+    grads = an.get(bnd.GRADS).reshape(K, an.P)
+    for nm, sl in orc.Dims(N, H).slices().items():
+        par.assert_close(grads[:, sl], ograds[:, sl], par.RTOL_FP32, f"grad {nm}")
+    theta, m, v = thetas.reshape(-1).copy(), np.zeros(K * an.P, np.float32), np.zeros(K * an.P, np.float32)
+    orc.adam(theta, grads.reshape(-1), m, v, 1, np.float32(w.lr), np.float32(w.adam_b1), np.float32(w.adam_b2), np.float32(w.adam_eps))
+    for which, want in ((bnd.ADAM_M, m), (bnd.ADAM_V, v), (bnd.PARAMS, theta)):
+        par.assert_close(an.get(which), want, par.RTOL_FP32, f"blob {which}")
+    assert an.status() == 0
