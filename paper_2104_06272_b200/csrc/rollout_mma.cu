@@ -548,12 +548,14 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
         if (!a.replay && ctas <= 148 && smem + w1 <= MAX_DYN_SMEM) return launch<k_rollout_mma<H, NW, PREC, false, 1, true, false, 32, true>>(grid, NW * 32 + 32, smem + w1, s, a);
     // The owner warp costs a CTA of the 128-wide kernel its second place on an SM: only where every CTA gets an SM of its own.
     // (H = 64: three CTAs per SM where there are that many)
-    // ... in fp32 with the agent rows of W1 beside them where the steps gather many times what the load takes and the GPU is full more
-    // than once (B200: 44158 envs, 100 cells, T = 45 425 -> 390 us, 30000 envs, 81 cells, T = 16 124 -> 113 us; but 104889 envs, 81
-    // cells, T = 6 145 -> 147 us, 12000 envs 76.4 -> 77.6 us, bf16 44158 envs 333 -> 345 us)
+    // ... in fp32 with the agent rows of W1 beside them where the GPU is full more than once and the rollout is ten steps or longer: a CTA
+    // loads them once and gathers from them every step.  B200, gather from shared memory / from L2, 14300 to 131072 envs on 9 to 121 cells:
+    // T = 2, 4 0.99 to 1.13, T = 6, 8 0.92 to 1.05, T = 12 0.90 to 0.98, T = 16 to 64 0.85 to 1.00 of the time, whatever the board (30000
+    // envs, 81 cells, T = 16: 128 -> 116 us).  Up to 444 CTAs 0.94 to 1.08 without a pattern; bf16 loses (44158 envs, T = 45: 333 ->
+    // 345 us).
     if constexpr (H == 64 && PREC == 0) {
         const size_t w1b = (size_t)a.d.C * H * 4;
-        if (!a.replay && (size_t)grid.x * grid.y > 444 && a.T * Cfg::ME >= 6 * a.d.C && smem + w1b <= 75 * 1024)
+        if (!a.replay && (size_t)grid.x * grid.y > 444 && a.T >= 10 && smem + w1b <= 75 * 1024)
             return launch<k_rollout_mma<H, NW, PREC, GROUPED, 3, true, false, 32, true>>(grid, NW * 32 + 32, smem + w1b, s, a);
     }
     if constexpr (H == 64)
