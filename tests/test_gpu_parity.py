@@ -3,6 +3,10 @@
 Stages are teacher-forced: one flipped action would send a free-running comparison down a different
 trajectory, so each stage of the library is fed to the oracle and compared there.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -528,3 +532,41 @@ def test_asynchronous_copies_through_page_locked_host_memory(bnd):
     assert np.array_equal(an.get(bnd.PARAMS), src.numpy())
     with pytest.raises(bnd.AnakinError):
         an._ck(bnd._lib.anakin_get(an._h, bnd.PARAMS, bufs[bnd.PARAMS].data_ptr(), bufs[bnd.PARAMS].numel() * 4, 3))
+
+
+_THREADS = """
+import threading
+import numpy as np, torch
+from paper_2104_06272_b200 import binding as bnd
+
+torch.zeros(1, device="cuda")
+SHAPES = [(256, 0), (128, 0), (64, 0), (512, 1), (384, 0), (96, 0), (256, 1), (1024, 1)]
+go, out = threading.Barrier(len(SHAPES)), {}
+
+def work(i, H, prec, wait):
+    an = bnd.Anakin(bnd.make_cfg(300, 6, H, 4, precision=prec), stream=torch.cuda.Stream())
+    an.reset(i)
+    if wait:
+        go.wait()
+    an.run(2)
+    got = an.get(bnd.PARAMS), an.status()
+    out.setdefault(i, []).append(got)
+
+ts = [threading.Thread(target=work, args=(i, H, p, True)) for i, (H, p) in enumerate(SHAPES)]
+for t in ts: t.start()
+for t in ts: t.join()
+for i, (H, p) in enumerate(SHAPES): work(i, H, p, False)
+for i in range(len(SHAPES)):
+    (a, sa), (b, sb) = out[i]
+    assert sa == sb == 0 and (a.view(np.uint32) == b.view(np.uint32)).all(), (i, SHAPES[i])
+print("ok")
+"""
+
+
+def test_handles_in_their_own_threads_and_streams_give_what_they_give_alone():
+    """Different handles are independent: the first calls of a process from eight threads at once (what the library sets up once per
+    process or device among them), each on a handle and a stream of its own, against the same work done one after the other."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _THREADS], env={**os.environ, "PYTHONPATH": root}, cwd=root, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stderr
