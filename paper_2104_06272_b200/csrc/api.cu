@@ -110,12 +110,16 @@ size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* o
     // wide layers: bf16 planes of h1 (three exact terms in fp32 workloads) with room for the bootstrap step's rows; h2 likewise
     b.h1 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 6 : 2) : R * H * (x3 ? 6 : 4));
     b.gate1 = (dh1_agent_tc_supported(d) && policies_of(c) <= 1) ? (uint8_t*)take(R * (H / 8)) : nullptr;  // what the fused dh1 kernel gates with
-    b.h2 = (float*)take(wide ? wide_h1_rows(d) * H * (f32 ? 4 : 2) : R * H * 4);
+    // dh1 of the widths where it leaves the chip lies over h2: the heads kernel is the last to read h2 (its 16-bit planes, dh2, are what
+    // follows), and an update ends with the saved activations marked as gone.  On the wide path the buffer is also where the operands of
+    // the base GEMM go, which runs before a forward pass fills h2.
+    const bool dh1_on_chip = H == 64 || (dh1_agent_tc_supported(d) && policies_of(c) <= 1);
+    const size_t h2_bytes = wide ? wide_h1_rows(d) * H * (f32 ? 4 : 2) : R * H * 4;
+    b.h2 = (float*)take(wide ? std::max(h2_bytes, wide_scratch_bytes(d)) : h2_bytes);
     b.out5 = (float*)take(R * 8 * 4);
     b.vboot = (float*)take(B * 4);
     b.dh2 = (float*)take(R * H * (x3 ? 6 : wide ? 2 : 4));
-    const bool dh1_on_chip = H == 64 || (dh1_agent_tc_supported(d) && policies_of(c) <= 1);
-    b.dh1 = dh1_on_chip ? nullptr : (float*)take(!wide ? R * H * 4 : std::max(R * H * (f32 ? 4 : 2), wide_scratch_bytes(d)));
+    b.dh1 = dh1_on_chip ? nullptr : b.h2;
     // t-slices of two 16-bit planes, or three planes
     b.S = (float*)take((dh1_on_chip ? (size_t)most_s_rows((int)B) : 4 * B) * H * 4);
     LearnPlan pl;
@@ -362,11 +366,6 @@ int anakin_gae(anakin_t* h) {
 // The update proper, from ADV/RET as they stand.  phase 0: through Adam; phase 1: stop at the batch-mean gradient.
 static int learn_after_gae(anakin_t* h, int phase, float ppo_clip = 0.f, bool consume = true) {
     cudaError_t e;
-    if (!h->base_valid) {
-        e = launch_env_base(h->d, h->b, h->ctx());
-        if (e != cudaSuccess) return fail_cuda(h, e);
-        h->base_valid = true;
-    }
     if (!h->frags_valid) {
         e = pack_w2(h);
         if (e != cudaSuccess) return fail_cuda(h, e);
@@ -453,17 +452,6 @@ int anakin_learn_vtrace(anakin_t* h, int epochs, float rho_bar, float c_bar) {
     const bool offered = H == 64 || H == 128 || H == 256 || (h->cfg.precision == ANAKIN_PRECISION_BF16 && (H == 512 || H == 1024));
     if (h->K > 1 || !offered) return ANAKIN_E_UNSUPPORTED_CFG;
     for (int ep = 0; ep < epochs; ++ep) {
-        cudaError_t e;
-        if (!h->base_valid) {
-            e = launch_env_base(h->d, h->b, h->ctx());
-            if (e != cudaSuccess) return fail_cuda(h, e);
-            h->base_valid = true;
-        }
-        if (!h->frags_valid) {
-            e = pack_w2(h);
-            if (e != cudaSuccess) return fail_cuda(h, e);
-            h->frags_valid = true;
-        }
         // Head outputs of the recorded rows under the current parameters: the rollout's own when nothing has changed since
         // (then the recorded bootstrap row is the current one too), else a replay that also evaluates the final state.
         const float* boot = h->b.tval + (size_t)h->last_T * h->d.B;
@@ -472,7 +460,7 @@ int anakin_learn_vtrace(anakin_t* h, int epochs, float rho_bar, float c_bar) {
             if (rc != ANAKIN_OK) return rc;
             boot = h->b.vboot;
         }
-        e = launch_vtrace(h->d, h->b, h->last_T, h->cfg.gamma, rho_bar, c_bar, boot, h->ctx());
+        const cudaError_t e = launch_vtrace(h->d, h->b, h->last_T, h->cfg.gamma, rho_bar, c_bar, boot, h->ctx());
         if (e != cudaSuccess) return fail_cuda(h, e);
         h->adv_valid = true;
         const int rc = learn_after_gae(h, 0, 0.f, ep == epochs - 1);

@@ -1598,6 +1598,12 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
                 return cudaErrorNotSupported;
         }
     }
+    if (b.dbg_gates) {  // (before the backward kernels: dh1 goes over h2)
+        Scope sc(c, K_PACK_GATES);
+        if (d.npol > 1) launch<k_pack_gates2<true>>(dim3(64, d.npol), 256, 0, s, DimsBuffers{d, b}, R, 0);
+        else launch<k_pack_gates2<false>>(148 * 8, 256, 0, s, DimsBuffers{d, b}, R, wide && PREC == 1 ? 1 : 0);
+        CK(cudaGetLastError());
+    }
     a.ts = 1;  // slices of the steps (rows of S per env)
     bool fused_agent = false;  // dh1, S and the agent plane of dW1 in one kernel (dh1 stays on chip)
     const bool back64 = H == 64;  // ... and dW2 too
@@ -1717,12 +1723,6 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
             if (grp > 1) launch<k_reduce_adam2<PREC, false, 4>>(nb, 256, 0, s, a, R, pl.loss_blocks);
             else launch<k_reduce_adam2<PREC, false, 1>>(nb, 256, 0, s, a, R, pl.loss_blocks);
         }
-        CK(cudaGetLastError());
-    }
-    if (b.dbg_gates) {
-        Scope sc(c, K_PACK_GATES);
-        if (d.npol > 1) launch<k_pack_gates2<true>>(dim3(64, d.npol), 256, 0, s, DimsBuffers{d, b}, R, 0);
-        else launch<k_pack_gates2<false>>(148 * 8, 256, 0, s, DimsBuffers{d, b}, R, wide && PREC == 1 ? 1 : 0);
         CK(cudaGetLastError());
     }
     return cudaSuccess;

@@ -525,7 +525,7 @@ size_t wide_h1_rows(const Dims& d) { return (size_t)d.B * d.Tmax + d.B; }
 // times the K: the smallest term's rows first, X repeated.  cudaErrorNotSupported for the
 // buffers of other paths and for small batches, where the gather kernel's single launch is quicker (B H = 2^20: 11 us each): up to the
 // sizes that act without a workspace, which has no room for the operands, so that both give the same bits.
-// Uses the dh1 buffer, which is dead outside the update, as scratch for the operands.
+// Uses the dh1 buffer (the one h2 is in) as scratch for the operands: base is computed ahead of the forward passes that fill it.
 cudaError_t launch_env_base_wide(const Dims& d, const Buffers& b, const Ctx& c) {
     if (!b.w2p_hi || !wide_supported(d.H, 0) || (size_t)d.B * d.H <= ANAKIN_NOALLOC_MAX_BH) return cudaErrorNotSupported;
     const bool f32 = is_f32(b);

@@ -115,3 +115,17 @@ def test_binding_fails_loudly_without_the_library(tmp_path):
         shutil.copy(os.path.join(ROOT, "paper_2104_06272_b200", f), pkg / f)
     r = subprocess.run([sys.executable, "-c", "import paper_2104_06272_b200.binding"], cwd=tmp_path, capture_output=True, text=True)
     assert r.returncode != 0 and "libanakin.so is missing" in r.stderr and "no CPU or PyTorch fallback" in r.stderr
+
+
+@pytest.mark.parametrize("H,precision,n_policies,per", [
+    (32, 0, 0, 16), (96, 0, 0, 16), (512, 0, 0, 16), (1024, 0, 0, 16),   # h1 and dh2 as three 16-bit terms, h2 / dh1 fp32
+    (96, 1, 0, 12), (192, 1, 0, 12), (512, 1, 0, 6), (1024, 1, 0, 6),    # bf16: one plane each on the wide path
+    (64, 0, 0, 12), (128, 0, 0, 12.125), (256, 0, 0, 12.125), (256, 1, 0, 12.125), (128, 0, 64, 12),  # dh1 on chip, or over h2; a gate bit
+])
+def test_workspace_holds_one_buffer_for_h2_and_dh1(bnd, H, precision, n_policies, per):
+    """Bytes per recorded row and hidden unit at a size where nothing else counts for much: the rest (trajectory, head outputs, S, partials,
+    parameters) is bounded by a tenth of it plus 96 bytes a row and eight steps' worth of rows."""
+    B, T = 32768, 128
+    got = bnd.workspace_bytes(bnd.make_cfg(B, 5, H, T, precision=precision, n_policies=n_policies))
+    rows = B * T * H * per
+    assert rows <= got <= 1.1 * rows + 96 * B * T + 8 * B * H * per
