@@ -392,18 +392,36 @@ bool three_terms(int H, int prec);             // fp32 operands as three bf16 te
 bool rollout_uses_fragments(int H, int prec);  // the warp-level kernel (and with it the fragment copies of W2) serves this shape
 cudaError_t launch_rollout_tc128(const RolloutArgs& a, int prec, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, large batches); cudaErrorNotSupported otherwise
 cudaError_t launch_rollout_pair2(const RolloutArgs& a, int prec, cudaStream_t s);  // two env groups per CTA pair (H = 256, large batches); cudaErrorNotSupported otherwise
-// Slices of a replay (grid.y) for kernels of one CTA per SM: its steps are independent, so few CTAs take fewer steps each, at least
-// two.  The number that takes the fewest steps over all waves, with one more per slice for the weights' load; none empty.
-inline int replay_slices(const RolloutArgs& a, int ctas) {
+// Slices of a replay (grid.y) for a kernel of per_sm CTAs to an SM: its steps are independent, so few CTAs take fewer steps each, at
+// least two.  The number whose last CTA ends first, a CTA taking its steps and one more for the weights' load; none empty.  With several
+// such the smallest for the tcgen05 kernels (H = 256 in bf16, 6000 envs, T = 5: 32.7 us in one, 34.8 in two or three), the largest
+// for the warp-level ones (H = 192, 3000 envs, T = 5: 45 us in one, 41 in two or three).  (A rule that only asked for enough CTAs, with
+// no look at the last wave: H = 192, 3000 envs, T = 64 450 -> 317 us; H = 96, 12000 envs, T = 33 312 -> 221 us; H = 64, 30000 envs,
+// T = 64 428 -> 368 us.)
+inline int replay_slices(const RolloutArgs& a, int ctas, int per_sm = 1, bool largest = false) {
     if (!a.replay) return 1;
-    const int steps = a.T + (a.replay == 2 ? 1 : 0);
+    const int steps = a.T + (a.replay == 2 ? 1 : 0), slots = 148 * per_sm;
+    // CTAs are placed slice by slice: those of `l` steps fill `waves` waves and `rem` slots of another, then come `ctas` shorter ones
+    auto end_of = [&](int n, int l) {
+        const long long full = (long long)(n - 1) * ctas, waves = full / slots, rem = full % slots;
+        const int L = l + 1, S = steps - (n - 1) * l + 1;
+        long long t = waves * L + (ctas + slots - 1) / slots * S;  // (not before: with all slots free at once)
+        for (;;) {  // the next time at which a slot of either kind ends a CTA
+            const long long early = (t - waves * L) / S, late = t > (waves + 1) * L ? (t - (waves + 1) * L) / S : 0;
+            if ((slots - rem) * early + rem * late >= ctas) break;
+            const long long e = waves * L + (early + 1) * S, f = (waves + 1) * L + (late + 1) * S;
+            t = rem == 0 || e < f ? e : f;
+        }
+        return rem > 0 && t < (waves + 1) * L ? (waves + 1) * L : t;
+    };
     long long best = 1ll << 60;
     int len = steps;
-    for (int n = 1; n <= 16 || n <= 148 / ctas; ++n) {
+    for (int n = 1; n <= 16 || n <= slots / ctas; ++n) {
         const int l = (steps + n - 1) / n;
         if (l < 2 && n > 1) break;
-        const long long t = (long long)(((long long)n * ctas + 147) / 148) * (l + 1);
-        if (t < best) { best = t; len = l; }
+        if ((n - 1) * l >= steps) continue;  // (an empty last slice: fewer slices of the same length do)
+        const long long t = end_of(n, l);
+        if (t < best || (largest && t == best)) { best = t; len = l; }
     }
     return (steps + len - 1) / len;
 }

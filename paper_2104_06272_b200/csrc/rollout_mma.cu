@@ -534,12 +534,7 @@ static cudaError_t launch_t(const RolloutArgs& a0, cudaStream_t s) {
         smem += Cfg::gae_bytes(a.T);
     }
     const int ctas = (a.d.B + Cfg::ME - 1) / Cfg::ME;
-    int slices = 1;
-    if (a.replay && !GROUPED) {  // independent steps: enough CTAs for every SM (two per SM up to H = 128), at least two steps each
-        const int want = (H <= 128 ? 2 : 1) * 148, steps = a.T + (a.replay == 2 ? 1 : 0);
-        slices = (want + ctas - 1) / ctas;
-        if (slices > (steps + 1) / 2) slices = (steps + 1) / 2;
-    }
+    const int slices = GROUPED ? 1 : replay_slices(a, ctas, H <= 32 ? 4 : H <= 64 ? 3 : H <= 128 ? 2 : 1 /*as many as an SM holds*/, true);
     const dim3 grid(ctas, GROUPED ? a.d.npol : slices);
     // Three-term operands at H = 96, a CTA to an SM: the registers of a whole SM, and the agent rows of W1 (B200, T = 16, 4736 envs:
     // 70 -> 48 us; the other widths and bf16 gain nothing from these rows, their gathers hide behind twice the MMAs).

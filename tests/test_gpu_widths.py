@@ -86,7 +86,8 @@ def test_gradients_of_long_sums(bnd, H, prec, B, N, T, bias):
 
 
 @pytest.mark.parametrize("H,prec,B,T", [(32, 0, 40, 7), (64, 0, 33, 9), (96, 1, 70, 5), (128, 0, 65, 11), (128, 1, 200, 4), (256, 0, 127, 6), (256, 0, 300, 9),
-                                        (256, 1, 129, 7), (384, 0, 70, 5)])
+                                        (256, 1, 129, 7), (384, 0, 70, 5), (32, 0, 3000, 17), (64, 0, 6000, 9), (96, 1, 3000, 16), (192, 0, 1500, 16),
+                                        (192, 1, 5000, 3)])
 def test_replayed_forward_pass_equals_the_rollouts_own(bnd, H, prec, B, T):
     """The update of a trajectory handed back through set() recomputes the forward pass in slices of steps (few envs), and must
     give the gradient of the update that reuses the rollout's activations."""
