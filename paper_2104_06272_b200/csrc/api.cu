@@ -99,10 +99,10 @@ size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* o
     b.dbg_gates = c.debug_logits ? (uint32_t*)take(2 * R * (H / 32) * 4) : nullptr;
     b.base = (float*)take(B * H * 4);
     const bool mma = rollout_mma_supported(d.H);
-    const bool frags = mma && rollout_uses_fragments(d.H, c.precision);
+    const bool frags = mma && rollout_uses_fragments(d.H);
     b.w2f_hi = frags ? (uint2*)take(H * H * 2) : nullptr;
     b.w2f_lo = frags ? (uint2*)take(H * H * 2) : nullptr;
-    const bool wide = wide_supported(d.H, c.precision), f32 = c.precision == ANAKIN_PRECISION_FP32;
+    const bool wide = wide_supported(d.H), f32 = c.precision == ANAKIN_PRECISION_FP32;
     const bool x3 = three_terms(d.H, c.precision);
     b.w2f_lo2 = frags && x3 ? (uint2*)take(H * H * 2) : nullptr;
     b.w2p_hi = (uint16_t*)take(H * H * 2 * (x3 ? 3 : 1));
@@ -186,7 +186,7 @@ size_t blob_total(anakin_t* h, int which) {
 
 // 16-bit copies of W2 in the layouts the tensor-core kernels read.
 cudaError_t pack_w2(anakin_t* h) {
-    if (wide_supported(h->d.H, h->cfg.precision)) return launch_pack_w2_wide(h->d, h->b, h->ctx());
+    if (wide_supported(h->d.H)) return launch_pack_w2_wide(h->d, h->b, h->ctx());
     return launch_pack_w2(h->d, h->b, h->cfg.precision, h->ctx());
 }
 
@@ -255,7 +255,7 @@ int replay_activations(anakin_t* h, bool with_boot = false) {
     a.replay = with_boot ? 2 : 1;
     a.fuse_gae = 0;
     a.gamma = a.lambda = 0.f;
-    if (wide_supported(h->d.H, h->cfg.precision)) {
+    if (wide_supported(h->d.H)) {
         e = launch_rollout_wide(a, h->ctx());
     } else {
         Scope sc(h->ctx(), K_REPLAY);

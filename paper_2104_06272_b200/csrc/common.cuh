@@ -389,7 +389,7 @@ cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c);
 cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s);  // cudaErrorNotSupported if not covered
 bool rollout_mma_supported(int H);
 bool three_terms(int H, int prec);             // fp32 operands as three bf16 terms instead of two fp16 terms
-bool rollout_uses_fragments(int H, int prec);  // the warp-level kernel (and with it the fragment copies of W2) serves this shape
+bool rollout_uses_fragments(int H);  // the warp-level kernel (and with it the fragment copies of W2) serves this shape
 cudaError_t launch_rollout_tc128(const RolloutArgs& a, int prec, cudaStream_t s);  // two-group tcgen05 rollout (H = 128, large batches); cudaErrorNotSupported otherwise
 cudaError_t launch_rollout_pair2(const RolloutArgs& a, int prec, cudaStream_t s);  // two env groups per CTA pair (H = 256, large batches); cudaErrorNotSupported otherwise
 // Slices of a replay (grid.y) for a kernel of per_sm CTAs to an SM: its steps are independent, so few CTAs take fewer steps each, at
@@ -427,7 +427,7 @@ inline int replay_slices(const RolloutArgs& a, int ctas, int per_sm = 1, bool la
 }
 cudaError_t launch_rollout_pair(const RolloutArgs& a, int prec, cudaStream_t s);  // CTA-pair tcgen05 rollout (H = 256); cudaErrorNotSupported otherwise
 cudaError_t noalloc_wide_scratch(Buffers* b);  // acting without a workspace: h1, h2 and W2's planes of the wide layers
-bool wide_supported(int H, int prec);         // hidden layer too wide for the persistent rollouts (either precision)
+bool wide_supported(int H);                   // hidden layer too wide for the persistent rollouts (either precision)
 size_t wide_h1_rows(const Dims& d);           // rows of one h1 / h2 plane on that path: the recorded ones and the bootstrap step's
 size_t wide_scratch_bytes(const Dims& d);     // operands of the base GEMM (kept in the dh1 buffer)
 int agent_plane_splits(const Dims& d);

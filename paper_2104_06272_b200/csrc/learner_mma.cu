@@ -1430,10 +1430,7 @@ static int env_splits(const Dims& d, int rows) {
 }
 
 // dW2 inside the heads kernel: hidden width 128 or 256, one policy.
-static bool heads_fuse_dw2(const Dims& d, size_t R, int heads_grid, int prec) {
-    (void)R; (void)prec;
-    return (d.H == 128 || d.H == 256) && d.npol <= 1 && heads_grid >= 1;
-}
+static bool heads_fuse_dw2(const Dims& d) { return (d.H == 128 || d.H == 256) && d.npol <= 1; }
 
 // dW2 with three-term operands: 128 x 128 tiles, one wave of CTAs, ranges of at least 256 rows.
 static int x3_w2_splits(int H, size_t R) {
@@ -1483,7 +1480,7 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     if (d.npol > 1) hg = (size_t)std::max(4 * heads_grid_max(H) / d.npol, 1);  // many policies: the CTAs of all policies fill the GPU together
     p->heads_grid = (int)(tiles32 < hg ? tiles32 : hg);
     // (the fused heads + dW2 kernel writes one dW2 partial per CTA: room for the larger of the two partial counts)
-    int w2_slots = heads_fuse_dw2(d, R, p->heads_grid, 1) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;
+    int w2_slots = heads_fuse_dw2(d) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;
     if (three_terms(H, 0) && x3_w2_splits(H, R) > w2_slots) w2_slots = x3_w2_splits(H, R);
     p->ns_small = p->heads_grid;
     p->small_stride = (size_t)6 * H + 8;
@@ -1546,7 +1543,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const int H = d.H, C = d.C, B = d.B, T = a.T;
     const size_t R = (size_t)B * T, RH = (size_t)B * d.Tmax * H;
     cudaStream_t s = c.s;
-    const bool wide = wide_supported(H, PREC);  // bf16 activations in HBM, layer-2 products as large tcgen05 GEMMs
+    const bool wide = wide_supported(H);  // bf16 activations in HBM, layer-2 products as large tcgen05 GEMMs
     // many policies: every kernel gets one grid slice per policy and moves its workspace pointers there; the tcgen05
     // kernels bake addresses into tensor maps, so this path stays on the warp-level kernels
     const bool grouped = d.npol > 1;
@@ -1567,7 +1564,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     a.reg[7] = PartRegion{b.part + pl.off_small + (size_t)6 * H, pl.ns_small, pl.small_stride, d.obh};
 
     // dW2 = h1^T dh2 rides in the heads kernel where its rows per CTA allow (it then has one partial per heads CTA)
-    const bool fuse_dw2 = !wide && !grouped && b.w2p_hi != nullptr && heads_fuse_dw2(d, R, pl.heads_grid, PREC);
+    const bool fuse_dw2 = heads_fuse_dw2(d);
     if (fuse_dw2) a.reg[4].ns = pl.heads_grid;
     {
         Scope sc(c, K_HEADS_BWD);

@@ -100,7 +100,7 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
         b.w2f_lo = reinterpret_cast<uint2*>(frag + plane);
         b.w2f_lo2 = reinterpret_cast<uint2*>(frag + 2 * plane);
     } else if (rollout_mma_supported(cfg->H)) {  // same kernel choice as the handle-based rollout
-        if (rollout_uses_fragments(cfg->H, cfg->precision)) {
+        if (rollout_uses_fragments(cfg->H)) {
             b.w2f_hi = reinterpret_cast<uint2*>(frag);
             b.w2f_lo = reinterpret_cast<uint2*>(frag + kW2FragBytes / 2);
         }
@@ -124,7 +124,7 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
     uint64_t launches = 0;
     const Ctx ctx{s, &launches, nullptr};
     if (launch_env_base(a.d, b, ctx) != cudaSuccess) return ANAKIN_E_CUDA;  // fills `base`: nothing of the last call survives
-    if (wide_supported(cfg->H, cfg->precision)) {
+    if (wide_supported(cfg->H)) {
         if (noalloc_wide_scratch(&b) != cudaSuccess) return ANAKIN_E_CUDA;
         a.d.Tmax = 0;  // the activations of one step
         if (launch_pack_w2_wide(a.d, b, ctx) != cudaSuccess) return ANAKIN_E_CUDA;

@@ -67,7 +67,7 @@ cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c) {
 }
 
 cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
-    if (wide_supported(a.d.H, prec)) return launch_rollout_wide(a, c);  // two launches per step
+    if (wide_supported(a.d.H)) return launch_rollout_wide(a, c);  // two launches per step
     Scope sc(c, K_ROLLOUT);
     return launch_rollout_mma(a, prec, c.s);
 }

@@ -567,7 +567,7 @@ bool rollout_mma_supported(int H) { return H == 32 || H == 64 || H == 96 || H ==
 // fp32 operands as three exact bf16 terms (the widths beside 64, 128 and 256, which take two fp16 terms).
 bool three_terms(int H, int prec) { return prec == 0 && !(H == 64 || H == 128 || H == 256); }
 // H = 256 runs the CTA-pair tcgen05 kernels, which read the row-major planes of W2 only.
-bool rollout_uses_fragments(int H, int prec) { (void)prec; return rollout_mma_supported(H) && H != 256; }
+bool rollout_uses_fragments(int H) { return rollout_mma_supported(H) && H != 256; }
 
 // Returns cudaErrorNotSupported when the shape is not covered by the tensor-pipe kernel.
 cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s) {

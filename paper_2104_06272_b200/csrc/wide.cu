@@ -23,7 +23,7 @@
 namespace anakin {
 
 // Hidden layers too wide for the persistent rollouts, in either precision (bf16 at 512 / 1024 is the headline form).
-bool wide_supported(int H, int prec) { (void)prec; return H == 384 || H == 512 || H == 768 || H == 1024; }
+bool wide_supported(int H) { return H == 384 || H == 512 || H == 768 || H == 1024; }
 
 namespace {
 
@@ -527,7 +527,7 @@ size_t wide_h1_rows(const Dims& d) { return (size_t)d.B * d.Tmax + d.B; }
 // sizes that act without a workspace, which has no room for the operands, so that both give the same bits.
 // Uses the dh1 buffer (the one h2 is in) as scratch for the operands: base is computed ahead of the forward passes that fill it.
 cudaError_t launch_env_base_wide(const Dims& d, const Buffers& b, const Ctx& c) {
-    if (!b.w2p_hi || !wide_supported(d.H, 0) || (size_t)d.B * d.H <= ANAKIN_NOALLOC_MAX_BH) return cudaErrorNotSupported;
+    if (!b.w2p_hi || !wide_supported(d.H) || (size_t)d.B * d.H <= ANAKIN_NOALLOC_MAX_BH) return cudaErrorNotSupported;
     const bool f32 = is_f32(b);
     const int Cp = (d.C + 63) / 64 * 64, terms = f32 ? 3 : 1;
     uint16_t* X = reinterpret_cast<uint16_t*>(b.dh1);
