@@ -1,18 +1,19 @@
-// Wide-network path (bf16 workload, hidden width 512 / 1024 / 2048): the layer-2 products of the Anakin minimal unit
+// Wide-network path (hidden widths 384, 512, 768, 1024, both precisions): the layer-2 products of the Anakin minimal unit
 // (Podracer paper, Section 3.1; Figure 2, top) as large GEMMs on the 5th-generation tensor cores.
 //
-// With a hidden layer this wide W2 no longer fits on chip next to a CTA's activations, so the acting half runs as three
-// launches per environment step instead of one persistent kernel:
-//   k_h1_wide      h1 = bf16(relu(base[env] + W1[agent row]))                  gather-add, HBM-bound
-//   k_gemm_nt_tc   h2 = bf16(relu(h1 W2 + b2))                                 tcgen05, persistent, bias/ReLU epilogue
-//   k_heads_wide   out = h2 Wh + bh, then softmax / Philox sample / env step   warp per env, then thread per env
-// h1 and h2 of every recorded row stay in HBM as bf16 for the update, which calls k_gemm_nt_tc once more for
-// dh1 = (dh2 W2^T) gated by h1 > 0 over all B*T rows, and k_sum_t_wide for S = sum over t of dh1.
+// With a hidden layer this wide W2 no longer fits on chip next to a CTA's activations, so the acting half runs as two
+// launches per environment step instead of one persistent kernel, after one for the first step's h1:
+//   k_h1_wide      h1 = relu(base[env] + W1[agent row])                        gather-add, HBM-bound (first step, replays)
+//   GEMM           h2 = relu(h1 W2 + b2)                                       tcgen05, persistent, bias/ReLU epilogue
+//   k_heads_wide   out = h2 Wh + bh, softmax / Philox sample / env step, then h1 of the next step
+// h1 and h2 of every recorded row stay in HBM for the update, which runs the GEMM once more for dh1 = (dh2 W2^T) gated by
+// h1 > 0 over all B*T rows.  In bf16 the GEMM is k_gemm_nt_tc (below) or the CTA-pair kernel (wide2.cu), activations are one bf16
+// plane and k_sum_t_wide forms S = sum over t of dh1; fp32 runs x3_gemm.cu on three bf16 terms and k_agent_plane for S.
 //
 // k_gemm_nt_tc: C[m][n] = sum_k A[m][k] Bop[k][n] with A row-major (K-major for the MMA).  One persistent CTA per SM walks
 // 128 x 256 output tiles (n fastest, so that the CTAs running together share A tiles through L2):
 //   warp 0 (one lane)  TMA producer: 64-wide k chunks of A (128 rows) and B (256 columns) into a 3-stage ring
-//   warp 1 (one lane)  tcgen05.mma issuer, four k16 MMAs per chunk into one of two 256-column fp32 accumulators in TMEM
+//   warp 1             tcgen05.mma issuer (the whole warp walks the loop, an elected lane issues), four k16 MMAs per chunk into one of two 256-column fp32 accumulators in TMEM
 //   warps 2-9          epilogue of tile i while the MMAs of tile i+1 run: tcgen05.ld, bias + ReLU (or gate), bf16, store
 // B is either K-major (rows = n: W2 as stored, for dh2 W2^T) or MN-major (rows = k: W2 as stored, for h1 W2).
 // Every wait is bounded; a timeout raises DEV_E_WAIT_TIMEOUT and the CTA unwinds (tensor memory freed).
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(256) k_h1_wide(Dims d, Buffers b, const uint8_
     }
 }
 
-// Heads, sampling and env step for RW = 32 or 8 rows per CTA (eight where 32 would leave SMs without a CTA: a step is a
+// Heads, sampling and env step for HW_ROWS = 32 or 8 rows per CTA (eight where 32 would leave SMs without a CTA: a step is a
 // dependent launch, so its latency counts): eight warps share the rows for the head products, then warp 0
 // takes one row per lane for the per-env part (its env state and wall words were requested at kernel start).
 //   mode 0: step t of the rollout (row = env): saves the head outputs and the value, samples, steps the env, records.
@@ -265,10 +266,11 @@ __global__ void __launch_bounds__(256, HW_ROWS >= 16 && H >= 768 ? 4 : 5) k_head
         }
     }
     const uint16_t* h2b = reinterpret_cast<const uint16_t*>(b.h2);
-    // A warp walks rows wid, wid + 8, ...; WIN trips of h2 are in flight.  The widest layers take two rows at a time, so that a piece of
-    // Wh read from shared memory serves both (B200, H = 1024: 16384 rows in bf16 37.8 -> 32.2 us, 12000 in fp32 33.1 -> 28.8 us; below
-    // H = 768 the registers cost the fifth CTA per SM, 22.5 -> 23.7 us for 20000 rows of 512 in bf16).
-    constexpr int RB = HW_ROWS >= 16 && H >= 768 ? 2 : 1, WIN = RB == 2 && F32 ? (TRIPS % 2 == 0 ? 2 : 3) : TRIPS % 4 == 0 ? 4 : 3;
+    // A warp walks rows wid, wid + 8, ...; WIN trips of h2 are in flight.  In CTAs of 32 rows it takes two at a time, so that a piece of
+    // Wh read from shared memory serves both (B200, one row / two: bf16 H = 1024, 16384 rows 39.8 / 34.8 us, 768 32.5 / 27.4, 512, 20000
+    // rows 26.6 / 22.8, 384 21.4 / 18.0; fp32 H = 1024, 12000 rows 39.4 / 34.2).  In fp32 below 768 the second row's registers cost
+    // what it gains in the largest batches (H = 512, 12000 rows 24.2 / 22.4, 120000 rows 138.8 / 142.0), so those keep one.
+    constexpr int RB = HW_ROWS >= 16 && (H >= 768 || !F32) ? 2 : 1, WIN = RB == 2 && F32 ? (TRIPS % 2 == 0 ? 2 : 3) : TRIPS % 4 == 0 ? 4 : 3;
     using H2x4 = typename std::conditional<F32, float4, uint2>::type;  // four consecutive units of h2: fp32, or bf16
     static_assert(TRIPS % WIN == 0, "a trip keeps its slot from one pass to the next");
     H2x4 v[WIN][RB];

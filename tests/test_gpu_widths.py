@@ -12,6 +12,7 @@ CASES = [
     # (H, precision, B, N, T)
     (384, 0, 3, 3, 2), (384, 0, 129, 11, 5), (384, 1, 77, 5, 4), (512, 0, 70, 8, 6), (512, 0, 2049, 7, 3), (768, 0, 33, 16, 3),
     (768, 1, 257, 6, 3), (1024, 0, 130, 9, 2), (1024, 0, 1025, 4, 2), (1024, 1, 9, 7, 3), (384, 0, 9500, 3, 2),
+    (384, 1, 9500, 3, 2), (512, 1, 9473, 4, 2), (768, 0, 9490, 2, 2),
     # the warp-level kernels' widths: batches around a CTA's 32 envs and a dh1 tile's 64, one and several t-slices
     (32, 0, 33, 5, 3), (32, 1, 65, 4, 2), (96, 0, 2, 3, 4), (96, 0, 777, 7, 20), (96, 1, 64, 12, 5), (192, 0, 100, 6, 9),
     (192, 0, 5, 4, 55), (192, 1, 2100, 5, 3), (64, 0, 1500, 5, 9), (64, 1, 31, 6, 33),
