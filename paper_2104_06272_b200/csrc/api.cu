@@ -55,7 +55,7 @@ int validate(const anakin_cfg* c) {
         default: return ANAKIN_E_UNSUPPORTED_CFG;
     }
     if ((double)c->B * (double)c->T_max > 2.0e9) return ANAKIN_E_UNSUPPORTED_CFG;
-    if (c->n_policies >= 2) {  // many policies: fp32 on the warp-level tensor path, every policy with at least one env
+    if (c->n_policies >= 2) {  // many policies: fp32 at 64 and 128 units, every policy with at least one env
         const int K = c->n_policies, Bp = (c->B + K - 1) / K;
         if (K > c->B || (long long)(K - 1) * Bp >= c->B) return ANAKIN_E_INVALID_ARG;
         if (K > 65535 || c->precision != ANAKIN_PRECISION_FP32 || (c->H != 64 && c->H != 128)) return ANAKIN_E_UNSUPPORTED_CFG;

@@ -10,7 +10,7 @@
 // owns 128 hidden units (accumulator lanes) and walks units of (128 envs, slice of the steps), unit blockIdx.x,
 // blockIdx.x + gridDim.x, ..., step by step:
 //   warp 0 (one lane)  TMA producer: the dh2 planes of every step through a ring of 128 x 64 K-major boxes
-//   warp 1 (one lane)  tcgen05.mma issuer.  Per step: the dh1 product (K = H; three fp16 terms per k16, one in the bf16
+//   warp 1             tcgen05.mma issuer (the whole warp walks the loop, an elected lane issues).  Per step: the dh1 product (K = H; three fp16 terms per k16, one in the bf16
 //                      workload, all into one of two 128-column accumulators); then, for the step before, the agent-plane
 //                      product  D[unit][cell] += sum over the 128 envs of dh1[env][unit] * onehot[env][cell]  (K = 128,
 //                      operand tiles that the epilogue warps wrote) into a third accumulator, restarted after every GROUP

@@ -1,16 +1,17 @@
 // Weight-gradient GEMMs on the 5th-generation tensor cores:  C[m][n] = sum_k A[k][m] B[k][n],  K = B*T rows.
 //
 // These are the batch-mean reductions of the update (the single-device form of the paper's cross-core gradient average,
-// Podracer paper, Section 3.1): dW2 = h1^T dh2 and the agent plane of dW1 = onehot(pos)^T dh1.  Both operands have the
+// Podracer paper, Section 3.1): dW2 = h1^T dh2 of the widths that have no fused kernel for it, the agent plane of dW1 =
+// onehot(pos)^T dh1 of the bf16 widths outside 64, 128, 256, and the wall and goal planes of every width.  Both operands have the
 // contraction index as their slow (row) index, i.e. they are "MN-major" for the MMA.
 //
 // One CTA owns a 128 x BN output tile (BN = the hidden width up to 256, else column tiles of 256; the accumulator
 // columns live in tensor memory) and a
 // K range (split-K; partials are summed later in a fixed order).  Per 64-row K chunk:
-//   warp 0 (one lane)  issues TMA loads of the operand planes (64 x 64 boxes, 128-byte swizzle) into a 2-stage ring,
+//   warp 0 (one lane)  issues TMA loads of the operand planes (64 x 64 boxes, 128-byte swizzle) into a ring of two to four stages,
 //   warps 2-5          for the one-hot A operand: write the 0/1 tile straight into the swizzled layout instead of loading it,
-//   warp 1 (one lane)  issues tcgen05.mma: for fp32 workloads three MMAs per k16 (lo*hi, hi*lo, hi*hi fp16 terms) into one
-//                      fp32 accumulator; commits free the stage,
+//   warp 1             issues tcgen05.mma (the whole warp walks the loop, an elected lane issues): for fp32 workloads three MMAs per
+//                      k16 (lo*hi, hi*lo, hi*hi fp16 terms) into one fp32 accumulator, six with three-term operands; commits free the stage,
 //   warps 2-5          after the last chunk: tcgen05.ld the accumulator and store the partial tile.
 // Long K ranges (plane operands): the tensor core's fp32 accumulation rounds toward zero, which biases a sum of many
 // thousand MMAs by more than the fp32 workloads' 1e-4 bound (measured: -2e-4 after 65,536 rows; fp32 workloads only).  The K range of a CTA

@@ -1,18 +1,19 @@
 // Learning half of the Anakin minimal unit on the tensor pipe (Podracer paper, Section 3.1; Figure 2, top), for the
 // hidden sizes the tensor-pipe rollout covers.  The update reuses the policy's forward pass (Section 3.1): the rollout
-// kernel saved h1 (as bf16 hi/lo planes) and h2 for every recorded row, so the learner starts at the heads.
+// kernel saved h1 (as 16-bit planes) and h2 for every recorded row, so the learner starts at the heads.
 //
 //   k_heads_bwd   flat 32-row tiles: saved head outputs -> softmax / loss terms -> dOut -> dh2 (fp32 FMA, HBM-bound).
-//                 Emits dh2 as 16-bit hi/lo planes and per-CTA partial sums of dWh, dbh, db2 and the loss terms.
-//                 At hidden width 256 (few enough rows per CTA) it also takes dW2 = h1^T dh2 for its rows: the dh2 tile it
+//                 Emits dh2 as 16-bit planes and per-CTA partial sums of dWh, dbh, db2 and the loss terms.
+//                 At hidden widths 128 and 256 (one policy) it also takes dW2 = h1^T dh2 for its rows: the dh2 tile it
 //                 has just computed and the matching h1 tile (TMA) are the operands of tcgen05 MMAs into tensor memory,
 //                 so dh2 is not read back for that product and the stand-alone dW2 GEMM is not launched.
-//   k_dh1         dh1 = (dh2 W2^T) gated by h1 > 0 with mma.sync; a CTA keeps its slice of W2 in shared memory and
-//                 walks t for 64 envs, so S = sum_t dh1 accumulates in registers.  Emits dh1 planes and S planes.
-//   k_gemm_tn     C[m][n] = sum_k A[k][m] B[k][n] with split-K partial outputs, bf16 hi/lo planes as operands and
-//                 three MMAs per product (two when A is an exact 0/1 plane, one in the bf16 workload):
-//                 dW2 = h1^T dh2 (K = B*T), dW1[agent plane] = X^T dh1 (K = B*T), dW1[wall, goal planes] = X^T S
-//                 (K = B; an extra all-ones row of A yields db1 = sum_b S[b]).
+//   k_dh1         (bf16 at widths 32, 96, 192; many policies at 128) dh1 = (dh2 W2^T) gated by h1 > 0 with mma.sync; a CTA
+//                 keeps its slice of W2 in shared memory and walks t for 64 envs, so S = sum_t dh1 accumulates in
+//                 registers.  The other widths have tcgen05 kernels of their own (back64_tc.cu, dh1a_tc.cu, x3_gemm.cu).
+//   k_gemm_tn     (many policies) C[m][n] = sum_k A[k][m] B[k][n] with split-K partial outputs, three MMAs per product, two
+//                 when A is an exact 0/1 plane.  dW2 = h1^T dh2 (K = B*T) and the agent plane of dW1 (K = B*T) at H = 128,
+//                 the wall and goal planes X^T S (K = B; an extra all-ones row of A yields db1 = sum_b S[b]).  One policy:
+//                 gemm_tc.cu.
 //   k_reduce_adam2  fixed-order sum of every region's partials (= the batch-mean gradient, the single-device form of
 //                 the paper's cross-core average), Adam, loss statistics.
 // No floating-point atomics: every sum has a fixed order, so runs are bitwise reproducible.
@@ -32,7 +33,7 @@ namespace anakin {
 // ----------------------------------------------------------------------------------------------------
 // HS = width of the column slab one CTA covers (blockIdx.y picks the slab; HS = H for H <= 256); H2BF: h2 is stored as
 // bf16 (the wide bf16 path) instead of fp32.
-// FUSE (H = 256 only): the kernel also takes dW2 = h1^T dh2 for its rows on the tcgen05 pipe (see k_heads_bwd).
+// FUSE (H = 128, 256): the kernel also takes dW2 = h1^T dh2 for its rows on the tcgen05 pipe (see k_heads_bwd).
 __host__ __device__ constexpr int heads_per_sm(int H) { return H == 32 ? 8 : H == 64 ? 5 : H == 96 ? 4 : 2; }
 template <int H, int NW, int PREC, int HS = H, bool H2BF = false, bool FUSE = false>
 struct HeadsCfg {
@@ -1544,8 +1545,8 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const size_t R = (size_t)B * T, RH = (size_t)B * d.Tmax * H;
     cudaStream_t s = c.s;
     const bool wide = wide_supported(H);  // bf16 activations in HBM, layer-2 products as large tcgen05 GEMMs
-    // many policies: every kernel gets one grid slice per policy and moves its workspace pointers there; the tcgen05
-    // kernels bake addresses into tensor maps, so this path stays on the warp-level kernels
+    // many policies: every kernel gets one grid slice per policy and moves its workspace pointers there.  At H = 64 the backward kernel
+    // is the tcgen05 one (its tensor maps have a policy dimension); the rest, and H = 128, run the warp-level kernels
     const bool grouped = d.npol > 1;
     LearnPlan pl;
     learn_mma_plan(d, &pl);

@@ -1,15 +1,16 @@
-// Persistent rollout on the tensor pipe (warp-level mma.sync), second-layer weights resident on chip.
+// Persistent rollout on the tensor pipe (warp-level mma.sync), second-layer weights resident on chip: hidden widths 32, 64, 96, 128
+// and 192, and many policies.  (128 beyond one wave of batches: rollout_tc128.cu; 256: rollout_pair.cu, rollout_pair2.cu.)
 //
-// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top).  A CTA owns 32 envs for all
-// T+1 forward passes of a rollout; nothing is exchanged between CTAs.  Per step:
+// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top).  A CTA owns 32 envs, or 16 in small batches,
+// for all T+1 forward passes of a rollout; nothing is exchanged between CTAs.  Per step:
 //   layer 1   h1 = relu(base + W1[agent row])            gather-add, written to smem as 16-bit (hi, lo) planes
 //   layer 2   h2 = relu(h1 W2 + b2)                      mma.sync m16n8k16; warp w owns output columns [NC*w, NC*w+NC)
 //   heads     out = h2 Wh + bh                           fp32 FMA on the accumulator fragments, fixed-order reduction
 //   env       softmax, Philox inverse-CDF sample, gridworld step, time-major records   (one thread per env)
-// fp32 workloads use a two-term fp16 split of both operands and three MMAs per product (hi*hi + lo*hi + hi*lo,
-// fp32 accumulate).  W2's "hi" B-fragments stay in shared memory and its "lo" B-fragments in registers for the
-// whole kernel (H = 256: 128 KB + 128 KB), so after the prologue the loop touches no weight bytes beyond the
-// agent's W1 row.  The bf16 workload needs one MMA per product and no lo planes.
+// fp32 workloads at 64 and 128 use a two-term fp16 split of both operands and three MMAs per product (hi*hi + lo*hi + hi*lo,
+// fp32 accumulate), at 32, 96 and 192 three bf16 terms and six MMAs.  W2's leading B-fragments stay in shared memory and those of
+// its last term in registers for the whole kernel, so after the prologue the loop touches no weight bytes beyond the
+// agent's W1 row (from L2, or from shared memory where the launch says so).  The bf16 workload needs one MMA per product.
 #include "env_step.cuh"
 
 namespace anakin {

@@ -1,7 +1,8 @@
 // Persistent rollout on the 5th-generation tensor cores: a pair of CTAs (a cluster of two, on neighbouring SMs) owns
 // 64 envs for all T+1 forward passes of a rollout and shares the second-layer weights between its two SMs.
 //
-// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top), hidden width 256, fp32 workloads.
+// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top), hidden width 256; the fp32 form
+// (bf16 workloads have one plane of each operand and one MMA per k16).
 // The second layer is computed transposed,  D[j][env] = sum_k W2[k][j] h1[env][k],  as tcgen05.mma.cta_group::2 with
 // M = 256 hidden units, so that each CTA keeps only ITS 128 columns of W2 on chip (two fp16 planes in TENSOR memory, the A
 // operand of every MMA, transposed into it once) and builds only the h1 rows of ITS 32 envs; the tensor cores of the pair read
@@ -433,8 +434,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<ME_>::THREAD
 
 }  // namespace
 
-// Covers hidden width 256 with fp32 parameters (two-term fp16 operands) when the row-major 16-bit planes of W2 exist;
-// anything else returns cudaErrorNotSupported and the caller takes the warp-level kernel.
 template <int ME>
 static cudaError_t launch_pair(const RolloutArgs& a0, int prec, cudaStream_t s) {
     using Cfg = PairCfg<ME>;
@@ -458,6 +457,7 @@ static cudaError_t launch_pair(const RolloutArgs& a0, int prec, cudaStream_t s) 
     return w1s ? go(std::true_type{}) : go(std::false_type{});
 }
 
+// Hidden width 256 in either precision, given the row-major 16-bit planes of W2; cudaErrorNotSupported otherwise.
 cudaError_t launch_rollout_pair(const RolloutArgs& a, int prec, cudaStream_t s) {
     if (a.d.H != 256 || !a.b.w2p_hi || (prec == 0 && !a.b.w2p_lo) || !a.b.base) return cudaErrorNotSupported;
     // 16 envs per CTA while one wave of pairs covers the batch

@@ -1,7 +1,8 @@
 // Persistent rollout on the 5th-generation tensor cores for hidden width 256 and large batches: a pair of CTAs (a
 // cluster of two, on neighbouring SMs) owns 128 envs for all T+1 forward passes, in TWO independent groups of 64.
 //
-// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top), fp32 workloads.  The layout of one
+// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top); the fp32 form (bf16 workloads have one
+// plane of each operand and one MMA per k16).  The layout of one
 // group is that of the one-group CTA-pair kernel: layer 2 transposed, D[j][env] = sum_k W2[k][j] h1[env][k], as
 // tcgen05.mma.cta_group::2 with M = 256 hidden units, each CTA keeping ITS 128 columns of W2 on chip (the fp16 hi
 // plane transposed in tensor memory as the A operand, the lo plane in shared memory) and building the h1 rows of ITS 32 envs of the group.  With many envs per SM the rollout is a
@@ -446,7 +447,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Pair2Cfg::THREADS, 1
 
 }  // namespace
 
-// Covers hidden width 256 with fp32 parameters on batches large enough to give every SM pair a cluster of 128 envs;
+// Hidden width 256 in either precision, on batches beyond one wave of the one-group kernel and on replays of 128 envs and more;
 // anything else returns cudaErrorNotSupported and the caller takes the one-group CTA-pair kernel.
 cudaError_t launch_rollout_pair2(const RolloutArgs& a0, int prec, cudaStream_t s) {
     using Cfg = Pair2Cfg;

@@ -1,7 +1,8 @@
 // Persistent rollout on the 5th-generation tensor cores for hidden width 128 and large batches: one CTA owns 128 envs
 // for all T+1 forward passes of a rollout and keeps the whole second layer on chip.
 //
-// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top), fp32 workloads.  With many envs per
+// Acting half of the Anakin minimal unit (Podracer paper, Section 3.1; Figure 2, top); the fp32 form (bf16 workloads have one
+// plane of each operand and one MMA per k16).  With many envs per
 // SM the rollout is a throughput problem, but a single env group still walks a strictly serial chain per step (gather the
 // agent's first-layer row -> tensor cores -> heads -> sample -> next gather).  The CTA therefore holds TWO independent
 // groups of 64 envs, each with eight worker warps of its own, so that one group's tensor-core phase and sampling phase
@@ -434,8 +435,8 @@ __global__ void __launch_bounds__(Tc128Cfg::THREADS, 1) k_rollout_tc128(RolloutA
 
 }  // namespace
 
-// Covers hidden width 128 with fp32 parameters (two-term fp16 operands) on batches large enough to give every SM a CTA
-// of 128 envs; anything else returns cudaErrorNotSupported and the caller takes the warp-level kernel.
+// Hidden width 128 in either precision, on batches beyond one wave of the warp-level kernel and on replays of more than 64
+// envs; anything else returns cudaErrorNotSupported and the caller takes the warp-level kernel.
 cudaError_t launch_rollout_tc128(const RolloutArgs& a0, int prec, cudaStream_t s) {
     using Cfg = Tc128Cfg;
     if (a0.d.H != Cfg::H || !a0.b.w2p_hi || (prec == 0 && !a0.b.w2p_lo) || !a0.b.base || a0.d.npol > 1) return cudaErrorNotSupported;

@@ -8,7 +8,7 @@
 // ends up with its 128 rows x 256 columns of the accumulator in its own tensor memory.
 //   warp 0 (one lane, both CTAs)   TMA producer of its CTA's halves; the byte counts of both CTAs are credited to the
 //                                  LEADER's "full" barrier, which the leader's producer arms for both
-//   warp 1 (one lane, leader only) MMA issuer; commits are multicast to the "empty" / "accumulator full" barriers of both CTAs
+//   warp 1 (leader only)           MMA issuer (the whole warp walks the loop, an elected lane issues); commits are multicast to the "empty" / "accumulator full" barriers of both CTAs
 //   warps 2-9 (both CTAs)          epilogue of tile i under the MMAs of tile i+1 (two 256-column accumulators); their
 //                                  "accumulator drained" arrivals all go to the leader's barrier
 // Tensor memory is allocated and freed by one warp of each CTA.  Every wait is bounded (a timeout raises

@@ -12,7 +12,7 @@
 // PAIR: a cluster of two CTAs owns a 256 x 256 tile (cta_group::2), 96 KB per stage and CTA for 24 x 128 clocks of MMAs; otherwise
 // one CTA owns 128 x BN (BN = 128, 64) for launches with few tiles.
 //   warp 0 (one lane)        TMA producer (PAIR: of its CTA's halves, credited to the leader's barrier)
-//   warp 1 (one lane)        MMA issuer (PAIR: the leader's)
+//   warp 1                   MMA issuer (PAIR: the leader's): the whole warp walks the loop, an elected lane issues
 //   warps 2-9                accumulate the groups, then bias / ReLU / gate and store through a staging buffer, 64-byte row segments
 // Every wait is bounded; a timeout raises DEV_E_WAIT_TIMEOUT and the CTA unwinds (tensor memory freed).
 #include <cstring>

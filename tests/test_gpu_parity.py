@@ -47,8 +47,8 @@ SMALL = {
     "tp_ragged_64": Workload("tp_ragged_64", B=97, N=3, H=64, T=3, iters=1, episode_cap=2),
     "tp_bf16_128": Workload("tp_bf16_128", B=210, N=7, H=128, T=6, iters=1, precision=1, episode_cap=5),
     "tp_bf16_256": Workload("tp_bf16_256", B=131, N=16, H=256, T=5, iters=1, precision=1),
-    # the second env (torus: moves wrap around the edges) on every rollout path: persistent tensor-pipe kernel,
-    # FFMA kernel, wide bf16 path
+    # the second env (torus: moves wrap around the edges) on every rollout path: CTA-pair tcgen05 kernel,
+    # warp-level tensor kernel (three-term operands), wide bf16 path
     "torus_tp_256": Workload("torus_tp_256", B=140, N=6, H=256, T=12, iters=1, episode_cap=9, env_kind=1),
     "torus_ffma_96": Workload("torus_ffma_96", B=77, N=5, H=96, T=12, iters=1, episode_cap=9, env_kind=1),
     "torus_wide_512": Workload("torus_wide_512", B=70, N=8, H=512, T=6, iters=1, precision=1, episode_cap=9, env_kind=1),

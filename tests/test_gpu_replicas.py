@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = {
     "mma_h64": WORKLOADS["tiny"].scaled(name="mma_h64", B=256, T=16),
+    # (a width with three-term operands on the warp-level tensor rollout)
     "ffma_h96": WORKLOADS["tiny"].scaled(name="ffma_h96", B=192, H=96, T=8),
     "wide_bf16": WORKLOADS["tensor_core"].scaled(name="wide_bf16", B=256, H=512, T=4),
     # the kernels the large workloads run: the warp-level tensor rollout at H = 128 and the CTA-pair tcgen05 rollout at
