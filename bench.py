@@ -141,6 +141,10 @@ PROFILE_OF = {
     ("throughput", "reduce_adam"): ("reduce_adam2__throughput.md", "learner_mma.cu"),
     ("throughput", "env_base"): ("env_base__throughput.md", "rollout.cu"),
     ("throughput", "dw1_walls"): ("gemm_tn_tc_env_planes__throughput.md", "gemm_tc.cu"),
+    ("many_policies", "rollout"): ("rollout_mma__many_policies.md", "rollout_mma.cu"),
+    ("many_policies", "dh1"): ("back64__many_policies.md", "back64_tc.cu"),
+    ("many_policies", "heads_bwd"): ("heads_bwd__many_policies.md", "learner_mma.cu"),
+    ("many_policies", "reduce_adam"): ("reduce_adam2__many_policies.md", "learner_mma.cu"),
 }
 
 
