@@ -17,7 +17,7 @@ CASES = [
     (32, 0, 33, 5, 3), (32, 1, 65, 4, 2), (96, 0, 2, 3, 4), (96, 0, 777, 7, 20), (96, 1, 64, 12, 5), (192, 0, 100, 6, 9),
     (192, 0, 5, 4, 55), (192, 1, 2100, 5, 3), (64, 0, 1500, 5, 9), (64, 1, 31, 6, 33),
     # width 64: several steps in a 128-row tile (rows left over, slices that end short), one env more than fits, a CTA that walks
-    # more than 32 tiles; boards of more than 128 cells there and at 128 and 256
+    # 24 tiles (longer ones: LONG_SUMS below); boards of more than 128 cells there and at 128 and 256
     (64, 0, 1, 12, 5), (64, 0, 5, 16, 40), (64, 1, 64, 12, 7), (64, 0, 65, 5, 20), (64, 1, 129, 16, 3), (64, 0, 18945, 3, 17),
     (128, 0, 130, 16, 5), (128, 1, 77, 12, 9), (256, 0, 40, 12, 7), (256, 1, 300, 16, 4), (32, 1, 300, 16, 9), (192, 1, 70, 13, 6),
     # units of (128-env tile, slice) that do not come out even: more units than CTAs, a short last slice, 5 and 16 slices
