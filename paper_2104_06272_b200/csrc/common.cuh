@@ -79,7 +79,7 @@ struct Buffers {
     float* h2;       // [R][H]
     float* out5;     // [R][8] head outputs (4 logits, value) of every recorded row, saved by the tensor-pipe rollout
     float* vboot;    // [B] value of the state after the last recorded step under the CURRENT parameters (replay mode 2)
-    float* dh2;      // [R][H]
+    float* dh2;      // [R][H] (null where it stays on chip)
     float* dh1;      // [R][H]
     float* S;        // [B][H]  sum over t of dh1
     float* part;     // split-K partial gradients (LearnPlan)
@@ -467,6 +467,9 @@ inline int most_slices(int m_tiles, int cap) { return m_tiles * 4 > cap ? 4 : (c
 inline int most_s_rows(int B) { return 4 * B > 148 * 128 ? 4 * B : (MAX_SLICES * B < 148 * 128 ? MAX_SLICES * B : 148 * 128); }
 void back64_shape(const Dims& d, int T, int* nx, int* ts);  // hidden width 64: dh1, S, dW2 and the agent plane in one kernel
 cudaError_t launch_back64(const LearnArgs& a, int prec, int nx, float* part_w2, float* part_agent, size_t stride_agent, cudaStream_t s);
+bool back128_supported(const Dims& d);  // hidden width 128, up to 128 cells, one policy: everything from the head outputs to dh1 in one kernel
+void back128_shape(const Dims& d, int T, int* nx, int* ts);
+cudaError_t launch_back128(const LearnArgs& a, int prec, int nx, float* part_w2, float* part_agent, size_t stride_agent, cudaStream_t s);
 cudaError_t launch_selftest_wait(int* status, long long limit_clocks, long long* waited_clocks, cudaStream_t s);
 cudaError_t launch_refresh_compute_params(const Dims& d, const Buffers& b, int prec, const Ctx& c);
 

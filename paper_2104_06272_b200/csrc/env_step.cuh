@@ -270,6 +270,43 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
         lo = *reinterpret_cast<const uint32_t*>(&l);
     }
 }
+// Two fp32 operations in one instruction (each half rounded on its own, exactly as the scalar one).
+__device__ __forceinline__ uint64_t pack_f32x2(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack_f32x2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// The 32 x 32 bit matrix whose row l is lane l's word, transposed: lane l gets bit l of every lane's word (bit k from lane k).
+__device__ __forceinline__ uint32_t transpose_bits32(uint32_t x, int lane) {
+    uint32_t m = 0x0000FFFFu;  // bits whose index has bit `s` clear
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, s);
+        x = (lane & s) ? (x & ~m) | ((y & ~m) >> s) : (x & m) | ((y & m) << s);
+        m ^= m << (s >> 1);
+    }
+    return x;
+}
 // PREC 2: two consecutive elements as three packed bf16 terms, x = t[0] + t[1] + t[2] (both subtractions are exact).
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t (&t)[3]) {
 #pragma unroll

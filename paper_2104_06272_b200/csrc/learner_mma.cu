@@ -2,6 +2,9 @@
 // hidden sizes the tensor-pipe rollout covers.  The update reuses the policy's forward pass (Section 3.1): the rollout
 // kernel saved h1 (as 16-bit planes) and h2 for every recorded row, so the learner starts at the heads.
 //
+// Hidden width 128 on boards of up to 128 cells (one policy) has all of it up to dh1 and the agent plane in one kernel (back128_tc.cu); the
+// kernels below serve the rest.
+//
 //   k_heads_bwd   flat 32-row tiles: saved head outputs -> softmax / loss terms -> dOut -> dh2 (fp32 FMA, HBM-bound).
 //                 Emits dh2 as 16-bit planes and per-CTA partial sums of dWh, dbh, db2 and the loss terms.
 //                 At hidden widths 128 and 256 (one policy) it also takes dW2 = h1^T dh2 for its rows: the dh2 tile it
@@ -1471,6 +1474,9 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         p->ns_agent = std::max(p->ns_agent, std::min(cap, (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax)));
         p->ns_env = env_splits(d, most_s_rows(d.B));
     }
+    if (back128_supported(d)) {  // (one partial of everything per CTA)
+        p->ns_w2 = p->ns_agent = std::min(148, (d.B + 63) / 64 * std::min(MAX_SLICES, d.Tmax));
+    }
     if (H == 64) {  // (one partial per CTA of the fused kernel; its slices of the steps are rows of S)
         const int units = d.B > 64 ? (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax) : (d.Tmax + 128 / d.B - 1) / (128 / d.B);  // (of any T <= Tmax)
         p->ns_w2 = p->ns_agent = std::min(std::max(148 / d.npol, 1), units);
@@ -1480,6 +1486,7 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     size_t hg = (size_t)heads_grid_max(H);
     if (d.npol > 1) hg = (size_t)std::max(4 * heads_grid_max(H) / d.npol, 1);  // many policies: the CTAs of all policies fill the GPU together
     p->heads_grid = (int)(tiles32 < hg ? tiles32 : hg);
+    if (back128_supported(d)) p->heads_grid = p->ns_w2;
     // (the fused heads + dW2 kernel writes one dW2 partial per CTA: room for the larger of the two partial counts)
     int w2_slots = heads_fuse_dw2(d) && p->heads_grid > p->ns_w2 ? p->heads_grid : p->ns_w2;
     if (three_terms(H, 0) && x3_w2_splits(H, R) > w2_slots) w2_slots = x3_w2_splits(H, R);
@@ -1567,7 +1574,10 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     // dW2 = h1^T dh2 rides in the heads kernel where its rows per CTA allow (it then has one partial per heads CTA)
     const bool fuse_dw2 = heads_fuse_dw2(d);
     if (fuse_dw2) a.reg[4].ns = pl.heads_grid;
-    {
+    // Everything from the head outputs to dh1 and the agent plane in one kernel: it beats the two at every size that was timed (2500 to
+    // 131072 envs).  Beyond 128 cells its accumulators do not fit in tensor memory.
+    const bool back128 = back128_supported(d);
+    if (!back128) {
         Scope sc(c, K_HEADS_BWD);
         switch (H) {
             case 64: if constexpr (PREC != 2) { CK((launch_heads_t<64, 4, PREC>(a, pl.heads_grid, s))); break; }
@@ -1612,6 +1622,15 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
         Scope sc(c, K_DH1);
         CK(launch_back64(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
+        fused_agent = true;
+    } else if (back128) {
+        int nx;
+        back128_shape(d, T, &nx, &a.ts);
+        for (int q = 4; q < 8; ++q) a.reg[q].ns = nx;
+        a.reg[1].ns = pl.loss_blocks = nx;
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
+        Scope sc(c, K_DH1);
+        CK(launch_back128(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
     } else if (!wide && !grouped && dh1_agent_tc_supported(d)) {
         int nx;

@@ -22,6 +22,9 @@ CASES = [
     (128, 0, 130, 16, 5), (128, 1, 77, 12, 9), (256, 0, 40, 12, 7), (256, 1, 300, 16, 4), (32, 1, 300, 16, 9), (192, 1, 70, 13, 6),
     # units of (128-env tile, slice) that do not come out even: more units than CTAs, a short last slice, 5 and 16 slices
     (128, 0, 2500, 5, 24), (128, 1, 1300, 5, 11), (256, 0, 6000, 5, 7), (256, 1, 1000, 4, 17), (256, 0, 100, 6, 33),
+    # width 128 on boards of up to 128 cells (tiles of 64 envs, one kernel from the head outputs to dh1): batches around a tile's edge,
+    # the largest board, several units a CTA with a short last tile, a CTA without a whole slice
+    (128, 0, 1, 11, 3), (128, 1, 63, 2, 70), (128, 0, 64, 3, 9), (128, 0, 65, 11, 20), (128, 1, 9537, 8, 3), (128, 0, 19000, 6, 5),
     # the agent rows of W1 beside three CTAs per SM at width 64, and one step or one CTA short of it
     (64, 0, 14241, 3, 3), (64, 0, 14300, 9, 16), (64, 0, 14241, 3, 9), (64, 0, 14209, 11, 10), (64, 0, 14208, 5, 10),
     # just beyond one wave of the smaller-batch rollouts at H = 128 and 256
