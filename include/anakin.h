@@ -247,9 +247,9 @@ int anakin_run(anakin_t* h, int iters);
  * stream, anakin_set only enqueues: see the conventions above) or a device pointer (ptr_is_device = 1; asynchronous
  * on the stream), or a PAGE-LOCKED host pointer (ptr_is_device = 2; asynchronous on the stream in both directions: the
  * data of an anakin_get is there once the caller has synchronised the stream, e.g. with anakin_status).  `bytes` must equal the blob's
- * size.  A device pointer may be any that cudaMemcpyAsync takes, another GPU's memory included; with many policies, memory of the
- * handle's own GPU (while that is the current device) is read or written by one kernel on the stream, anything else by one copy per
- * policy.  Setting any TRAJ_* / ADV / RET blob marks a rollout of the last used length as pending, so the stages
+ * size.  A device pointer may be any that cudaMemcpyAsync takes, another GPU's memory included; memory of the handle's own GPU
+ * (while that is the current device) is read or written by a kernel on the stream, one policy's blobs up to 16 MiB, anything else by
+ * cudaMemcpyAsync, with many policies one per policy.  Setting any TRAJ_* / ADV / RET blob marks a rollout of the last used length as pending, so the stages
  * can be driven with the other side's data.  Errors: INVALID_ARG (unknown blob, wrong size, read-only blob).
  */
 int anakin_get(anakin_t* h, int which, void* ptr, size_t bytes, int ptr_is_device);

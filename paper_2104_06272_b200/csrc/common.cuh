@@ -385,6 +385,7 @@ inline cudaError_t launch(dim3 grid, dim3 block, size_t smem, cudaStream_t s, A.
 cudaError_t launch_reset(const Dims& d, const Buffers& b, uint64_t seed, double density, int prec, const Ctx& c);
 cudaError_t launch_env_base(const Dims& d, const Buffers& b, const Ctx& c);
 cudaError_t launch_copy_blocks(void* dst, size_t dpitch, const void* src, size_t spitch, size_t bytes, size_t rows, cudaStream_t s);
+cudaError_t launch_copy_flat(void* dst, const void* src, size_t bytes, cudaStream_t s);
 cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c);
 cudaError_t launch_rollout_mma(const RolloutArgs& a, int prec, cudaStream_t s);  // cudaErrorNotSupported if not covered
 bool rollout_mma_supported(int H);

@@ -563,6 +563,36 @@ print("ok")
 """
 
 
+@pytest.mark.parametrize("shift", [0, 1, 4, 20])
+def test_blobs_copied_within_the_gpu_at_any_alignment(bnd, shift):
+    """A blob of up to 16 MiB goes to or from this GPU's memory by a kernel (sixteen, four or one byte a thread, and a tail), larger ones
+    and everything else by the runtime's copy: both directions, sizes of 77 bytes to 19 MB, offsets that are and are not aligned."""
+    w = Workload("copies", B=77, N=5, H=32, T=3, iters=1)
+    big = Workload("copies_big", B=60000, N=2, H=32, T=80, iters=1)
+    for wl, names in ((w, (bnd.PARAMS, bnd.ENV_POS, bnd.ENV_WALLS, bnd.TRAJ_ACTION, bnd.TRAJ_VALUE)), (big, (bnd.TRAJ_ACTION, bnd.TRAJ_REWARD))):
+        an = bnd.Anakin(bnd.cfg_from_workload(wl))
+        an.reset(5)
+        an.run(1)
+        for which in names:
+            want = an.get(which).view(np.uint8).reshape(-1)
+            room = torch.full((want.size + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+            out = room[shift: shift + want.size]
+            before = an.launch_count()
+            an.get_into(which, out)
+            assert (an.launch_count() > before) == (want.size <= 16 << 20)
+            got = room.cpu().numpy()
+            assert np.array_equal(got[shift: shift + want.size], want)
+            assert (got[:shift] == 0xA5).all() and (got[shift + want.size:] == 0xA5).all()
+            an.set(which, torch.zeros(want.size, dtype=torch.uint8, device="cuda"))
+            assert not an.get(which).view(np.uint8).any()
+            an.set(which, out)
+            assert np.array_equal(an.get(which).view(np.uint8).reshape(-1), want)
+        pin = torch.zeros(an.blob_bytes(bnd.ENV_POS), dtype=torch.uint8).pin_memory()  # (no memory of this GPU: the runtime's copy)
+        before = an.launch_count()
+        assert bnd.lib().anakin_get(an._h, bnd.ENV_POS, pin.data_ptr(), pin.numel(), 1) == bnd.OK
+        assert an.launch_count() == before and an.status() == 0 and (pin.numpy() == an.get(bnd.ENV_POS)).all()
+
+
 def test_handles_in_their_own_threads_and_streams_give_what_they_give_alone():
     """Different handles are independent: the first calls of a process from eight threads at once (what the library sets up once per
     process or device among them), each on a handle and a stream of its own, against the same work done one after the other."""
