@@ -190,11 +190,8 @@ def kernel_work(w):
         # name: (bound, executed flops, bytes)
         "rollout": ("tensor", p3 * 2.0 * B * (T + 1) * H * H, R * (15.0 + pl * H + 4.0 * H) + B * 4),
         # fused kernels.  H = 128, 256 (one policy): also the agent plane of dW1 over 128 or 256 padded cells; reads the dh2 planes and
-        # one gate bit per element.  H = 128 on boards of up to 128 cells: everything from the head outputs on, dW2 too; reads h2, the h1 planes
-        # and the gates.  H = 64: also dW2; reads the dh2 and h1 planes.  Otherwise: dh2 in, 16-bit h1 gates in, dh1 out.
-        "dh1": (("tensor", p3 * 4.0 * R * H * H + p2 * 2.0 * R * 128 * H, R * H * (pl + 4.125) + R * 33.0)
-                if H == 128 and C <= 128 and getattr(w, "n_policies", 0) <= 1
-                else ("tensor", p3 * 2.0 * R * H * H + p2 * 2.0 * R * (128 if C <= 128 else 256) * H, R * H * (pl + 0.125))
+        # one gate bit per element.  H = 64: also dW2; reads the dh2 and h1 planes.  Otherwise: dh2 in, 16-bit h1 gates in, dh1 out.
+        "dh1": (("tensor", p3 * 2.0 * R * H * H + p2 * 2.0 * R * (128 if C <= 128 else 256) * H, R * H * (pl + 0.125))
                 if H in (128, 256) and getattr(w, "n_policies", 0) <= 1
                 else ("tensor", p3 * 4.0 * R * H * H + p2 * 2.0 * R * (128 if C <= 128 else 256) * H, R * H * 2.0 * pl) if H == 64
                 else ("tensor", p3 * 2.0 * R * H * H, R * H * (2.0 * pl + 2.0))),
@@ -202,8 +199,11 @@ def kernel_work(w):
         "dw1_agent": ("tensor", p2 * 2.0 * R * C * H, R * H * 1.0 * pl + R),
         "dw1_walls": ("tensor", 2 * 2.0 * B * (2 * C + 1) * H, B * H * 4.0),  # (wall and goal planes in one launch; many policies: the walls)
         "dw1_goal": ("tensor", 2 * 2.0 * B * C * H, B * H * 4.0),
-        # hidden width 128 / 256 (one policy): the kernel also takes dW2 = h1^T dh2 on the tensor pipe and reads the h1 planes
-        "heads_bwd": (("hbm", R * H * 22.0 + p3 * 2.0 * R * H * H, R * H * (4.0 + 2.0 * pl) + R * 10.0)
+        # hidden width 128 / 256 (one policy): the kernel also takes dW2 = h1^T dh2 on the tensor pipe and reads the h1 planes; at 128 on boards of
+        # up to 128 cells dh1 and the agent plane too, and no dh2 goes out
+        "heads_bwd": (("tensor", p3 * 4.0 * R * H * H + p2 * 2.0 * R * 128 * H, R * H * (pl + 4.125) + R * 45.0)
+                      if H == 128 and C <= 128 and getattr(w, "n_policies", 0) <= 1
+                      else ("hbm", R * H * 22.0 + p3 * 2.0 * R * H * H, R * H * (4.0 + 2.0 * pl) + R * 10.0)
                       if H in (128, 256) and getattr(w, "n_policies", 0) <= 1
                       else ("hbm", R * H * 22.0, R * H * (4.0 + pl) + R * 10.0)),
         "gae": ("hbm", R * 6.0, R * 17.0),

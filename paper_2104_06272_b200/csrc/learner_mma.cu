@@ -1629,7 +1629,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         for (int q = 4; q < 8; ++q) a.reg[q].ns = nx;
         a.reg[1].ns = pl.loss_blocks = nx;
         a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
-        Scope sc(c, K_DH1);
+        Scope sc(c, K_HEADS_BWD);  // (profiled under the name of what it starts with)
         CK(launch_back128(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
     } else if (!wide && !grouped && dh1_agent_tc_supported(d)) {
