@@ -73,76 +73,177 @@ cudaError_t launch_rollout(const RolloutArgs& a, int prec, const Ctx& c) {
 }
 
 // ----------------------------------------------------------------------------------------------------
-// GAE reverse scan: lane = env, so every load and store of a warp is one contiguous segment per t.
-//   d_t = 1 - done_t; delta_t = r_t + gamma d_t V_{t+1} - V_t; A_t = delta_t + gamma lambda d_t A_{t+1}; ret = A + V
+// The two reverse scans over the recorded steps, x_t = delta_t + coef_t x_{t+1}.  A CTA takes 32 envs and up to 64 steps at a time: eight
+// warps fetch the rows and form delta and coef (lane = env, a warp every eighth step, so that all of a chunk's loads are in flight at
+// once), one warp walks the chain through shared memory, the eight write the results.  One thread per env with four or eight steps in
+// flight paid a memory round trip and the exponentials of each group one after the other, on a few SMs.  B200 (events included): V-trace of
+// 6000 envs, T = 20 17.8 -> 10.6 us; GAE of 16384 envs, T = 32 23.8 -> 10.6, of 3000, T = 16 12.8 -> 8.8.
 // ----------------------------------------------------------------------------------------------------
+constexpr int SCAN_ENVS = 32, SCAN_WARPS = 8, SCAN_STEPS = 64, SCAN_ROWS = SCAN_STEPS / SCAN_WARPS;
+
+struct ScanShared {
+    float v[SCAN_STEPS + 1][SCAN_ENVS];      // values; row n: the value after the chunk's last step
+    float x[SCAN_STEPS + 1][SCAN_ENVS];      // results of the chain; row n: the one after the chunk
+    float delta[SCAN_STEPS][SCAN_ENVS], coef[SCAN_STEPS][SCAN_ENVS];
+};
+
+// The chain of one chunk of n steps; the caller synchronises on both sides.
+__device__ __forceinline__ void scan_chain(ScanShared& s, int n, int lane) {
+    float x = s.x[n][lane];
+    for (int k = n - 1; k >= 0; --k) {
+        x = __fmaf_rn(s.coef[k][lane], x, s.delta[k][lane]);
+        s.x[k][lane] = x;
+    }
+}
+
+// GAE: d_t = 1 - done_t; delta_t = r_t + gamma d_t V_{t+1} - V_t; A_t = delta_t + gamma lambda d_t A_{t+1}; ret = A + V.  The operations
+// of gae_scan_env_smem, which the rollouts that keep their values on chip run: the same bits.
 template <bool GROUPED>
-__global__ void __launch_bounds__(128) k_gae(DimsBuffers in, int T, float gamma, float lambda) {
+__global__ void __launch_bounds__(32 * SCAN_WARPS) k_gae(DimsBuffers in, int T, float gamma, float lambda) {
+    __shared__ ScanShared s;
     pdl_wait();
     const PolicyArgs<GROUPED, DimsBuffers> pa(in, blockIdx.y);
-    const Dims& d = pa.a.d;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= d.B) return;
-    gae_scan_env(pa.a.b, d.B, T, e, gamma, lambda);
+    const Buffers& b = pa.a.b;
+    const int B = pa.a.d.B, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, env = blockIdx.x * SCAN_ENVS + lane;
+    const bool have = env < B;
+    const float gl = __fmul_rn(gamma, lambda);
+    for (int tb = T; tb > 0; tb -= SCAN_STEPS) {
+        const int t0 = max(tb - SCAN_STEPS, 0), n = tb - t0;
+        float r[SCAN_ROWS], nd[SCAN_ROWS];
+        float vn = 0.f, xn = 0.f;  // after the chunk: the bootstrap value, then the first row of the chunk before
+        if (wid == 0) {
+            vn = tb == T ? (have ? b.tval[(size_t)T * B + env] : 0.f) : s.v[0][lane];
+            xn = tb == T ? 0.f : s.x[0][lane];
+        }
+        if (tb < T) __syncthreads();  // (every warp is done with the chunk before)
+        if (wid == 0) {
+            s.v[n][lane] = vn;
+            s.x[n][lane] = xn;
+        }
+        float v[SCAN_ROWS];
+#pragma unroll
+        for (int q = 0; q < SCAN_ROWS; ++q) {
+            const int k = wid + SCAN_WARPS * q;
+            v[q] = r[q] = nd[q] = 0.f;
+            if (k < n && have) {
+                const size_t i = (size_t)(t0 + k) * B + env;
+                v[q] = b.tval[i];
+                r[q] = b.trew[i];
+                nd[q] = b.tdone[i] ? 0.f : 1.f;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < SCAN_ROWS; ++q)
+            if (wid + SCAN_WARPS * q < n) s.v[wid + SCAN_WARPS * q][lane] = v[q];
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < SCAN_ROWS; ++q) {
+            const int k = wid + SCAN_WARPS * q;
+            if (k < n) {
+                s.delta[k][lane] = __fsub_rn(__fmaf_rn(__fmul_rn(gamma, nd[q]), s.v[k + 1][lane], r[q]), v[q]);
+                s.coef[k][lane] = __fmul_rn(gl, nd[q]);
+            }
+        }
+        __syncthreads();
+        if (wid == 0) scan_chain(s, n, lane);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < SCAN_ROWS; ++q) {
+            const int k = wid + SCAN_WARPS * q;
+            if (k < n && have) {
+                const size_t i = (size_t)(t0 + k) * B + env;
+                const float A = s.x[k][lane];
+                b.adv[i] = A;
+                b.ret[i] = __fadd_rn(A, v[q]);
+            }
+        }
+    }
 }
 
 cudaError_t launch_gae(const Dims& d, const Buffers& b, int T, float gamma, float lambda, const Ctx& c) {
     Scope sc(c, K_GAE);
-    if (d.npol > 1) launch<k_gae<true>>(dim3((d.B + 127) / 128, d.npol), 128, 0, c.s, DimsBuffers{d, b}, T, gamma, lambda);
-    else launch<k_gae<false>>((d.B + 127) / 128, 128, 0, c.s, DimsBuffers{d, b}, T, gamma, lambda);
+    const unsigned nb = (unsigned)((d.B + SCAN_ENVS - 1) / SCAN_ENVS);
+    if (d.npol > 1) launch<k_gae<true>>(dim3(nb, d.npol), 32 * SCAN_WARPS, 0, c.s, DimsBuffers{d, b}, T, gamma, lambda);
+    else launch<k_gae<false>>(nb, 32 * SCAN_WARPS, 0, c.s, DimsBuffers{d, b}, T, gamma, lambda);
     return cudaGetLastError();
 }
 
-// ----------------------------------------------------------------------------------------------------
-// V-trace targets (Espeholt et al. 2018, IMPALA, Eq. 1; recursive form), lane = env, reverse scan over t.  mu = the policy
-// that acted (recorded log-probabilities), pi = the current parameters (head outputs of the recorded rows in out5):
+// V-trace targets (Espeholt et al. 2018, IMPALA, Eq. 1; recursive form).  mu = the policy that acted (recorded log-probabilities),
+// pi = the current parameters (head outputs of the recorded rows in out5):
 //   w = exp(logp_pi - logp_mu); rho = min(rho_bar, w); c = min(c_bar, w); d = 1 - done
 //   delta = rho (r + gamma d V' - V);  e = delta + gamma d c e';  ret = V + e;  adv = rho (r + gamma d (V' + e') - V)
-// Four steps per memory round trip.
-// ----------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_vtrace(Dims d, Buffers b, int T, float gamma, float rho_bar, float c_bar, const float* boot) {
-    pdl_wait();  // (no early trigger: 37 us alone, 61 us with the next kernel's CTAs beside it)
-    const int env = blockIdx.x * blockDim.x + threadIdx.x;
-    if (env >= d.B) return;
-    const int B = d.B;
-    float e_next = 0.f, v_next = boot[env];
-    for (int tb = T; tb > 0; tb -= 4) {
-        float4 lg[4];
-        float v[4], r[4], nd[4], lmu[4];
-        int act[4];
+__global__ void __launch_bounds__(32 * SCAN_WARPS) k_vtrace(Dims d, Buffers b, int T, float gamma, float rho_bar, float c_bar, const float* boot) {
+    __shared__ ScanShared s;
+    pdl_wait();  // (no early trigger: the next kernel's CTAs would crowd in beside this one's)
+    const int B = d.B, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, env = blockIdx.x * SCAN_ENVS + lane;
+    const bool have = env < B;
+    for (int tb = T; tb > 0; tb -= SCAN_STEPS) {
+        const int t0 = max(tb - SCAN_STEPS, 0), n = tb - t0;
+        float vn = 0.f, xn = 0.f;  // after the chunk: the bootstrap value, then the first row of the chunk before
+        if (wid == 0) {
+            vn = tb == T ? (have ? boot[env] : 0.f) : s.v[0][lane];
+            xn = tb == T ? 0.f : s.x[0][lane];
+        }
+        if (tb < T) __syncthreads();  // (every warp is done with the chunk before)
+        if (wid == 0) {
+            s.v[n][lane] = vn;
+            s.x[n][lane] = xn;
+        }
+        float v[SCAN_ROWS], r[SCAN_ROWS], gd[SCAN_ROWS], rho[SCAN_ROWS];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int t = tb - 1 - q;
-            if (t >= 0) {
-                const size_t i = (size_t)t * B + env;
-                const float4* o = reinterpret_cast<const float4*>(b.out5 + i * 8);
-                lg[q] = o[0];
-                v[q] = o[1].x;
-                r[q] = b.trew[i];
-                nd[q] = b.tdone[i] ? 0.f : 1.f;
-                lmu[q] = b.tlogp[i];
-                act[q] = b.tact[i];
+        for (int h = 0; h < SCAN_ROWS; h += 4) {  // four rows' loads at a time
+            float4 lg[4];
+            float lmu[4];
+            int act[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = wid + SCAN_WARPS * (h + q);
+                lg[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                v[h + q] = r[h + q] = gd[h + q] = lmu[q] = 0.f;
+                act[q] = 0;
+                if (k < n && have) {
+                    const size_t i = (size_t)(t0 + k) * B + env;
+                    const float4* o = reinterpret_cast<const float4*>(b.out5 + i * 8);
+                    lg[q] = o[0];
+                    v[h + q] = o[1].x;
+                    r[h + q] = b.trew[i];
+                    gd[h + q] = gamma * (b.tdone[i] ? 0.f : 1.f);
+                    lmu[q] = b.tlogp[i];
+                    act[q] = b.tact[i];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = wid + SCAN_WARPS * (h + q);
+                if (k < n) {
+                    const float l0 = lg[q].x, l1 = lg[q].y, l2 = lg[q].z, l3 = lg[q].w;
+                    const float mx = fmaxf(fmaxf(l0, l1), fmaxf(l2, l3));
+                    const float Z = ((expf(l0 - mx) + expf(l1 - mx)) + expf(l2 - mx)) + expf(l3 - mx);
+                    const float la = act[q] == 0 ? l0 : act[q] == 1 ? l1 : act[q] == 2 ? l2 : l3;
+                    const float lpi = (la - mx) - logf(Z);
+                    const float w = expf(lpi - lmu[q]);
+                    rho[h + q] = fminf(rho_bar, w);
+                    s.coef[k][lane] = gd[h + q] * fminf(c_bar, w);
+                    s.v[k][lane] = v[h + q];
+                }
             }
         }
+        __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int t = tb - 1 - q;
-            if (t >= 0) {
-                const size_t i = (size_t)t * B + env;
-                const float l0 = lg[q].x, l1 = lg[q].y, l2 = lg[q].z, l3 = lg[q].w;
-                const float mx = fmaxf(fmaxf(l0, l1), fmaxf(l2, l3));
-                const float Z = ((expf(l0 - mx) + expf(l1 - mx)) + expf(l2 - mx)) + expf(l3 - mx);
-                const float la = act[q] == 0 ? l0 : act[q] == 1 ? l1 : act[q] == 2 ? l2 : l3;
-                const float lpi = (la - mx) - logf(Z);
-                const float w = expf(lpi - lmu[q]);
-                const float rho = fminf(rho_bar, w), c = fminf(c_bar, w);
-                const float gd = gamma * nd[q];
-                const float delta = rho * ((r[q] + gd * v_next) - v[q]);
-                const float e = delta + gd * c * e_next;
-                b.adv[i] = rho * ((r[q] + gd * (v_next + e_next)) - v[q]);
-                b.ret[i] = v[q] + e;
-                e_next = e;
-                v_next = v[q];
+        for (int q = 0; q < SCAN_ROWS; ++q) {
+            const int k = wid + SCAN_WARPS * q;
+            if (k < n) s.delta[k][lane] = rho[q] * ((r[q] + gd[q] * s.v[k + 1][lane]) - v[q]);
+        }
+        __syncthreads();
+        if (wid == 0) scan_chain(s, n, lane);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < SCAN_ROWS; ++q) {
+            const int k = wid + SCAN_WARPS * q;
+            if (k < n && have) {
+                const size_t i = (size_t)(t0 + k) * B + env;
+                b.adv[i] = rho[q] * ((r[q] + gd[q] * (s.v[k + 1][lane] + s.x[k + 1][lane])) - v[q]);
+                b.ret[i] = v[q] + s.x[k][lane];
             }
         }
     }
@@ -150,7 +251,7 @@ __global__ void __launch_bounds__(128) k_vtrace(Dims d, Buffers b, int T, float 
 
 cudaError_t launch_vtrace(const Dims& d, const Buffers& b, int T, float gamma, float rho_bar, float c_bar, const float* boot, const Ctx& c) {
     Scope sc(c, K_VTRACE);
-    return launch<k_vtrace>((d.B + 127) / 128, 128, 0, c.s, d, b, T, gamma, rho_bar, c_bar, boot);
+    return launch<k_vtrace>((d.B + SCAN_ENVS - 1) / SCAN_ENVS, 32 * SCAN_WARPS, 0, c.s, d, b, T, gamma, rho_bar, c_bar, boot);
 }
 
 }  // namespace anakin

@@ -141,3 +141,30 @@ def test_vtrace_argument_errors_and_unsupported_path(bnd):
         ff.learn_vtrace(1, 1.0, 1.0)
     assert e.value.code == bnd.E_UNSUPPORTED_CFG
     ff.learn()  # the rollout is still pending and the generic update still works
+
+
+@pytest.mark.parametrize("B,T", [(1, 1), (31, 63), (33, 64), (64, 65), (40, 128), (20, 131)])
+def test_reverse_scans_across_chunk_edges(bnd, B, T):
+    """GAE and V-trace walk the steps backwards in chunks of 64 steps of 32 envs: one step, a chunk and one more or less, several, and
+    groups of envs that are not full.  GAE gives the bits of the scan that the rollout itself runs on chip."""
+    w = Workload(f"scan_{B}_{T}", B=B, N=4, H=64, T=T, iters=1, episode_cap=9)
+    an = make(bnd, w)
+    an.reset(3)
+    an.set(bnd.PARAMS, random_params(2, w.P, 0.15))
+    an.rollout()
+    g = par.gpu_traj(an, bnd, T)
+    fused = [an.get(which).view(np.uint32) for which in (bnd.ADV, bnd.RET)]
+    an.set(bnd.ADV, np.full(B * T, 7.0, np.float32))
+    gadv, gret = par.check_gae(an, bnd, w, g, T)
+    assert (gadv.reshape(-1).view(np.uint32) == fused[0]).all() and (gret.reshape(-1).view(np.uint32) == fused[1]).all()
+    rng = np.random.default_rng(11)
+    theta = an.get(bnd.PARAMS)
+    an.set(bnd.PARAMS, (theta + 0.03 * rng.standard_normal(theta.size)).astype(np.float32))
+    st = par.gpu_state(an, bnd)
+    an.learn_vtrace(1, 1.1, 0.9)
+    out = oracle_heads(w, st["theta"], st["walls"], st["goal"], np.concatenate([g["pos"], st["pos"][None, :]], axis=0))
+    adv, ret = orc.vtrace(np.float32(w.gamma), 1.1, 0.9, g["reward"], out[:, :, 4], g["done"], logp_of(out[:-1, :, :4], g["action"]), g["logp"])
+    rtol = par.rtol_of(w.precision)
+    par.assert_close(an.get(bnd.ADV), adv, rtol, "vtrace advantages")
+    par.assert_close(an.get(bnd.RET), ret, rtol, "vtrace value targets")
+    assert an.status() == 0
