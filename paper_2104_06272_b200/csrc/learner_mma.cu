@@ -1427,10 +1427,18 @@ static void dh1a_shape(const Dims& d, int T, int* nx, int* ts) {
     *nx = std::min(m_tiles * *ts, cap);
 }
 
-// Splits of the wall and goal planes' K range (rows of S).
+// Splits of the wall and goal planes' K range (rows of S), at least two 64-row chunks each: one wave of the launch's tiles (128 cells of
+// either plane x 256 columns), of CTAs that take an SM each above 128 columns and share one below.  B200 (events included), this rule / as
+// many as two waves of the wall tiles alone: 65536 envs, 10 x 10, H = 256 29 / 39 us and 21 / 24 in the reduction, 6000 envs, 12 x 12,
+// H = 256 21 / 29 and 21 / 26, 2500 envs, 9 x 9, H = 128 12.2 / 15.4 and 12 / 13; one chunk at least instead of two gains nothing more.
 static int env_splits(const Dims& d, int rows) {
-    const int bt = d.H == 128 || d.H >= 256 ? 128 : 64;
-    return splits_for(rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
+    if (d.npol > 1) {  // (the warp-level kernel's tiles)
+        const int bt = d.H == 128 ? 128 : 64;
+        return splits_for(rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
+    }
+    const int tiles = ((d.C + 128) / 128 + (d.C + 127) / 128) * ((d.H + 255) / 256), slots = d.H > 128 ? 148 : 296;
+    const int most = rows / 128 > 0 ? rows / 128 : 1, least = (rows + 8191) / 8192;  // (one accumulator takes at most 8192 rows)
+    return std::max(std::min(std::min(slots / tiles, 128), most), std::min(least, 128));
 }
 
 // dW2 inside the heads kernel: hidden width 128 or 256, one policy.
@@ -1468,7 +1476,7 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
     }
-    p->ns_env = splits_for(d.B, tiles_ch, 128);
+    p->ns_env = d.npol > 1 ? splits_for(d.B, tiles_ch, 128) : env_splits(d, d.B);
     if (dh1_agent_tc_supported(d) && d.npol <= 1) {  // (one agent-plane partial per CTA of the fused kernel, any T <= Tmax)
         const int cap = 148 / (H / DH1A_UNITS);
         p->ns_agent = std::max(p->ns_agent, std::min(cap, (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax)));
