@@ -91,9 +91,8 @@ __global__ void __launch_bounds__(Back128Cfg<PREC>::THREADS, 1)
     uint64_t* qempty = qfull + 2;          // [2] ... and read (the builder warps arrive)
     uint64_t* dfull = qempty + 2;          // [2] dh2 written (the builder warps arrive)
     uint64_t* mdone = dfull + 2;           // [2] dW2 and dh1 of a tile have finished
-    uint64_t* tiles_full = mdone + 2;      // [2] dh1^T and the one-hot of a tile written (the epilogue warps arrive; two barriers: a warp
-                                           // may arrive for the next tile before another has for this one)
-    uint64_t* tiles_free = tiles_full + 2; // the agent MMAs of a tile have finished
+    uint64_t* tiles_full = mdone + 2;      // dh1^T and the one-hot of a tile written (the epilogue warps arrive)
+    uint64_t* tiles_free = tiles_full + 1; // the agent MMAs of a tile have finished
     uint64_t* wstage = tiles_free + 1;     // W2 landed in its staging boxes
     uint64_t* wfull = wstage + 1;          // ... and is in tensor memory (the epilogue warps arrive)
     uint32_t* tmem_slot = (uint32_t*)(wfull + 1);
@@ -120,8 +119,8 @@ __global__ void __launch_bounds__(Back128Cfg<PREC>::THREADS, 1)
             tc::mbar_init(&qempty[i], Cfg::BUILD_WARPS);
             tc::mbar_init(&dfull[i], Cfg::BUILD_WARPS);
             tc::mbar_init(&mdone[i], 1);
-            tc::mbar_init(&tiles_full[i], Cfg::EPI_WARPS);
         }
+        tc::mbar_init(tiles_full, Cfg::EPI_WARPS);
         tc::mbar_init(tiles_free, 1);
         tc::mbar_init(wstage, 1);
         tc::mbar_init(wfull, Cfg::EPI_WARPS);
@@ -189,7 +188,7 @@ __global__ void __launch_bounds__(Back128Cfg<PREC>::THREADS, 1)
             const uint32_t id_w2 = tc::umma_idesc<PREC>(128, H, true, true), id_dh1 = tc::umma_idesc<PREC>(128, BM, false, false);
             const uint32_t id_agent = tc::umma_idesc<PREC>(128, 128, false, true);
             auto agent_mma = [&](int v) {
-                ok = tc::warp_all(tc::mbar_wait(&tiles_full[v & 1], (uint32_t)(v >> 1) & 1u));
+                ok = tc::warp_all(tc::mbar_wait(tiles_full, (uint32_t)v & 1u));
                 if (!ok) return;
                 tc::tc_fence_after();
                 if (tc::elect_one()) {
@@ -570,8 +569,11 @@ __global__ void __launch_bounds__(Back128Cfg<PREC>::THREADS, 1)
                     if (PL == 2) tc::tmem_st8(acc + 8, lo);
                 }
                 tc::tmem_st_wait();
+                // The MMAs of the tile before have read the one-hot tile.  Every warp waits for every tile's, also those that write no row of it: a
+                // wait for a phase is only right from the one before it (two behind, it returns at once, and the accumulator would be read
+                // before its last MMAs), and no warp arrives for a tile before all have for the one before.
+                if (g >= 1) ok = tc::mbar_wait(tiles_free, (uint32_t)(g - 1) & 1u);
                 if (half == 0 && q < BM / 32) {  // the one-hot row of env j
-                    if (g >= 1) ok = tc::mbar_wait(tiles_free, (uint32_t)(g - 1) & 1u);  // the MMAs of the tile before have read the tile
                     if (prev_off >= 0) *reinterpret_cast<uint16_t*>(sO + prev_off) = 0;
                     prev_off = -1;
                     if (cell >= 0 && cell < 128) {
@@ -584,7 +586,7 @@ __global__ void __launch_bounds__(Back128Cfg<PREC>::THREADS, 1)
                 tc::tc_fence_before();
                 __syncwarp();
                 if (!ok) break;
-                if (lane == 0) tc::mbar_arrive(&tiles_full[buf]);
+                if (lane == 0) tc::mbar_arrive(tiles_full);
             }
             // S (sum over t of dh1) as two 16-bit planes [ts*B][H]: an fp32 sum keeps two terms in either workload
             if (ok) {

@@ -1,6 +1,8 @@
 // dh1 = (dh2 W2^T) gated by h1 > 0, S = sum over t of dh1, AND the agent plane of dW1 = onehot(pos)^T dh1, in one
 // tcgen05 kernel: dh1 never goes to HBM.
 //
+// Serves H = 256, and H = 128 on boards of more than 128 cells (smaller ones run back128_tc.cu).
+//
 // Backward pass through the second layer of the policy/value MLP and the first-layer weight gradient of the rows the
 // agent's position selects (the update half of the Anakin minimal unit, Podracer paper, Section 3.1; Figure 2, top).
 //
@@ -574,7 +576,8 @@ cudaError_t launch_t(const LearnArgs& a, int grid_x, float* part_agent, size_t p
 template <int NC>
 cudaError_t launch_nc(const LearnArgs& a, int prec, int grid_x, float* part_agent, size_t part_stride, cudaStream_t s) {
     if (a.d.H == 256) return prec == 1 ? launch_t<256, 1, NC>(a, grid_x, part_agent, part_stride, s) : launch_t<256, 0, NC>(a, grid_x, part_agent, part_stride, s);
-    return prec == 1 ? launch_t<128, 1, NC>(a, grid_x, part_agent, part_stride, s) : launch_t<128, 0, NC>(a, grid_x, part_agent, part_stride, s);
+    if constexpr (NC == 2) return prec == 1 ? launch_t<128, 1, NC>(a, grid_x, part_agent, part_stride, s) : launch_t<128, 0, NC>(a, grid_x, part_agent, part_stride, s);
+    return cudaErrorNotSupported;  // (H = 128 on boards of up to 128 cells: back128_tc.cu)
 }
 
 }  // namespace

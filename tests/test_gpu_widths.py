@@ -1,6 +1,7 @@
 """Hidden widths besides the headline ones, in both precisions, on the GPU against the oracle stage by stage (needs a B200):
 partial column tiles (384 is one and a half of 256), the smallest batches, row counts around the tiles' edges, boards whose
 cell count is and is not a multiple of 64, batches on either side of the base-GEMM and tile-size rules."""
+import numpy as np
 import pytest
 
 from paper_2104_06272_b200.workloads import Workload, random_params
@@ -54,6 +55,24 @@ def test_width_one_iteration_stage_by_stage(bnd, H, prec, B, N, T):
         par.check_iteration(an, bnd, w, 11)
     finally:
         print(w.name, "worst error / bound:", {k: round(v, 3) for k, v in par.MARGINS.items()})
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_width_128_gradients_do_not_depend_on_timing(bnd, prec):
+    """Two handles in lockstep over 60 passes of two to three tiles of 64 envs a CTA: the same bits.  (The warps of the fused backward
+    kernel hand tiles on through mbarriers; one that read the agent plane's accumulator ahead of its last MMAs showed here in one
+    pass of fifteen in bf16.)"""
+    pair = []
+    for _ in range(2):
+        an = bnd.Anakin(bnd.make_cfg(148 * 128 + 77, 8, 128, 5, precision=prec, episode_cap=4))
+        an.reset(6)
+        pair.append(an)
+    for i in range(60):
+        grads = []
+        for an in pair:
+            an.run(1)
+            grads.append(an.get(bnd.GRADS))
+        assert (grads[0].view(np.uint32) == grads[1].view(np.uint32)).all(), f"pass {i}"
 
 
 LONG_SUMS = [
