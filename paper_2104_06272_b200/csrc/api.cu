@@ -118,7 +118,9 @@ size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* o
     b.h2 = (float*)take(wide ? std::max(h2_bytes, wide_scratch_bytes(d)) : h2_bytes);
     b.out5 = (float*)take(R * 8 * 4);
     b.vboot = (float*)take(B * 4);
-    b.dh2 = back128_supported(d) ? nullptr : (float*)take(R * H * (x3 ? 6 : wide ? 2 : 4));
+    // (at H = 128 on boards of up to 128 cells nothing goes there any more, dh2 stays on chip; the workspace keeps its size, the same on every
+    // board)
+    b.dh2 = (float*)take(R * H * (x3 ? 6 : wide ? 2 : 4));
     b.dh1 = dh1_on_chip ? nullptr : b.h2;
     // t-slices of two 16-bit planes, or three planes
     b.S = (float*)take((dh1_on_chip ? (size_t)most_s_rows((int)B) : 4 * B) * H * 4);

@@ -79,7 +79,7 @@ struct Buffers {
     float* h2;       // [R][H]
     float* out5;     // [R][8] head outputs (4 logits, value) of every recorded row, saved by the tensor-pipe rollout
     float* vboot;    // [B] value of the state after the last recorded step under the CURRENT parameters (replay mode 2)
-    float* dh2;      // [R][H] (null where it stays on chip)
+    float* dh2;      // [R][H] (not written where it stays on chip)
     float* dh1;      // [R][H]
     float* S;        // [B][H]  sum over t of dh1
     float* part;     // split-K partial gradients (LearnPlan)

@@ -1431,8 +1431,8 @@ static void dh1a_shape(const Dims& d, int T, int* nx, int* ts) {
 // either plane x 256 columns), of CTAs that take an SM each above 128 columns and share one below.  B200 (events included), this rule / as
 // many as two waves of the wall tiles alone: 65536 envs, 10 x 10, H = 256 29 / 39 us and 21 / 24 in the reduction, 6000 envs, 12 x 12,
 // H = 256 21 / 29 and 21 / 26, 2500 envs, 9 x 9, H = 128 12.2 / 15.4 and 12 / 13; one chunk at least instead of two gains nothing more.
-static int env_splits(const Dims& d, int rows) {
-    if (d.npol > 1) {  // (the warp-level kernel's tiles)
+static int env_splits(const Dims& d, int rows, bool many) {
+    if (many) {  // (many policies: the warp-level kernel's tiles)
         const int bt = d.H == 128 ? 128 : 64;
         return splits_for(rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
     }
@@ -1476,11 +1476,13 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
     }
-    p->ns_env = d.npol > 1 ? splits_for(d.B, tiles_ch, 128) : env_splits(d, d.B);
+    p->ns_env = d.npol > 1 ? splits_for(d.B, tiles_ch, 128) : env_splits(d, d.B, false);
+    int env_room = std::max(splits_for(d.B, tiles_ch, 128), env_splits(d, d.B, false));  // (the same for one policy and for many)
     if (dh1_agent_tc_supported(d) && d.npol <= 1) {  // (one agent-plane partial per CTA of the fused kernel, any T <= Tmax)
         const int cap = 148 / (H / DH1A_UNITS);
         p->ns_agent = std::max(p->ns_agent, std::min(cap, (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax)));
-        p->ns_env = env_splits(d, most_s_rows(d.B));
+        p->ns_env = env_splits(d, most_s_rows(d.B), false);
+        env_room = std::max(env_room, p->ns_env);
     }
     if (back128_supported(d)) {  // (one partial of everything per CTA)
         p->ns_w2 = p->ns_agent = std::min(148, (d.B + 63) / 64 * std::min(MAX_SLICES, d.Tmax));
@@ -1488,7 +1490,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     if (H == 64) {  // (one partial per CTA of the fused kernel; its slices of the steps are rows of S)
         const int units = d.B > 64 ? (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax) : (d.Tmax + 128 / d.B - 1) / (128 / d.B);  // (of any T <= Tmax)
         p->ns_w2 = p->ns_agent = std::min(std::max(148 / d.npol, 1), units);
-        p->ns_env = env_splits(d, most_s_rows(d.B));
+        p->ns_env = env_splits(d, most_s_rows(d.B), d.npol > 1);
+        env_room = std::max({env_room, env_splits(d, most_s_rows(d.B), false), env_splits(d, most_s_rows(d.B), true)});
     }
     const size_t tiles32 = (R + 31) / 32;
     size_t hg = (size_t)heads_grid_max(H);
@@ -1503,8 +1506,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     size_t off = 0;
     p->off_w2 = off; off += (size_t)w2_slots * H * H;
     p->off_agent = off; off += (size_t)p->ns_agent * C * H;
-    p->off_walls = off; off += (size_t)p->ns_env * (C + 1) * H;
-    p->off_goal = off; off += (size_t)p->ns_env * C * H;
+    p->off_walls = off; off += (size_t)env_room * (C + 1) * H;
+    p->off_goal = off; off += (size_t)env_room * C * H;
     p->off_small = off; off += (size_t)p->ns_small * p->small_stride;
     p->part_floats = off;
     p->loss_blocks = p->heads_grid;
@@ -1627,7 +1630,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         int nx;
         back64_shape(d, T, &nx, &a.ts);
         a.reg[1].ns = a.reg[4].ns = nx;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped);
         Scope sc(c, K_DH1);
         CK(launch_back64(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
@@ -1636,7 +1639,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         back128_shape(d, T, &nx, &a.ts);
         for (int q = 4; q < 8; ++q) a.reg[q].ns = nx;
         a.reg[1].ns = pl.loss_blocks = nx;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped);
         Scope sc(c, K_HEADS_BWD);  // (profiled under the name of what it starts with)
         CK(launch_back128(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
@@ -1644,7 +1647,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         int nx;
         dh1a_shape(d, T, &nx, &a.ts);
         a.reg[1].ns = nx;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped);
         Scope sc(c, K_DH1);
         CK(launch_dh1_agent_tc(a, PREC, nx, b.part + pl.off_agent, CH, s));
         fused_agent = true;
