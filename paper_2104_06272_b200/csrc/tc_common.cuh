@@ -52,11 +52,6 @@ __device__ __forceinline__ float lds_f1(uint32_t addr) {
     asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
     return v;
 }
-__device__ __forceinline__ uint64_t lds_b64(uint32_t addr) {
-    uint64_t v;
-    asm("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
-    return v;
-}
 __device__ __forceinline__ float4 lds_f4(uint32_t addr) {
     float4 v;
     asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
