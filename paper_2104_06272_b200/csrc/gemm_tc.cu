@@ -11,7 +11,8 @@
 //   warp 0 (one lane)  issues TMA loads of the operand planes (64 x 64 boxes, 128-byte swizzle) into a ring of two to four stages,
 //   warps 2-5          for the one-hot A operand: write the 0/1 tile straight into the swizzled layout instead of loading it,
 //   warp 1             issues tcgen05.mma (the whole warp walks the loop, an elected lane issues): for fp32 workloads three MMAs per
-//                      k16 (lo*hi, hi*lo, hi*hi fp16 terms) into one fp32 accumulator, six with three-term operands; commits free the stage,
+//                      k16 (lo*hi, hi*lo, hi*hi fp16 terms) into one fp32 accumulator, six with three-term operands;
+//                      the small terms of the wall and goal planes go into an accumulator of their own; commits free the stage,
 //   warps 2-5          after the last chunk: tcgen05.ld the accumulator and store the partial tile.
 // Long K ranges (plane operands): the tensor core's fp32 accumulation rounds toward zero, which biases a sum of many
 // thousand MMAs by more than the fp32 workloads' 1e-4 bound (measured: -2e-4 after 65,536 rows; fp32 workloads only).  The K range of a CTA
@@ -120,9 +121,11 @@ struct GemmTcCfg {
     static constexpr bool X3 = PREC == 2 && DEEP;
     static constexpr int GROUP = X3 ? 1 : 64;
     static constexpr int EPI_THREADS = X3 ? 256 : 128;
-    // three-term B beside an exact synthesized A: the leading products in one accumulator, the small terms in a second one (every
-    // MMA rounds toward zero at its accumulator's magnitude), added at the end
-    static constexpr bool SPLIT = PREC == 2 && !DEEP;
+    // several terms of B beside an exact synthesized A: the leading products in one accumulator, the small terms in a second one (every
+    // MMA rounds toward zero at its accumulator's magnitude), added at the end.  8192 rows, the most that one split has, are then 512
+    // MMAs in the accumulator that counts; in one for both terms they were 1024.  In time it is nothing: 65536 envs,
+    // 10 x 10, H = 256 29.1 us with and without, 16384, 16 x 16, H = 1024 55.6, 303104, 12 x 12, H = 256 154.
+    static constexpr bool SPLIT = !DEEP && BPL >= 2;
     static constexpr int TMEM_COLS = FLUSH || SPLIT ? 2 * BN : BN;
 };
 
@@ -232,10 +235,10 @@ __global__ void __launch_bounds__((GemmTcCfg<BN, APL, BPL, AMODE == A_PLANES, PR
                     uint32_t accum = (cg > 0 || k16 > 0) ? 1u : 0u;
                     if (APL == 2) { tc::umma(acc, tc::umma_desc(sa + Cfg::A_PLANE + k16 * 2048, Cfg::BOX, 1024), b_hi, idesc, accum); accum = 1u; }
                     if (Cfg::SPLIT) {
-                        tc::umma(acc + BN, a_hi, tc::umma_desc(sb + 2 * Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum);
-                        tc::umma(acc + BN, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, 1u);
+                        if (BPL == 3) tc::umma(acc + BN, a_hi, tc::umma_desc(sb + 2 * Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum);
+                        tc::umma(acc + BN, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, BPL == 3 ? 1u : accum);
                     }
-                    if (BPL == 2) { tc::umma(acc, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
+                    if (BPL == 2 && !Cfg::SPLIT) { tc::umma(acc, a_hi, tc::umma_desc(sb + Cfg::B_PLANE + k16 * 2048, Cfg::BOX, 1024), idesc, accum); accum = 1u; }
                     tc::umma(acc, a_hi, b_hi, idesc, accum);
                 }
                 tc::umma_commit(&bars[STAGES + s]);  // frees the stage when these MMAs are done

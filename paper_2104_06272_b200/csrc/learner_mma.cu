@@ -1437,8 +1437,8 @@ static int env_splits(const Dims& d, int rows, bool many) {
         return splits_for(rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
     }
     const int tiles = ((d.C + 128) / 128 + (d.C + 127) / 128) * ((d.H + 255) / 256), slots = d.H > 128 ? 148 : 296;
-    const int most = rows / 128 > 0 ? rows / 128 : 1, least = (rows + 8191) / 8192;  // (one accumulator takes at most 8192 rows)
-    return std::max(std::min(std::min(slots / tiles, 128), most), std::min(least, 128));
+    const int most = rows / 128 > 0 ? rows / 128 : 1, least = (rows + 8191) / 8192;  // (one split has at most 8192 rows, whatever the batch)
+    return std::max(std::min(std::min(slots / tiles, 128), most), least);
 }
 
 // dW2 inside the heads kernel: hidden width 128 or 256, one policy.

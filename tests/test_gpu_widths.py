@@ -4,6 +4,7 @@ cell count is and is not a multiple of 64, batches on either side of the base-GE
 import numpy as np
 import pytest
 
+from oracle import binding as orc
 from paper_2104_06272_b200.workloads import Workload, random_params
 from tests import parity as par
 
@@ -106,6 +107,48 @@ def test_gradients_of_long_sums(bnd, H, prec, B, N, T, bias):
     finally:
         print(w.name, "worst error / bound:", {k: round(v, 3) for k, v in par.MARGINS.items()})
     assert an.status() == 0
+
+
+@pytest.mark.parametrize("H,B,N", [(64, 606208, 12), (256, 303104, 12), (64, 4194304, 3), (32, 606208, 5), (1024, 65536, 16)])
+def test_wall_plane_sums_are_not_biased(bnd, H, B, N):
+    """fp32 sums over the envs on the tensor core, which rounds every addition toward zero.  Every row adds the same value here (all gates
+    open, no policy gradient, returns off by a constant), so what the additions lose has one sign.  The leading 16-bit terms of the at most
+    8192 rows of a split are equal numbers of 11 bits: 24 bits hold their sum, and it loses nothing as long as no other term goes into the
+    same accumulator.  What is left: a value as two fp16 terms, 2^-22, and dh1 itself, 3 H / 16 MMAs each of which loses less than a unit in
+    the last place, 2^-23, of a sum that is on average half grown.  Boards of two row tiles a plane, where a split has most rows, a batch of
+    more than 128 such splits, three-term operands.  (With both terms in one accumulator: 6e-6 to 8e-6, 1e-4 in one of 128 splits.)"""
+    an = bnd.Anakin(bnd.make_cfg(B, N, H, 1, entropy_coef=0.0))
+    an.reset(7)
+    rng = np.random.default_rng(3)
+    sl = orc.Dims(N, H).slices()
+    theta = np.zeros(an.P, np.float32)
+    theta[sl["W1"]] = 0.1 * rng.standard_normal(3 * N * N * H) / N
+    theta[sl["b1"]] = 2.0
+    theta[sl["W2"]] = rng.uniform(0.5, 1.5, H * H) / H
+    theta[sl["b2"]] = 1.0
+    theta[sl["Wh"]].reshape(H, 5)[:, 4] = rng.uniform(0.5, 1.5, H) / H
+    an.set(bnd.PARAMS, theta)
+    an.rollout()
+    value = an.get(bnd.TRAJ_VALUE)[:B]
+    ret = (value + 64).astype(np.float32)  # (far off, so that rounding of the values themselves does not count)
+    an.set(bnd.ADV, np.zeros(B, np.float32))
+    an.set(bnd.RET, ret)
+    an.update()
+    assert an.status() == 0
+    grads = an.get(bnd.GRADS)
+    # in double: dL/dvalue of a row, down through open gates, times the number of rows of a bias, of a wall cell, of a goal cell
+    d_out = 2 * float(bnd.make_cfg(B, N, H, 1).value_coef) * (value.astype(np.float64) - ret).mean()
+    d_h1 = d_out * theta[sl["W2"]].reshape(H, H).astype(np.float64) @ theta[sl["Wh"]].reshape(H, 5)[:, 4]
+    walls, goal = an.get(bnd.ENV_WALLS).reshape(B, -1), an.get(bnd.ENV_GOAL)
+    cells = np.arange(N * N)
+    n_wall = np.array([((walls[:, c >> 5] >> (c & 31)) & 1).sum() for c in cells])
+    n_goal = np.bincount(goal, minlength=N * N)
+    dW1 = grads[sl["W1"]].reshape(3, N * N, H)
+    for name, got, want in (("b1", grads[sl["b1"]], d_h1), ("walls", dW1[0], np.outer(n_wall / B, d_h1)), ("goal", dW1[2], np.outer(n_goal / B, d_h1))):
+        bias = (np.asarray(got, np.float64) - want).sum() / want.sum()
+        print(f"H = {H}, {B} envs: {name} off by {bias:+.2e}")
+        assert abs(bias) <= 2.0**-22 + 3 * H / 16 * 2.0**-24, name
+        par.assert_close(got, want, par.RTOL_FP32, name)
 
 
 @pytest.mark.parametrize("H,prec,B,T", [(32, 0, 40, 7), (64, 0, 33, 9), (96, 1, 70, 5), (128, 0, 65, 11), (128, 1, 200, 4), (256, 0, 127, 6), (256, 0, 300, 9),
