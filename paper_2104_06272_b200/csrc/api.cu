@@ -136,6 +136,7 @@ size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* o
 
 int fail_cuda(anakin_t* h, cudaError_t e) {
     snprintf(h->cuda_err, sizeof(h->cuda_err), "%s: %s", cudaGetErrorName(e), cudaGetErrorString(e));
+    cudaGetLastError();  // (reported here: the next call's launches must not find it again)
     return ANAKIN_E_CUDA;
 }
 
@@ -316,6 +317,7 @@ int anakin_create(const anakin_cfg* cfg, void* dev_workspace, size_t bytes, void
     cudaError_t e = cudaGetDevice(&cur);
     if (e == cudaSuccess && cur != cfg->device) e = cudaSetDevice(cfg->device);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         delete h;
         return ANAKIN_E_CUDA;
     }

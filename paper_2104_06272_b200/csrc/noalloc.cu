@@ -49,6 +49,12 @@ cudaError_t scratch_for_current_device(unsigned char** out) {
     return cudaSuccess;
 }
 
+// A CUDA error is reported by the return code: the next call's launches must not find it again.
+int fail_cuda() {
+    cudaGetLastError();
+    return ANAKIN_E_CUDA;
+}
+
 }  // namespace
 
 extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int64_t global_step, int T,
@@ -72,7 +78,7 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
         return ANAKIN_E_WORKSPACE_TOO_SMALL;
     }
     unsigned char* scratch = nullptr;
-    if (scratch_for_current_device(&scratch) != cudaSuccess) return ANAKIN_E_CUDA;
+    if (scratch_for_current_device(&scratch) != cudaSuccess) return fail_cuda();
     cudaStream_t s = (cudaStream_t)cuda_stream;
 
     RolloutArgs a;
@@ -111,7 +117,7 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
     b.stats = reinterpret_cast<anakin_stats*>(tail);
     b.status = reinterpret_cast<int*>(tail + 128);
     // the tail holds accumulators and a sticky status word left by the previous call: start them at zero
-    if (cudaMemsetAsync(tail, 0, kTailBytes, s) != cudaSuccess) return ANAKIN_E_CUDA;
+    if (cudaMemsetAsync(tail, 0, kTailBytes, s) != cudaSuccess) return fail_cuda();
     a.T = T;
     a.cap = cfg->episode_cap;
     a.gstep0 = (uint32_t)global_step;
@@ -123,15 +129,15 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
     a.fuse_gae = 0;  // the caller gets the trajectory only
     uint64_t launches = 0;
     const Ctx ctx{s, &launches, nullptr};
-    if (launch_env_base(a.d, b, ctx) != cudaSuccess) return ANAKIN_E_CUDA;  // fills `base`: nothing of the last call survives
+    if (launch_env_base(a.d, b, ctx) != cudaSuccess) return fail_cuda();  // fills `base`: nothing of the last call survives
     if (wide_supported(cfg->H)) {
-        if (noalloc_wide_scratch(&b) != cudaSuccess) return ANAKIN_E_CUDA;
+        if (noalloc_wide_scratch(&b) != cudaSuccess) return fail_cuda();
         a.d.Tmax = 0;  // the activations of one step
-        if (launch_pack_w2_wide(a.d, b, ctx) != cudaSuccess) return ANAKIN_E_CUDA;
+        if (launch_pack_w2_wide(a.d, b, ctx) != cudaSuccess) return fail_cuda();
     } else if (launch_pack_w2(a.d, b, cfg->precision, ctx) != cudaSuccess) {  // likewise the weight fragments
-        return ANAKIN_E_CUDA;
+        return fail_cuda();
     }
-    if (launch_rollout(a, cfg->precision, ctx) != cudaSuccess) return ANAKIN_E_CUDA;
+    if (launch_rollout(a, cfg->precision, ctx) != cudaSuccess) return fail_cuda();
     return ANAKIN_OK;
 }
 
@@ -140,13 +146,13 @@ extern "C" int anakin_rollout_noalloc(const anakin_cfg* cfg, uint64_t seed, int6
 extern "C" int anakin_noalloc_status(void* cuda_stream, int* device_status) {
     if (!device_status) return ANAKIN_E_INVALID_ARG;
     unsigned char* scratch = nullptr;
-    if (scratch_for_current_device(&scratch) != cudaSuccess) return ANAKIN_E_CUDA;
+    if (scratch_for_current_device(&scratch) != cudaSuccess) return fail_cuda();
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const unsigned char* tail = scratch + kMaxBaseFloats * sizeof(float) + kW2FragBytes + kW2PlaneBytes;
     int st = 0;
     cudaError_t e = cudaMemcpyAsync(&st, tail + 128, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return ANAKIN_E_CUDA;
+    if (e != cudaSuccess) return fail_cuda();
     *device_status = st;
     return st == 0 ? ANAKIN_OK : ANAKIN_E_DEVICE_STATUS;
 }

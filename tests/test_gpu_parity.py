@@ -3,6 +3,7 @@
 Stages are teacher-forced: one flipped action would send a free-running comparison down a different
 trajectory, so each stage of the library is fed to the oracle and compared there.
 """
+import ctypes as C
 import os
 import subprocess
 import sys
@@ -591,6 +592,52 @@ def test_blobs_copied_within_the_gpu_at_any_alignment(bnd, shift):
         before = an.launch_count()
         assert bnd.lib().anakin_get(an._h, bnd.ENV_POS, pin.data_ptr(), pin.numel(), 1) == bnd.OK
         assert an.launch_count() == before and an.status() == 0 and (pin.numpy() == an.get(bnd.ENV_POS)).all()
+
+
+@pytest.fixture()
+def side_by_side():
+    """Three allocations of 256 KiB side by side in one 2 MiB page, so that no byte near them is unmapped: (address of the first, a
+    function that frees one of them)."""
+    cu, size = C.CDLL("libcuda.so.1"), 256 << 10
+    torch.zeros(1, device="cuda")  # (the context)
+    ptrs = []
+    for _ in range(24):
+        p = C.c_uint64()
+        assert cu.cuMemAlloc_v2(C.byref(p), C.c_size_t(size)) == 0
+        ptrs.append(p.value)
+
+    def free(p):
+        ptrs.remove(p)
+        assert cu.cuMemFree_v2(C.c_uint64(p)) == 0
+
+    at = next((p for p in ptrs if p % (2 << 20) <= 5 * size and p + size in ptrs and p + 2 * size in ptrs), None)
+    if at is not None:
+        yield at, size, free
+    torch.cuda.synchronize()
+    for p in list(ptrs):
+        free(p)
+    if at is None:
+        pytest.skip("no three allocations side by side")
+
+
+def copy_pos(bnd, an, what, p):
+    return getattr(bnd.lib(), "anakin_" + what)(an._h, bnd.ENV_POS, C.c_void_p(p), an.blob_bytes(bnd.ENV_POS), 1)
+
+
+def test_a_refused_copy_leaves_no_error_behind(bnd, side_by_side):
+    """A caller's buffer that is too short for its blob: an error code, and the next calls, which launch kernels, succeed."""
+    at, size, free = side_by_side
+    free(at + size)
+    free(at + 2 * size)
+    an = bnd.Anakin(bnd.make_cfg(2 * size + 77, 2, 32, 1))
+    an.reset(3)
+    want = an.get(bnd.ENV_POS)
+    for what in ("get", "set"):
+        assert copy_pos(bnd, an, what, at) == bnd.E_CUDA
+        assert (an.get(bnd.ENV_POS) == want).all()
+        an.set(bnd.ENV_POS, torch.from_numpy(want).cuda())
+    an.run(1)
+    assert an.status() == 0
 
 
 def test_handles_in_their_own_threads_and_streams_give_what_they_give_alone():
