@@ -7,6 +7,8 @@
 #include <cstring>
 #include <new>
 
+#include <cuda.h>  // pointer attributes (types only; the entry is fetched through the runtime)
+
 #include "common.cuh"
 
 using namespace anakin;
@@ -526,19 +528,46 @@ size_t anakin_blob_bytes(anakin_t* h, int which) {
     return blob_total(h, which);
 }
 
-// Whether a kernel launched now may address [p, p + bytes): the current device is the handle's, and both ends are plain memory of
-// that GPU.  Anything else (another GPU's memory, which needs peer access; managed or host memory; a range that runs out of its
-// allocation) is left to the runtime's copies, which take or refuse it themselves.
+// Looked up once, by whichever thread is first (the others wait for it); null where the driver has no such entry.
+static decltype(&cuPointerGetAttributes) pointer_attributes_fn() {
+    static const auto fn = []() -> decltype(&cuPointerGetAttributes) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();  // (not this call's error)
+            return nullptr;
+        }
+        return reinterpret_cast<decltype(&cuPointerGetAttributes)>(p);
+    }();
+    return fn;
+}
+
+// Whether a kernel launched now may address [p, p + bytes): the current device is the handle's, and the whole range is plain memory of
+// that GPU inside one allocation.  Anything else (another GPU's memory, which needs peer access; managed or host memory; a range that
+// runs out of its allocation, even into another one) is left to the runtime's copies, which take or refuse it themselves: what they
+// refuse with an error code would be a fault in a kernel.  The address range of a virtual-memory reservation may hold several mappings
+// and holes between them, so the mappings are walked; of every other allocation the first one holds it all, and this is one call.
 static bool kernel_can_copy(const anakin_t* h, const void* p, size_t bytes) {
     int cur = -1;
     if (cudaGetDevice(&cur) != cudaSuccess || cur != h->cfg.device) return false;
-    for (const size_t at : {(size_t)0, bytes - 1}) {
-        cudaPointerAttributes pa;
-        if (cudaPointerGetAttributes(&pa, static_cast<const char*>(p) + at) != cudaSuccess) {
-            cudaGetLastError();  // (not this call's error)
-            return false;
-        }
-        if (pa.type != cudaMemoryTypeDevice || pa.device != h->cfg.device) return false;
+    const auto query = pointer_attributes_fn();
+    if (!query) return false;
+    const CUdeviceptr beg = (CUdeviceptr)(uintptr_t)p, end = beg + bytes;
+    if (end <= beg) return false;
+    for (CUdeviceptr at = beg; at < end;) {
+        unsigned type = 0, managed = 0, access = 0;
+        int dev = -1, mapped = 0;
+        CUdeviceptr range = 0, map = 0;
+        size_t range_size = 0, map_size = 0;
+        CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS,
+                                      CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_MAPPED, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                      CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_MAPPING_BASE_ADDR, CU_POINTER_ATTRIBUTE_MAPPING_SIZE};
+        void* data[] = {&type, &managed, &access, &dev, &mapped, &range, &range_size, &map, &map_size};
+        if (query(sizeof(what) / sizeof(what[0]), what, data, at) != CUDA_SUCCESS) return false;
+        if (type != CU_MEMORYTYPE_DEVICE || managed || access != CU_POINTER_ATTRIBUTE_ACCESS_FLAG_READWRITE || dev != h->cfg.device || !mapped) return false;
+        if (beg < range || end > range + range_size) return false;
+        if (at < map || at >= map + map_size) return false;
+        at = map + map_size;
     }
     return true;
 }

@@ -640,6 +640,24 @@ def test_a_refused_copy_leaves_no_error_behind(bnd, side_by_side):
     assert an.status() == 0
 
 
+def test_a_blob_that_runs_out_of_its_allocation_is_not_copied_by_a_kernel(bnd, side_by_side):
+    """A caller's buffer that ends in another allocation, with or without a hole between: the runtime's copy refuses it with an error code (a
+    kernel would write over the neighbour, or fault in the hole); one that fills its allocation to the last byte goes by the kernel."""
+    at, size, free = side_by_side
+    an, full = (bnd.Anakin(bnd.make_cfg(B, 2, 32, 1)) for B in (2 * size + 77, size))
+    an.reset(3)
+    full.reset(3)
+    want = an.get(bnd.ENV_POS)
+    for hole in (False, True):
+        if hole:
+            free(at + size)
+        before = an.launch_count()
+        assert copy_pos(bnd, an, "get", at) == bnd.E_CUDA and copy_pos(bnd, an, "set", at) == bnd.E_CUDA and an.launch_count() == before
+        assert (an.get(bnd.ENV_POS) == want).all()
+        before = full.launch_count()
+        assert copy_pos(bnd, full, "get", at) == bnd.OK and copy_pos(bnd, full, "set", at) == bnd.OK and full.launch_count() == before + 2
+
+
 def test_handles_in_their_own_threads_and_streams_give_what_they_give_alone():
     """Different handles are independent: the first calls of a process from eight threads at once (what the library sets up once per
     process or device among them), each on a handle and a stream of its own, against the same work done one after the other."""
