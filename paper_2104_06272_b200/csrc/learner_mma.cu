@@ -1418,6 +1418,18 @@ static int splits_for(int K, int tiles, int min_k) {
     return ns < 1 ? 1 : ns;
 }
 
+// Many policies: the splits of the warp-level kernel.  The tensor core rounds toward zero, so one split, which is one accumulator, has at most
+// 4096 rows (768 MMAs).  With 128 splits at most, 49152 rows of the same sign each (two policies of 65536 envs, H = 128, T = 96, 2 x 2 boards)
+// came out 2.4e-4 low in dW2, 3.6 times the bound.  More splits than splits_for gives come in whole waves of two CTAs an SM.  B200: two
+// policies of 100,000 envs, 10 x 10, T = 8 dW2 453 -> 394, agent plane 377 -> 336, reduction 93 -> 183 us; of 65536 envs, 2 x 2, T = 96 3439 ->
+// 2886, 2911 -> 2485, 93 -> 941.  (Restarts inside the kernel: dW2 of the first 487 us, and the agent plane of every shape 5 to 8 % slower.)
+static int grouped_splits(const Dims& d, size_t rows, int tiles, int min_k) {
+    const int ns = splits_for((int)rows, tiles, min_k), least = (int)((rows + 4095) / 4096);
+    if (ns >= least) return ns;
+    const long long one = (long long)d.npol * tiles, waves = (least * one + 295) / 296;
+    return (int)(waves * 296 / one);
+}
+
 // Launch shape of the fused dh1 + agent-plane kernel: nx CTAs (H = 256: pairs), one per SM, walk the units (128-env tile, slice of
 // the steps); one agent-plane partial each.  (Four slices at most and one unit per CTA: 2500 envs, H = 128, T = 24 21.3 -> 18.8 us,
 // 6000 envs, H = 256, T = 20 58 -> 44 us.)
@@ -1434,7 +1446,7 @@ static void dh1a_shape(const Dims& d, int T, int* nx, int* ts) {
 static int env_splits(const Dims& d, int rows, bool many) {
     if (many) {  // (many policies: the warp-level kernel's tiles)
         const int bt = d.H == 128 ? 128 : 64;
-        return splits_for(rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
+        return grouped_splits(d, rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
     }
     const int tiles = ((d.C + 128) / 128 + (d.C + 127) / 128) * ((d.H + 255) / 256), slots = d.H > 128 ? 148 : 296;
     const int most = rows / 128 > 0 ? rows / 128 : 1, least = (rows + 8191) / 8192;  // (one split has at most 8192 rows, whatever the batch)
@@ -1463,8 +1475,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         tiles_hh = (H / 128) * ((H + 255) / 256);
         tiles_agent = ((C + 127) / 128) * ((H + 255) / 256);
     }
-    p->ns_w2 = splits_for((int)R, tiles_hh, 256);
-    p->ns_agent = splits_for((int)R, tiles_agent, 256);
+    p->ns_w2 = d.npol > 1 ? grouped_splits(d, R, tiles_hh, 256) : splits_for((int)R, tiles_hh, 256);
+    p->ns_agent = d.npol > 1 ? grouped_splits(d, R, tiles_agent, 256) : splits_for((int)R, tiles_agent, 256);
     if (H > 256) {  // the bf16 GEMM CTAs of the wide path take a whole SM each (four 48 KB stages): one wave
         p->ns_w2 = 148 / tiles_hh > 0 ? 148 / tiles_hh : 1;
     }
@@ -1476,8 +1488,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
     }
-    p->ns_env = d.npol > 1 ? splits_for(d.B, tiles_ch, 128) : env_splits(d, d.B, false);
-    int env_room = std::max(splits_for(d.B, tiles_ch, 128), env_splits(d, d.B, false));  // (the same for one policy and for many)
+    p->ns_env = d.npol > 1 ? grouped_splits(d, d.B, tiles_ch, 128) : env_splits(d, d.B, false);
+    int env_room = std::max(grouped_splits(d, d.B, tiles_ch, 128), env_splits(d, d.B, false));  // (the same for one policy and for many)
     if (dh1_agent_tc_supported(d) && d.npol <= 1) {  // (one agent-plane partial per CTA of the fused kernel, any T <= Tmax)
         const int cap = 148 / (H / DH1A_UNITS);
         p->ns_agent = std::max(p->ns_agent, std::min(cap, (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax)));

@@ -291,14 +291,18 @@ def test_policies_blobs_outside_the_handles_gpu_go_by_the_runtimes_copies(bnd, n
         an.set(bnd.ENV_POS, want)
 
 
-def test_policies_gradients_of_long_sums(bnd):
+@pytest.mark.parametrize("H,per,N,T,bias", [(64, 9472, 3, 97, 0.0), (128, 65536, 2, 48, 3.0)])
+def test_policies_gradients_of_long_sums(bnd, H, per, N, T, bias):
     """Two policies share the 148 CTAs of the fused backward kernel at H = 64: 74 tiles of 128 envs times 97 steps are at least 97 tiles
     for the busiest of a policy's 74 CTAs, so both accumulators are emptied and restarted on the way (dW2 every 32, the agent plane
-    every 96 tiles).  The last policy is a few envs short."""
-    w = Workload("k2_h64_long", B=2 * 9472 - 50, N=3, H=64, T=97, iters=1, n_policies=2)
+    every 96 tiles).  At H = 128 the 128 splits of dW2 have 24576 rows each, six groups of 4096, of the same sign (a value head that is
+    off by 3 on boards of four cells): what the tensor core's rounding loses in one accumulator adds up.  The last policy is a few envs
+    short."""
+    w = Workload(f"k2_h{H}_long", B=2 * per - 50, N=N, H=H, T=T, iters=1, n_policies=2)
     an = make(bnd, w)
     an.reset(21)
     thetas = policy_thetas(w, an.K, seed=31)
+    thetas[:, -1] += bias
     an.set(bnd.PARAMS, thetas)
     an.rollout()
     an.gae()
