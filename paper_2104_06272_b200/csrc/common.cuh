@@ -313,9 +313,9 @@ struct GemmTnArgs {
     int M2;
     float* part2;
     size_t stride2;
-    // many policies (npol > 1): grid.z = policy * nsplit + split; every pointer above moves by pstride bytes per policy;
+    // many policies (npol > 1): z0 + blockIdx.z = policy * nsplit + split; every pointer above moves by pstride bytes per policy;
     // the last policy has K_last rows (period kmod_last)
-    int npol, nsplit, K_last, kmod_last;
+    int npol, nsplit, z0, K_last, kmod_last;
     size_t pstride;
     size_t alo_off_last, blo_off_last;  // Alo - Ahi and Blo - Bhi (elements) in the last policy's more compact planes
 };

@@ -917,8 +917,8 @@ struct GemmTnCfg {
 template <int BM, int BN, int AMODE>
 __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
     pdl_wait();  // (the trigger comes after the products: CTAs of the next kernel beside these from the start cost more than the gap)
-    // many policies: grid.z = policy * nsplit + split
-    const PolicyArgs<true, GemmTnArgs> pa(g_in, (int)blockIdx.z / g_in.nsplit);
+    const int pol_split = g_in.z0 + (int)blockIdx.z;  // policy * nsplit + split
+    const PolicyArgs<true, GemmTnArgs> pa(g_in, pol_split / g_in.nsplit);
     const GemmTnArgs& g = pa.a;
     using Cfg = GemmTnCfg<BM, BN, AMODE>;
     constexpr int APL = Cfg::APL, BPL = Cfg::BPL, PREC = 0;
@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
     __nv_bfloat16* sB = sA + STAGES * Cfg::A_STAGE;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int wm = wid >> 2, wn = wid & 3;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN, split = (int)blockIdx.z % g.nsplit;
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN, split = pol_split % g.nsplit;
     const int kbeg = split * g.klen, kend = min(g.K, kbeg + g.klen);
     const int ntiles = kend > kbeg ? (kend - kbeg + BK - 1) / BK : 0;
 
@@ -1063,10 +1063,17 @@ __global__ void __launch_bounds__(256) k_gemm_tn(GemmTnArgs g_in) {
 template <int BM, int BN, int AMODE>
 static cudaError_t launch_gemm_tn(const GemmTnArgs& g, int rows_m, int splits, cudaStream_t s) {
     using Cfg = GemmTnCfg<BM, BN, AMODE>;
-    if ((size_t)g.npol * splits > 65535) return cudaErrorNotSupported;
+    const long long all = (long long)g.npol * splits, most = 65535;  // (the third dimension of a grid)
+    if (all > 0x7FFFFFFF) return cudaErrorNotSupported;
     GemmTnArgs gg = g;
     gg.nsplit = splits;
-    return launch<k_gemm_tn<BM, BN, AMODE>>(dim3((rows_m + BM - 1) / BM, (g.N + BN - 1) / BN, g.npol * splits), 256, Cfg::smem_bytes, s, gg);
+    cudaError_t e = cudaSuccess;
+    for (long long z0 = 0; z0 < all && e == cudaSuccess; z0 += most) {
+        gg.z0 = (int)z0;
+        const dim3 grid((rows_m + BM - 1) / BM, (g.N + BN - 1) / BN, (unsigned)std::min(all - z0, most));
+        e = launch<k_gemm_tn<BM, BN, AMODE>>(grid, 256, Cfg::smem_bytes, s, gg);
+    }
+    return e;
 }
 
 // One Adam step of parameter i with gradient g (Kingma & Ba, Algorithm 1), plus the refreshed 16-bit copies.

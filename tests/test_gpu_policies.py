@@ -319,6 +319,31 @@ def test_policies_gradients_of_long_sums(bnd, H, per, N, T, bias):
     assert an.status() == 0
 
 
+def test_policies_times_splits_beyond_a_grid_dimension(bnd):
+    """1025 policies of 16384 rows at H = 128: 64 splits each of dW2 and the agent plane, 65600 in all, more than the second and third
+    dimension of a grid hold.  The first and the last policy's gradients against the oracle."""
+    w = Workload("k1025_h128", B=1025 * 1024 - 40, N=3, H=128, T=16, iters=1, n_policies=1025)
+    an = make(bnd, w)
+    an.reset(21)
+    theta = np.tile(random_params(31, w.P, 0.15), (an.K, 1))
+    an.set(bnd.PARAMS, theta)
+    an.rollout()
+    an.learn()
+    assert an.status() == 0
+    walls, goal, gates = an.get(bnd.ENV_WALLS).reshape(w.B, -1), an.get(bnd.ENV_GOAL), an.get(bnd.DEBUG_GATES)
+    traj = [an.get(which) for which in (bnd.TRAJ_POS, bnd.TRAJ_ACTION, bnd.ADV, bnd.RET)]
+    grads = an.get(bnd.GRADS).reshape(an.K, an.P)
+    for p in (0, an.K - 1):
+        e0, n = an.policy_envs(p)
+        words = n * w.T * (w.H // 32)
+        own = gates[2 * e0 * w.T * (w.H // 32):][:2 * words].reshape(2, n * w.T, w.H // 32)
+        blocks = [np.ascontiguousarray(an.policy_block(x, p, w.T)) for x in traj]
+        ograds, _, _ = orc.learn(w.N, w.H, 0, theta[p], np.ascontiguousarray(walls[e0:e0 + n]), goal[e0:e0 + n].copy(), *blocks,
+                                 np.float32(w.value_coef), np.float32(w.entropy_coef), gates=(own[0], own[1]))
+        for nm, sl in orc.Dims(w.N, w.H).slices().items():
+            par.assert_close(grads[p][sl], ograds[sl], par.RTOL_FP32, f"policy {p} grad {nm}")
+
+
 @pytest.mark.parametrize("K,H,N", [(40, 64, 5), (64, 128, 16), (300, 64, 16), (1024, 64, 9)])
 def test_policies_every_parameter_is_reduced_and_stepped_once(bnd, K, H, N):
     """One, two, three and four pieces of a policy's parameters per CTA of the reduction: gradient, moments and parameters of every policy."""
