@@ -334,6 +334,7 @@ __device__ __forceinline__ void select_policy(GemmTnArgs& g, int pol) {
 #endif
 
 // tcgen05 version (tensor memory accumulators, TMA-fed); cudaErrorNotSupported when the shape is not covered.
+int gemm_tn_tc_env_per_sm(int H, bool three);
 cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int prec, int splits, int* status, cudaStream_t s);
 
 // ---- launches ----

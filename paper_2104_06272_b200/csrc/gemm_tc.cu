@@ -423,6 +423,15 @@ static cudaError_t launch_p(const GemmTnArgs& g, int amode, int splits, int* sta
     return launch_bn<64, PREC>(g, amode, splits, status, s);
 }
 
+// CTAs of the wall and goal planes' launch that an SM holds at once (its 228 KB of shared memory decide, 1 KB of them a CTA's own).
+int gemm_tn_tc_env_per_sm(int H, bool three) {
+    constexpr size_t sm = 228 * 1024;
+    auto fit = [](size_t smem) { return (int)(sm / (smem + 1024)); };
+    if (H > 128) return three ? fit(GemmTcCfg<256, 1, 3, false, 2>::smem_bytes) : fit(GemmTcCfg<256, 1, 2, false, 0>::smem_bytes);
+    if (H > 64) return three ? fit(GemmTcCfg<128, 1, 3, false, 2>::smem_bytes) : fit(GemmTcCfg<128, 1, 2, false, 0>::smem_bytes);
+    return three ? fit(GemmTcCfg<64, 1, 3, false, 2>::smem_bytes) : fit(GemmTcCfg<64, 1, 2, false, 0>::smem_bytes);
+}
+
 // Covered: N = ldb a multiple of 32 (column tiles of 64, 128 or 256; columns past N read as zeros and are not stored), klen a
 // multiple of 64, the planes of the workload's precision.
 cudaError_t launch_gemm_tn_tc(const GemmTnArgs& g, int amode, int prec, int splits, int* status, cudaStream_t s) {

@@ -1447,15 +1447,19 @@ static void dh1a_shape(const Dims& d, int T, int* nx, int* ts) {
 }
 
 // Splits of the wall and goal planes' K range (rows of S), at least two 64-row chunks each: one wave of the launch's tiles (128 cells of
-// either plane x 256 columns), of CTAs that take an SM each above 128 columns and share one below.  B200 (events included), this rule / as
-// many as two waves of the wall tiles alone: 65536 envs, 10 x 10, H = 256 29 / 39 us and 21 / 24 in the reduction, 6000 envs, 12 x 12,
-// H = 256 21 / 29 and 21 / 26, 2500 envs, 9 x 9, H = 128 12.2 / 15.4 and 12 / 13; one chunk at least instead of two gains nothing more.
-static int env_splits(const Dims& d, int rows, bool many) {
+// either plane x 256 columns), of as many CTAs as an SM holds; a third one (up to 64 columns) only where a split then still has 512 rows.
+// B200 (events included), one wave / as many as two waves of the wall tiles alone: 65536 envs, 10 x 10, H = 256 29 / 39 us and 21 / 24 in
+// the reduction, 6000 envs, 12 x 12, H = 256 21 / 29 and 21 / 26, 2500 envs, 9 x 9, H = 128 12.2 / 15.4 and 12 / 13; one chunk at least
+// instead of two gains nothing more.  H = 96 in fp32, where one CTA fits, one wave / two (whole iterations): 12000 envs, 16 x 16, T = 2 127 /
+// 132 us, 20000, 10 x 10 131 / 135.  H = 64, three / two CTAs an SM: 65536 envs, 12 x 12, T = 2 167 / 175, 16 x 16 202 / 210, but 6000 envs,
+// 16 x 16, T = 16 (24000 rows) 125 / 122.
+static int env_splits(const Dims& d, int rows, bool many, bool three) {
     if (many) {  // (many policies: the warp-level kernel's tiles)
         const int bt = d.H == 128 ? 128 : 64;
         return grouped_splits(d, rows, ((d.C + 1 + bt - 1) / bt) * ((d.H + bt - 1) / bt), 256);
     }
-    const int tiles = ((d.C + 128) / 128 + (d.C + 127) / 128) * ((d.H + 255) / 256), slots = d.H > 128 ? 148 : 296;
+    const int tiles = ((d.C + 128) / 128 + (d.C + 127) / 128) * ((d.H + 255) / 256), fit = gemm_tn_tc_env_per_sm(d.H, three);
+    const int slots = 148 * (rows / 512 >= 148 * fit / tiles ? fit : std::min(fit, 2));
     const int most = rows / 128 > 0 ? rows / 128 : 1, least = (rows + 8191) / 8192;  // (one split has at most 8192 rows, whatever the batch)
     return std::max(std::min(std::min(slots / tiles, 128), most), least);
 }
@@ -1495,12 +1499,12 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
         const int ap = agent_plane_splits(d);
         if (ap > p->ns_agent) p->ns_agent = ap;
     }
-    p->ns_env = d.npol > 1 ? grouped_splits(d, d.B, tiles_ch, 128) : env_splits(d, d.B, false);
-    int env_room = std::max(grouped_splits(d, d.B, tiles_ch, 128), env_splits(d, d.B, false));  // (the same for one policy and for many)
+    p->ns_env = d.npol > 1 ? grouped_splits(d, d.B, tiles_ch, 128) : env_splits(d, d.B, false, false);
+    int env_room = std::max(grouped_splits(d, d.B, tiles_ch, 128), env_splits(d, d.B, false, false));  // (the same for one policy and for many)
     if (dh1_agent_tc_supported(d) && d.npol <= 1) {  // (one agent-plane partial per CTA of the fused kernel, any T <= Tmax)
         const int cap = 148 / (H / DH1A_UNITS);
         p->ns_agent = std::max(p->ns_agent, std::min(cap, (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax)));
-        p->ns_env = env_splits(d, most_s_rows(d.B), false);
+        p->ns_env = env_splits(d, most_s_rows(d.B), false, false);
         env_room = std::max(env_room, p->ns_env);
     }
     if (back128_supported(d)) {  // (one partial of everything per CTA)
@@ -1509,8 +1513,8 @@ void learn_mma_plan(const Dims& d, LearnPlan* p) {
     if (H == 64) {  // (one partial per CTA of the fused kernel; its slices of the steps are rows of S)
         const int units = d.B > 64 ? (d.B + 127) / 128 * std::min(MAX_SLICES, d.Tmax) : (d.Tmax + 128 / d.B - 1) / (128 / d.B);  // (of any T <= Tmax)
         p->ns_w2 = p->ns_agent = std::min(std::max(148 / d.npol, 1), units);
-        p->ns_env = env_splits(d, most_s_rows(d.B), d.npol > 1);
-        env_room = std::max({env_room, env_splits(d, most_s_rows(d.B), false), env_splits(d, most_s_rows(d.B), true)});
+        p->ns_env = env_splits(d, most_s_rows(d.B), d.npol > 1, false);
+        env_room = std::max({env_room, env_splits(d, most_s_rows(d.B), false, false), env_splits(d, most_s_rows(d.B), true, false)});
     }
     const size_t tiles32 = (R + 31) / 32;
     size_t hg = (size_t)heads_grid_max(H);
@@ -1587,7 +1591,10 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
     const bool grouped = d.npol > 1;
     LearnPlan pl;
     learn_mma_plan(d, &pl);
-    if (PREC == 2) pl.ns_w2 = x3_w2_splits(H, R);
+    if (PREC == 2) {
+        pl.ns_w2 = x3_w2_splits(H, R);
+        pl.ns_env = env_splits(d, B, false, true);
+    }
     a.part_small = b.part + pl.off_small;
     a.small_stride = pl.small_stride;
     // parameter regions in flat order: W1 walls | W1 agent | W1 goal | b1 | W2 | b2 | Wh | bh
@@ -1649,7 +1656,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         int nx;
         back64_shape(d, T, &nx, &a.ts);
         a.reg[1].ns = a.reg[4].ns = nx;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped, false);
         Scope sc(c, K_DH1);
         CK(launch_back64(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
@@ -1658,7 +1665,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         back128_shape(d, T, &nx, &a.ts);
         for (int q = 4; q < 8; ++q) a.reg[q].ns = nx;
         a.reg[1].ns = pl.loss_blocks = nx;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped, false);
         Scope sc(c, K_HEADS_BWD);  // (profiled under the name of what it starts with)
         CK(launch_back128(a, PREC, nx, b.part + pl.off_w2, b.part + pl.off_agent, CH, s));
         fused_agent = true;
@@ -1666,7 +1673,7 @@ static cudaError_t launch_learn_mma_p(LearnArgs a, const Ctx& c) {
         int nx;
         dh1a_shape(d, T, &nx, &a.ts);
         a.reg[1].ns = nx;
-        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped);
+        a.reg[0].ns = a.reg[2].ns = a.reg[3].ns = pl.ns_env = env_splits(d, a.ts * B, grouped, false);
         Scope sc(c, K_DH1);
         CK(launch_dh1_agent_tc(a, PREC, nx, b.part + pl.off_agent, CH, s));
         fused_agent = true;
