@@ -156,13 +156,15 @@ def test_reverse_scans_across_chunk_edges(bnd, B, T):
     an.rollout()
     g = par.gpu_traj(an, bnd, T)
     fused = [an.get(which).view(np.uint32) for which in (bnd.ADV, bnd.RET)]
-    an.set(bnd.ADV, np.full(B * T, 7.0, np.float32))
+    poison = lambda: [an.set(which, np.full(B * T, 7.0, np.float32)) for which in (bnd.ADV, bnd.RET)]  # noqa: E731
+    poison()
     gadv, gret = par.check_gae(an, bnd, w, g, T)
     assert (gadv.reshape(-1).view(np.uint32) == fused[0]).all() and (gret.reshape(-1).view(np.uint32) == fused[1]).all()
     rng = np.random.default_rng(11)
     theta = an.get(bnd.PARAMS)
     an.set(bnd.PARAMS, (theta + 0.03 * rng.standard_normal(theta.size)).astype(np.float32))
     st = par.gpu_state(an, bnd)
+    poison()
     an.learn_vtrace(1, 1.1, 0.9)
     sel = np.arange(B) if B <= 200 else np.r_[:100, B - 100:B]
     g = {k: np.ascontiguousarray(v[:, sel]) for k, v in g.items()}

@@ -58,17 +58,17 @@ def test_width_one_iteration_stage_by_stage(bnd, H, prec, B, N, T):
         print(w.name, "worst error / bound:", {k: round(v, 3) for k, v in par.MARGINS.items()})
 
 
-@pytest.mark.parametrize("prec", [0, 1])
-def test_width_128_gradients_do_not_depend_on_timing(bnd, prec):
-    """Two handles in lockstep over 60 passes of two to three tiles of 64 envs a CTA: the same bits.  (The warps of the fused backward
-    kernel hand tiles on through mbarriers; one that read the agent plane's accumulator ahead of its last MMAs showed here in one
-    pass of fifteen in bf16.)"""
+@pytest.mark.parametrize("prec,B,T,passes", [(0, 148 * 128 + 77, 5, 60), (1, 148 * 128 + 77, 5, 60), (0, 148 * 64, 97, 20), (1, 148 * 64, 97, 20)])
+def test_width_128_gradients_do_not_depend_on_timing(bnd, prec, B, T, passes):
+    """Two handles in lockstep over many passes: the same bits.  Two to three units of 64 envs a CTA, some fifteen tiles; one unit of 97 tiles a
+    CTA, where in fp32 both accumulators are emptied and restarted on the way.  (The warps of the fused backward kernel hand tiles on
+    through mbarriers; one that read the agent plane's accumulator ahead of its last MMAs showed here in one pass of fifteen in bf16.)"""
     pair = []
     for _ in range(2):
-        an = bnd.Anakin(bnd.make_cfg(148 * 128 + 77, 8, 128, 5, precision=prec, episode_cap=4))
+        an = bnd.Anakin(bnd.make_cfg(B, 8, 128, T, precision=prec, episode_cap=4))
         an.reset(6)
         pair.append(an)
-    for i in range(60):
+    for i in range(passes):
         grads = []
         for an in pair:
             an.run(1)
@@ -78,13 +78,16 @@ def test_width_128_gradients_do_not_depend_on_timing(bnd, prec):
 
 LONG_SUMS = [
     # (H, precision, B, N, T, bias of the value head).  Many rows a CTA: the accumulators of the backward kernels are emptied and
-    # restarted on the way (the agent plane every 48 tiles of 128 rows at H = 128 and 256, 96 tiles at 64; dW2 at 64 every 32).  However the tiles are dealt out, one of
-    # the 148 CTAs (74 pairs at H = 256) has at least the mean of them.
+    # restarted on the way: the agent plane every 48 tiles of 128 rows at H = 256 and, on boards of more than 128 cells, 128, every 96 tiles
+    # at 64; dW2 at 64 every 32; at H = 128 on smaller boards, in tiles of 64 rows, the agent plane every 96 and dW2 every 64.  However the
+    # tiles are dealt out, one of the 148 CTAs (74 pairs at H = 256) has at least the mean of them.
     # The tensor core rounds toward zero, so a sum that is left in one accumulator is biased, most where nearly every MMA adds to
     # it: four cells, and a value head that is off by 3 (every row pulls the same way).
     (128, 0, 131072, 2, 96, 3.0), (64, 0, 131072, 2, 160, 3.0),
     (128, 0, 18945, 13, 49, 0.0), (256, 0, 30000, 3, 20, 3.0), (256, 0, 7000, 12, 70, 0.0),
     (64, 0, 18945, 3, 98, 0.0), (64, 0, 18945, 12, 98, 0.0), (64, 1, 18945, 5, 34, 0.0), (64, 1, 18945, 12, 34, 0.0),
+    # one unit of T tiles a CTA: exactly one group of either accumulator, and one tile more
+    (128, 0, 148 * 64, 3, 64, 0.0), (128, 0, 148 * 64, 3, 65, 0.0), (128, 0, 148 * 64, 3, 96, 0.0), (128, 0, 148 * 64, 3, 97, 0.0),
 ]
 
 
