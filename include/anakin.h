@@ -143,7 +143,8 @@ typedef struct anakin_stats {
 /*
  * Size of the device workspace a configuration needs.  Validates cfg.  For large batches nearly all of it is the activations and
  * their gradients, per recorded row (B * T_max of them) and hidden unit: 12 bytes for H = 64, 128, 256, and below 384 in bf16; 16
- * bytes in fp32 at the other widths (three 16-bit terms an operand); 6 bytes in bf16 from 384 on.
+ * bytes in fp32 at the other widths (three 16-bit terms an operand); 6 bytes in bf16 from 384 on.  The bytes a row and unit do not
+ * depend on the board: at H = 128 with one policy a third of them is unused on boards of up to 128 cells.
  */
 int anakin_workspace_bytes(const anakin_cfg* cfg, size_t* bytes);
 

@@ -120,8 +120,8 @@ size_t carve(const anakin_cfg& c, const Dims& d, unsigned char* base, Buffers* o
     b.h2 = (float*)take(wide ? std::max(h2_bytes, wide_scratch_bytes(d)) : h2_bytes);
     b.out5 = (float*)take(R * 8 * 4);
     b.vboot = (float*)take(B * 4);
-    // (at H = 128 on boards of up to 128 cells nothing goes there any more, dh2 stays on chip; the workspace keeps its size, the same on every
-    // board)
+    // (at H = 128 on boards of up to 128 cells nothing goes there, dh2 stays on chip; the bytes a row and unit are part of the interface and the
+    // same on every board)
     b.dh2 = (float*)take(R * H * (x3 ? 6 : wide ? 2 : 4));
     b.dh1 = dh1_on_chip ? nullptr : b.h2;
     // t-slices of two 16-bit planes, or three planes
@@ -572,9 +572,10 @@ static bool kernel_can_copy(const anakin_t* h, const void* p, size_t bytes) {
     return true;
 }
 
-// Largest blob of one policy that a kernel copies within the GPU.  As a memcpy each costs about 3 us on the stream whatever its size and
+// Largest blob of one policy that a kernel copies within the GPU.  As a memcpy each costs 3.5 us on the stream whatever its size and
 // is no programmatic dependent.  B200, six blobs after each pass: 64 envs at H = 64, two iterations 105.6 -> 96.3 us, 4096 at H = 256
 // 316.5 -> 307.0; back to back, host included, 37 KB 8.2 -> 6.4 us each, 7.4 MB 8.8 -> 4.9.
+// At addresses that only bytes fit, a byte a thread: 64 KB 3.9 -> 3.5 us each, 4 MB 8.2 -> 3.8, 16 MB 13.3 -> 11.1 out, 10.3 -> 9.9 in.
 constexpr size_t COPY_KERNEL_MAX = 16u << 20;
 
 static int copy_blob(anakin_t* h, int which, void* ptr, size_t bytes, int ptr_is_device, bool to_lib) {

@@ -19,8 +19,9 @@
 // groups are added with round-to-nearest.
 // Every wait is bounded; a timeout raises DEV_E_WAIT_TIMEOUT and the CTA unwinds.
 //
-// What bounds it: no single thing.  A tile takes about 4200 clocks; HBM and the tensor pipe are each half busy (its 44 MMAs are
-// 2050 clocks), and the issuer, the builders and the epilogue are each at work for 3200 of them (with the builders' loop cut to an
+// What bounds it: no single thing.  A tile takes about 4200 clocks; HBM is half busy; the tensor pipe is taken for 2600 of them (20 MMAs
+// with N = 128 at 64 clocks, and the 24 of dh1, N = 64, at the 55 that one takes instead of 32; its counter, of useful clocks, says 48 %),
+// and the issuer, the builders and the epilogue are each at work for 3200 (with the builders' loop cut to an
 // eighth, or most MMAs left out, 2.25 ms become 2.1).  B200, 131072 envs, 8 x 8, T = 64, fp32: the two kernels this one replaces (heads with
 // dW2; dh1 with the agent plane; dh2 out to HBM and back) 2.18 + 1.19 ms, this one 2.25; the whole iteration 5.94 -> 4.95 ms.  2500 envs,
 // 9 x 9, T = 24: 26 + 19 -> 33 us; rollout and four PPO epochs 420 -> 367 us.  Tried: sixteen builder warps 2.39 ms (fewer registers);
@@ -318,7 +319,6 @@ __global__ void __launch_bounds__(Back128Cfg<PREC>::THREADS, 1)
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&qfull[buf]);
             };
-            // (each set of loads stays in registers of its own until it is used: moved from one to the next it would be waited for)
             RowIn in;
             row_load(in);
 #pragma unroll 1
