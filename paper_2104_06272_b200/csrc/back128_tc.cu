@@ -20,7 +20,7 @@
 // Every wait is bounded; a timeout raises DEV_E_WAIT_TIMEOUT and the CTA unwinds.
 //
 // What bounds it: no single thing.  A tile takes about 4200 clocks; HBM is half busy; the tensor pipe is taken for 2600 of them (20 MMAs
-// with N = 128 at 64 clocks, and the 24 of dh1, N = 64, at the 55 that one takes instead of 32; its counter, of useful clocks, says 48 %),
+// with N = 128 at 64 clocks, and the 24 of dh1, N = 64, at the 55 that one takes instead of 32; its counter, of useful clocks, says 47 %),
 // and the issuer, the builders and the epilogue are each at work for 3200 (with the builders' loop cut to an
 // eighth, or most MMAs left out, 2.25 ms become 2.1).  B200, 131072 envs, 8 x 8, T = 64, fp32: the two kernels this one replaces (heads with
 // dW2; dh1 with the agent plane; dh2 out to HBM and back) 2.18 + 1.19 ms, this one 2.25; the whole iteration 5.94 -> 4.95 ms.  2500 envs,
